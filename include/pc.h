@@ -118,9 +118,8 @@ PC_API int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q,
  * flight and return; the host then treats the call's results as undefined (PC_ERR_TIMEOUT).
  *   wait_limit_cycles      limit for all later launches of this process (0: the default of
  *                          about 2e9 cycles, a second);
- *   skip_final_publication non-zero: the single-CTA chunk-prefill kernel (head size 64, or an
- *                          odd number of q-heads per kv-head) leaves out ONE signal that carries
- *                          no data - the "no more work" message to its consumer warps after the
+ *   skip_final_publication non-zero: the single-CTA chunk-prefill kernel (head size 64)
+ *                          leaves out ONE signal that carries no data - the "no more work" message to its consumer warps after the
  *                          last work item, when nothing is in flight any more - so that their
  *                          wait runs out.  Outputs of such a call are complete; its status_word
  *                          is non-zero.  Zero switches the hook off again.

@@ -995,8 +995,8 @@ static cudaError_t launch_prefill_t(const CUtensorMap* maps, const PrefillParams
   return cudaGetLastError();
 }
 
-cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int d, int grid, cudaStream_t st) {
-  return d == 128 ? launch_prefill_t<128>(maps, prm, grid, st) : launch_prefill_t<64>(maps, prm, grid, st);
+cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int grid, cudaStream_t st) {
+  return launch_prefill_t<64>(maps, prm, grid, st);
 }
 
 template <int D>

@@ -16,12 +16,13 @@ struct PrefillParams {
   float* win_score;              // [C,Hkv,L]
   int* status;                   // device status word or null
   int* counter;                  // work-queue counter, zeroed before launch
+  float* lse2;                   // [C,Hq,wp] scratch: log-sum-exp of the window rows (log2 units), wp = w rounded up to 8
   int wait_kcycles;              // limit of every device-side wait, in units of 1024 cycles
   int skip_final_publication;    // test hook of the bounded waits (see pc_debug_bounded_wait_test in pc.h)
 };
 
-// maps: rotated q (box 64x1x128x1), k_rot, v, o (store), rotated q with a w-row box
-cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int d, int grid, cudaStream_t st);
+// Head size 64.  maps: rotated q (box 64x1x128x1), k_rot, v, o (store), rotated q with a wp-row box
+cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int grid, cudaStream_t st);
 
 // Head size 128: CTA-pair kernel (pc_prefill2.cu).  maps as above plus maps[5] = rotated keys with a 64-token box.
 cudaError_t launch_prefill_pair(const CUtensorMap* maps, const PrefillParams& prm, int sm_count, cudaStream_t st);

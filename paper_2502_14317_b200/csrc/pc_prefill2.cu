@@ -1,33 +1,23 @@
 // Chunk-local causal attention with fused query-window scores (Eq. 1-2, Eq. 5-6) for head
 // size 128 on CTA pairs.
 //
-// Two CTAs of a cluster work as one unit (tcgen05 cta_group::2).  Each CTA owns ONE 128-row
-// query block; the two blocks of a pair read the same K/V (two q-heads of one kv-head at the
-// same query tile, or two adjacent query tiles of one head), so every 128-key tile is split
-// between the two shared memories: each CTA stages 64 keys of K and 64 head-dim columns of V
-// and the tensor cores of both SMs read both halves.  That halves the shared-memory traffic
-// per MMA, which is what limits a single CTA with two blocks at this head size.
+// Two CTAs of a cluster work as one unit (tcgen05 cta_group::2).  Each CTA owns TWO 128-row query blocks A and B, so
+// four blocks walk the same K/V tiles at a time: every 128-key tile is split between the two shared memories (each CTA
+// stages 64 keys of K and 64 head-dim columns of V) and one MMA of M = 256 feeds both SMs.  While the softmax of one
+// block runs the tensor cores work for the other.
 //
-// Per CTA, TMEM holds two S buffers (one per softmax warpgroup, 128 columns each), two P buffers
-// (64 columns of bf16 each) and one accumulator (128 columns).  Two softmax warpgroups take
-// alternate key tiles (thread = query row), chained only through the short per-row decision on the
-// running maximum.  As soon as a warpgroup has S(j) in registers, Q K^T of its next tile S(j+2)
-// may run into the same buffer, so that S is waiting when the warpgroup comes back; P(j) goes to
-// the warpgroup's P buffer once P V of its previous tile has run.
+// Per CTA, TMEM holds S and (over its first half) P of both blocks, 128 columns each, and both accumulators.
 //
-// Warps (12 per CTA): 0-3 softmax of even tiles, 4-7 softmax of odd tiles (both: epilogue and score
-// sweep split by halves),
-// 8 TMA producer, 9 issuer of Q K^T, 10 and 11 issuers of P V for even / odd tiles (issuers run in
-// the leader CTA only).  Several issuers because a tcgen05.mma issue blocks while the pipe is busy
-// and every barrier wait or commit of an issuing thread costs it about a hundred cycles.
+// Warps (16 per CTA): 0-3 softmax of block A, 4-7 softmax of block B (thread = query row = TMEM lane), 8-11 epilogue (the
+// softmax warps go straight on to the next block), 12 TMA producer, 13 issuer of all MMAs (leader CTA only), 14-15 idle.
+// Registers are dealt out by role: 184 / 80 / 64.
 //
-// Window scores: the pair that runs the last query tiles of a (chunk, kv-head) group keeps the
-// window rows' log-sum-exp in both shared memories, then sweeps the keys once more with the
-// transposed product K_j Qw^T (each CTA takes every other key tile; keys on TMEM lanes, window
+// Window scores: the pair that runs the last query tiles of a (chunk, kv-head) group then sweeps the keys once more
+// with the transposed product K_j Qw^T (each CTA takes every other key tile; keys on TMEM lanes, window
 // rows on columns), so Eq. 6 is a per-thread sum in a fixed order: deterministic, fp32, no atomics.
-#include "pc_kernels.h"
 #include "pc_attn.h"
-#include "pc_sm100.cuh"
+#include "pc_kernels.h"
+#include "pc_softmax.cuh"
 
 namespace pc {
 
@@ -35,108 +25,102 @@ namespace {
 
 constexpr int TILE = 128;
 constexpr int D = 128;
-constexpr int NT2 = 384;                     // threads per CTA
-constexpr int WARP_PRODUCER = 8, WARP_QK = 9, WARP_PV = 10;
-constexpr int NKS = 4, NVS = 4;              // K / V ring stages (16 KB each)
-constexpr int NSB = 2;                       // S buffers in TMEM (one per warpgroup); P has buffers of its own
-constexpr uint32_t TM_P = 256;               // two P buffers of 64 columns (128 bf16 keys each), one per warpgroup
-constexpr int HALF_BYTES = 16384;            // 64 keys x 128 d of K, or 128 keys x 64 d of V
+constexpr int NT2 = 512;                     // threads per CTA
+constexpr int WARP_EPI = 8, WARP_PRODUCER = 12, WARP_MMA = 13;
+constexpr int REGS_SOFTMAX = 184, REGS_EPI = 80, REGS_SERVICE = 64;      // 128 * (2 * 184 + 80 + 64) = 64 K registers
+constexpr int NQ = 4;                        // query slots: the two blocks in work and the two that come next
+constexpr int NS = 6;                        // K/V ring stages (16 KB: 64 keys x 128 d of K, or 128 keys x 64 d of V)
+constexpr int NDESC = 4;                     // work descriptors in flight
+constexpr int HALF_BYTES = 16384;
 constexpr int Q_BYTES = 32768;
-constexpr uint32_t TM_O = 384;               // accumulator columns
-constexpr float LAZY_RESCALE = 8.0f;         // log2 units
+constexpr uint32_t TM_O = 256;               // accumulator columns (block b: + 128 b)
 
-enum { W2_QFULL = 201, W2_QFREE, W2_KFULL, W2_KFREE, W2_VFULL, W2_VFREE, W2_SFULL, W2_PA, W2_PB,
-       W2_PVDONE, W2_OFULL, W2_ACCFREE, W2_LSE, W2_TFULL, W2_TFREE, W2_MPUB, W2_TURN };
+enum { W2_ITEM = 201, W2_QFULL, W2_QFREE, W2_KVFULL, W2_KVFREE, W2_DESC, W2_SFULL, W2_PHALF, W2_PFULL, W2_OFULL, W2_OFREE, W2_LM,
+       W2_LMFREE, W2_LSE, W2_TFULL, W2_TFREE };
+
+enum { KIND_DONE = 0, KIND_FLASH = 1, KIND_SWEEP = 2 };
+struct __align__(16) Desc {
+  int kind, c, hkv, len;       // chunk, kv-head, tokens of the chunk
+  int h[2], t[2];              // FLASH: q-head and query tile of this CTA's block A / B (t < 0 or behind the chunk: no such
+                               // tile, the rows are computed on zeros and not stored);  SWEEP: h[0] = pass
+  int n[2];                    // FLASH: key tiles the pair walks for block A / B; 0: block absent in both CTAs
+};
 
 struct __align__(16) Misc2 {
-  uint64_t q_full[2], q_free[2];             // q_full: leader only, counts the bytes of both CTAs' query tiles
-  uint64_t k_full[NKS], k_free[NKS], v_full[NVS], v_free[NVS];
-  uint64_t s_full[2][NSB];                   // [owning warpgroup][buffer]: a waiter must see every phase of its barrier
-  uint64_t p_a[2][NSB], p_b[2][NSB];         // [owning warpgroup = P V issuer][buffer]
-  uint64_t s_read[NSB];                      // leader only: S of the tile in this buffer is in registers (8 warps of the pair)
-  uint64_t pv_turn[2];                       // leader only: issue token of the two P V issuers
-  uint64_t o_full, acc_free, lse_ready;
-  uint64_t t_full[2], t_free[2];
-  uint64_t m_pub[2][4];                      // [owner warpgroup][warp]: its reference maxima of a tile are in mref
-  uint64_t mma_done;                         // every tensor-core operation of the three issuers has completed (teardown)
+  uint64_t q_full[NQ], q_free[NQ];           // q_full, kv_full: leader only, count the bytes of both CTAs
+  uint64_t kv_full[NS], kv_free[NS];
+  uint64_t s_full[2], o_full[2], t_full[2];  // completion of MMAs, signalled in both CTAs
+  uint64_t p_half[2], p_full[2], o_free[2], t_free[2];   // leader only, arrivals of both CTAs
+  uint64_t lm_full[2], lm_free[2];
+  uint64_t d_full[NDESC], d_free[NDESC];
+  uint64_t item_full, item_free;             // work items from the leader's producer to its peer's
+  uint64_t lse_rdy;
+  uint64_t mma_done;
+  Desc desc[NDESC];
+  int item;
   uint32_t tmem_base;
   int abort_flag;                            // the two words after tmem_base stay adjacent: bounded waits read the limit
   int wait_kcycles;                          // through the flag's address
-  float lse2[1024];                          // window-row log-sum-exp (log2 units) of all G heads, G * w <= 1024
-  float mref[2][TILE];                       // [tile parity][row]: reference maximum (log2 units) after that tile
-  float xl[2][TILE];                         // [key half][row]: half-row sums
-  float xs[2][2][TILE];                      // [buffer][column half][key]: partial window scores
+  float lm[2][2][TILE];                      // [block][max / sum][row]: final statistics of a block; in the score sweep
+                                             // [buffer][key]: partial window scores of the second column half
 };
 
 constexpr int OFF_Q = 0;
-constexpr int OFF_RK = 2 * Q_BYTES;
-constexpr int OFF_RV = OFF_RK + NKS * HALF_BYTES;
-constexpr int OFF_MISC = OFF_RV + NVS * HALF_BYTES;
-constexpr int SMEM2_BYTES = OFF_MISC + (int)sizeof(Misc2) + 1024;
+constexpr int OFF_RING = NQ * Q_BYTES;
+constexpr int OFF_MISC = OFF_RING + NS * HALF_BYTES;
+constexpr int SMEM2_BYTES = OFF_MISC + (int)sizeof(Misc2);
+static_assert(SMEM2_BYTES <= 232448, "shared memory of a CTA");
 
 __device__ __forceinline__ uint32_t full_par(uint32_t n) { return n & 1u; }           // n-th completion of a barrier
 __device__ __forceinline__ uint32_t free_par(uint32_t n) { return (n & 1u) ^ 1u; }    // completion n-1 (passes for n = 0)
 
 // ------------------------------------------------------------------ work decomposition
-// Groups = (chunk, kv-head); the items of a group are ordered heaviest first; item 0 of a
-// group (the tail item) holds the query tiles with window rows for all G heads, then the sweep.
-// The two CTAs of a pair take the same query tile of two q-heads of the kv-head, so G must be even (an odd
-// group size would leave a pair with two different query tiles of one head, one of them walking a masked
-// key tile; such shapes run on the single-CTA kernel instead).
-// Division of n < 2^31 by a fixed divisor as a multiplication (round-up method with a 32-bit multiplier).
-struct FastDiv {
-  uint32_t d, mul, shr;
-  __device__ __forceinline__ void init(uint32_t div) {
-    d = div;
-    uint32_t l = 0;
-    while ((1u << l) < div) ++l;                           // ceil(log2(div))
-    shr = 31u + l;
-    mul = static_cast<uint32_t>(((1ull << shr) + div - 1) / div);
-  }
-  __device__ __forceinline__ int quot(int n) const {
-    return static_cast<int>((static_cast<uint64_t>(static_cast<uint32_t>(n)) * mul) >> shr);
-  }
-  __device__ __forceinline__ void divmod(int n, int& q, int& r) const {
-    q = quot(n);
-    r = n - q * static_cast<int>(d);
-  }
-};
-
+// Groups = (chunk, kv-head).  A unit is what the four blocks of a pair take at a time:
+//   G % 4 == 0   one query tile of four q-heads (block A: heads 0, 1 of the four; B: heads 2, 3; one per CTA)
+//   G % 2 == 0   two adjacent tiles of two q-heads (A: lower tile; B: upper tile; one head per CTA)
+//   G odd        four adjacent tiles of one q-head (A: the lower two, B: the upper two; one per CTA; the lower tile of a
+//                block walks one fully masked key tile, 3 % of the tiles at 32 tiles a chunk)
+// counted from the last tile of the chunk.  Item 0 of a group (the tail item) holds the units with window rows for all
+// q-heads, then the score sweep; the other items are one unit each, heaviest first.
+// Items are dealt out in batches of groups whose keys and values stay in L2 together, heaviest first over the whole
+// batch, so that what is dealt last is light (one group at a time, the last blocks ended 4 % after the median one).
 // With per-chunk lengths the query tiles of a shorter chunk are numbered from the END: slot v of the static
-// decomposition (v = T - 1 is the last tile of a full-length chunk) is tile v - (T - T_c) of a chunk with T_c tiles,
-// and slots below T - T_c are empty.  The window then always sits in the last one or two slots, which the tail item
-// of the group owns together with the score sweep.
+// decomposition (v = T - 1 is the last tile of a full-length chunk) is tile v - (T - T_c) of a chunk with T_c tiles.
+// The window then always sits in the last one or two slots, which the tail item owns together with the score sweep.
 struct Sched2 {
-  int T, t_w, ntt, G, P, ipg, hp, n_pass, wp;
-  FastDiv d_ipg, d_hkv, d_ntt, d_P;
+  int T, G, hpu, tpu, P, U, ntu, ipg, batch, hp, n_pass, wp;
 };
 __device__ __forceinline__ Sched2 make_sched2(const PrefillParams& p) {
   Sched2 s;
   s.T = (p.L + TILE - 1) / TILE;
   s.G = p.Hq / p.Hkv;
-  s.P = s.G / 2;
-  // slots of the tail item: the tiles that can hold window rows (with per-chunk lengths the window of some chunk
-  // may straddle two tiles even where that of a full-length chunk does not)
-  s.ntt = (p.chunk_len != nullptr) ? (p.w > 1 ? 2 : 1) : s.T - (p.L - p.w) / TILE;
-  if (s.ntt > s.T) s.ntt = s.T;
-  s.t_w = s.T - s.ntt;
-  s.ipg = 1 + s.t_w * s.P;
+  s.hpu = s.G % 4 == 0 ? 4 : (s.G % 2 == 0 ? 2 : 1);      // q-heads and tiles of a unit
+  s.tpu = 4 / s.hpu;
+  s.P = s.G / s.hpu;
+  s.U = (s.T + s.tpu - 1) / s.tpu;
+  // tail units: those that can hold window rows (with per-chunk lengths the window of some chunk may straddle two
+  // tiles even where that of a full-length chunk does not)
+  const int ntt = (p.chunk_len != nullptr) ? (p.w > 1 ? 2 : 1) : s.T - (p.L - p.w) / TILE;
+  s.ntu = (ntt + s.tpu - 1) / s.tpu;
+  if (s.ntu > s.U) s.ntu = s.U;
+  s.ipg = 1 + (s.U - s.ntu) * s.P;
+  const long long kv_bytes = (long long)p.L * (4 * D);    // K and V of a group
+  s.batch = (int)((48ll << 20) / kv_bytes);
+  if (s.batch < 1) s.batch = 1;
   s.wp = (p.w + 7) & ~7;                                  // window rows of a head in the sweep operand (multiple of 8)
-  const int cap = TILE / s.wp, want = s.G / 2;
+  const int cap = TILE / s.wp, want = (s.G + 1) / 2;
   s.hp = cap < want ? cap : want;                         // window heads per CTA and sweep pass
   s.n_pass = (s.G + 2 * s.hp - 1) / (2 * s.hp);
-  s.d_ipg.init(s.ipg); s.d_hkv.init(p.Hkv); s.d_ntt.init(s.ntt); s.d_P.init(s.P);
   return s;
 }
-__device__ __forceinline__ int n_subitems2(const Sched2& s, int within) {
-  if (within != 0) return 1;
-  return s.P * s.ntt;
+// item -> (group, item within the group)
+__device__ __forceinline__ void decode_item(const Sched2& s, int n_groups, int item, int& group, int& within) {
+  const int per_batch = s.batch * s.ipg;
+  const int b = item / per_batch, rem = item - b * per_batch, g0 = b * s.batch;
+  const int size = n_groups - g0 < s.batch ? n_groups - g0 : s.batch;
+  within = rem / size;
+  group = g0 + rem - within * size;
 }
-struct Blk {
-  int h;       // q-head of this CTA's block
-  int t;       // query tile of this CTA's block
-  int n;       // key tiles the pair walks
-};
 // length of chunk c in tokens (window included), clamped to (w, L]
 __device__ __forceinline__ int chunk_length(const PrefillParams& p, int c) {
   if (p.chunk_len == nullptr) return p.L;
@@ -144,36 +128,47 @@ __device__ __forceinline__ int chunk_length(const PrefillParams& p, int c) {
   len = len > p.L ? p.L : len;
   return len <= p.w ? p.w + 1 : len;
 }
-// len: length of the block's chunk.  b.n == 0: an empty slot, every role skips the block.
-__device__ __forceinline__ Blk decode_blk(const Sched2& s, int rank, int hkv, int within, int sub, int len) {
-  Blk b;
-  const int h0 = hkv * s.G;
-  int pair, tile;
-  if (within == 0) { int rem; s.d_ntt.divmod(sub, pair, rem); tile = s.T - 1 - rem; }
-  else { int q; s.d_P.divmod(within - 1, q, pair); tile = s.t_w - 1 - q; }
-  tile -= s.T - (len + TILE - 1) / TILE;
-  b.h = h0 + 2 * pair + rank;
-  b.t = tile;
-  b.n = tile < 0 ? 0 : tile + 1;
-  return b;
+// blocks of sub-item `sub` (of the tail item, or 0)
+__device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, int within, int sub, Desc& d) {
+  const int x = within == 0 ? sub : s.ntu * s.P + within - 1;
+  const int unit = x / s.P, set = x - unit * s.P;
+  const int hi = s.T - 1 - unit * s.tpu - (s.T - (d.len + TILE - 1) / TILE);      // upper tile of the unit
+  const int h0 = hkv * s.G + set * s.hpu;
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    int top;                                              // upper tile of the block over both CTAs
+    if (s.hpu == 4) { d.h[b] = h0 + 2 * b + rank; top = hi; d.t[b] = hi; }
+    else if (s.hpu == 2) { d.h[b] = h0 + rank; top = hi - 1 + b; d.t[b] = top; }
+    else { d.h[b] = h0; top = hi - 2 + 2 * b; d.t[b] = top - 1 + rank; }
+    d.n[b] = top < 0 ? 0 : top + 1;
+  }
 }
 
 struct Ctx2 {
   Misc2* mi;
-  uint8_t* sQ[2];
-  uint8_t* rK;
-  uint8_t* rV;
+  uint8_t* sQ;
+  uint8_t* ring;
   uint32_t tmem;
-  uint32_t rank;
   volatile int* abort_flag;
   int* status;
 };
 
-// waits of the single-thread service roles (long pause between polls) / of the softmax warps
+// waits of the single-thread service roles (long pause between polls) / of the softmax and epilogue warps
 #define WAIT2(bar, par, code) mbar_wait_ns<SERVICE_BACKOFF_NS>((bar), (par), cx.abort_flag, cx.status, (code))
 #define WAIT2S(bar, par, code) mbar_wait((bar), (par), cx.abort_flag, cx.status, (code))
 
-// wait whose completion also makes the peer CTA's earlier shared-memory writes visible
+__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+// one arrival of the warp on a barrier of the leader CTA; guards TMEM data, ordered by the tcgen05 fence
+__device__ __forceinline__ void warp_arrive_leader(uint32_t leader_addr) {
+  tc_fence_before_sync();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive_remote(leader_addr);
+}
+
+// wait whose completion also makes the peer CTA's earlier writes visible
 __device__ __forceinline__ void mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                   int where) {
   if (mbar_try_wait_cluster(bar, parity)) return;
@@ -191,24 +186,75 @@ __device__ __forceinline__ void mbar_wait_cluster(uint64_t* bar, uint32_t parity
   }
 }
 
-__device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles) {
+__device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool leader) {
+  for (int i = 0; i < NQ; ++i) { mbar_init(&mi.q_full[i], 1); mbar_init(&mi.q_free[i], 1); }
+  for (int i = 0; i < NS; ++i) { mbar_init(&mi.kv_full[i], 1); mbar_init(&mi.kv_free[i], 1); }
   for (int b = 0; b < 2; ++b) {
-    mbar_init(&mi.q_full[b], 1); mbar_init(&mi.q_free[b], 1);
-    mbar_init(&mi.t_full[b], 1); mbar_init(&mi.t_free[b], 16);
+    mbar_init(&mi.s_full[b], 1); mbar_init(&mi.o_full[b], 1); mbar_init(&mi.t_full[b], 1);
+    mbar_init(&mi.p_half[b], 8); mbar_init(&mi.p_full[b], 8);         // 4 softmax warps of the block in each CTA
+    mbar_init(&mi.o_free[b], 8); mbar_init(&mi.t_free[b], 16);        // epilogue warps / softmax warps of both CTAs
+    mbar_init(&mi.lm_full[b], 4); mbar_init(&mi.lm_free[b], 4);
   }
-  for (int s = 0; s < NKS; ++s) { mbar_init(&mi.k_full[s], 1); mbar_init(&mi.k_free[s], 1); }
-  for (int s = 0; s < NVS; ++s) { mbar_init(&mi.v_full[s], 1); mbar_init(&mi.v_free[s], 1); }
-  for (int s = 0; s < NSB; ++s) {
-    mbar_init(&mi.s_full[0][s], 1); mbar_init(&mi.s_full[1][s], 1); mbar_init(&mi.s_read[s], 8);
-    for (int g = 0; g < 2; ++g) { mbar_init(&mi.p_a[g][s], 8); mbar_init(&mi.p_b[g][s], 8); }   // 4 warps of the owning warpgroup in each CTA
-  }
-  mbar_init(&mi.pv_turn[0], 1); mbar_init(&mi.pv_turn[1], 1);
-  mbar_init(&mi.o_full, 1); mbar_init(&mi.acc_free, 16); mbar_init(&mi.lse_ready, 16);
-  for (int w = 0; w < 4; ++w) { mbar_init(&mi.m_pub[0][w], 1); mbar_init(&mi.m_pub[1][w], 1); }   // warp to warp (same rows)
-  mbar_init(&mi.mma_done, 3);
+  for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 13 : 12); }   // softmax and epilogue warps, issuer
+  mbar_init(&mi.item_full, 1); mbar_init(&mi.item_free, 1);
+  mbar_init(&mi.lse_rdy, 8);
+  mbar_init(&mi.mma_done, 1);
   mi.abort_flag = 0;
   mi.wait_kcycles = wait_kcycles;
   fence_mbar_init();
+}
+
+// consumers of the descriptor ring.  whole_warp: all 32 threads call.
+__device__ __forceinline__ Desc next_desc(const Ctx2& cx, uint32_t& n, bool whole_warp) {
+  Misc2& mi = *cx.mi;
+  const int slot = n % NDESC;
+  Desc d;
+  if (!WAIT2S(&mi.d_full[slot], full_par(n / NDESC), W2_DESC) || *cx.abort_flag) { d.kind = KIND_DONE; return d; }
+  d = mi.desc[slot];
+  if (whole_warp) warp_arrive(&mi.d_free[slot]); else mbar_arrive(&mi.d_free[slot]);
+  ++n;
+  return d;
+}
+
+// ------------------------------------------------------------------ producer
+struct Prod { uint32_t kv = 0, q = 0, d = 0, item = 0; };
+__device__ __forceinline__ void publish(const Ctx2& cx, Prod& p, const Desc& d) {
+  Misc2& mi = *cx.mi;
+  const int slot = p.d % NDESC;
+  WAIT2(&mi.d_free[slot], free_par(p.d / NDESC), W2_DESC);
+  mi.desc[slot] = d;
+  mbar_arrive(&mi.d_full[slot]);
+  ++p.d;
+}
+// The leader's producer draws items from the queue and hands each to its peer's.
+__device__ __forceinline__ int next_item(const Ctx2& cx, Prod& p, bool leader, int* counter, int n_items) {
+  Misc2& mi = *cx.mi;
+  int item;
+  if (leader) {
+    item = atomicAdd(counter, 1);
+    if (item > n_items) item = n_items;
+    WAIT2(&mi.item_free, free_par(p.item), W2_ITEM);      // the peer has read the previous one
+    st_async_u32(map_to_cta(&mi.item, 1), static_cast<uint32_t>(item), map_to_cta(&mi.item_full, 1));
+  } else {
+    mbar_arrive_expect_tx(&mi.item_full, 4);
+    if (!WAIT2(&mi.item_full, full_par(p.item), W2_ITEM)) return n_items;
+    item = *reinterpret_cast<volatile int*>(&mi.item);
+    mbar_arrive_remote(map_to_cta(&mi.item_free, 0));
+  }
+  ++p.item;
+  return item;
+}
+// expects a stage's bytes over both CTAs on the leader's barrier of the next ring stage; returns that barrier's address
+// for the copies and the stage's place; 0 once a wait has run out (no copy is issued into a ring that nobody drains)
+__device__ __forceinline__ uint32_t ring_stage(const Ctx2& cx, Prod& p, bool leader, uint8_t** dst) {
+  Misc2& mi = *cx.mi;
+  if (*cx.abort_flag) return 0;
+  const int s = p.kv % NS;
+  if (!WAIT2(&mi.kv_free[s], free_par(p.kv / NS), W2_KVFREE)) return 0;
+  if (leader) mbar_arrive_expect_tx(&mi.kv_full[s], 2 * HALF_BYTES);
+  *dst = cx.ring + s * HALF_BYTES;
+  ++p.kv;
+  return map_to_cta(&mi.kv_full[s], 0);
 }
 
 }  // namespace
@@ -218,557 +264,435 @@ __device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles) {
 // ====================================================================================
 // tensor maps: tm_q (box 64 d x 128 tokens), tm_kh (rotated keys, box 64 d x 64 tokens),
 // tm_k (rotated keys, box 64 d x 128 tokens), tm_v (box 64 d x 128 tokens), tm_o (store,
-// box 64 d x 128 tokens), tm_qw (box 64 d x w tokens)
+// box 64 d x 128 tokens), tm_qw (box 64 d x wp tokens)
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT2, 1)
 prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kh,
                     const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                     const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ CUtensorMap tm_qw,
                     const __grid_constant__ PrefillParams prm) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  extern __shared__ __align__(1024) uint8_t smem[];
   Misc2& mi = *reinterpret_cast<Misc2*>(smem + OFF_MISC);
   Ctx2 cx;
   cx.mi = &mi;
-  cx.sQ[0] = smem + OFF_Q;
-  cx.sQ[1] = smem + OFF_Q + Q_BYTES;
-  cx.rK = smem + OFF_RK;
-  cx.rV = smem + OFF_RV;
+  cx.sQ = smem + OFF_Q;
+  cx.ring = smem + OFF_RING;
   cx.abort_flag = &mi.abort_flag;
   cx.status = prm.status;
-  cx.rank = cluster_ctarank();
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t rank = cx.rank;
+  const uint32_t rank = cluster_ctarank();
   const bool leader = (rank == 0);
-  const Sched2 sch = make_sched2(prm);
-  const int n_items = prm.C * prm.Hkv * sch.ipg;
-  const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int rows_half = sch.hp * sch.wp;                 // sweep operand rows per CTA and pass (B operand half)
 
-  if (tid == 0) init_barriers2(mi, prm.wait_kcycles);
-  if (warp == WARP_QK) tmem_alloc_pair(&mi.tmem_base, 512);
+  if (tid == 0) init_barriers2(mi, prm.wait_kcycles, leader);
+  if (warp == WARP_MMA) tmem_alloc_pair(&mi.tmem_base, 512);
   tc_fence_before_sync();
   __syncthreads();
   cluster_sync_all();                                    // both CTAs' barriers exist before any remote arrive
   tc_fence_after_sync();
   cx.tmem = mi.tmem_base;
 
-  if (warp == WARP_PRODUCER) {
-    // ================================================================ TMA producer (both CTAs)
-    if (lane == 0) {
-      tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kh); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
-      tma_prefetch_desc(&tm_qw);
-      uint32_t cQ = 0, cK = 0, cV = 0;
-      // Once a wait has run out (abort flag) no new work is started: every role leaves its loops at the next item,
-      // this one also at the next tile, so that no copy is issued into a ring that nobody drains any more.
-      for (int item = pair_id; item < n_items && !*cx.abort_flag; item += n_pairs) {
-        int group, within, c, hkv;
-        sch.d_ipg.divmod(item, group, within);
-        sch.d_hkv.divmod(group, c, hkv);
-        const int nsub = n_subitems2(sch, within);
-        const int len = chunk_length(prm, c);
-        for (int sub = 0; sub < nsub; ++sub) {
-          const Blk bk = decode_blk(sch, rank, hkv, within, sub, len);
-          if (bk.n == 0) continue;
-          {
-            const int qb = cQ & 1;
-            WAIT2(&mi.q_free[qb], free_par(cQ >> 1), W2_QFREE);
-            if (leader) mbar_arrive_expect_tx(&mi.q_full[qb], 2 * Q_BYTES);
-            const uint32_t bar = map_to_cta(&mi.q_full[qb], 0);
-            for (int a = 0; a < 2; ++a) tma_load_4d_pair(cx.sQ[qb] + a * 16384, &tm_q, bar, a * 64, bk.h, bk.t * TILE, c);
-            ++cQ;
-          }
-          for (int j = 0; j < bk.n && !*cx.abort_flag; ++j) {
-            {
-              const int s = cK % NKS;
-              WAIT2(&mi.k_free[s], free_par(cK / NKS), W2_KFREE);
-              if (leader) mbar_arrive_expect_tx(&mi.k_full[s], 2 * HALF_BYTES);
-              const uint32_t bar = map_to_cta(&mi.k_full[s], 0);
+  if (warp >= WARP_PRODUCER) {
+    setmaxnreg_dec<REGS_SERVICE>();
+    if (warp == WARP_PRODUCER) {
+      // ================================================================ TMA producer (both CTAs)
+      if (elect_one()) {
+        const Sched2 sch = make_sched2(prm);
+        const int n_groups = prm.C * prm.Hkv, n_items = n_groups * sch.ipg;
+        const int rows_half = sch.hp * sch.wp;           // sweep operand rows per CTA and pass (B operand half)
+        tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kh); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
+        tma_prefetch_desc(&tm_qw);
+        Prod p;
+        // Once a wait has run out (abort flag) no new work is started: every role leaves its loops at the next
+        // descriptor, this one also at the next tile, so that no copy is issued into a ring that nobody drains.
+        while (!*cx.abort_flag) {
+          const int item = next_item(cx, p, leader, prm.counter, n_items);
+          if (item >= n_items) break;
+          int group, within;
+          decode_item(sch, n_groups, item, group, within);
+          Desc d;
+          d.c = group / prm.Hkv;
+          d.hkv = group - d.c * prm.Hkv;
+          d.len = chunk_length(prm, d.c);
+          uint8_t* dst;
+          const int nsub = within == 0 ? sch.ntu * sch.P : 1;
+          for (int sub = 0; sub < nsub; ++sub) {
+            d.kind = KIND_FLASH;
+            decode_unit(sch, rank, d.hkv, within, sub, d);
+            if (d.n[1] == 0) continue;                    // (n[0] <= n[1])
+            publish(cx, p, d);
+            for (int b = 0; b < 2; ++b) {
+              if (d.n[b] == 0) continue;
+              const int qs = p.q % NQ;
+              WAIT2(&mi.q_free[qs], free_par(p.q / NQ), W2_QFREE);
+              if (leader) mbar_arrive_expect_tx(&mi.q_full[qs], 2 * Q_BYTES);
+              const uint32_t bar = map_to_cta(&mi.q_full[qs], 0);
               for (int a = 0; a < 2; ++a)
-                tma_load_4d_pair(cx.rK + s * HALF_BYTES + a * 8192, &tm_kh, bar, a * 64, hkv, j * TILE + (int)rank * 64, c);
-              ++cK;
+                tma_load_4d_pair(cx.sQ + qs * Q_BYTES + a * 16384, &tm_q, bar, a * 64, d.h[b], d.t[b] * TILE, d.c);
+              ++p.q;
             }
-            {
-              const int s = cV % NVS;
-              WAIT2(&mi.v_free[s], free_par(cV / NVS), W2_VFREE);
-              if (leader) mbar_arrive_expect_tx(&mi.v_full[s], 2 * HALF_BYTES);
-              tma_load_4d_pair(cx.rV + s * HALF_BYTES, &tm_v, map_to_cta(&mi.v_full[s], 0), (int)rank * 64, hkv, j * TILE, c);
-              ++cV;
+            for (int j = 0; j < d.n[1]; ++j) {
+              const uint32_t kbar = ring_stage(cx, p, leader, &dst);
+              if (kbar)
+                for (int a = 0; a < 2; ++a) tma_load_4d_pair(dst + a * 8192, &tm_kh, kbar, a * 64, d.hkv, j * TILE + (int)rank * 64, d.c);
+              const uint32_t vbar = ring_stage(cx, p, leader, &dst);
+              if (vbar) tma_load_4d_pair(dst, &tm_v, vbar, (int)rank * 64, d.hkv, j * TILE, d.c);
             }
           }
-        }
-        if (within == 0) {
-          // ---- score sweep: window queries of hp heads per CTA and pass, then this CTA's key tiles.  A head's rows
-          // in the operand are the wp tokens that end with the chunk (wp = w rounded up to 8: the first wp - w rows
-          // are not window rows and are left out of the sums; a start before token 0 reads zeros)
-          const int n_sweep_tiles = ((len + TILE - 1) / TILE + 1) / 2;
-          for (int u = 0; u < sch.n_pass; ++u) {
-            const int qb = cQ & 1;
-            WAIT2(&mi.q_free[qb], free_par(cQ >> 1), W2_QFREE);
-            if (leader) mbar_arrive_expect_tx(&mi.q_full[qb], 2 * rows_half * D * 2);
-            const uint32_t bar = map_to_cta(&mi.q_full[qb], 0);
-            for (int i = 0; i < sch.hp; ++i) {
-              int g = u * 2 * sch.hp + (int)rank * sch.hp + i;
-              if (g >= sch.G) g = sch.G - 1;              // filler rows: loaded, never summed
-              for (int a = 0; a < 2; ++a)
-                tma_load_4d_pair(cx.sQ[qb] + a * 16384 + i * sch.wp * 128, &tm_qw, bar, a * 64, hkv * sch.G + g,
-                                 len - sch.wp, c);
-            }
-            ++cQ;
-            if (cK & 1) {                                 // a full key tile takes an even-aligned pair of stages
-              const int s = cK % NKS;
-              WAIT2(&mi.k_free[s], free_par(cK / NKS), W2_KFREE);
-              if (leader) mbar_arrive(&mi.k_full[s]);
-              ++cK;
-            }
-            for (int jj = 0; jj < n_sweep_tiles && !*cx.abort_flag; ++jj) {
-              const int tile = 2 * jj + (int)rank;
-              for (int a = 0; a < 2; ++a) {
-                const int s = cK % NKS;
-                WAIT2(&mi.k_free[s], free_par(cK / NKS), W2_KFREE);
-                if (leader) mbar_arrive_expect_tx(&mi.k_full[s], 2 * HALF_BYTES);
-                tma_load_4d_pair(cx.rK + s * HALF_BYTES, &tm_k, map_to_cta(&mi.k_full[s], 0), a * 64, hkv, tile * TILE, c);
-                ++cK;
+          if (within == 0) {
+            // ---- score sweep: window queries of hp heads per CTA and pass, then this CTA's key tiles.  A head's rows
+            // in the operand are the wp tokens that end with the chunk (wp = w rounded up to 8: the first wp - w rows
+            // are not window rows and are left out of the sums; a start before token 0 reads zeros)
+            const int n_steps = ((d.len + TILE - 1) / TILE + 1) / 2;
+            for (int u = 0; u < sch.n_pass; ++u) {
+              d.kind = KIND_SWEEP;
+              d.h[0] = u;
+              publish(cx, p, d);
+              const int qs = p.q % NQ;
+              WAIT2(&mi.q_free[qs], free_par(p.q / NQ), W2_QFREE);
+              if (leader) mbar_arrive_expect_tx(&mi.q_full[qs], 2 * rows_half * D * 2);
+              const uint32_t bar = map_to_cta(&mi.q_full[qs], 0);
+              for (int i = 0; i < sch.hp; ++i) {
+                int g = u * 2 * sch.hp + (int)rank * sch.hp + i;
+                if (g >= sch.G) g = sch.G - 1;            // filler rows: loaded, never summed
+                for (int a = 0; a < 2; ++a)
+                  tma_load_4d_pair(cx.sQ + qs * Q_BYTES + a * 16384 + i * sch.wp * 128, &tm_qw, bar, a * 64,
+                                   d.hkv * sch.G + g, d.len - sch.wp, d.c);
               }
+              ++p.q;
+              // a full key tile takes two consecutive stages that start on an even one: everything uses stages in twos
+              for (int jj = 0; jj < n_steps; ++jj)
+                for (int a = 0; a < 2; ++a) {
+                  const uint32_t kbar = ring_stage(cx, p, leader, &dst);
+                  if (kbar) tma_load_4d_pair(dst, &tm_k, kbar, a * 64, d.hkv, (2 * jj + (int)rank) * TILE, d.c);
+                }
             }
           }
         }
-      }
-      // Every copy issued must have landed before a CTA may exit.  In a run without a timed-out wait that follows
-      // from the last uses of the rings having been consumed (the teardown below waits for every tensor-core
-      // operation).  After an abort nothing is consumed any more: the leader, whose barriers count the bytes of both
-      // CTAs' copies, waits on them (ignoring the abort flag, bounded); the peer cannot observe the completion of
-      // its own last copies and lets a fixed pause pass that outlasts any copy in flight.
-      if (*cx.abort_flag) {
-        if (leader) {
-          for (uint32_t i = (cK > NKS ? cK - NKS : 0); i < cK; ++i) mbar_wait_drain(&mi.k_full[i % NKS], full_par(i / NKS), cx.abort_flag);
-          for (uint32_t i = (cV > NVS ? cV - NVS : 0); i < cV; ++i) mbar_wait_drain(&mi.v_full[i % NVS], full_par(i / NVS), cx.abort_flag);
-          for (uint32_t i = (cQ > 2 ? cQ - 2 : 0); i < cQ; ++i) mbar_wait_drain(&mi.q_full[i & 1], full_par(i >> 1), cx.abort_flag);
-        }
-        abort_grace_pause(cx.abort_flag);
-      }
-    }
-    __syncwarp();
-  } else if (warp == WARP_QK) {
-    // ================================================================ issuer of S = Q K^T (leader CTA)
-    if (lane == 0 && leader) {
-      const uint32_t idesc_qk = make_idesc_bf16_f32(256, TILE, false, false);
-      const uint32_t idesc_sw = make_idesc_bf16_f32(256, 2 * rows_half, false, false);
-      const uint32_t rk_u32 = smem_u32(cx.rK);
-      uint32_t cQ = 0, cK = 0, cS = 0, cT = 0, n_done = 0;
-      for (int item = pair_id; item < n_items && !*cx.abort_flag; item += n_pairs) {
-        int group, within, c, hkv;
-        sch.d_ipg.divmod(item, group, within);
-        sch.d_hkv.divmod(group, c, hkv);
-        const int nsub = n_subitems2(sch, within);
-        const int len = chunk_length(prm, c);
-        for (int sub = 0; sub < nsub; ++sub) {
-          const Blk bk = decode_blk(sch, rank, hkv, within, sub, len);
-          if (bk.n == 0) continue;
-          const int qb = cQ & 1;
-          WAIT2(&mi.q_full[qb], full_par(cQ >> 1), W2_QFULL);           // the query tiles of both CTAs have landed
-          ++cQ;
-          const uint32_t q_u32 = smem_u32(cx.sQ[qb]);
-          for (int j = 0; j < bk.n; ++j) {
-            const int sb = cS % NSB;
-            // S(t) of a warpgroup overwrites its S(t-2): wait until that is in registers.  (P lives elsewhere.)
-            WAIT2(&mi.s_read[sb], free_par(cS / NSB), W2_PVDONE);
-            const int s = cK % NKS;
-            WAIT2(&mi.k_full[s], full_par(cK / NKS), W2_KFULL);
-            tc_fence_after_sync();
-            const uint32_t k_u32 = rk_u32 + s * HALF_BYTES;
-#pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks)
-              mma_ss_pair(cx.tmem + sb * TILE, make_smem_desc_sw128(q_u32 + (ks / 4) * 16384 + (ks % 4) * 32, 16, 1024),
-                          make_smem_desc_sw128(k_u32 + (ks / 4) * 8192 + (ks % 4) * 32, 16, 1024), idesc_qk, ks > 0);
-            mma_commit_pair(&mi.s_full[cS & 1][sb]);   // tile cS belongs to warpgroup cS & 1
-            mma_commit_pair(&mi.k_free[s]);
-            ++cK;
-            ++cS;
+        Desc d;
+        d.kind = KIND_DONE; d.c = d.hkv = d.len = 0;
+        publish(cx, p, d);
+        // Every copy issued must have landed before a CTA may exit.  In a run without a timed-out wait that follows
+        // from the last uses of the rings having been consumed (the teardown below waits for every tensor-core
+        // operation).  After an abort nothing is consumed any more: the leader, whose barriers count the bytes of both
+        // CTAs' copies, waits on them (ignoring the abort flag, bounded); the peer cannot observe the completion of
+        // its own last copies and lets a fixed pause pass that outlasts any copy in flight.
+        if (*cx.abort_flag) {
+          if (leader) {
+            for (uint32_t i = (p.kv > NS ? p.kv - NS : 0); i < p.kv; ++i) mbar_wait_drain(&mi.kv_full[i % NS], full_par(i / NS), cx.abort_flag);
+            for (uint32_t i = (p.q > NQ ? p.q - NQ : 0); i < p.q; ++i) mbar_wait_drain(&mi.q_full[i % NQ], full_par(i / NQ), cx.abort_flag);
           }
-          ++n_done;
-        }
-        if (within == 0) {
-          // ---- score sweep.  Its two [128 keys x 256 rows] buffers overlay all of TMEM: every S/P
-          // buffer is consumed and the accumulator has been read out once acc_free completes.
-          WAIT2(&mi.acc_free, free_par(n_done), W2_ACCFREE);
-          const int n_sweep_tiles = ((len + TILE - 1) / TILE + 1) / 2;
-          for (int u = 0; u < sch.n_pass; ++u) {
-            const int qb = cQ & 1;
-            WAIT2(&mi.q_full[qb], full_par(cQ >> 1), W2_QFULL);
-            ++cQ;
-            const uint32_t q_u32 = smem_u32(cx.sQ[qb]);
-            if (cK & 1) {
-              const int s = cK % NKS;
-              WAIT2(&mi.k_full[s], full_par(cK / NKS), W2_KFULL);
-              mma_commit_pair(&mi.k_free[s]);
-              ++cK;
-            }
-            for (int jj = 0; jj < n_sweep_tiles; ++jj) {
-              const int e = cT & 1;
-              WAIT2(&mi.t_free[e], free_par(cT >> 1), W2_TFREE);
-              const int s = cK % NKS;
-              WAIT2(&mi.k_full[s], full_par(cK / NKS), W2_KFULL);
-              WAIT2(&mi.k_full[s + 1], full_par((cK + 1) / NKS), W2_KFULL);
-              tc_fence_after_sync();
-              const uint32_t k_u32 = rk_u32 + s * HALF_BYTES;
-#pragma unroll
-              for (int ks = 0; ks < D / 16; ++ks)
-                mma_ss_pair(cx.tmem + e * 256, make_smem_desc_sw128(k_u32 + (ks / 4) * 16384 + (ks % 4) * 32, 16, 1024),
-                            make_smem_desc_sw128(q_u32 + (ks / 4) * 16384 + (ks % 4) * 32, 16, 1024), idesc_sw, ks > 0);
-              mma_commit_pair(&mi.t_full[e]);
-              mma_commit_pair(&mi.k_free[s]);
-              mma_commit_pair(&mi.k_free[s + 1]);
-              cK += 2;
-              ++cT;
-            }
-          }
-          // the next item's S buffers overlay the sweep buffers: wait until both were read
-          WAIT2(&mi.t_free[0], free_par((cT + 1) >> 1), W2_TFREE);
-          WAIT2(&mi.t_free[1], free_par(cT >> 1), W2_TFREE);
+          abort_grace_pause(cx.abort_flag);
         }
       }
-      mma_commit_pair(&mi.mma_done);                         // teardown waits for everything this thread issued
-    }
-    __syncwarp();
-  } else if (warp == WARP_PV || warp == WARP_PV + 1) {
-    // ================================================================ issuers of O += P V (leader CTA)
-    // Two threads take alternate tiles: the barrier waits and commits of one (a few hundred cycles
-    // per tile, during which a blocked-issue pipe would run dry) overlap the issue of the other.
-    // A token keeps the accumulation in tile order, so the result does not depend on timing.
-    if (lane == 0 && leader) {
-      const int me = warp - WARP_PV;
-      constexpr uint32_t idesc_pv = make_idesc_bf16_f32(256, D, false, true);
-      const uint32_t rv_u32 = smem_u32(cx.rV);
-      uint32_t cS = 0, n_done = 0, n_turn = 0;
-      for (int item = pair_id; item < n_items && !*cx.abort_flag; item += n_pairs) {
-        int group, within, c, hkv;
-        sch.d_ipg.divmod(item, group, within);
-        sch.d_hkv.divmod(group, c, hkv);
-        const int nsub = n_subitems2(sch, within);
-        const int len = chunk_length(prm, c);
-        for (int sub = 0; sub < nsub; ++sub) {
-          const Blk bk = decode_blk(sch, rank, hkv, within, sub, len);
-          if (bk.n == 0) continue;
-          WAIT2(&mi.acc_free, free_par(n_done), W2_ACCFREE);                   // accumulator of the previous block read out
-          for (int j = 0; j < bk.n; ++j, ++cS) {
-            if ((int)(cS & 1) != me) continue;
-            const int sb = cS % NSB;
-            const int s = cS % NVS;                                            // one V stage per tile
-            WAIT2(&mi.v_full[s], full_par(cS / NVS), W2_VFULL);
-            const uint32_t v_u32 = rv_u32 + s * HALF_BYTES;
-            const uint32_t tP = cx.tmem + TM_P + (cS & 1) * 64;
-            WAIT2(&mi.p_a[me][sb], full_par(cS / NSB), W2_PA);           // keys 0..63 of P
-            WAIT2(&mi.pv_turn[me], me == 0 ? free_par(n_turn) : full_par(n_turn), W2_TURN);   // P V of tile cS-1 issued
-            tc_fence_after_sync();
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-              mma_ts_pair(cx.tmem + TM_O, tP + ks * 8, make_smem_desc_sw128(v_u32 + ks * 2048, 16384, 1024), idesc_pv,
-                          j > 0 || ks > 0);
-            WAIT2(&mi.p_b[me][sb], full_par(cS / NSB), W2_PB);           // keys 64..127
-            tc_fence_after_sync();
-#pragma unroll
-            for (int ks = 4; ks < 8; ++ks)
-              mma_ts_pair(cx.tmem + TM_O, tP + ks * 8, make_smem_desc_sw128(v_u32 + ks * 2048, 16384, 1024), idesc_pv, true);
-            tc_fence_before_sync();
-            mbar_arrive(&mi.pv_turn[me ^ 1]);
-            ++n_turn;
-            mma_commit_pair(&mi.v_free[s]);
-            if (j == bk.n - 1) mma_commit_pair(&mi.o_full);
-          }
-          ++n_done;
-        }
-      }
-      mma_commit_pair(&mi.mma_done);
-    }
-    __syncwarp();
-  } else if (warp < 8) {
-    // ================================================================ softmax: two threads per query row
-    const int r = tid & 127;                                 // row of the block = TMEM lane
-    const int hlf = tid >> 7;                                // which 64 keys of every tile / which 64 head-dim columns
-    const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const float scale_log2 = prm.scale_log2;
-    const uint32_t a_acc_free = map_to_cta(&mi.acc_free, 0);
-    uint32_t cQ = 0, cS = 0, cT = 0, n_done = 0, n_tail = 0;
-    uint32_t n_pub_mine = 0, n_pub_other = 0;                // publications made by this warpgroup / seen from the other
-    // The output tile is stored from the block's Q buffer.  The thread that issued the store does not wait for
-    // it there (its warp would reach the next block's first tile a few thousand cycles after the others, and a
-    // tile is only as fast as its slowest warp): it waits, and hands the buffer back to the producer, after its
-    // first tile of the next block, when the store has long been read.
-    int store_pending = -1;                                  // thread 0: Q buffer of a store that may still be reading it
-    auto finish_store = [&]() {
-      if (tid == 0 && store_pending >= 0) {
-        tma_store_wait_read();
-        mbar_arrive(&mi.q_free[store_pending]);
-        store_pending = -1;
-      }
-    };
-    for (int item = pair_id; item < n_items && !*cx.abort_flag; item += n_pairs) {
-      int group, within, c, hkv;
-      sch.d_ipg.divmod(item, group, within);
-      sch.d_hkv.divmod(group, c, hkv);
-      const int nsub = n_subitems2(sch, within);
-      const int len = chunk_length(prm, c);
-      for (int sub = 0; sub < nsub; ++sub) {
-        const Blk bk = decode_blk(sch, rank, hkv, within, sub, len);
-        if (bk.n == 0) continue;
-        const int token = bk.t * TILE + r;
-        const int qb = cQ & 1;                               // this block's query buffer (its output is staged there)
-        ++cQ;
-        uint8_t* const myQ = cx.sQ[qb];
-        // ---- key tiles: the two warpgroups take alternate tiles (whole rows, one thread per row), so the
-        // load / maximum phase of one tile runs under the exponentials of the other.  The running
-        // maximum is decided tile by tile in order: the owner of tile j waits for the owner of tile
-        // j-1 to publish its per-row reference maximum, decides (lazy rescale) and publishes its own.
-        float m_seen = -INFINITY, l_run = 0.0f;                // l_run: sum over this thread's tiles, relative to m_seen
-        for (int j = 0; j < bk.n; ++j, ++cS) {
-          const int owner = cS & 1;
-          if (owner != hlf) continue;
-          const int sb = cS % NSB;
-          WAIT2S(&mi.s_full[owner][sb], full_par(cS / NSB), W2_SFULL);
+      __syncwarp();
+    } else if (warp == WARP_MMA && leader) {
+      // ================================================================ issuer (leader CTA)
+      // Per key tile and block: O += P V as soon as P is there (in two halves), then S of the block's next tile, which
+      // overwrites P: the pipe runs them in order.  The next unit's first S follows the last tile without a gap.
+      if (elect_one()) {
+        const Sched2 sch = make_sched2(prm);
+        constexpr uint32_t idesc_qk = make_idesc_bf16_f32(256, TILE, false, false), idesc_pv = make_idesc_bf16_f32(256, D, false, true);
+        const int rows_half = sch.hp * sch.wp;
+        const uint32_t idesc_sw = make_idesc_bf16_f32(256, 2 * rows_half, false, false);
+        const uint32_t ring_u32 = smem_u32(cx.ring), q_u32 = smem_u32(cx.sQ);
+        uint32_t nd = 0, kv = 0, nq = 0, np[2] = {0, 0}, no[2] = {0, 0}, nt = 0;
+        uint32_t qa[2];                                          // query operands of the two blocks in work
+        Desc d = next_desc(cx, nd, false);
+        bool primed = false;
+        auto issue_first_qk = [&](int b, uint32_t k_smem) {
+          qa[b] = q_u32 + (nq % NQ) * Q_BYTES;
+          WAIT2S(&mi.q_full[nq % NQ], full_par(nq / NQ), W2_QFULL);
+          ++nq;
           tc_fence_after_sync();
-          const uint32_t tS = cx.tmem + sb * TILE + lane_sel;
-          uint32_t s[4][32];
+          mma_ss_pair_k128<true>(cx.tmem + b * 128, qa[b], k_smem, idesc_qk);
+          mma_commit_pair(&mi.s_full[b]);
+        };
+        while (d.kind != KIND_DONE) {
+          if (d.kind == KIND_FLASH) {
+            const int n0 = d.n[0], n = d.n[1];
+            if (!primed) {
+              const int st = kv % NS;
+              WAIT2S(&mi.kv_full[st], full_par(kv / NS), W2_KVFULL);
+              for (int b = 0; b < 2; ++b) if (d.n[b] > 0) issue_first_qk(b, ring_u32 + st * HALF_BYTES);
+              mma_commit_pair(&mi.kv_free[st]);
+              ++kv;
+            }
+            Desc nx;
+            nx.kind = KIND_DONE; nx.n[0] = nx.n[1] = 0;
+            for (int j = 0; j < n; ++j) {
+              const int sv = kv % NS, sk = (kv + 1) % NS;
+              WAIT2S(&mi.kv_full[sv], full_par(kv / NS), W2_KVFULL);
+              const uint32_t v_u32 = ring_u32 + sv * HALF_BYTES, k_u32 = ring_u32 + sk * HALF_BYTES;
+              bool more = j + 1 < n;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) tmem_ld32(tS + q * 32, s[q]);
-          tmem_wait_ld();
-          tc_fence_before_sync();
+              for (int b = 0; b < 2; ++b) {
+                const uint32_t tS = cx.tmem + b * 128, tO = cx.tmem + TM_O + b * 128;
+                const int nb = b ? n : n0;
+                if (j < nb) {
+                  if (j == 0) { WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE); ++no[b]; }   // accumulator of the previous block read out
+                  WAIT2S(&mi.p_half[b], full_par(np[b]), W2_PHALF);                            // keys 0..63 of P
+                  tc_fence_after_sync();
+                  mma_ts_k64<true>(tO, tS, v_u32, idesc_pv, j > 0);
+                  WAIT2S(&mi.p_full[b], full_par(np[b]), W2_PFULL);
+                  ++np[b];
+                  tc_fence_after_sync();
+                  mma_ts_k64<true>(tO, tS + 32, v_u32 + 8192, idesc_pv, true);
+                  if (j == nb - 1) mma_commit_pair(&mi.o_full[b]);
+                }
+                if (b == 0) {
+                  if (j + 1 == n) { nx = next_desc(cx, nd, false); more = nx.kind == KIND_FLASH; }
+                  if (more) WAIT2S(&mi.kv_full[sk], full_par((kv + 1) / NS), W2_KVFULL);
+                }
+                if (j + 1 < nb) {
+                  tc_fence_after_sync();
+                  mma_ss_pair_k128<true>(tS, qa[b], k_u32, idesc_qk);
+                  mma_commit_pair(&mi.s_full[b]);
+                } else if (j + 1 == n && more && nx.n[b] > 0) {
+                  issue_first_qk(b, k_u32);
+                }
+              }
+              mma_commit_pair(&mi.kv_free[sv]);
+              ++kv;
+              if (more) { mma_commit_pair(&mi.kv_free[sk]); ++kv; }
+            }
+            primed = nx.kind == KIND_FLASH;
+            d = nx;
+          } else {
+            // ---- score sweep, one pass: S^T = K_j Qw^T.  Its two [128 keys x 256 rows] buffers overlay all of TMEM:
+            // every S / P buffer is consumed and the accumulators have been read out once o_free completes.
+            const int n_steps = ((d.len + TILE - 1) / TILE + 1) / 2;
+            for (int b = 0; b < 2; ++b) WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE);
+            const uint32_t qw = q_u32 + (nq % NQ) * Q_BYTES;
+            WAIT2S(&mi.q_full[nq % NQ], full_par(nq / NQ), W2_QFULL);
+            ++nq;
+            for (int jj = 0; jj < n_steps; ++jj, ++nt) {
+              const int e = nt & 1, st = kv % NS;
+              WAIT2S(&mi.t_free[e], free_par(nt >> 1), W2_TFREE);
+              WAIT2S(&mi.kv_full[st], full_par(kv / NS), W2_KVFULL);
+              WAIT2S(&mi.kv_full[st + 1], full_par((kv + 1) / NS), W2_KVFULL);
+              tc_fence_after_sync();
+              mma_ss_pair_k128<false>(cx.tmem + e * 256, ring_u32 + st * HALF_BYTES, qw, idesc_sw);
+              mma_commit_pair(&mi.t_full[e]);
+              mma_commit_pair(&mi.kv_free[st]);
+              mma_commit_pair(&mi.kv_free[st + 1]);
+              kv += 2;
+            }
+            // what follows overwrites the sweep buffers: wait until both were read
+            WAIT2S(&mi.t_free[nt & 1], free_par(nt >> 1), W2_TFREE);
+            WAIT2S(&mi.t_free[(nt + 1) & 1], free_par((nt + 1) >> 1), W2_TFREE);
+            d = next_desc(cx, nd, false);
+          }
+        }
+        mma_commit_pair(&mi.mma_done);                           // teardown waits for everything this thread issued
+      }
+      __syncwarp();
+    }
+  } else if (warp >= WARP_EPI) {
+    // ================================================================ epilogue: normalise, stage bf16 rows in the block's
+    // (now idle) query slot, TMA store
+    setmaxnreg_dec<REGS_EPI>();
+    const Sched2 sch = make_sched2(prm);
+    const int r = tid & 127;
+    const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    uint32_t nd = 0, nq = 0, no[2] = {0, 0};
+    while (true) {
+      const Desc d = next_desc(cx, nd, true);
+      if (d.kind == KIND_DONE) break;
+      if (d.kind == KIND_SWEEP) {
+        if (d.h[0] == 0) {                                       // the window rows' log-sum-exp of this CTA's blocks is in memory
+          __threadfence();
           __syncwarp();
-          if (lane == 0) mbar_arrive_remote(map_to_cta(&mi.s_read[sb], 0));   // Q K^T of this warpgroup's next tile may start
-          const int vis = token - j * TILE + 1;                // visible columns (causal); >= 128: all
-          if (vis < TILE) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (q * 32 + i >= vis) s[q][i] = 0xFF800000u;            // -inf
+          if (lane == 0) {
+            mbar_arrive_cluster(map_to_cta(&mi.lse_rdy, 0));
+            mbar_arrive_cluster(map_to_cta(&mi.lse_rdy, 1));
           }
-          float mq[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            float a = fmax3(__uint_as_float(s[q][0]), __uint_as_float(s[q][1]), __uint_as_float(s[q][2]));
-#pragma unroll
-            for (int i = 3; i < 31; i += 2) a = fmax3(a, __uint_as_float(s[q][i]), __uint_as_float(s[q][i + 1]));
-            mq[q] = fmaxf(a, __uint_as_float(s[q][31]));
-          }
-          const float m_tile = fmaxf(fmaxf(mq[0], mq[1]), fmaxf(mq[2], mq[3])) * scale_log2;   // -inf: nothing visible
-          // reference maximum after tile j-1 (published by the other warpgroup)
-          float m_prev = -INFINITY;
-          if (j > 0) {                                         // the partner's publication of tile j-1
-            WAIT2S(&mi.m_pub[hlf ^ 1][warp & 3], full_par(n_pub_other), W2_MPUB);
-            ++n_pub_other;
-            m_prev = mi.mref[(j - 1) & 1][r];
-          }
-          const bool first_tile = (j == 0);
-          const bool raise = first_tile || (m_tile > m_prev + LAZY_RESCALE);
-          const float m_new = raise ? fmaxf(m_prev, m_tile) : m_prev;
-          mi.mref[j & 1][r] = m_new;
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&mi.m_pub[hlf][warp & 3]);   // the warp with the same rows may decide tile j+1
-          ++n_pub_mine;
-          if (m_new != m_seen) {                               // bring this thread's partial sum to the new reference
-            l_run *= (m_seen == -INFINITY) ? 0.0f : fast_exp2(m_seen - m_new);
-            m_seen = m_new;
-          }
-          if (!first_tile && __any_sync(0xFFFFFFFFu, raise)) {
-            // rare: rescale the accumulator rows of this warp.  P V of tile j-1 may still be running
-            // (it is not ordered before this tile's S): wait for it; P V of tile j cannot start before
-            // this thread publishes P.
-            const float alpha = (m_prev == -INFINITY) ? 0.0f : fast_exp2(m_prev - m_new);
-            const uint32_t prev = cS - 1;
-            WAIT2S(&mi.v_free[prev % NVS], full_par(prev / NVS), W2_PVDONE);   // committed after P V of tile `prev`
-            tc_fence_after_sync();
-            const uint32_t tO = cx.tmem + TM_O + lane_sel;
+        }
+        ++nq;
+        continue;
+      }
 #pragma unroll 1
-            for (int q = 0; q < D / 8; ++q) {
-              uint32_t o[8];
-              tmem_ld8(tO + q * 8, o);
-              tmem_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-              tmem_st8(tO + q * 8, o);
-            }
-          }
-          if (cS >= 2) {
-            // the P buffer of this warpgroup is free once P V of its previous tile has run; this wait also keeps
-            // the softmax at most one own tile ahead of the P V issuer, whose barriers have one phase bit
-            const uint32_t prev2 = cS - 2;
-            WAIT2S(&mi.v_free[prev2 % NVS], full_par(prev2 / NVS), W2_PVDONE);
-            tc_fence_after_sync();
-          }
-          const float neg_m = (m_new == -INFINITY) ? 0.0f : -m_new;
-          const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2), negm2 = pack_f32x2(neg_m, neg_m);
-          uint64_t sum2[2] = {0ull, 0ull};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint32_t packed[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(s[q][2 * i]), __uint_as_float(s[q][2 * i + 1])), scale2, negm2);
-              float x0, x1, p0, p1;
-              unpack_f32x2(x2, x0, x1);
-              p0 = fast_exp2(x0);                                // MUFU pipe
-              p1 = fast_exp2(x1);
-              sum2[i & 1] = add_f32x2(sum2[i & 1], pack_f32x2(p0, p1));
-              packed[i] = pack_bf16x2(p0, p1);
-            }
-            tmem_st16(cx.tmem + TM_P + hlf * 64 + q * 16 + lane_sel, packed);   // P: 64 bf16 columns
-            if (q == 1) {                                      // keys 0..63 are final: P V may start on them
-              tmem_wait_st();
-              tc_fence_before_sync();
-              __syncwarp();
-              if (lane == 0) mbar_arrive_remote(map_to_cta(&mi.p_a[hlf][sb], 0));
-            }
-          }
-          float a0, a1, a2, a3;
-          unpack_f32x2(sum2[0], a0, a1);
-          unpack_f32x2(sum2[1], a2, a3);
-          l_run += (a0 + a1) + (a2 + a3);
-          tmem_wait_st();
-          tc_fence_before_sync();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_remote(map_to_cta(&mi.p_b[hlf][sb], 0));
-          finish_store();
-        }
-        // the warpgroup that did not own the last tile consumes its owner's publication; then both
-        // bring their partial sums to the final reference maximum
-        {
-          const int last_owner = (cS - 1) & 1;
-          if (hlf != last_owner) {
-            WAIT2S(&mi.m_pub[hlf ^ 1][warp & 3], full_par(n_pub_other), W2_MPUB);
-            ++n_pub_other;
-          }
-          const float m_fin = mi.mref[(bk.n - 1) & 1][r];
-          if (m_fin != m_seen) {
-            l_run *= (m_seen == -INFINITY) ? 0.0f : fast_exp2(m_seen - m_fin);
-            m_seen = m_fin;
-          }
-        }
-        const float m_used = m_seen;
-        finish_store();
-        // ---- epilogue: combine the two half-row sums, normalise, stage bf16 rows in this block's
-        // (now idle) Q buffer, TMA store
-        WAIT2S(&mi.o_full, full_par(n_done), W2_OFULL);
-        ++n_done;
+      for (int b = 0; b < 2; ++b) {
+        if ((b ? d.n[1] : d.n[0]) == 0) continue;
+        const int h = b ? d.h[1] : d.h[0], t = b ? d.t[1] : d.t[0];
+        const uint32_t ph = b ? no[1]++ : no[0]++;
+        uint8_t* const myQ = cx.sQ + (nq % NQ) * Q_BYTES;
+        uint64_t* const q_free = &mi.q_free[nq % NQ];
+        ++nq;
+        const int token = t * TILE + r;
+        WAIT2(&mi.lm_full[b], full_par(ph), W2_LM);
+        const float m_used = mi.lm[b][0][r], l_run = mi.lm[b][1][r];
+        warp_arrive(&mi.lm_free[b]);
+        WAIT2S(&mi.o_full[b], full_par(ph), W2_OFULL);
         tc_fence_after_sync();
-        mi.xl[hlf][r] = l_run;
-        named_barrier_sync(1, 256);
-        const float l_tot = mi.xl[0][r] + mi.xl[1][r];
-        const float inv_l = token < len ? 1.0f / l_tot : 0.0f;   // rows behind the end of the chunk are written as zeros
-        {
-          const uint32_t tO = cx.tmem + TM_O + hlf * 64 + lane_sel;
+        const bool in_chunk = token >= 0 && token < d.len;       // rows behind the end of the chunk are written as zeros
+        const float inv_l = in_chunk ? 1.0f / l_run : 0.0f;
+        const uint32_t tO = cx.tmem + TM_O + b * 128 + lane_sel;
+#pragma unroll 1
+        for (int q = 0; q < D / 32; ++q) {
+          uint32_t o[32];
+          tmem_ld32(tO + q * 32, o);
+          tmem_wait_ld();
+          loaded(o);
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            uint32_t o[32];
-            tmem_ld32(tO + q * 32, o);
-            tmem_wait_ld();
+          for (int g4 = 0; g4 < 4; ++g4) {
+            uint32_t pk[4];
 #pragma unroll
-            for (int g4 = 0; g4 < 4; ++g4) {
-              uint32_t pk[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e)
-                pk[e] = token < len ? pack_bf16x2(__uint_as_float(o[g4 * 8 + 2 * e]) * inv_l, __uint_as_float(o[g4 * 8 + 2 * e + 1]) * inv_l) : 0u;
-              *reinterpret_cast<uint4*>(myQ + hlf * 16384 + sw128_offset(r, q * 4 + g4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-            }
+            for (int e = 0; e < 4; ++e)
+              pk[e] = in_chunk ? pack_bf16x2(__uint_as_float(o[g4 * 8 + 2 * e]) * inv_l, __uint_as_float(o[g4 * 8 + 2 * e + 1]) * inv_l) : 0u;
+            const int col = q * 32 + g4 * 8;
+            *reinterpret_cast<uint4*>(myQ + (col / 64) * 16384 + sw128_offset(r, (col % 64) / 8)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
         }
-        tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_remote(a_acc_free);
-        if (hlf == 0 && token < len) {
-          const float lse2 = m_used + log2f(l_tot);
-          if (prm.lse) prm.lse[((size_t)c * prm.Hq + bk.h) * prm.L + token] = lse2 * 0.6931471805599453f;
-          const int wi = token - (len - prm.w);
+        warp_arrive_leader(map_to_cta(&mi.o_free[b], 0));
+        if (in_chunk) {
+          const float lse2 = m_used + log2f(l_run);
+          const size_t row = (size_t)d.c * prm.Hq + h;
+          if (prm.lse) prm.lse[row * prm.L + token] = lse2 * 0.6931471805599453f;
+          const int wi = token - (d.len - prm.w);
           if (wi >= 0) {
-            prm.win_lse[((size_t)c * prm.Hq + bk.h) * prm.w + wi] = lse2 * 0.6931471805599453f;
-            if (within == 0) {                               // the sweep of both CTAs needs it
-              float* slot = &mi.lse2[(bk.h - hkv * sch.G) * prm.w + wi];
-              *slot = lse2;
-              st_shared_cluster_f32(map_to_cta(slot, rank ^ 1u), lse2);
-            }
+            prm.win_lse[row * prm.w + wi] = lse2 * 0.6931471805599453f;
+            float* const slot = prm.lse2 + row * sch.wp + (sch.wp - prm.w);
+            slot[wi] = lse2;
+            if (wi == 0)                                         // operand rows that are not window rows: probability 0
+              for (int i = 1; i <= sch.wp - prm.w; ++i) slot[-i] = INFINITY;
           }
         }
         fence_proxy_async_smem();
-        named_barrier_sync(1, 256);
-        if (tid == 0) {
-          if (bk.t * TILE < prm.L) {
-            for (int a = 0; a < 2; ++a) tma_store_4d(&tm_o, myQ + a * 16384, a * 64, bk.h, bk.t * TILE, c);
+        named_barrier_sync(1, 128);
+        if (r == 0) {
+          if (t >= 0 && t * TILE < prm.L) {
+            for (int a = 0; a < 2; ++a) tma_store_4d(&tm_o, myQ + a * 16384, a * 64, h, t * TILE, d.c);
             tma_store_commit();
+            tma_store_wait_read();
           }
-          store_pending = qb;                                // released by finish_store() once the store has read it
-        }
-      }
-      if (within == 0) {
-        finish_store();                                      // a later sweep pass loads window queries into that buffer
-        // ---- score sweep.  First make the window rows' log-sum-exp of all heads visible in both CTAs.
-        __syncwarp();
-        if (lane == 0) {
-          mbar_arrive_cluster(map_to_cta(&mi.lse_ready, 0));
-          mbar_arrive_cluster(map_to_cta(&mi.lse_ready, 1));
-        }
-        mbar_wait_cluster(&mi.lse_ready, full_par(n_tail), cx.abort_flag, cx.status, W2_LSE);
-        ++n_tail;
-        const int n_sweep_tiles = ((len + TILE - 1) / TILE + 1) / 2;
-        const int w0 = len - prm.w;                          // first window token of this chunk
-        for (int u = 0; u < sch.n_pass; ++u) {
-          const int qb = cQ & 1;                             // window queries of this pass (loaded and consumed by other warps)
-          ++cQ;
-          // this thread sums the columns of the heads that CTA `hlf` loaded: local head i = ncol / w
-          const int g_base = u * 2 * sch.hp + hlf * sch.hp;
-          for (int jj = 0; jj < n_sweep_tiles; ++jj) {
-            const int e = cT & 1;
-            WAIT2S(&mi.t_full[e], full_par(cT >> 1), W2_TFULL);
-            tc_fence_after_sync();
-            const int key = (2 * jj + (int)rank) * TILE + r;
-            const bool need_mask = (2 * jj + (int)rank) * TILE + TILE - 1 > w0;
-            const uint32_t tT = cx.tmem + e * 256 + hlf * rows_half + lane_sel;
-            float part = 0.0f;
-            for (int ih = 0; ih < sch.hp; ++ih) {            // heads of this column half; a head has wp columns, the last w are window rows
-              const int g = g_base + ih;
-              if (g >= sch.G) break;                         // filler head
-              const float* lse_head = mi.lse2 + g * prm.w;
-              for (int col = 0; col < sch.wp; col += 8) {
-                uint32_t sv[8];
-                tmem_ld8(tT + ih * sch.wp + col, sv);
-                tmem_wait_ld();
-                const int wi0 = col - (sch.wp - prm.w);      // window row of the first of these 8 columns (negative: not a window row)
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                  const int wi = wi0 + i;
-                  float pv = fast_exp2(fmaf(__uint_as_float(sv[i]), scale_log2, -lse_head[wi < 0 ? 0 : wi]));
-                  if (wi < 0 || (need_mask && key > w0 + wi)) pv = 0.0f;
-                  part += pv;
-                }
-              }
-            }
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_remote(map_to_cta(&mi.t_free[e], 0));
-            mi.xs[e][hlf][r] = part;
-            named_barrier_sync(1, 256);
-            if (hlf == 0 && key < len) {
-              float* dst = prm.win_score + ((size_t)c * prm.Hkv + hkv) * prm.L + key;
-              const float total = part + mi.xs[e][1][r];
-              *dst = (u == 0) ? total : (*dst + total);
-            }
-            ++cT;
-          }
-          named_barrier_sync(1, 256);                        // everyone is past its last use of sQ[qb]
-          if (tid == 0) mbar_arrive(&mi.q_free[qb]);
+          mbar_arrive(q_free);
         }
       }
     }
-    finish_store();
-    if (tid == 0) tma_store_wait_all();
+    if (r == 0) tma_store_wait_all();
+  } else {
+    // ================================================================ softmax
+    setmaxnreg_inc<REGS_SOFTMAX>();
+    const Sched2 sch = make_sched2(prm);
+    const int b = warp >> 2;
+    const int r = tid & 127;
+    const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    const uint32_t tS = cx.tmem + b * 128 + lane_sel, tO = cx.tmem + TM_O + b * 128 + lane_sel;
+    const float scale_log2 = prm.scale_log2;
+    struct Hooks {
+      uint32_t p_half, p_full;                                   // barriers of the leader CTA
+      __device__ __forceinline__ void on_read() const {}
+      __device__ __forceinline__ void before_rescale() const {}  // S of this tile was issued after P V of the tile before
+      __device__ __forceinline__ void before_p() const {}        // P overwrites S, which is in registers
+      __device__ __forceinline__ void on_half() const { warp_arrive_leader(p_half); }
+      __device__ __forceinline__ void on_full() const { warp_arrive_leader(p_full); }
+    } hk = {map_to_cta(&mi.p_half[b], 0), map_to_cta(&mi.p_full[b], 0)};
+    uint32_t nd = 0, n_s = 0, n_blk = 0, nq = 0, nt = 0, n_lse = 0;
+    while (true) {
+      const Desc d = next_desc(cx, nd, true);
+      if (d.kind == KIND_DONE) break;
+      if (d.kind == KIND_FLASH) {
+        nq += d.n[0] > 0 ? 2 : 1;
+        const int n = b ? d.n[1] : d.n[0], t = b ? d.t[1] : d.t[0];
+        if (n == 0) continue;
+        RowState st = {-INFINITY, 0.0f};
+#pragma unroll 1
+        for (int j = 0; j < n; ++j) {
+          WAIT2S(&mi.s_full[b], full_par(n_s), W2_SFULL);
+          ++n_s;
+          tc_fence_after_sync();
+          if (j > 0 && j < t) softmax_tile<D, false>(tS, tS, tO, TILE, false, scale_log2, st, hk);
+          else softmax_tile<D, true>(tS, tS, tO, (t - j) * TILE + r + 1, j == 0, scale_log2, st, hk);   // causal: keys <= token
+        }
+        WAIT2S(&mi.lm_free[b], free_par(n_blk), W2_LMFREE);
+        ++n_blk;
+        mi.lm[b][0][r] = st.m;
+        mi.lm[b][1][r] = st.l;
+        warp_arrive(&mi.lm_full[b]);
+      } else {
+        // ---- score sweep: this thread owns a key; its warpgroup sums the columns of the heads that CTA b loaded
+        const int u = d.h[0];
+        if (u == 0) { mbar_wait_cluster(&mi.lse_rdy, full_par(n_lse), cx.abort_flag, cx.status, W2_LSE); ++n_lse; }
+        const int rows_half = sch.hp * sch.wp;
+        const int g0 = u * 2 * sch.hp + b * sch.hp;
+        const int heads = sch.G - g0 < sch.hp ? (sch.G > g0 ? sch.G - g0 : 0) : sch.hp;
+        const int cols = heads * sch.wp;
+        const float* const lse_rows = prm.lse2 + ((size_t)d.c * prm.Hq + d.hkv * sch.G + g0) * sch.wp;
+        const int n_steps = ((d.len + TILE - 1) / TILE + 1) / 2;
+        const int w0 = d.len - prm.w, pad = sch.wp - prm.w;      // first window token of this chunk
+        float* const xch = &mi.lm[0][0][0];                      // [buffer][key]
+        const uint32_t t_free0 = map_to_cta(&mi.t_free[0], 0), t_free1 = map_to_cta(&mi.t_free[1], 0);
+        for (int jj = 0; jj < n_steps; ++jj, ++nt) {
+          const int e = nt & 1;
+          WAIT2S(&mi.t_full[e], full_par(nt >> 1), W2_TFULL);
+          tc_fence_after_sync();
+          const int key0 = (2 * jj + (int)rank) * TILE, key = key0 + r;
+          const uint32_t tT = cx.tmem + e * 256 + b * rows_half + lane_sel;
+          float part = 0.0f;
+          int col = 0;
+          if (key0 + TILE - 1 <= w0) {                           // every window row sees every key of the tile
+            const uint64_t scale2 = dup2(scale_log2);
+            uint64_t sum2 = 0ull;
+#pragma unroll 1
+            for (; col + 32 <= cols; col += 32) {
+              uint32_t sv[32];
+              tmem_ld32(tT + col, sv);
+              float4 ls[8];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) ls[i] = __ldcg(reinterpret_cast<const float4*>(lse_rows + col) + i);
+              tmem_wait_ld();
+              loaded(sv);
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                const float4 l4 = ls[i / 2];
+                const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), scale2,
+                                              (i & 1) ? pack_f32x2(-l4.z, -l4.w) : pack_f32x2(-l4.x, -l4.y));
+                float x0, x1;
+                unpack_f32x2(x2, x0, x1);
+                sum2 = add_f32x2(sum2, pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
+              }
+            }
+            float a0, a1;
+            unpack_f32x2(sum2, a0, a1);
+            part = a0 + a1;
+          }
+#pragma unroll 1
+          for (; col < cols; col += 8) {                         // the rest, and tiles that reach into the window
+            uint32_t sv[8];
+            tmem_ld8(tT + col, sv);
+            const float4 la = __ldcg(reinterpret_cast<const float4*>(lse_rows + col)), lb = __ldcg(reinterpret_cast<const float4*>(lse_rows + col + 4));
+            const float ls[8] = {la.x, la.y, la.z, la.w, lb.x, lb.y, lb.z, lb.w};
+            const int wi0 = col % sch.wp - pad;                  // window row of the first of these columns (negative: none)
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const float pv = fast_exp2(fmaf(__uint_as_float(sv[i]), scale_log2, -ls[i]));
+              part += key <= w0 + wi0 + i ? pv : 0.0f;
+            }
+          }
+          warp_arrive_leader(e ? t_free1 : t_free0);
+          if (b == 1) xch[e * TILE + r] = part;
+          named_barrier_sync(3, 256);
+          if (b == 0 && key < d.len) {
+            float* dst = prm.win_score + ((size_t)d.c * prm.Hkv + d.hkv) * prm.L + key;
+            const float total = part + xch[e * TILE + r];
+            *dst = (u == 0) ? total : (*dst + total);
+          }
+        }
+        named_barrier_sync(3, 256);                              // everyone is past the exchange buffer
+        if (tid == 0) mbar_arrive(&mi.q_free[nq % NQ]);          // the window queries were read by MMAs that have completed
+        ++nq;
+      }
+    }
   }
 
   // ---- teardown: no CTA may exit while its peer can still signal it or read its shared memory
   tc_fence_before_sync();
   __syncthreads();
   cluster_sync_all();
-  if (warp == WARP_QK) {
-    // no tensor-core operation may still be running when its accumulators are freed: every issuer ended with a
-    // commit to mma_done (three arrivals in both CTAs).  Immediate in a clean run; after an abort this is what
+  if (warp == WARP_MMA) {
+    // no tensor-core operation may still be running when its accumulators are freed: the issuer ended with a
+    // commit to mma_done (an arrival in both CTAs).  Immediate in a clean run; after an abort this is what
     // makes the exit safe.  The wait ignores the abort flag and is bounded.
     mbar_wait_drain(&mi.mma_done, 0, cx.abort_flag);
     tc_fence_after_sync();
@@ -780,14 +704,13 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 //                                   host launcher
 // ====================================================================================
 // maps: 0 q (box 64 x 128 tokens), 1 rotated keys (64 x 128), 2 v (64 x 128), 3 o (store), 4 q with a
-// w-token box, 5 rotated keys with a 64-token box.  The grid is a whole number of CTA pairs.
+// wp-token box, 5 rotated keys with a 64-token box.  The grid is a whole number of CTA pairs.
 cudaError_t launch_prefill_pair(const CUtensorMap* maps, const PrefillParams& prm, int sm_count, cudaStream_t st) {
   // the opt-in to large dynamic shared memory is a per-device attribute of the function: set it on every call
   // (a host-side call of a few hundred nanoseconds) rather than remember which devices have it
   if (cudaError_t e = cudaFuncSetAttribute(prefill_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES); e != cudaSuccess) return e;
   const int grid = (sm_count / 2) * 2;
   if (grid < 2) return cudaErrorInvalidConfiguration;
-  if ((prm.Hq / prm.Hkv) % 2 != 0) return cudaErrorInvalidValue;   // the pair kernel takes even group sizes
   note_launch();
   prefill_pair_kernel<<<grid, NT2, SMEM2_BYTES, st>>>(maps[0], maps[5], maps[1], maps[2], maps[3], maps[4], prm);
   return cudaGetLastError();

@@ -413,4 +413,65 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
                : "memory");
 }
 
+// One thread of a converged warp (elect.sync).  Unlike `lane == 0` the compiler knows that the branch is taken by a
+// single thread, and keeps the operands of tcgen05 instructions in uniform registers: issuing the eight k-steps of a
+// 128 x 128 x 128 product takes 121 to 200 cycles in such a branch and 410 to 470 under `lane == 0`.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
+  return pred != 0;
+}
+template <int N> __device__ __forceinline__ void setmaxnreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void setmaxnreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+
+// ------------------------------------------------------------------ whole products as one asm block
+// The k-steps of a product are one asm statement whose descriptors differ by immediates in the low word (121 cycles to
+// issue the eight steps, against 200 for eight statements under elect_one), so that the issuing thread stays ahead of
+// the pipe, which needs 512 cycles for them.  Operand tiles: rows of 64 elements, 128-byte swizzle; a k-step is 16
+// elements = 32 bytes, the next 64 elements of a row are an atom of 8 KB (64 rows) or 16 KB (128 rows) further.
+constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);        // SBO 1024, sm_100 descriptor, 128-byte swizzle
+__device__ __forceinline__ uint32_t desc_lo(uint32_t smem, uint32_t lbo) { return ((smem & 0x3FFFFu) >> 4) | ((lbo >> 4) << 16); }
+#define PC_MMA_SS0(G) "setp.ne.b32 p, 0, 0;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\ttcgen05.mma.cta_group::" #G ".kind::f16 [%0], a, b, %4, p;\n\tsetp.eq.b32 p, 0, 0;\n\t"
+#define PC_MMA_SS(G, oa, ob) "add.s32 x, %1, " #oa ";\n\tadd.s32 y, %2, " #ob ";\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %3};\n\ttcgen05.mma.cta_group::" #G ".kind::f16 [%0], a, b, %4, p;\n\t"
+#define PC_MMA_TS(G, t, o) "add.s32 x, %1, " #t ";\n\tadd.s32 y, %2, " #o ";\n\tmov.b64 b, {y, %3};\n\ttcgen05.mma.cta_group::" #G ".kind::f16 [%0], [x], b, %4, p;\n\t"
+#define PC_SS_REGS "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\t"
+// S = A B^T over 64 elements (one atom), single CTA
+__device__ __forceinline__ void mma_ss_k64(uint32_t d_tmem, uint32_t a_smem, uint32_t b_smem, uint32_t idesc) {
+  asm volatile(PC_SS_REGS PC_MMA_SS0(1) PC_MMA_SS(1, 2, 2) PC_MMA_SS(1, 4, 4) PC_MMA_SS(1, 6, 6) "}\n"
+               ::"r"(d_tmem), "r"(desc_lo(a_smem, 16)), "r"(desc_lo(b_smem, 16)), "r"(DESC_HI), "r"(idesc) : "memory");
+}
+// S = A B^T over 128 elements on a CTA pair; A 128 rows per CTA, B 64 rows (B64) or up to 128 rows per CTA
+template <bool B64>
+__device__ __forceinline__ void mma_ss_pair_k128(uint32_t d_tmem, uint32_t a_smem, uint32_t b_smem, uint32_t idesc) {
+  if constexpr (B64)
+    asm volatile(PC_SS_REGS PC_MMA_SS0(2) PC_MMA_SS(2, 2, 2) PC_MMA_SS(2, 4, 4) PC_MMA_SS(2, 6, 6)
+                 PC_MMA_SS(2, 1024, 512) PC_MMA_SS(2, 1026, 514) PC_MMA_SS(2, 1028, 516) PC_MMA_SS(2, 1030, 518) "}\n"
+                 ::"r"(d_tmem), "r"(desc_lo(a_smem, 16)), "r"(desc_lo(b_smem, 16)), "r"(DESC_HI), "r"(idesc) : "memory");
+  else
+    asm volatile(PC_SS_REGS PC_MMA_SS0(2) PC_MMA_SS(2, 2, 2) PC_MMA_SS(2, 4, 4) PC_MMA_SS(2, 6, 6)
+                 PC_MMA_SS(2, 1024, 1024) PC_MMA_SS(2, 1026, 1026) PC_MMA_SS(2, 1028, 1028) PC_MMA_SS(2, 1030, 1030) "}\n"
+                 ::"r"(d_tmem), "r"(desc_lo(a_smem, 16)), "r"(desc_lo(b_smem, 16)), "r"(DESC_HI), "r"(idesc) : "memory");
+}
+// four k-steps (64 keys) of O (+)= P V, P in TMEM; p_tmem and v_smem point at the first of them
+template <bool PAIR>
+__device__ __forceinline__ void mma_ts_k64(uint32_t o_tmem, uint32_t p_tmem, uint32_t v_smem, uint32_t idesc, bool accumulate) {
+  if constexpr (PAIR)
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t.reg .b32 x, y;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 b, {%2, %3};\n\t"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], b, %4, p;\n\tsetp.eq.b32 p, 0, 0;\n\t"
+                 PC_MMA_TS(2, 8, 128) PC_MMA_TS(2, 16, 256) PC_MMA_TS(2, 24, 384) "}\n"
+                 ::"r"(o_tmem), "r"(p_tmem), "r"(desc_lo(v_smem, 16384)), "r"(DESC_HI), "r"(idesc), "r"(static_cast<uint32_t>(accumulate)) : "memory");
+  else
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t.reg .b32 x, y;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 b, {%2, %3};\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\tsetp.eq.b32 p, 0, 0;\n\t"
+                 PC_MMA_TS(1, 8, 128) PC_MMA_TS(1, 16, 256) PC_MMA_TS(1, 24, 384) "}\n"
+                 ::"r"(o_tmem), "r"(p_tmem), "r"(desc_lo(v_smem, 16384)), "r"(DESC_HI), "r"(idesc), "r"(static_cast<uint32_t>(accumulate)) : "memory");
+}
+
+// 32-bit store into the shared memory of a CTA of the cluster whose completion is counted (4 bytes) on an mbarrier there
+__device__ __forceinline__ void st_async_u32(uint32_t cluster_addr, uint32_t v, uint32_t bar_cluster_addr) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(cluster_addr), "r"(v),
+               "r"(bar_cluster_addr)
+               : "memory");
+}
+
 }  // namespace pc

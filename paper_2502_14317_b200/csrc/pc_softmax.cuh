@@ -1,0 +1,174 @@
+// Softmax of one key tile, shared by the chunk-local attention kernels (thread = query row = TMEM lane).
+#pragma once
+#include "pc_sm100.cuh"
+
+namespace pc {
+
+constexpr float LAZY_RESCALE_LOG2 = 8.0f;      // the reference maximum is raised only when it grows by more than 2^8
+// Every POLY_EVERY-th pair of exponentials is evaluated on the FMA pipe.  A tile needs 128 exponentials a row, 1024
+// cycles of a scheduler's MUFU pipe for its warp; measured on two warps a scheduler (cycles a tile): none 2305, every
+// eighth 2170, fifth 2038, fourth 1972, third 2186 (then the issue slots are what is short).
+constexpr int POLY_EVERY = 4;
+
+__device__ __forceinline__ float fmax_nan(float a, float b) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t dup2(float v) { return pack_f32x2(v, v); }
+
+// 2^x of a pair on the FMA pipe: x = n + f with n the nearest integer (magic-number addition); a polynomial of degree 5
+// in f on [-1/2, 1/2] with p(0) = 1, fitted for the least relative error (1.7e-7 evaluated in fp32, as good as the
+// MUFU's 2^-22); n added to the exponent field.  Arguments below -127 give 0, NaN stays NaN.
+__device__ __forceinline__ void exp2_pair_fma(uint64_t x2, float& p0, float& p1) {
+  float x0, x1;
+  unpack_f32x2(x2, x0, x1);
+  x2 = pack_f32x2(fmax_nan(x0, -127.0f), fmax_nan(x1, -127.0f));          // 2^-127 comes out as exactly 0
+  const uint64_t r2 = add_f32x2(x2, dup2(12582912.0f));
+  const uint64_t n2 = add_f32x2(r2, dup2(-12582912.0f));
+  const uint64_t f2 = fma_f32x2(n2, dup2(-1.0f), x2);
+  uint64_t p = fma_f32x2(f2, dup2(0.001326472731307149f), dup2(0.009671512991189957f));
+  p = fma_f32x2(f2, p, dup2(0.05550733581185341f));
+  p = fma_f32x2(f2, p, dup2(0.24022242426872253f));
+  p = fma_f32x2(f2, p, dup2(0.6931470036506653f));
+  p = fma_f32x2(f2, p, dup2(1.0f));
+  float r0, r1;
+  unpack_f32x2(r2, r0, r1);
+  unpack_f32x2(p, p0, p1);
+  p0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(r0) << 23));
+  p1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(r1) << 23));
+}
+
+// 32 logits -> 16 packed bf16 pairs; partial sums in sum2
+__device__ __forceinline__ void exps32(const uint32_t (&s)[32], uint64_t scale2, uint64_t negm2, uint64_t (&sum2)[2],
+                                       uint32_t (&packed)[16]) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), scale2, negm2);
+    float p0, p1;
+    if (i % POLY_EVERY == POLY_EVERY - 1) {
+      exp2_pair_fma(x2, p0, p1);
+    } else {
+      float x0, x1;
+      unpack_f32x2(x2, x0, x1);
+      p0 = fast_exp2(x0);
+      p1 = fast_exp2(x1);
+    }
+    sum2[i & 1] = add_f32x2(sum2[i & 1], pack_f32x2(p0, p1));
+    packed[i] = pack_bf16x2(p0, p1);
+  }
+}
+__device__ __forceinline__ float max32(const uint32_t (&s)[32]) {
+  float a = fmax3(__uint_as_float(s[0]), __uint_as_float(s[1]), __uint_as_float(s[2]));
+#pragma unroll
+  for (int j = 3; j < 31; j += 2) a = fmax3(a, __uint_as_float(s[j]), __uint_as_float(s[j + 1]));
+  return fmaxf(a, __uint_as_float(s[31]));
+}
+// masked columns (>= vis) of a 32-column piece whose first column is `col0`
+__device__ __forceinline__ void mask32(uint32_t (&s)[32], int col0, int vis) {
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (col0 + j >= vis) s[j] = 0xFF800000u;                       // -inf
+}
+// after tmem_wait_ld: ties the loaded registers to the wait, so that no use of them moves above it
+__device__ __forceinline__ void loaded(uint32_t (&r)[32]) {
+#pragma unroll
+  for (int i = 0; i < 32; i += 8)
+    asm volatile("" : "+r"(r[i]), "+r"(r[i + 1]), "+r"(r[i + 2]), "+r"(r[i + 3]), "+r"(r[i + 4]), "+r"(r[i + 5]), "+r"(r[i + 6]), "+r"(r[i + 7]));
+}
+
+struct RowState { float m, l; };               // reference maximum (log2 units) of a row and its sum relative to that
+
+// multiplies the accumulator rows of this warp by alpha
+template <int D>
+__device__ __forceinline__ void rescale_rows(uint32_t o_taddr, float alpha) {
+#pragma unroll 1
+  for (int q = 0; q < D / 8; ++q) {
+    uint32_t o[8];
+    tmem_ld8(o_taddr + q * 8, o);
+    tmem_wait_ld();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
+    tmem_st8(o_taddr + q * 8, o);
+  }
+}
+
+// One 128-key tile.  The exponentials of the first 64 keys are taken against the reference maximum of the tiles BEFORE
+// this one, while the maximum of this tile is found on the ALU pipe beside them; they are stored only when that maximum
+// is known not to exceed the reference by more than 2^8 in any row of the warp (otherwise the reference is raised, the
+// accumulator rescaled and the first half repeated).  So the row maximum is off the path from logits to exponentials.
+// GEN: tiles with masked columns (columns >= vis; vis <= 0: all) and the first tile of a block; the tiles between
+// run straight-line code (the branches around the masks cost 300 of 1240 cycles).
+// Hooks: on_read() - all logits are in registers; before_rescale() - called before the accumulator is touched;
+// before_p() - called before probabilities are stored at p_taddr (64 columns); on_half(), on_full() - keys 0..63 / all
+// keys of P are in TMEM.
+template <int D, bool GEN, class Hooks>
+__device__ __forceinline__ void softmax_tile(uint32_t s_taddr, uint32_t p_taddr, uint32_t o_taddr, int vis, bool first_tile,
+                                             float scale_log2, RowState& st, const Hooks& hk) {
+  const uint64_t scale2 = dup2(scale_log2);
+  uint64_t sum2[2] = {0ull, 0ull};
+  uint32_t pk[2][16], c2[32], c3[32];
+  float mx;
+  {
+    uint32_t c0[32], c1[32];
+    tmem_ld32(s_taddr, c0);
+    tmem_ld32(s_taddr + 32, c1);
+    tmem_wait_ld();
+    loaded(c0); loaded(c1);
+    tmem_ld32(s_taddr + 64, c2);
+    tmem_ld32(s_taddr + 96, c3);
+    if (GEN) { mask32(c0, 0, vis); mask32(c1, 32, vis); }
+    const uint64_t negm2 = dup2(st.m == -INFINITY ? 0.0f : -st.m);  // nothing visible so far: exp2(-inf) = 0
+    mx = fmaxf(max32(c0), max32(c1));
+    if (!GEN || !first_tile) {
+      exps32(c0, scale2, negm2, sum2, pk[0]);
+      exps32(c1, scale2, negm2, sum2, pk[1]);
+    }
+  }
+  tmem_wait_ld();
+  loaded(c2); loaded(c3);
+  if (GEN) { mask32(c2, 64, vis); mask32(c3, 96, vis); }
+  mx = fmaxf(mx, fmaxf(max32(c2), max32(c3))) * scale_log2;
+  const bool raise = mx > st.m + LAZY_RESCALE_LOG2 || (GEN && first_tile);
+  if (__any_sync(0xFFFFFFFFu, raise)) {                            // rare; warp-uniform: each warp owns its 32 lanes of O
+    float alpha = 1.0f;
+    if (raise) {
+      const float m_new = fmaxf(st.m, mx);
+      alpha = (st.m == -INFINITY) ? 0.0f : fast_exp2(st.m - m_new);
+      st.m = m_new;
+      st.l *= alpha;
+    }
+    if (!GEN || !first_tile) {
+      hk.before_rescale();
+      rescale_rows<D>(o_taddr, alpha);
+    }
+    uint32_t c0[32], c1[32];
+    tmem_ld32(s_taddr, c0);
+    tmem_ld32(s_taddr + 32, c1);
+    tmem_wait_ld();
+    loaded(c0); loaded(c1);
+    if (GEN) { mask32(c0, 0, vis); mask32(c1, 32, vis); }
+    const uint64_t negm2 = dup2(st.m == -INFINITY ? 0.0f : -st.m);
+    sum2[0] = sum2[1] = 0ull;
+    exps32(c0, scale2, negm2, sum2, pk[0]);
+    exps32(c1, scale2, negm2, sum2, pk[1]);
+  }
+  hk.on_read();
+  hk.before_p();
+  tmem_st16(p_taddr, pk[0]);
+  tmem_st16(p_taddr + 16, pk[1]);
+  tmem_wait_st();
+  hk.on_half();
+  const uint64_t negm2 = dup2(st.m == -INFINITY ? 0.0f : -st.m);
+  exps32(c2, scale2, negm2, sum2, pk[0]);
+  tmem_st16(p_taddr + 32, pk[0]);
+  exps32(c3, scale2, negm2, sum2, pk[1]);
+  tmem_st16(p_taddr + 48, pk[1]);
+  tmem_wait_st();
+  hk.on_full();
+  float a0, a1;
+  unpack_f32x2(add_f32x2(sum2[0], sum2[1]), a0, a1);
+  st.l += a0 + a1;
+}
+
+}  // namespace pc

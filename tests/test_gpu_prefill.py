@@ -74,6 +74,36 @@ def test_shapes(C, L, w, Hq, Hkv, d, theta):
     _run_and_compare(q, k, v, w, theta)
 
 
+@pytest.mark.parametrize("L,Hq,Hkv,chunk_len", [
+    (128, 1, 1, None), (129, 1, 1, None), (384, 3, 1, None), (512, 2, 2, None), (513, 1, 1, None), (770, 7, 1, None),   # G odd: units of 4 tiles
+    (127, 2, 1, None), (256, 6, 1, None), (640, 4, 2, None),                     # G = 2 mod 4: units of 2 tiles, odd and even counts
+    (385, 8, 1, None), (260, 12, 1, None),                                       # G = 0 mod 4: two and three sets of 4 heads
+    (700, 5, 1, [700, 41, 129, 512]), (700, 2, 1, [257, 700]), (513, 4, 1, [384, 513, 41]),   # shorter chunks: absent blocks
+])
+def test_units_of_a_cta_pair(L, Hq, Hkv, chunk_len):
+    """Head size 128: a pair of CTAs takes four (q-head, query tile) blocks at a time, which blocks depends on the
+    group size; the edges are tile counts that do not fill a unit, windows that cross tiles and shorter chunks."""
+    import paper_2502_14317_b200 as pc
+    w, d, theta = 40, 128, 10000.0
+    C = len(chunk_len) if chunk_len else 2
+    rng = np.random.default_rng(L + 31 * Hq)
+    q, k, v = (pc_inputs.f32_to_bf16_bits(rng.standard_normal((C, L, h, d)).astype(np.float32)) for h in (Hq, Hkv, Hkv))
+    if chunk_len is None:
+        _run_and_compare(q, k, v, w, theta)
+        return
+    cl = torch.tensor(chunk_len, dtype=torch.int32, device="cuda")
+    res = pc.chunk_prefill_attn(to_dev(q), to_dev(k), to_dev(v), w=w, rope_theta=theta, want_lse=True, chunk_len=cl)
+    torch.cuda.synchronize()
+    assert int(res["status"].item()) == 0
+    for c, n in enumerate(chunk_len):
+        O, LSE, k_rot = orc.local_attention(q[c:c + 1, :n], k[c:c + 1, :n], v[c:c + 1, :n], theta)
+        S, _, _ = orc.window_scores(orc.rope_bf16(q[c:c + 1, :n], theta), k_rot, v[c:c + 1, :n], w, 1.0 / np.sqrt(d))
+        check_attention_output(to_f64(res["o"][c:c + 1, :n]), O)
+        assert np.abs(res["lse"][c:c + 1, :, :n].cpu().numpy() - LSE).max() <= 2e-3
+        check_scores(res["win_score"][c:c + 1, :, :n].cpu().numpy(), S, Hq // Hkv, w, n)
+        assert not res["o"][c, n:].any() and not res["win_score"][c, :, n:].any()
+
+
 @pytest.mark.parametrize("d", [64, 128])
 def test_growing_logits_rescale_path(d):
     """Keys whose norm grows along the chunk make the running row maximum jump by more than the lazy
