@@ -51,7 +51,7 @@ void fill_strides(const int64_t in[3], int64_t out[3], int64_t tokens, int64_t h
 bool strides_ok(const int64_t s[3], int64_t d) { return s[0] > 0 && s[1] > 0 && s[2] >= d && s[0] % 8 == 0 && s[1] % 8 == 0 && s[2] % 8 == 0; }
 
 struct PrefillLayout {
-  size_t off_counter, off_table, off_table32, off_qrot, off_lse2, off_krot, total;
+  size_t off_counter, off_table, off_table32, off_qrot, off_krot, total;
 };
 PrefillLayout prefill_layout(const pc_prefill_desc* d, bool krot_in_ws) {
   PrefillLayout l;
@@ -60,7 +60,6 @@ PrefillLayout prefill_layout(const pc_prefill_desc* d, bool krot_in_ws) {
   l.off_table = off; off += align_up((size_t)d->L * (d->d / 2) * sizeof(double2));
   l.off_table32 = off; off += align_up((size_t)d->L * (d->d / 2) * sizeof(float4));   // fp32 heads, then fp32 tails
   l.off_qrot = off; off += align_up((size_t)d->C * d->L * d->Hq * d->d * 2);         // rotated queries
-  l.off_lse2 = off; off += align_up((size_t)d->C * d->Hq * ((d->w + 7) & ~7) * sizeof(float));
   l.off_krot = off;
   if (krot_in_ws) off += align_up((size_t)d->C * d->L * d->Hkv * d->d * 2);
   l.total = off;
@@ -180,7 +179,6 @@ int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q, const 
   prm.scale_log2 = (float)(scale * 1.4426950408889634);
   prm.lse = lse; prm.win_lse = win_lse; prm.win_score = win_score;
   prm.status = status_word; prm.counter = counter;
-  prm.lse2 = reinterpret_cast<float*>(ws + lay.off_lse2);
   prm.wait_kcycles = pc::g_wait_kcycles.load();
   prm.skip_final_publication = pc::g_skip_final_publication.load();
   // Head size 128 runs on CTA pairs: halved shared-memory operands (a single CTA's 128 x 128 x 128 product reads 128 bytes

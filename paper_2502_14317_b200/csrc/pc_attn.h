@@ -16,7 +16,6 @@ struct PrefillParams {
   float* win_score;              // [C,Hkv,L]
   int* status;                   // device status word or null
   int* counter;                  // work-queue counter, zeroed before launch
-  float* lse2;                   // [C,Hq,wp] scratch: log-sum-exp of the window rows (log2 units), wp = w rounded up to 8
   int wait_kcycles;              // limit of every device-side wait, in units of 1024 cycles
   int skip_final_publication;    // test hook of the bounded waits (see pc_debug_bounded_wait_test in pc.h)
 };

@@ -61,8 +61,9 @@ struct __align__(16) Misc2 {
   uint32_t tmem_base;
   int abort_flag;                            // the two words after tmem_base stay adjacent: bounded waits read the limit
   int wait_kcycles;                          // through the flag's address
-  float lm[2][2][TILE];                      // [block][max / sum][row]: final statistics of a block; in the score sweep
-                                             // [buffer][key]: partial window scores of the second column half
+  alignas(16) float lm[2][2][TILE];          // [block][max / sum][row]: final statistics of a block; in the score sweep [0]:
+                                             // [buffer][key] partial window scores of the second column half, [1]:
+                                             // [column half][column] log-sum-exp of the window rows
 };
 
 constexpr int OFF_Q = 0;
@@ -549,13 +550,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           const size_t row = (size_t)d.c * prm.Hq + h;
           if (prm.lse) prm.lse[row * prm.L + token] = lse2 * 0.6931471805599453f;
           const int wi = token - (d.len - prm.w);
-          if (wi >= 0) {
-            prm.win_lse[row * prm.w + wi] = lse2 * 0.6931471805599453f;
-            float* const slot = prm.lse2 + row * sch.wp + (sch.wp - prm.w);
-            slot[wi] = lse2;
-            if (wi == 0)                                         // operand rows that are not window rows: probability 0
-              for (int i = 1; i <= sch.wp - prm.w; ++i) slot[-i] = INFINITY;
-          }
+          if (wi >= 0) prm.win_lse[row * prm.w + wi] = lse2 * 0.6931471805599453f;
         }
         fence_proxy_async_smem();
         named_barrier_sync(1, 128);
@@ -617,7 +612,19 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const int g0 = u * 2 * sch.hp + b * sch.hp;
         const int heads = sch.G - g0 < sch.hp ? (sch.G > g0 ? sch.G - g0 : 0) : sch.hp;
         const int cols = heads * sch.wp;
-        const float* const lse_rows = prm.lse2 + ((size_t)d.c * prm.Hq + d.hkv * sch.G + g0) * sch.wp;
+        // log-sum-exp of the columns' window rows in log2 units; +inf (probability 0) in columns that are no window rows.
+        // (The outputs win_lse are read back, from both CTAs: exact to half an ulp of the natural logarithm.)
+        float* const lse_cols = &mi.lm[1][b][0];
+        if (r < cols) {
+          const int wi = r % sch.wp - (sch.wp - prm.w);
+          float x = INFINITY;
+          if (wi >= 0) {
+            const float nat = __ldcg(prm.win_lse + ((size_t)d.c * prm.Hq + d.hkv * sch.G + g0 + r / sch.wp) * prm.w + wi);
+            x = fmaf(nat, 1.442695040888963f, nat * 1.925963033500e-8f);     // log2(e) as a sum of two floats
+          }
+          lse_cols[r] = x;
+        }
+        named_barrier_sync(3, 256);
         const int n_steps = ((d.len + TILE - 1) / TILE + 1) / 2;
         const int w0 = d.len - prm.w, pad = sch.wp - prm.w;      // first window token of this chunk
         float* const xch = &mi.lm[0][0][0];                      // [buffer][key]
@@ -637,14 +644,11 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             for (; col + 32 <= cols; col += 32) {
               uint32_t sv[32];
               tmem_ld32(tT + col, sv);
-              float4 ls[8];
-#pragma unroll
-              for (int i = 0; i < 8; ++i) ls[i] = __ldcg(reinterpret_cast<const float4*>(lse_rows + col) + i);
               tmem_wait_ld();
               loaded(sv);
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
-                const float4 l4 = ls[i / 2];
+                const float4 l4 = *reinterpret_cast<const float4*>(lse_cols + col + (i / 2) * 4);
                 const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), scale2,
                                               (i & 1) ? pack_f32x2(-l4.z, -l4.w) : pack_f32x2(-l4.x, -l4.y));
                 float x0, x1;
@@ -660,7 +664,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           for (; col < cols; col += 8) {                         // the rest, and tiles that reach into the window
             uint32_t sv[8];
             tmem_ld8(tT + col, sv);
-            const float4 la = __ldcg(reinterpret_cast<const float4*>(lse_rows + col)), lb = __ldcg(reinterpret_cast<const float4*>(lse_rows + col + 4));
+            const float4 la = *reinterpret_cast<const float4*>(lse_cols + col), lb = *reinterpret_cast<const float4*>(lse_cols + col + 4);
             const float ls[8] = {la.x, la.y, la.z, la.w, lb.x, lb.y, lb.z, lb.w};
             const int wi0 = col % sch.wp - pad;                  // window row of the first of these columns (negative: none)
             tmem_wait_ld();
