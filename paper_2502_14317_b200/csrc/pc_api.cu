@@ -370,6 +370,7 @@ struct ParallelPlan {
   int Gs, n_rg, n_cache_tiles, n_split, tiles_per_split;
   bool alt;                        // single-CTA kernel, rows of an item fit one block: two streams on alternate key tiles
   int n_part;                      // partial results to merge per (sequence, q-head)
+  int few_split;                   // few query rows (pc_decode.cu, no workspace): CTAs of a cluster per (sequence, kv-head)
   bool pair;                       // CTA-pair kernel: 256-row groups, no key split
   int hpc, n_rg_pair;              // pair kernel: q-heads per CTA, 256-row groups per kv-head
   size_t off_counter, off_table, off_table_hi, off_table_lo, off_qrot, off_ml, off_o, total;
@@ -390,7 +391,6 @@ ParallelPlan parallel_plan(int B, int w, int Hq, int Hkv, int d, int Nk, int sm_
   p.n_cache_tiles = (Nk + 127) / 128;
   const long long base = (long long)B * Hkv * p.n_rg;
   p.pair = false;
-  p.hpc = 0; p.n_rg_pair = 0;
   if (d == 128 && w >= 8 && (G * w) % 256 == 0 && sm_count >= 2) {
     const long long pairs = sm_count / 2, groups = (long long)B * Hkv * (G * w / 256);
     const long long rounds = (groups + pairs - 1) / pairs;
@@ -429,6 +429,21 @@ ParallelPlan parallel_plan(int B, int w, int Hq, int Hkv, int d, int Nk, int sm_
   p.off_o = off;
   if (p.n_part > 1) off += align_up((size_t)B * Hq * p.n_part * w * d * sizeof(float));
   p.total = off;
+  // few query rows (at most 32 per kv-head: the line is drawn where the transposed kernel stops winning, figures in
+  // pc_decode.cu): CTAs per (sequence, kv-head), 0: another kernel.  Least time by a model in microseconds - rounds of the
+  // grid (two CTAs per SM) x (about 6 for prologue, pipeline fill and merge + a tile at the CTA's share of
+  // the memory bandwidth, no faster than the 0.6 that the chain through the tensor cores takes)
+  p.few_split = 0;
+  if (G * w <= 32) {
+    const double slots = 2.0 * sm_count, tile_us = 512.0 * d / 6.5e6;
+    double least = -1.0;
+    for (int s = 1; s <= 16 && s <= p.n_cache_tiles + 1; s *= 2) {
+      const double ctas = (double)base * s, rounds = std::ceil(ctas / slots), active = ctas < slots ? ctas : slots;
+      const double per_tile = tile_us * active > 0.6 ? tile_us * active : 0.6;
+      const double cost = rounds * (6.0 + per_tile * std::ceil((p.n_cache_tiles + 1.0) / s));
+      if (least < 0.0 || cost < least) { least = cost; p.few_split = s; }
+    }
+  }
   return p;
 }
 
@@ -462,7 +477,7 @@ namespace {
 int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_t d, int32_t Nk, int64_t Nk_cap,
                            const void* q_win, int32_t q_pos0, float rope_theta, float softmax_scale, const void* k_cache,
                            const void* v_cache, const void* k_win, const void* v_win, void* out, float* lse_out,
-                           int32_t* status_word, void* workspace, size_t workspace_bytes, void* stream) {
+                           int32_t* status_word, void* workspace, size_t workspace_bytes, void* stream, bool append) {
   int32_t rc = check_parallel_args(B, w, Hq, Hkv, d, Nk);
   if (rc != PC_OK) return rc;
   if (Nk_cap < Nk || Nk_cap > (1ll << 28)) return PC_ERR_INVALID_ARG;
@@ -492,6 +507,30 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   const uint32_t box_kc[4] = {64, 128, 1, 1};
   const uint32_t box_kw[4] = {64, 1, 128, 1};
 
+  const double softmax_scale_d = softmax_scale > 0.0f ? (double)softmax_scale : 1.0 / std::sqrt((double)d);
+  if (plan.few_split > 0) {
+    CUtensorMap dm[4];
+    if (!pc::make_tmap_bf16_4d(&dm[0], k_cache, kc_dims, kc_str, box_kc) ||
+        !pc::make_tmap_bf16_4d(&dm[1], v_cache, kc_dims, kc_str, box_kc) ||
+        !pc::make_tmap_bf16_4d(&dm[2], k_win, kw_dims, kw_str, box_kw) ||
+        !pc::make_tmap_bf16_4d(&dm[3], v_win, kw_dims, kw_str, box_kw))
+      return PC_ERR_CUDA;
+    pc::DecodeParams dp;
+    dp.B = B; dp.w = w; dp.Hq = Hq; dp.Hkv = Hkv; dp.Nk = Nk;
+    dp.n_cache_tiles = plan.n_cache_tiles; dp.n_split = plan.few_split;
+    dp.q_pos0 = q_pos0; dp.rope_theta = rope_theta;
+    dp.scale_log2 = (float)(softmax_scale_d * 1.4426950408889634);
+    dp.q_win = q_win; dp.k_win = k_win; dp.v_win = v_win;
+    dp.k_append = append ? const_cast<void*>(k_cache) : nullptr;
+    dp.v_append = append ? const_cast<void*>(v_cache) : nullptr;
+    dp.Nk_cap = Nk_cap;
+    dp.out = static_cast<__nv_bfloat16*>(out);
+    dp.lse_out = lse_out;
+    dp.status = status_word;
+    dp.wait_kcycles = pc::g_wait_kcycles.load();
+    return pc::launch_decode_attn(dm, dp, d, st) == cudaSuccess ? PC_OK : PC_ERR_CUDA;
+  }
+
   // rotated queries first (the same pass that serves the chunk-local kernels)
   float4* table_hi = reinterpret_cast<float4*>(ws + plan.off_table_hi);
   float4* table_lo = reinterpret_cast<float4*>(ws + plan.off_table_lo);
@@ -499,6 +538,16 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   pc::launch_rope_table(table, table_hi, table_lo, w, d, (double)rope_theta, q_pos0, st);
   const long long q_stride[3] = {(long long)w * Hq * d, (long long)Hq * d, (long long)d};
   pc::launch_rope_rows(q_win, q_stride, q_rot, table, table_hi, table_lo, B, w, Hq, d, st);
+
+  // the attention reads entries below Nk only (rows behind them read as zeros and are masked): the new rows can follow
+  // on the same stream
+  auto append_kv = [&]() -> int32_t {
+    if (!append) return PC_OK;
+    return pc::launch_append_kv(k_win, v_win, B, w, Hkv, d, Nk, Nk_cap, const_cast<void*>(k_cache), const_cast<void*>(v_cache), st) ==
+                   cudaSuccess
+               ? PC_OK
+               : PC_ERR_CUDA;
+  };
 
   if (plan.pair) {
     CUtensorMap pm[6];
@@ -514,13 +563,12 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
     pc::ParallelPairParams pp;
     pp.B = B; pp.w = w; pp.Hq = Hq; pp.Hkv = Hkv; pp.Nk = Nk;
     pp.hpc = plan.hpc; pp.n_rg = plan.n_rg_pair;
-    const double scale = softmax_scale > 0.0f ? (double)softmax_scale : 1.0 / std::sqrt((double)d);
-    pp.scale_log2 = (float)(scale * 1.4426950408889634);
+    pp.scale_log2 = (float)(softmax_scale_d * 1.4426950408889634);
     pp.lse_out = lse_out;
     pp.status = status_word;
     pp.wait_kcycles = pc::g_wait_kcycles.load();
     if (pc::launch_parallel_pair(pm, pp, dev.sm_count, st) != cudaSuccess) return PC_ERR_CUDA;
-    return PC_OK;
+    return append_kv();
   }
 
   CUtensorMap maps[5];
@@ -538,8 +586,7 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   prm.Gs = plan.Gs; prm.n_rg = plan.n_rg;
   prm.n_cache_tiles = plan.n_cache_tiles; prm.n_split = plan.n_split; prm.tiles_per_split = plan.tiles_per_split;
   prm.alt = plan.alt ? 1 : 0; prm.n_part = plan.n_part;
-  const double scale = softmax_scale > 0.0f ? (double)softmax_scale : 1.0 / std::sqrt((double)d);
-  prm.scale_log2 = (float)(scale * 1.4426950408889634);
+  prm.scale_log2 = (float)(softmax_scale_d * 1.4426950408889634);
   prm.part_ml = reinterpret_cast<float*>(ws + plan.off_ml);
   prm.part_o = reinterpret_cast<float*>(ws + plan.off_o);
   prm.out = static_cast<__nv_bfloat16*>(out);
@@ -550,7 +597,7 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   const long long n_items = (long long)B * Hkv * plan.n_rg * plan.n_split;
   const int grid = (int)(n_items < dev.sm_count ? n_items : dev.sm_count);
   if (pc::launch_parallel_attn(maps, prm, d, grid, st) != cudaSuccess) return PC_ERR_CUDA;
-  return PC_OK;
+  return append_kv();
 }
 
 }  // namespace
@@ -562,7 +609,7 @@ int32_t pc_parallel_attn(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_t 
                          const void* v_cache, const void* k_win, const void* v_win, void* out, float* lse_out,
                          int32_t* status_word, void* workspace, size_t workspace_bytes, void* stream) {
   return parallel_attn_impl(B, w, Hq, Hkv, d, Nk, Nk, q_win, q_pos0, rope_theta, softmax_scale, k_cache, v_cache, k_win,
-                            v_win, out, lse_out, status_word, workspace, workspace_bytes, stream);
+                            v_win, out, lse_out, status_word, workspace, workspace_bytes, stream, false);
 }
 
 int32_t pc_parallel_attn_append(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_t d, int32_t Nk, int32_t Nk_cap,
@@ -570,16 +617,8 @@ int32_t pc_parallel_attn_append(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, i
                                 void* v_cache, const void* k_win, const void* v_win, void* out, float* lse_out,
                                 int32_t* status_word, void* workspace, size_t workspace_bytes, void* stream) {
   if (Nk_cap < 1 || (int64_t)Nk + w > (int64_t)Nk_cap) return PC_ERR_INVALID_ARG;
-  const int32_t rc = parallel_attn_impl(B, w, Hq, Hkv, d, Nk, Nk_cap, q_win, q_pos0, rope_theta, softmax_scale, k_cache,
-                                        v_cache, k_win, v_win, out, lse_out, status_word, workspace, workspace_bytes,
-                                        stream);
-  if (rc != PC_OK) return rc;
-  // the attention above reads entries below Nk only (rows behind them read as zeros and are masked): the new rows
-  // can follow on the same stream
-  if (pc::launch_append_kv(k_win, v_win, B, w, Hkv, d, Nk, Nk_cap, k_cache, v_cache, static_cast<cudaStream_t>(stream)) !=
-      cudaSuccess)
-    return PC_ERR_CUDA;
-  return PC_OK;
+  return parallel_attn_impl(B, w, Hq, Hkv, d, Nk, Nk_cap, q_win, q_pos0, rope_theta, softmax_scale, k_cache, v_cache, k_win,
+                            v_win, out, lse_out, status_word, workspace, workspace_bytes, stream, true);
 }
 
 }  // extern "C"

@@ -45,6 +45,23 @@ struct ParallelParams {
 // maps: rotated q_win (w-row box), k_cache, v_cache (128-key box), k_win, v_win (128-row box over w tokens)
 cudaError_t launch_parallel_attn(const CUtensorMap* maps, const ParallelParams& prm, int d, int grid, cudaStream_t st);
 
+// Parallel attention for few query rows (pc_decode.cu): Hq / Hkv * w <= 32.  One launch, no workspace.
+struct DecodeParams {
+  int B, w, Hq, Hkv, Nk;
+  int n_cache_tiles, n_split;    // 128-key tiles of the cache; CTAs (of a cluster) per (sequence, kv-head), 1 .. 16
+  int q_pos0;
+  float rope_theta, scale_log2;
+  const void *q_win, *k_win, *v_win;
+  void *k_append, *v_append;     // caches to append the new entries to at Nk (rows Nk_cap apart), or null
+  long long Nk_cap;
+  __nv_bfloat16* out;            // [B,w,Hq,d]
+  float* lse_out;                // [B,Hq,w] or null
+  int* status;
+  int wait_kcycles;
+};
+// maps: k_cache, v_cache (128-key box), k_win, v_win (128-row box over w tokens)
+cudaError_t launch_decode_attn(const CUtensorMap* maps, const DecodeParams& prm, int d, cudaStream_t st);
+
 // Parallel attention on CTA pairs (head size 128, G * w a multiple of 256, no key split): every pair takes the
 // windows of 2 * hpc q-heads of one kv-head (hpc * w = 128 rows per CTA) over the whole cache.
 struct ParallelPairParams {

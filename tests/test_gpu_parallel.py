@@ -51,6 +51,32 @@ def test_parallel_attn_shapes(B, w, Hq, Hkv, d, Nk, q_pos0, theta):
     assert np.abs(res["lse"].cpu().numpy() - LSE).max() <= 2e-3
 
 
+@pytest.mark.parametrize("B,w,Hq,Hkv,d,Nk,grow", [
+    (1, 1, 1, 1, 128, 1, 0), (1, 1, 3, 1, 64, 127, 0), (2, 1, 2, 2, 128, 129, 0),    # one and two tiles: fewer than key splits
+    (1, 2, 8, 1, 128, 2050, 0), (1, 1, 17, 1, 128, 700, 0), (2, 4, 8, 1, 64, 640, 0),   # 16, 17 and 32 rows per kv-head
+    (1, 1, 33, 1, 64, 513, 0), (3, 8, 4, 1, 128, 1500, 0), (1, 32, 2, 2, 64, 900, 0),   # 33 rows (the row-major kernel), 32 rows
+    (150, 1, 8, 2, 128, 140, 0), (40, 16, 16, 8, 64, 260, 0),                     # more items than CTAs fit
+    (1, 4, 8, 2, 128, 3000, 1), (30, 8, 4, 1, 64, 600, 1),                            # growing keys: the reference maxima are raised in most tiles
+])
+def test_few_query_rows(B, w, Hq, Hkv, d, Nk, grow):
+    """Up to 32 query rows per (sequence, kv-head): the transposed kernel, its row paddings, key splits and merge."""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(Nk + 3 * w + Hq)
+    qw = _bits(rng, (B, w, Hq, d))
+    kc, vc = rng.standard_normal((B, Hkv, Nk, d)).astype(np.float32), _bits(rng, (B, Hkv, Nk, d))
+    if grow:
+        kc *= np.linspace(1.0, 40.0, Nk, dtype=np.float32)[None, None, :, None]
+    kc = pc_inputs.f32_to_bf16_bits(kc)
+    kw, vw = _bits(rng, (B, w, Hkv, d)), _bits(rng, (B, w, Hkv, d))
+    res = pc.parallel_attn(to_dev(qw), to_dev(kc), to_dev(vc), to_dev(kw), to_dev(vw), q_pos0=500, rope_theta=1e4,
+                           want_lse=True)
+    torch.cuda.synchronize()
+    assert int(res["status"].item()) == 0
+    Fg, LSE = orc.parallel_attention(qw, 500, 1e4, None, kc, vc, kw, vw)
+    check_attention_output(to_f64(res["out"]), Fg, "Fg", sharp=bool(grow))
+    assert np.abs(res["lse"].cpu().numpy() - LSE).max() <= 2e-3
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,d,Nk0,cap,steps", [
     (2, 8, 2, 128, 250, 260, (1, 1, 4, 1)),   # crosses a tile boundary of the cache (256) while generating
     (3, 4, 4, 64, 40, 48, (1, 2, 1)),         # MHA, head size 64
