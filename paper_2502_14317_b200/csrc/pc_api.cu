@@ -181,11 +181,7 @@ int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q, const 
   prm.status = status_word; prm.counter = counter;
   prm.wait_kcycles = pc::g_wait_kcycles.load();
   prm.skip_final_publication = pc::g_skip_final_publication.load();
-  // Head size 128 runs on CTA pairs: halved shared-memory operands (a single CTA's 128 x 128 x 128 product reads 128 bytes
-  // a cycle, all that shared memory gives) and halved L2 traffic are worth 6 % at equal structure.  Head size 64 runs on
-  // single CTAs: its products are half as long and the softmax is what bounds it.
-  const cudaError_t le = d == 128 ? pc::launch_prefill_pair(maps, prm, dev.sm_count, st)
-                                  : pc::launch_prefill_attn(maps, prm, dev.sm_count, st);
+  const cudaError_t le = pc::launch_prefill_attn(maps, prm, d, dev.sm_count, st);
   if (le != cudaSuccess) return PC_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? PC_OK : PC_ERR_CUDA;
 }

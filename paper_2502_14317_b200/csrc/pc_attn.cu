@@ -1,5 +1,5 @@
-// Attention kernels for sm_100a: chunk-local causal attention with fused query-window
-// scores (Eq. 1-2, Eq. 5-6) and parallel attention over the compressed cache (Eq. 9-11).
+// Parallel attention over the compressed cache (Eq. 9-11) on single CTAs: batches and shapes that neither the CTA-pair
+// kernel (pc_parallel2.cu) nor the kernel for few query rows (pc_decode.cu) takes.
 //
 // One persistent CTA per SM, 12 warps in 3 warpgroups:
 //   warps 0-3  softmax group 0   (one 128-row query block, thread = row = TMEM lane)
@@ -20,12 +20,6 @@
 // Queries and keys arrive rotated (the RoPE pre-pass of pc_rope.cu runs before these kernels).
 // In the parallel attention an item whose rows fill one block only (a decoding step) is run by
 // BOTH groups on alternate key tiles and merged afterwards, like two key splits.
-//
-// Window scores (prefill only): the item that owns the last query tiles of a
-// (chunk, kv-head) group runs them for all G q-heads, keeps the window rows' final
-// log-sum-exp in shared memory, then sweeps the keys once more computing the transposed
-// product K_j Qw^T (keys on TMEM lanes, the G*w window rows on columns), so the column
-// sum of Eq. 6 is a per-thread sum in a fixed order: deterministic, no atomics.
 #include "pc_kernels.h"
 #include "pc_attn.h"
 #include "pc_sm100.cuh"
@@ -44,22 +38,19 @@ constexpr float LAZY_RESCALE = 8.0f;        // log2 units
 constexpr int ITEM_DONE = -1;
 
 // where-codes stored in the status word when a wait gives up
-enum { W_ITEM = 101, W_QFULL, W_QROT /* unused, keeps the later codes */, W_QFREE, W_KVFULL, W_KVFREE, W_SFULL, W_PFULL, W_OFULL, W_ACCFREE, W_TFULL, W_TFREE, W_TURN, W_PHALF };
+enum { W_ITEM = 101, W_QFULL, W_QROT /* unused, keeps the later codes */, W_QFREE, W_KVFULL, W_KVFREE, W_SFULL, W_PFULL, W_OFULL, W_ACCFREE, W_TFULL /* unused */, W_TFREE /* unused */, W_TURN, W_PHALF };
 
 struct __align__(16) Misc {
   uint64_t q_full[2], q_free[2];
   uint64_t kv_full[NS], kv_free[NS];
   uint64_t s_full[2], p_half[2], p_full[2], o_full[2], acc_free[2];
   uint64_t item_full[2], item_empty[2];
-  uint64_t t_full[2], t_free[2];
   uint64_t turn[2];                        // issue token passed between the two tcgen05 issuers
   uint64_t mma_done;                       // every tensor-core operation of both issuers has completed (teardown)
   int item_slot[2];
   uint32_t tmem_base;
   int abort_flag;                          // these two words stay adjacent: bounded waits read the limit through the
   int wait_kcycles;                        // flag's address
-  float lse2[1024];                        // window-row log-sum-exp (log2 domain), G * w <= 1024
-  float xch[2][TILE];
 };
 
 template <int D>
@@ -71,99 +62,6 @@ struct Cfg {
   static constexpr int OFF_MISC = OFF_RING + NS * TILE_BYTES;
   static constexpr int SMEM_BYTES = OFF_MISC + (int)sizeof(Misc) + 1024;   // + alignment slack
 };
-
-// One pair of 128-row query blocks that share K/V tiles.
-struct SubItem {
-  int hA, tA, hB, tB;        // q-head and query tile of block A / B; hB < 0: block B absent
-};
-
-// ------------------------------------------------------------------ item decoding (prefill)
-// With per-chunk lengths the query tiles of a shorter chunk are numbered from the END: slot v of the static
-// decomposition (v = T - 1 is the last tile of a full-length chunk) is tile v - (T - T_c) of a chunk with T_c
-// tiles; slots below T - T_c are empty.  The window then always sits in the last two slots, which the tail item
-// of the group owns together with the score sweep.
-struct Sched {
-  int T, t_w, ntt, G, P, hp_mode, ipg, n_lp;
-  int wp, hb, Gs, n_pass;                    // score sweep: operand rows per head (w rounded up to 8), heads per 128-row
-                                             // block, heads per pass, passes
-};
-
-// length of chunk c in tokens (window included), clamped to (w, L]
-__device__ __forceinline__ int chunk_length(const PrefillParams& p, int c) {
-  if (p.chunk_len == nullptr) return p.L;
-  int len = __ldg(p.chunk_len + c);
-  len = len > p.L ? p.L : len;
-  return len <= p.w ? p.w + 1 : len;
-}
-
-__device__ __forceinline__ Sched make_sched(const PrefillParams& p) {
-  Sched s;
-  s.T = (p.L + TILE - 1) / TILE;
-  s.G = p.Hq / p.Hkv;
-  s.hp_mode = (s.G % 2 == 0);
-  s.P = s.G / 2;
-  s.wp = (p.w + 7) & ~7;
-  s.hb = TILE / s.wp;
-  s.Gs = 2 * s.hb < s.G ? 2 * s.hb : s.G;
-  s.n_pass = (s.G + s.Gs - 1) / s.Gs;
-  if (s.hp_mode) {
-    // tail slots: the tiles that can hold window rows (two with per-chunk lengths: the window of some chunk may
-    // straddle two tiles even where that of a full-length chunk does not)
-    s.ntt = (p.chunk_len != nullptr) ? (p.w > 1 ? 2 : 1) : s.T - (p.L - p.w) / TILE;
-    if (s.ntt > s.T) s.ntt = s.T;
-    s.t_w = s.T - s.ntt;
-    s.n_lp = 0;
-    s.ipg = 1 + s.t_w * s.P;
-  } else {
-    s.ntt = s.T >= 2 ? 2 : 1;
-    s.t_w = s.T - s.ntt;
-    s.n_lp = (s.t_w + 1) / 2;                // tile pairs below the tail, from the top
-    s.ipg = 1 + s.n_lp * s.G;
-  }
-  return s;
-}
-
-// score sweep: q-heads whose window rows sit in block b (0 / 1) of pass u
-__device__ __forceinline__ int sweep_heads(const Sched& s, int u, int b) {
-  const int heads = (s.G - u * s.Gs) < s.Gs ? (s.G - u * s.Gs) : s.Gs;
-  const int first = heads < s.hb ? heads : s.hb;
-  return b ? heads - first : first;
-}
-
-// number of sub-items of item `within` (0 = tail item of the group)
-__device__ __forceinline__ int n_subitems(const Sched& s, int within) {
-  if (within != 0) return 1;
-  return s.hp_mode ? s.P * s.ntt : s.G;
-}
-
-// len: length of the sub-item's chunk.  Returns hA < 0 for an empty sub-item (every role skips it).
-__device__ __forceinline__ SubItem decode_sub(const Sched& s, int hkv, int within, int sub, int len) {
-  SubItem it;
-  const int h0 = hkv * s.G;
-  if (s.hp_mode) {
-    int pair, tile;
-    if (within == 0) { pair = sub / s.ntt; tile = s.T - 1 - (sub % s.ntt); }
-    else { const int x = within - 1; tile = s.t_w - 1 - x / s.P; pair = x % s.P; }
-    it.hA = h0 + 2 * pair; it.hB = it.hA + 1; it.tA = tile; it.tB = tile;
-  } else {
-    int g, hi;
-    if (within == 0) { g = sub; hi = s.T - 1; }
-    else { const int x = within - 1; g = x % s.G; hi = s.t_w - 1 - 2 * (x / s.G); }
-    if (hi >= 1) { it.hA = h0 + g; it.tA = hi - 1; it.hB = h0 + g; it.tB = hi; }
-    else { it.hA = h0 + g; it.tA = hi; it.hB = -1; it.tB = 0; }
-  }
-  const int shift = s.T - (len + TILE - 1) / TILE;          // empty slots of a shorter chunk
-  if (shift > 0) {
-    it.tA -= shift;
-    it.tB -= shift;
-    if (it.hB >= 0 && it.tB < 0) it.hB = -1;
-    if (it.tA < 0) {
-      if (it.hB >= 0 && s.hp_mode == 0) { it.tA = it.tB; it.hB = -1; it.tB = 0; }   // only the upper tile of the pair exists
-      else { it.hA = -1; it.hB = -1; }
-    }
-  }
-  return it;
-}
 
 // One arrival for a whole warp (an arrival per thread costs the barrier 32 serialised shared-memory operations).
 __device__ __forceinline__ void warp_arrive(uint64_t* bar) {
@@ -260,11 +158,6 @@ __device__ __forceinline__ void issue_qk(uint32_t d_tmem, uint32_t q_smem, uint3
            ks > 0);
   }
 }
-// transposed product for the score sweep: D[keys, rows] = K_tile * Qw^T
-template <int D>
-__device__ __forceinline__ void issue_kq(uint32_t d_tmem, uint32_t k_smem, uint32_t q_smem, int n_cols) {
-  issue_qk<D>(d_tmem, k_smem, q_smem, n_cols);
-}
 // k-steps [ks0, ks1) of O += P V (16 keys per step)
 template <int D>
 __device__ __forceinline__ void issue_pv(uint32_t o_tmem, uint32_t p_tmem, uint32_t v_smem, bool accumulate, int ks0,
@@ -282,7 +175,6 @@ struct Waits {                                 // how many times each barrier ha
   uint32_t q[2] = {0, 0};                      // q_full / q_free (one use per block load)
   uint32_t kv = 0;                             // ring position (monotone)
   uint32_t s[2] = {0, 0}, p[2] = {0, 0}, o[2] = {0, 0}, acc[2] = {0, 0};   // p counts p_half and p_full alike
-  uint32_t t[2] = {0, 0};
   uint32_t turn = 0;                           // batches issued so far by this issuer
   uint32_t item = 0;
 };
@@ -306,7 +198,6 @@ __device__ __forceinline__ void init_barriers(Misc& mi, int wait_kcycles) {
     mbar_init(&mi.s_full[b], 1); mbar_init(&mi.p_half[b], 4); mbar_init(&mi.p_full[b], 4); mbar_init(&mi.o_full[b], 1);
     mbar_init(&mi.acc_free[b], 4);
     mbar_init(&mi.item_full[b], 1); mbar_init(&mi.item_empty[b], 10);      // 8 softmax warps + 2 issuer threads
-    mbar_init(&mi.t_full[b], 2); mbar_init(&mi.t_free[b], 8);
     mbar_init(&mi.turn[b], 1);
   }
   for (int s = 0; s < NS; ++s) { mbar_init(&mi.kv_full[s], 1); mbar_init(&mi.kv_free[s], 2); }   // both issuers release a stage
@@ -317,16 +208,14 @@ __device__ __forceinline__ void init_barriers(Misc& mi, int wait_kcycles) {
 }
 
 // producer: publish the next work item (dynamic queue); returns it
-// skip_final: test hook - the "no more work" message is written but never signalled, so that the consumers' wait for
-// it runs out.  Nothing is in flight at that point: every copy has been consumed and every accumulator read out.
-__device__ __forceinline__ int producer_next_item(const Ctx& cx, Waits& wt, int* counter, int n_items, bool skip_final = false) {
+__device__ __forceinline__ int producer_next_item(const Ctx& cx, Waits& wt, int* counter, int n_items) {
   Misc& mi = *cx.mi;
   const int slot = wt.item & 1;
   mbar_wait(&mi.item_empty[slot], free_par(wt.item >> 1), cx.abort_flag, cx.status, W_ITEM);
   int item = atomicAdd(counter, 1);
   if (item >= n_items || *cx.abort_flag) item = ITEM_DONE;
   mi.item_slot[slot] = item;
-  if (!(skip_final && item == ITEM_DONE)) mbar_arrive(&mi.item_full[slot]);
+  mbar_arrive(&mi.item_full[slot]);
   ++wt.item;
   return item;
 }
@@ -394,10 +283,8 @@ __device__ __forceinline__ void mma_flash_block(const Ctx& cx, Waits& wt, int b,
   auto takes_part = [&](int j) { return has_b && j < n && (alternate ? ((j & 1) == b) : (j < nb_b)); };
   const int last = alternate ? (((n - 1) & 1) == b ? n - 1 : n - 2) : nb_b - 1;     // last tile of this block
   if (has_b) {
-    // accumulator and score buffers of earlier work must have been read out
+    // the accumulator of earlier work must have been read out
     mbar_wait(&mi.acc_free[b], free_par(wt.acc[b]), cx.abort_flag, cx.status, W_ACCFREE);
-#pragma unroll
-    for (int e = 0; e < 2; ++e) mbar_wait(&mi.t_free[e], free_par(wt.t[e]), cx.abort_flag, cx.status, W_TFREE);
     // the query block (rotated by the pre-pass, in global memory) is ready as soon as its copy has landed
     mbar_wait(&mi.q_full[b], full_par(wt.q[b]), cx.abort_flag, cx.status, W_QFULL);
     ++wt.q[b];
@@ -488,278 +375,6 @@ __device__ __forceinline__ void wg_flash_loop(const Ctx& cx, uint32_t& n_s, uint
 }
 
 }  // namespace
-
-// ====================================================================================
-//                                   PREFILL KERNEL
-// ====================================================================================
-template <int D>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
-prefill_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
-                    const __grid_constant__ CUtensorMap tm_qw, const __grid_constant__ PrefillParams prm) {
-  using C = Cfg<D>;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  Misc& mi = *reinterpret_cast<Misc*>(smem + C::OFF_MISC);
-  Ctx cx;
-  cx.mi = &mi;
-  cx.sQ[0] = smem + C::OFF_Q;
-  cx.sQ[1] = smem + C::OFF_Q + C::TILE_BYTES;
-  cx.ring = smem + C::OFF_RING;
-  cx.abort_flag = &mi.abort_flag;
-  cx.status = prm.status;
-
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const Sched sch = make_sched(prm);
-  const int n_items = prm.C * prm.Hkv * sch.ipg;
-  const int n_pass = sch.n_pass;
-
-  if (tid == 0) init_barriers(mi, prm.wait_kcycles);
-  if (warp == WARP_MMA) tmem_alloc(&mi.tmem_base, 512);
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  cx.tmem = mi.tmem_base;
-
-  Waits wt;
-
-  if (warp == WARP_PRODUCER) {
-    // ================================================================ TMA producer
-    if (lane == 0) {
-      tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); tma_prefetch_desc(&tm_qw);
-      while (true) {
-        const int item = producer_next_item(cx, wt, prm.counter, n_items, prm.skip_final_publication != 0);
-        if (item == ITEM_DONE) break;
-        const int group = item / sch.ipg, within = item % sch.ipg;
-        const int c = group / prm.Hkv, hkv = group % prm.Hkv;
-        const int nsub = n_subitems(sch, within);
-        const int len = chunk_length(prm, c);
-        const int T_c = (len + TILE - 1) / TILE;
-        for (int sub = 0; sub < nsub; ++sub) {
-          const SubItem it = decode_sub(sch, hkv, within, sub, len);
-          if (it.hA < 0) continue;
-#pragma unroll
-          for (int b = 0; b < 2; ++b) {
-            const int h = b ? it.hB : it.hA, t = b ? it.tB : it.tA;
-            if (h < 0) continue;
-            mbar_wait(&mi.q_free[b], free_par(wt.q[b]), cx.abort_flag, cx.status, W_QFREE);
-            mbar_arrive_expect_tx(&mi.q_full[b], C::TILE_BYTES);
-            for (int a = 0; a < C::ATOMS; ++a)
-              tma_load_4d(cx.sQ[b] + a * 16384, &tm_q, &mi.q_full[b], a * 64, h, t * TILE, c);
-            ++wt.q[b];
-          }
-          const int n = (it.hB >= 0 ? it.tB : it.tA) + 1;
-          for (int j = 0; j < n; ++j) {
-            producer_ring_tile<D>(cx, wt, &tm_k, hkv, j * TILE, c);
-            producer_ring_tile<D>(cx, wt, &tm_v, hkv, j * TILE, c);
-          }
-        }
-        if (within == 0) {
-          // ---- score sweep: window queries of Gs heads per pass, then all key tiles.  A head's rows in the operand
-          // are the wp tokens that end with the chunk (wp = w rounded up to 8: the first wp - w of them are not
-          // window rows and are left out of the sums; a start before token 0 reads zeros)
-          for (int u = 0; u < n_pass; ++u) {
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-              const int heads_b = sweep_heads(sch, u, b);
-              if (heads_b == 0) continue;
-              mbar_wait(&mi.q_free[b], free_par(wt.q[b]), cx.abort_flag, cx.status, W_QFREE);
-              mbar_arrive_expect_tx(&mi.q_full[b], heads_b * sch.wp * D * 2);
-              for (int ih = 0; ih < heads_b; ++ih) {
-                const int g = u * sch.Gs + b * sch.hb + ih;
-                for (int a = 0; a < C::ATOMS; ++a)
-                  tma_load_4d(cx.sQ[b] + a * 16384 + ih * sch.wp * 128, &tm_qw, &mi.q_full[b], a * 64, hkv * sch.G + g,
-                              len - sch.wp, c);
-              }
-              ++wt.q[b];
-            }
-            for (int j = 0; j < T_c; ++j) producer_ring_tile<D>(cx, wt, &tm_k, hkv, j * TILE, c);
-          }
-        }
-      }
-      producer_drain(cx, wt);
-    }
-    __syncwarp();
-  } else if (warp == WARP_MMA || warp == WARP_MMA + 1) {
-    // ================================================================ tcgen05 issuers (one per block)
-    if (lane == 0) {
-      const int b = warp - WARP_MMA;
-      const uint32_t ring_u32 = smem_u32(cx.ring);
-      const uint32_t q_u32 = smem_u32(cx.sQ[b]);
-      while (true) {
-        const int item = consumer_next_item(cx, wt, false);
-        if (item == ITEM_DONE) break;
-        const int group = item / sch.ipg, within = item % sch.ipg;
-        const int hkv = group % prm.Hkv;
-        const int nsub = n_subitems(sch, within);
-        const int len = chunk_length(prm, group / prm.Hkv);
-        const int T_c = (len + TILE - 1) / TILE;
-        for (int sub = 0; sub < nsub; ++sub) {
-          const SubItem it = decode_sub(sch, hkv, within, sub, len);
-          if (it.hA < 0) continue;
-          const bool has_b = (b == 0) || it.hB >= 0;
-          const int nb_b = (b == 0) ? it.tA + 1 : (it.hB >= 0 ? it.tB + 1 : 0);
-          const int n = (it.hB >= 0 ? it.tB : it.tA) + 1;
-          mma_flash_block<D>(cx, wt, b, has_b, nb_b, n);
-        }
-        if (within == 0) {
-          // ---- score sweep: this issuer computes the columns of its own block (window rows b*128..)
-          mbar_wait(&mi.acc_free[b], free_par(wt.acc[b]), cx.abort_flag, cx.status, W_ACCFREE);
-          for (int u = 0; u < n_pass; ++u) {
-            const int rows_b = sweep_heads(sch, u, b) * sch.wp;
-            if (rows_b > 0) { mbar_wait(&mi.q_full[b], full_par(wt.q[b]), cx.abort_flag, cx.status, W_QROT); ++wt.q[b]; }
-            for (int j = 0; j < T_c; ++j) {
-              const int e = j & 1;
-              mbar_wait(&mi.t_free[e], free_par(wt.t[e]), cx.abort_flag, cx.status, W_TFREE);
-              const int st = wt.kv % NS;
-              mbar_wait(&mi.kv_full[st], full_par(wt.kv / NS), cx.abort_flag, cx.status, W_KVFULL);
-              ++wt.kv;
-              if (rows_b > 0) {
-                tc_fence_after_sync();
-                issue_kq<D>(cx.tmem + e * 256 + b * 128, ring_u32 + st * C::TILE_BYTES, q_u32, (rows_b + 15) & ~15);
-                mma_commit(&mi.t_full[e]);
-                mma_commit(&mi.kv_free[st]);
-              } else {
-                mbar_arrive(&mi.t_full[e]);
-                mbar_arrive(&mi.kv_free[st]);
-              }
-              ++wt.t[e];
-            }
-          }
-        }
-      }
-      mma_commit(&mi.mma_done);                              // teardown waits for everything this thread issued
-    }
-    __syncwarp();
-  } else if (warp < 8) {
-    // ================================================================ softmax groups
-    const int b = warp >> 2;                                 // block / group index
-    const int r = tid & 127;                                 // row in the block = TMEM lane
-    const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tS = cx.tmem + b * 128 + lane_sel, tO = cx.tmem + 256 + b * 128 + lane_sel;
-    const float scale_log2 = prm.scale_log2;
-    uint8_t* const myQ = b ? cx.sQ[1] : cx.sQ[0];
-    uint32_t n_s = 0, n_o = 0, n_t0 = 0, n_t1 = 0;            // barrier use counts of this group
-    while (true) {
-      const int item = consumer_next_item(cx, wt, true);
-      if (item == ITEM_DONE) break;
-      const int group = item / sch.ipg, within = item % sch.ipg;
-      const int c = group / prm.Hkv, hkv = group % prm.Hkv;
-      const int nsub = n_subitems(sch, within);
-      const int len = chunk_length(prm, c);
-      const int T_c = (len + TILE - 1) / TILE;
-      for (int sub = 0; sub < nsub; ++sub) {
-        const SubItem it = decode_sub(sch, hkv, within, sub, len);
-        const int h = b ? it.hB : it.hA, t = b ? it.tB : it.tA;
-        if (h < 0) continue;
-        const int token = t * TILE + r;
-        // ---- main loop over key tiles (causal: keys <= token; only the diagonal tile is masked)
-        float m_used, l_run;
-        const int n = t + 1;
-        wg_flash_loop<D>(cx, n_s, n_o, b, tS, tO, n, scale_log2,
-                         [&](int j) { return (j == n - 1) ? (token - j * TILE + 1) : TILE; }, m_used, l_run);
-        // ---- epilogue: normalise, stage bf16 rows in the (now idle) Q buffer, TMA store
-        const float inv_l = 1.0f / l_run;
-        const bool in_chunk = token < len;                   // rows behind the end of the chunk are written as zeros
-#pragma unroll
-        for (int q = 0; q < D / 32; ++q) {
-          uint32_t o[32];
-          tmem_ld32(tO + q * 32, o);
-          tmem_wait_ld();
-#pragma unroll
-          for (int g4 = 0; g4 < 4; ++g4) {
-            uint32_t pk[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              pk[e] = in_chunk ? pack_bf16x2(__uint_as_float(o[g4 * 8 + 2 * e]) * inv_l, __uint_as_float(o[g4 * 8 + 2 * e + 1]) * inv_l) : 0u;
-            const int col = q * 32 + g4 * 8;
-            *reinterpret_cast<uint4*>(myQ + (col / 64) * 16384 + sw128_offset(r, (col % 64) / 8)) =
-                make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          }
-        }
-        tc_fence_before_sync();
-        warp_arrive(&mi.acc_free[b]);
-        const float lse2 = m_used + log2f(l_run);
-        if (in_chunk) {
-          if (prm.lse) prm.lse[((size_t)c * prm.Hq + h) * prm.L + token] = lse2 * 0.6931471805599453f;
-          const int wi = token - (len - prm.w);
-          if (wi >= 0) {
-            prm.win_lse[((size_t)c * prm.Hq + h) * prm.w + wi] = lse2 * 0.6931471805599453f;
-            if (within == 0) mi.lse2[(h - hkv * sch.G) * prm.w + wi] = lse2;
-          }
-        }
-        fence_proxy_async_smem();
-        named_barrier_sync(1 + b, 128);
-        if (r == 0) {
-          for (int a = 0; a < C::ATOMS; ++a) tma_store_4d(&tm_o, myQ + a * 16384, a * 64, h, t * TILE, c);
-          tma_store_commit();
-          tma_store_wait_read();
-          mbar_arrive(&mi.q_free[b]);
-        }
-      }
-      if (within == 0) {
-        // ---- score sweep: this thread owns key (j * 128 + r); columns are the window rows
-        named_barrier_sync(3, 256);                           // lse2 complete and visible to both groups
-        const int w0 = len - prm.w;                           // first window token of this chunk
-        for (int u = 0; u < n_pass; ++u) {
-          const int heads_b = sweep_heads(sch, u, b);          // heads whose rows sit in this group's columns
-          const int rows_b = heads_b * sch.wp;
-          const float* lse_rows = mi.lse2 + (u * sch.Gs + b * sch.hb) * prm.w;   // log-sum-exp of this group's first head
-          for (int j = 0; j < T_c; ++j) {
-            const int e = j & 1;
-            mbar_wait(&mi.t_full[e], full_par(e ? n_t1 : n_t0), cx.abort_flag, cx.status, W_TFULL);
-            if (e) ++n_t1; else ++n_t0;
-            tc_fence_after_sync();
-            const int key = j * TILE + r;
-            const bool need_mask = (j * TILE + TILE - 1) > w0;
-            float part = 0.0f;
-            const uint32_t tT = cx.tmem + e * 256 + b * 128 + lane_sel;
-            for (int ih = 0; ih < heads_b; ++ih) {             // a head has wp columns, the last w of them are window rows
-              for (int col = 0; col < sch.wp; col += 8) {
-                uint32_t sv[8];
-                tmem_ld8(tT + ih * sch.wp + col, sv);
-                tmem_wait_ld();
-                const int wi0 = col - (sch.wp - prm.w);        // window row of the first of these columns (negative: none)
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) {
-                  const int wi = wi0 + jj;
-                  float pv = fast_exp2(fmaf(__uint_as_float(sv[jj]), scale_log2, -lse_rows[ih * prm.w + (wi < 0 ? 0 : wi)]));
-                  if (wi < 0 || (need_mask && key > w0 + wi)) pv = 0.0f;
-                  part += pv;
-                }
-              }
-            }
-            tc_fence_before_sync();
-            warp_arrive(&mi.t_free[e]);
-            if (b == 1) mi.xch[e][r] = part;
-            named_barrier_sync(3, 256);
-            if (b == 0 && key < len) {
-              float* dst = prm.win_score + ((size_t)c * prm.Hkv + hkv) * prm.L + key;
-              const float total = part + mi.xch[e][r];
-              *dst = (u == 0) ? total : (*dst + total);
-            }
-          }
-          if (rows_b > 0) {
-            named_barrier_sync(1 + b, 128);                   // every thread of the group is past its last use of sQ[b]
-            if (r == 0) mbar_arrive(&mi.q_free[b]);
-          }
-        }
-      }
-    }
-    if (r == 0) tma_store_wait_all();
-  }
-
-  tc_fence_before_sync();
-  __syncthreads();
-  if (warp == WARP_MMA) {
-    // no tensor-core operation may still be running when its accumulators are freed: both issuers ended with a
-    // commit to mma_done.  Immediate in a clean run; after an abort this is what makes the exit safe (the wait
-    // ignores the abort flag and is bounded).
-    mbar_wait_drain(&mi.mma_done, 0, cx.abort_flag);
-    tc_fence_after_sync();
-    tmem_dealloc(cx.tmem, 512);
-  }
-}
 
 // ====================================================================================
 //                          PARALLEL (GLOBAL) ATTENTION KERNEL
@@ -984,21 +599,6 @@ __global__ void __launch_bounds__(256) parallel_merge_kernel(const float* __rest
 // ====================================================================================
 //                                   host launchers
 // ====================================================================================
-template <int D>
-static cudaError_t launch_prefill_t(const CUtensorMap* maps, const PrefillParams& prm, int grid, cudaStream_t st) {
-  // the opt-in to large dynamic shared memory is a per-device attribute of the function: set it on every call
-  // (a host-side call of a few hundred nanoseconds) rather than remember which devices have it
-  if (cudaError_t e = cudaFuncSetAttribute(prefill_attn_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         Cfg<D>::SMEM_BYTES); e != cudaSuccess) return e;
-  note_launch();
-  prefill_attn_kernel<D><<<grid, NUM_THREADS, Cfg<D>::SMEM_BYTES, st>>>(maps[0], maps[1], maps[2], maps[3], maps[4], prm);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int grid, cudaStream_t st) {
-  return launch_prefill_t<64>(maps, prm, grid, st);
-}
-
 template <int D>
 static cudaError_t launch_parallel_t(const CUtensorMap* maps, const ParallelParams& prm, int grid, cudaStream_t st) {
   // the opt-in to large dynamic shared memory is a per-device attribute of the function: set it on every call

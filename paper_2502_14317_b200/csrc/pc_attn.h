@@ -20,11 +20,8 @@ struct PrefillParams {
   int skip_final_publication;    // test hook of the bounded waits (see pc_debug_bounded_wait_test in pc.h)
 };
 
-// Head size 64.  maps: rotated q (box 64x1x128x1), k_rot, v, o (store), rotated q with a wp-row box
-cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int grid, cudaStream_t st);
-
-// Head size 128: CTA-pair kernel (pc_prefill2.cu).  maps as above plus maps[5] = rotated keys with a 64-token box.
-cudaError_t launch_prefill_pair(const CUtensorMap* maps, const PrefillParams& prm, int sm_count, cudaStream_t st);
+// maps: rotated q (box 64 x 1 x 128 tokens), k_rot, v, o (store), rotated q with a wp-row box, k_rot with a 64-token box
+cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int d, int sm_count, cudaStream_t st);
 
 struct ParallelParams {
   int B, w, Hq, Hkv, Nk;

@@ -1,19 +1,22 @@
-// Chunk-local causal attention with fused query-window scores (Eq. 1-2, Eq. 5-6) for head
-// size 128 on CTA pairs.
+// Chunk-local causal attention with fused query-window scores (Eq. 1-2, Eq. 5-6).
 //
-// Two CTAs of a cluster work as one unit (tcgen05 cta_group::2).  Each CTA owns TWO 128-row query blocks A and B, so
-// four blocks walk the same K/V tiles at a time: every 128-key tile is split between the two shared memories (each CTA
-// stages 64 keys of K and 64 head-dim columns of V) and one MMA of M = 256 feeds both SMs.  While the softmax of one
-// block runs the tensor cores work for the other.
+// A CTA owns TWO 128-row query blocks A and B that walk the same K/V tiles; while the softmax of one block runs the
+// tensor cores work for the other.
 //
-// Per CTA, TMEM holds S and (over its first half) P of both blocks, 128 columns each, and both accumulators.
+// Head size 128 runs on CTA pairs (cluster of two, tcgen05 cta_group::2): four blocks share the tiles, every
+// 128-key tile is split between the two shared memories (each CTA stages 64 keys of K and 64 head-dim columns of V) and
+// one MMA of M = 256 feeds both SMs.  A single CTA's 128 x 128 x 128 product reads 128 bytes a cycle, all that shared
+// memory gives; on a pair it reads 96, and the L2 traffic is halved.  TMEM of a CTA: S of both blocks with P over
+// its first half (128 columns each) and both accumulators (128 each).
+// Head size 64 runs on single CTAs: its products are half as long, the softmax is what bounds it, and there is room in
+// TMEM for P beside S, so the next tile's S is computed as soon as the present one is in registers.
 //
 // Warps (16 per CTA): 0-3 softmax of block A, 4-7 softmax of block B (thread = query row = TMEM lane), 8-11 epilogue (the
-// softmax warps go straight on to the next block), 12 TMA producer, 13 issuer of all MMAs (leader CTA only), 14-15 idle.
-// Registers are dealt out by role: 184 / 80 / 64.
+// softmax warps go straight on to the next block), 12 TMA producer, 13 issuer of all MMAs (of a pair: in the leader CTA
+// only), 14-15 idle.  Registers are dealt out by role: 184 / 80 / 64.
 //
-// Window scores: the pair that runs the last query tiles of a (chunk, kv-head) group then sweeps the keys once more
-// with the transposed product K_j Qw^T (each CTA takes every other key tile; keys on TMEM lanes, window
+// Window scores: the unit that runs the last query tiles of a (chunk, kv-head) group then sweeps the keys once more
+// with the transposed product K_j Qw^T (the CTAs of a pair take alternate key tiles; keys on TMEM lanes, window
 // rows on columns), so Eq. 6 is a per-thread sum in a fixed order: deterministic, fp32, no atomics.
 #include "pc_attn.h"
 #include "pc_kernels.h"
@@ -24,33 +27,43 @@ namespace pc {
 namespace {
 
 constexpr int TILE = 128;
-constexpr int D = 128;
 constexpr int NT2 = 512;                     // threads per CTA
 constexpr int WARP_EPI = 8, WARP_PRODUCER = 12, WARP_MMA = 13;
 constexpr int REGS_SOFTMAX = 184, REGS_EPI = 80, REGS_SERVICE = 64;      // 128 * (2 * 184 + 80 + 64) = 64 K registers
 constexpr int NQ = 4;                        // query slots: the two blocks in work and the two that come next
-constexpr int NS = 6;                        // K/V ring stages (16 KB: 64 keys x 128 d of K, or 128 keys x 64 d of V)
+constexpr int NS = 6;                        // K/V ring stages (16 KB: of a pair 64 keys x 128 d of K or 128 keys x 64 d of V;
+                                             // of a single CTA 128 keys x 64 d)
 constexpr int NDESC = 4;                     // work descriptors in flight
-constexpr int HALF_BYTES = 16384;
-constexpr int Q_BYTES = 32768;
-constexpr uint32_t TM_O = 256;               // accumulator columns (block b: + 128 b)
+constexpr int STAGE_BYTES = 16384;
+template <int D>
+struct Cfg {
+  static constexpr bool PAIR = D == 128;
+  static constexpr int NCTA = PAIR ? 2 : 1;
+  static constexpr int ATOMS = D / 64;
+  static constexpr int Q_BYTES = TILE * D * 2;
+  static constexpr uint32_t TM_O = 256;      // accumulator columns (block b: + D b)
+  static constexpr uint32_t TM_P = 384;      // head size 64: P of block b: + 64 b (head size 128: over S)
+  static constexpr int CODE = PAIR ? 200 : 100;        // wait codes in the status word
+};
 
-enum { W2_ITEM = 201, W2_QFULL, W2_QFREE, W2_KVFULL, W2_KVFREE, W2_DESC, W2_SFULL, W2_PHALF, W2_PFULL, W2_OFULL, W2_OFREE, W2_LM,
-       W2_LMFREE, W2_LSE, W2_TFULL, W2_TFREE };
+enum { W2_DESC = 1, W2_ITEM, W2_QFULL, W2_QFREE, W2_KVFULL, W2_KVFREE, W2_SFULL, W2_PHALF, W2_PFULL, W2_OFULL, W2_OFREE, W2_LM,
+       W2_LMFREE, W2_LSE, W2_TFULL, W2_TFREE, W2_SREAD, W2_PV };
 
 enum { KIND_DONE = 0, KIND_FLASH = 1, KIND_SWEEP = 2 };
 struct __align__(16) Desc {
   int kind, c, hkv, len;       // chunk, kv-head, tokens of the chunk
   int h[2], t[2];              // FLASH: q-head and query tile of this CTA's block A / B (t < 0 or behind the chunk: no such
                                // tile, the rows are computed on zeros and not stored);  SWEEP: h[0] = pass
-  int n[2];                    // FLASH: key tiles the pair walks for block A / B; 0: block absent in both CTAs
+  int n[2];                    // FLASH: key tiles walked for block A / B; 0: block absent (in both CTAs of a pair)
 };
 
 struct __align__(16) Misc2 {
-  uint64_t q_full[NQ], q_free[NQ];           // q_full, kv_full: leader only, count the bytes of both CTAs
+  // of a pair: q_full, kv_full, p_*, o_free, t_free, s_read in the leader only; completions of MMAs in both CTAs
+  uint64_t q_full[NQ], q_free[NQ];
   uint64_t kv_full[NS], kv_free[NS];
-  uint64_t s_full[2], o_full[2], t_full[2];  // completion of MMAs, signalled in both CTAs
-  uint64_t p_half[2], p_full[2], o_free[2], t_free[2];   // leader only, arrivals of both CTAs
+  uint64_t s_full[2], o_full[2], t_full[2];
+  uint64_t p_half[2], p_full[2], o_free[2], t_free[2];
+  uint64_t s_read[2], pv_done[2];            // head size 64: S is in registers / P V of a tile has run
   uint64_t lm_full[2], lm_free[2];
   uint64_t d_full[NDESC], d_free[NDESC];
   uint64_t item_full, item_free;             // work items from the leader's producer to its peer's
@@ -66,21 +79,22 @@ struct __align__(16) Misc2 {
                                              // [column half][column] log-sum-exp of the window rows
 };
 
-constexpr int OFF_Q = 0;
-constexpr int OFF_RING = NQ * Q_BYTES;
-constexpr int OFF_MISC = OFF_RING + NS * HALF_BYTES;
-constexpr int SMEM2_BYTES = OFF_MISC + (int)sizeof(Misc2);
-static_assert(SMEM2_BYTES <= 232448, "shared memory of a CTA");
+template <int D>
+struct Off {
+  static constexpr int Q = 0, RING = NQ * Cfg<D>::Q_BYTES, MISC = RING + NS * STAGE_BYTES, TOTAL = MISC + (int)sizeof(Misc2);
+  static_assert(TOTAL <= 232448, "shared memory of a CTA");
+};
 
 __device__ __forceinline__ uint32_t full_par(uint32_t n) { return n & 1u; }           // n-th completion of a barrier
 __device__ __forceinline__ uint32_t free_par(uint32_t n) { return (n & 1u) ^ 1u; }    // completion n-1 (passes for n = 0)
 
 // ------------------------------------------------------------------ work decomposition
-// Groups = (chunk, kv-head).  A unit is what the four blocks of a pair take at a time:
+// Groups = (chunk, kv-head).  A unit is what the blocks (four of a pair, two of a single CTA) take at a time.  Pair:
 //   G % 4 == 0   one query tile of four q-heads (block A: heads 0, 1 of the four; B: heads 2, 3; one per CTA)
 //   G % 2 == 0   two adjacent tiles of two q-heads (A: lower tile; B: upper tile; one head per CTA)
 //   G odd        four adjacent tiles of one q-head (A: the lower two, B: the upper two; one per CTA; the lower tile of a
 //                block walks one fully masked key tile, 3 % of the tiles at 32 tiles a chunk)
+// single CTA: one tile of two q-heads, or (G odd) two adjacent tiles of one;
 // counted from the last tile of the chunk.  Item 0 of a group (the tail item) holds the units with window rows for all
 // q-heads, then the score sweep; the other items are one unit each, heaviest first.
 // Items are dealt out in batches of groups whose keys and values stay in L2 together, heaviest first over the whole
@@ -91,12 +105,14 @@ __device__ __forceinline__ uint32_t free_par(uint32_t n) { return (n & 1u) ^ 1u;
 struct Sched2 {
   int T, G, hpu, tpu, P, U, ntu, ipg, batch, hp, n_pass, wp;
 };
+template <int D>
 __device__ __forceinline__ Sched2 make_sched2(const PrefillParams& p) {
   Sched2 s;
   s.T = (p.L + TILE - 1) / TILE;
   s.G = p.Hq / p.Hkv;
-  s.hpu = s.G % 4 == 0 ? 4 : (s.G % 2 == 0 ? 2 : 1);      // q-heads and tiles of a unit
-  s.tpu = 4 / s.hpu;
+  constexpr int BLOCKS = 2 * Cfg<D>::NCTA;
+  s.hpu = s.G % BLOCKS == 0 ? BLOCKS : (s.G % 2 == 0 ? 2 : 1);      // q-heads and tiles of a unit
+  s.tpu = BLOCKS / s.hpu;
   s.P = s.G / s.hpu;
   s.U = (s.T + s.tpu - 1) / s.tpu;
   // tail units: those that can hold window rows (with per-chunk lengths the window of some chunk may straddle two
@@ -130,6 +146,7 @@ __device__ __forceinline__ int chunk_length(const PrefillParams& p, int c) {
   return len <= p.w ? p.w + 1 : len;
 }
 // blocks of sub-item `sub` (of the tail item, or 0)
+template <int D>
 __device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, int within, int sub, Desc& d) {
   const int x = within == 0 ? sub : s.ntu * s.P + within - 1;
   const int unit = x / s.P, set = x - unit * s.P;
@@ -138,7 +155,11 @@ __device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, 
 #pragma unroll
   for (int b = 0; b < 2; ++b) {
     int top;                                              // upper tile of the block over both CTAs
-    if (s.hpu == 4) { d.h[b] = h0 + 2 * b + rank; top = hi; d.t[b] = hi; }
+    if (!Cfg<D>::PAIR) {
+      d.h[b] = s.hpu == 2 ? h0 + b : h0;
+      top = s.hpu == 2 ? hi : hi - 1 + b;
+      d.t[b] = top;
+    } else if (s.hpu == 4) { d.h[b] = h0 + 2 * b + rank; top = hi; d.t[b] = hi; }
     else if (s.hpu == 2) { d.h[b] = h0 + rank; top = hi - 1 + b; d.t[b] = top; }
     else { d.h[b] = h0; top = hi - 2 + 2 * b; d.t[b] = top - 1 + rank; }
     d.n[b] = top < 0 ? 0 : top + 1;
@@ -155,12 +176,28 @@ struct Ctx2 {
 };
 
 // waits of the single-thread service roles (long pause between polls) / of the softmax and epilogue warps
-#define WAIT2(bar, par, code) mbar_wait_ns<SERVICE_BACKOFF_NS>((bar), (par), cx.abort_flag, cx.status, (code))
-#define WAIT2S(bar, par, code) mbar_wait((bar), (par), cx.abort_flag, cx.status, (code))
+#define WAIT2(bar, par, code) mbar_wait_ns<SERVICE_BACKOFF_NS>((bar), (par), cx.abort_flag, cx.status, Cfg<D>::CODE + (code))
+#define WAIT2S(bar, par, code) mbar_wait((bar), (par), cx.abort_flag, cx.status, Cfg<D>::CODE + (code))
 
 __device__ __forceinline__ void warp_arrive(uint64_t* bar) {
   __syncwarp();
   if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+// cluster address of the same barrier in CTA `rank` of a pair / of this CTA
+template <int D>
+__device__ __forceinline__ uint32_t in_cta(const void* p, uint32_t rank) {
+  if constexpr (Cfg<D>::PAIR) return map_to_cta(p, rank);
+  else return smem_u32(p);
+}
+template <int D>
+__device__ __forceinline__ void commit(uint64_t* bar) {           // in both CTAs of a pair
+  if constexpr (Cfg<D>::PAIR) mma_commit_pair(bar);
+  else mma_commit(bar);
+}
+template <int D>
+__device__ __forceinline__ void load_box(void* dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2, int c3) {
+  if constexpr (Cfg<D>::PAIR) tma_load_4d_pair(dst, tm, bar, c0, c1, c2, c3);
+  else tma_load_4d_addr(dst, tm, bar, c0, c1, c2, c3);
 }
 // one arrival of the warp on a barrier of the leader CTA; guards TMEM data, ordered by the tcgen05 fence
 __device__ __forceinline__ void warp_arrive_leader(uint32_t leader_addr) {
@@ -187,18 +224,21 @@ __device__ __forceinline__ void mbar_wait_cluster(uint64_t* bar, uint32_t parity
   }
 }
 
+template <int D>
 __device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool leader) {
+  constexpr int N = Cfg<D>::NCTA;
   for (int i = 0; i < NQ; ++i) { mbar_init(&mi.q_full[i], 1); mbar_init(&mi.q_free[i], 1); }
   for (int i = 0; i < NS; ++i) { mbar_init(&mi.kv_full[i], 1); mbar_init(&mi.kv_free[i], 1); }
   for (int b = 0; b < 2; ++b) {
     mbar_init(&mi.s_full[b], 1); mbar_init(&mi.o_full[b], 1); mbar_init(&mi.t_full[b], 1);
-    mbar_init(&mi.p_half[b], 8); mbar_init(&mi.p_full[b], 8);         // 4 softmax warps of the block in each CTA
-    mbar_init(&mi.o_free[b], 8); mbar_init(&mi.t_free[b], 16);        // epilogue warps / softmax warps of both CTAs
+    mbar_init(&mi.p_half[b], 4 * N); mbar_init(&mi.p_full[b], 4 * N); // 4 softmax warps of the block in each CTA
+    mbar_init(&mi.o_free[b], 4 * N); mbar_init(&mi.t_free[b], 8 * N); // epilogue warps / softmax warps of the CTAs
+    mbar_init(&mi.s_read[b], 4); mbar_init(&mi.pv_done[b], 1);
     mbar_init(&mi.lm_full[b], 4); mbar_init(&mi.lm_free[b], 4);
   }
   for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 13 : 12); }   // softmax and epilogue warps, issuer
   mbar_init(&mi.item_full, 1); mbar_init(&mi.item_free, 1);
-  mbar_init(&mi.lse_rdy, 8);
+  mbar_init(&mi.lse_rdy, 4 * N);
   mbar_init(&mi.mma_done, 1);
   mi.abort_flag = 0;
   mi.wait_kcycles = wait_kcycles;
@@ -206,6 +246,7 @@ __device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool
 }
 
 // consumers of the descriptor ring.  whole_warp: all 32 threads call.
+template <int D>
 __device__ __forceinline__ Desc next_desc(const Ctx2& cx, uint32_t& n, bool whole_warp) {
   Misc2& mi = *cx.mi;
   const int slot = n % NDESC;
@@ -219,21 +260,24 @@ __device__ __forceinline__ Desc next_desc(const Ctx2& cx, uint32_t& n, bool whol
 
 // ------------------------------------------------------------------ producer
 struct Prod { uint32_t kv = 0, q = 0, d = 0, item = 0; };
-__device__ __forceinline__ void publish(const Ctx2& cx, Prod& p, const Desc& d) {
+template <int D>
+__device__ __forceinline__ void publish(const Ctx2& cx, Prod& p, const Desc& d, bool signal = true) {
   Misc2& mi = *cx.mi;
   const int slot = p.d % NDESC;
   WAIT2(&mi.d_free[slot], free_par(p.d / NDESC), W2_DESC);
   mi.desc[slot] = d;
-  mbar_arrive(&mi.d_full[slot]);
+  if (signal) mbar_arrive(&mi.d_full[slot]);
   ++p.d;
 }
 // The leader's producer draws items from the queue and hands each to its peer's.
+template <int D>
 __device__ __forceinline__ int next_item(const Ctx2& cx, Prod& p, bool leader, int* counter, int n_items) {
   Misc2& mi = *cx.mi;
   int item;
   if (leader) {
     item = atomicAdd(counter, 1);
     if (item > n_items) item = n_items;
+    if (!Cfg<D>::PAIR) return item;
     WAIT2(&mi.item_free, free_par(p.item), W2_ITEM);      // the peer has read the previous one
     st_async_u32(map_to_cta(&mi.item, 1), static_cast<uint32_t>(item), map_to_cta(&mi.item_full, 1));
   } else {
@@ -247,15 +291,16 @@ __device__ __forceinline__ int next_item(const Ctx2& cx, Prod& p, bool leader, i
 }
 // expects a stage's bytes over both CTAs on the leader's barrier of the next ring stage; returns that barrier's address
 // for the copies and the stage's place; 0 once a wait has run out (no copy is issued into a ring that nobody drains)
+template <int D>
 __device__ __forceinline__ uint32_t ring_stage(const Ctx2& cx, Prod& p, bool leader, uint8_t** dst) {
   Misc2& mi = *cx.mi;
   if (*cx.abort_flag) return 0;
   const int s = p.kv % NS;
   if (!WAIT2(&mi.kv_free[s], free_par(p.kv / NS), W2_KVFREE)) return 0;
-  if (leader) mbar_arrive_expect_tx(&mi.kv_full[s], 2 * HALF_BYTES);
-  *dst = cx.ring + s * HALF_BYTES;
+  if (leader) mbar_arrive_expect_tx(&mi.kv_full[s], Cfg<D>::NCTA * STAGE_BYTES);
+  *dst = cx.ring + s * STAGE_BYTES;
   ++p.kv;
-  return map_to_cta(&mi.kv_full[s], 0);
+  return in_cta<D>(&mi.kv_full[s], 0);
 }
 
 }  // namespace
@@ -263,41 +308,44 @@ __device__ __forceinline__ uint32_t ring_stage(const Ctx2& cx, Prod& p, bool lea
 // ====================================================================================
 //                                   KERNEL
 // ====================================================================================
-// tensor maps: tm_q (box 64 d x 128 tokens), tm_kh (rotated keys, box 64 d x 64 tokens),
-// tm_k (rotated keys, box 64 d x 128 tokens), tm_v (box 64 d x 128 tokens), tm_o (store,
-// box 64 d x 128 tokens), tm_qw (box 64 d x wp tokens)
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT2, 1)
-prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kh,
-                    const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                    const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ CUtensorMap tm_qw,
-                    const __grid_constant__ PrefillParams prm) {
+// tensor maps (boxes of 64 d): tm_q (128 tokens), tm_kh (rotated keys, 64 tokens), tm_k (rotated keys, 128 tokens), tm_v
+// (128 tokens), tm_o (store, 128 tokens), tm_qw (wp tokens)
+template <int D>
+__global__ void __launch_bounds__(NT2, 1)
+prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kh,
+               const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+               const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ CUtensorMap tm_qw,
+               const __grid_constant__ PrefillParams prm) {
+  constexpr bool PAIR = Cfg<D>::PAIR;
+  constexpr int NCTA = Cfg<D>::NCTA, Q_BYTES = Cfg<D>::Q_BYTES;
+  constexpr uint32_t TM_O = Cfg<D>::TM_O, TM_P = Cfg<D>::TM_P;
   extern __shared__ __align__(1024) uint8_t smem[];
-  Misc2& mi = *reinterpret_cast<Misc2*>(smem + OFF_MISC);
+  Misc2& mi = *reinterpret_cast<Misc2*>(smem + Off<D>::MISC);
   Ctx2 cx;
   cx.mi = &mi;
-  cx.sQ = smem + OFF_Q;
-  cx.ring = smem + OFF_RING;
+  cx.sQ = smem + Off<D>::Q;
+  cx.ring = smem + Off<D>::RING;
   cx.abort_flag = &mi.abort_flag;
   cx.status = prm.status;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t rank = cluster_ctarank();
+  const uint32_t rank = PAIR ? cluster_ctarank() : 0;
   const bool leader = (rank == 0);
 
-  if (tid == 0) init_barriers2(mi, prm.wait_kcycles, leader);
-  if (warp == WARP_MMA) tmem_alloc_pair(&mi.tmem_base, 512);
+  if (tid == 0) init_barriers2<D>(mi, prm.wait_kcycles, leader);
+  if (warp == WARP_MMA) { if constexpr (PAIR) tmem_alloc_pair(&mi.tmem_base, 512); else tmem_alloc(&mi.tmem_base, 512); }
   tc_fence_before_sync();
   __syncthreads();
-  cluster_sync_all();                                    // both CTAs' barriers exist before any remote arrive
+  if constexpr (PAIR) cluster_sync_all();                // both CTAs' barriers exist before any remote arrive
   tc_fence_after_sync();
   cx.tmem = mi.tmem_base;
 
   if (warp >= WARP_PRODUCER) {
     setmaxnreg_dec<REGS_SERVICE>();
     if (warp == WARP_PRODUCER) {
-      // ================================================================ TMA producer (both CTAs)
+      // ================================================================ TMA producer (both CTAs of a pair)
       if (elect_one()) {
-        const Sched2 sch = make_sched2(prm);
+        const Sched2 sch = make_sched2<D>(prm);
         const int n_groups = prm.C * prm.Hkv, n_items = n_groups * sch.ipg;
         const int rows_half = sch.hp * sch.wp;           // sweep operand rows per CTA and pass (B operand half)
         tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kh); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
@@ -306,7 +354,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         // Once a wait has run out (abort flag) no new work is started: every role leaves its loops at the next
         // descriptor, this one also at the next tile, so that no copy is issued into a ring that nobody drains.
         while (!*cx.abort_flag) {
-          const int item = next_item(cx, p, leader, prm.counter, n_items);
+          const int item = next_item<D>(cx, p, leader, prm.counter, n_items);
           if (item >= n_items) break;
           int group, within;
           decode_item(sch, n_groups, item, group, within);
@@ -318,60 +366,66 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           const int nsub = within == 0 ? sch.ntu * sch.P : 1;
           for (int sub = 0; sub < nsub; ++sub) {
             d.kind = KIND_FLASH;
-            decode_unit(sch, rank, d.hkv, within, sub, d);
+            decode_unit<D>(sch, rank, d.hkv, within, sub, d);
             if (d.n[1] == 0) continue;                    // (n[0] <= n[1])
-            publish(cx, p, d);
+            publish<D>(cx, p, d);
             for (int b = 0; b < 2; ++b) {
               if (d.n[b] == 0) continue;
               const int qs = p.q % NQ;
               WAIT2(&mi.q_free[qs], free_par(p.q / NQ), W2_QFREE);
-              if (leader) mbar_arrive_expect_tx(&mi.q_full[qs], 2 * Q_BYTES);
-              const uint32_t bar = map_to_cta(&mi.q_full[qs], 0);
-              for (int a = 0; a < 2; ++a)
-                tma_load_4d_pair(cx.sQ + qs * Q_BYTES + a * 16384, &tm_q, bar, a * 64, d.h[b], d.t[b] * TILE, d.c);
+              if (leader) mbar_arrive_expect_tx(&mi.q_full[qs], NCTA * Q_BYTES);
+              const uint32_t bar = in_cta<D>(&mi.q_full[qs], 0);
+              for (int a = 0; a < Cfg<D>::ATOMS; ++a)
+                load_box<D>(cx.sQ + qs * Q_BYTES + a * 16384, &tm_q, bar, a * 64, d.h[b], d.t[b] * TILE, d.c);
               ++p.q;
             }
             for (int j = 0; j < d.n[1]; ++j) {
-              const uint32_t kbar = ring_stage(cx, p, leader, &dst);
-              if (kbar)
-                for (int a = 0; a < 2; ++a) tma_load_4d_pair(dst + a * 8192, &tm_kh, kbar, a * 64, d.hkv, j * TILE + (int)rank * 64, d.c);
-              const uint32_t vbar = ring_stage(cx, p, leader, &dst);
-              if (vbar) tma_load_4d_pair(dst, &tm_v, vbar, (int)rank * 64, d.hkv, j * TILE, d.c);
+              const uint32_t kbar = ring_stage<D>(cx, p, leader, &dst);
+              if (kbar) {
+                if constexpr (PAIR)
+                  for (int a = 0; a < 2; ++a) load_box<D>(dst + a * 8192, &tm_kh, kbar, a * 64, d.hkv, j * TILE + (int)rank * 64, d.c);
+                else load_box<D>(dst, &tm_k, kbar, 0, d.hkv, j * TILE, d.c);
+              }
+              const uint32_t vbar = ring_stage<D>(cx, p, leader, &dst);
+              if (vbar) load_box<D>(dst, &tm_v, vbar, (int)rank * 64, d.hkv, j * TILE, d.c);
             }
           }
           if (within == 0) {
             // ---- score sweep: window queries of hp heads per CTA and pass, then this CTA's key tiles.  A head's rows
             // in the operand are the wp tokens that end with the chunk (wp = w rounded up to 8: the first wp - w rows
             // are not window rows and are left out of the sums; a start before token 0 reads zeros)
-            const int n_steps = ((d.len + TILE - 1) / TILE + 1) / 2;
+            const int n_steps = ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
             for (int u = 0; u < sch.n_pass; ++u) {
               d.kind = KIND_SWEEP;
               d.h[0] = u;
-              publish(cx, p, d);
-              const int qs = p.q % NQ;
-              WAIT2(&mi.q_free[qs], free_par(p.q / NQ), W2_QFREE);
-              if (leader) mbar_arrive_expect_tx(&mi.q_full[qs], 2 * rows_half * D * 2);
-              const uint32_t bar = map_to_cta(&mi.q_full[qs], 0);
-              for (int i = 0; i < sch.hp; ++i) {
-                int g = u * 2 * sch.hp + (int)rank * sch.hp + i;
-                if (g >= sch.G) g = sch.G - 1;            // filler rows: loaded, never summed
-                for (int a = 0; a < 2; ++a)
-                  tma_load_4d_pair(cx.sQ + qs * Q_BYTES + a * 16384 + i * sch.wp * 128, &tm_qw, bar, a * 64,
-                                   d.hkv * sch.G + g, d.len - sch.wp, d.c);
+              publish<D>(cx, p, d);
+              for (int b = 0; b < 3 - NCTA; ++b) {        // a pair's CTAs load a column half each, a single CTA both
+                const int qs = p.q % NQ;
+                WAIT2(&mi.q_free[qs], free_par(p.q / NQ), W2_QFREE);
+                if (leader) mbar_arrive_expect_tx(&mi.q_full[qs], NCTA * rows_half * D * 2);
+                const uint32_t bar = in_cta<D>(&mi.q_full[qs], 0);
+                for (int i = 0; i < sch.hp; ++i) {
+                  int g = u * 2 * sch.hp + ((int)rank + b) * sch.hp + i;
+                  if (g >= sch.G) g = sch.G - 1;          // filler rows: loaded, never summed
+                  for (int a = 0; a < Cfg<D>::ATOMS; ++a)
+                    load_box<D>(cx.sQ + qs * Q_BYTES + a * 16384 + i * sch.wp * 128, &tm_qw, bar, a * 64, d.hkv * sch.G + g,
+                                d.len - sch.wp, d.c);
+                }
+                ++p.q;
               }
-              ++p.q;
-              // a full key tile takes two consecutive stages that start on an even one: everything uses stages in twos
+              // a full key tile takes ATOMS consecutive stages (of a pair: two that start on an even one, everything uses
+              // stages in twos)
               for (int jj = 0; jj < n_steps; ++jj)
-                for (int a = 0; a < 2; ++a) {
-                  const uint32_t kbar = ring_stage(cx, p, leader, &dst);
-                  if (kbar) tma_load_4d_pair(dst, &tm_k, kbar, a * 64, d.hkv, (2 * jj + (int)rank) * TILE, d.c);
+                for (int a = 0; a < Cfg<D>::ATOMS; ++a) {
+                  const uint32_t kbar = ring_stage<D>(cx, p, leader, &dst);
+                  if (kbar) load_box<D>(dst, &tm_k, kbar, a * 64, d.hkv, (NCTA * jj + (int)rank) * TILE, d.c);
                 }
             }
           }
         }
         Desc d;
         d.kind = KIND_DONE; d.c = d.hkv = d.len = 0;
-        publish(cx, p, d);
+        publish<D>(cx, p, d, PAIR || prm.skip_final_publication == 0);
         // Every copy issued must have landed before a CTA may exit.  In a run without a timed-out wait that follows
         // from the last uses of the rings having been consumed (the teardown below waits for every tensor-core
         // operation).  After an abort nothing is consumed any more: the leader, whose barriers count the bytes of both
@@ -387,104 +441,128 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       __syncwarp();
     } else if (warp == WARP_MMA && leader) {
-      // ================================================================ issuer (leader CTA)
-      // Per key tile and block: O += P V as soon as P is there (in two halves), then S of the block's next tile, which
-      // overwrites P: the pipe runs them in order.  The next unit's first S follows the last tile without a gap.
+      // ================================================================ issuer (of a pair: leader CTA)
       if (elect_one()) {
-        const Sched2 sch = make_sched2(prm);
-        constexpr uint32_t idesc_qk = make_idesc_bf16_f32(256, TILE, false, false), idesc_pv = make_idesc_bf16_f32(256, D, false, true);
+        const Sched2 sch = make_sched2<D>(prm);
+        constexpr uint32_t idesc_qk = make_idesc_bf16_f32(TILE * NCTA, TILE, false, false), idesc_pv = make_idesc_bf16_f32(TILE * NCTA, D, false, true);
         const int rows_half = sch.hp * sch.wp;
-        const uint32_t idesc_sw = make_idesc_bf16_f32(256, 2 * rows_half, false, false);
+        const uint32_t idesc_sw = make_idesc_bf16_f32(TILE * NCTA, PAIR ? 2 * rows_half : (rows_half + 15) & ~15, false, false);
         const uint32_t ring_u32 = smem_u32(cx.ring), q_u32 = smem_u32(cx.sQ);
         uint32_t nd = 0, kv = 0, nq = 0, np[2] = {0, 0}, no[2] = {0, 0}, nt = 0;
-        uint32_t qa[2];                                          // query operands of the two blocks in work
-        Desc d = next_desc(cx, nd, false);
-        bool primed = false;
-        auto issue_first_qk = [&](int b, uint32_t k_smem) {
+        uint32_t qa[2] = {0, 0};                                          // query operands of the two blocks in work
+        auto wait_kv = [&](uint32_t i) {
+          WAIT2S(&mi.kv_full[i % NS], full_par(i / NS), W2_KVFULL);
+          return ring_u32 + (i % NS) * STAGE_BYTES;
+        };
+        auto qk = [&](int b, uint32_t k_smem) {
+          tc_fence_after_sync();
+          if constexpr (PAIR) mma_ss_pair_k128<true>(cx.tmem + b * 128, qa[b], k_smem, idesc_qk);
+          else mma_ss_k64(cx.tmem + b * 128, qa[b], k_smem, idesc_qk);
+          commit<D>(&mi.s_full[b]);
+        };
+        auto first_qk = [&](int b, uint32_t k_smem) {
           qa[b] = q_u32 + (nq % NQ) * Q_BYTES;
           WAIT2S(&mi.q_full[nq % NQ], full_par(nq / NQ), W2_QFULL);
           ++nq;
-          tc_fence_after_sync();
-          mma_ss_pair_k128<true>(cx.tmem + b * 128, qa[b], k_smem, idesc_qk);
-          mma_commit_pair(&mi.s_full[b]);
+          qk(b, k_smem);
         };
+        // O += P V of a tile, in two halves as P arrives
+        auto pv = [&](int b, uint32_t v_smem, bool first, bool last) {
+          const uint32_t tO = cx.tmem + TM_O + b * D, tP = PAIR ? cx.tmem + b * 128 : cx.tmem + TM_P + b * 64;
+          if (first) { WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE); ++no[b]; }       // accumulator of the previous block read out
+          WAIT2S(&mi.p_half[b], full_par(np[b]), W2_PHALF);                                // keys 0..63 of P
+          tc_fence_after_sync();
+          mma_ts_k64<PAIR>(tO, tP, v_smem, idesc_pv, !first);
+          WAIT2S(&mi.p_full[b], full_par(np[b]), W2_PFULL);
+          ++np[b];
+          tc_fence_after_sync();
+          mma_ts_k64<PAIR>(tO, tP + 32, v_smem + 8192, idesc_pv, true);
+          if (!PAIR) mma_commit(&mi.pv_done[b]);
+          if (last) commit<D>(&mi.o_full[b]);
+        };
+        Desc d = next_desc<D>(cx, nd, false);
+        bool primed = false;                                     // first S of the unit already issued
         while (d.kind != KIND_DONE) {
           if (d.kind == KIND_FLASH) {
             const int n0 = d.n[0], n = d.n[1];
             if (!primed) {
-              const int st = kv % NS;
-              WAIT2S(&mi.kv_full[st], full_par(kv / NS), W2_KVFULL);
-              for (int b = 0; b < 2; ++b) if (d.n[b] > 0) issue_first_qk(b, ring_u32 + st * HALF_BYTES);
-              mma_commit_pair(&mi.kv_free[st]);
+              const uint32_t k_u32 = wait_kv(kv);
+              for (int b = 0; b < 2; ++b) if (d.n[b] > 0) first_qk(b, k_u32);
+              commit<D>(&mi.kv_free[kv % NS]);
               ++kv;
             }
             Desc nx;
             nx.kind = KIND_DONE; nx.n[0] = nx.n[1] = 0;
-            for (int j = 0; j < n; ++j) {
-              const int sv = kv % NS, sk = (kv + 1) % NS;
-              WAIT2S(&mi.kv_full[sv], full_par(kv / NS), W2_KVFULL);
-              const uint32_t v_u32 = ring_u32 + sv * HALF_BYTES, k_u32 = ring_u32 + sk * HALF_BYTES;
+            // the next unit's first S follows the last tile without a gap
+            for (int j = 0; j < n; ++j) {                        // kv: V of tile j; kv + 1: the next K
               bool more = j + 1 < n;
-#pragma unroll
-              for (int b = 0; b < 2; ++b) {
-                const uint32_t tS = cx.tmem + b * 128, tO = cx.tmem + TM_O + b * 128;
-                const int nb = b ? n : n0;
-                if (j < nb) {
-                  if (j == 0) { WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE); ++no[b]; }   // accumulator of the previous block read out
-                  WAIT2S(&mi.p_half[b], full_par(np[b]), W2_PHALF);                            // keys 0..63 of P
-                  tc_fence_after_sync();
-                  mma_ts_k64<true>(tO, tS, v_u32, idesc_pv, j > 0);
-                  WAIT2S(&mi.p_full[b], full_par(np[b]), W2_PFULL);
-                  ++np[b];
-                  tc_fence_after_sync();
-                  mma_ts_k64<true>(tO, tS + 32, v_u32 + 8192, idesc_pv, true);
-                  if (j == nb - 1) mma_commit_pair(&mi.o_full[b]);
-                }
-                if (b == 0) {
-                  if (j + 1 == n) { nx = next_desc(cx, nd, false); more = nx.kind == KIND_FLASH; }
-                  if (more) WAIT2S(&mi.kv_full[sk], full_par((kv + 1) / NS), W2_KVFULL);
-                }
-                if (j + 1 < nb) {
-                  tc_fence_after_sync();
-                  mma_ss_pair_k128<true>(tS, qa[b], k_u32, idesc_qk);
-                  mma_commit_pair(&mi.s_full[b]);
-                } else if (j + 1 == n && more && nx.n[b] > 0) {
-                  issue_first_qk(b, k_u32);
-                }
+              uint32_t k_u32 = 0;
+              auto look_ahead = [&]() {
+                if (j + 1 == n) { nx = next_desc<D>(cx, nd, false); more = nx.kind == KIND_FLASH; }
+                if (more) k_u32 = wait_kv(kv + 1);
+              };
+              auto next_s = [&](int b, int nb) {
+                if (j + 1 < nb) qk(b, k_u32);
+                else if (j + 1 == n && more && nx.n[b] > 0) first_qk(b, k_u32);
+              };
+              if constexpr (PAIR) {
+                // per block: P V, then the next S over P; the pipe runs them in order
+                const uint32_t v_u32 = wait_kv(kv);
+                if (j < n0) pv(0, v_u32, j == 0, j == n0 - 1);
+                look_ahead();
+                next_s(0, n0);
+                pv(1, v_u32, j == 0, j == n - 1);
+                next_s(1, n);
+              } else {
+                // next S as soon as the present one is in registers, then P V
+                look_ahead();
+                if (j < n0) WAIT2S(&mi.s_read[0], full_par(np[0]), W2_SREAD);
+                next_s(0, n0);
+                WAIT2S(&mi.s_read[1], full_par(np[1]), W2_SREAD);
+                next_s(1, n);
+                if (more) commit<D>(&mi.kv_free[(kv + 1) % NS]);
+                const uint32_t v_u32 = wait_kv(kv);
+                if (j < n0) pv(0, v_u32, j == 0, j == n0 - 1);
+                pv(1, v_u32, j == 0, j == n - 1);
               }
-              mma_commit_pair(&mi.kv_free[sv]);
-              ++kv;
-              if (more) { mma_commit_pair(&mi.kv_free[sk]); ++kv; }
+              commit<D>(&mi.kv_free[kv % NS]);
+              if (PAIR && more) commit<D>(&mi.kv_free[(kv + 1) % NS]);
+              kv += more ? 2 : 1;
             }
             primed = nx.kind == KIND_FLASH;
             d = nx;
           } else {
             // ---- score sweep, one pass: S^T = K_j Qw^T.  Its two [128 keys x 256 rows] buffers overlay all of TMEM:
             // every S / P buffer is consumed and the accumulators have been read out once o_free completes.
-            const int n_steps = ((d.len + TILE - 1) / TILE + 1) / 2;
+            const int n_steps = ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
             for (int b = 0; b < 2; ++b) WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE);
-            const uint32_t qw = q_u32 + (nq % NQ) * Q_BYTES;
-            WAIT2S(&mi.q_full[nq % NQ], full_par(nq / NQ), W2_QFULL);
-            ++nq;
+            for (int b = 0; b < 3 - NCTA; ++b) {
+              qa[b] = q_u32 + (nq % NQ) * Q_BYTES;
+              WAIT2S(&mi.q_full[nq % NQ], full_par(nq / NQ), W2_QFULL);
+              ++nq;
+            }
             for (int jj = 0; jj < n_steps; ++jj, ++nt) {
-              const int e = nt & 1, st = kv % NS;
+              const int e = nt & 1;
               WAIT2S(&mi.t_free[e], free_par(nt >> 1), W2_TFREE);
-              WAIT2S(&mi.kv_full[st], full_par(kv / NS), W2_KVFULL);
-              WAIT2S(&mi.kv_full[st + 1], full_par((kv + 1) / NS), W2_KVFULL);
-              tc_fence_after_sync();
-              mma_ss_pair_k128<false>(cx.tmem + e * 256, ring_u32 + st * HALF_BYTES, qw, idesc_sw);
-              mma_commit_pair(&mi.t_full[e]);
-              mma_commit_pair(&mi.kv_free[st]);
-              mma_commit_pair(&mi.kv_free[st + 1]);
-              kv += 2;
+              const uint32_t k_u32 = wait_kv(kv);
+              if constexpr (PAIR) {
+                wait_kv(kv + 1);
+                tc_fence_after_sync();
+                mma_ss_pair_k128<false>(cx.tmem + e * 256, k_u32, qa[0], idesc_sw);
+              } else {
+                tc_fence_after_sync();
+                for (int b = 0; b < 2; ++b) mma_ss_k64(cx.tmem + e * 256 + b * 128, k_u32, qa[b], idesc_sw);
+              }
+              commit<D>(&mi.t_full[e]);
+              for (int a = 0; a < Cfg<D>::ATOMS; ++a, ++kv) commit<D>(&mi.kv_free[kv % NS]);
             }
             // what follows overwrites the sweep buffers: wait until both were read
             WAIT2S(&mi.t_free[nt & 1], free_par(nt >> 1), W2_TFREE);
             WAIT2S(&mi.t_free[(nt + 1) & 1], free_par((nt + 1) >> 1), W2_TFREE);
-            d = next_desc(cx, nd, false);
+            d = next_desc<D>(cx, nd, false);
           }
         }
-        mma_commit_pair(&mi.mma_done);                           // teardown waits for everything this thread issued
+        commit<D>(&mi.mma_done);                                 // teardown waits for everything this thread issued
       }
       __syncwarp();
     }
@@ -492,23 +570,23 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // ================================================================ epilogue: normalise, stage bf16 rows in the block's
     // (now idle) query slot, TMA store
     setmaxnreg_dec<REGS_EPI>();
-    const Sched2 sch = make_sched2(prm);
+    const Sched2 sch = make_sched2<D>(prm);
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
     uint32_t nd = 0, nq = 0, no[2] = {0, 0};
     while (true) {
-      const Desc d = next_desc(cx, nd, true);
+      const Desc d = next_desc<D>(cx, nd, true);
       if (d.kind == KIND_DONE) break;
       if (d.kind == KIND_SWEEP) {
         if (d.h[0] == 0) {                                       // the window rows' log-sum-exp of this CTA's blocks is in memory
           __threadfence();
           __syncwarp();
           if (lane == 0) {
-            mbar_arrive_cluster(map_to_cta(&mi.lse_rdy, 0));
-            mbar_arrive_cluster(map_to_cta(&mi.lse_rdy, 1));
+            mbar_arrive_cluster(in_cta<D>(&mi.lse_rdy, 0));
+            if (PAIR) mbar_arrive_cluster(in_cta<D>(&mi.lse_rdy, 1));
           }
         }
-        ++nq;
+        nq += 3 - NCTA;
         continue;
       }
 #pragma unroll 1
@@ -527,7 +605,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         tc_fence_after_sync();
         const bool in_chunk = token >= 0 && token < d.len;       // rows behind the end of the chunk are written as zeros
         const float inv_l = in_chunk ? 1.0f / l_run : 0.0f;
-        const uint32_t tO = cx.tmem + TM_O + b * 128 + lane_sel;
+        const uint32_t tO = cx.tmem + TM_O + b * D + lane_sel;
 #pragma unroll 1
         for (int q = 0; q < D / 32; ++q) {
           uint32_t o[32];
@@ -544,7 +622,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             *reinterpret_cast<uint4*>(myQ + (col / 64) * 16384 + sw128_offset(r, (col % 64) / 8)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
         }
-        warp_arrive_leader(map_to_cta(&mi.o_free[b], 0));
+        warp_arrive_leader(in_cta<D>(&mi.o_free[b], 0));
         if (in_chunk) {
           const float lse2 = m_used + log2f(l_run);
           const size_t row = (size_t)d.c * prm.Hq + h;
@@ -556,7 +634,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         named_barrier_sync(1, 128);
         if (r == 0) {
           if (t >= 0 && t * TILE < prm.L) {
-            for (int a = 0; a < 2; ++a) tma_store_4d(&tm_o, myQ + a * 16384, a * 64, h, t * TILE, d.c);
+            for (int a = 0; a < Cfg<D>::ATOMS; ++a) tma_store_4d(&tm_o, myQ + a * 16384, a * 64, h, t * TILE, d.c);
             tma_store_commit();
             tma_store_wait_read();
           }
@@ -568,23 +646,30 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   } else {
     // ================================================================ softmax
     setmaxnreg_inc<REGS_SOFTMAX>();
-    const Sched2 sch = make_sched2(prm);
+    const Sched2 sch = make_sched2<D>(prm);
     const int b = warp >> 2;
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tS = cx.tmem + b * 128 + lane_sel, tO = cx.tmem + TM_O + b * 128 + lane_sel;
+    const uint32_t tS = cx.tmem + b * 128 + lane_sel, tO = cx.tmem + TM_O + b * D + lane_sel;
+    const uint32_t tP = PAIR ? tS : cx.tmem + TM_P + b * 64 + lane_sel;
     const float scale_log2 = prm.scale_log2;
     struct Hooks {
-      uint32_t p_half, p_full;                                   // barriers of the leader CTA
-      __device__ __forceinline__ void on_read() const {}
-      __device__ __forceinline__ void before_rescale() const {}  // S of this tile was issued after P V of the tile before
-      __device__ __forceinline__ void before_p() const {}        // P overwrites S, which is in registers
+      const Ctx2& cx;
+      uint32_t p_half, p_full, s_read;                           // barriers (of the leader CTA)
+      uint64_t* pv_done;
+      uint32_t tiles;                                            // tiles of this block before the present one
+      __device__ __forceinline__ void on_read() const { if (!PAIR) warp_arrive_leader(s_read); }
+      // pair: S of this tile was issued after P V of the tile before, and P overwrites S, which is in registers
+      __device__ __forceinline__ void before_p() const {
+        if (!PAIR && tiles > 0) { WAIT2S(pv_done, full_par(tiles - 1), W2_PV); tc_fence_after_sync(); }
+      }
+      __device__ __forceinline__ void before_rescale() const { before_p(); }
       __device__ __forceinline__ void on_half() const { warp_arrive_leader(p_half); }
       __device__ __forceinline__ void on_full() const { warp_arrive_leader(p_full); }
-    } hk = {map_to_cta(&mi.p_half[b], 0), map_to_cta(&mi.p_full[b], 0)};
+    } hk = {cx, in_cta<D>(&mi.p_half[b], 0), in_cta<D>(&mi.p_full[b], 0), in_cta<D>(&mi.s_read[b], 0), &mi.pv_done[b], 0};
     uint32_t nd = 0, n_s = 0, n_blk = 0, nq = 0, nt = 0, n_lse = 0;
     while (true) {
-      const Desc d = next_desc(cx, nd, true);
+      const Desc d = next_desc<D>(cx, nd, true);
       if (d.kind == KIND_DONE) break;
       if (d.kind == KIND_FLASH) {
         nq += d.n[0] > 0 ? 2 : 1;
@@ -596,8 +681,9 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           WAIT2S(&mi.s_full[b], full_par(n_s), W2_SFULL);
           ++n_s;
           tc_fence_after_sync();
-          if (j > 0 && j < t) softmax_tile<D, false>(tS, tS, tO, TILE, false, scale_log2, st, hk);
-          else softmax_tile<D, true>(tS, tS, tO, (t - j) * TILE + r + 1, j == 0, scale_log2, st, hk);   // causal: keys <= token
+          if (j > 0 && j < t) softmax_tile<D, false>(tS, tP, tO, TILE, false, scale_log2, st, hk);
+          else softmax_tile<D, true>(tS, tP, tO, (t - j) * TILE + r + 1, j == 0, scale_log2, st, hk);   // causal: keys <= token
+          ++hk.tiles;
         }
         WAIT2S(&mi.lm_free[b], free_par(n_blk), W2_LMFREE);
         ++n_blk;
@@ -625,16 +711,16 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           lse_cols[r] = x;
         }
         named_barrier_sync(3, 256);
-        const int n_steps = ((d.len + TILE - 1) / TILE + 1) / 2;
+        const int n_steps = ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
         const int w0 = d.len - prm.w, pad = sch.wp - prm.w;      // first window token of this chunk
         float* const xch = &mi.lm[0][0][0];                      // [buffer][key]
-        const uint32_t t_free0 = map_to_cta(&mi.t_free[0], 0), t_free1 = map_to_cta(&mi.t_free[1], 0);
+        const uint32_t t_free0 = in_cta<D>(&mi.t_free[0], 0), t_free1 = in_cta<D>(&mi.t_free[1], 0);
         for (int jj = 0; jj < n_steps; ++jj, ++nt) {
           const int e = nt & 1;
           WAIT2S(&mi.t_full[e], full_par(nt >> 1), W2_TFULL);
           tc_fence_after_sync();
-          const int key0 = (2 * jj + (int)rank) * TILE, key = key0 + r;
-          const uint32_t tT = cx.tmem + e * 256 + b * rows_half + lane_sel;
+          const int key0 = (NCTA * jj + (int)rank) * TILE, key = key0 + r;
+          const uint32_t tT = cx.tmem + e * 256 + b * (PAIR ? rows_half : 128) + lane_sel;
           float part = 0.0f;
           int col = 0;
           if (key0 + TILE - 1 <= w0) {                           // every window row sees every key of the tile
@@ -684,40 +770,56 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           }
         }
         named_barrier_sync(3, 256);                              // everyone is past the exchange buffer
-        if (tid == 0) mbar_arrive(&mi.q_free[nq % NQ]);          // the window queries were read by MMAs that have completed
-        ++nq;
+        if (tid == 0)                                            // the window queries were read by MMAs that have completed
+          for (int i = 0; i < 3 - NCTA; ++i) mbar_arrive(&mi.q_free[(nq + i) % NQ]);
+        nq += 3 - NCTA;
       }
     }
   }
 
-  // ---- teardown: no CTA may exit while its peer can still signal it or read its shared memory
+  // ---- teardown: no CTA of a pair may exit while its peer can still signal it or read its shared memory
   tc_fence_before_sync();
   __syncthreads();
-  cluster_sync_all();
+  if constexpr (PAIR) cluster_sync_all();
   if (warp == WARP_MMA) {
     // no tensor-core operation may still be running when its accumulators are freed: the issuer ended with a
-    // commit to mma_done (an arrival in both CTAs).  Immediate in a clean run; after an abort this is what
+    // commit to mma_done (an arrival in both CTAs of a pair).  Immediate in a clean run; after an abort this is what
     // makes the exit safe.  The wait ignores the abort flag and is bounded.
     mbar_wait_drain(&mi.mma_done, 0, cx.abort_flag);
     tc_fence_after_sync();
-    tmem_dealloc_pair(cx.tmem, 512);
+    if constexpr (PAIR) tmem_dealloc_pair(cx.tmem, 512); else tmem_dealloc(cx.tmem, 512);
   }
 }
 
 // ====================================================================================
 //                                   host launcher
 // ====================================================================================
-// maps: 0 q (box 64 x 128 tokens), 1 rotated keys (64 x 128), 2 v (64 x 128), 3 o (store), 4 q with a
-// wp-token box, 5 rotated keys with a 64-token box.  The grid is a whole number of CTA pairs.
-cudaError_t launch_prefill_pair(const CUtensorMap* maps, const PrefillParams& prm, int sm_count, cudaStream_t st) {
+template <int D>
+static cudaError_t launch_prefill_t(const CUtensorMap* maps, const PrefillParams& prm, int sm_count, cudaStream_t st) {
   // the opt-in to large dynamic shared memory is a per-device attribute of the function: set it on every call
   // (a host-side call of a few hundred nanoseconds) rather than remember which devices have it
-  if (cudaError_t e = cudaFuncSetAttribute(prefill_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES); e != cudaSuccess) return e;
-  const int grid = (sm_count / 2) * 2;
-  if (grid < 2) return cudaErrorInvalidConfiguration;
+  if (cudaError_t e = cudaFuncSetAttribute(prefill_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Off<D>::TOTAL); e != cudaSuccess) return e;
+  constexpr int NCTA = Cfg<D>::NCTA;
+  const int grid = sm_count / NCTA * NCTA;               // one CTA per SM, a whole number of pairs
+  if (grid < 1) return cudaErrorInvalidConfiguration;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = NCTA; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(NT2);
+  cfg.dynamicSmemBytes = Off<D>::TOTAL;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   note_launch();
-  prefill_pair_kernel<<<grid, NT2, SMEM2_BYTES, st>>>(maps[0], maps[5], maps[1], maps[2], maps[3], maps[4], prm);
-  return cudaGetLastError();
+  return cudaLaunchKernelEx(&cfg, prefill_kernel<D>, maps[0], maps[5], maps[1], maps[2], maps[3], maps[4], prm);
+}
+
+// maps: 0 q (box 64 x 128 tokens), 1 rotated keys (64 x 128), 2 v (64 x 128), 3 o (store), 4 q with a
+// wp-token box, 5 rotated keys with a 64-token box
+cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int d, int sm_count, cudaStream_t st) {
+  return d == 128 ? launch_prefill_t<128>(maps, prm, sm_count, st) : launch_prefill_t<64>(maps, prm, sm_count, st);
 }
 
 }  // namespace pc
