@@ -428,14 +428,15 @@ ParallelPlan parallel_plan(int B, int w, int Hq, int Hkv, int d, int Nk, int sm_
   // few query rows (at most 32 per kv-head: the line is drawn where the transposed kernel stops winning, figures in
   // pc_decode.cu): CTAs per (sequence, kv-head), 0: another kernel.  Least time by a model in microseconds - rounds of the
   // grid (two CTAs per SM) x (about 6 for prologue, pipeline fill and merge + a tile at the CTA's share of
-  // the memory bandwidth, no faster than the 0.6 that the chain through the tensor cores takes)
+  // the memory bandwidth, no faster than the 50 GB/s that its three stages in flight give it: one sequence over 16401
+  // entries measured 26.7 us with 8 splits per head)
   p.few_split = 0;
   if (G * w <= 32) {
     const double slots = 2.0 * sm_count, tile_us = 512.0 * d / 6.5e6;
     double least = -1.0;
     for (int s = 1; s <= 16 && s <= p.n_cache_tiles + 1; s *= 2) {
       const double ctas = (double)base * s, rounds = std::ceil(ctas / slots), active = ctas < slots ? ctas : slots;
-      const double per_tile = tile_us * active > 0.6 ? tile_us * active : 0.6;
+      const double per_tile = tile_us * active > 512.0 * d / 5e4 ? tile_us * active : 512.0 * d / 5e4;
       const double cost = rounds * (6.0 + per_tile * std::ceil((p.n_cache_tiles + 1.0) / s));
       if (least < 0.0 || cost < least) { least = cost; p.few_split = s; }
     }
