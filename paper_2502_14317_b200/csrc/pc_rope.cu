@@ -11,8 +11,9 @@ namespace pc {
 // tab: (cos, sin) per (position, pair), fp64.  tab_hi / tab_lo: fp32 heads / tails of the same values, one float4
 // per two consecutive pairs (cos_2i, cos_2i+1, sin_2i, sin_2i+1); value = head + tail to 2^-48.
 __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict__ tab_hi, float4* __restrict__ tab_lo, int n_pos,
-                                  int half, double theta, int pos0) {
+                                  int half, double theta, int pos0, int* __restrict__ counter) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;      // one thread per two pairs
+  if (i == 0 && counter != nullptr) *counter = 0;           // work queue of the attention kernel that follows
   if (i >= n_pos * (half / 2)) return;
   const int p = i / (half / 2), t = 2 * (i % (half / 2));
   double c[2], s[2];
@@ -30,10 +31,11 @@ __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict_
   }
 }
 
-void launch_rope_table(double2* tab, float4* tab_hi, float4* tab_lo, int n_pos, int d, double theta, int pos0, cudaStream_t st) {
+void launch_rope_table(double2* tab, float4* tab_hi, float4* tab_lo, int n_pos, int d, double theta, int pos0, int* counter,
+                       cudaStream_t st) {
   const int n = n_pos * (d / 4);
   note_launch();
-  rope_table_kernel<<<(n + 255) / 256, 256, 0, st>>>(tab, tab_hi, tab_lo, n_pos, d / 2, theta, pos0);
+  rope_table_kernel<<<(n + 255) / 256, 256, 0, st>>>(tab, tab_hi, tab_lo, n_pos, d / 2, theta, pos0, counter);
 }
 
 // y[c,p,h,:] = bf16( RoPE(x[c,p,h,:], position p) ).  One warp owns one position: a lane holds 8 consecutive
@@ -45,10 +47,26 @@ void launch_rope_table(double2* tab, float4* tab_hi, float4* tab_lo, int n_pos, 
 // sixteen outputs of an undecided lane go to sixteen lanes, one each, and are patched into the row after the
 // vector store.  (Handling them in the lane that found them would make a third of the warp's passes wait for one
 // lane's slow path.)
-__global__ void __launch_bounds__(256, 4) rope_rows_kernel(const uint16_t* __restrict__ x, long long s_chunk, long long s_tok,
-                                                           long long s_head, uint16_t* __restrict__ y,
+//
+// One launch takes one or two tensors of the same chunks and positions (keys and queries): grid.y first deals out the slices of
+// the chunks of the first tensor, then those of the second.
+struct RopeTensor {
+  const uint16_t* x;
+  uint16_t* y;
+  long long s_chunk, s_tok, s_head;                         // element strides of x; y is contiguous
+  int H, ny, nz;                                            // heads; slices of the chunks; parts of the head passes
+};
+__global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant__ RopeTensor ta, const __grid_constant__ RopeTensor tb,
                                                            const float4* __restrict__ tab_hi, const float4* __restrict__ tab_lo,
-                                                           const double2* __restrict__ tab, int C, int L, int H, int d) {
+                                                           const double2* __restrict__ tab, int C, int L, int d) {
+  const bool second_tensor = (int)blockIdx.y >= ta.ny;      // the same for the whole block
+  const uint16_t* __restrict__ const x = second_tensor ? tb.x : ta.x;
+  uint16_t* __restrict__ const y = second_tensor ? tb.y : ta.y;
+  const long long s_chunk = second_tensor ? tb.s_chunk : ta.s_chunk, s_tok = second_tensor ? tb.s_tok : ta.s_tok,
+                  s_head = second_tensor ? tb.s_head : ta.s_head;
+  const int H = second_tensor ? tb.H : ta.H, ny = second_tensor ? tb.ny : ta.ny, zs = second_tensor ? tb.nz : ta.nz;
+  const int slice = second_tensor ? (int)blockIdx.y - ta.ny : (int)blockIdx.y;
+  if ((int)blockIdx.z >= zs) return;
   const int half = d / 2;
   const int groups = half / 8;                              // 16-byte groups per half row (4 or 8)
   const int lane = threadIdx.x & 31;
@@ -62,12 +80,12 @@ __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const uint16_t* __res
   float4 hi[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) hi[i] = __ldg(hi_row + g * 4 + i);
-  const int zs = gridDim.z;                                 // small inputs: the head passes are dealt out over grid.z
+  // small inputs: the head passes are dealt out over grid.z (zs parts)
   const long long step_src = (long long)h_step * zs * s_head;
   const size_t step_dst = (size_t)h_step * zs * d;
   const int n_pass = (H + h_step - 1) / h_step;
   const int h_mine = h_first + (int)blockIdx.z * h_step;    // this thread's head in its first pass
-  for (int c = blockIdx.y; c < C; c += gridDim.y) {
+  for (int c = slice; c < C; c += ny) {
     const uint16_t* src = x + (long long)c * s_chunk + (long long)p * s_tok + (long long)h_mine * s_head + g * 8;
     uint16_t* const dst_tok = y + ((size_t)c * L + p) * H * d;
     uint16_t* dst = dst_tok + (size_t)h_mine * d + g * 8;
@@ -125,21 +143,31 @@ __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const uint16_t* __res
   }
 }
 
-void launch_rope_rows(const void* x, const long long x_stride[3], void* y, const double2* tab, const float4* tab_hi,
-                      const float4* tab_lo, int C, int L, int H, int d, cudaStream_t st) {
+static RopeTensor rope_tensor(const RopeRows& r, int C, int L, int d) {
+  RopeTensor t;
+  t.x = (const uint16_t*)r.x; t.y = (uint16_t*)r.y;
+  t.s_chunk = r.stride[0]; t.s_tok = r.stride[1]; t.s_head = r.stride[2];
+  t.H = r.H;
   const int bx = (L + 7) / 8;                               // 8 positions per block
   // a slice of the chunks per block: the table entries are reused over the slice; enough blocks to fill the GPU
-  int ny = (4736 + bx - 1) / bx;
-  ny = ny < 1 ? 1 : (ny > C ? C : ny);
+  t.ny = (4736 + bx - 1) / bx;
+  t.ny = t.ny < 1 ? 1 : (t.ny > C ? C : t.ny);
   // a few positions and chunks only (the query window of one sequence): the passes over the heads, which a warp
   // would otherwise walk one after the other, become blocks of their own
-  const int n_pass = (H + 32 / (d / 16) - 1) / (32 / (d / 16));
-  int nz = bx * ny < 592 ? 592 / (bx * ny) : 1;
-  nz = nz > n_pass ? n_pass : (nz < 1 ? 1 : nz);
-  dim3 grid((unsigned)bx, (unsigned)ny, (unsigned)nz);
+  const int n_pass = (r.H + 32 / (d / 16) - 1) / (32 / (d / 16));
+  t.nz = bx * t.ny < 592 ? 592 / (bx * t.ny) : 1;
+  t.nz = t.nz > n_pass ? n_pass : (t.nz < 1 ? 1 : t.nz);
+  return t;
+}
+
+void launch_rope_rows(const RopeRows& a, const RopeRows* b, const double2* tab, const float4* tab_hi, const float4* tab_lo,
+                      int C, int L, int d, cudaStream_t st) {
+  const RopeTensor ta = rope_tensor(a, C, L, d);
+  RopeTensor tb = {};
+  if (b != nullptr) tb = rope_tensor(*b, C, L, d);
   note_launch();
-  rope_rows_kernel<<<grid, 256, 0, st>>>((const uint16_t*)x, x_stride[0], x_stride[1], x_stride[2], (uint16_t*)y, tab_hi,
-                                         tab_lo, tab, C, L, H, d);
+  rope_rows_kernel<<<dim3((unsigned)((L + 7) / 8), (unsigned)(ta.ny + tb.ny), (unsigned)(ta.nz > tb.nz ? ta.nz : tb.nz)), 256, 0, st>>>(
+      ta, tb, tab_hi, tab_lo, tab, C, L, d);
 }
 
 // Rows behind the end of a chunk that is shorter than L (per-chunk lengths): outputs read as zero there.
