@@ -362,68 +362,73 @@ int32_t pc_queue_emit(const int32_t* q_chunk, int32_t m, int32_t Hkv, int32_t k,
 namespace {
 
 struct ParallelPlan {
-  int Gs, n_rg, n_cache_tiles, n_split, tiles_per_split;
-  bool alt;                        // single-CTA kernel, rows of an item fit one block: two streams on alternate key tiles
-  int n_part;                      // partial results to merge per (sequence, q-head)
-  int few_split;                   // few query rows (pc_decode.cu, no workspace): CTAs of a cluster per (sequence, kv-head)
-  bool pair;                       // CTA-pair kernel: 256-row groups, no key split
-  int hpc, n_rg_pair;              // pair kernel: q-heads per CTA, 256-row groups per kv-head
+  int few_split;                   // few query rows (pc_decode.cu, no workspace): CTAs of a cluster per (sequence, kv-head); 0:
+  bool pair;                       // pc_parallel.cu on CTA pairs (else single CTAs)
+  int alt, n_rg, n_cache_tiles, n_split;   // see ParallelParams
   size_t off_counter, off_table, off_table_hi, off_table_lo, off_qrot, off_ml, off_o, total;
 };
 
-// The plan depends only on the sizes and the SM count.
-// Head size 128 with whole 256-row groups per (sequence, kv-head) runs on CTA pairs, one group per pair and
-// item, without a key split, when the groups fill the pairs' rounds to three quarters or more (the pair kernel is
-// about a third faster per tile, a partly filled last round costs it that advantage).
-// Otherwise the single-CTA kernel splits the keys.  The number of splits minimises a cost model in units of one
-// key tile: rounds of the persistent grid x (fixed cost of an item - query load, pipeline fill, write-out of
-// the partial result - of about four tiles + tiles per split).
-ParallelPlan parallel_plan(int B, int w, int Hq, int Hkv, int d, int Nk, int sm_count) {
-  ParallelPlan p;
-  const int G = Hq / Hkv;
-  p.Gs = (256 / w) < G ? (256 / w) : G;
-  p.n_rg = (G + p.Gs - 1) / p.Gs;
-  p.n_cache_tiles = (Nk + 127) / 128;
-  const long long base = (long long)B * Hkv * p.n_rg;
-  p.pair = false;
+// Partial results the workspace has room for per (sequence, q-head): the layout and with it the size that callers ask
+// for ahead follow from the sizes and the SM count alone.  One (nothing to merge) for whole 256-row groups of head size
+// 128 that fill three quarters or more of the CTA pairs' rounds; else as many key splits over single CTAs with
+// 256 rows as minimise rounds of the grid x (4 tiles of fixed cost + tiles per split), twice that for at most 128 rows.
+int part_room(int B, int w, int Hq, int Hkv, int d, int n_cache_tiles, int sm_count) {
+  const int G = Hq / Hkv, Gs = (256 / w) < G ? (256 / w) : G, n_rg = (G + Gs - 1) / Gs;
+  const long long base = (long long)B * Hkv * n_rg;
   if (d == 128 && w >= 8 && (G * w) % 256 == 0 && sm_count >= 2) {
     const long long pairs = sm_count / 2, groups = (long long)B * Hkv * (G * w / 256);
     const long long rounds = (groups + pairs - 1) / pairs;
-    if (4 * groups >= 3 * rounds * pairs) {
-      p.pair = true;
-      p.hpc = 128 / w;
-      p.n_rg_pair = G * w / 256;
-    }
+    if (4 * groups >= 3 * rounds * pairs) return 1;
   }
-  p.tiles_per_split = p.n_cache_tiles;
-  if (!p.pair) {
-    constexpr long long ITEM_COST_TILES = 4;
-    long long best = -1;
-    int max_split = p.n_cache_tiles / 2;                       // every split keeps at least two cache tiles
-    max_split = max_split < 1 ? 1 : (max_split > 64 ? 64 : max_split);
-    for (int s = 1; s <= max_split; ++s) {
-      const int tps = (p.n_cache_tiles + s - 1) / s;
-      const int ns = (p.n_cache_tiles + tps - 1) / tps;
-      const long long rounds = (base * ns + sm_count - 1) / sm_count;
-      const long long cost = rounds * (ITEM_COST_TILES + tps + (ns > 1 ? 1 : 0));   // a split run also pays for the merge
-      if (best < 0 || cost < best) { best = cost; p.tiles_per_split = tps; }
-    }
+  long long best = -1;
+  int tiles_per_split = n_cache_tiles, max_split = n_cache_tiles / 2;
+  max_split = max_split < 1 ? 1 : (max_split > 64 ? 64 : max_split);
+  for (int s = 1; s <= max_split; ++s) {
+    const int tps = (n_cache_tiles + s - 1) / s, ns = (n_cache_tiles + tps - 1) / tps;
+    const long long rounds = (base * ns + sm_count - 1) / sm_count, cost = rounds * (4 + tps + (ns > 1 ? 1 : 0));
+    if (best < 0 || cost < best) { best = cost; tiles_per_split = tps; }
   }
-  if (p.tiles_per_split < 1) p.tiles_per_split = 1;
-  p.n_split = p.n_cache_tiles > 0 ? (p.n_cache_tiles + p.tiles_per_split - 1) / p.tiles_per_split : 1;
+  if (tiles_per_split < 1) tiles_per_split = 1;
+  const int n_split = n_cache_tiles > 0 ? (n_cache_tiles + tiles_per_split - 1) / tiles_per_split : 1;
+  return Gs * w <= 128 ? 2 * n_split : n_split;
+}
+
+// The plan depends only on the sizes and the SM count.
+ParallelPlan parallel_plan(int B, int w, int Hq, int Hkv, int d, int Nk, int sm_count) {
+  ParallelPlan p;
+  const int G = Hq / Hkv;
+  p.n_cache_tiles = (Nk + 127) / 128;
+  const int room = part_room(B, w, Hq, Hkv, d, p.n_cache_tiles, sm_count);
   size_t off = 0;
   p.off_counter = off; off += ALIGN;
   p.off_table = off; off += align_up((size_t)w * (d / 2) * sizeof(double2));
   p.off_table_hi = off; off += align_up((size_t)w * (d / 4) * sizeof(float4));
   p.off_table_lo = off; off += align_up((size_t)w * (d / 4) * sizeof(float4));
   p.off_qrot = off; off += align_up((size_t)B * w * Hq * d * 2);
-  p.alt = !p.pair && p.Gs * w <= 128;
-  p.n_part = p.alt ? 2 * p.n_split : p.n_split;
   p.off_ml = off;
-  if (p.n_part > 1) off += align_up((size_t)B * Hq * p.n_part * w * 2 * sizeof(float));
+  if (room > 1) off += align_up((size_t)B * Hq * room * w * 2 * sizeof(float));
   p.off_o = off;
-  if (p.n_part > 1) off += align_up((size_t)B * Hq * p.n_part * w * d * sizeof(float));
+  if (room > 1) off += align_up((size_t)B * Hq * room * w * d * sizeof(float));
   p.total = off;
+
+  // Blocks of 128 rows per CTA (256 per pair) come in twos: an even number of them is filled with different rows that share
+  // every key tile, an odd number (in most cases one) holds the rows twice and takes alternate tiles.
+  p.pair = d == 128 && G * w > 128 && sm_count >= 2;
+  const int block_heads = (p.pair ? 256 : 128) / w, blocks = (G + block_heads - 1) / block_heads;
+  p.alt = blocks % 2;
+  p.n_rg = p.alt ? blocks : blocks / 2;
+  // Key splits: least time by a model in microseconds - rounds of the grid x (about 5 for an item + 1.4 a tile, twice that
+  // where a tile is used by two blocks of rows) + 4 for the merge of splits.
+  const int units = p.pair ? sm_count / 2 : sm_count, n_all = p.n_cache_tiles + 1;
+  const long long groups = (long long)B * Hkv * p.n_rg;
+  double least_us = -1.0;
+  p.n_split = 1;
+  for (int s = 1; s <= room && s <= 64 && 2 * s <= n_all + 1; ++s) {
+    const double rounds = std::ceil((double)groups * s / units);
+    const double cost = rounds * (5.0 + (p.alt ? 1.4 : 2.8) * std::ceil((double)n_all / s)) + (s > 1 ? 4.0 : 0.0);
+    if (least_us < 0.0 || cost < least_us) { least_us = cost; p.n_split = s; }
+  }
+
   // few query rows (at most 32 per kv-head: the line is drawn where the transposed kernel stops winning, figures in
   // pc_decode.cu): CTAs per (sequence, kv-head), 0: another kernel.  Least time by a model in microseconds - rounds of the
   // grid (two CTAs per SM) x (about 6 for prologue, pipeline fill and merge + a tile at the CTA's share of
@@ -434,7 +439,7 @@ ParallelPlan parallel_plan(int B, int w, int Hq, int Hkv, int d, int Nk, int sm_
     const double slots = 2.0 * sm_count, tile_us = 512.0 * d / 6.5e6;
     double least = -1.0;
     for (int s = 1; s <= 16 && s <= p.n_cache_tiles + 1; s *= 2) {
-      const double ctas = (double)base * s, rounds = std::ceil(ctas / slots), active = ctas < slots ? ctas : slots;
+      const double ctas = (double)B * Hkv * s, rounds = std::ceil(ctas / slots), active = ctas < slots ? ctas : slots;
       const double per_tile = tile_us * active > 512.0 * d / 5e4 ? tile_us * active : 512.0 * d / 5e4;
       const double cost = rounds * (6.0 + per_tile * std::ceil((p.n_cache_tiles + 1.0) / s));
       if (least < 0.0 || cost < least) { least = cost; p.few_split = s; }
@@ -535,51 +540,20 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   const pc::RopeRows rows = {q_win, {(long long)w * Hq * d, (long long)Hq * d, (long long)d}, q_rot, Hq};
   pc::launch_rope_rows(rows, nullptr, table, table_hi, table_lo, B, w, d, st);
 
-  // the attention reads entries below Nk only (rows behind them read as zeros and are masked): the new rows can follow
-  // on the same stream
-  auto append_kv = [&]() -> int32_t {
-    if (!append) return PC_OK;
-    return pc::launch_append_kv(k_win, v_win, B, w, Hkv, d, Nk, Nk_cap, const_cast<void*>(k_cache), const_cast<void*>(v_cache), st) ==
-                   cudaSuccess
-               ? PC_OK
-               : PC_ERR_CUDA;
-  };
-
-  if (plan.pair) {
-    CUtensorMap pm[6];
-    const uint32_t box_kch[4] = {64, 64, 1, 1};
-    const uint32_t box_kwh[4] = {64, 1, 64, 1};
-    if (!pc::make_tmap_bf16_4d(&pm[0], q_rot, qw_dims, qw_str, box_qw) ||
-        !pc::make_tmap_bf16_4d(&pm[1], out, qw_dims, qw_str, box_qw) ||
-        !pc::make_tmap_bf16_4d(&pm[2], k_cache, kc_dims, kc_str, box_kch) ||
-        !pc::make_tmap_bf16_4d(&pm[3], v_cache, kc_dims, kc_str, box_kc) ||
-        !pc::make_tmap_bf16_4d(&pm[4], k_win, kw_dims, kw_str, box_kwh) ||
-        !pc::make_tmap_bf16_4d(&pm[5], v_win, kw_dims, kw_str, box_kw))
-      return PC_ERR_CUDA;
-    pc::ParallelPairParams pp;
-    pp.B = B; pp.w = w; pp.Hq = Hq; pp.Hkv = Hkv; pp.Nk = Nk;
-    pp.hpc = plan.hpc; pp.n_rg = plan.n_rg_pair;
-    pp.scale_log2 = (float)(softmax_scale_d * 1.4426950408889634);
-    pp.lse_out = lse_out;
-    pp.status = status_word;
-    pp.wait_kcycles = pc::g_wait_kcycles.load();
-    if (pc::launch_parallel_pair(pm, pp, dev.sm_count, st) != cudaSuccess) return PC_ERR_CUDA;
-    return append_kv();
-  }
-
   CUtensorMap maps[5];
+  const uint32_t box_kch[4] = {64, plan.pair ? 64u : 128u, 1, 1};
+  const uint32_t box_kwh[4] = {64, 1, plan.pair ? 64u : 128u, 1};
   if (!pc::make_tmap_bf16_4d(&maps[0], q_rot, qw_dims, qw_str, box_qw) ||
-      !pc::make_tmap_bf16_4d(&maps[1], k_cache, kc_dims, kc_str, box_kc) ||
+      !pc::make_tmap_bf16_4d(&maps[1], k_cache, kc_dims, kc_str, box_kch) ||
       !pc::make_tmap_bf16_4d(&maps[2], v_cache, kc_dims, kc_str, box_kc) ||
-      !pc::make_tmap_bf16_4d(&maps[3], k_win, kw_dims, kw_str, box_kw) ||
+      !pc::make_tmap_bf16_4d(&maps[3], k_win, kw_dims, kw_str, box_kwh) ||
       !pc::make_tmap_bf16_4d(&maps[4], v_win, kw_dims, kw_str, box_kw))
     return PC_ERR_CUDA;
 
   pc::ParallelParams prm;
   prm.B = B; prm.w = w; prm.Hq = Hq; prm.Hkv = Hkv; prm.Nk = Nk;
-  prm.Gs = plan.Gs; prm.n_rg = plan.n_rg;
-  prm.n_cache_tiles = plan.n_cache_tiles; prm.n_split = plan.n_split; prm.tiles_per_split = plan.tiles_per_split;
-  prm.alt = plan.alt ? 1 : 0; prm.n_part = plan.n_part;
+  prm.alt = plan.alt; prm.n_rg = plan.n_rg;
+  prm.n_cache_tiles = plan.n_cache_tiles; prm.n_split = plan.n_split;
   prm.scale_log2 = (float)(softmax_scale_d * 1.4426950408889634);
   prm.part_ml = reinterpret_cast<float*>(ws + plan.off_ml);
   prm.part_o = reinterpret_cast<float*>(ws + plan.off_o);
@@ -588,10 +562,13 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   prm.status = status_word;
   prm.counter = counter;
   prm.wait_kcycles = pc::g_wait_kcycles.load();
-  const long long n_items = (long long)B * Hkv * plan.n_rg * plan.n_split;
-  const int grid = (int)(n_items < dev.sm_count ? n_items : dev.sm_count);
-  if (pc::launch_parallel_attn(maps, prm, d, grid, st) != cudaSuccess) return PC_ERR_CUDA;
-  return append_kv();
+  if (pc::launch_parallel_attn(maps, prm, d, plan.pair, dev.sm_count, st) != cudaSuccess) return PC_ERR_CUDA;
+  // the attention reads entries below Nk only (rows behind them read as zeros and are masked): the new rows can follow
+  // on the same stream
+  if (append && pc::launch_append_kv(k_win, v_win, B, w, Hkv, d, Nk, Nk_cap, const_cast<void*>(k_cache), const_cast<void*>(v_cache),
+                                     st) != cudaSuccess)
+    return PC_ERR_CUDA;
+  return PC_OK;
 }
 
 }  // namespace

@@ -23,24 +23,25 @@ struct PrefillParams {
 // maps: rotated q (box 64 x 1 x 128 tokens), k_rot, v, o (store), rotated q with a wp-row box, k_rot with a 64-token box
 cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int d, int sm_count, cudaStream_t st);
 
+// Parallel attention, more than 32 query rows per kv-head (pc_parallel.cu).
 struct ParallelParams {
   int B, w, Hq, Hkv, Nk;
-  int Gs, n_rg;                  // q-heads per row group (Gs * w <= 256), row groups per kv-head
-  int n_cache_tiles, n_split, tiles_per_split;
-  int alt;                       // 1: the item's rows fit one block; the two blocks take alternate key tiles of the split
-  int n_part;                    // partial results per (sequence, q-head): n_split, or 2 * n_split with alt
+  int alt;                       // 1: the two blocks of a CTA hold the same rows and take alternate key tiles; 0: they hold
+                                 // different rows and share the tiles
+  int n_rg;                      // row groups per kv-head (128 rows per CTA with alt, else 256; twice that on CTA pairs)
+  int n_cache_tiles, n_split;    // 128-key tiles of the cache; key splits (over those tiles and the window's own)
   float scale_log2;
-  float* part_o;                 // [B,Hq,n_part,w,d] fp32 unnormalised partial outputs (n_part > 1)
-  float* part_ml;                // [B,Hq,n_part,w,2] (running max in log2 units, sum)
+  float* part_o;                 // [B,Hq,n_split,w,d] fp32 unnormalised partial outputs (n_split > 1)
+  float* part_ml;                // [B,Hq,n_split,w,2] (running max in log2 units, sum)
   __nv_bfloat16* out;            // [B,w,Hq,d]
   float* lse_out;                // [B,Hq,w] or null
   int* status;
-  int* counter;
+  int* counter;                  // work-queue counter, zeroed before launch
   int wait_kcycles;              // limit of every device-side wait, in units of 1024 cycles
 };
-
-// maps: rotated q_win (w-row box), k_cache, v_cache (128-key box), k_win, v_win (128-row box over w tokens)
-cudaError_t launch_parallel_attn(const CUtensorMap* maps, const ParallelParams& prm, int d, int grid, cudaStream_t st);
+// maps: rotated q_win (w-row box), k_cache (128-key box; pair: 64), v_cache (128), k_win (128-row box over w tokens; pair:
+// 64), v_win (128)
+cudaError_t launch_parallel_attn(const CUtensorMap* maps, const ParallelParams& prm, int d, bool pair, int sm_count, cudaStream_t st);
 
 // Parallel attention for few query rows (pc_decode.cu): Hq / Hkv * w <= 32.  One launch, no workspace.
 struct DecodeParams {
@@ -58,20 +59,5 @@ struct DecodeParams {
 };
 // maps: k_cache, v_cache (128-key box), k_win, v_win (128-row box over w tokens)
 cudaError_t launch_decode_attn(const CUtensorMap* maps, const DecodeParams& prm, int d, cudaStream_t st);
-
-// Parallel attention on CTA pairs (head size 128, G * w a multiple of 256, no key split): every pair takes the
-// windows of 2 * hpc q-heads of one kv-head (hpc * w = 128 rows per CTA) over the whole cache.
-struct ParallelPairParams {
-  int B, w, Hq, Hkv, Nk;
-  int hpc, n_rg;                 // q-heads per CTA, 256-row groups per kv-head
-  float scale_log2;
-  float* lse_out;                // [B,Hq,w] or null
-  int* status;
-  int wait_kcycles;              // limit of every device-side wait, in units of 1024 cycles
-};
-
-// maps: rotated q_win (box 64 x 1 head x w tokens), out (same box), k_cache (64 x 64 keys), v_cache (64 x 128 keys),
-// k_win (64 x 1 head x 64 tokens), v_win (64 x 1 head x 128 tokens)
-cudaError_t launch_parallel_pair(const CUtensorMap* maps, const ParallelPairParams& prm, int sm_count, cudaStream_t st);
 
 }  // namespace pc

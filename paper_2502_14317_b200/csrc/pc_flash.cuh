@@ -1,0 +1,337 @@
+// What the flash-attention kernels on two query blocks per CTA share (chunk-local attention, pc_prefill2.cu; parallel
+// attention, pc_parallel.cu): roles, shared-memory layout, barriers, work descriptors, the K/V ring, MMA issue.
+//
+// A CTA owns two 128-row query blocks A and B, one softmax warpgroup each; while the softmax of one runs the tensor
+// cores work for the other.  Warps (16): 0-3 softmax of block A, 4-7 softmax of block B (thread = query row = TMEM lane),
+// 8-11 epilogue (the softmax warps go straight on to the next block), 12 TMA producer, 13 issuer of all MMAs (of a
+// CTA pair: in the leader only), 14-15 idle.  Registers are dealt out by role: 184 / 80 / 64.
+// Cfg<D, PAIR>: head size, and whether two CTAs of a cluster work as one unit (cta_group::2: blocks of 2 x 128 rows, every
+// K/V tile split between the two shared memories).
+#pragma once
+#include "pc_softmax.cuh"
+
+namespace pc {
+namespace flash {
+
+constexpr int TILE = 128;
+constexpr int NT2 = 512;                     // threads per CTA
+constexpr int WARP_EPI = 8, WARP_PRODUCER = 12, WARP_MMA = 13;
+constexpr int REGS_SOFTMAX = 184, REGS_EPI = 80, REGS_SERVICE = 64;      // 128 * (2 * 184 + 80 + 64) = 64 K registers
+constexpr int NDESC = 4;                     // work descriptors in flight
+constexpr int MAX_NQ = 4, MAX_NS = 6;
+template <int D_, bool PAIR_>
+struct Cfg {
+  static constexpr int D = D_;
+  static constexpr bool PAIR = PAIR_;
+  static constexpr int NCTA = PAIR ? 2 : 1;
+  static constexpr int ATOMS = D / 64;
+  static constexpr int Q_BYTES = TILE * D * 2;
+  static constexpr int STAGE_BYTES = TILE * D * 2 / NCTA;  // K/V ring: a tile, or of a pair 64 keys of K / half the columns of V
+  static constexpr int NQ = STAGE_BYTES == 16384 ? 4 : 2;  // query slots
+  static constexpr int NS = STAGE_BYTES == 16384 ? 6 : 5;
+  // TMEM: S of block b at 128 b, its accumulator at TM_O + D b.  Head size 128 has no room for P but over S; head size 64
+  // keeps it apart, so that the next S can be computed as soon as the present one is in registers
+  static constexpr bool SEP_P = D == 64;
+  static constexpr uint32_t TM_O = 256, TM_P = 384;
+  static constexpr int CODE = PAIR ? 200 : 100;            // wait codes in the status word
+};
+
+enum { W2_DESC = 1, W2_ITEM, W2_QFULL, W2_QFREE, W2_KVFULL, W2_KVFREE, W2_SFULL, W2_PHALF, W2_PFULL, W2_OFULL, W2_OFREE, W2_LM,
+       W2_LMFREE, W2_LSE, W2_TFULL, W2_TFREE, W2_SREAD, W2_PV };
+
+enum { KIND_DONE = 0, KIND_FLASH = 1, KIND_SWEEP = 2 };
+struct __align__(16) Desc {
+  int kind, c, hkv, len;       // chunk, kv-head, tokens of the chunk
+  int h[2], t[2];              // FLASH: q-head and query tile of this CTA's block A / B (t < 0 or behind the chunk: no such
+                               // tile, the rows are computed on zeros and not stored);  SWEEP: h[0] = pass
+  int n[2];                    // FLASH: key tiles walked for block A / B; 0: block absent (in both CTAs of a pair)
+};
+
+struct __align__(16) Misc2 {
+  // of a pair: q_full, kv_full, p_*, o_free, t_free, s_read in the leader only; completions of MMAs in both CTAs
+  uint64_t q_full[MAX_NQ], q_free[MAX_NQ];
+  uint64_t kv_full[MAX_NS], kv_free[MAX_NS];
+  uint64_t s_full[2], o_full[2], t_full[2];
+  uint64_t p_half[2], p_full[2], o_free[2], t_free[2];
+  uint64_t s_read[2], pv_done[2];            // head size 64: S is in registers / P V of a tile has run
+  uint64_t lm_full[2], lm_free[2];
+  uint64_t d_full[NDESC], d_free[NDESC];
+  uint64_t item_full, item_free;             // work items from the leader's producer to its peer's
+  uint64_t lse_rdy;
+  uint64_t mma_done;
+  Desc desc[NDESC];
+  int item;
+  uint32_t tmem_base;
+  int abort_flag;                            // the two words after tmem_base stay adjacent: bounded waits read the limit
+  int wait_kcycles;                          // through the flag's address
+  alignas(16) float lm[2][2][TILE];          // [block][max / sum][row]: final statistics of a block; in the score sweep [0]:
+                                             // [buffer][key] partial window scores of the second column half, [1]:
+                                             // [column half][column] log-sum-exp of the window rows
+};
+
+template <class C>
+struct Off {
+  static constexpr int Q = 0, RING = C::NQ * C::Q_BYTES, MISC = RING + C::NS * C::STAGE_BYTES, TOTAL = MISC + (int)sizeof(Misc2);
+  static_assert(TOTAL <= 232448, "shared memory of a CTA");
+};
+
+__device__ __forceinline__ uint32_t full_par(uint32_t n) { return n & 1u; }           // n-th completion of a barrier
+__device__ __forceinline__ uint32_t free_par(uint32_t n) { return (n & 1u) ^ 1u; }    // completion n-1 (passes for n = 0)
+
+struct Ctx2 {
+  Misc2* mi;
+  uint8_t* sQ;
+  uint8_t* ring;
+  uint32_t tmem;
+  volatile int* abort_flag;
+  int* status;
+};
+
+// waits of the single-thread service roles (long pause between polls) / of the softmax and epilogue warps
+#define WAIT2(bar, par, code) mbar_wait_ns<SERVICE_BACKOFF_NS>((bar), (par), cx.abort_flag, cx.status, C::CODE + (code))
+#define WAIT2S(bar, par, code) mbar_wait((bar), (par), cx.abort_flag, cx.status, C::CODE + (code))
+
+__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+// cluster address of the same barrier in CTA `rank` of a pair / of this CTA
+template <class C>
+__device__ __forceinline__ uint32_t in_cta(const void* p, uint32_t rank) {
+  if constexpr (C::PAIR) return map_to_cta(p, rank);
+  else return smem_u32(p);
+}
+template <class C>
+__device__ __forceinline__ void commit(uint64_t* bar) {           // in both CTAs of a pair
+  if constexpr (C::PAIR) mma_commit_pair(bar);
+  else mma_commit(bar);
+}
+template <class C>
+__device__ __forceinline__ void load_box(void* dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2, int c3) {
+  if constexpr (C::PAIR) tma_load_4d_pair(dst, tm, bar, c0, c1, c2, c3);
+  else tma_load_4d_addr(dst, tm, bar, c0, c1, c2, c3);
+}
+// one arrival of the warp on a barrier of the leader CTA; guards TMEM data, ordered by the tcgen05 fence
+__device__ __forceinline__ void warp_arrive_leader(uint32_t leader_addr) {
+  tc_fence_before_sync();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive_remote(leader_addr);
+}
+
+// wait whose completion also makes the peer CTA's earlier writes visible
+__device__ __forceinline__ void mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
+                                                  int where) {
+  if (mbar_try_wait_cluster(bar, parity)) return;
+  const long long t0 = clock64();
+  uint32_t spins = 0;
+  while (!mbar_try_wait_cluster(bar, parity)) {
+    if ((++spins & 63u) == 0u) {
+      if (*abort_flag) return;
+      if (clock64() - t0 > (static_cast<long long>(abort_flag[1]) << 10)) {
+        *abort_flag = 1;
+        if (status) atomicCAS(status, 0, where);
+        return;
+      }
+    }
+  }
+}
+
+template <class C>
+__device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool leader) {
+  constexpr int N = C::NCTA;
+  for (int i = 0; i < C::NQ; ++i) { mbar_init(&mi.q_full[i], 1); mbar_init(&mi.q_free[i], 1); }
+  for (int i = 0; i < C::NS; ++i) { mbar_init(&mi.kv_full[i], 1); mbar_init(&mi.kv_free[i], 1); }
+  for (int b = 0; b < 2; ++b) {
+    mbar_init(&mi.s_full[b], 1); mbar_init(&mi.o_full[b], 1); mbar_init(&mi.t_full[b], 1);
+    mbar_init(&mi.p_half[b], 4 * N); mbar_init(&mi.p_full[b], 4 * N); // 4 softmax warps of the block in each CTA
+    mbar_init(&mi.o_free[b], 4 * N); mbar_init(&mi.t_free[b], 8 * N); // epilogue warps / softmax warps of the CTAs
+    mbar_init(&mi.s_read[b], 4); mbar_init(&mi.pv_done[b], 1);
+    mbar_init(&mi.lm_full[b], 4); mbar_init(&mi.lm_free[b], 4);
+  }
+  for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 13 : 12); }   // softmax and epilogue warps, issuer
+  mbar_init(&mi.item_full, 1); mbar_init(&mi.item_free, 1);
+  mbar_init(&mi.lse_rdy, 4 * N);
+  mbar_init(&mi.mma_done, 1);
+  mi.abort_flag = 0;
+  mi.wait_kcycles = wait_kcycles;
+  fence_mbar_init();
+}
+
+// consumers of the descriptor ring.  whole_warp: all 32 threads call.
+template <class C>
+__device__ __forceinline__ Desc next_desc(const Ctx2& cx, uint32_t& n, bool whole_warp) {
+  Misc2& mi = *cx.mi;
+  const int slot = n % NDESC;
+  Desc d;
+  if (!WAIT2S(&mi.d_full[slot], full_par(n / NDESC), W2_DESC) || *cx.abort_flag) { d.kind = KIND_DONE; return d; }
+  d = mi.desc[slot];
+  if (whole_warp) warp_arrive(&mi.d_free[slot]); else mbar_arrive(&mi.d_free[slot]);
+  ++n;
+  return d;
+}
+
+// ------------------------------------------------------------------ producer
+struct Prod { uint32_t kv = 0, q = 0, d = 0, item = 0; };
+template <class C>
+__device__ __forceinline__ void publish(const Ctx2& cx, Prod& p, const Desc& d, bool signal = true) {
+  Misc2& mi = *cx.mi;
+  const int slot = p.d % NDESC;
+  WAIT2(&mi.d_free[slot], free_par(p.d / NDESC), W2_DESC);
+  mi.desc[slot] = d;
+  if (signal) mbar_arrive(&mi.d_full[slot]);
+  ++p.d;
+}
+// The leader's producer draws items from the queue and hands each to its peer's.
+template <class C>
+__device__ __forceinline__ int next_item(const Ctx2& cx, Prod& p, bool leader, int* counter, int n_items) {
+  Misc2& mi = *cx.mi;
+  int item;
+  if (leader) {
+    item = atomicAdd(counter, 1);
+    if (item > n_items) item = n_items;
+    if (!C::PAIR) return item;
+    WAIT2(&mi.item_free, free_par(p.item), W2_ITEM);      // the peer has read the previous one
+    st_async_u32(map_to_cta(&mi.item, 1), static_cast<uint32_t>(item), map_to_cta(&mi.item_full, 1));
+  } else {
+    mbar_arrive_expect_tx(&mi.item_full, 4);
+    if (!WAIT2(&mi.item_full, full_par(p.item), W2_ITEM)) return n_items;
+    item = *reinterpret_cast<volatile int*>(&mi.item);
+    mbar_arrive_remote(map_to_cta(&mi.item_free, 0));
+  }
+  ++p.item;
+  return item;
+}
+// expects a stage's bytes over both CTAs on the leader's barrier of the next ring stage; returns that barrier's address
+// for the copies and the stage's place; 0 once a wait has run out (no copy is issued into a ring that nobody drains)
+template <class C>
+__device__ __forceinline__ uint32_t ring_stage(const Ctx2& cx, Prod& p, bool leader, uint8_t** dst) {
+  Misc2& mi = *cx.mi;
+  if (*cx.abort_flag) return 0;
+  const int s = p.kv % C::NS;
+  if (!WAIT2(&mi.kv_free[s], free_par(p.kv / C::NS), W2_KVFREE)) return 0;
+  if (leader) mbar_arrive_expect_tx(&mi.kv_full[s], C::NCTA * C::STAGE_BYTES);
+  *dst = cx.ring + s * C::STAGE_BYTES;
+  ++p.kv;
+  return in_cta<C>(&mi.kv_full[s], 0);
+}
+
+// start of a kernel: barriers, tensor memory; every thread of the CTA calls
+template <class C>
+__device__ __forceinline__ void setup(Ctx2& cx, uint8_t* smem, int* status, int wait_kcycles, bool leader) {
+  Misc2& mi = *reinterpret_cast<Misc2*>(smem + Off<C>::MISC);
+  cx.mi = &mi;
+  cx.sQ = smem + Off<C>::Q;
+  cx.ring = smem + Off<C>::RING;
+  cx.abort_flag = &mi.abort_flag;
+  cx.status = status;
+  if (threadIdx.x == 0) init_barriers2<C>(mi, wait_kcycles, leader);
+  if (threadIdx.x / 32 == WARP_MMA) { if constexpr (C::PAIR) tmem_alloc_pair(&mi.tmem_base, 512); else tmem_alloc(&mi.tmem_base, 512); }
+  tc_fence_before_sync();
+  __syncthreads();
+  if constexpr (C::PAIR) cluster_sync_all();             // both CTAs' barriers exist before any remote arrive
+  tc_fence_after_sync();
+  cx.tmem = mi.tmem_base;
+}
+
+// end of a kernel: no CTA of a pair may exit while its peer can still signal it or read its shared memory
+template <class C>
+__device__ __forceinline__ void teardown(const Ctx2& cx) {
+  tc_fence_before_sync();
+  __syncthreads();
+  if constexpr (C::PAIR) cluster_sync_all();
+  if (threadIdx.x / 32 == WARP_MMA) {
+    // no tensor-core operation may still be running when its accumulators are freed: the issuer ended with a
+    // commit to mma_done (an arrival in both CTAs of a pair).  Immediate in a clean run; after an abort this is what
+    // makes the exit safe.  The wait ignores the abort flag and is bounded.
+    mbar_wait_drain(&cx.mi->mma_done, 0, cx.abort_flag);
+    tc_fence_after_sync();
+    if constexpr (C::PAIR) tmem_dealloc_pair(cx.tmem, 512); else tmem_dealloc(cx.tmem, 512);
+  }
+}
+
+// Producer, at the end: every copy issued must have landed before a CTA may exit.  In a run without a timed-out wait that
+// follows from the last uses of the rings having been consumed (teardown waits for every tensor-core operation).  After
+// an abort nothing is consumed any more: the leader, whose barriers count the bytes of both CTAs' copies, waits on
+// them (ignoring the abort flag, bounded); its peer cannot observe the completion of its own last copies and lets a
+// fixed pause pass that outlasts any copy in flight.
+template <class C>
+__device__ __forceinline__ void drain_copies(const Ctx2& cx, const Prod& p, bool leader) {
+  Misc2& mi = *cx.mi;
+  if (!*cx.abort_flag) return;
+  if (leader) {
+    for (uint32_t i = (p.kv > C::NS ? p.kv - C::NS : 0); i < p.kv; ++i) mbar_wait_drain(&mi.kv_full[i % C::NS], full_par(i / C::NS), cx.abort_flag);
+    for (uint32_t i = (p.q > C::NQ ? p.q - C::NQ : 0); i < p.q; ++i) mbar_wait_drain(&mi.q_full[i % C::NQ], full_par(i / C::NQ), cx.abort_flag);
+  }
+  abort_grace_pause(cx.abort_flag);
+}
+
+// ------------------------------------------------------------------ issuer (one elected thread; of a pair: of the leader CTA)
+template <class C>
+struct Issuer {
+  const Ctx2& cx;
+  uint32_t ring_u32, q_u32;
+  uint32_t nd = 0, kv = 0, nq = 0, np[2] = {0, 0}, no[2] = {0, 0};   // descriptors, ring, query slots, tiles and blocks done
+  uint32_t qa[2] = {0, 0};                                           // query operands of the two blocks in work
+  __device__ __forceinline__ explicit Issuer(const Ctx2& c) : cx(c), ring_u32(smem_u32(c.ring)), q_u32(smem_u32(c.sQ)) {}
+  // operand of ring use i, once its copy has landed
+  __device__ __forceinline__ uint32_t wait_kv(uint32_t i) {
+    WAIT2S(&cx.mi->kv_full[i % C::NS], full_par(i / C::NS), W2_KVFULL);
+    return ring_u32 + (i % C::NS) * C::STAGE_BYTES;
+  }
+  __device__ __forceinline__ void free_kv(uint32_t i) { commit<C>(&cx.mi->kv_free[i % C::NS]); }
+  __device__ __forceinline__ uint32_t wait_q() {
+    WAIT2S(&cx.mi->q_full[nq % C::NQ], full_par(nq / C::NQ), W2_QFULL);
+    const uint32_t q = q_u32 + (nq % C::NQ) * C::Q_BYTES;
+    ++nq;
+    return q;
+  }
+  // S of block b = Q K^T
+  __device__ __forceinline__ void qk(int b, uint32_t k_smem) {
+    constexpr uint32_t idesc = make_idesc_bf16_f32(TILE * C::NCTA, TILE, false, false);
+    tc_fence_after_sync();
+    if constexpr (C::PAIR) mma_ss_pair_k128<true>(cx.tmem + b * 128, qa[b], k_smem, idesc);
+    else if constexpr (C::D == 128) mma_ss_k128(cx.tmem + b * 128, qa[b], k_smem, idesc);
+    else mma_ss_k64(cx.tmem + b * 128, qa[b], k_smem, idesc);
+    commit<C>(&cx.mi->s_full[b]);
+  }
+  // O of block b += P V of a tile, in two halves as P arrives
+  __device__ __forceinline__ void pv(int b, uint32_t v_smem, bool first, bool last) {
+    Misc2& mi = *cx.mi;
+    constexpr uint32_t idesc = make_idesc_bf16_f32(TILE * C::NCTA, C::D, false, true);
+    const uint32_t tO = cx.tmem + C::TM_O + b * C::D, tP = C::SEP_P ? cx.tmem + C::TM_P + b * 64 : cx.tmem + b * 128;
+    if (first) { WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE); ++no[b]; }       // accumulator of the previous block read out
+    WAIT2S(&mi.p_half[b], full_par(np[b]), W2_PHALF);                                // keys 0..63 of P
+    tc_fence_after_sync();
+    mma_ts_k64<C::PAIR>(tO, tP, v_smem, idesc, !first);
+    WAIT2S(&mi.p_full[b], full_par(np[b]), W2_PFULL);
+    ++np[b];
+    tc_fence_after_sync();
+    mma_ts_k64<C::PAIR>(tO, tP + 32, v_smem + 8192, idesc, true);
+    if (C::SEP_P) commit<C>(&mi.pv_done[b]);
+    if (last) commit<C>(&mi.o_full[b]);
+  }
+  __device__ __forceinline__ void wait_s_read(int b) { WAIT2S(&cx.mi->s_read[b], full_par(np[b]), W2_SREAD); }
+};
+
+// ------------------------------------------------------------------ softmax warps: hooks of softmax_tile for block b
+template <class C>
+struct Hooks {
+  const Ctx2& cx;
+  uint32_t p_half, p_full, s_read;                           // barriers (of the leader CTA)
+  uint64_t* pv_done;
+  uint32_t tiles;                                            // tiles of this block before the present one
+  __device__ __forceinline__ Hooks(const Ctx2& c, int b)
+      : cx(c), p_half(in_cta<C>(&c.mi->p_half[b], 0)), p_full(in_cta<C>(&c.mi->p_full[b], 0)), s_read(in_cta<C>(&c.mi->s_read[b], 0)),
+        pv_done(&c.mi->pv_done[b]), tiles(0) {}
+  __device__ __forceinline__ void on_read() const { if (C::SEP_P) warp_arrive_leader(s_read); }
+  // P over S: S of this tile was issued after P V of the tile before, and P overwrites S, which is in registers
+  __device__ __forceinline__ void before_p() const {
+    if (C::SEP_P && tiles > 0) { WAIT2S(pv_done, full_par(tiles - 1), W2_PV); tc_fence_after_sync(); }
+  }
+  __device__ __forceinline__ void before_rescale() const { before_p(); }
+  __device__ __forceinline__ void on_half() const { warp_arrive_leader(p_half); }
+  __device__ __forceinline__ void on_full() const { warp_arrive_leader(p_full); }
+};
+
+}  // namespace flash
+}  // namespace pc

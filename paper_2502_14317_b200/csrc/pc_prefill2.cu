@@ -11,82 +11,21 @@
 // Head size 64 runs on single CTAs: its products are half as long, the softmax is what bounds it, and there is room in
 // TMEM for P beside S, so the next tile's S is computed as soon as the present one is in registers.
 //
-// Warps (16 per CTA): 0-3 softmax of block A, 4-7 softmax of block B (thread = query row = TMEM lane), 8-11 epilogue (the
-// softmax warps go straight on to the next block), 12 TMA producer, 13 issuer of all MMAs (of a pair: in the leader CTA
-// only), 14-15 idle.  Registers are dealt out by role: 184 / 80 / 64.
+// Roles, rings and barriers: pc_flash.cuh.
 //
 // Window scores: the unit that runs the last query tiles of a (chunk, kv-head) group then sweeps the keys once more
 // with the transposed product K_j Qw^T (the CTAs of a pair take alternate key tiles; keys on TMEM lanes, window
 // rows on columns), so Eq. 6 is a per-thread sum in a fixed order: deterministic, fp32, no atomics.
 #include "pc_attn.h"
 #include "pc_kernels.h"
-#include "pc_softmax.cuh"
+#include "pc_flash.cuh"
 
 namespace pc {
 
 namespace {
 
-constexpr int TILE = 128;
-constexpr int NT2 = 512;                     // threads per CTA
-constexpr int WARP_EPI = 8, WARP_PRODUCER = 12, WARP_MMA = 13;
-constexpr int REGS_SOFTMAX = 184, REGS_EPI = 80, REGS_SERVICE = 64;      // 128 * (2 * 184 + 80 + 64) = 64 K registers
-constexpr int NQ = 4;                        // query slots: the two blocks in work and the two that come next
-constexpr int NS = 6;                        // K/V ring stages (16 KB: of a pair 64 keys x 128 d of K or 128 keys x 64 d of V;
-                                             // of a single CTA 128 keys x 64 d)
-constexpr int NDESC = 4;                     // work descriptors in flight
-constexpr int STAGE_BYTES = 16384;
-template <int D>
-struct Cfg {
-  static constexpr bool PAIR = D == 128;
-  static constexpr int NCTA = PAIR ? 2 : 1;
-  static constexpr int ATOMS = D / 64;
-  static constexpr int Q_BYTES = TILE * D * 2;
-  static constexpr uint32_t TM_O = 256;      // accumulator columns (block b: + D b)
-  static constexpr uint32_t TM_P = 384;      // head size 64: P of block b: + 64 b (head size 128: over S)
-  static constexpr int CODE = PAIR ? 200 : 100;        // wait codes in the status word
-};
-
-enum { W2_DESC = 1, W2_ITEM, W2_QFULL, W2_QFREE, W2_KVFULL, W2_KVFREE, W2_SFULL, W2_PHALF, W2_PFULL, W2_OFULL, W2_OFREE, W2_LM,
-       W2_LMFREE, W2_LSE, W2_TFULL, W2_TFREE, W2_SREAD, W2_PV };
-
-enum { KIND_DONE = 0, KIND_FLASH = 1, KIND_SWEEP = 2 };
-struct __align__(16) Desc {
-  int kind, c, hkv, len;       // chunk, kv-head, tokens of the chunk
-  int h[2], t[2];              // FLASH: q-head and query tile of this CTA's block A / B (t < 0 or behind the chunk: no such
-                               // tile, the rows are computed on zeros and not stored);  SWEEP: h[0] = pass
-  int n[2];                    // FLASH: key tiles walked for block A / B; 0: block absent (in both CTAs of a pair)
-};
-
-struct __align__(16) Misc2 {
-  // of a pair: q_full, kv_full, p_*, o_free, t_free, s_read in the leader only; completions of MMAs in both CTAs
-  uint64_t q_full[NQ], q_free[NQ];
-  uint64_t kv_full[NS], kv_free[NS];
-  uint64_t s_full[2], o_full[2], t_full[2];
-  uint64_t p_half[2], p_full[2], o_free[2], t_free[2];
-  uint64_t s_read[2], pv_done[2];            // head size 64: S is in registers / P V of a tile has run
-  uint64_t lm_full[2], lm_free[2];
-  uint64_t d_full[NDESC], d_free[NDESC];
-  uint64_t item_full, item_free;             // work items from the leader's producer to its peer's
-  uint64_t lse_rdy;
-  uint64_t mma_done;
-  Desc desc[NDESC];
-  int item;
-  uint32_t tmem_base;
-  int abort_flag;                            // the two words after tmem_base stay adjacent: bounded waits read the limit
-  int wait_kcycles;                          // through the flag's address
-  alignas(16) float lm[2][2][TILE];          // [block][max / sum][row]: final statistics of a block; in the score sweep [0]:
-                                             // [buffer][key] partial window scores of the second column half, [1]:
-                                             // [column half][column] log-sum-exp of the window rows
-};
-
-template <int D>
-struct Off {
-  static constexpr int Q = 0, RING = NQ * Cfg<D>::Q_BYTES, MISC = RING + NS * STAGE_BYTES, TOTAL = MISC + (int)sizeof(Misc2);
-  static_assert(TOTAL <= 232448, "shared memory of a CTA");
-};
-
-__device__ __forceinline__ uint32_t full_par(uint32_t n) { return n & 1u; }           // n-th completion of a barrier
-__device__ __forceinline__ uint32_t free_par(uint32_t n) { return (n & 1u) ^ 1u; }    // completion n-1 (passes for n = 0)
+using namespace flash;
+template <int D> using PCfg = Cfg<D, D == 128>;
 
 // ------------------------------------------------------------------ work decomposition
 // Groups = (chunk, kv-head).  A unit is what the blocks (four of a pair, two of a single CTA) take at a time.  Pair:
@@ -110,7 +49,7 @@ __device__ __forceinline__ Sched2 make_sched2(const PrefillParams& p) {
   Sched2 s;
   s.T = (p.L + TILE - 1) / TILE;
   s.G = p.Hq / p.Hkv;
-  constexpr int BLOCKS = 2 * Cfg<D>::NCTA;
+  constexpr int BLOCKS = 2 * PCfg<D>::NCTA;
   s.hpu = s.G % BLOCKS == 0 ? BLOCKS : (s.G % 2 == 0 ? 2 : 1);      // q-heads and tiles of a unit
   s.tpu = BLOCKS / s.hpu;
   s.P = s.G / s.hpu;
@@ -155,7 +94,7 @@ __device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, 
 #pragma unroll
   for (int b = 0; b < 2; ++b) {
     int top;                                              // upper tile of the block over both CTAs
-    if (!Cfg<D>::PAIR) {
+    if (!PCfg<D>::PAIR) {
       d.h[b] = s.hpu == 2 ? h0 + b : h0;
       top = s.hpu == 2 ? hi : hi - 1 + b;
       d.t[b] = top;
@@ -164,143 +103,6 @@ __device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, 
     else { d.h[b] = h0; top = hi - 2 + 2 * b; d.t[b] = top - 1 + rank; }
     d.n[b] = top < 0 ? 0 : top + 1;
   }
-}
-
-struct Ctx2 {
-  Misc2* mi;
-  uint8_t* sQ;
-  uint8_t* ring;
-  uint32_t tmem;
-  volatile int* abort_flag;
-  int* status;
-};
-
-// waits of the single-thread service roles (long pause between polls) / of the softmax and epilogue warps
-#define WAIT2(bar, par, code) mbar_wait_ns<SERVICE_BACKOFF_NS>((bar), (par), cx.abort_flag, cx.status, Cfg<D>::CODE + (code))
-#define WAIT2S(bar, par, code) mbar_wait((bar), (par), cx.abort_flag, cx.status, Cfg<D>::CODE + (code))
-
-__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-}
-// cluster address of the same barrier in CTA `rank` of a pair / of this CTA
-template <int D>
-__device__ __forceinline__ uint32_t in_cta(const void* p, uint32_t rank) {
-  if constexpr (Cfg<D>::PAIR) return map_to_cta(p, rank);
-  else return smem_u32(p);
-}
-template <int D>
-__device__ __forceinline__ void commit(uint64_t* bar) {           // in both CTAs of a pair
-  if constexpr (Cfg<D>::PAIR) mma_commit_pair(bar);
-  else mma_commit(bar);
-}
-template <int D>
-__device__ __forceinline__ void load_box(void* dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2, int c3) {
-  if constexpr (Cfg<D>::PAIR) tma_load_4d_pair(dst, tm, bar, c0, c1, c2, c3);
-  else tma_load_4d_addr(dst, tm, bar, c0, c1, c2, c3);
-}
-// one arrival of the warp on a barrier of the leader CTA; guards TMEM data, ordered by the tcgen05 fence
-__device__ __forceinline__ void warp_arrive_leader(uint32_t leader_addr) {
-  tc_fence_before_sync();
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) mbar_arrive_remote(leader_addr);
-}
-
-// wait whose completion also makes the peer CTA's earlier writes visible
-__device__ __forceinline__ void mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
-                                                  int where) {
-  if (mbar_try_wait_cluster(bar, parity)) return;
-  const long long t0 = clock64();
-  uint32_t spins = 0;
-  while (!mbar_try_wait_cluster(bar, parity)) {
-    if ((++spins & 63u) == 0u) {
-      if (*abort_flag) return;
-      if (clock64() - t0 > (static_cast<long long>(abort_flag[1]) << 10)) {
-        *abort_flag = 1;
-        if (status) atomicCAS(status, 0, where);
-        return;
-      }
-    }
-  }
-}
-
-template <int D>
-__device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool leader) {
-  constexpr int N = Cfg<D>::NCTA;
-  for (int i = 0; i < NQ; ++i) { mbar_init(&mi.q_full[i], 1); mbar_init(&mi.q_free[i], 1); }
-  for (int i = 0; i < NS; ++i) { mbar_init(&mi.kv_full[i], 1); mbar_init(&mi.kv_free[i], 1); }
-  for (int b = 0; b < 2; ++b) {
-    mbar_init(&mi.s_full[b], 1); mbar_init(&mi.o_full[b], 1); mbar_init(&mi.t_full[b], 1);
-    mbar_init(&mi.p_half[b], 4 * N); mbar_init(&mi.p_full[b], 4 * N); // 4 softmax warps of the block in each CTA
-    mbar_init(&mi.o_free[b], 4 * N); mbar_init(&mi.t_free[b], 8 * N); // epilogue warps / softmax warps of the CTAs
-    mbar_init(&mi.s_read[b], 4); mbar_init(&mi.pv_done[b], 1);
-    mbar_init(&mi.lm_full[b], 4); mbar_init(&mi.lm_free[b], 4);
-  }
-  for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 13 : 12); }   // softmax and epilogue warps, issuer
-  mbar_init(&mi.item_full, 1); mbar_init(&mi.item_free, 1);
-  mbar_init(&mi.lse_rdy, 4 * N);
-  mbar_init(&mi.mma_done, 1);
-  mi.abort_flag = 0;
-  mi.wait_kcycles = wait_kcycles;
-  fence_mbar_init();
-}
-
-// consumers of the descriptor ring.  whole_warp: all 32 threads call.
-template <int D>
-__device__ __forceinline__ Desc next_desc(const Ctx2& cx, uint32_t& n, bool whole_warp) {
-  Misc2& mi = *cx.mi;
-  const int slot = n % NDESC;
-  Desc d;
-  if (!WAIT2S(&mi.d_full[slot], full_par(n / NDESC), W2_DESC) || *cx.abort_flag) { d.kind = KIND_DONE; return d; }
-  d = mi.desc[slot];
-  if (whole_warp) warp_arrive(&mi.d_free[slot]); else mbar_arrive(&mi.d_free[slot]);
-  ++n;
-  return d;
-}
-
-// ------------------------------------------------------------------ producer
-struct Prod { uint32_t kv = 0, q = 0, d = 0, item = 0; };
-template <int D>
-__device__ __forceinline__ void publish(const Ctx2& cx, Prod& p, const Desc& d, bool signal = true) {
-  Misc2& mi = *cx.mi;
-  const int slot = p.d % NDESC;
-  WAIT2(&mi.d_free[slot], free_par(p.d / NDESC), W2_DESC);
-  mi.desc[slot] = d;
-  if (signal) mbar_arrive(&mi.d_full[slot]);
-  ++p.d;
-}
-// The leader's producer draws items from the queue and hands each to its peer's.
-template <int D>
-__device__ __forceinline__ int next_item(const Ctx2& cx, Prod& p, bool leader, int* counter, int n_items) {
-  Misc2& mi = *cx.mi;
-  int item;
-  if (leader) {
-    item = atomicAdd(counter, 1);
-    if (item > n_items) item = n_items;
-    if (!Cfg<D>::PAIR) return item;
-    WAIT2(&mi.item_free, free_par(p.item), W2_ITEM);      // the peer has read the previous one
-    st_async_u32(map_to_cta(&mi.item, 1), static_cast<uint32_t>(item), map_to_cta(&mi.item_full, 1));
-  } else {
-    mbar_arrive_expect_tx(&mi.item_full, 4);
-    if (!WAIT2(&mi.item_full, full_par(p.item), W2_ITEM)) return n_items;
-    item = *reinterpret_cast<volatile int*>(&mi.item);
-    mbar_arrive_remote(map_to_cta(&mi.item_free, 0));
-  }
-  ++p.item;
-  return item;
-}
-// expects a stage's bytes over both CTAs on the leader's barrier of the next ring stage; returns that barrier's address
-// for the copies and the stage's place; 0 once a wait has run out (no copy is issued into a ring that nobody drains)
-template <int D>
-__device__ __forceinline__ uint32_t ring_stage(const Ctx2& cx, Prod& p, bool leader, uint8_t** dst) {
-  Misc2& mi = *cx.mi;
-  if (*cx.abort_flag) return 0;
-  const int s = p.kv % NS;
-  if (!WAIT2(&mi.kv_free[s], free_par(p.kv / NS), W2_KVFREE)) return 0;
-  if (leader) mbar_arrive_expect_tx(&mi.kv_full[s], Cfg<D>::NCTA * STAGE_BYTES);
-  *dst = cx.ring + s * STAGE_BYTES;
-  ++p.kv;
-  return in_cta<D>(&mi.kv_full[s], 0);
 }
 
 }  // namespace
@@ -316,29 +118,16 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ CUtensorMap tm_qw,
                const __grid_constant__ PrefillParams prm) {
-  constexpr bool PAIR = Cfg<D>::PAIR;
-  constexpr int NCTA = Cfg<D>::NCTA, Q_BYTES = Cfg<D>::Q_BYTES;
-  constexpr uint32_t TM_O = Cfg<D>::TM_O, TM_P = Cfg<D>::TM_P;
+  using C = PCfg<D>;
+  constexpr bool PAIR = C::PAIR;
+  constexpr int NCTA = C::NCTA, Q_BYTES = C::Q_BYTES, NQ = C::NQ;
   extern __shared__ __align__(1024) uint8_t smem[];
-  Misc2& mi = *reinterpret_cast<Misc2*>(smem + Off<D>::MISC);
-  Ctx2 cx;
-  cx.mi = &mi;
-  cx.sQ = smem + Off<D>::Q;
-  cx.ring = smem + Off<D>::RING;
-  cx.abort_flag = &mi.abort_flag;
-  cx.status = prm.status;
-
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0;
   const bool leader = (rank == 0);
-
-  if (tid == 0) init_barriers2<D>(mi, prm.wait_kcycles, leader);
-  if (warp == WARP_MMA) { if constexpr (PAIR) tmem_alloc_pair(&mi.tmem_base, 512); else tmem_alloc(&mi.tmem_base, 512); }
-  tc_fence_before_sync();
-  __syncthreads();
-  if constexpr (PAIR) cluster_sync_all();                // both CTAs' barriers exist before any remote arrive
-  tc_fence_after_sync();
-  cx.tmem = mi.tmem_base;
+  Ctx2 cx;
+  setup<C>(cx, smem, prm.status, prm.wait_kcycles, leader);
+  Misc2& mi = *cx.mi;
 
   if (warp >= WARP_PRODUCER) {
     setmaxnreg_dec<REGS_SERVICE>();
@@ -354,7 +143,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         // Once a wait has run out (abort flag) no new work is started: every role leaves its loops at the next
         // descriptor, this one also at the next tile, so that no copy is issued into a ring that nobody drains.
         while (!*cx.abort_flag) {
-          const int item = next_item<D>(cx, p, leader, prm.counter, n_items);
+          const int item = next_item<C>(cx, p, leader, prm.counter, n_items);
           if (item >= n_items) break;
           int group, within;
           decode_item(sch, n_groups, item, group, within);
@@ -368,26 +157,26 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             d.kind = KIND_FLASH;
             decode_unit<D>(sch, rank, d.hkv, within, sub, d);
             if (d.n[1] == 0) continue;                    // (n[0] <= n[1])
-            publish<D>(cx, p, d);
+            publish<C>(cx, p, d);
             for (int b = 0; b < 2; ++b) {
               if (d.n[b] == 0) continue;
               const int qs = p.q % NQ;
               WAIT2(&mi.q_free[qs], free_par(p.q / NQ), W2_QFREE);
               if (leader) mbar_arrive_expect_tx(&mi.q_full[qs], NCTA * Q_BYTES);
-              const uint32_t bar = in_cta<D>(&mi.q_full[qs], 0);
-              for (int a = 0; a < Cfg<D>::ATOMS; ++a)
-                load_box<D>(cx.sQ + qs * Q_BYTES + a * 16384, &tm_q, bar, a * 64, d.h[b], d.t[b] * TILE, d.c);
+              const uint32_t bar = in_cta<C>(&mi.q_full[qs], 0);
+              for (int a = 0; a < C::ATOMS; ++a)
+                load_box<C>(cx.sQ + qs * Q_BYTES + a * 16384, &tm_q, bar, a * 64, d.h[b], d.t[b] * TILE, d.c);
               ++p.q;
             }
             for (int j = 0; j < d.n[1]; ++j) {
-              const uint32_t kbar = ring_stage<D>(cx, p, leader, &dst);
+              const uint32_t kbar = ring_stage<C>(cx, p, leader, &dst);
               if (kbar) {
                 if constexpr (PAIR)
-                  for (int a = 0; a < 2; ++a) load_box<D>(dst + a * 8192, &tm_kh, kbar, a * 64, d.hkv, j * TILE + (int)rank * 64, d.c);
-                else load_box<D>(dst, &tm_k, kbar, 0, d.hkv, j * TILE, d.c);
+                  for (int a = 0; a < 2; ++a) load_box<C>(dst + a * 8192, &tm_kh, kbar, a * 64, d.hkv, j * TILE + (int)rank * 64, d.c);
+                else load_box<C>(dst, &tm_k, kbar, 0, d.hkv, j * TILE, d.c);
               }
-              const uint32_t vbar = ring_stage<D>(cx, p, leader, &dst);
-              if (vbar) load_box<D>(dst, &tm_v, vbar, (int)rank * 64, d.hkv, j * TILE, d.c);
+              const uint32_t vbar = ring_stage<C>(cx, p, leader, &dst);
+              if (vbar) load_box<C>(dst, &tm_v, vbar, (int)rank * 64, d.hkv, j * TILE, d.c);
             }
           }
           if (within == 0) {
@@ -398,17 +187,17 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             for (int u = 0; u < sch.n_pass; ++u) {
               d.kind = KIND_SWEEP;
               d.h[0] = u;
-              publish<D>(cx, p, d);
+              publish<C>(cx, p, d);
               for (int b = 0; b < 3 - NCTA; ++b) {        // a pair's CTAs load a column half each, a single CTA both
                 const int qs = p.q % NQ;
                 WAIT2(&mi.q_free[qs], free_par(p.q / NQ), W2_QFREE);
                 if (leader) mbar_arrive_expect_tx(&mi.q_full[qs], NCTA * rows_half * D * 2);
-                const uint32_t bar = in_cta<D>(&mi.q_full[qs], 0);
+                const uint32_t bar = in_cta<C>(&mi.q_full[qs], 0);
                 for (int i = 0; i < sch.hp; ++i) {
                   int g = u * 2 * sch.hp + ((int)rank + b) * sch.hp + i;
                   if (g >= sch.G) g = sch.G - 1;          // filler rows: loaded, never summed
-                  for (int a = 0; a < Cfg<D>::ATOMS; ++a)
-                    load_box<D>(cx.sQ + qs * Q_BYTES + a * 16384 + i * sch.wp * 128, &tm_qw, bar, a * 64, d.hkv * sch.G + g,
+                  for (int a = 0; a < C::ATOMS; ++a)
+                    load_box<C>(cx.sQ + qs * Q_BYTES + a * 16384 + i * sch.wp * 128, &tm_qw, bar, a * 64, d.hkv * sch.G + g,
                                 d.len - sch.wp, d.c);
                 }
                 ++p.q;
@@ -416,118 +205,75 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               // a full key tile takes ATOMS consecutive stages (of a pair: two that start on an even one, everything uses
               // stages in twos)
               for (int jj = 0; jj < n_steps; ++jj)
-                for (int a = 0; a < Cfg<D>::ATOMS; ++a) {
-                  const uint32_t kbar = ring_stage<D>(cx, p, leader, &dst);
-                  if (kbar) load_box<D>(dst, &tm_k, kbar, a * 64, d.hkv, (NCTA * jj + (int)rank) * TILE, d.c);
+                for (int a = 0; a < C::ATOMS; ++a) {
+                  const uint32_t kbar = ring_stage<C>(cx, p, leader, &dst);
+                  if (kbar) load_box<C>(dst, &tm_k, kbar, a * 64, d.hkv, (NCTA * jj + (int)rank) * TILE, d.c);
                 }
             }
           }
         }
         Desc d;
         d.kind = KIND_DONE; d.c = d.hkv = d.len = 0;
-        publish<D>(cx, p, d, PAIR || prm.skip_final_publication == 0);
-        // Every copy issued must have landed before a CTA may exit.  In a run without a timed-out wait that follows
-        // from the last uses of the rings having been consumed (the teardown below waits for every tensor-core
-        // operation).  After an abort nothing is consumed any more: the leader, whose barriers count the bytes of both
-        // CTAs' copies, waits on them (ignoring the abort flag, bounded); the peer cannot observe the completion of
-        // its own last copies and lets a fixed pause pass that outlasts any copy in flight.
-        if (*cx.abort_flag) {
-          if (leader) {
-            for (uint32_t i = (p.kv > NS ? p.kv - NS : 0); i < p.kv; ++i) mbar_wait_drain(&mi.kv_full[i % NS], full_par(i / NS), cx.abort_flag);
-            for (uint32_t i = (p.q > NQ ? p.q - NQ : 0); i < p.q; ++i) mbar_wait_drain(&mi.q_full[i % NQ], full_par(i / NQ), cx.abort_flag);
-          }
-          abort_grace_pause(cx.abort_flag);
-        }
+        publish<C>(cx, p, d, PAIR || prm.skip_final_publication == 0);
+        drain_copies<C>(cx, p, leader);
       }
       __syncwarp();
     } else if (warp == WARP_MMA && leader) {
       // ================================================================ issuer (of a pair: leader CTA)
       if (elect_one()) {
         const Sched2 sch = make_sched2<D>(prm);
-        constexpr uint32_t idesc_qk = make_idesc_bf16_f32(TILE * NCTA, TILE, false, false), idesc_pv = make_idesc_bf16_f32(TILE * NCTA, D, false, true);
         const int rows_half = sch.hp * sch.wp;
         const uint32_t idesc_sw = make_idesc_bf16_f32(TILE * NCTA, PAIR ? 2 * rows_half : (rows_half + 15) & ~15, false, false);
-        const uint32_t ring_u32 = smem_u32(cx.ring), q_u32 = smem_u32(cx.sQ);
-        uint32_t nd = 0, kv = 0, nq = 0, np[2] = {0, 0}, no[2] = {0, 0}, nt = 0;
-        uint32_t qa[2] = {0, 0};                                          // query operands of the two blocks in work
-        auto wait_kv = [&](uint32_t i) {
-          WAIT2S(&mi.kv_full[i % NS], full_par(i / NS), W2_KVFULL);
-          return ring_u32 + (i % NS) * STAGE_BYTES;
-        };
-        auto qk = [&](int b, uint32_t k_smem) {
-          tc_fence_after_sync();
-          if constexpr (PAIR) mma_ss_pair_k128<true>(cx.tmem + b * 128, qa[b], k_smem, idesc_qk);
-          else mma_ss_k64(cx.tmem + b * 128, qa[b], k_smem, idesc_qk);
-          commit<D>(&mi.s_full[b]);
-        };
-        auto first_qk = [&](int b, uint32_t k_smem) {
-          qa[b] = q_u32 + (nq % NQ) * Q_BYTES;
-          WAIT2S(&mi.q_full[nq % NQ], full_par(nq / NQ), W2_QFULL);
-          ++nq;
-          qk(b, k_smem);
-        };
-        // O += P V of a tile, in two halves as P arrives
-        auto pv = [&](int b, uint32_t v_smem, bool first, bool last) {
-          const uint32_t tO = cx.tmem + TM_O + b * D, tP = PAIR ? cx.tmem + b * 128 : cx.tmem + TM_P + b * 64;
-          if (first) { WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE); ++no[b]; }       // accumulator of the previous block read out
-          WAIT2S(&mi.p_half[b], full_par(np[b]), W2_PHALF);                                // keys 0..63 of P
-          tc_fence_after_sync();
-          mma_ts_k64<PAIR>(tO, tP, v_smem, idesc_pv, !first);
-          WAIT2S(&mi.p_full[b], full_par(np[b]), W2_PFULL);
-          ++np[b];
-          tc_fence_after_sync();
-          mma_ts_k64<PAIR>(tO, tP + 32, v_smem + 8192, idesc_pv, true);
-          if (!PAIR) mma_commit(&mi.pv_done[b]);
-          if (last) commit<D>(&mi.o_full[b]);
-        };
-        Desc d = next_desc<D>(cx, nd, false);
+        Issuer<C> is(cx);
+        uint32_t nt = 0;
+        auto first_qk = [&](int b, uint32_t k_smem) { is.qa[b] = is.wait_q(); is.qk(b, k_smem); };
+        Desc d = next_desc<C>(cx, is.nd, false);
         bool primed = false;                                     // first S of the unit already issued
         while (d.kind != KIND_DONE) {
           if (d.kind == KIND_FLASH) {
             const int n0 = d.n[0], n = d.n[1];
             if (!primed) {
-              const uint32_t k_u32 = wait_kv(kv);
+              const uint32_t k_u32 = is.wait_kv(is.kv);
               for (int b = 0; b < 2; ++b) if (d.n[b] > 0) first_qk(b, k_u32);
-              commit<D>(&mi.kv_free[kv % NS]);
-              ++kv;
+              is.free_kv(is.kv++);
             }
             Desc nx;
             nx.kind = KIND_DONE; nx.n[0] = nx.n[1] = 0;
             // the next unit's first S follows the last tile without a gap
-            for (int j = 0; j < n; ++j) {                        // kv: V of tile j; kv + 1: the next K
+            for (int j = 0; j < n; ++j) {                        // is.kv: V of tile j; is.kv + 1: the next K
               bool more = j + 1 < n;
               uint32_t k_u32 = 0;
               auto look_ahead = [&]() {
-                if (j + 1 == n) { nx = next_desc<D>(cx, nd, false); more = nx.kind == KIND_FLASH; }
-                if (more) k_u32 = wait_kv(kv + 1);
+                if (j + 1 == n) { nx = next_desc<C>(cx, is.nd, false); more = nx.kind == KIND_FLASH; }
+                if (more) k_u32 = is.wait_kv(is.kv + 1);
               };
               auto next_s = [&](int b, int nb) {
-                if (j + 1 < nb) qk(b, k_u32);
+                if (j + 1 < nb) is.qk(b, k_u32);
                 else if (j + 1 == n && more && nx.n[b] > 0) first_qk(b, k_u32);
               };
-              if constexpr (PAIR) {
+              if constexpr (!C::SEP_P) {
                 // per block: P V, then the next S over P; the pipe runs them in order
-                const uint32_t v_u32 = wait_kv(kv);
-                if (j < n0) pv(0, v_u32, j == 0, j == n0 - 1);
+                const uint32_t v_u32 = is.wait_kv(is.kv);
+                if (j < n0) is.pv(0, v_u32, j == 0, j == n0 - 1);
                 look_ahead();
                 next_s(0, n0);
-                pv(1, v_u32, j == 0, j == n - 1);
+                is.pv(1, v_u32, j == 0, j == n - 1);
                 next_s(1, n);
               } else {
                 // next S as soon as the present one is in registers, then P V
                 look_ahead();
-                if (j < n0) WAIT2S(&mi.s_read[0], full_par(np[0]), W2_SREAD);
+                if (j < n0) is.wait_s_read(0);
                 next_s(0, n0);
-                WAIT2S(&mi.s_read[1], full_par(np[1]), W2_SREAD);
+                is.wait_s_read(1);
                 next_s(1, n);
-                if (more) commit<D>(&mi.kv_free[(kv + 1) % NS]);
-                const uint32_t v_u32 = wait_kv(kv);
-                if (j < n0) pv(0, v_u32, j == 0, j == n0 - 1);
-                pv(1, v_u32, j == 0, j == n - 1);
+                if (more) is.free_kv(is.kv + 1);
+                const uint32_t v_u32 = is.wait_kv(is.kv);
+                if (j < n0) is.pv(0, v_u32, j == 0, j == n0 - 1);
+                is.pv(1, v_u32, j == 0, j == n - 1);
               }
-              commit<D>(&mi.kv_free[kv % NS]);
-              if (PAIR && more) commit<D>(&mi.kv_free[(kv + 1) % NS]);
-              kv += more ? 2 : 1;
+              is.free_kv(is.kv);
+              if (!C::SEP_P && more) is.free_kv(is.kv + 1);
+              is.kv += more ? 2 : 1;
             }
             primed = nx.kind == KIND_FLASH;
             d = nx;
@@ -535,34 +281,30 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             // ---- score sweep, one pass: S^T = K_j Qw^T.  Its two [128 keys x 256 rows] buffers overlay all of TMEM:
             // every S / P buffer is consumed and the accumulators have been read out once o_free completes.
             const int n_steps = ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
-            for (int b = 0; b < 2; ++b) WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE);
-            for (int b = 0; b < 3 - NCTA; ++b) {
-              qa[b] = q_u32 + (nq % NQ) * Q_BYTES;
-              WAIT2S(&mi.q_full[nq % NQ], full_par(nq / NQ), W2_QFULL);
-              ++nq;
-            }
+            for (int b = 0; b < 2; ++b) WAIT2S(&mi.o_free[b], free_par(is.no[b]), W2_OFREE);
+            for (int b = 0; b < 3 - NCTA; ++b) is.qa[b] = is.wait_q();
             for (int jj = 0; jj < n_steps; ++jj, ++nt) {
               const int e = nt & 1;
               WAIT2S(&mi.t_free[e], free_par(nt >> 1), W2_TFREE);
-              const uint32_t k_u32 = wait_kv(kv);
+              const uint32_t k_u32 = is.wait_kv(is.kv);
               if constexpr (PAIR) {
-                wait_kv(kv + 1);
+                is.wait_kv(is.kv + 1);
                 tc_fence_after_sync();
-                mma_ss_pair_k128<false>(cx.tmem + e * 256, k_u32, qa[0], idesc_sw);
+                mma_ss_pair_k128<false>(cx.tmem + e * 256, k_u32, is.qa[0], idesc_sw);
               } else {
                 tc_fence_after_sync();
-                for (int b = 0; b < 2; ++b) mma_ss_k64(cx.tmem + e * 256 + b * 128, k_u32, qa[b], idesc_sw);
+                for (int b = 0; b < 2; ++b) mma_ss_k64(cx.tmem + e * 256 + b * 128, k_u32, is.qa[b], idesc_sw);
               }
-              commit<D>(&mi.t_full[e]);
-              for (int a = 0; a < Cfg<D>::ATOMS; ++a, ++kv) commit<D>(&mi.kv_free[kv % NS]);
+              commit<C>(&mi.t_full[e]);
+              for (int a = 0; a < C::ATOMS; ++a) is.free_kv(is.kv++);
             }
             // what follows overwrites the sweep buffers: wait until both were read
             WAIT2S(&mi.t_free[nt & 1], free_par(nt >> 1), W2_TFREE);
             WAIT2S(&mi.t_free[(nt + 1) & 1], free_par((nt + 1) >> 1), W2_TFREE);
-            d = next_desc<D>(cx, nd, false);
+            d = next_desc<C>(cx, is.nd, false);
           }
         }
-        commit<D>(&mi.mma_done);                                 // teardown waits for everything this thread issued
+        commit<C>(&mi.mma_done);                                 // teardown waits for everything this thread issued
       }
       __syncwarp();
     }
@@ -575,15 +317,15 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
     uint32_t nd = 0, nq = 0, no[2] = {0, 0};
     while (true) {
-      const Desc d = next_desc<D>(cx, nd, true);
+      const Desc d = next_desc<C>(cx, nd, true);
       if (d.kind == KIND_DONE) break;
       if (d.kind == KIND_SWEEP) {
         if (d.h[0] == 0) {                                       // the window rows' log-sum-exp of this CTA's blocks is in memory
           __threadfence();
           __syncwarp();
           if (lane == 0) {
-            mbar_arrive_cluster(in_cta<D>(&mi.lse_rdy, 0));
-            if (PAIR) mbar_arrive_cluster(in_cta<D>(&mi.lse_rdy, 1));
+            mbar_arrive_cluster(in_cta<C>(&mi.lse_rdy, 0));
+            if (PAIR) mbar_arrive_cluster(in_cta<C>(&mi.lse_rdy, 1));
           }
         }
         nq += 3 - NCTA;
@@ -605,7 +347,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         tc_fence_after_sync();
         const bool in_chunk = token >= 0 && token < d.len;       // rows behind the end of the chunk are written as zeros
         const float inv_l = in_chunk ? 1.0f / l_run : 0.0f;
-        const uint32_t tO = cx.tmem + TM_O + b * D + lane_sel;
+        const uint32_t tO = cx.tmem + C::TM_O + b * D + lane_sel;
 #pragma unroll 1
         for (int q = 0; q < D / 32; ++q) {
           uint32_t o[32];
@@ -622,7 +364,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             *reinterpret_cast<uint4*>(myQ + (col / 64) * 16384 + sw128_offset(r, (col % 64) / 8)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
         }
-        warp_arrive_leader(in_cta<D>(&mi.o_free[b], 0));
+        warp_arrive_leader(in_cta<C>(&mi.o_free[b], 0));
         if (in_chunk) {
           const float lse2 = m_used + log2f(l_run);
           const size_t row = (size_t)d.c * prm.Hq + h;
@@ -634,7 +376,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         named_barrier_sync(1, 128);
         if (r == 0) {
           if (t >= 0 && t * TILE < prm.L) {
-            for (int a = 0; a < Cfg<D>::ATOMS; ++a) tma_store_4d(&tm_o, myQ + a * 16384, a * 64, h, t * TILE, d.c);
+            for (int a = 0; a < C::ATOMS; ++a) tma_store_4d(&tm_o, myQ + a * 16384, a * 64, h, t * TILE, d.c);
             tma_store_commit();
             tma_store_wait_read();
           }
@@ -650,26 +392,13 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const int b = warp >> 2;
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tS = cx.tmem + b * 128 + lane_sel, tO = cx.tmem + TM_O + b * D + lane_sel;
-    const uint32_t tP = PAIR ? tS : cx.tmem + TM_P + b * 64 + lane_sel;
+    const uint32_t tS = cx.tmem + b * 128 + lane_sel, tO = cx.tmem + C::TM_O + b * D + lane_sel;
+    const uint32_t tP = C::SEP_P ? cx.tmem + C::TM_P + b * 64 + lane_sel : tS;
     const float scale_log2 = prm.scale_log2;
-    struct Hooks {
-      const Ctx2& cx;
-      uint32_t p_half, p_full, s_read;                           // barriers (of the leader CTA)
-      uint64_t* pv_done;
-      uint32_t tiles;                                            // tiles of this block before the present one
-      __device__ __forceinline__ void on_read() const { if (!PAIR) warp_arrive_leader(s_read); }
-      // pair: S of this tile was issued after P V of the tile before, and P overwrites S, which is in registers
-      __device__ __forceinline__ void before_p() const {
-        if (!PAIR && tiles > 0) { WAIT2S(pv_done, full_par(tiles - 1), W2_PV); tc_fence_after_sync(); }
-      }
-      __device__ __forceinline__ void before_rescale() const { before_p(); }
-      __device__ __forceinline__ void on_half() const { warp_arrive_leader(p_half); }
-      __device__ __forceinline__ void on_full() const { warp_arrive_leader(p_full); }
-    } hk = {cx, in_cta<D>(&mi.p_half[b], 0), in_cta<D>(&mi.p_full[b], 0), in_cta<D>(&mi.s_read[b], 0), &mi.pv_done[b], 0};
+    Hooks<C> hk(cx, b);
     uint32_t nd = 0, n_s = 0, n_blk = 0, nq = 0, nt = 0, n_lse = 0;
     while (true) {
-      const Desc d = next_desc<D>(cx, nd, true);
+      const Desc d = next_desc<C>(cx, nd, true);
       if (d.kind == KIND_DONE) break;
       if (d.kind == KIND_FLASH) {
         nq += d.n[0] > 0 ? 2 : 1;
@@ -714,7 +443,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const int n_steps = ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
         const int w0 = d.len - prm.w, pad = sch.wp - prm.w;      // first window token of this chunk
         float* const xch = &mi.lm[0][0][0];                      // [buffer][key]
-        const uint32_t t_free0 = in_cta<D>(&mi.t_free[0], 0), t_free1 = in_cta<D>(&mi.t_free[1], 0);
+        const uint32_t t_free0 = in_cta<C>(&mi.t_free[0], 0), t_free1 = in_cta<C>(&mi.t_free[1], 0);
         for (int jj = 0; jj < n_steps; ++jj, ++nt) {
           const int e = nt & 1;
           WAIT2S(&mi.t_full[e], full_par(nt >> 1), W2_TFULL);
@@ -777,18 +506,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   }
 
-  // ---- teardown: no CTA of a pair may exit while its peer can still signal it or read its shared memory
-  tc_fence_before_sync();
-  __syncthreads();
-  if constexpr (PAIR) cluster_sync_all();
-  if (warp == WARP_MMA) {
-    // no tensor-core operation may still be running when its accumulators are freed: the issuer ended with a
-    // commit to mma_done (an arrival in both CTAs of a pair).  Immediate in a clean run; after an abort this is what
-    // makes the exit safe.  The wait ignores the abort flag and is bounded.
-    mbar_wait_drain(&mi.mma_done, 0, cx.abort_flag);
-    tc_fence_after_sync();
-    if constexpr (PAIR) tmem_dealloc_pair(cx.tmem, 512); else tmem_dealloc(cx.tmem, 512);
-  }
+  teardown<C>(cx);
 }
 
 // ====================================================================================
@@ -798,8 +516,8 @@ template <int D>
 static cudaError_t launch_prefill_t(const CUtensorMap* maps, const PrefillParams& prm, int sm_count, cudaStream_t st) {
   // the opt-in to large dynamic shared memory is a per-device attribute of the function: set it on every call
   // (a host-side call of a few hundred nanoseconds) rather than remember which devices have it
-  if (cudaError_t e = cudaFuncSetAttribute(prefill_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Off<D>::TOTAL); e != cudaSuccess) return e;
-  constexpr int NCTA = Cfg<D>::NCTA;
+  if (cudaError_t e = cudaFuncSetAttribute(prefill_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Off<PCfg<D>>::TOTAL); e != cudaSuccess) return e;
+  constexpr int NCTA = PCfg<D>::NCTA;
   const int grid = sm_count / NCTA * NCTA;               // one CTA per SM, a whole number of pairs
   if (grid < 1) return cudaErrorInvalidConfiguration;
   cudaLaunchAttribute attr[1];
@@ -808,7 +526,7 @@ static cudaError_t launch_prefill_t(const CUtensorMap* maps, const PrefillParams
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(NT2);
-  cfg.dynamicSmemBytes = Off<D>::TOTAL;
+  cfg.dynamicSmemBytes = Off<PCfg<D>>::TOTAL;
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;

@@ -447,6 +447,12 @@ __device__ __forceinline__ void mma_ss_k64(uint32_t d_tmem, uint32_t a_smem, uin
   asm volatile(PC_SS_REGS PC_MMA_SS0(1) PC_MMA_SS(1, 2, 2) PC_MMA_SS(1, 4, 4) PC_MMA_SS(1, 6, 6) "}\n"
                ::"r"(d_tmem), "r"(desc_lo(a_smem, 16)), "r"(desc_lo(b_smem, 16)), "r"(DESC_HI), "r"(idesc) : "memory");
 }
+// the same over 128 elements, operands of 128 rows
+__device__ __forceinline__ void mma_ss_k128(uint32_t d_tmem, uint32_t a_smem, uint32_t b_smem, uint32_t idesc) {
+  asm volatile(PC_SS_REGS PC_MMA_SS0(1) PC_MMA_SS(1, 2, 2) PC_MMA_SS(1, 4, 4) PC_MMA_SS(1, 6, 6)
+               PC_MMA_SS(1, 1024, 1024) PC_MMA_SS(1, 1026, 1026) PC_MMA_SS(1, 1028, 1028) PC_MMA_SS(1, 1030, 1030) "}\n"
+               ::"r"(d_tmem), "r"(desc_lo(a_smem, 16)), "r"(desc_lo(b_smem, 16)), "r"(DESC_HI), "r"(idesc) : "memory");
+}
 // S = A B^T over 128 elements on a CTA pair; A 128 rows per CTA, B 64 rows (B64) or up to 128 rows per CTA
 template <bool B64>
 __device__ __forceinline__ void mma_ss_pair_k128(uint32_t d_tmem, uint32_t a_smem, uint32_t b_smem, uint32_t idesc) {
