@@ -122,6 +122,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
       mi.abort_flag = 0;
       mi.wait_kcycles = prm.wait_kcycles;
       fence_mbar_init();
+      chain();
       for (uint32_t kv = 0; kv < n_first; ++kv) load_half(kv);
     }
     __syncwarp();
@@ -134,10 +135,13 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
     auto q_slot = [&](int r, int e) -> uint16_t* {
       return reinterpret_cast<uint16_t*>(smem + Y::OFF_Q + (e / 64) * (N * 128) + sw128_offset(r, (e % 64) / 8) + (e % 8) * 2);
     };
+    double sn = 0.0, cs = 0.0;
+    auto turn = [&](int e) { sincos((double)(prm.q_pos0 + e / HALF) * pow((double)prm.rope_theta, -2.0 * (double)(e % HALF) / (double)D), &sn, &cs); };
+    if (rt < w * HALF) turn(rt);                              // needs nothing from before this launch
+    chain();
     for (int e = rt; e < w * HALF; e += NTD - 32) {
       const int i = e / HALF, t = e % HALF;
-      double sn, cs;
-      sincos((double)(prm.q_pos0 + i) * pow((double)prm.rope_theta, -2.0 * (double)t / (double)D), &sn, &cs);
+      if (e != rt) turn(e);
       for (int g = 0; g < G; ++g) {
         const uint16_t* const x = qs + ((size_t)i * prm.Hq + g) * D + t;
         const double a = (double)__uint_as_float((uint32_t)x[0] << 16), b = (double)__uint_as_float((uint32_t)x[HALF] << 16);
@@ -392,18 +396,8 @@ static cudaError_t launch_decode_t(const CUtensorMap* maps, const DecodeParams& 
   if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM); e != cudaSuccess) return e;
   if (prm.n_split > 8)
     if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)prm.n_split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(prm.B * prm.Hkv * prm.n_split));
-  cfg.blockDim = dim3(NTD);
-  cfg.dynamicSmemBytes = SMEM;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  note_launch();
-  return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], prm);
+  return launch_chained(kernel, dim3((unsigned)(prm.B * prm.Hkv * prm.n_split)), dim3(NTD), SMEM, st, prm.n_split, maps[0], maps[1], maps[2],
+                        maps[3], prm);
 }
 
 cudaError_t launch_decode_attn(const CUtensorMap* maps, const DecodeParams& prm, int d, cudaStream_t st) {

@@ -10,6 +10,35 @@ namespace pc {
 // Every kernel launch of the library is counted here (see pc_launch_count in pc.h).
 void note_launch();
 
+// Launches of one call, and of calls on one stream, follow each other closely: every kernel is launched with programmatic
+// stream serialisation, so that it is set up while its predecessor drains, and begins with chain() (kernels with a
+// costly start after that start), which waits until everything before it on the stream has completed and then lets
+// its successor be set up.  The successor is released AFTER the wait: at most two kernels overlap, so a kernel never
+// shares an SM's L1 with a reader of the data that its predecessor replaces.
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, A... args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  note_launch();
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
+#endif
+
 // ---- pc_rope.cu
 // cos/sin table: tab[p * (d/2) + t] = (cos, sin)(  (pos0 + p) * theta^(-2t/d) ), fp64; tab_hi, tab_lo (may be null): the
 // same entries split into an fp32 head and an fp32 tail (value = head + tail to 2^-48), one float4 per two pairs:

@@ -64,6 +64,7 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
   Ctx2 cx;
   setup<C>(cx, smem, prm.status, prm.wait_kcycles, leader);
   Misc2& mi = *cx.mi;
+  chain();
 
   if (warp >= WARP_PRODUCER) {
     setmaxnreg_dec<REGS_SERVICE>();
@@ -319,6 +320,7 @@ template <int D>
 __global__ void __launch_bounds__(128) parallel_merge_kernel(const float* __restrict__ part_o, const float* __restrict__ part_ml,
                                                              int n_rows, int w, int Hq, int n_split,
                                                              __nv_bfloat16* __restrict__ out, float* __restrict__ lse_out) {
+  chain();
   const int row = blockIdx.x * 4 + (threadIdx.x >> 5);                       // (seq * Hq + h) * w + i
   const int lane = threadIdx.x & 31;
   if (row >= n_rows) return;
@@ -368,25 +370,13 @@ static cudaError_t launch_parallel_t(const CUtensorMap* maps, const ParallelPara
   const long long n_items = (long long)prm.B * prm.Hkv * prm.n_rg * prm.n_split;
   const int units = sm_count / C::NCTA;
   if (units < 1) return cudaErrorInvalidConfiguration;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = C::NCTA; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n_items < units ? (int)n_items : units) * C::NCTA));
-  cfg.blockDim = dim3(NT2);
-  cfg.dynamicSmemBytes = Off<C>::TOTAL;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  note_launch();
-  if (cudaError_t e = cudaLaunchKernelEx(&cfg, parallel_attn_kernel<D, PAIR>, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
+  if (cudaError_t e = launch_chained(parallel_attn_kernel<D, PAIR>, dim3((unsigned)((n_items < units ? (int)n_items : units) * C::NCTA)), dim3(NT2),
+                                     Off<C>::TOTAL, st, C::NCTA, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
       e != cudaSuccess) return e;
   if (prm.n_split > 1) {
     const int rows = prm.B * prm.Hq * prm.w;
-    note_launch();
-    parallel_merge_kernel<D><<<(rows + 3) / 4, 128, 0, st>>>(prm.part_o, prm.part_ml, rows, prm.w, prm.Hq, prm.n_split, prm.out,
-                                                             prm.lse_out);
-    return cudaGetLastError();
+    return launch_chained(parallel_merge_kernel<D>, dim3((rows + 3) / 4), dim3(128), 0, st, 1, prm.part_o, prm.part_ml, rows, prm.w, prm.Hq,
+                          prm.n_split, prm.out, prm.lse_out);
   }
   return cudaSuccess;
 }

@@ -128,6 +128,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   Ctx2 cx;
   setup<C>(cx, smem, prm.status, prm.wait_kcycles, leader);
   Misc2& mi = *cx.mi;
+  chain();
 
   if (warp >= WARP_PRODUCER) {
     setmaxnreg_dec<REGS_SERVICE>();
@@ -520,18 +521,8 @@ static cudaError_t launch_prefill_t(const CUtensorMap* maps, const PrefillParams
   constexpr int NCTA = PCfg<D>::NCTA;
   const int grid = sm_count / NCTA * NCTA;               // one CTA per SM, a whole number of pairs
   if (grid < 1) return cudaErrorInvalidConfiguration;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = NCTA; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(NT2);
-  cfg.dynamicSmemBytes = Off<PCfg<D>>::TOTAL;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  note_launch();
-  return cudaLaunchKernelEx(&cfg, prefill_kernel<D>, maps[0], maps[5], maps[1], maps[2], maps[3], maps[4], prm);
+  return launch_chained(prefill_kernel<D>, dim3((unsigned)grid), dim3(NT2), Off<PCfg<D>>::TOTAL, st, NCTA, maps[0], maps[5], maps[1], maps[2],
+                        maps[3], maps[4], prm);
 }
 
 // maps: 0 q (box 64 x 128 tokens), 1 rotated keys (64 x 128), 2 v (64 x 128), 3 o (store), 4 q with a

@@ -17,6 +17,7 @@ constexpr int QUEUE_MAX = 1024;                                // slots + chunks
 constexpr int EMPTY_ID = 0x7FFFFFFF;                           // an empty slot loses every tie
 
 __global__ void queue_init_kernel(float* q_score, int* q_chunk, int m) {
+  chain();
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     q_score[i] = 0.0f;
     q_chunk[i] = -1;
@@ -24,8 +25,7 @@ __global__ void queue_init_kernel(float* q_score, int* q_chunk, int m) {
 }
 
 void launch_queue_init(float* q_score, int* q_chunk, int m, cudaStream_t st) {
-  note_launch();
-  queue_init_kernel<<<1, 256, 0, st>>>(q_score, q_chunk, m);
+  launch_chained(queue_init_kernel, dim3(1), dim3(256), 0, st, 1, q_score, q_chunk, m);
 }
 
 // Candidates 0..m-1 are the slots, m..m+Cb-1 the chunks of the batch.  A candidate survives when fewer
@@ -34,6 +34,7 @@ void launch_queue_init(float* q_score, int* q_chunk, int m, cudaStream_t st) {
 __global__ void __launch_bounds__(QUEUE_MAX) queue_update_kernel(const float* __restrict__ score, int Cb, int chunk_id0,
                                                                  int lower_is_better, int m, float* __restrict__ q_score,
                                                                  int* __restrict__ q_chunk, int* __restrict__ slot_src) {
+  chain();
   __shared__ uint32_t key[QUEUE_MAX];
   __shared__ int id[QUEUE_MAX];
   __shared__ int keep[QUEUE_MAX];
@@ -82,13 +83,13 @@ __global__ void __launch_bounds__(QUEUE_MAX) queue_update_kernel(const float* __
 
 void launch_queue_update(const float* score, int Cb, int chunk_id0, int lower_is_better, int m, float* q_score,
                          int* q_chunk, int* slot_src, cudaStream_t st) {
-  note_launch();
-  queue_update_kernel<<<1, QUEUE_MAX, 0, st>>>(score, Cb, chunk_id0, lower_is_better, m, q_score, q_chunk, slot_src);
+  launch_chained(queue_update_kernel, dim3(1), dim3(QUEUE_MAX), 0, st, 1, score, Cb, chunk_id0, lower_is_better, m, q_score, q_chunk, slot_src);
 }
 
 // slot_order[i] = the slot holding the i-th smallest chunk id (-1 past the filled slots); kept_out[i] = that id.
 __global__ void __launch_bounds__(QUEUE_MAX) queue_order_kernel(const int* __restrict__ q_chunk, int m,
                                                                 int* __restrict__ kept_out, int* __restrict__ slot_order) {
+  chain();
   __shared__ int id[QUEUE_MAX];
   const int i = threadIdx.x;
   if (i < m) {
@@ -112,6 +113,7 @@ __global__ void __launch_bounds__(256) queue_emit_kernel(const uint4* __restrict
                                                          const int* __restrict__ q_pos, const int* __restrict__ slot_order,
                                                          int m, int Hkv, int k, uint4* __restrict__ k_out,
                                                          uint4* __restrict__ v_out, int* __restrict__ pos_out) {
+  chain();
   constexpr int LPR = D / 8;
   const long long n_rows = (long long)Hkv * m * k;
   const long long gthreads = (long long)gridDim.x * blockDim.x;
@@ -138,19 +140,17 @@ __global__ void __launch_bounds__(256) queue_emit_kernel(const uint4* __restrict
 cudaError_t launch_queue_emit(const int* q_chunk, int m, int Hkv, int k, int d, const void* q_k, const void* q_v,
                               const int* q_pos, int* kept_out, int* slot_order, void* k_out, void* v_out, int* pos_out,
                               int sm_count, cudaStream_t st) {
-  note_launch();
-  queue_order_kernel<<<1, QUEUE_MAX, 0, st>>>(q_chunk, m, kept_out, slot_order);
+  launch_chained(queue_order_kernel, dim3(1), dim3(QUEUE_MAX), 0, st, 1, q_chunk, m, kept_out, slot_order);
   const long long n_rows = (long long)Hkv * m * k;
   const int lpr = d / 8;
   const long long want = (n_rows * lpr + 255) / 256;
   int blocks = (int)(want < (long long)sm_count * 8 ? want : (long long)sm_count * 8);
   if (blocks < 1) blocks = 1;
-  note_launch();
   if (d == 128)
-    queue_emit_kernel<128><<<blocks, 256, 0, st>>>((const uint4*)q_k, (const uint4*)q_v, q_pos, slot_order, m, Hkv, k,
+    launch_chained(queue_emit_kernel<128>, dim3(blocks), dim3(256), 0, st, 1, (const uint4*)q_k, (const uint4*)q_v, q_pos, slot_order, m, Hkv, k,
                                                    (uint4*)k_out, (uint4*)v_out, pos_out);
   else
-    queue_emit_kernel<64><<<blocks, 256, 0, st>>>((const uint4*)q_k, (const uint4*)q_v, q_pos, slot_order, m, Hkv, k,
+    launch_chained(queue_emit_kernel<64>, dim3(blocks), dim3(256), 0, st, 1, (const uint4*)q_k, (const uint4*)q_v, q_pos, slot_order, m, Hkv, k,
                                                   (uint4*)k_out, (uint4*)v_out, pos_out);
   return cudaGetLastError();
 }

@@ -13,16 +13,20 @@ namespace pc {
 __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict__ tab_hi, float4* __restrict__ tab_lo, int n_pos,
                                   int half, double theta, int pos0, int* __restrict__ counter) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;      // one thread per two pairs
-  if (i == 0 && counter != nullptr) *counter = 0;           // work queue of the attention kernel that follows
-  if (i >= n_pos * (half / 2)) return;
   const int p = i / (half / 2), t = 2 * (i % (half / 2));
+  const bool mine = i < n_pos * (half / 2);
   double c[2], s[2];
+  if (mine) {
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const double inv_freq = pow(theta, -2.0 * (double)(t + e) / (double)(2 * half));
-    sincos((double)(pos0 + p) * inv_freq, &s[e], &c[e]);
-    tab[(size_t)p * half + t + e] = make_double2(c[e], s[e]);
+    for (int e = 0; e < 2; ++e) {
+      const double inv_freq = pow(theta, -2.0 * (double)(t + e) / (double)(2 * half));
+      sincos((double)(pos0 + p) * inv_freq, &s[e], &c[e]);
+    }
   }
+  chain();                                                  // the arithmetic needs nothing from before; the tables may still be in use
+  if (i == 0 && counter != nullptr) *counter = 0;           // work queue of the attention kernel that follows
+  if (!mine) return;
+  for (int e = 0; e < 2; ++e) tab[(size_t)p * half + t + e] = make_double2(c[e], s[e]);
   if (tab_hi != nullptr) {
     const float c0 = (float)c[0], c1 = (float)c[1], s0 = (float)s[0], s1 = (float)s[1];
     tab_hi[i] = make_float4(c0, c1, s0, s1);
@@ -34,8 +38,7 @@ __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict_
 void launch_rope_table(double2* tab, float4* tab_hi, float4* tab_lo, int n_pos, int d, double theta, int pos0, int* counter,
                        cudaStream_t st) {
   const int n = n_pos * (d / 4);
-  note_launch();
-  rope_table_kernel<<<(n + 255) / 256, 256, 0, st>>>(tab, tab_hi, tab_lo, n_pos, d / 2, theta, pos0, counter);
+  launch_chained(rope_table_kernel, dim3((n + 255) / 256), dim3(256), 0, st, 1, tab, tab_hi, tab_lo, n_pos, d / 2, theta, pos0, counter);
 }
 
 // y[c,p,h,:] = bf16( RoPE(x[c,p,h,:], position p) ).  One warp owns one position: a lane holds 8 consecutive
@@ -59,6 +62,7 @@ struct RopeTensor {
 __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant__ RopeTensor ta, const __grid_constant__ RopeTensor tb,
                                                            const float4* __restrict__ tab_hi, const float4* __restrict__ tab_lo,
                                                            const double2* __restrict__ tab, int C, int L, int d) {
+  chain();
   const bool second_tensor = (int)blockIdx.y >= ta.ny;      // the same for the whole block
   const uint16_t* __restrict__ const x = second_tensor ? tb.x : ta.x;
   uint16_t* __restrict__ const y = second_tensor ? tb.y : ta.y;
@@ -165,8 +169,7 @@ void launch_rope_rows(const RopeRows& a, const RopeRows* b, const double2* tab, 
   const RopeTensor ta = rope_tensor(a, C, L, d);
   RopeTensor tb = {};
   if (b != nullptr) tb = rope_tensor(*b, C, L, d);
-  note_launch();
-  rope_rows_kernel<<<dim3((unsigned)((L + 7) / 8), (unsigned)(ta.ny + tb.ny), (unsigned)(ta.nz > tb.nz ? ta.nz : tb.nz)), 256, 0, st>>>(
+  launch_chained(rope_rows_kernel, dim3((unsigned)((L + 7) / 8), (unsigned)(ta.ny + tb.ny), (unsigned)(ta.nz > tb.nz ? ta.nz : tb.nz)), dim3(256), 0, st, 1, 
       ta, tb, tab_hi, tab_lo, tab, C, L, d);
 }
 
@@ -174,6 +177,7 @@ void launch_rope_rows(const RopeRows& a, const RopeRows* b, const double2* tab, 
 __global__ void zero_chunk_tails_kernel(const int* __restrict__ chunk_len, int L, int w, int Hq, int Hkv, int d,
                                         uint16_t* __restrict__ o, long long so_chunk, long long so_tok, long long so_head,
                                         float* __restrict__ lse, float* __restrict__ win_score) {
+  chain();
   const int c = blockIdx.y;
   int len = chunk_len[c];
   len = len > L ? L : (len <= w ? w + 1 : len);
@@ -195,8 +199,7 @@ __global__ void zero_chunk_tails_kernel(const int* __restrict__ chunk_len, int L
 
 void launch_zero_chunk_tails(const int* chunk_len, int C, int L, int w, int Hq, int Hkv, int d, void* o,
                              const long long o_stride[3], float* lse, float* win_score, cudaStream_t st) {
-  note_launch();
-  zero_chunk_tails_kernel<<<dim3(64, (unsigned)C), 256, 0, st>>>(chunk_len, L, w, Hq, Hkv, d, (uint16_t*)o, o_stride[0],
+  launch_chained(zero_chunk_tails_kernel, dim3(64, (unsigned)C), dim3(256), 0, st, 1, chunk_len, L, w, Hq, Hkv, d, (uint16_t*)o, o_stride[0],
                                                                 o_stride[1], o_stride[2], lse, win_score);
 }
 

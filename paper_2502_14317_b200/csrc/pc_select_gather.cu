@@ -8,6 +8,7 @@ namespace pc {
 
 // ------------------------------------------------------------------ chunk score stand-in
 __global__ void chunk_score_kernel(const float* __restrict__ win_lse, int n_per_chunk, float* __restrict__ score) {
+  chain();
   __shared__ double part[256];
   const int c = blockIdx.x;
   double acc = 0.0;
@@ -22,14 +23,14 @@ __global__ void chunk_score_kernel(const float* __restrict__ win_lse, int n_per_
 }
 
 void launch_chunk_score(const float* win_lse, int C, int n_per_chunk, float* score, cudaStream_t st) {
-  note_launch();
-  chunk_score_kernel<<<C, 256, 0, st>>>(win_lse, n_per_chunk, score);
+  launch_chained(chunk_score_kernel, dim3(C), dim3(256), 0, st, 1, win_lse, n_per_chunk, score);
 }
 
 // ------------------------------------------------------------------ chunk top-m
 // One block; thread i ranks chunk i against all others (C <= 1024).
 __global__ void select_chunks_kernel(const float* __restrict__ score, int C, int m, int lower_is_better,
                                      int* __restrict__ kept) {
+  chain();
   __shared__ uint32_t key[1024];
   __shared__ int flag[1024];
   const int i = threadIdx.x;
@@ -56,6 +57,7 @@ __global__ void select_chunks_kernel(const float* __restrict__ score, int C, int
 __global__ void __launch_bounds__(1024) score_select_chunks_kernel(const float* __restrict__ win_lse, int n_per_chunk, int C,
                                                                    int m, int lower_is_better, float* __restrict__ score,
                                                                    int* __restrict__ kept) {
+  chain();
   __shared__ double part[4][256];
   __shared__ uint32_t key[64];
   __shared__ int flag[64];
@@ -98,8 +100,7 @@ __global__ void __launch_bounds__(1024) score_select_chunks_kernel(const float* 
 void launch_score_select_chunks(const float* win_lse, int C, int n_per_chunk, int m, int lower_is_better, float* score,
                                 int* kept, cudaStream_t st) {
   if (C <= 64) {
-    note_launch();
-    score_select_chunks_kernel<<<1, 1024, 0, st>>>(win_lse, n_per_chunk, C, m, lower_is_better, score, kept);
+    launch_chained(score_select_chunks_kernel, dim3(1), dim3(1024), 0, st, 1, win_lse, n_per_chunk, C, m, lower_is_better, score, kept);
   } else {
     launch_chunk_score(win_lse, C, n_per_chunk, score, st);
     launch_select_chunks(score, C, m, lower_is_better, kept, st);
@@ -107,8 +108,7 @@ void launch_score_select_chunks(const float* win_lse, int C, int n_per_chunk, in
 }
 
 void launch_select_chunks(const float* score, int C, int m, int lower_is_better, int* kept, cudaStream_t st) {
-  note_launch();
-  select_chunks_kernel<<<1, 1024, 0, st>>>(score, C, m, lower_is_better, kept);
+  launch_chained(select_chunks_kernel, dim3(1), dim3(1024), 0, st, 1, score, C, m, lower_is_better, kept);
 }
 
 // ------------------------------------------------------------------ token top-k
@@ -200,6 +200,7 @@ __global__ void __launch_bounds__(SMALL ? 256 : SEL_MAX_THREADS, SMALL ? SEL_SMA
                                                                         const int* __restrict__ kept, int Hkv, int L,
                                                                         int n_cand, int k, int* __restrict__ idx,
                                                                         const SelCalib cal, const SelGather ga = SelGather()) {
+  chain();
   extern __shared__ int sel_stage[];                           // STAGE: [min(k, n_cand)]
   __shared__ int s_part[2][32];                                // [round parity][warp]: undecided keys of the warp with the bit set
   __shared__ int s_tot[2][32];
@@ -403,13 +404,12 @@ cudaError_t launch_select_tokens(const float* win_score, const int* kept, int m,
   const int grid = m * Hkv;
 #define PC_SELECT(C, S)                                                                                               \
   do {                                                                                                                \
-    note_launch();                                                                                                    \
     if (threads <= 256)                                                                                               \
-      select_tokens_kernel<C, S, true><<<grid, threads, S ? stage_bytes : 0, st>>>(win_score, kept, Hkv, L, n_cand, k, \
-                                                                                    idx, cal);                        \
+      launch_chained(select_tokens_kernel<C, S, true>, dim3(grid), dim3(threads), S ? stage_bytes : 0, st, 1, win_score, kept, Hkv, L, n_cand, k, \
+                     idx, cal, SelGather());                        \
     else                                                                                                              \
-      select_tokens_kernel<C, S, false><<<grid, threads, S ? stage_bytes : 0, st>>>(win_score, kept, Hkv, L, n_cand,   \
-                                                                                     k, idx, cal);                    \
+      launch_chained(select_tokens_kernel<C, S, false>, dim3(grid), dim3(threads), S ? stage_bytes : 0, st, 1, win_score, kept, Hkv, L, n_cand,   \
+                     k, idx, cal, SelGather());                    \
   } while (0)
   if (calib) {
     if (stage) PC_SELECT(true, true); else PC_SELECT(true, false);
@@ -436,12 +436,11 @@ cudaError_t launch_select_gather_slots(const float* win_score, const int* slot_s
   ga.s_chunk = stride_elems[0] / 8; ga.s_tok = stride_elems[1] / 8; ga.s_head = stride_elems[2] / 8;
   ga.k_out = (uint4*)q_k; ga.v_out = (uint4*)q_v; ga.pos_out = q_pos;
   ga.lpr = d / 8;
-  note_launch();
   if (threads <= 256)
-    select_tokens_kernel<false, true, true, true><<<m * Hkv, threads, stage_bytes, st>>>(win_score, slot_src, Hkv, L, n_cand, k,
+    launch_chained(select_tokens_kernel<false, true, true, true>, dim3(m * Hkv), dim3(threads), stage_bytes, st, 1, win_score, slot_src, Hkv, L, n_cand, k,
                                                                                         nullptr, cal, ga);
   else
-    select_tokens_kernel<false, true, false, true><<<m * Hkv, threads, stage_bytes, st>>>(win_score, slot_src, Hkv, L, n_cand, k,
+    launch_chained(select_tokens_kernel<false, true, false, true>, dim3(m * Hkv), dim3(threads), stage_bytes, st, 1, win_score, slot_src, Hkv, L, n_cand, k,
                                                                                          nullptr, cal, ga);
   return cudaGetLastError();
 }
@@ -457,6 +456,7 @@ __global__ void __launch_bounds__(256) gather_kv_kernel(const uint4* __restrict_
                                                         const int* __restrict__ kept, const int* __restrict__ idx, int m,
                                                         int Hkv, int k, uint4* __restrict__ k_out,
                                                         uint4* __restrict__ v_out, int* __restrict__ pos_out) {
+  chain();
   constexpr int LPR = D / 8;                                   // lanes per row
   const long long n_rows = (long long)Hkv * m * k;
   const long long gthreads = (long long)gridDim.x * blockDim.x;
@@ -490,9 +490,8 @@ cudaError_t launch_gather_kv(const void* k_src, const void* v_src, const long lo
   if (blocks < 1) blocks = 1;
   const long long sc = stride_elems[0] / 8, stok = stride_elems[1] / 8, sh = stride_elems[2] / 8;
 #define PC_GATHER(D, S)                                                                                              \
-  gather_kv_kernel<D, S><<<blocks, 256, 0, st>>>((const uint4*)k_src, (const uint4*)v_src, sc, stok, sh, kept, idx, m, \
+  launch_chained(gather_kv_kernel<D, S>, dim3(blocks), dim3(256), 0, st, 1, (const uint4*)k_src, (const uint4*)v_src, sc, stok, sh, kept, idx, m, \
                                                  Hkv, k, (uint4*)k_out, (uint4*)v_out, pos_out)
-  note_launch();
   if (d == 128) {
     if (by_slot) PC_GATHER(128, true); else PC_GATHER(128, false);
   } else {
@@ -507,6 +506,7 @@ cudaError_t launch_gather_kv(const void* k_src, const void* v_src, const long lo
 __global__ void append_kv_kernel(const uint4* __restrict__ k_win, const uint4* __restrict__ v_win, int B, int w, int Hkv,
                                  int lpr, long long Nk, long long Nk_cap, uint4* __restrict__ k_cache,
                                  uint4* __restrict__ v_cache) {
+  chain();
   const long long n = (long long)B * w * Hkv * lpr;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const int piece = (int)(i % lpr);
@@ -525,8 +525,7 @@ cudaError_t launch_append_kv(const void* k_win, const void* v_win, int B, int w,
   const int lpr = d / 8;
   const long long n = (long long)B * w * Hkv * lpr;
   const int blocks = (int)((n + 255) / 256 < 1184 ? (n + 255) / 256 : 1184);
-  note_launch();
-  append_kv_kernel<<<blocks < 1 ? 1 : blocks, 256, 0, st>>>((const uint4*)k_win, (const uint4*)v_win, B, w, Hkv, lpr, Nk, Nk_cap,
+  launch_chained(append_kv_kernel, dim3(blocks < 1 ? 1 : blocks), dim3(256), 0, st, 1, (const uint4*)k_win, (const uint4*)v_win, B, w, Hkv, lpr, Nk, Nk_cap,
                                                         (uint4*)k_cache, (uint4*)v_cache);
   return cudaGetLastError();
 }
