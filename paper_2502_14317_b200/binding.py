@@ -124,6 +124,20 @@ def _stream():
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
+def _like(t, shape):
+    """New contiguous bf16 tensor on t's device (empty_like is the cheapest way to get one)."""
+    if t.dtype is torch.bfloat16 and t.shape == shape and t.is_contiguous():
+        return torch.empty_like(t)
+    return t.new_empty(shape, dtype=torch.bfloat16)
+
+
+def _window(t, L, w):
+    """The window rows of chunk 0, [1,w,H,d], contiguous: a view where the storage allows it."""
+    s = t.stride()
+    v = t.as_strided((1, w, t.shape[2], t.shape[3]), s, t.storage_offset() + (L - w) * s[1])
+    return v if v.is_contiguous() else v.contiguous()
+
+
 def _need_cuda(*tensors):
     for t in tensors:
         if t is not None and not t.is_cuda:
@@ -159,9 +173,9 @@ def chunk_prefill_attn(q, k, v, *, w, rope_theta, softmax_scale=0.0, want_lse=Fa
     C, L, Hq, d = q.shape
     Hkv = k.shape[2]
     dev = q.device
-    o = q.new_empty((C, L, Hq, d)) if out is None else out
+    o = _like(q, q.shape) if out is None else out
     if k_rot is None:
-        k_rot = k.new_empty((C, L, Hkv, d))
+        k_rot = _like(k, k.shape)
     if win_score is None:
         win_score = torch.empty((C, Hkv, L), dtype=torch.float32, device=dev)
     if win_lse is None:
@@ -268,8 +282,8 @@ def gather_kv(k_src, v_src, kept, idx, k_out=None, v_out=None, pos_out=None, wan
     dev = k_src.device
     if k_src.stride() != v_src.stride() or k_src.stride(3) != 1:
         raise PcError("k_src and v_src must share strides with a contiguous head dimension")
-    k_out = torch.empty((Hkv, m * k, d), dtype=torch.bfloat16, device=dev) if k_out is None else k_out
-    v_out = torch.empty((Hkv, m * k, d), dtype=torch.bfloat16, device=dev) if v_out is None else v_out
+    k_out = _like(k_src, (Hkv, m * k, d)) if k_out is None else k_out
+    v_out = _like(k_out, (Hkv, m * k, d)) if v_out is None else v_out
     if pos_out is None and want_pos:
         pos_out = torch.empty((Hkv, m * k), dtype=torch.int32, device=dev)
     strides = (c_int64 * 3)(k_src.stride(0), k_src.stride(1), k_src.stride(2))
@@ -372,7 +386,7 @@ def parallel_attn(q_win, k_cache, v_cache, k_win, v_win, *, q_pos0, rope_theta, 
     for t in (q_win, k_cache, v_cache, k_win, v_win):
         if not t.is_contiguous():
             raise PcError("pc_parallel_attn takes contiguous tensors")
-    out = torch.empty((B, w, Hq, d), dtype=torch.bfloat16, device=dev) if out is None else out
+    out = _like(q_win, q_win.shape) if out is None else out
     if lse_out is None and want_lse:
         lse_out = torch.empty((B, Hq, w), dtype=torch.float32, device=dev)
     if status is None:
@@ -399,7 +413,7 @@ def parallel_attn_append(q_win, k_cache, v_cache, n_valid, k_win, v_win, *, q_po
     for t in (q_win, k_cache, v_cache, k_win, v_win):
         if not t.is_contiguous():
             raise PcError("pc_parallel_attn_append takes contiguous tensors")
-    out = torch.empty((B, w, Hq, d), dtype=torch.bfloat16, device=dev) if out is None else out
+    out = _like(q_win, q_win.shape) if out is None else out
     if lse_out is None and want_lse:
         lse_out = torch.empty((B, Hq, w), dtype=torch.float32, device=dev)
     if status is None:
@@ -462,12 +476,8 @@ def hot_path(q, k, v, *, w, rope_theta, m, k_keep, softmax_scale=0.0, chunk_scor
         score, kept = score_select_chunks(pre["win_lse"], m, True, score_out=b.get("chunk_score"), kept_out=b.get("kept"))
     idx = select_tokens(pre["win_score"], kept, L - w, k_keep, out=b.get("idx"))
     kc, vc, pos = gather_kv(pre["k_rot"], v, kept, idx, k_out=b.get("kc"), v_out=b.get("vc"), pos_out=b.get("pos"))
-    # the window is the same in every chunk: take it from chunk 0 (views, no copy)
-    q_win = q[0:1, L - w:].contiguous() if not q[0:1, L - w:].is_contiguous() else q[0:1, L - w:]
-    k_win = pre["k_rot"][0:1, L - w:]
-    v_win = v[0:1, L - w:]
-    if not v_win.is_contiguous():
-        v_win = v_win.contiguous()
+    # the window is the same in every chunk: take it from chunk 0
+    q_win, k_win, v_win = (_window(t, L, w) for t in (q, pre["k_rot"], v))
     pa = parallel_attn(q_win, kc.unsqueeze(0), vc.unsqueeze(0), k_win, v_win, q_pos0=L - w, rope_theta=rope_theta,
                        softmax_scale=softmax_scale, out=b.get("fg"), status=pre["status"], workspace=b.get("ws_par"))
     res = {"o": pre["o"], "k_rot": pre["k_rot"], "win_score": pre["win_score"], "win_lse": pre["win_lse"],
@@ -553,10 +563,7 @@ def hot_path_streaming(q, k, v, *, w, rope_theta, m, k_keep, batch=None, softmax
         c0 += n
     kept, kc, vc, pos = queue_emit(qu, k_out=b.get("kc"), v_out=b.get("vc"), pos_out=b.get("pos"), kept_out=b.get("kept"))
     b.update({"kc": kc, "vc": vc, "pos": pos, "kept": kept})
-    q_win = q0[0:1, L0 - w:]
-    q_win = q_win if q_win.is_contiguous() else q_win.contiguous()
-    v_win = v0[0:1, L0 - w:]
-    v_win = v_win if v_win.is_contiguous() else v_win.contiguous()
+    q_win, v_win = _window(q0, L0, w), _window(v0, L0, w)
     pa = parallel_attn(q_win, kc.unsqueeze(0), vc.unsqueeze(0), k_win, v_win, q_pos0=L0 - w, rope_theta=rope_theta,
                        softmax_scale=softmax_scale, out=b.get("fg"), status=b["status"], workspace=b.get("ws_par"))
     b.update({"fg": pa["out"], "ws_par": pa["workspace"]})
