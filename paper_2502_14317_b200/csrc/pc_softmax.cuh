@@ -5,39 +5,12 @@
 namespace pc {
 
 constexpr float LAZY_RESCALE_LOG2 = 8.0f;      // the reference maximum is raised only when it grows by more than 2^8
-// Every POLY_EVERY-th pair of exponentials is evaluated on the FMA pipe.  A tile needs 128 exponentials a row, 1024
-// cycles of a scheduler's MUFU pipe for its warp; measured on two warps a scheduler (cycles a tile): none 2305, every
-// eighth 2170, fifth 2038, fourth 1972, third 2186 (then the issue slots are what is short).
-constexpr int POLY_EVERY = 4;
+// All exponentials run on the MUFU pipe (ex2), 1024 cycles a tile and warp.  Evaluating every fourth pair as a polynomial on
+// the FMA pipe took a seventh off a tile's cycles and made every workload slower: these kernels run at the board's
+// power cap, and twenty FMA-pipe instructions cost more energy than the two ex2 they replace (128K tokens, 32/8 heads
+// 9244 us with every fourth pair, 8946 with every eighth, 8725 with none; head size 64 at 32K tokens 1018, 977, 953).
 
-__device__ __forceinline__ float fmax_nan(float a, float b) {
-  float d;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
-  return d;
-}
 __device__ __forceinline__ uint64_t dup2(float v) { return pack_f32x2(v, v); }
-
-// 2^x of a pair on the FMA pipe: x = n + f with n the nearest integer (magic-number addition); a polynomial of degree 5
-// in f on [-1/2, 1/2] with p(0) = 1, fitted for the least relative error (1.7e-7 evaluated in fp32, as good as the
-// MUFU's 2^-22); n added to the exponent field.  Arguments below -127 give 0, NaN stays NaN.
-__device__ __forceinline__ void exp2_pair_fma(uint64_t x2, float& p0, float& p1) {
-  float x0, x1;
-  unpack_f32x2(x2, x0, x1);
-  x2 = pack_f32x2(fmax_nan(x0, -127.0f), fmax_nan(x1, -127.0f));          // 2^-127 comes out as exactly 0
-  const uint64_t r2 = add_f32x2(x2, dup2(12582912.0f));
-  const uint64_t n2 = add_f32x2(r2, dup2(-12582912.0f));
-  const uint64_t f2 = fma_f32x2(n2, dup2(-1.0f), x2);
-  uint64_t p = fma_f32x2(f2, dup2(0.001326472731307149f), dup2(0.009671512991189957f));
-  p = fma_f32x2(f2, p, dup2(0.05550733581185341f));
-  p = fma_f32x2(f2, p, dup2(0.24022242426872253f));
-  p = fma_f32x2(f2, p, dup2(0.6931470036506653f));
-  p = fma_f32x2(f2, p, dup2(1.0f));
-  float r0, r1;
-  unpack_f32x2(r2, r0, r1);
-  unpack_f32x2(p, p0, p1);
-  p0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(r0) << 23));
-  p1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(r1) << 23));
-}
 
 // 32 logits -> 16 packed bf16 pairs; partial sums in sum2
 __device__ __forceinline__ void exps32(const uint32_t (&s)[32], uint64_t scale2, uint64_t negm2, uint64_t (&sum2)[2],
@@ -45,15 +18,9 @@ __device__ __forceinline__ void exps32(const uint32_t (&s)[32], uint64_t scale2,
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), scale2, negm2);
-    float p0, p1;
-    if (i % POLY_EVERY == POLY_EVERY - 1) {
-      exp2_pair_fma(x2, p0, p1);
-    } else {
-      float x0, x1;
-      unpack_f32x2(x2, x0, x1);
-      p0 = fast_exp2(x0);
-      p1 = fast_exp2(x1);
-    }
+    float x0, x1;
+    unpack_f32x2(x2, x0, x1);
+    const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
     sum2[i & 1] = add_f32x2(sum2[i & 1], pack_f32x2(p0, p1));
     packed[i] = pack_bf16x2(p0, p1);
   }
