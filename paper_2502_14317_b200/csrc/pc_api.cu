@@ -162,11 +162,10 @@ int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q, const 
       !pc::make_tmap_bf16_4d(&maps[5], krot, kv_dims, kr_str, box_half))
     return PC_ERR_CUDA;
 
-  pc::launch_rope_table(table, table_hi, table_lo, desc->L, d, (double)desc->rope_theta, 0, counter, st);
   // queries and keys are rotated once, ahead of the attention kernel (positions 0 .. L-1 in every chunk)
   const long long os_ll[3] = {os[0], os[1], os[2]};
   const pc::RopeRows rk = {k, {ks[0], ks[1], ks[2]}, krot, desc->Hkv}, rq = {q, {qs[0], qs[1], qs[2]}, qrot, desc->Hq};
-  pc::launch_rope_rows(rk, &rq, table, table_hi, table_lo, desc->C, desc->L, d, st);
+  pc::launch_rope(rk, &rq, {table, table_hi, table_lo}, desc->C, desc->L, d, (double)desc->rope_theta, 0, counter, st);
 
   if (chunk_len != nullptr)   // rows and scores behind the end of a shorter chunk read as zero: the kernels below skip them
     pc::launch_zero_chunk_tails(chunk_len, desc->C, desc->L, desc->w, desc->Hq, desc->Hkv, d, o, os_ll, lse, win_score, st);
@@ -204,9 +203,8 @@ int32_t pc_rope_position_reuse(const void* x, int32_t C, int32_t L, int32_t H, i
   double2* table = reinterpret_cast<double2*>(ws);
   float4* table_hi = reinterpret_cast<float4*>(ws + align_up((size_t)L * (d / 2) * sizeof(double2)));
   float4* table_lo = table_hi + (size_t)L * (d / 4);
-  pc::launch_rope_table(table, table_hi, table_lo, L, d, (double)rope_theta, 0, nullptr, st);
   const pc::RopeRows rows = {x, {(long long)L * H * d, (long long)H * d, d}, y, H};
-  pc::launch_rope_rows(rows, nullptr, table, table_hi, table_lo, C, L, d, st);
+  pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, C, L, d, (double)rope_theta, 0, nullptr, st);
   return cudaGetLastError() == cudaSuccess ? PC_OK : PC_ERR_CUDA;
 }
 
@@ -536,9 +534,8 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   float4* table_hi = reinterpret_cast<float4*>(ws + plan.off_table_hi);
   float4* table_lo = reinterpret_cast<float4*>(ws + plan.off_table_lo);
   void* q_rot = ws + plan.off_qrot;
-  pc::launch_rope_table(table, table_hi, table_lo, w, d, (double)rope_theta, q_pos0, counter, st);
   const pc::RopeRows rows = {q_win, {(long long)w * Hq * d, (long long)Hq * d, (long long)d}, q_rot, Hq};
-  pc::launch_rope_rows(rows, nullptr, table, table_hi, table_lo, B, w, d, st);
+  pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, B, w, d, (double)rope_theta, q_pos0, counter, st);
 
   CUtensorMap maps[5];
   const uint32_t box_kch[4] = {64, plan.pair ? 64u : 128u, 1, 1};

@@ -40,12 +40,10 @@ __device__ __forceinline__ void chain() {
 #endif
 
 // ---- pc_rope.cu
-// cos/sin table: tab[p * (d/2) + t] = (cos, sin)(  (pos0 + p) * theta^(-2t/d) ), fp64; tab_hi, tab_lo (may be null): the
-// same entries split into an fp32 head and an fp32 tail (value = head + tail to 2^-48), one float4 per two pairs:
-// (cos_2i, cos_2i+1, sin_2i, sin_2i+1).
-// counter (may be null) is set to 0.
-void launch_rope_table(double2* tab, float4* tab_hi, float4* tab_lo, int n_pos, int d, double theta, int pos0, int* counter,
-                       cudaStream_t st);
+// Room for the cos/sin table of n_pos positions: exact[p * (d/2) + t] = (cos, sin)(  (pos0 + p) * theta^(-2t/d) ), fp64; hi, lo:
+// the same entries split into an fp32 head and an fp32 tail (value = head + tail to 2^-48), one float4 per two pairs:
+// (cos_2i, cos_2i+1, sin_2i, sin_2i+1).  Small inputs leave it unused.
+struct RopeTable { double2* exact; float4 *hi, *lo; };
 // y[c,p,h,:] = bf16( RoPE(x[c,p,h,:], position p) ), the fp64 rotation rounded once; x addressed by element strides
 // (chunk, token, head), y contiguous [C,L,H,d].
 struct RopeRows {
@@ -54,9 +52,9 @@ struct RopeRows {
   void* y;
   int H;
 };
-// one tensor, or two (b not null) in the same launch
-void launch_rope_rows(const RopeRows& a, const RopeRows* b, const double2* tab, const float4* tab_hi, const float4* tab_lo,
-                      int C, int L, int d, cudaStream_t st);
+// one tensor, or two (b not null) in the same launch; positions pos0 .. pos0 + L - 1; counter (may be null) is set to 0
+void launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int C, int L, int d, double theta, int pos0,
+                 int* counter, cudaStream_t st);
 
 // Per-chunk lengths: zero o[c, p, :, :], lse[c, :, p] and win_score[c, :, p] for p >= clamp(chunk_len[c], w + 1, L).
 void launch_zero_chunk_tails(const int* chunk_len, int C, int L, int w, int Hq, int Hkv, int d, void* o,

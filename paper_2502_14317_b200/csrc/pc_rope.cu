@@ -8,6 +8,11 @@
 
 namespace pc {
 
+__device__ __forceinline__ void rope_angle(double theta, int half, int pos, int t, double& c, double& s) {
+  const double inv_freq = pow(theta, -2.0 * (double)t / (double)(2 * half));
+  sincos((double)pos * inv_freq, &s, &c);
+}
+
 // tab: (cos, sin) per (position, pair), fp64.  tab_hi / tab_lo: fp32 heads / tails of the same values, one float4
 // per two consecutive pairs (cos_2i, cos_2i+1, sin_2i, sin_2i+1); value = head + tail to 2^-48.
 __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict__ tab_hi, float4* __restrict__ tab_lo, int n_pos,
@@ -18,27 +23,15 @@ __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict_
   double c[2], s[2];
   if (mine) {
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const double inv_freq = pow(theta, -2.0 * (double)(t + e) / (double)(2 * half));
-      sincos((double)(pos0 + p) * inv_freq, &s[e], &c[e]);
-    }
+    for (int e = 0; e < 2; ++e) rope_angle(theta, half, pos0 + p, t + e, c[e], s[e]);
   }
   chain();                                                  // the arithmetic needs nothing from before; the tables may still be in use
   if (i == 0 && counter != nullptr) *counter = 0;           // work queue of the attention kernel that follows
   if (!mine) return;
   for (int e = 0; e < 2; ++e) tab[(size_t)p * half + t + e] = make_double2(c[e], s[e]);
-  if (tab_hi != nullptr) {
-    const float c0 = (float)c[0], c1 = (float)c[1], s0 = (float)s[0], s1 = (float)s[1];
-    tab_hi[i] = make_float4(c0, c1, s0, s1);
-    tab_lo[i] = make_float4((float)(c[0] - (double)c0), (float)(c[1] - (double)c1), (float)(s[0] - (double)s0),
-                            (float)(s[1] - (double)s1));
-  }
-}
-
-void launch_rope_table(double2* tab, float4* tab_hi, float4* tab_lo, int n_pos, int d, double theta, int pos0, int* counter,
-                       cudaStream_t st) {
-  const int n = n_pos * (d / 4);
-  launch_chained(rope_table_kernel, dim3((n + 255) / 256), dim3(256), 0, st, 1, tab, tab_hi, tab_lo, n_pos, d / 2, theta, pos0, counter);
+  const float c0 = (float)c[0], c1 = (float)c[1], s0 = (float)s[0], s1 = (float)s[1];
+  tab_hi[i] = make_float4(c0, c1, s0, s1);
+  tab_lo[i] = make_float4((float)(c[0] - (double)c0), (float)(c[1] - (double)c1), (float)(s[0] - (double)s0), (float)(s[1] - (double)s1));
 }
 
 // y[c,p,h,:] = bf16( RoPE(x[c,p,h,:], position p) ).  One warp owns one position: a lane holds 8 consecutive
@@ -53,16 +46,40 @@ void launch_rope_table(double2* tab, float4* tab_hi, float4* tab_lo, int n_pos, 
 //
 // One launch takes one or two tensors of the same chunks and positions (keys and queries): grid.y first deals out the slices of
 // the chunks of the first tensor, then those of the second.
+//
+// OWN_TABLE: a warp computes the table row of its position itself, in shared memory, before it waits for the kernel ahead
+// (see launch_rope).
+struct RopeAngles { double theta; int pos0; int* counter; };   // for OWN_TABLE; counter (may be null) is set to 0
+struct RopeRow { float4 hi[32], lo[32]; double2 exact[64]; };
 struct RopeTensor {
   const uint16_t* x;
   uint16_t* y;
   long long s_chunk, s_tok, s_head;                         // element strides of x; y is contiguous
   int H, ny, nz;                                            // heads; slices of the chunks; parts of the head passes
 };
+template <bool OWN_TABLE>
 __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant__ RopeTensor ta, const __grid_constant__ RopeTensor tb,
                                                            const float4* __restrict__ tab_hi, const float4* __restrict__ tab_lo,
-                                                           const double2* __restrict__ tab, int C, int L, int d) {
+                                                           const double2* __restrict__ tab, int C, int L, int d, RopeAngles ang) {
+  __shared__ RopeRow own[OWN_TABLE ? 8 : 1];
+  const int half = d / 2, lane = threadIdx.x & 31;
+  const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  RopeRow& row = own[OWN_TABLE ? threadIdx.x >> 5 : 0];
+  if (OWN_TABLE && p < L) {
+    for (int t = lane; t < half; t += 32) {
+      double2 e;
+      rope_angle(ang.theta, half, ang.pos0 + p, t, e.x, e.y);
+      const float c0 = (float)e.x, s0 = (float)e.y;
+      float* const hi = reinterpret_cast<float*>(&row.hi[t >> 1]) + (t & 1);
+      float* const lo = reinterpret_cast<float*>(&row.lo[t >> 1]) + (t & 1);
+      hi[0] = c0; hi[2] = s0;
+      lo[0] = (float)(e.x - (double)c0); lo[2] = (float)(e.y - (double)s0);
+      row.exact[t] = e;
+    }
+    __syncwarp();
+  }
   chain();
+  if (OWN_TABLE && ang.counter != nullptr && (blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *ang.counter = 0;
   const bool second_tensor = (int)blockIdx.y >= ta.ny;      // the same for the whole block
   const uint16_t* __restrict__ const x = second_tensor ? tb.x : ta.x;
   uint16_t* __restrict__ const y = second_tensor ? tb.y : ta.y;
@@ -71,19 +88,16 @@ __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant
   const int H = second_tensor ? tb.H : ta.H, ny = second_tensor ? tb.ny : ta.ny, zs = second_tensor ? tb.nz : ta.nz;
   const int slice = second_tensor ? (int)blockIdx.y - ta.ny : (int)blockIdx.y;
   if ((int)blockIdx.z >= zs) return;
-  const int half = d / 2;
   const int groups = half / 8;                              // 16-byte groups per half row (4 or 8)
-  const int lane = threadIdx.x & 31;
-  const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (p >= L) return;                                       // whole warps leave together
   const int g = lane % groups, h_first = lane / groups, h_step = 32 / groups;
   const size_t row0 = (size_t)p * half;                     // first pair of this position in the tables
-  const float4* hi_row = tab_hi + row0 / 2;
-  const float4* lo_row = tab_lo + row0 / 2;
-  const double2* d_row = tab + row0;
+  const float4* hi_row = OWN_TABLE ? row.hi : tab_hi + row0 / 2;
+  const float4* lo_row = OWN_TABLE ? row.lo : tab_lo + row0 / 2;
+  const double2* d_row = OWN_TABLE ? row.exact : tab + row0;
   float4 hi[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) hi[i] = __ldg(hi_row + g * 4 + i);
+  for (int i = 0; i < 4; ++i) hi[i] = table_entry<OWN_TABLE>(hi_row + g * 4 + i);
   // small inputs: the head passes are dealt out over grid.z (zs parts)
   const long long step_src = (long long)h_step * zs * s_head;
   const size_t step_dst = (size_t)h_step * zs * d;
@@ -136,8 +150,8 @@ __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant
             const float b = __uint_as_float((t & 1) ? (u2 & 0xFFFF0000u) : (u2 << 16));
             const int sg = srcl % groups, sh = srcl / groups + ps * h_step;      // pair group and head of that lane
             const int pair = sg * 8 + t;
-            const uint32_t r = second ? rope_one_exact(b, -a, pair, hi_row, lo_row, d_row)
-                                      : rope_one_exact(a, b, pair, hi_row, lo_row, d_row);
+            const uint32_t r = second ? rope_one_exact<OWN_TABLE>(b, -a, pair, hi_row, lo_row, d_row)
+                                      : rope_one_exact<OWN_TABLE>(a, b, pair, hi_row, lo_row, d_row);
             dst_tok[(size_t)sh * d + (second ? half : 0) + pair] = (uint16_t)r;
           }
         } while (todo != 0u);
@@ -164,13 +178,25 @@ static RopeTensor rope_tensor(const RopeRows& r, int C, int L, int d) {
   return t;
 }
 
-void launch_rope_rows(const RopeRows& a, const RopeRows* b, const double2* tab, const float4* tab_hi, const float4* tab_lo,
-                      int C, int L, int d, cudaStream_t st) {
+void launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int C, int L, int d, double theta, int pos0,
+                 int* counter, cudaStream_t st) {
   const RopeTensor ta = rope_tensor(a, C, L, d);
   RopeTensor tb = {};
   if (b != nullptr) tb = rope_tensor(*b, C, L, d);
-  launch_chained(rope_rows_kernel, dim3((unsigned)((L + 7) / 8), (unsigned)(ta.ny + tb.ny), (unsigned)(ta.nz > tb.nz ? ta.nz : tb.nz)), dim3(256), 0, st, 1, 
-      ta, tb, tab_hi, tab_lo, tab, C, L, d);
+  const dim3 grid((unsigned)((L + 7) / 8), (unsigned)(ta.ny + tb.ny), (unsigned)(ta.nz > tb.nz ? ta.nz : tb.nz));
+  const RopeAngles ang = {theta, pos0, counter};
+  // Up to 2 M values the warps compute their own table rows: one launch less, and the angles are found while the kernel ahead
+  // still runs (us, table kernel / own rows; B x L x H x d: 1x64x32x128 5.2 / 3.8, 4x256x8x64 5.3 / 4.2, 1x1024x8x128
+  // 7.3 / 5.5, 4x1024x8x64 8.1 / 7.7).  Above it, repeating the fp64 angles in every slice of the chunks and fewer free
+  // registers cost more than the launch (16x64x32x128 9.9 / 10.4, 64x64x32x128 18.7 / 23.3, 4x8192x32x128 118 / 152).
+  const long long values = (long long)C * L * d * (a.H + (b != nullptr ? b->H : 0));
+  if (values <= (1 << 21)) {
+    launch_chained(rope_rows_kernel<true>, grid, dim3(256), 0, st, 1, ta, tb, tab.hi, tab.lo, tab.exact, C, L, d, ang);
+    return;
+  }
+  launch_chained(rope_table_kernel, dim3((unsigned)((L * (d / 4) + 255) / 256)), dim3(256), 0, st, 1, tab.exact, tab.hi, tab.lo, L, d / 2,
+                 theta, pos0, counter);
+  launch_chained(rope_rows_kernel<false>, grid, dim3(256), 0, st, 1, ta, tb, tab.hi, tab.lo, tab.exact, C, L, d, ang);
 }
 
 // Rows behind the end of a chunk that is shorter than L (per-chunk lengths): outputs read as zero there.

@@ -49,15 +49,20 @@ __device__ __forceinline__ uint32_t rope_out_dd(float a, float b, float ch, floa
 //
 // Levels 2 and 3 for ONE output y = a * c - b * s (pass (b, -a) for the second output of a pair, b c + a s) at
 // table entry `pair` of a position's row: heads in hi_row, tails in lo_row (float4 per two pairs), fp64 (cos, sin)
-// in d_row.  Returns the bf16 bits.
-__device__ __forceinline__ uint32_t rope_one_exact(float a, float b, int pair, const float4* __restrict__ hi_row,
-                                                   const float4* __restrict__ lo_row, const double2* __restrict__ d_row) {
+// in d_row (SHARED: the rows are in shared memory).  Returns the bf16 bits.
+template <bool SHARED, class T>
+__device__ __forceinline__ T table_entry(const T* p) { return SHARED ? *p : __ldg(p); }
+
+template <bool SHARED>
+__device__ __forceinline__ uint32_t rope_one_exact(float a, float b, int pair, const float4* hi_row, const float4* lo_row,
+                                                   const double2* d_row) {
   const float* h = reinterpret_cast<const float*>(hi_row + (pair >> 1));
   const float* l = reinterpret_cast<const float*>(lo_row + (pair >> 1));
   const int e = pair & 1;
-  uint32_t r = rope_out_dd(a, b, __ldg(h + e), __ldg(h + 2 + e), __ldg(l + e), __ldg(l + 2 + e));
+  uint32_t r = rope_out_dd(a, b, table_entry<SHARED>(h + e), table_entry<SHARED>(h + 2 + e), table_entry<SHARED>(l + e),
+                           table_entry<SHARED>(l + 2 + e));
   if (r == 0xFFFFFFFFu) {
-    const double2 t = __ldg(d_row + pair);
+    const double2 t = table_entry<SHARED>(d_row + pair);
     r = f64_to_bf16_rne((double)a * t.x - (double)b * t.y);
   }
   return r;

@@ -216,6 +216,18 @@ def test_rope_position_reuse_equals_fp64_rotation_rounded_once(C, L, H, d, theta
     assert bad.shape[0] == 0, f"{bad.shape[0]} of {ref.size} rotated values differ from the fp64 rotation, first at {bad[0]}"
 
 
+@pytest.mark.parametrize("C,L,H,d", [(1, 1, 1, 64), (1, 1, 1, 128), (5, 9, 3, 64), (2, 1024, 8, 128), (1, 2049, 8, 128), (1, 4097, 8, 64)])
+def test_rope_with_and_without_a_table_kernel(C, L, H, d):
+    """Up to 2^21 values the warps of the rotation pass compute their own table rows, above that a kernel of its own does: the
+    smallest inputs, the last size of the first kind and the first two above it give the oracle's bits."""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(L + d)
+    bits = pc_inputs.f32_to_bf16_bits(rng.standard_normal((C, L, H, d)).astype(np.float32))
+    got = to_bits(pc.rope_position_reuse(to_dev(bits), rope_theta=10000.0))
+    torch.cuda.synchronize()
+    assert np.array_equal(got, orc.rope_bf16(bits, 10000.0))
+
+
 @pytest.mark.parametrize("L,w,Hq,Hkv,d,lens", [
     (640, 64, 4, 2, 128, [640, 500, 129, 65, 384]),      # CTA pairs: full, ragged, two tiles, one tile, tile-aligned
     (520, 24, 4, 1, 128, [300, 520, 25, 256]),           # w = 24, the shortest chunk has a single context token
