@@ -315,6 +315,46 @@ PC_API int32_t pc_parallel_attn_append(int32_t B, int32_t w, int32_t Hq, int32_t
                                 void* workspace, size_t workspace_bytes, void* stream);
 
 /* ------------------------------------------------------------------------------------
+ * The whole path for chunks on the device, as one call: pc_chunk_prefill_attn,
+ * pc_score_select_chunks (pc_select_chunks on given_score if that is not NULL; lower is
+ * better), pc_select_tokens on the L - w context tokens, pc_gather_kv and pc_parallel_attn
+ * (B = 1, q_pos0 = L - w) of chunk 0's window over the m * k_keep kept entries.  Same kernels,
+ * same results; what it saves is the host time between them, which bounds a short prompt.
+ * Shapes as in those calls; v and k_rot contiguous, q_win [w,Hq,d] contiguous (the window rows
+ * of chunk 0: for a contiguous q, q + (L-w)*Hq*d).  With clear_status the status word, which
+ * both attention calls share, is set to 0 first.  Returns the first failing call's code and
+ * names that call in *failed (may be NULL; 0: none).
+ * pc_hot_path_workspace_bytes gives the size of ws_prefill and, in *parallel_bytes, that of
+ * ws_parallel.
+ */
+typedef struct {
+  const void *q, *k, *v, *q_win;
+  void *o, *k_rot;
+  float *win_score, *win_lse;
+  const float* given_score;            /* [n_score] or NULL */
+  float* chunk_score;                  /* [C], unused with given_score */
+  int32_t *kept, *idx;
+  void *kc, *vc;
+  int32_t* pos;                        /* or NULL */
+  void* fg;
+  int32_t* status_word;                /* or NULL */
+  void* ws_prefill;
+  size_t ws_prefill_bytes;
+  void* ws_parallel;
+  size_t ws_parallel_bytes;
+  int32_t m, k_keep, n_score, clear_status;
+} pc_hot_path_args;
+
+enum {
+  PC_STAGE_PREFILL = 1, PC_STAGE_SELECT_CHUNKS, PC_STAGE_SCORE_SELECT_CHUNKS, PC_STAGE_SELECT_TOKENS, PC_STAGE_GATHER,
+  PC_STAGE_PARALLEL
+};
+
+PC_API size_t pc_hot_path_workspace_bytes(const pc_prefill_desc* desc, int32_t m, int32_t k_keep, size_t* parallel_bytes);
+
+PC_API int32_t pc_hot_path(const pc_prefill_desc* desc, const pc_hot_path_args* args, int32_t* failed, void* stream);
+
+/* ------------------------------------------------------------------------------------
  * pc_parallel_attn without a workspace argument, for callers that must not allocate.
  * The paper has no counterpart of this call: it computes exactly what pc_parallel_attn
  * computes (same kernels, same split plan, same results) and exists for the callers

@@ -27,6 +27,17 @@ class _PrefillDesc(Structure):
                 ("o_stride", c_int64 * 3)]
 
 
+class _HotPathArgs(Structure):
+    _fields_ = [(n, c_void_p) for n in ("q", "k", "v", "q_win", "o", "k_rot", "win_score", "win_lse", "given_score", "chunk_score",
+                                        "kept", "idx", "kc", "vc", "pos", "fg", "status_word", "ws_prefill")] + \
+               [("ws_prefill_bytes", c_size_t), ("ws_parallel", c_void_p), ("ws_parallel_bytes", c_size_t),
+                ("m", c_int32), ("k_keep", c_int32), ("n_score", c_int32), ("clear_status", c_int32)]
+
+
+_STAGES = (None, "pc_chunk_prefill_attn", "pc_select_chunks", "pc_score_select_chunks", "pc_select_tokens", "pc_gather_kv",
+           "pc_parallel_attn")
+
+
 def lib_path() -> str:
     return os.path.join(_HERE, "libpc.so")
 
@@ -88,6 +99,10 @@ def load_library():
     lib.pc_parallel_attn_append.restype = c_int32
     lib.pc_parallel_attn_append.argtypes = [c_int32] * 7 + [c_void_p, c_int32, c_float, c_float] + [c_void_p] * 8 + \
                                            [c_size_t, c_void_p]
+    lib.pc_hot_path_workspace_bytes.restype = c_size_t
+    lib.pc_hot_path_workspace_bytes.argtypes = [POINTER(_PrefillDesc), c_int32, c_int32, POINTER(c_size_t)]
+    lib.pc_hot_path.restype = c_int32
+    lib.pc_hot_path.argtypes = [POINTER(_PrefillDesc), POINTER(_HotPathArgs), POINTER(c_int32), c_void_p]
     lib.pc_parallel_attn_static_scratch_bytes.restype = c_size_t
     lib.pc_parallel_attn_static_scratch_bytes.argtypes = []
     lib.pc_parallel_attn_static.restype = c_int32
@@ -129,6 +144,16 @@ def _like(t, shape):
     if t.dtype is torch.bfloat16 and t.shape == shape and t.is_contiguous():
         return torch.empty_like(t)
     return t.new_empty(shape, dtype=torch.bfloat16)
+
+
+def _new(t, dtype, *shape):
+    """New contiguous tensor on t's device (torch.empty takes 2.4 us for a shape of several dimensions, this 1.5)."""
+    strides, n = [], 1
+    for s in reversed(shape):
+        strides.append(n)
+        n *= s if s > 1 else 1
+    strides.reverse()
+    return torch.empty_strided(shape, strides, dtype=dtype, device=t.device)
 
 
 def _window(t, L, w):
@@ -459,35 +484,77 @@ def parallel_attn_static(q_win, k_cache, v_cache, k_win, v_win, out, *, q_pos0, 
 
 
 def hot_path(q, k, v, *, w, rope_theta, m, k_keep, softmax_scale=0.0, chunk_score=None, buffers=None):
-    """One pass of the whole path on the current stream: the five C-ABI calls chained, no host sync.
+    """pc_hot_path: one pass of the whole path on the current stream, no host sync.
 
     ``chunk_score`` (device fp32 [C]) stands for the self-information of Eq. 3; if None the
     single-layer stand-in computed from the window log-sum-exp is used.
     ``buffers`` (dict) lets repeated calls reuse outputs and workspaces.
     """
     b = {} if buffers is None else buffers
+    lib = load_library()
+    _need_cuda(q, k, v, chunk_score)
     C, L, Hq, d = q.shape
-    pre = chunk_prefill_attn(q, k, v, w=w, rope_theta=rope_theta, softmax_scale=softmax_scale, out=b.get("o"),
-                             k_rot=b.get("k_rot"), win_score=b.get("win_score"), win_lse=b.get("win_lse"),
-                             status=b.get("status"), workspace=b.get("ws_prefill"))
+    Hkv = k.shape[2]
+    m, k_keep = int(m), int(k_keep)
+    get = b.get
+    o, k_rot, win_score, win_lse = get("o"), get("k_rot"), get("win_score"), get("win_lse")
+    kept, idx, kc, vc, pos, fg = get("kept"), get("idx"), get("kc"), get("vc"), get("pos"), get("fg")
+    score, status, ws_prefill, ws_par = get("chunk_score"), get("status"), get("ws_prefill"), get("ws_par")
+    clear = status is None
+    if o is None:
+        o = _like(q, q.shape)
+    if k_rot is None:
+        k_rot = _like(k, k.shape)
+    if win_score is None:
+        win_score = _new(q, torch.float32, C, Hkv, L)
+    if win_lse is None:
+        win_lse = _new(q, torch.float32, C, Hq, w)
     if chunk_score is not None:
-        score, kept = chunk_score, select_chunks(chunk_score, m, True, out=b.get("kept"))
-    else:
-        score, kept = score_select_chunks(pre["win_lse"], m, True, score_out=b.get("chunk_score"), kept_out=b.get("kept"))
-    idx = select_tokens(pre["win_score"], kept, L - w, k_keep, out=b.get("idx"))
-    kc, vc, pos = gather_kv(pre["k_rot"], v, kept, idx, k_out=b.get("kc"), v_out=b.get("vc"), pos_out=b.get("pos"))
+        score = chunk_score
+    elif score is None:
+        score = _new(q, torch.float32, C)
+    if kept is None:
+        kept = _new(q, torch.int32, m)
+    if idx is None:
+        idx = _new(q, torch.int32, m, Hkv, k_keep)
+    if kc is None:
+        kc = _new(q, torch.bfloat16, Hkv, m * k_keep, d)
+    if vc is None:
+        vc = _new(q, torch.bfloat16, Hkv, m * k_keep, d)
+    if pos is None:
+        pos = _new(q, torch.int32, Hkv, m * k_keep)
+    if fg is None:
+        fg = _new(q, torch.bfloat16, 1, w, Hq, d)
+    if status is None:
+        status = _new(q, torch.int32, 1)
+    desc = _make_desc(q, k, v, o, w, rope_theta, softmax_scale)
+    ref = ctypes.byref(desc)
+    need_par = c_size_t()
+    need = lib.pc_hot_path_workspace_bytes(ref, m, k_keep, ctypes.byref(need_par))
+    need_par = need_par.value
+    if ws_prefill is None or ws_prefill.numel() < need:        # 0: a bad argument, which the call below names
+        ws_prefill = _new(q, torch.uint8, max(need, 16))
+    if ws_par is None or ws_par.numel() < need_par:
+        ws_par = _new(q, torch.uint8, max(need_par, 16))
+    if k_rot.stride() != v.stride():
+        raise PcError("k_src and v_src must share strides with a contiguous head dimension")
     # the window is the same in every chunk: take it from chunk 0
-    q_win, k_win, v_win = (_window(t, L, w) for t in (q, pre["k_rot"], v))
-    pa = parallel_attn(q_win, kc.unsqueeze(0), vc.unsqueeze(0), k_win, v_win, q_pos0=L - w, rope_theta=rope_theta,
-                       softmax_scale=softmax_scale, out=b.get("fg"), status=pre["status"], workspace=b.get("ws_par"))
-    res = {"o": pre["o"], "k_rot": pre["k_rot"], "win_score": pre["win_score"], "win_lse": pre["win_lse"],
-           "chunk_score": score, "kept": kept, "idx": idx, "kc": kc, "vc": vc, "pos": pos, "fg": pa["out"],
-           "status": pre["status"], "ws_prefill": pre["workspace"], "ws_par": pa["workspace"]}
+    q_win = None if q.is_contiguous() else _window(q, L, w)
+    args = _HotPathArgs(q.data_ptr(), k.data_ptr(), v.data_ptr(),
+                        q.data_ptr() + (L - w) * Hq * d * 2 if q_win is None else q_win.data_ptr(), o.data_ptr(), k_rot.data_ptr(),
+                        win_score.data_ptr(), win_lse.data_ptr(), _ptr(chunk_score), score.data_ptr(), kept.data_ptr(),
+                        idx.data_ptr(), kc.data_ptr(), vc.data_ptr(), pos.data_ptr(), fg.data_ptr(), status.data_ptr(),
+                        ws_prefill.data_ptr(), ws_prefill.numel(), ws_par.data_ptr(), ws_par.numel(), m, k_keep, score.numel(), clear)
+    failed = c_int32()
+    rc = lib.pc_hot_path(ref, ctypes.byref(args), ctypes.byref(failed), _stream())
+    if rc != 0:
+        _check(rc, _STAGES[failed.value])
+    res = {"o": o, "k_rot": k_rot, "win_score": win_score, "win_lse": win_lse, "chunk_score": score, "kept": kept, "idx": idx,
+           "kc": kc, "vc": vc, "pos": pos, "fg": fg, "status": status, "ws_prefill": ws_prefill, "ws_par": ws_par}
     if buffers is not None:
-        buffers.update({"o": res["o"], "k_rot": res["k_rot"], "win_score": res["win_score"], "win_lse": res["win_lse"],
-                        "chunk_score": score if chunk_score is None else b.get("chunk_score"), "kept": kept, "idx": idx,
-                        "kc": kc, "vc": vc, "pos": pos, "fg": res["fg"], "status": res["status"],
-                        "ws_prefill": res["ws_prefill"], "ws_par": res["ws_par"]})
+        given = get("chunk_score") if chunk_score is not None else score
+        buffers.update(res)
+        buffers["chunk_score"] = given                         # a caller's scores are not a buffer
     return res
 
 

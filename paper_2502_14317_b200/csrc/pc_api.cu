@@ -112,10 +112,15 @@ size_t pc_chunk_prefill_attn_workspace_bytes(const pc_prefill_desc* desc) {
   return prefill_layout(desc, false).total;
 }
 
-int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q, const void* k, const void* v,
-                              const int32_t* chunk_len, void* o, void* k_rot, float* lse, float* win_score,
-                              float* win_lse, int32_t* status_word, void* workspace, size_t workspace_bytes,
-                              void* stream) {
+}  // extern "C"
+
+namespace {
+
+// clear_status: the status word is set to 0 first (by a kernel that runs anyway)
+int32_t prefill_attn_impl(const pc_prefill_desc* desc, const void* q, const void* k, const void* v,
+                          const int32_t* chunk_len, void* o, void* k_rot, float* lse, float* win_score,
+                          float* win_lse, int32_t* status_word, void* workspace, size_t workspace_bytes,
+                          void* stream, bool clear_status) {
   int32_t rc = check_prefill_desc(desc);
   if (rc != PC_OK) return rc;
   if (!q || !k || !v || !o || !win_score || !win_lse) return PC_ERR_INVALID_ARG;
@@ -165,7 +170,8 @@ int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q, const 
   // queries and keys are rotated once, ahead of the attention kernel (positions 0 .. L-1 in every chunk)
   const long long os_ll[3] = {os[0], os[1], os[2]};
   const pc::RopeRows rk = {k, {ks[0], ks[1], ks[2]}, krot, desc->Hkv}, rq = {q, {qs[0], qs[1], qs[2]}, qrot, desc->Hq};
-  pc::launch_rope(rk, &rq, {table, table_hi, table_lo}, desc->C, desc->L, d, (double)desc->rope_theta, 0, counter, st);
+  pc::launch_rope(rk, &rq, {table, table_hi, table_lo}, desc->C, desc->L, d, (double)desc->rope_theta, 0, counter,
+                  clear_status ? status_word : nullptr, st);
 
   if (chunk_len != nullptr)   // rows and scores behind the end of a shorter chunk read as zero: the kernels below skip them
     pc::launch_zero_chunk_tails(chunk_len, desc->C, desc->L, desc->w, desc->Hq, desc->Hkv, d, o, os_ll, lse, win_score, st);
@@ -182,6 +188,18 @@ int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q, const 
   const cudaError_t le = pc::launch_prefill_attn(maps, prm, d, dev.sm_count, st);
   if (le != cudaSuccess) return PC_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? PC_OK : PC_ERR_CUDA;
+}
+
+}  // namespace
+
+extern "C" {
+
+int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q, const void* k, const void* v,
+                              const int32_t* chunk_len, void* o, void* k_rot, float* lse, float* win_score,
+                              float* win_lse, int32_t* status_word, void* workspace, size_t workspace_bytes,
+                              void* stream) {
+  return prefill_attn_impl(desc, q, k, v, chunk_len, o, k_rot, lse, win_score, win_lse, status_word, workspace, workspace_bytes,
+                           stream, false);
 }
 
 // ------------------------------------------------------------------------------------ RoPE with position reuse
@@ -204,7 +222,7 @@ int32_t pc_rope_position_reuse(const void* x, int32_t C, int32_t L, int32_t H, i
   float4* table_hi = reinterpret_cast<float4*>(ws + align_up((size_t)L * (d / 2) * sizeof(double2)));
   float4* table_lo = table_hi + (size_t)L * (d / 4);
   const pc::RopeRows rows = {x, {(long long)L * H * d, (long long)H * d, d}, y, H};
-  pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, C, L, d, (double)rope_theta, 0, nullptr, st);
+  pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, C, L, d, (double)rope_theta, 0, nullptr, nullptr, st);
   return cudaGetLastError() == cudaSuccess ? PC_OK : PC_ERR_CUDA;
 }
 
@@ -535,7 +553,7 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   float4* table_lo = reinterpret_cast<float4*>(ws + plan.off_table_lo);
   void* q_rot = ws + plan.off_qrot;
   const pc::RopeRows rows = {q_win, {(long long)w * Hq * d, (long long)Hq * d, (long long)d}, q_rot, Hq};
-  pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, B, w, d, (double)rope_theta, q_pos0, counter, st);
+  pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, B, w, d, (double)rope_theta, q_pos0, counter, nullptr, st);
 
   CUtensorMap maps[5];
   const uint32_t box_kch[4] = {64, plan.pair ? 64u : 128u, 1, 1};
@@ -587,6 +605,44 @@ int32_t pc_parallel_attn_append(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, i
   if (Nk_cap < 1 || (int64_t)Nk + w > (int64_t)Nk_cap) return PC_ERR_INVALID_ARG;
   return parallel_attn_impl(B, w, Hq, Hkv, d, Nk, Nk_cap, q_win, q_pos0, rope_theta, softmax_scale, k_cache, v_cache, k_win,
                             v_win, out, lse_out, status_word, workspace, workspace_bytes, stream, true);
+}
+
+// ------------------------------------------------------------------------------------ the whole path
+size_t pc_hot_path_workspace_bytes(const pc_prefill_desc* desc, int32_t m, int32_t k, size_t* parallel_bytes) {
+  if (parallel_bytes != nullptr)
+    *parallel_bytes = desc != nullptr && m >= 1 && k >= 1 && (int64_t)m * k < (1ll << 31)
+                          ? pc_parallel_attn_workspace_bytes(1, desc->w, desc->Hq, desc->Hkv, desc->d, m * k) : 0;
+  return pc_chunk_prefill_attn_workspace_bytes(desc);
+}
+
+int32_t pc_hot_path(const pc_prefill_desc* desc, const pc_hot_path_args* a, int32_t* failed, void* stream) {
+  int32_t stage = PC_STAGE_PREFILL, rc = PC_ERR_INVALID_ARG;
+  if (desc != nullptr && a != nullptr) do {
+    rc = prefill_attn_impl(desc, a->q, a->k, a->v, nullptr, a->o, a->k_rot, nullptr, a->win_score, a->win_lse, a->status_word,
+                           a->ws_prefill, a->ws_prefill_bytes, stream, a->clear_status != 0);
+    if (rc != PC_OK) break;
+    const int32_t C = desc->C, L = desc->L, w = desc->w, Hq = desc->Hq, Hkv = desc->Hkv, d = desc->d;
+    if (a->given_score != nullptr) {
+      stage = PC_STAGE_SELECT_CHUNKS;
+      rc = pc_select_chunks(a->given_score, a->n_score, a->m, 1, a->kept, stream);
+    } else {
+      stage = PC_STAGE_SCORE_SELECT_CHUNKS;
+      rc = pc_score_select_chunks(a->win_lse, C, Hq, w, a->m, 1, a->chunk_score, a->kept, stream);
+    }
+    if (rc != PC_OK) break;
+    stage = PC_STAGE_SELECT_TOKENS;
+    if ((rc = pc_select_tokens(a->win_score, a->kept, C, a->m, Hkv, L, L - w, a->k_keep, a->idx, stream)) != PC_OK) break;
+    stage = PC_STAGE_GATHER;
+    const int64_t row = (int64_t)Hkv * d, kv_stride[3] = {L * row, row, d};
+    if ((rc = pc_gather_kv(a->k_rot, a->v, kv_stride, a->kept, a->idx, a->m, Hkv, a->k_keep, d, a->kc, a->vc, a->pos, stream)) != PC_OK) break;
+    stage = PC_STAGE_PARALLEL;
+    // the window is the same in every chunk: the keys and values of chunk 0's
+    rc = pc_parallel_attn(1, w, Hq, Hkv, d, a->m * a->k_keep, a->q_win, L - w, desc->rope_theta, desc->softmax_scale, a->kc, a->vc,
+                          static_cast<const uint16_t*>(a->k_rot) + (L - w) * row, static_cast<const uint16_t*>(a->v) + (L - w) * row,
+                          a->fg, nullptr, a->status_word, a->ws_parallel, a->ws_parallel_bytes, stream);
+  } while (false);
+  if (failed != nullptr) *failed = rc == PC_OK ? 0 : stage;
+  return rc;
 }
 
 }  // extern "C"

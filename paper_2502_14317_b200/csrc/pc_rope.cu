@@ -16,7 +16,7 @@ __device__ __forceinline__ void rope_angle(double theta, int half, int pos, int 
 // tab: (cos, sin) per (position, pair), fp64.  tab_hi / tab_lo: fp32 heads / tails of the same values, one float4
 // per two consecutive pairs (cos_2i, cos_2i+1, sin_2i, sin_2i+1); value = head + tail to 2^-48.
 __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict__ tab_hi, float4* __restrict__ tab_lo, int n_pos,
-                                  int half, double theta, int pos0, int* __restrict__ counter) {
+                                  int half, double theta, int pos0, int* __restrict__ counter, int* __restrict__ clear) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;      // one thread per two pairs
   const int p = i / (half / 2), t = 2 * (i % (half / 2));
   const bool mine = i < n_pos * (half / 2);
@@ -27,6 +27,7 @@ __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict_
   }
   chain();                                                  // the arithmetic needs nothing from before; the tables may still be in use
   if (i == 0 && counter != nullptr) *counter = 0;           // work queue of the attention kernel that follows
+  if (i == 0 && clear != nullptr) *clear = 0;
   if (!mine) return;
   for (int e = 0; e < 2; ++e) tab[(size_t)p * half + t + e] = make_double2(c[e], s[e]);
   const float c0 = (float)c[0], c1 = (float)c[1], s0 = (float)s[0], s1 = (float)s[1];
@@ -49,7 +50,7 @@ __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict_
 //
 // OWN_TABLE: a warp computes the table row of its position itself, in shared memory, before it waits for the kernel ahead
 // (see launch_rope).
-struct RopeAngles { double theta; int pos0; int* counter; };   // for OWN_TABLE; counter (may be null) is set to 0
+struct RopeAngles { double theta; int pos0; int *counter, *clear; };   // for OWN_TABLE; counter and clear (may be null) are set to 0
 struct RopeRow { float4 hi[32], lo[32]; double2 exact[64]; };
 struct RopeTensor {
   const uint16_t* x;
@@ -79,7 +80,10 @@ __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant
     __syncwarp();
   }
   chain();
-  if (OWN_TABLE && ang.counter != nullptr && (blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *ang.counter = 0;
+  if (OWN_TABLE && (blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) {
+    if (ang.counter != nullptr) *ang.counter = 0;
+    if (ang.clear != nullptr) *ang.clear = 0;
+  }
   const bool second_tensor = (int)blockIdx.y >= ta.ny;      // the same for the whole block
   const uint16_t* __restrict__ const x = second_tensor ? tb.x : ta.x;
   uint16_t* __restrict__ const y = second_tensor ? tb.y : ta.y;
@@ -179,12 +183,12 @@ static RopeTensor rope_tensor(const RopeRows& r, int C, int L, int d) {
 }
 
 void launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int C, int L, int d, double theta, int pos0,
-                 int* counter, cudaStream_t st) {
+                 int* counter, int* clear, cudaStream_t st) {
   const RopeTensor ta = rope_tensor(a, C, L, d);
   RopeTensor tb = {};
   if (b != nullptr) tb = rope_tensor(*b, C, L, d);
   const dim3 grid((unsigned)((L + 7) / 8), (unsigned)(ta.ny + tb.ny), (unsigned)(ta.nz > tb.nz ? ta.nz : tb.nz));
-  const RopeAngles ang = {theta, pos0, counter};
+  const RopeAngles ang = {theta, pos0, counter, clear};
   // Up to 2 M values the warps compute their own table rows: one launch less, and the angles are found while the kernel ahead
   // still runs (us, table kernel / own rows; B x L x H x d: 1x64x32x128 5.2 / 3.8, 4x256x8x64 5.3 / 4.2, 1x1024x8x128
   // 7.3 / 5.5, 4x1024x8x64 8.1 / 7.7).  Above it, repeating the fp64 angles in every slice of the chunks and fewer free
@@ -195,7 +199,7 @@ void launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int
     return;
   }
   launch_chained(rope_table_kernel, dim3((unsigned)((L * (d / 4) + 255) / 256)), dim3(256), 0, st, 1, tab.exact, tab.hi, tab.lo, L, d / 2,
-                 theta, pos0, counter);
+                 theta, pos0, counter, clear);
   launch_chained(rope_rows_kernel<false>, grid, dim3(256), 0, st, 1, ta, tb, tab.hi, tab.lo, tab.exact, C, L, d, ang);
 }
 

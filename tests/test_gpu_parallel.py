@@ -180,6 +180,45 @@ def test_single_chunk_keep_all_equals_local_attention():
     check_attention_output(fg, O[0, L - w:], "Fg vs full causal attention")
 
 
+@pytest.mark.parametrize("C,L,w,Hq,Hkv,d,m,k,given,strided", [
+    (4, 256, 16, 4, 2, 64, 2, 64, False, False), (3, 200, 32, 6, 3, 128, 2, 100, True, False),
+    (1, 129, 8, 2, 1, 128, 1, 121, False, True), (5, 300, 64, 4, 4, 64, 3, 77, True, True),
+])
+def test_hot_path_equals_its_stages(C, L, w, Hq, Hkv, d, m, k, given, strided):
+    """The whole path as one call gives the bits of the five calls made one by one, with fresh outputs (the status word
+    starts from whatever was in memory) and with kept ones, and names the stage that refuses its arguments."""
+    import paper_2502_14317_b200 as pc
+    g = torch.Generator(device="cuda").manual_seed(C + L)
+    q, kk, v = (torch.randn((C, L, h, d), generator=g, device="cuda").bfloat16() for h in (Hq, Hkv, Hkv))
+    if strided:
+        q = torch.cat([q, q], dim=2)[:, :, :Hq]
+    score = torch.randn(C, generator=g, device="cuda") if given else None
+    pre = pc.chunk_prefill_attn(q, kk, v, w=w, rope_theta=1e4)
+    if given:
+        want_score, kept = score, pc.select_chunks(score, m, True)
+    else:
+        want_score, kept = pc.score_select_chunks(pre["win_lse"], m, True)
+    idx = pc.select_tokens(pre["win_score"], kept, L - w, k)
+    kc, vc, pos = pc.gather_kv(pre["k_rot"], v, kept, idx)
+    fg = pc.parallel_attn(q[0:1, L - w:].contiguous(), kc[None], vc[None], pre["k_rot"][0:1, L - w:].contiguous(),
+                          v[0:1, L - w:].contiguous(), q_pos0=L - w, rope_theta=1e4)["out"]
+    want = {"o": pre["o"], "k_rot": pre["k_rot"], "win_score": pre["win_score"], "win_lse": pre["win_lse"], "chunk_score": want_score,
+            "kept": kept, "idx": idx, "kc": kc, "vc": vc, "pos": pos, "fg": fg}
+    junk = [torch.full((n,), -1, dtype=torch.int32, device="cuda") for n in (1, 2, 64)]        # freed: fresh memory is not zero
+    del junk
+    buffers = {}
+    for b in (None, buffers, buffers):
+        got = pc.hot_path(q, kk, v, w=w, rope_theta=1e4, m=m, k_keep=k, chunk_score=score, buffers=b)
+        torch.cuda.synchronize()
+        assert int(got["status"].item()) == 0
+        for key, t in want.items():
+            assert torch.equal(got[key], t), key
+    for bad, stage in ((dict(w=L), "pc_chunk_prefill_attn"), (dict(k_keep=0), "pc_select_tokens"),
+                       (dict(m=C + 1), "pc_select_chunks" if given else "pc_score_select_chunks")):
+        with pytest.raises(pc.PcError, match=stage):
+            pc.hot_path(q, kk, v, **{**dict(w=w, rope_theta=1e4, m=m, k_keep=k, chunk_score=score), **bad})
+
+
 def test_hot_path_from_host_matches_device_path(cfg0_inputs):
     """Uploading the chunks in groups on a copy stream must give exactly what the all-on-device path gives."""
     import paper_2502_14317_b200 as pc
