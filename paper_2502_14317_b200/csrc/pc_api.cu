@@ -378,7 +378,6 @@ int32_t pc_queue_emit(const int32_t* q_chunk, int32_t m, int32_t Hkv, int32_t k,
 namespace {
 
 struct ParallelPlan {
-  int few_split;                   // few query rows (pc_decode.cu, no workspace): CTAs of a cluster per (sequence, kv-head); 0:
   bool pair;                       // pc_parallel.cu on CTA pairs (else single CTAs)
   int alt, n_rg, n_cache_tiles, n_split;   // see ParallelParams
   size_t off_counter, off_table, off_table_hi, off_table_lo, off_qrot, off_ml, off_o, total;
@@ -444,23 +443,6 @@ ParallelPlan parallel_plan(int B, int w, int Hq, int Hkv, int d, int Nk, int sm_
     const double cost = rounds * (5.0 + (p.alt ? 1.4 : 2.8) * std::ceil((double)n_all / s)) + (s > 1 ? 4.0 : 0.0);
     if (least_us < 0.0 || cost < least_us) { least_us = cost; p.n_split = s; }
   }
-
-  // few query rows (at most 32 per kv-head: the line is drawn where the transposed kernel stops winning, figures in
-  // pc_decode.cu): CTAs per (sequence, kv-head), 0: another kernel.  Least time by a model in microseconds - rounds of the
-  // grid (two CTAs per SM) x (about 6 for prologue, pipeline fill and merge + a tile at the CTA's share of
-  // the memory bandwidth, no faster than the 50 GB/s that its three stages in flight give it: one sequence over 16401
-  // entries measured 26.7 us with 8 splits per head)
-  p.few_split = 0;
-  if (G * w <= 32) {
-    const double slots = 2.0 * sm_count, tile_us = 512.0 * d / 6.5e6;
-    double least = -1.0;
-    for (int s = 1; s <= 16 && s <= p.n_cache_tiles + 1; s *= 2) {
-      const double ctas = (double)B * Hkv * s, rounds = std::ceil(ctas / slots), active = ctas < slots ? ctas : slots;
-      const double per_tile = tile_us * active > 512.0 * d / 5e4 ? tile_us * active : 512.0 * d / 5e4;
-      const double cost = rounds * (6.0 + per_tile * std::ceil((p.n_cache_tiles + 1.0) / s));
-      if (least < 0.0 || cost < least) { least = cost; p.few_split = s; }
-    }
-  }
   return p;
 }
 
@@ -470,6 +452,45 @@ int32_t check_parallel_args(int B, int w, int Hq, int Hkv, int d, int Nk) {
   if (!pow2_between(w, 1, 128)) return PC_ERR_UNSUPPORTED;      // w = 1: one new token decoding over the cache
   if ((long long)B * Hq > (1 << 24) || Nk > (1 << 28)) return PC_ERR_UNSUPPORTED;
   return PC_OK;
+}
+
+// Clusters of n CTAs of the few-row kernel that the current device runs at a time (asked once per device).
+int few_clusters(int n, bool deep) {
+  static std::atomic<int> known[64][2][17];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  std::atomic<int>& k = known[dev][deep][n];
+  int v = k.load(std::memory_order_relaxed);
+  if (v == 0) k.store(v = pc::decode_clusters(n, deep) + 1, std::memory_order_relaxed);
+  return v - 1;
+}
+
+// Few query rows (pc_decode.cu, no workspace): CTAs of a cluster per (sequence, kv-head), 0: another kernel.  At most 32
+// rows per kv-head: the line is drawn where the transposed kernel stops winning, figures in pc_decode.cu.
+struct FewPlan { int split; bool deep; };
+FewPlan few_plan(int B, int w, int Hq, int Hkv, int d, int n_cache_tiles) {
+  FewPlan p = {0, false};
+  if (Hq / Hkv * w > 32) return p;
+  // Least time by a model in microseconds: rounds of clusters x (6.5 for prologue, pipeline fill and merge + a tile at the
+  // CTA's share of the memory bandwidth, no faster than one CTA alone takes it).  Head size 128 has a build with six 32 KB stages and one
+  // CTA per SM: alone it takes a tile in 0.67 us, with three stages in 1.43 (the load of the next but one tile then waits for
+  // the products of this one).  Measured, us, three stages / six, best split of each: 16401 entries x 8 kv-heads, one
+  // sequence 20.5 (16 CTAs) / 17.0 (10), two 27.9 (12) / 26.0 (6), four 44.7 (8) / 43.4 (4); 4 kv-heads 18.0 (16) / 13.5 (16);
+  // 16 sequences of 8192 81.6 (2) / 81.1 (1).
+  const bool wide = Hq / Hkv * w > 16;
+  const double tile_us = 512.0 * d / 6.5e6;
+  double least = -1.0;
+  for (int deep = 0; deep <= (d == 128 ? 1 : 0); ++deep) {
+    const double alone = d == 128 ? (deep ? (wide ? 1.25 : 0.67) : (wide ? 1.5 : 1.43)) : (wide ? 1.3 : 0.62);
+    for (int s = 1; s <= 16 && s <= n_cache_tiles + 1; ++s) {
+      const int fit = few_clusters(s, deep != 0);
+      if (fit < 1) continue;
+      const double items = (double)B * Hkv, rounds = std::ceil(items / fit), active = (items < fit ? items : fit) * s;
+      const double cost = rounds * (6.5 + (tile_us * active > alone ? tile_us * active : alone) * std::ceil((n_cache_tiles + 1.0) / s));
+      if (least < 0.0 || cost < least) { least = cost; p = {s, deep != 0}; }
+    }
+  }
+  return p;
 }
 
 int plan_sm_count() {
@@ -525,7 +546,8 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   const uint32_t box_kw[4] = {64, 1, 128, 1};
 
   const double softmax_scale_d = softmax_scale > 0.0f ? (double)softmax_scale : 1.0 / std::sqrt((double)d);
-  if (plan.few_split > 0) {
+  const FewPlan few = few_plan(B, w, Hq, Hkv, d, plan.n_cache_tiles);
+  if (few.split > 0) {
     CUtensorMap dm[4];
     if (!pc::make_tmap_bf16_4d(&dm[0], k_cache, kc_dims, kc_str, box_kc) ||
         !pc::make_tmap_bf16_4d(&dm[1], v_cache, kc_dims, kc_str, box_kc) ||
@@ -534,7 +556,7 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
       return PC_ERR_CUDA;
     pc::DecodeParams dp;
     dp.B = B; dp.w = w; dp.Hq = Hq; dp.Hkv = Hkv; dp.Nk = Nk;
-    dp.n_cache_tiles = plan.n_cache_tiles; dp.n_split = plan.few_split;
+    dp.n_cache_tiles = plan.n_cache_tiles; dp.n_split = few.split; dp.deep = few.deep;
     dp.q_pos0 = q_pos0; dp.rope_theta = rope_theta;
     dp.scale_log2 = (float)(softmax_scale_d * 1.4426950408889634);
     dp.q_win = q_win; dp.k_win = k_win; dp.v_win = v_win;

@@ -47,6 +47,7 @@ cudaError_t launch_parallel_attn(const CUtensorMap* maps, const ParallelParams& 
 struct DecodeParams {
   int B, w, Hq, Hkv, Nk;
   int n_cache_tiles, n_split;    // 128-key tiles of the cache; CTAs (of a cluster) per (sequence, kv-head), 1 .. 16
+  int deep;                      // head size 128: six stages and one CTA per SM, not three and two
   int q_pos0;
   float rope_theta, scale_log2;
   const void *q_win, *k_win, *v_win;
@@ -59,5 +60,7 @@ struct DecodeParams {
 };
 // maps: k_cache, v_cache (128-key box), k_win, v_win (128-row box over w tokens)
 cudaError_t launch_decode_attn(const CUtensorMap* maps, const DecodeParams& prm, int d, cudaStream_t st);
+// clusters of n_split CTAs that the current device runs at a time
+int decode_clusters(int n_split, bool deep);
 
 }  // namespace pc

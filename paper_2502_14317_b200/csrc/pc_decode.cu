@@ -13,10 +13,17 @@
 // 2^8 times it needs one barrier vote and no reduction over keys.  Row sums stay per thread until the end.
 //
 // A (sequence, kv-head) is split over the CTAs of a cluster (1 to 16), which merge through distributed shared memory.
-// Two CTAs per SM, three 32 KB stages each: the prologue of one runs under the copies of the other.
+// Many items: two CTAs per SM, three 32 KB stages each, the prologue of one under the copies of the other.  Few items of head size
+// 128, where a CTA alone must take its tiles fast: one CTA per SM with six stages (rule and figures: few_plan in pc_api.cu).
+//
+// What bounds it: many sequences, the copy bandwidth; one sequence, latencies - of 39 K cycles over 16401 entries (one token,
+// 8 kv-heads, ten CTAs each, caches cold) 27 K pass in the tiles, 3 K before the queries are asked for (their
+// angles, under the kernel ahead where there is one), 5 K in the queries' rotation, 4 K in the merge.
 //
 // Measured on caches of 16401 entries, 32 q-heads over 8 kv-heads of size 128, against the row-major kernel with its
-// five other launches: 64 sequences, one token 867 -> 652 us (6.6 TB/s, the copy bandwidth); one sequence 46.6 -> 28.7 us.
+// five other launches: 64 sequences, one token 867 -> 642 us (6.7 TB/s, the copy bandwidth); one sequence 46.6 -> 16.7 us
+// (28.7 with three stages everywhere, a load per query row where it is used and the splits read one after the other
+// in the merge).  8 tokens, 4096 entries, one sequence: 20.4 -> 13.2 us with those three changed.
 // 32 rows (64 sequences, 8 tokens, 8000 entries): 521 -> 434 us.  With 64 rows the chain of a tile (64 exponentials a
 // thread between two products) outlasts the copies: 500 -> 626 us, so those stay with the row-major kernel.
 // Warps: 0-3 softmax and epilogue, 4 TMA producer, 5 MMA issuer; all but 4 rotate queries first.
@@ -35,10 +42,11 @@ constexpr int MAX_STAGES = 6;
 
 enum { WD_KV = 301, WD_FREE, WD_S, WD_P, WD_PV };
 
-template <int D, int N>
+// DEEP: twice the stages, one CTA per SM (head size 128 only)
+template <int D, int N, bool DEEP>
 struct Lay {
   static constexpr int TILE_BYTES = TILE * D * 2;
-  static constexpr int NS = D == 128 ? 3 : 6;
+  static constexpr int NS = (D == 128 ? 3 : 6) * (DEEP ? 2 : 1);
   static constexpr int OFF_Q = NS * TILE_BYTES;
   static constexpr int OFF_P = OFF_Q + N * D * 2;
   static constexpr int OFF_MISC = OFF_P + N * TILE * 2;
@@ -74,6 +82,39 @@ __device__ __forceinline__ float warp_max(float x) {               // order-pres
   i = __reduce_max_sync(0xFFFFFFFFu, i);
   return __int_as_float(i ^ ((i >> 31) & 0x7FFFFFFF));
 }
+// Sums over the lanes of N values per lane: the sum of x[i] in lane i (N = 16: also in lane i + 16).  Halves the values a lane
+// holds with every exchange, N - 1 exchanges in all instead of 5 N.
+template <int N>
+__device__ __forceinline__ float lane_sums(float (&x)[N], int lane) {
+#pragma unroll
+  for (int o = N / 2; o > 0; o >>= 1) {
+    const bool upper = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < o; ++j) {
+      const float give = upper ? x[j] : x[j + o], keep = upper ? x[j + o] : x[j];
+      x[j] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+    }
+  }
+  return N == 16 ? x[0] + __shfl_xor_sync(0xFFFFFFFFu, x[0], 16) : x[0];
+}
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+// sum over the CTAs s < ns of weight[s] * (four floats at addr in CTA s); all reads are in flight together
+template <int MAX>
+__device__ __forceinline__ float4 sum_splits(const float* addr, const float* weight, int ns, int self) {
+  float4 x[MAX], acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+  for (int s = 0; s < MAX; ++s) x[s] = ld_cluster_f32x4(map_to_cta(addr, s < ns ? s : self));   // (weight 0 there)
+#pragma unroll
+  for (int s = 0; s < MAX; ++s) {
+    acc.x = fmaf(weight[s], x[s].x, acc.x); acc.y = fmaf(weight[s], x[s].y, acc.y);
+    acc.z = fmaf(weight[s], x[s].z, acc.z); acc.w = fmaf(weight[s], x[s].w, acc.w);
+  }
+  return acc;
+}
 template <int N>
 __device__ __forceinline__ void load_cols(uint32_t taddr, float (&s)[N]) {
   uint32_t a[N];
@@ -85,12 +126,12 @@ __device__ __forceinline__ void load_cols(uint32_t taddr, float (&s)[N]) {
 
 }  // namespace
 
-template <int D, int N>
-__global__ void __launch_bounds__(NTD, 2)
+template <int D, int N, bool DEEP>
+__global__ void __launch_bounds__(NTD, DEEP ? 1 : 2)
 decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_constant__ CUtensorMap tm_vc,
                    const __grid_constant__ CUtensorMap tm_kw, const __grid_constant__ CUtensorMap tm_vw,
                    const __grid_constant__ DecodeParams prm) {
-  using Y = Lay<D, N>;
+  using Y = Lay<D, N, DEEP>;
   extern __shared__ __align__(1024) uint8_t smem[];
   Misc<N>& mi = *reinterpret_cast<Misc<N>*>(smem + Y::OFF_MISC);
   volatile int* const abort_flag = &mi.abort_flag;
@@ -135,25 +176,47 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
     auto q_slot = [&](int r, int e) -> uint16_t* {
       return reinterpret_cast<uint16_t*>(smem + Y::OFF_Q + (e / 64) * (N * 128) + sw128_offset(r, (e % 64) / 8) + (e % 8) * 2);
     };
-    double sn = 0.0, cs = 0.0;
-    auto turn = [&](int e) { sincos((double)(prm.q_pos0 + e / HALF) * pow((double)prm.rope_theta, -2.0 * (double)(e % HALF) / (double)D), &sn, &cs); };
-    if (rt < w * HALF) turn(rt);                              // needs nothing from before this launch
+    // a thread keeps its pair over the tokens: one pow, and the angles of its first tokens need nothing from before this launch
+    constexpr int TURNERS = (NTD - 32) / HALF * HALF, STEP = TURNERS / HALF, AHEAD = 3;
+    const int t = rt % HALF, i_first = rt < TURNERS ? rt / HALF : w;
+    double sn[AHEAD], cs[AHEAD], freq = 0.0;
+    auto turn = [&](int i, double& s, double& c) { sincos((double)(prm.q_pos0 + i) * freq, &s, &c); };
+    if (i_first < w) freq = pow((double)prm.rope_theta, -2.0 * (double)t / (double)D);
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k)
+      if (i_first + k * STEP < w) turn(i_first + k * STEP, sn[k], cs[k]);
     chain();
-    for (int e = rt; e < w * HALF; e += NTD - 32) {
-      const int i = e / HALF, t = e % HALF;
-      if (e != rt) turn(e);
+    // the rows as they are first go to the P buffer, all loads in flight at once (a load per row and pair where it is needed
+    // puts their latencies in a row)
+    uint16_t* const raw = reinterpret_cast<uint16_t*>(smem + Y::OFF_P);             // [token * G + g][D]
+    for (int e = rt; e < R * (D / 8); e += NTD - 32) {
+      const int i = e / (G * (D / 8)), c = e - i * (G * (D / 8));
+      reinterpret_cast<uint4*>(raw)[e] = __ldg(reinterpret_cast<const uint4*>(qs + (size_t)i * prm.Hq * D) + c);
+    }
+    named_barrier_sync(3, NTD - 32);
+    auto rotate = [&](int i, double s, double c) {
+#pragma unroll 4
       for (int g = 0; g < G; ++g) {
-        const uint16_t* const x = qs + ((size_t)i * prm.Hq + g) * D + t;
+        const uint16_t* const x = raw + (i * G + g) * D + t;
         const double a = (double)__uint_as_float((uint32_t)x[0] << 16), b = (double)__uint_as_float((uint32_t)x[HALF] << 16);
-        *q_slot(g * w + i, t) = f64_to_bf16_rne(a * cs - b * sn);
-        *q_slot(g * w + i, t + HALF) = f64_to_bf16_rne(b * cs + a * sn);
+        *q_slot(g * w + i, t) = f64_to_bf16_rne(a * c - b * s);
+        *q_slot(g * w + i, t + HALF) = f64_to_bf16_rne(b * c + a * s);
       }
+    };
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k)
+      if (i_first + k * STEP < w) rotate(i_first + k * STEP, sn[k], cs[k]);
+    for (int i = i_first + AHEAD * STEP; i < w; i += STEP) {
+      double s, c;
+      turn(i, s, c);
+      rotate(i, s, c);
     }
     // operand rows that are no query rows: zero queries and zero probabilities
     for (int e = rt; e < (N - R) * (D / 8); e += NTD - 32) {
       const int r = R + e / (D / 8), c = e % (D / 8);
       *reinterpret_cast<uint4*>(smem + Y::OFF_Q + (c / 8) * (N * 128) + sw128_offset(r, c % 8)) = make_uint4(0, 0, 0, 0);
     }
+    named_barrier_sync(3, NTD - 32);
     for (int e = rt; e < (N - R) * (TILE / 8); e += NTD - 32) {
       const int r = R + e / (TILE / 8), c = e % (TILE / 8);
       *reinterpret_cast<uint4*>(smem + Y::OFF_P + (c / 8) * (N * 128) + sw128_offset(r, c % 8)) = make_uint4(0, 0, 0, 0);
@@ -321,15 +384,8 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
     // ---- row sums over the keys, then O^T (thread = head-dim column)
     mbar_wait(&mi.pv_done, full_par(n - 1), abort_flag, prm.status, WD_PV);
     tc_fence_after_sync();
-#pragma unroll
-    for (int r = 0; r < N; ++r) {
-      if (r < R) {
-        float x = l[r];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-        if (lane == 0) mi.red[warp][r] = x;
-      }
-    }
+    const float row_sum = lane_sums<N>(l, lane);
+    if (lane < N) mi.red[warp][lane] = row_sum;
     named_barrier_sync(1, 128);
     float o[N];
     load_cols<N>(tO + lane_sel, o);
@@ -357,23 +413,38 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
   }
 
   if (ns > 1) {
-    // ---- merge of the splits: every CTA takes a slice of the output, reading all CTAs' partial results
+    // ---- merge of the splits: every CTA takes a slice of the output.  First the weights of the splits in its rows, a warp
+    // per row and a lane per split, then the sums; the remote reads of a step are all in flight together.
     cluster_sync_all();
-    const int total = R * D, chunk = (total + ns - 1) / ns;
-    for (int e = split * chunk + tid; e < total && e < (split + 1) * chunk; e += NTD) {
-      const int r = e / D, dd = e % D, wi = r % w, g = r / w;
-      float m = -INFINITY;
-      for (int s = 0; s < ns; ++s) m = fmaxf(m, -ld_cluster_f32(map_to_cta(&mi.negm[r], s)));
-      float acc = 0.0f, lt = 0.0f;
-      for (int s = 0; s < ns; ++s) {
-        const float f = exp2f(-ld_cluster_f32(map_to_cta(&mi.negm[r], s)) - m);
-        const float ls = (ld_cluster_f32(map_to_cta(&mi.red[0][r], s)) + ld_cluster_f32(map_to_cta(&mi.red[1][r], s))) +
-                         (ld_cluster_f32(map_to_cta(&mi.red[2][r], s)) + ld_cluster_f32(map_to_cta(&mi.red[3][r], s)));
-        acc = fmaf(f, ld_cluster_f32(map_to_cta(smem + (size_t)e * 4, s)), acc);
-        lt = fmaf(f, ls, lt);
+    const int total = R * D, chunk = (total / 4 + ns - 1) / ns * 4, e0 = split * chunk, e1 = e0 + chunk < total ? e0 + chunk : total;
+    float* const weight = reinterpret_cast<float*>(smem + Y::TILE_BYTES);           // [row][16], behind the partial results
+    for (int r = e0 / D + warp; r * D < e1; r += NTD / 32) {
+      float m = -INFINITY, l = 0.0f;
+      if (lane < ns) {
+        m = -ld_cluster_f32(map_to_cta(&mi.negm[r], lane));
+        l = (ld_cluster_f32(map_to_cta(&mi.red[0][r], lane)) + ld_cluster_f32(map_to_cta(&mi.red[1][r], lane))) +
+            (ld_cluster_f32(map_to_cta(&mi.red[2][r], lane)) + ld_cluster_f32(map_to_cta(&mi.red[3][r], lane)));
       }
-      prm.out[(((size_t)seq * w + wi) * prm.Hq + hkv * G + g) * D + dd] = __float2bfloat16_rn(acc / lt);
-      if (prm.lse_out != nullptr && dd == 0) prm.lse_out[((size_t)seq * prm.Hq + hkv * G) * w + r] = (m + log2f(lt)) * 0.6931471805599453f;
+      float top = m;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+      const float f = lane < ns ? exp2f(m - top) : 0.0f;
+      float sum = f * l;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+      if (lane < 16) weight[r * 16 + lane] = f / sum;
+      if (prm.lse_out != nullptr && lane == 0 && r * D >= e0)
+        prm.lse_out[((size_t)seq * prm.Hq + hkv * G) * w + r] = (top + log2f(sum)) * 0.6931471805599453f;
+    }
+    __syncthreads();
+    for (int e = e0 + 4 * tid; e < e1; e += 4 * NTD) {
+      const int r = e / D, dd = e % D, wi = r % w, g = r / w;
+      const float* const part = reinterpret_cast<const float*>(smem) + e;
+      const float* const wr = weight + r * 16;
+      const float4 o = ns > 8 ? sum_splits<16>(part, wr, ns, split) : ns > 4 ? sum_splits<8>(part, wr, ns, split) :
+                       ns > 2 ? sum_splits<4>(part, wr, ns, split) : sum_splits<2>(part, wr, ns, split);
+      *reinterpret_cast<uint2*>(prm.out + (((size_t)seq * w + wi) * prm.Hq + hkv * G + g) * D + dd) =
+          make_uint2(pack_bf16x2(o.x, o.y), pack_bf16x2(o.z, o.w));
     }
     cluster_sync_all();                                       // no CTA exits while another may read its shared memory
   }
@@ -387,23 +458,50 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
   }
 }
 
-template <int D, int N>
-static cudaError_t launch_decode_t(const CUtensorMap* maps, const DecodeParams& prm, cudaStream_t st) {
-  using Y = Lay<D, N>;
+template <int D, int N, bool DEEP>
+static cudaError_t prepare(int n_split) {
+  using Y = Lay<D, N, DEEP>;
   constexpr int SMEM = Y::OFF_MISC + (int)sizeof(Misc<N>);
-  static_assert(2 * (SMEM + 1024) <= 233472, "two CTAs per SM");
-  auto* const kernel = decode_attn_kernel<D, N>;
+  static_assert((DEEP ? 1 : 2) * (SMEM + 1024) <= 233472, "CTAs per SM");
+  auto* const kernel = decode_attn_kernel<D, N, DEEP>;
   if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM); e != cudaSuccess) return e;
-  if (prm.n_split > 8)
-    if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); e != cudaSuccess) return e;
-  return launch_chained(kernel, dim3((unsigned)(prm.B * prm.Hkv * prm.n_split)), dim3(NTD), SMEM, st, prm.n_split, maps[0], maps[1], maps[2],
-                        maps[3], prm);
+  return n_split > 8 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess;
+}
+template <int D, int N, bool DEEP>
+static cudaError_t launch_decode_t(const CUtensorMap* maps, const DecodeParams& prm, cudaStream_t st) {
+  if (cudaError_t e = prepare<D, N, DEEP>(prm.n_split); e != cudaSuccess) return e;
+  return launch_chained(decode_attn_kernel<D, N, DEEP>, dim3((unsigned)(prm.B * prm.Hkv * prm.n_split)), dim3(NTD),
+                        Lay<D, N, DEEP>::OFF_MISC + sizeof(Misc<N>), st, prm.n_split, maps[0], maps[1], maps[2], maps[3], prm);
+}
+template <int D, int N>
+static cudaError_t launch_decode_n(const CUtensorMap* maps, const DecodeParams& prm, cudaStream_t st) {
+  if constexpr (D == 128)
+    if (prm.deep) return launch_decode_t<D, N, true>(maps, prm, st);
+  return launch_decode_t<D, N, false>(maps, prm, st);
 }
 
 cudaError_t launch_decode_attn(const CUtensorMap* maps, const DecodeParams& prm, int d, cudaStream_t st) {
   const int rows = prm.Hq / prm.Hkv * prm.w;
-  if (d == 128) return rows <= 16 ? launch_decode_t<128, 16>(maps, prm, st) : launch_decode_t<128, 32>(maps, prm, st);
-  return rows <= 16 ? launch_decode_t<64, 16>(maps, prm, st) : launch_decode_t<64, 32>(maps, prm, st);
+  if (d == 128) return rows <= 16 ? launch_decode_n<128, 16>(maps, prm, st) : launch_decode_n<128, 32>(maps, prm, st);
+  return rows <= 16 ? launch_decode_n<64, 16>(maps, prm, st) : launch_decode_n<64, 32>(maps, prm, st);
 }
+
+template <bool DEEP>
+static int clusters_t(int n_split) {                          // the largest of the builds: what fits there fits everywhere
+  if (prepare<128, 32, DEEP>(n_split) != cudaSuccess) { cudaGetLastError(); return 0; }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)n_split);
+  cfg.blockDim = dim3(NTD);
+  cfg.dynamicSmemBytes = Lay<128, 32, DEEP>::OFF_MISC + sizeof(Misc<32>);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {(unsigned)n_split, 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, decode_attn_kernel<128, 32, DEEP>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return n;
+}
+int decode_clusters(int n_split, bool deep) { return deep ? clusters_t<true>(n_split) : clusters_t<false>(n_split); }
 
 }  // namespace pc

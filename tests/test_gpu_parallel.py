@@ -77,6 +77,26 @@ def test_few_query_rows(B, w, Hq, Hkv, d, Nk, grow):
     assert np.abs(res["lse"].cpu().numpy() - LSE).max() <= 2e-3
 
 
+@pytest.mark.parametrize("B,w,Hq,Hkv,d,Nk", [
+    (1, 1, 4, 1, 128, 20000), (1, 1, 10, 10, 128, 5000), (3, 1, 12, 6, 128, 3000),   # deep ring, 16, 9 or 10 and fewer CTAs; stages reused
+    (1, 16, 4, 2, 128, 300), (80, 8, 8, 2, 128, 300),                            # 16 tokens: angles found in the loop; three stages, 32 rows
+    (75, 1, 4, 2, 128, 1000), (2, 32, 1, 1, 64, 2500),
+])
+def test_few_query_rows_deep_and_shallow_rings(B, w, Hq, Hkv, d, Nk):
+    """The two builds of the transposed kernel (few items: six stages; many: three), odd cluster sizes and long token loops."""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(Nk + B)
+    qw, kw, vw = (_bits(rng, (B, w, h, d)) for h in (Hq, Hkv, Hkv))
+    kc, vc = _bits(rng, (B, Hkv, Nk, d)), _bits(rng, (B, Hkv, Nk, d))
+    res = pc.parallel_attn(to_dev(qw), to_dev(kc), to_dev(vc), to_dev(kw), to_dev(vw), q_pos0=777, rope_theta=1e4, want_lse=True)
+    torch.cuda.synchronize()
+    assert int(res["status"].item()) == 0
+    for b in sorted({0, B // 2, B - 1}):
+        Fg, LSE = orc.parallel_attention(qw[b:b + 1], 777, 1e4, None, *(x[b:b + 1] for x in (kc, vc, kw, vw)))
+        check_attention_output(to_f64(res["out"][b:b + 1]), Fg, "Fg")
+        assert np.abs(res["lse"][b:b + 1].cpu().numpy() - LSE).max() <= 2e-3
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,d,Nk0,cap,steps", [
     (2, 8, 2, 128, 250, 260, (1, 1, 4, 1)),   # crosses a tile boundary of the cache (256) while generating
     (3, 4, 4, 64, 40, 48, (1, 2, 1)),         # MHA, head size 64
