@@ -61,6 +61,7 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     for (int i = tid; i < NQ * C::Q_BYTES / 16; i += NT2) reinterpret_cast<uint4*>(smem + Off<C>::Q)[i] = make_uint4(0, 0, 0, 0);
     fence_proxy_async_smem();
   }
+  if (tid == WARP_PRODUCER * 32) { tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kc); tma_prefetch_desc(&tm_vc); }
   Ctx2 cx;
   setup<C>(cx, smem, prm.status, prm.wait_kcycles, leader);
   Misc2& mi = *cx.mi;
@@ -72,7 +73,6 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
       // ================================================================ TMA producer (both CTAs of a pair)
       if (elect_one()) {
         const int n_items = prm.B * prm.Hkv * prm.n_rg * prm.n_split;
-        tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kc); tma_prefetch_desc(&tm_vc);
         Prod p;
         // once a wait has run out (abort flag) no new work is started
         while (!*cx.abort_flag) {
@@ -263,9 +263,7 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                                           pack_bf16x2(x[i * 8 + 4], x[i * 8 + 5]), pack_bf16x2(x[i * 8 + 6], x[i * 8 + 7]));
           } else if (valid) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-              out[q * 4 + i] = make_uint4(__float_as_uint(x[i * 4]), __float_as_uint(x[i * 4 + 1]), __float_as_uint(x[i * 4 + 2]),
-                                          __float_as_uint(x[i * 4 + 3]));
+            for (int i = 0; i < 2; ++i) st_global_f32x8(out + q * 4 + i * 2, &x[i * 8]);
           }
         }
         warp_arrive_leader(in_cta<C>(&mi.o_free[alt ? 0 : b0], 0));

@@ -125,6 +125,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0;
   const bool leader = (rank == 0);
+  if (tid == WARP_PRODUCER * 32) {
+    tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kh); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
+    tma_prefetch_desc(&tm_qw);
+  }
   Ctx2 cx;
   setup<C>(cx, smem, prm.status, prm.wait_kcycles, leader);
   Misc2& mi = *cx.mi;
@@ -138,8 +142,6 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const Sched2 sch = make_sched2<D>(prm);
         const int n_groups = prm.C * prm.Hkv, n_items = n_groups * sch.ipg;
         const int rows_half = sch.hp * sch.wp;           // sweep operand rows per CTA and pass (B operand half)
-        tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kh); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
-        tma_prefetch_desc(&tm_qw);
         Prod p;
         // Once a wait has run out (abort flag) no new work is started: every role leaves its loops at the next
         // descriptor, this one also at the next tile, so that no copy is issued into a ring that nobody drains.
