@@ -40,10 +40,10 @@ __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict_
 // piece of the token's row (1 KB for d = 128), and a block of 8 warps streams 8 adjacent rows: the DRAM pages
 // are walked front to back, as a copy would.  The table entries of (position, pairs) stay in registers across
 // the heads and across the chunks of the block's slice.
-// Outputs that the fp32 arithmetic cannot decide (about one in 1300) are redone exactly by the whole warp: the
-// sixteen outputs of an undecided lane go to sixteen lanes, one each, and are patched into the row after the
-// vector store.  (Handling them in the lane that found them would make a third of the warp's passes wait for one
-// lane's slow path.)
+// Outputs that the fp32 arithmetic cannot decide (about one in 1300, so something in a third of a warp's passes) are redone
+// exactly: a lane that has any leaves its sixteen inputs in a list of the warp, and whenever there are two such lanes
+// on the list their thirty-two outputs go to the thirty-two lanes and are patched into the rows.  (One lane at a time, its
+// inputs spread by shuffles: a third of all instructions, 117 us where this takes 112.)
 //
 // One launch takes one or two tensors of the same chunks and positions (keys and queries): grid.y first deals out the slices of
 // the chunks of the first tensor, then those of the second.
@@ -51,6 +51,13 @@ __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict_
 // OWN_TABLE: a warp computes the table row of its position itself, in shared memory, before it waits for the kernel ahead
 // (see launch_rope).
 struct RopeAngles { double theta; int pos0; int *counter, *clear; };   // for OWN_TABLE; counter and clear (may be null) are set to 0
+__device__ __forceinline__ void copy_async16(void* smem_dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
+struct RopeTodo { uint4 x1, x2; uint16_t* dst; int g; };       // a lane's inputs, where its outputs go, its group of pairs
 struct RopeRow { float4 hi[32], lo[32]; double2 exact[64]; };
 struct RopeTensor {
   const uint16_t* x;
@@ -66,6 +73,9 @@ __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant
   const int half = d / 2, lane = threadIdx.x & 31;
   const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   RopeRow& row = own[OWN_TABLE ? threadIdx.x >> 5 : 0];
+  __shared__ RopeTodo todo_lists[8][33];
+  RopeTodo* const todo = todo_lists[threadIdx.x >> 5];
+  int n_todo = 0;                                           // the same in all lanes
   if (OWN_TABLE && p < L) {
     for (int t = lane; t < half; t += 32) {
       double2 e;
@@ -107,25 +117,57 @@ __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant
   const size_t step_dst = (size_t)h_step * zs * d;
   const int n_pass = (H + h_step - 1) / h_step;
   const int h_mine = h_first + (int)blockIdx.z * h_step;    // this thread's head in its first pass
-  for (int c = slice; c < C; c += ny) {
-    const uint16_t* src = x + (long long)c * s_chunk + (long long)p * s_tok + (long long)h_mine * s_head + g * 8;
-    uint16_t* const dst_tok = y + ((size_t)c * L + p) * H * d;
-    uint16_t* dst = dst_tok + (size_t)h_mine * d + g * 8;
-    uint4 n1 = make_uint4(0, 0, 0, 0), n2 = make_uint4(0, 0, 0, 0);
-    if (h_mine < H) {
-      n1 = __ldg(reinterpret_cast<const uint4*>(src));
-      n2 = __ldg(reinterpret_cast<const uint4*>(src + half));
+  // outputs of entries i and i + 1 (an entry below 0 is none)
+  auto redo = [&](int i) {
+    __syncwarp();                                           // the list, and the vector stores that the patches follow
+    const int t = (lane >> 1) & 7, second = lane & 1, e = i + (lane >> 4);
+    if (e >= 0) {
+      const RopeTodo& d = todo[e];
+      const float a = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(&d.x1)[t] << 16);
+      const float b = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(&d.x2)[t] << 16);
+      const int pair = d.g * 8 + t;
+      const uint32_t r = second ? rope_one_exact<OWN_TABLE>(b, -a, pair, hi_row, lo_row, d_row)
+                                : rope_one_exact<OWN_TABLE>(a, b, pair, hi_row, lo_row, d_row);
+      d.dst[(second ? half : 0) + t] = (uint16_t)r;
     }
-#pragma unroll 1
-    for (int ps = blockIdx.z; ps < n_pass; ps += zs, src += step_src, dst += step_dst) {
-      const bool active = h_first + ps * h_step < H;
-      const uint4 x1 = n1, x2 = n2;
-      if (ps + zs < n_pass && h_first + (ps + zs) * h_step < H) {                // the next pass's row is in flight during this one's arithmetic
-        n1 = __ldg(reinterpret_cast<const uint4*>(src + step_src));
-        n2 = __ldg(reinterpret_cast<const uint4*>(src + step_src + half));
-      } else {
-        n1 = make_uint4(0, 0, 0, 0); n2 = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+  };
+  // A lane's inputs of the next passes come through a ring in shared memory (its own slots only: nothing to synchronise), so that
+  // DEPTH - 1 passes are in flight; with one in registers the pass was bound by the latency of memory (4 x 8192 x 32 x 128: 110
+  // us, 97 with two or three passes in the ring, 83 at the copy bandwidth; 16 x 8192 x 8 x 128: 116 and 100).
+  constexpr int DEPTH = OWN_TABLE ? 2 : 3;
+  __shared__ uint4 ring[8][DEPTH][2][32];
+  uint4(*const mine)[2][32] = ring[threadIdx.x >> 5];
+  int c_next = slice, ps_next = blockIdx.z;
+  const uint16_t* src = x + (long long)slice * s_chunk + (long long)p * s_tok + (long long)h_mine * s_head + g * 8;
+  auto fetch = [&](int slot) {
+    if (c_next < C) {
+      if (h_first + ps_next * h_step < H) {                 // (lanes without a row compute on what is there and store nothing)
+        copy_async16(&mine[slot][0][lane], src);
+        copy_async16(&mine[slot][1][lane], src + half);
       }
+      ps_next += zs;
+      src += step_src;
+      if (ps_next >= n_pass) {
+        ps_next = blockIdx.z;
+        c_next += ny;
+        src = x + (long long)c_next * s_chunk + (long long)p * s_tok + (long long)h_mine * s_head + g * 8;
+      }
+    }
+    copy_async_commit();
+  };
+#pragma unroll
+  for (int i = 0; i < DEPTH - 1; ++i) fetch(i);
+  int slot = 0;
+  for (int c = slice; c < C; c += ny) {
+    uint16_t* dst = y + ((size_t)c * L + p) * H * d + (size_t)h_mine * d + g * 8;
+#pragma unroll 1
+    for (int ps = blockIdx.z; ps < n_pass; ps += zs, dst += step_dst) {
+      const bool active = h_first + ps * h_step < H;
+      fetch((slot + DEPTH - 1) % DEPTH);
+      copy_async_wait<DEPTH - 1>();
+      const uint4 x1 = mine[slot][0][lane], x2 = mine[slot][1][lane];
+      slot = (slot + 1) % DEPTH;
       uint4 y1, y2;
       uint32_t amb = rope_two_pairs_fast(x1.x, x2.x, hi[0], y1.x, y2.x);
       amb |= rope_two_pairs_fast(x1.y, x2.y, hi[1], y1.y, y2.y);
@@ -135,34 +177,15 @@ __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant
         *reinterpret_cast<uint4*>(dst) = y1;
         *reinterpret_cast<uint4*>(dst + half) = y2;
       }
-      unsigned todo = __ballot_sync(0xFFFFFFFFu, active && amb != 0u);
-      if (todo != 0u) {                                     // warp-uniform
-        __syncwarp();                                       // the vector stores above precede the patches below
-        const int t = (lane >> 1) & 7, second = lane & 1;   // lanes 0..15: pair t of the undecided lane, first / second output
-        do {
-          const int srcl = __ffs(todo) - 1;
-          todo &= todo - 1;
-          const uint32_t w1[4] = {__shfl_sync(0xFFFFFFFFu, x1.x, srcl), __shfl_sync(0xFFFFFFFFu, x1.y, srcl),
-                                  __shfl_sync(0xFFFFFFFFu, x1.z, srcl), __shfl_sync(0xFFFFFFFFu, x1.w, srcl)};
-          const uint32_t w2[4] = {__shfl_sync(0xFFFFFFFFu, x2.x, srcl), __shfl_sync(0xFFFFFFFFu, x2.y, srcl),
-                                  __shfl_sync(0xFFFFFFFFu, x2.z, srcl), __shfl_sync(0xFFFFFFFFu, x2.w, srcl)};
-          if (lane < 16) {
-            const int wsel = t >> 1;
-            const uint32_t u1 = wsel == 0 ? w1[0] : wsel == 1 ? w1[1] : wsel == 2 ? w1[2] : w1[3];
-            const uint32_t u2 = wsel == 0 ? w2[0] : wsel == 1 ? w2[1] : wsel == 2 ? w2[2] : w2[3];
-            const float a = __uint_as_float((t & 1) ? (u1 & 0xFFFF0000u) : (u1 << 16));
-            const float b = __uint_as_float((t & 1) ? (u2 & 0xFFFF0000u) : (u2 << 16));
-            const int sg = srcl % groups, sh = srcl / groups + ps * h_step;      // pair group and head of that lane
-            const int pair = sg * 8 + t;
-            const uint32_t r = second ? rope_one_exact<OWN_TABLE>(b, -a, pair, hi_row, lo_row, d_row)
-                                      : rope_one_exact<OWN_TABLE>(a, b, pair, hi_row, lo_row, d_row);
-            dst_tok[(size_t)sh * d + (second ? half : 0) + pair] = (uint16_t)r;
-          }
-        } while (todo != 0u);
-        __syncwarp();
+      const unsigned undecided = __ballot_sync(0xFFFFFFFFu, active && amb != 0u);
+      if (undecided != 0u) {                                // warp-uniform
+        if ((undecided >> lane) & 1u) todo[n_todo + __popc(undecided & ((1u << lane) - 1u))] = {x1, x2, dst, g};
+        n_todo += __popc(undecided);
+        for (; n_todo >= 2; n_todo -= 2) redo(n_todo - 2);
       }
     }
   }
+  if (n_todo != 0) redo(n_todo - 2);
 }
 
 static RopeTensor rope_tensor(const RopeRows& r, int C, int L, int d) {
@@ -189,12 +212,13 @@ void launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int
   if (b != nullptr) tb = rope_tensor(*b, C, L, d);
   const dim3 grid((unsigned)((L + 7) / 8), (unsigned)(ta.ny + tb.ny), (unsigned)(ta.nz > tb.nz ? ta.nz : tb.nz));
   const RopeAngles ang = {theta, pos0, counter, clear};
-  // Up to 2 M values the warps compute their own table rows: one launch less, and the angles are found while the kernel ahead
-  // still runs (us, table kernel / own rows; B x L x H x d: 1x64x32x128 5.2 / 3.8, 4x256x8x64 5.3 / 4.2, 1x1024x8x128
-  // 7.3 / 5.5, 4x1024x8x64 8.1 / 7.7).  Above it, repeating the fp64 angles in every slice of the chunks and fewer free
-  // registers cost more than the launch (16x64x32x128 9.9 / 10.4, 64x64x32x128 18.7 / 23.3, 4x8192x32x128 118 / 152).
+  // Up to 1 M values the warps compute their own table rows: one launch less, and the angles are found while the kernel ahead
+  // still runs (us, table kernel / own rows; C x L x H x d: 1x64x32x128 4.1 / 2.8, 4x256x8x64 4.2 / 2.9, 1x1024x8x128
+  // 5.5 / 4.8, 4x64x32x128 4.7 / 5.1 and 2 us less host time).  Above it, repeating the fp64 angles in every slice of the
+  // chunks and fewer free registers cost more than the launch (8x64x32x128 5.7 / 6.8, 64x64x32x128 14.7 / 18.1, 4x8192x32x128
+  // 97 / 129).
   const long long values = (long long)C * L * d * (a.H + (b != nullptr ? b->H : 0));
-  if (values <= (1 << 21)) {
+  if (values <= (1 << 20)) {
     launch_chained(rope_rows_kernel<true>, grid, dim3(256), 0, st, 1, ta, tb, tab.hi, tab.lo, tab.exact, C, L, d, ang);
     return;
   }

@@ -75,21 +75,21 @@ __device__ __forceinline__ uint32_t rope_two_pairs_fast(uint32_t x1w, uint32_t x
                                                         uint32_t& up_out) {
   const float a0 = __uint_as_float(x1w << 16), a1 = __uint_as_float(x1w & 0xFFFF0000u);
   const float b0 = __uint_as_float(x2w << 16), b1 = __uint_as_float(x2w & 0xFFFF0000u);
-  const uint64_t A = pack_f32x2(a0, a1), B = pack_f32x2(b0, b1), NB = pack_f32x2(-b0, -b1);
+  const uint64_t A = pack_f32x2(a0, a1), B = pack_f32x2(b0, b1);
   const uint64_t C = pack_f32x2(hi.x, hi.y), S = pack_f32x2(hi.z, hi.w);
-  const uint64_t Y1 = fma_f32x2(NB, S, mul_f32x2(A, C));                 // a c - b s
-  const uint64_t Y2 = fma_f32x2(A, S, mul_f32x2(B, C));                  // b c + a s
-  const float m0 = fabsf(a0) + fabsf(b0), m1 = fabsf(a1) + fabsf(b1);
-  const uint64_t T = pack_f32x2(2.3841858e-7f * m0, 2.3841858e-7f * m1);     // 2^-22 (|a| + |b|)
-  const uint64_t NT = pack_f32x2(-2.3841858e-7f * m0, -2.3841858e-7f * m1);
+  // table entry, product and sum round by 2^-24 each, the test below once more: 4 * 2^-24 (|a c| + |b s|) in all
+  const uint64_t Y1 = fma_f32x2(mul_f32x2(B, S), pack_f32x2(-1.0f, -1.0f), mul_f32x2(A, C));    // a c - b s
+  const uint64_t Y2 = fma_f32x2(A, S, mul_f32x2(B, C));                                         // b c + a s
+  const uint64_t M = pack_f32x2(fabsf(a0) + fabsf(b0), fabsf(a1) + fabsf(b1));
+  const uint64_t T = pack_f32x2(2.3841858e-7f, 2.3841858e-7f), NT = pack_f32x2(-2.3841858e-7f, -2.3841858e-7f);   // 2^-22
   float p, q;
-  unpack_f32x2(add_f32x2(Y1, NT), p, q);
+  unpack_f32x2(fma_f32x2(M, NT, Y1), p, q);
   lo_out = pack_bf16x2(p, q);
-  unpack_f32x2(add_f32x2(Y1, T), p, q);
+  unpack_f32x2(fma_f32x2(M, T, Y1), p, q);
   const uint32_t lo_up = pack_bf16x2(p, q);
-  unpack_f32x2(add_f32x2(Y2, NT), p, q);
+  unpack_f32x2(fma_f32x2(M, NT, Y2), p, q);
   up_out = pack_bf16x2(p, q);
-  unpack_f32x2(add_f32x2(Y2, T), p, q);
+  unpack_f32x2(fma_f32x2(M, T, Y2), p, q);
   const uint32_t up_up = pack_bf16x2(p, q);
   return (lo_out ^ lo_up) | (up_out ^ up_up);
 }
