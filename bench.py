@@ -291,9 +291,9 @@ def run_gpu(args, cfg):
                        kc=kc, vc=vc, pos=pos, fg=pa["out"], ws_par=pa["workspace"])
         return pa["out"]
 
-    # kernels of one step (counted by the library, see pc_launch_count): cos/sin table, rotation of keys and of
-    # queries, chunk attention, stand-in score + chunk top-m, token top-k, gather, window cos/sin table, parallel
-    # attention, merge of its key splits
+    # kernels of one step (counted by the library, see pc_launch_count): cos/sin table, rotation of keys and queries, chunk
+    # attention, stand-in score + chunk top-m, token top-k, gather, rotation of the window, parallel attention, merge of
+    # its key splits
 
     def barrier():
         torch.cuda.synchronize()
@@ -399,8 +399,7 @@ def run_gpu(args, cfg):
                     "h2d_bytes_per_step": int(hq.numel() + hk.numel() + hv.numel()) * 2,
                     "d2h_bytes_per_step": int(h_out.numel()) * 2, "ms_per_step": e2e_ms, "steps": e2e_steps},
             "gpu_launches": launches_timed,
-            "roofline": {"bound": "tensor", "kernel": ("prefill_pair_kernel" if pair_path else "prefill_attn_kernel") +
-                                   " (+ RoPE table and key pre-pass inside the same call)",
+            "roofline": {"bound": "tensor", "kernel": "prefill_kernel (+ RoPE table and rotation pass inside the same call)",
                          "achieved": ach_tflops, "peak": peak_tflops, "unit": "TFLOP/s",
                          "frac": ach_tflops / peak_tflops,
                          "frac_of_burst_peak": ach_tflops / peaks["bf16_tflops"],

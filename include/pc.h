@@ -280,8 +280,7 @@ PC_API int32_t pc_queue_emit(const int32_t* q_chunk, int32_t m, int32_t Hkv, int
  * keys.  Keys arrive already rotated; the queries are rotated into the workspace first
  * (B * w * Hq * d * 2 bytes of it).  Small batches are split over key ranges with an fp32
  * merge; with at most 32 query rows per kv-head (Hq / Hkv * w: decoding steps, short windows) all of it is
- * one launch that needs no workspace (the size asked for is the same); head size 128 with G * w a multiple of 256 and enough (sequence, kv-head) groups to fill the
- * GPU runs unsplit, one 256-row group per CTA pair.
+ * one launch that needs no workspace (the size asked for is the same).
  * q_win [B,w,Hq,d]; k_cache, v_cache [B,Hkv,Nk,d]; k_win, v_win [B,w,Hkv,d];
  * out [B,w,Hq,d] bf16; lse_out [B,Hq,w] fp32 natural log (may be NULL).  All contiguous.
  * Here w may be any power of two in [1, 128]: w = 1 is a decoding step over the compressed

@@ -349,9 +349,10 @@ int32_t pc_queue_select_gather(const float* win_score, const void* k_src, const 
   if (!aligned16(k_src) || !aligned16(v_src) || !aligned16(q_k) || !aligned16(q_v)) return PC_ERR_INVALID_ARG;
   const long long s[3] = {kv_stride[0], kv_stride[1], kv_stride[2]};
   if (s[0] <= 0 || s[1] <= 0 || s[2] < d || s[0] % 8 || s[1] % 8 || s[2] % 8) return PC_ERR_INVALID_ARG;
-  if (device_info().ok != 1) return PC_ERR_UNSUPPORTED;
+  const DeviceInfo& dev = device_info();
+  if (dev.ok != 1) return PC_ERR_UNSUPPORTED;
   const cudaError_t e = pc::launch_select_gather_slots(win_score, slot_src, m, Hkv, L, n_cand, k, k_src, v_src, s, d, q_k,
-                                                       q_v, q_pos, static_cast<cudaStream_t>(stream));
+                                                       q_v, q_pos, dev.sm_count, static_cast<cudaStream_t>(stream));
   if (e == cudaErrorNotSupported) return PC_ERR_UNSUPPORTED;     // k too large to stage: pc_select_tokens + pc_queue_gather
   return e == cudaSuccess ? PC_OK : PC_ERR_CUDA;
 }

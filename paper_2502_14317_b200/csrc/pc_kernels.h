@@ -78,7 +78,7 @@ cudaError_t launch_select_tokens(const float* win_score, const int* kept, int m,
 // storage, in one launch; cudaErrorNotSupported when k is too large for that (then rank and gather separately)
 cudaError_t launch_select_gather_slots(const float* win_score, const int* slot_src, int m, int Hkv, int L, int n_cand,
                                        int k, const void* k_src, const void* v_src, const long long stride_elems[3],
-                                       int d, void* q_k, void* q_v, int* q_pos, cudaStream_t st);
+                                       int d, void* q_k, void* q_v, int* q_pos, int sm_count, cudaStream_t st);
 cudaError_t launch_gather_kv(const void* k_src, const void* v_src, const long long stride_elems[3], const int* kept,
                              const int* idx, int m, int Hkv, int k, int d, void* k_out, void* v_out, int* pos_out,
                              int sm_count, bool by_slot, cudaStream_t st);

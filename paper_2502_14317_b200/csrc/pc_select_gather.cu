@@ -194,7 +194,10 @@ struct SelGather {
 // otherwise (k too large for that) they are stored straight to the index row.
 // SMALL: rows of at most 8192 candidates (256 threads), compiled for five CTAs per SM.
 // GATHER (with STAGE): kept[r] is the batch chunk that moves into queue slot r (-1: the slot keeps its contents and
-// the block returns); positions go to pos_out[hkv, r*k + t] and the rows k_src / v_src[kept[r], pos, hkv] to slot r.
+// the block returns); positions go to pos_out[hkv, r*k + t] and the rows k_src / v_src[kept[r], pos, hkv] to slot r.  The blocks
+// (r * Hkv + hkv, y) all rank the row and each moves its share of the kept rows: one block alone is bound by the latency of
+// its copies (8 kv-heads, 8192 tokens; 4 slots of 512 kept rows 16.2 us with one block a row, 8.6 with eight; 8 slots of 2048 92
+// and 34 with four).
 template <bool CAL, bool STAGE, bool SMALL, bool GATHER = false>
 __global__ void __launch_bounds__(SMALL ? 256 : SEL_MAX_THREADS, SMALL ? SEL_SMALL_CTAS : 1) select_tokens_kernel(const float* __restrict__ win_score,
                                                                         const int* __restrict__ kept, int Hkv, int L,
@@ -361,12 +364,13 @@ __global__ void __launch_bounds__(SMALL ? 256 : SEL_MAX_THREADS, SMALL ? SEL_SMA
       }
     }
     __syncthreads();
-    for (int j = tid; j < k_out; j += blockDim.x) out[j] = j < n_emit ? sel_stage[j] : -1;
+    const int share = GATHER ? (k_out + gridDim.y - 1) / gridDim.y : k_out, j_lo = GATHER ? share * blockIdx.y : 0;
+    const int j_hi = j_lo + share < k_out ? j_lo + share : k_out;
+    for (int j = j_lo + tid; j < j_hi; j += blockDim.x) out[j] = j < n_emit ? sel_stage[j] : -1;
     if (GATHER) {                                              // rows of the kept positions, lpr lanes per row, K and V together
       const int rows_per_warp = 32 / ga.lpr, piece = lane % ga.lpr;
-      for (int j0 = warp * rows_per_warp; j0 < k_out; j0 += nwarps * rows_per_warp) {
-        const int j = j0 + lane / ga.lpr;
-        if (j >= k_out) continue;
+#pragma unroll 4
+      for (int j = j_lo + warp * rows_per_warp + lane / ga.lpr; j < j_hi; j += nwarps * rows_per_warp) {
         const int pos = j < n_emit ? sel_stage[j] : -1;
         uint4 kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
         if (pos >= 0) {
@@ -424,7 +428,7 @@ cudaError_t launch_select_tokens(const float* win_score, const int* kept, int m,
 // the kept positions of a row do not fit the staging buffer (the caller then ranks and gathers in two launches).
 cudaError_t launch_select_gather_slots(const float* win_score, const int* slot_src, int m, int Hkv, int L, int n_cand,
                                        int k, const void* k_src, const void* v_src, const long long stride_elems[3],
-                                       int d, void* q_k, void* q_v, int* q_pos, cudaStream_t st) {
+                                       int d, void* q_k, void* q_v, int* q_pos, int sm_count, cudaStream_t st) {
   int threads = (n_cand + SEL_SPAN - 1) / SEL_SPAN * 32;
   if (threads < 32) threads = 32;
   if (threads > SEL_MAX_THREADS) return cudaErrorInvalidValue;
@@ -436,11 +440,16 @@ cudaError_t launch_select_gather_slots(const float* win_score, const int* slot_s
   ga.s_chunk = stride_elems[0] / 8; ga.s_tok = stride_elems[1] / 8; ga.s_head = stride_elems[2] / 8;
   ga.k_out = (uint4*)q_k; ga.v_out = (uint4*)q_v; ga.pos_out = q_pos;
   ga.lpr = d / 8;
+  // blocks per row: up to eight while there are SMs for them and every block has 32 rows to move
+  int parts = 2 * sm_count / (m * Hkv);
+  if (parts > k / 32) parts = k / 32;
+  parts = parts < 1 ? 1 : (parts > 8 ? 8 : parts);
+  const dim3 grid((unsigned)(m * Hkv), (unsigned)parts);
   if (threads <= 256)
-    launch_chained(select_tokens_kernel<false, true, true, true>, dim3(m * Hkv), dim3(threads), stage_bytes, st, 1, win_score, slot_src, Hkv, L, n_cand, k,
+    launch_chained(select_tokens_kernel<false, true, true, true>, grid, dim3(threads), stage_bytes, st, 1, win_score, slot_src, Hkv, L, n_cand, k,
                                                                                         nullptr, cal, ga);
   else
-    launch_chained(select_tokens_kernel<false, true, false, true>, dim3(m * Hkv), dim3(threads), stage_bytes, st, 1, win_score, slot_src, Hkv, L, n_cand, k,
+    launch_chained(select_tokens_kernel<false, true, false, true>, grid, dim3(threads), stage_bytes, st, 1, win_score, slot_src, Hkv, L, n_cand, k,
                                                                                          nullptr, cal, ga);
   return cudaGetLastError();
 }

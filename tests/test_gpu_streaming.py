@@ -236,3 +236,9 @@ def test_rank_and_compact_in_one_launch_equals_the_two_calls(Cb, L, w, Hkv, d, k
         assert torch.equal(states[0][key].view(torch.int16), states[1][key].view(torch.int16)), key
     assert torch.equal(states[0]["q_pos"], states[1]["q_pos"])
     assert int((states[1]["q_pos"][:, k:2 * k] == -7).all()) == 1     # slot 1 keeps its contents
+
+
+@pytest.mark.parametrize("Cb,L,w,Hkv,d,k,m", [(2, 200, 8, 1, 64, 33, 3), (2, 9000, 64, 4, 128, 1021, 4), (2, 300, 16, 40, 64, 100, 4)])
+def test_rank_and_compact_with_several_blocks_a_row(Cb, L, w, Hkv, d, k, m):
+    """One block a row (33 kept), eight with uneven shares, and more rows than there are SMs."""
+    test_rank_and_compact_in_one_launch_equals_the_two_calls(Cb, L, w, Hkv, d, k, m)
