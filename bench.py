@@ -155,14 +155,26 @@ class ClockSampler:
         self.uuid = uuid
         self.proc = None
         self.tmp = None
+        self.skip = 0
 
     def start(self):
         try:
             self.tmp = tempfile.NamedTemporaryFile("w+", suffix=".csv", delete=False)
             self.proc = subprocess.Popen(["nvidia-smi", f"--query-gpu={self.FIELDS}", "--format=csv,noheader,nounits",
-                                          "-lms", "50", "-i", self.uuid], stdout=self.tmp, stderr=subprocess.DEVNULL)
+                                          "-lms", "20", "-i", self.uuid], stdout=self.tmp, stderr=subprocess.DEVNULL)
         except Exception:
             self.proc = None
+
+    def rows(self) -> int:
+        """Samples written so far."""
+        if self.proc is None:
+            return 0
+        with open(self.tmp.name) as f:
+            return f.read().count("\n")
+
+    def mark(self):
+        """The timed region starts: samples taken before this do not count."""
+        self.skip = self.rows()
 
     def stop(self) -> dict:
         out = {"sm_mhz": None, "sm_max_mhz": None, "reasons": [], "samples": 0}
@@ -175,7 +187,7 @@ class ClockSampler:
             self.proc.kill()
         self.tmp.flush()
         self.tmp.seek(0)
-        rows = [r.strip().split(",") for r in self.tmp.read().strip().splitlines() if r.strip()]
+        rows = [r.strip().split(",") for r in self.tmp.read().strip().splitlines() if r.strip()][self.skip:]
         self.tmp.close()
         os.unlink(self.tmp.name)
         sm, reasons, mx, pw = [], set(), None, []
@@ -301,14 +313,20 @@ def run_gpu(args, cfg):
             dist.barrier()
             torch.cuda.synchronize()
 
+    props = torch.cuda.get_device_properties(dev)
+    sampler = ClockSampler("GPU-" + str(props.uuid)) if rank == 0 else None
+    if sampler: sampler.start()
     for _ in range(args.warmup):
         step()
     barrier()
     assert int(buffers["status"].item()) == 0, "a device-side wait ran out during warm-up"
-
-    props = torch.cuda.get_device_properties(dev)
-    sampler = ClockSampler("GPU-" + str(props.uuid)) if rank == 0 else None
-    if sampler: sampler.start()
+    # the sampler takes a while to start, longer than the timed region may last: keep the GPU busy until it writes
+    if sampler:
+        t0 = time.time()
+        while sampler.rows() == 0 and time.time() - t0 < 2.0:
+            step()
+            torch.cuda.synchronize()
+        sampler.mark()
 
     # ---- timed region: K steps, inputs resident in HBM
     ev = [[torch.cuda.Event(enable_timing=True) for _ in range(5)] for _ in range(args.steps)]
@@ -373,12 +391,11 @@ def run_gpu(args, cfg):
     if rank == 0:
         # DRAM bytes per launch of the dominant kernel: read from the committed ncu summary (a 2-chunk launch
         # of the same shape, scaled by the chunk count); null once the kernel sources differ from the captured ones
-        pair_path = cfg.d == 128 and cfg.G % 2 == 0
         traffic, traffic_note = args.traffic_bytes, "command line"
         if traffic is None:
-            if pair_path and cfg.L == 8192 and cfg.Hq == 32 and cfg.Hkv == 8:
-                traffic, traffic_note = recorded_traffic(["pc_prefill2.cu", "pc_sm100.cuh"],
-                                                         "prefill_pair_kernel_cfg1_C2_ncu_full.md", cfg.C / 2.0)
+            if cfg.d == 128 and cfg.L == 8192 and cfg.Hq == 32 and cfg.Hkv == 8:
+                traffic, traffic_note = recorded_traffic(["pc_prefill2.cu", "pc_flash.cuh", "pc_softmax.cuh", "pc_sm100.cuh"],
+                                                         "prefill_kernel_cfg1_C2_ncu_full.md", cfg.C / 2.0)
             else:
                 traffic_note = "no ncu capture of this shape"
         flops = prefill_flops(cfg)
@@ -496,7 +513,7 @@ def _extra_prefill(pc, torch, dev, peaks, g, out):
         assert int(buf["status"].item()) == 0
         tf = prefill_flops(cfg) / us / 1e6
         out["prefill_" + name] = {"us": us, "tflops": tf, "frac_of_measured_bf16_burst": tf / peaks["bf16_tflops"],
-                                  "kernel": "prefill_pair_kernel" if (cfg.d == 128 and cfg.G % 2 == 0) else "prefill_attn_kernel",
+                                  "kernel": "prefill_kernel",
                                   "workload": workload_description(cfg)["workload"]}
         del q, k, v, buf
         torch.cuda.empty_cache()
