@@ -7,6 +7,9 @@
 
 namespace pc {
 
+// Words that follow a work counter, zeroed with it: blocks with window rows that are done, by (chunk, kv-head) group.
+constexpr int COUNTER_WORDS = 64, MAX_SPREAD_GROUPS = COUNTER_WORDS - 1;
+
 struct PrefillParams {
   int C, L, w, Hq, Hkv;
   float scale_log2;              // softmax scale * log2(e)
@@ -15,7 +18,8 @@ struct PrefillParams {
   float* win_lse;                // [C,Hq,w]
   float* win_score;              // [C,Hkv,L]
   int* status;                   // device status word or null
-  int* counter;                  // work-queue counter, zeroed before launch
+  int* counter;                  // work-queue counter and COUNTER_WORDS - 1 words behind it, zeroed before launch
+  int sweep_slices;              // 0: a group's score sweep belongs to its tail item; n: it is n items of its own (few groups)
   int wait_kcycles;              // limit of every device-side wait, in units of 1024 cycles
   int skip_final_publication;    // test hook of the bounded waits (see pc_debug_bounded_wait_test in pc.h)
 };

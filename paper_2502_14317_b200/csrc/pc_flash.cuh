@@ -118,6 +118,22 @@ __device__ __forceinline__ void warp_arrive_leader(uint32_t leader_addr) {
   if ((threadIdx.x & 31) == 0) mbar_arrive_remote(leader_addr);
 }
 
+// waits until a counter in global memory has reached n (bounded as every wait); the writes before its increments are visible then
+__device__ __forceinline__ void wait_count(const int* count, int n, volatile int* abort_flag, int* status, int where) {
+  const long long t0 = clock64();
+  while (!*abort_flag) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+    if (v >= n) break;
+    if (clock64() - t0 > (static_cast<long long>(abort_flag[1]) << 10)) {
+      if (status) atomicCAS(status, 0, where);
+      *abort_flag = 1;
+    }
+    __nanosleep(100);
+  }
+  __threadfence();
+}
+
 // wait whose completion also makes the peer CTA's earlier writes visible
 __device__ __forceinline__ void mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                   int where) {

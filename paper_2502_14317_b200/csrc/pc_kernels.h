@@ -52,8 +52,8 @@ struct RopeRows {
   void* y;
   int H;
 };
-// one tensor, or two (b not null) in the same launch; positions pos0 .. pos0 + L - 1; counter and clear (may be
-// null) are set to 0
+// one tensor, or two (b not null) in the same launch; positions pos0 .. pos0 + L - 1; the COUNTER_WORDS
+// of counter (pc_attn.h) and clear (each may be null) are set to 0
 void launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int C, int L, int d, double theta, int pos0,
                  int* counter, int* clear, cudaStream_t st);
 

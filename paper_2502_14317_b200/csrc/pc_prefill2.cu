@@ -44,13 +44,17 @@ template <int D> using PCfg = Cfg<D, D == 128>;
 // q-heads, then the score sweep; the other items are one unit each, heaviest first.
 // Items are dealt out in batches of groups whose keys and values stay in L2 together, heaviest first over the whole
 // batch, so that what is dealt last is light (one group at a time, the last blocks ended 4 % after the median one).
+// Few groups (SPREAD, a build of its own: the other's code stays as it is): a tail item would outlast everything else (d = 64, G = 4: two units and as many sweep steps as a
+// unit has tiles, on one CTA), so every unit is an item, and the sweeps follow as items of their own, each over a slice of
+// the keys.  A sweep waits until the blocks with the group's window rows, wherever they run, have counted themselves
+// done: all of them were dealt out before the first sweep, and no unit waits for a sweep.
 // With per-chunk lengths the query tiles of a shorter chunk are numbered from the END: slot v of the static
 // decomposition (v = T - 1 is the last tile of a full-length chunk) is tile v - (T - T_c) of a chunk with T_c tiles.
 // The window then always sits in the last one or two slots, which the tail item owns together with the score sweep.
 struct Sched2 {
   int T, G, hpu, tpu, P, U, ntu, ipg, batch, hp, n_pass, wp;
 };
-template <int D>
+template <int D, bool SPREAD>
 __device__ __forceinline__ Sched2 make_sched2(const PrefillParams& p) {
   Sched2 s;
   s.T = (p.L + TILE - 1) / TILE;
@@ -65,7 +69,7 @@ __device__ __forceinline__ Sched2 make_sched2(const PrefillParams& p) {
   const int ntt = (p.chunk_len != nullptr) ? (p.w > 1 ? 2 : 1) : s.T - (p.L - p.w) / TILE;
   s.ntu = (ntt + s.tpu - 1) / s.tpu;
   if (s.ntu > s.U) s.ntu = s.U;
-  s.ipg = 1 + (s.U - s.ntu) * s.P;
+  s.ipg = SPREAD ? s.U * s.P : 1 + (s.U - s.ntu) * s.P;
   const long long kv_bytes = (long long)p.L * (4 * D);    // K and V of a group
   s.batch = (int)((48ll << 20) / kv_bytes);
   if (s.batch < 1) s.batch = 1;
@@ -90,10 +94,9 @@ __device__ __forceinline__ int chunk_length(const PrefillParams& p, int c) {
   len = len > p.L ? p.L : len;
   return len <= p.w ? p.w + 1 : len;
 }
-// blocks of sub-item `sub` (of the tail item, or 0)
+// blocks of unit x of a group, counted from the last tile of the chunk
 template <int D>
-__device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, int within, int sub, Desc& d) {
-  const int x = within == 0 ? sub : s.ntu * s.P + within - 1;
+__device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, int x, Desc& d) {
   const int unit = x / s.P, set = x - unit * s.P;
   const int hi = s.T - 1 - unit * s.tpu - (s.T - (d.len + TILE - 1) / TILE);      // upper tile of the unit
   const int h0 = hkv * s.G + set * s.hpu;
@@ -118,7 +121,7 @@ __device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, 
 // ====================================================================================
 // tensor maps (boxes of 64 d): tm_q (128 tokens), tm_kh (rotated keys, 64 tokens), tm_k (rotated keys, 128 tokens), tm_v
 // (128 tokens), tm_o (store, 128 tokens), tm_qw (wp tokens)
-template <int D>
+template <int D, bool SPREAD>
 __global__ void __launch_bounds__(NT2, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kh,
                const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -145,8 +148,9 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     if (warp == WARP_PRODUCER) {
       // ================================================================ TMA producer (both CTAs of a pair)
       if (elect_one()) {
-        const Sched2 sch = make_sched2<D>(prm);
-        const int n_groups = prm.C * prm.Hkv, n_items = n_groups * sch.ipg;
+        const Sched2 sch = make_sched2<D, SPREAD>(prm);
+        const int n_groups = prm.C * prm.Hkv, n_unit_items = n_groups * sch.ipg, slices = SPREAD ? prm.sweep_slices : 1;
+        const int n_items = n_unit_items + (SPREAD ? n_groups * slices : 0);
         const int rows_half = sch.hp * sch.wp;           // sweep operand rows per CTA and pass (B operand half)
         Prod p;
         // Once a wait has run out (abort flag) no new work is started: every role leaves its loops at the next
@@ -155,16 +159,20 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           const int item = next_item<C>(cx, p, leader, prm.counter, n_items);
           if (item >= n_items) break;
           int group, within;
-          decode_item(sch, n_groups, item, group, within);
+          const bool unit_item = !SPREAD || item < n_unit_items;
+          if (unit_item) decode_item(sch, n_groups, item, group, within);
+          else { within = (item - n_unit_items) / n_groups; group = item - n_unit_items - within * n_groups; }      // within: slice
           Desc d;
           d.c = group / prm.Hkv;
           d.hkv = group - d.c * prm.Hkv;
           d.len = chunk_length(prm, d.c);
           uint8_t* dst;
-          const int nsub = within == 0 ? sch.ntu * sch.P : 1;
+          const bool tail = !SPREAD && within == 0;
+          const int first = SPREAD ? within : (tail ? 0 : sch.ntu * sch.P + within - 1);
+          const int nsub = tail ? sch.ntu * sch.P : (unit_item ? 1 : 0);
           for (int sub = 0; sub < nsub; ++sub) {
             d.kind = KIND_FLASH;
-            decode_unit<D>(sch, rank, d.hkv, within, sub, d);
+            decode_unit<D>(sch, rank, d.hkv, first + sub, d);
             if (d.n[1] == 0) continue;                    // (n[0] <= n[1])
             publish<C>(cx, p, d);
             for (int b = 0; b < 2; ++b) {
@@ -188,12 +196,15 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               if (vbar) load_box<C>(dst, &tm_v, vbar, (int)rank * 64, d.hkv, j * TILE, d.c);
             }
           }
-          if (within == 0) {
+          if (tail || !unit_item) {
             // ---- score sweep: window queries of hp heads per CTA and pass, then this CTA's key tiles.  A head's rows
             // in the operand are the wp tokens that end with the chunk (wp = w rounded up to 8: the first wp - w rows
             // are not window rows and are left out of the sums; a start before token 0 reads zeros)
-            const int n_steps = ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
-            for (int u = 0; u < sch.n_pass; ++u) {
+            const int all_steps = ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
+            const int step0 = unit_item ? 0 : all_steps * within / slices;
+            const int n_steps = (unit_item ? all_steps : all_steps * (within + 1) / slices) - step0;
+            if (SPREAD) { d.t[0] = step0; d.t[1] = n_steps; }
+            for (int u = 0; u < sch.n_pass && (!SPREAD || n_steps > 0); ++u) {
               d.kind = KIND_SWEEP;
               d.h[0] = u;
               publish<C>(cx, p, d);
@@ -216,7 +227,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               for (int jj = 0; jj < n_steps; ++jj)
                 for (int a = 0; a < C::ATOMS; ++a) {
                   const uint32_t kbar = ring_stage<C>(cx, p, leader, &dst);
-                  if (kbar) load_box<C>(dst, &tm_k, kbar, a * 64, d.hkv, (NCTA * jj + (int)rank) * TILE, d.c);
+                  if (kbar) load_box<C>(dst, &tm_k, kbar, a * 64, d.hkv, (NCTA * (step0 + jj) + (int)rank) * TILE, d.c);
                 }
             }
           }
@@ -230,7 +241,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     } else if (warp == WARP_MMA && leader) {
       // ================================================================ issuer (of a pair: leader CTA)
       if (elect_one()) {
-        const Sched2 sch = make_sched2<D>(prm);
+        const Sched2 sch = make_sched2<D, SPREAD>(prm);
         const int rows_half = sch.hp * sch.wp;
         const uint32_t idesc_sw = make_idesc_bf16_f32(TILE * NCTA, PAIR ? 2 * rows_half : (rows_half + 15) & ~15, false, false);
         Issuer<C> is(cx);
@@ -289,7 +300,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           } else {
             // ---- score sweep, one pass: S^T = K_j Qw^T.  Its two [128 keys x 256 rows] buffers overlay all of TMEM:
             // every S / P buffer is consumed and the accumulators have been read out once o_free completes.
-            const int n_steps = ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
+            const int n_steps = SPREAD ? d.t[1] : ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
             for (int b = 0; b < 2; ++b) WAIT2S(&mi.o_free[b], free_par(is.no[b]), W2_OFREE);
             for (int b = 0; b < 3 - NCTA; ++b) is.qa[b] = is.wait_q();
             for (int jj = 0; jj < n_steps; ++jj, ++nt) {
@@ -321,7 +332,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     // ================================================================ epilogue: normalise, stage bf16 rows in the block's
     // (now idle) query slot, TMA store
     setmaxnreg_dec<REGS_EPI>();
-    const Sched2 sch = make_sched2<D>(prm);
+    const Sched2 sch = make_sched2<D, SPREAD>(prm);
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
     uint32_t nd = 0, nq = 0, no[2] = {0, 0};
@@ -333,6 +344,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           __threadfence();
           __syncwarp();
           if (lane == 0) {
+            if (SPREAD) {                                        // ... and that of the group's other blocks
+              const int tiles = (d.len + TILE - 1) / TILE - (d.len - prm.w) / TILE;
+              wait_count(prm.counter + 1 + d.c * prm.Hkv + d.hkv, tiles * sch.G, cx.abort_flag, cx.status, C::CODE + W2_LSE);
+            }
             mbar_arrive_cluster(in_cta<C>(&mi.lse_rdy, 0));
             if (PAIR) mbar_arrive_cluster(in_cta<C>(&mi.lse_rdy, 1));
           }
@@ -383,6 +398,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
         fence_proxy_async_smem();
         named_barrier_sync(1, 128);
+        if (SPREAD && r == 0 && (t + 1) * TILE > d.len - prm.w && t * TILE < d.len) {     // a block with window rows
+          __threadfence();
+          atomicAdd(prm.counter + 1 + d.c * prm.Hkv + d.hkv, 1);
+        }
         if (r == 0) {
           if (t >= 0 && t * TILE < prm.L) {
             for (int a = 0; a < C::ATOMS; ++a) tma_store_4d(&tm_o, myQ + a * 16384, a * 64, h, t * TILE, d.c);
@@ -397,7 +416,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   } else {
     // ================================================================ softmax
     setmaxnreg_inc<REGS_SOFTMAX>();
-    const Sched2 sch = make_sched2<D>(prm);
+    const Sched2 sch = make_sched2<D, SPREAD>(prm);
     const int b = warp >> 2;
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
@@ -449,7 +468,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           lse_cols[r] = x;
         }
         named_barrier_sync(3, 256);
-        const int n_steps = ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
+        const int n_steps = SPREAD ? d.t[1] : ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
         const int w0 = d.len - prm.w, pad = sch.wp - prm.w;      // first window token of this chunk
         float* const xch = &mi.lm[0][0][0];                      // [buffer][key]
         const uint32_t t_free0 = in_cta<C>(&mi.t_free[0], 0), t_free1 = in_cta<C>(&mi.t_free[1], 0);
@@ -457,7 +476,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           const int e = nt & 1;
           WAIT2S(&mi.t_full[e], full_par(nt >> 1), W2_TFULL);
           tc_fence_after_sync();
-          const int key0 = (NCTA * jj + (int)rank) * TILE, key = key0 + r;
+          const int key0 = (NCTA * ((SPREAD ? d.t[0] : 0) + jj) + (int)rank) * TILE, key = key0 + r;
           const uint32_t tT = cx.tmem + e * 256 + b * (PAIR ? rows_half : 128) + lane_sel;
           float part = 0.0f;
           int col = 0;
@@ -521,16 +540,42 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 // ====================================================================================
 //                                   host launcher
 // ====================================================================================
+// Slices of a group's score sweep as items of their own (SPREAD), or 0 for sweeps inside the tail items.  Where a tail item has more
+// steps (tiles of its units and of the sweep) than 1.2 times what a CTA or pair gets on average: us without / with, C x L,
+// heads, d: 1 x 2048, 32/8, 64 (3.1 times) 99 / 54; 1 x 8192, 16/4, 64 (1.7) 332 / 231; 2 x 1024, 8/2, 128 (5.5) 41.6 / 38.1;
+// 2 x 2048, 32/8, 128 (0.8) 100 / 105; 3 x 3000, 24/8, 128 (1.0) 215 / 223.  Not for two tiles, where the count in memory costs more
+// than it spreads (1 x 192, 32/8, 128 20.5 / 21.6; 4 x 256, 4/2, 64 18.4 / 19.1).
 template <int D>
-static cudaError_t launch_prefill_t(const CUtensorMap* maps, const PrefillParams& prm, int sm_count, cudaStream_t st) {
+static int sweep_slices(const PrefillParams& p, int units) {
+  constexpr int NCTA = PCfg<D>::NCTA, BLOCKS = 2 * NCTA;
+  const long long groups = (long long)p.C * p.Hkv;
+  const int T = (p.L + TILE - 1) / TILE;
+  if (groups > MAX_SPREAD_GROUPS || T < 6) return 0;
+  const int G = p.Hq / p.Hkv, hpu = G % BLOCKS == 0 ? BLOCKS : (G % 2 == 0 ? 2 : 1), tpu = BLOCKS / hpu;
+  const int P = G / hpu, U = (T + tpu - 1) / tpu, steps = (T + NCTA - 1) / NCTA;
+  const double all = (double)groups * (P * U * (T + tpu) / 2.0 + steps), tail = (double)P * T + steps;
+  if (tail < 1.2 * all / units) return 0;
+  int n = (int)(units / groups) < 8 ? (int)(units / groups) : 8;
+  n = n < steps ? n : steps;
+  return n < 1 ? 1 : n;
+}
+
+template <int D, bool SPREAD>
+static cudaError_t launch_build(const CUtensorMap* maps, const PrefillParams& prm, int grid, cudaStream_t st) {
   // the opt-in to large dynamic shared memory is a per-device attribute of the function: set it on every call
   // (a host-side call of a few hundred nanoseconds) rather than remember which devices have it
-  if (cudaError_t e = cudaFuncSetAttribute(prefill_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Off<PCfg<D>>::TOTAL); e != cudaSuccess) return e;
+  constexpr auto kernel = prefill_kernel<D, SPREAD>;
+  if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Off<PCfg<D>>::TOTAL); e != cudaSuccess) return e;
+  return launch_chained(kernel, dim3((unsigned)grid), dim3(NT2), Off<PCfg<D>>::TOTAL, st, PCfg<D>::NCTA, maps[0], maps[5], maps[1], maps[2],
+                        maps[3], maps[4], prm);
+}
+template <int D>
+static cudaError_t launch_prefill_t(const CUtensorMap* maps, PrefillParams prm, int sm_count, cudaStream_t st) {
   constexpr int NCTA = PCfg<D>::NCTA;
   const int grid = sm_count / NCTA * NCTA;               // one CTA per SM, a whole number of pairs
   if (grid < 1) return cudaErrorInvalidConfiguration;
-  return launch_chained(prefill_kernel<D>, dim3((unsigned)grid), dim3(NT2), Off<PCfg<D>>::TOTAL, st, NCTA, maps[0], maps[5], maps[1], maps[2],
-                        maps[3], maps[4], prm);
+  prm.sweep_slices = sweep_slices<D>(prm, grid / NCTA);
+  return prm.sweep_slices > 0 ? launch_build<D, true>(maps, prm, grid, st) : launch_build<D, false>(maps, prm, grid, st);
 }
 
 // maps: 0 q (box 64 x 128 tokens), 1 rotated keys (64 x 128), 2 v (64 x 128), 3 o (store), 4 q with a

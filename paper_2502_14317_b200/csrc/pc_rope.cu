@@ -3,6 +3,7 @@
 // before the attention kernel, by a bandwidth-bound pass: the result is the fp64 rotation
 // rounded once to bf16 (see pc_rope_exact.cuh for how fp32 arithmetic gets there), so rotated
 // keys - an output that the gather copies - are reproducible to the bit.
+#include "pc_attn.h"
 #include "pc_kernels.h"
 #include "pc_rope_exact.cuh"
 
@@ -26,7 +27,7 @@ __global__ void rope_table_kernel(double2* __restrict__ tab, float4* __restrict_
     for (int e = 0; e < 2; ++e) rope_angle(theta, half, pos0 + p, t + e, c[e], s[e]);
   }
   chain();                                                  // the arithmetic needs nothing from before; the tables may still be in use
-  if (i == 0 && counter != nullptr) *counter = 0;           // work queue of the attention kernel that follows
+  if (i < COUNTER_WORDS && counter != nullptr) counter[i] = 0;   // work queue of the attention kernel that follows
   if (i == 0 && clear != nullptr) *clear = 0;
   if (!mine) return;
   for (int e = 0; e < 2; ++e) tab[(size_t)p * half + t + e] = make_double2(c[e], s[e]);
@@ -90,9 +91,9 @@ __global__ void __launch_bounds__(256, 4) rope_rows_kernel(const __grid_constant
     __syncwarp();
   }
   chain();
-  if (OWN_TABLE && (blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) {
-    if (ang.counter != nullptr) *ang.counter = 0;
-    if (ang.clear != nullptr) *ang.clear = 0;
+  if (OWN_TABLE && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) {
+    if (ang.counter != nullptr && threadIdx.x < COUNTER_WORDS) ang.counter[threadIdx.x] = 0;
+    if (ang.clear != nullptr && threadIdx.x == 0) *ang.clear = 0;
   }
   const bool second_tensor = (int)blockIdx.y >= ta.ny;      // the same for the whole block
   const uint16_t* __restrict__ const x = second_tensor ? tb.x : ta.x;

@@ -216,6 +216,32 @@ def test_rope_position_reuse_equals_fp64_rotation_rounded_once(C, L, H, d, theta
     assert bad.shape[0] == 0, f"{bad.shape[0]} of {ref.size} rotated values differ from the fp64 rotation, first at {bad[0]}"
 
 
+@pytest.mark.parametrize("C,L,w,Hq,Hkv,d,chunk_len", [
+    (1, 700, 32, 8, 2, 64, None), (1, 1500, 100, 8, 2, 128, None), (2, 900, 64, 3, 1, 128, None), (1, 1100, 40, 6, 3, 64, None),
+    (3, 1000, 24, 4, 1, 128, [1000, 129, 41]), (2, 1030, 128, 5, 1, 64, [200, 1030]),
+])
+def test_score_sweeps_as_items_of_their_own(C, L, w, Hq, Hkv, d, chunk_len):
+    """Few (chunk, kv-head) groups: units and slices of the score sweep are dealt out one by one and a sweep waits for the group's
+    window rows; windows over one and two tiles, short chunks with fewer steps than slices."""
+    import paper_2502_14317_b200 as pc
+    theta = 10000.0
+    rng = np.random.default_rng(L + w)
+    q, k, v = (pc_inputs.f32_to_bf16_bits(rng.standard_normal((C, L, h, d)).astype(np.float32)) for h in (Hq, Hkv, Hkv))
+    if chunk_len is None:
+        _run_and_compare(q, k, v, w, theta)
+        return
+    cl = torch.tensor(chunk_len, dtype=torch.int32, device="cuda")
+    res = pc.chunk_prefill_attn(to_dev(q), to_dev(k), to_dev(v), w=w, rope_theta=theta, want_lse=True, chunk_len=cl)
+    torch.cuda.synchronize()
+    assert int(res["status"].item()) == 0
+    for c, n in enumerate(chunk_len):
+        O, LSE, k_rot = orc.local_attention(q[c:c + 1, :n], k[c:c + 1, :n], v[c:c + 1, :n], theta)
+        S, _, _ = orc.window_scores(orc.rope_bf16(q[c:c + 1, :n], theta), k_rot, v[c:c + 1, :n], w, 1.0 / np.sqrt(d))
+        check_attention_output(to_f64(res["o"][c:c + 1, :n]), O)
+        check_scores(res["win_score"][c:c + 1, :, :n].cpu().numpy(), S, Hq // Hkv, w, n)
+        assert not res["o"][c, n:].any() and not res["win_score"][c, :, n:].any()
+
+
 @pytest.mark.parametrize("C,L,H,d", [(1, 1, 1, 64), (1, 1, 1, 128), (5, 9, 3, 64), (2, 512, 8, 128), (1, 1025, 8, 128), (1, 2049, 8, 64), (3, 700, 37, 128)])
 def test_rope_with_and_without_a_table_kernel(C, L, H, d):
     """Up to 2^20 values the warps of the rotation pass compute their own table rows, above that a kernel of its own does: the
