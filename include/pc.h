@@ -121,7 +121,8 @@ PC_API int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q,
  *   skip_final_publication non-zero: the single-CTA chunk-prefill kernel (head size 64)
  *                          leaves out ONE signal that carries no data - the "no more work" message to its consumer warps after the
  *                          last work item, when nothing is in flight any more - so that their
- *                          wait runs out.  Outputs of such a call are complete; its status_word
+ *                          wait runs out.  Outputs of such a call are complete (not the scores of a call whose
+ *                          sweeps are items of their own: they wait for blocks that end with that signal); its status_word
  *                          is non-zero.  Zero switches the hook off again.
  * Host-side settings, read at every launch.
  */
