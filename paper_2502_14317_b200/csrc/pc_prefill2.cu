@@ -340,14 +340,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const Desc d = next_desc<C>(cx, nd, true);
       if (d.kind == KIND_DONE) break;
       if (d.kind == KIND_SWEEP) {
-        if (d.h[0] == 0) {                                       // the window rows' log-sum-exp of this CTA's blocks is in memory
+        if (!SPREAD && d.h[0] == 0) {                            // the window rows' log-sum-exp of this CTA's blocks is in memory
           __threadfence();
           __syncwarp();
           if (lane == 0) {
-            if (SPREAD) {                                        // ... and that of the group's other blocks
-              const int tiles = (d.len + TILE - 1) / TILE - (d.len - prm.w) / TILE;
-              wait_count(prm.counter + 1 + d.c * prm.Hkv + d.hkv, tiles * sch.G, cx.abort_flag, cx.status, C::CODE + W2_LSE);
-            }
             mbar_arrive_cluster(in_cta<C>(&mi.lse_rdy, 0));
             if (PAIR) mbar_arrive_cluster(in_cta<C>(&mi.lse_rdy, 1));
           }
@@ -450,7 +446,23 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       } else {
         // ---- score sweep: this thread owns a key; its warpgroup sums the columns of the heads that CTA b loaded
         const int u = d.h[0];
-        if (u == 0) { mbar_wait_cluster(&mi.lse_rdy, full_par(n_lse), cx.abort_flag, cx.status, W2_LSE); ++n_lse; }
+        if (u == 0) {
+          if constexpr (SPREAD) {
+            // Sweeps follow one another here without a block between them, so the epilogue warps, which would be several sweeps
+            // ahead, cannot hand this over through a barrier's parity.  The log-sum-exp of all the group's window rows is in
+            // memory once its blocks have counted themselves done, and the epilogue has read this CTA's last
+            // statistics (lm, reused below) once each warpgroup has seen its own lm_free.
+            WAIT2S(&mi.lm_free[b], free_par(n_blk), W2_LMFREE);
+            if (lane == 0) {
+              const int tiles = (d.len + TILE - 1) / TILE - (d.len - prm.w) / TILE;
+              wait_count(prm.counter + 1 + d.c * prm.Hkv + d.hkv, tiles * sch.G, cx.abort_flag, cx.status, C::CODE + W2_LSE);
+            }
+            named_barrier_sync(3, 256);
+          } else {
+            mbar_wait_cluster(&mi.lse_rdy, full_par(n_lse), cx.abort_flag, cx.status, W2_LSE);
+            ++n_lse;
+          }
+        }
         const int rows_half = sch.hp * sch.wp;
         const int g0 = u * 2 * sch.hp + b * sch.hp;
         const int heads = sch.G - g0 < sch.hp ? (sch.G > g0 ? sch.G - g0 : 0) : sch.hp;

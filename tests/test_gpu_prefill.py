@@ -242,6 +242,17 @@ def test_score_sweeps_as_items_of_their_own(C, L, w, Hq, Hkv, d, chunk_len):
         assert not res["o"][c, n:].any() and not res["win_score"][c, :, n:].any()
 
 
+@pytest.mark.parametrize("C,L,w,Hq,Hkv,d,chunk_len", [
+    (1, 2048, 128, 24, 8, 128, None),                         # 64 sweeps of one step and two passes each
+    (4, 1500, 50, 5, 1, 128, [1500, 100, 900, 1300]),         # sweeps of one step or none
+    (4, 1536, 50, 8, 8, 64, [1536, 100, 900, 1300]), (1, 2304, 8, 16, 8, 64, None), (1, 900, 16, 62, 62, 64, None),
+])
+def test_several_short_score_sweeps_on_one_cta(C, L, w, Hq, Hkv, d, chunk_len):
+    """Sweeps of a few steps: the CTA that is through its units first takes several of them, whose descriptors its warps reach
+    well apart; a warp that could be a whole sweep ahead of another must not signal it through a barrier's parity."""
+    test_score_sweeps_as_items_of_their_own(C, L, w, Hq, Hkv, d, chunk_len)
+
+
 @pytest.mark.parametrize("C,L,H,d", [(1, 1, 1, 64), (1, 1, 1, 128), (5, 9, 3, 64), (2, 512, 8, 128), (1, 1025, 8, 128), (1, 2049, 8, 64), (3, 700, 37, 128)])
 def test_rope_with_and_without_a_table_kernel(C, L, H, d):
     """Up to 2^20 values the warps of the rotation pass compute their own table rows, above that a kernel of its own does: the
