@@ -201,6 +201,7 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     setmaxnreg_dec<REGS_EPI>();
     const int r = tid & 127, wi = r % w;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    const bool sectors = (reinterpret_cast<uintptr_t>(prm.part_o) & 31) == 0;  // a workspace is aligned to 16 bytes only
     uint32_t nd = 0, nq = 0, no[2] = {0, 0};
     while (true) {
       const Desc d = next_desc<C>(cx, nd, true);
@@ -268,7 +269,10 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                                           pack_bf16x2(x[i * 8 + 4], x[i * 8 + 5]), pack_bf16x2(x[i * 8 + 6], x[i * 8 + 7]));
           } else if (valid) {
 #pragma unroll
-            for (int i = 0; i < 2; ++i) st_global_f32x8(out + q * 4 + i * 2, &x[i * 8]);
+            for (int i = 0; i < 4; ++i)
+              if (!sectors) out[q * 4 + i] = make_uint4(__float_as_uint(x[i * 4]), __float_as_uint(x[i * 4 + 1]), __float_as_uint(x[i * 4 + 2]),
+                                                        __float_as_uint(x[i * 4 + 3]));
+              else if (i % 2 == 0) st_global_f32x8(out + q * 4 + i, &x[i * 4]);
           }
         }
         warp_arrive_leader(in_cta<C>(&mi.o_free[alt ? 0 : b0], 0));

@@ -147,7 +147,7 @@ __device__ __forceinline__ void tma_store_wait_read() {   // smem source may be 
 __device__ __forceinline__ void tma_store_wait_all() {    // writes complete
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
-// one 32-byte store (a whole sector: rows that threads write each on their own)
+// one 32-byte store (a whole sector: rows that threads write each on their own); p aligned to 32 bytes
 __device__ __forceinline__ void st_global_f32x8(void* p, const float* x) {
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                :: "l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7]) : "memory");

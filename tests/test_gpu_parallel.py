@@ -51,6 +51,26 @@ def test_parallel_attn_shapes(B, w, Hq, Hkv, d, Nk, q_pos0, theta):
     assert np.abs(res["lse"].cpu().numpy() - LSE).max() <= 2e-3
 
 
+@pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 128), (4, 2, 128), (4, 2, 64)])
+@pytest.mark.parametrize("shift", [16, 32, 48])
+def test_workspace_at_any_multiple_of_16_bytes(Hq, Hkv, d, shift):
+    """Keys split, so that partial results go through the workspace: its address needs 16 bytes of alignment, no more (pairs,
+    single CTAs, head size 64)."""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(shift + d)
+    B, w, Nk = 1, 64, 2500
+    t = [to_dev(_bits(rng, s)) for s in ((B, w, Hq, d), (B, Hkv, Nk, d), (B, Hkv, Nk, d), (B, w, Hkv, d), (B, w, Hkv, d))]
+    need = pc.parallel_attn_workspace_bytes(B, w, Hq, Hkv, d, Nk)
+    assert need > B * Hq * w * d * 4                                          # room for partial results: the keys are split
+    room = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+    at = -room.data_ptr() % 64 + shift
+    want = pc.parallel_attn(*t, q_pos0=100, rope_theta=1e4, want_lse=True)
+    got = pc.parallel_attn(*t, q_pos0=100, rope_theta=1e4, want_lse=True, workspace=room[at:at + need])
+    torch.cuda.synchronize()
+    assert int(got["status"].item()) == 0
+    assert torch.equal(got["out"], want["out"]) and torch.equal(got["lse"], want["lse"])
+
+
 @pytest.mark.parametrize("B,w,Hq,Hkv,d,Nk,grow", [
     (1, 1, 1, 1, 128, 1, 0), (1, 1, 3, 1, 64, 127, 0), (2, 1, 2, 2, 128, 129, 0),    # one and two tiles: fewer than key splits
     (1, 2, 8, 1, 128, 2050, 0), (1, 1, 17, 1, 128, 700, 0), (2, 4, 8, 1, 64, 640, 0),   # 16, 17 and 32 rows per kv-head
