@@ -42,6 +42,12 @@ const DeviceInfo& device_info() {
   return info[dev];
 }
 
+// Result of a call's launches.  A failure is reported by the call that made it and not left pending for a later one.
+int32_t launched(cudaError_t e) {
+  const cudaError_t pending = cudaGetLastError();
+  return e == cudaSuccess && pending == cudaSuccess ? PC_OK : PC_ERR_CUDA;
+}
+
 bool pow2_between(int x, int lo, int hi) { return x >= lo && x <= hi && (x & (x - 1)) == 0; }
 
 void fill_strides(const int64_t in[3], int64_t out[3], int64_t tokens, int64_t heads, int64_t d) {
@@ -170,8 +176,9 @@ int32_t prefill_attn_impl(const pc_prefill_desc* desc, const void* q, const void
   // queries and keys are rotated once, ahead of the attention kernel (positions 0 .. L-1 in every chunk)
   const long long os_ll[3] = {os[0], os[1], os[2]};
   const pc::RopeRows rk = {k, {ks[0], ks[1], ks[2]}, krot, desc->Hkv}, rq = {q, {qs[0], qs[1], qs[2]}, qrot, desc->Hq};
-  pc::launch_rope(rk, &rq, {table, table_hi, table_lo}, desc->C, desc->L, d, (double)desc->rope_theta, 0, counter,
-                  clear_status ? status_word : nullptr, st);
+  if (cudaError_t e = pc::launch_rope(rk, &rq, {table, table_hi, table_lo}, desc->C, desc->L, d, (double)desc->rope_theta, 0, counter,
+                                      clear_status ? status_word : nullptr, st);
+      e != cudaSuccess) return launched(e);
 
   if (chunk_len != nullptr)   // rows and scores behind the end of a shorter chunk read as zero: the kernels below skip them
     pc::launch_zero_chunk_tails(chunk_len, desc->C, desc->L, desc->w, desc->Hq, desc->Hkv, d, o, os_ll, lse, win_score, st);
@@ -185,9 +192,7 @@ int32_t prefill_attn_impl(const pc_prefill_desc* desc, const void* q, const void
   prm.status = status_word; prm.counter = counter;
   prm.wait_kcycles = pc::g_wait_kcycles.load();
   prm.skip_final_publication = pc::g_skip_final_publication.load();
-  const cudaError_t le = pc::launch_prefill_attn(maps, prm, d, dev.sm_count, st);
-  if (le != cudaSuccess) return PC_ERR_CUDA;
-  return cudaGetLastError() == cudaSuccess ? PC_OK : PC_ERR_CUDA;
+  return launched(pc::launch_prefill_attn(maps, prm, d, dev.sm_count, st));
 }
 
 }  // namespace
@@ -222,8 +227,7 @@ int32_t pc_rope_position_reuse(const void* x, int32_t C, int32_t L, int32_t H, i
   float4* table_hi = reinterpret_cast<float4*>(ws + align_up((size_t)L * (d / 2) * sizeof(double2)));
   float4* table_lo = table_hi + (size_t)L * (d / 4);
   const pc::RopeRows rows = {x, {(long long)L * H * d, (long long)H * d, d}, y, H};
-  pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, C, L, d, (double)rope_theta, 0, nullptr, nullptr, st);
-  return cudaGetLastError() == cudaSuccess ? PC_OK : PC_ERR_CUDA;
+  return launched(pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, C, L, d, (double)rope_theta, 0, nullptr, nullptr, st));
 }
 
 // ------------------------------------------------------------------------------------ chunk score stand-in
@@ -568,7 +572,7 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
     dp.lse_out = lse_out;
     dp.status = status_word;
     dp.wait_kcycles = pc::g_wait_kcycles.load();
-    return pc::launch_decode_attn(dm, dp, d, st) == cudaSuccess ? PC_OK : PC_ERR_CUDA;
+    return launched(pc::launch_decode_attn(dm, dp, d, st));
   }
 
   // rotated queries first (the same pass that serves the chunk-local kernels)
@@ -576,7 +580,8 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   float4* table_lo = reinterpret_cast<float4*>(ws + plan.off_table_lo);
   void* q_rot = ws + plan.off_qrot;
   const pc::RopeRows rows = {q_win, {(long long)w * Hq * d, (long long)Hq * d, (long long)d}, q_rot, Hq};
-  pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, B, w, d, (double)rope_theta, q_pos0, counter, nullptr, st);
+  if (cudaError_t e = pc::launch_rope(rows, nullptr, {table, table_hi, table_lo}, B, w, d, (double)rope_theta, q_pos0, counter, nullptr, st);
+      e != cudaSuccess) return launched(e);
 
   CUtensorMap maps[5];
   const uint32_t box_kch[4] = {64, plan.pair ? 64u : 128u, 1, 1};
@@ -600,13 +605,12 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   prm.status = status_word;
   prm.counter = counter;
   prm.wait_kcycles = pc::g_wait_kcycles.load();
-  if (pc::launch_parallel_attn(maps, prm, d, plan.pair, dev.sm_count, st) != cudaSuccess) return PC_ERR_CUDA;
+  cudaError_t e = pc::launch_parallel_attn(maps, prm, d, plan.pair, dev.sm_count, st);
   // the attention reads entries below Nk only (rows behind them read as zeros and are masked): the new rows can follow
   // on the same stream
-  if (append && pc::launch_append_kv(k_win, v_win, B, w, Hkv, d, Nk, Nk_cap, const_cast<void*>(k_cache), const_cast<void*>(v_cache),
-                                     st) != cudaSuccess)
-    return PC_ERR_CUDA;
-  return PC_OK;
+  if (append && e == cudaSuccess)
+    e = pc::launch_append_kv(k_win, v_win, B, w, Hkv, d, Nk, Nk_cap, const_cast<void*>(k_cache), const_cast<void*>(v_cache), st);
+  return launched(e);
 }
 
 }  // namespace

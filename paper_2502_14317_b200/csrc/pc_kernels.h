@@ -54,8 +54,8 @@ struct RopeRows {
 };
 // one tensor, or two (b not null) in the same launch; positions pos0 .. pos0 + L - 1; the COUNTER_WORDS
 // of counter (pc_attn.h) and clear (each may be null) are set to 0
-void launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int C, int L, int d, double theta, int pos0,
-                 int* counter, int* clear, cudaStream_t st);
+cudaError_t launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int C, int L, int d, double theta, int pos0,
+                        int* counter, int* clear, cudaStream_t st);
 
 // Per-chunk lengths: zero o[c, p, :, :], lse[c, :, p] and win_score[c, :, p] for p >= clamp(chunk_len[c], w + 1, L).
 void launch_zero_chunk_tails(const int* chunk_len, int C, int L, int w, int Hq, int Hkv, int d, void* o,

@@ -206,8 +206,8 @@ static RopeTensor rope_tensor(const RopeRows& r, int C, int L, int d) {
   return t;
 }
 
-void launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int C, int L, int d, double theta, int pos0,
-                 int* counter, int* clear, cudaStream_t st) {
+cudaError_t launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int C, int L, int d, double theta, int pos0,
+                        int* counter, int* clear, cudaStream_t st) {
   const RopeTensor ta = rope_tensor(a, C, L, d);
   RopeTensor tb = {};
   if (b != nullptr) tb = rope_tensor(*b, C, L, d);
@@ -219,13 +219,12 @@ void launch_rope(const RopeRows& a, const RopeRows* b, const RopeTable& tab, int
   // chunks and fewer free registers cost more than the launch (8x64x32x128 5.7 / 6.8, 64x64x32x128 14.7 / 18.1, 4x8192x32x128
   // 97 / 129).
   const long long values = (long long)C * L * d * (a.H + (b != nullptr ? b->H : 0));
-  if (values <= (1 << 20)) {
-    launch_chained(rope_rows_kernel<true>, grid, dim3(256), 0, st, 1, ta, tb, tab.hi, tab.lo, tab.exact, C, L, d, ang);
-    return;
-  }
-  launch_chained(rope_table_kernel, dim3((unsigned)((L * (d / 4) + 255) / 256)), dim3(256), 0, st, 1, tab.exact, tab.hi, tab.lo, L, d / 2,
-                 theta, pos0, counter, clear);
-  launch_chained(rope_rows_kernel<false>, grid, dim3(256), 0, st, 1, ta, tb, tab.hi, tab.lo, tab.exact, C, L, d, ang);
+  if (values <= (1 << 20))
+    return launch_chained(rope_rows_kernel<true>, grid, dim3(256), 0, st, 1, ta, tb, tab.hi, tab.lo, tab.exact, C, L, d, ang);
+  if (cudaError_t e = launch_chained(rope_table_kernel, dim3((unsigned)((L * (d / 4) + 255) / 256)), dim3(256), 0, st, 1, tab.exact, tab.hi,
+                                     tab.lo, L, d / 2, theta, pos0, counter, clear);
+      e != cudaSuccess) return e;
+  return launch_chained(rope_rows_kernel<false>, grid, dim3(256), 0, st, 1, ta, tb, tab.hi, tab.lo, tab.exact, C, L, d, ang);
 }
 
 // Rows behind the end of a chunk that is shorter than L (per-chunk lengths): outputs read as zero there.

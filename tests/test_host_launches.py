@@ -1,0 +1,59 @@
+"""CPU checks of what the C ABI does around its launches: its host code and the rotation's linked with a fake CUDA runtime
+(fake_runtime.cpp), in which a chosen launch fails."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_2502_14317_b200 import binding, build
+    csrc, out = build.CSRC, str(tmp_path_factory.mktemp("fake") / "libpc_fake.so")
+    subprocess.run([build._nvcc(), "-shared", "-cudart", "none", "-gencode", "arch=compute_100a,code=sm_100a", "-O1", "-std=c++17",
+                    "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", "-I", csrc, "-Xlinker", "-Bsymbolic", "-Xlinker", "--no-undefined",
+                    os.path.join(ROOT, "tests", "fake_runtime.cpp"), "-o", out] +
+                   [os.path.join(csrc, f) for f in ("pc_api.cu", "pc_rope.cu", "pc_static_scratch.cu")],
+                   check=True, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)
+    with pytest.MonkeyPatch.context() as mp:
+        mp.setattr(binding, "_LIB", None)
+        mp.setattr(binding, "lib_path", lambda: out)
+        return binding.load_library()
+
+
+P = 1 << 20                                                       # a device address that nothing follows
+
+
+def _desc(C=2, L=300, w=16, Hq=4, Hkv=2, d=128, v_stride=(0, 0, 0)):
+    from paper_2502_14317_b200.binding import _PrefillDesc
+    return _PrefillDesc(C, L, w, Hq, Hkv, d, 1e4, 0.0, (0, 0, 0), (0, 0, 0), v_stride, (0, 0, 0))
+
+
+def _calls(lib):
+    """name, call, launches of the rotation ahead of the attention"""
+    big = 1 << 40
+    desc = lambda **kw: ctypes.byref(_desc(**kw))
+    prefill = lambda **kw: lib.pc_chunk_prefill_attn(desc(**kw), P, P, P, None, P, P, None, P, P, None, P, big, None)
+    parallel = lambda B, w: lib.pc_parallel_attn(B, w, 8, 2, 128, 3000, P, 0, 1e4, 0.0, P, P, P, P, P, None, None, P, big, None)
+    return [("rope, own tables", lambda: lib.pc_rope_position_reuse(P, 1, 100, 4, 64, 1e4, P, P, big, None), 1),
+            ("rope, table kernel", lambda: lib.pc_rope_position_reuse(P, 4, 4096, 8, 128, 1e4, P, P, big, None), 2),
+            ("prefill, own tables", lambda: prefill(), 1), ("prefill, table kernel", lambda: prefill(C=8, L=2000), 2),
+            ("window", lambda: parallel(1, 64), 1), ("window, table kernel", lambda: parallel(64, 64), 2), ("few rows", lambda: parallel(1, 1), 0)]
+
+
+@pytest.mark.parametrize("which", range(7))
+def test_a_failed_launch_is_reported_by_the_call_that_made_it(fake, which):
+    name, call, rotation = _calls(fake)[which]
+    fake.fake_reset(-1)
+    assert call() == 0
+    n_attention = fake.fake_attention_launches()
+    for at in range(rotation + n_attention):
+        fake.fake_reset(at)
+        assert call() == -4, f"{name}: launch {at} failed"
+        if at < rotation:
+            assert fake.fake_attention_launches() == 0, f"{name}: the attention ran on what a failed rotation left"
+        assert fake.fake_last_error() == 0, f"{name}: the error is left to a later call"
+        assert call() == 0
