@@ -331,7 +331,7 @@ typedef struct {
   const void *q, *k, *v, *q_win;
   void *o, *k_rot;
   float *win_score, *win_lse;
-  const float* given_score;            /* [n_score] or NULL */
+  const float* given_score;            /* [n_score] or NULL; more scores than chunks are refused */
   float* chunk_score;                  /* [C], unused with given_score */
   int32_t *kept, *idx;
   void *kc, *vc;

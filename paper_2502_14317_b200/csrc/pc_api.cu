@@ -645,6 +645,8 @@ size_t pc_hot_path_workspace_bytes(const pc_prefill_desc* desc, int32_t m, int32
 int32_t pc_hot_path(const pc_prefill_desc* desc, const pc_hot_path_args* a, int32_t* failed, void* stream) {
   int32_t stage = PC_STAGE_PREFILL, rc = PC_ERR_INVALID_ARG;
   if (desc != nullptr && a != nullptr) do {
+    // more scores than chunks: chunks that do not exist could be kept, and their rows be read
+    if (a->given_score != nullptr && a->n_score > desc->C) { stage = PC_STAGE_SELECT_CHUNKS; break; }
     rc = prefill_attn_impl(desc, a->q, a->k, a->v, nullptr, a->o, a->k_rot, nullptr, a->win_score, a->win_lse, a->status_word,
                            a->ws_prefill, a->ws_prefill_bytes, stream, a->clear_status != 0);
     if (rc != PC_OK) break;

@@ -57,3 +57,21 @@ def test_a_failed_launch_is_reported_by_the_call_that_made_it(fake, which):
             assert fake.fake_attention_launches() == 0, f"{name}: the attention ran on what a failed rotation left"
         assert fake.fake_last_error() == 0, f"{name}: the error is left to a later call"
         assert call() == 0
+
+
+def _hot_path(lib, desc, n_score=None):
+    from paper_2502_14317_b200.binding import _HotPathArgs
+    a = _HotPathArgs(**{n: P for n, t in _HotPathArgs._fields_ if t is ctypes.c_void_p}, ws_prefill_bytes=1 << 40, ws_parallel_bytes=1 << 40,
+                     m=1, k_keep=64, n_score=n_score or 0, clear_status=0)
+    if n_score is None:
+        a.given_score = None
+    failed = ctypes.c_int32(-1)
+    lib.fake_reset(-1)
+    return lib.pc_hot_path(ctypes.byref(desc), ctypes.byref(a), ctypes.byref(failed), None), failed.value, lib.fake_attention_launches()
+
+
+def test_whole_path_refuses_scores_of_chunks_that_do_not_exist(fake):
+    """Before anything is launched; fewer scores than chunks rank the first chunks, as pc_select_chunks does."""
+    assert _hot_path(fake, _desc(C=3), n_score=4) == (-1, 2, 0)
+    for n in (1, 3, None):
+        assert _hot_path(fake, _desc(C=3), n_score=n) == (0, 0, 2)
