@@ -320,7 +320,7 @@ PC_API int32_t pc_parallel_attn_append(int32_t B, int32_t w, int32_t Hq, int32_t
  * better), pc_select_tokens on the L - w context tokens, pc_gather_kv and pc_parallel_attn
  * (B = 1, q_pos0 = L - w) of chunk 0's window over the m * k_keep kept entries.  Same kernels,
  * same results; what it saves is the host time between them, which bounds a short prompt.
- * Shapes as in those calls; v and k_rot contiguous, q_win [w,Hq,d] contiguous (the window rows
+ * Shapes as in those calls; v and k_rot contiguous (PC_ERR_INVALID_ARG for other strides of v), q_win [w,Hq,d] contiguous (the window rows
  * of chunk 0: for a contiguous q, q + (L-w)*Hq*d).  With clear_status the status word, which
  * both attention calls share, is set to 0 first.  Returns the first failing call's code and
  * names that call in *failed (may be NULL; 0: none).

@@ -645,6 +645,13 @@ size_t pc_hot_path_workspace_bytes(const pc_prefill_desc* desc, int32_t m, int32
 int32_t pc_hot_path(const pc_prefill_desc* desc, const pc_hot_path_args* a, int32_t* failed, void* stream) {
   int32_t stage = PC_STAGE_PREFILL, rc = PC_ERR_INVALID_ARG;
   if (desc != nullptr && a != nullptr) do {
+    // the gather and the window's own values take v as it would be contiguous (the stride of a dimension of one entry does not matter)
+    const int64_t packed[3] = {(int64_t)desc->L * desc->Hkv * desc->d, (int64_t)desc->Hkv * desc->d, desc->d}, n[3] = {desc->C, desc->L, desc->Hkv};
+    int64_t vs[3];
+    fill_strides(desc->v_stride, vs, desc->L, desc->Hkv, desc->d);
+    bool contiguous = true;
+    for (int i = 0; i < 3; ++i) contiguous = contiguous && (vs[i] == packed[i] || n[i] == 1);
+    if (!contiguous) break;
     // more scores than chunks: chunks that do not exist could be kept, and their rows be read
     if (a->given_score != nullptr && a->n_score > desc->C) { stage = PC_STAGE_SELECT_CHUNKS; break; }
     rc = prefill_attn_impl(desc, a->q, a->k, a->v, nullptr, a->o, a->k_rot, nullptr, a->win_score, a->win_lse, a->status_word,

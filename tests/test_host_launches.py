@@ -75,3 +75,11 @@ def test_whole_path_refuses_scores_of_chunks_that_do_not_exist(fake):
     assert _hot_path(fake, _desc(C=3), n_score=4) == (-1, 2, 0)
     for n in (1, 3, None):
         assert _hot_path(fake, _desc(C=3), n_score=n) == (0, 0, 2)
+
+
+def test_whole_path_refuses_values_that_are_not_contiguous(fake):
+    """The prefill takes strides of v, the stages behind it do not."""
+    for v_stride in ((2 * 300 * 256, 256, 128), (300 * 256, 128, 300 * 128), (300 * 512, 512, 128)):
+        assert _hot_path(fake, _desc(v_stride=v_stride)) == (-1, 1, 0), v_stride
+    for C, Hkv, v_stride in ((2, 2, (0, 0, 0)), (2, 2, (300 * 256, 256, 128)), (1, 2, (900 * 256, 256, 128)), (2, 1, (300 * 128, 128, 38400))):
+        assert _hot_path(fake, _desc(C=C, Hkv=Hkv, v_stride=v_stride)) == (0, 0, 2), v_stride
