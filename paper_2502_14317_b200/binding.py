@@ -140,10 +140,17 @@ def _stream():
 
 
 def _like(t, shape):
-    """New contiguous bf16 tensor on t's device (empty_like is the cheapest way to get one)."""
+    """New contiguous bf16 tensor on t's device (empty_like is the cheapest way to get one).  Its strides are those of its
+    shape: t may count as contiguous with any stride in a dimension of one entry."""
     if t.dtype is torch.bfloat16 and t.shape == shape and t.is_contiguous():
-        return torch.empty_like(t)
+        return torch.empty_like(t, memory_format=torch.contiguous_format)
     return t.new_empty(shape, dtype=torch.bfloat16)
+
+
+def _same_rows(a, b):
+    """Whether the strides of a serve b too: equal wherever a dimension has more than one entry, the innermost contiguous."""
+    sa, sb = a.stride(), b.stride()
+    return sa[3] == 1 and (sa == sb or (sb[3] == 1 and all(x == y or n == 1 for x, y, n in zip(sa, sb, a.shape))))
 
 
 def _window(t, L, w):
@@ -295,7 +302,7 @@ def gather_kv(k_src, v_src, kept, idx, k_out=None, v_out=None, pos_out=None, wan
     C, L, Hkv, d = k_src.shape
     m, _, k = idx.shape
     dev = k_src.device
-    if k_src.stride() != v_src.stride() or k_src.stride(3) != 1:
+    if not _same_rows(k_src, v_src):
         raise PcError("k_src and v_src must share strides with a contiguous head dimension")
     k_out = _like(k_src, (Hkv, m * k, d)) if k_out is None else k_out
     v_out = _like(k_out, (Hkv, m * k, d)) if v_out is None else v_out
@@ -346,7 +353,7 @@ def queue_gather(state, k_src, v_src, idx):
     Cb, L, Hkv, d = k_src.shape
     if idx.shape != (Cb, Hkv, state["k"]) or Hkv != state["Hkv"] or d != state["d"]:
         raise PcError("idx must be [Cb, Hkv, k] for the queue's k; Hkv and d must match the queue")
-    if k_src.stride() != v_src.stride() or k_src.stride(3) != 1:
+    if not _same_rows(k_src, v_src):
         raise PcError("k_src and v_src must share strides with a contiguous head dimension")
     strides = (c_int64 * 3)(k_src.stride(0), k_src.stride(1), k_src.stride(2))
     _check(lib.pc_queue_gather(_ptr(k_src), _ptr(v_src), strides, _ptr(state["slot_src"]), _ptr(idx), state["m"], Hkv,
@@ -362,7 +369,7 @@ def queue_select_gather(state, win_score, k_src, v_src, n_cand):
     Cb, L, Hkv, d = k_src.shape
     if Hkv != state["Hkv"] or d != state["d"] or win_score.shape != (Cb, Hkv, L) or not win_score.is_contiguous():
         raise PcError("win_score must be contiguous [Cb, Hkv, L]; Hkv and d must match the queue")
-    if k_src.stride() != v_src.stride() or k_src.stride(3) != 1:
+    if not _same_rows(k_src, v_src):
         raise PcError("k_src and v_src must share strides with a contiguous head dimension")
     strides = (c_int64 * 3)(k_src.stride(0), k_src.stride(1), k_src.stride(2))
     _check(lib.pc_queue_select_gather(_ptr(win_score), _ptr(k_src), _ptr(v_src), strides, _ptr(state["slot_src"]), state["m"],
@@ -528,7 +535,7 @@ def hot_path(q, k, v, *, w, rope_theta, m, k_keep, softmax_scale=0.0, chunk_scor
         ws_prefill = torch.empty(max(need, need_par, 16), dtype=torch.uint8, device=dev)
     if ws_par is None or ws_par.numel() < need_par:            # (the prefill is done with its own by then)
         ws_par = ws_prefill if ws_prefill.numel() >= need_par else torch.empty(max(need_par, 16), dtype=torch.uint8, device=dev)
-    if k_rot.stride() != v.stride():
+    if not (k_rot.is_contiguous() and v.is_contiguous()):
         raise PcError("k_src and v_src must share strides with a contiguous head dimension")
     # the window is the same in every chunk: take it from chunk 0
     q_win = None if q.is_contiguous() else _window(q, L, w)

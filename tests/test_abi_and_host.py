@@ -93,6 +93,16 @@ def test_host_side_argument_errors_need_no_gpu(lib):
     assert lib.pc_queue_emit(o, 2, 2, 64, 128, p, p, o, o, None, p, p, None, None) == -1    # no slot_order array
 
 
+def test_new_tensors_have_the_strides_of_their_shape():
+    import torch
+    from paper_2502_14317_b200.binding import _like, _same_rows
+    t = torch.zeros((2, 1, 5, 8), dtype=torch.bfloat16).transpose(1, 2)         # contiguous, the stride of the one head is 40
+    new = _like(t, t.shape)
+    assert t.is_contiguous() and new.stride() == (40, 8, 8, 1)
+    assert _same_rows(t, new) and _same_rows(new, t)
+    assert not _same_rows(new, torch.zeros((2, 10, 1, 8))[:, ::2]) and not _same_rows(new, torch.zeros((2, 5, 1, 16))[..., ::2])
+
+
 def test_binding_fails_loudly_without_library(tmp_path, monkeypatch):
     from paper_2502_14317_b200 import binding
     monkeypatch.setattr(binding, "_LIB", None)

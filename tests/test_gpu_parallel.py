@@ -259,6 +259,36 @@ def test_hot_path_equals_its_stages(C, L, w, Hq, Hkv, d, m, k, given, strided):
             pc.hot_path(q, kk, v, **{**dict(w=w, rope_theta=1e4, m=m, k_keep=k, chunk_score=score), **bad})
 
 
+@pytest.mark.parametrize("C,Hkv,odd", [(2, 1, "k"), (2, 1, "v"), (2, 1, "kv"), (1, 2, "k"), (1, 2, "v"), (1, 2, "kv")])
+def test_strides_of_dimensions_of_one_entry_do_not_matter(C, Hkv, odd):
+    """One kv-head seen through a transposed view, or one chunk cut out of longer ones: contiguous all the same."""
+    import paper_2502_14317_b200 as pc
+    L, w, Hq, d, m, k_keep = 300, 16, 2, 64, 1, 50
+    g = torch.Generator(device="cuda").manual_seed(C)
+    q, k, v = (torch.randn((C, L, h, d), generator=g, device="cuda").bfloat16() for h in (Hq, Hkv, Hkv))
+
+    def same_values_other_strides(t):
+        if Hkv == 1:
+            t = t[:, :, 0].clone()[:, None].transpose(1, 2)
+        else:
+            t = torch.cat([t, t], dim=1)[:, :L]
+        assert t.is_contiguous() and t.stride() != q.new_empty(t.shape).stride()
+        return t
+
+    k2, v2 = (same_values_other_strides(t) if n in odd else t for n, t in (("k", k), ("v", v)))
+    args = dict(w=w, rope_theta=1e4, m=m, k_keep=k_keep)
+    want, got = pc.hot_path(q, k, v, **args), pc.hot_path(q, k2, v2, **args)
+    by_batch = pc.hot_path_streaming(q, k2, v2, batch=1, **args)
+    kc, vc, pos = pc.gather_kv(k2, v2, want["kept"], want["idx"])
+    want_kc, want_vc, _ = pc.gather_kv(k, v, want["kept"], want["idx"])
+    for key in ("o", "k_rot", "idx", "kc", "vc", "fg"):
+        assert torch.equal(got[key], want[key]) and got[key].stride() == want[key].stride(), key
+    assert torch.equal(by_batch["kc"], want["kc"]) and torch.equal(by_batch["vc"], want["vc"])
+    assert torch.equal(kc, want_kc) and torch.equal(vc, want_vc)
+    with pytest.raises(pc.PcError, match="strides"):
+        pc.hot_path(q, k, torch.cat([v, v], dim=3)[..., :d], **args)
+
+
 def test_hot_path_from_host_matches_device_path(cfg0_inputs):
     """Uploading the chunks in groups on a copy stream must give exactly what the all-on-device path gives."""
     import paper_2502_14317_b200 as pc
