@@ -490,6 +490,8 @@ def hot_path(q, k, v, *, w, rope_theta, m, k_keep, softmax_scale=0.0, chunk_scor
     b = {} if buffers is None else buffers
     lib = load_library()
     _need_cuda(q, k, v, chunk_score)
+    if chunk_score is not None and (chunk_score.dtype != torch.float32 or not chunk_score.is_contiguous()):
+        raise PcError("chunk_score must be contiguous float32")
     C, L, Hq, d = q.shape
     Hkv = k.shape[2]
     m, k_keep = int(m), int(k_keep)

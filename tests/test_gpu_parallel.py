@@ -259,6 +259,16 @@ def test_hot_path_equals_its_stages(C, L, w, Hq, Hkv, d, m, k, given, strided):
             pc.hot_path(q, kk, v, **{**dict(w=w, rope_theta=1e4, m=m, k_keep=k, chunk_score=score), **bad})
 
 
+def test_hot_path_takes_scores_as_contiguous_float32_of_its_chunks_only():
+    import paper_2502_14317_b200 as pc
+    q, k = (torch.zeros((4, 200, h, 64), dtype=torch.bfloat16, device="cuda") for h in (4, 2))
+    score = torch.zeros(8, device="cuda")
+    for bad, why in ((score[:4].double(), "float32"), (score[::2], "contiguous"), (score[:1].expand(4), "contiguous"), (score, "invalid")):
+        with pytest.raises(pc.PcError, match=why):
+            pc.hot_path(q, k, k, w=16, rope_theta=1e4, m=2, k_keep=50, chunk_score=bad)
+    torch.cuda.synchronize()
+
+
 @pytest.mark.parametrize("C,Hkv,odd", [(2, 1, "k"), (2, 1, "v"), (2, 1, "kv"), (1, 2, "k"), (1, 2, "v"), (1, 2, "kv")])
 def test_strides_of_dimensions_of_one_entry_do_not_matter(C, Hkv, odd):
     """One kv-head seen through a transposed view, or one chunk cut out of longer ones: contiguous all the same."""
