@@ -328,10 +328,11 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
   return d;
 }
 
-// Round an fp64 value to bf16, ties to even, in one rounding (no fp32 detour).
+// Round an fp64 value to bf16, ties to even, in one rounding (no fp32 detour).  NaN stays NaN.
 __device__ __forceinline__ uint16_t f64_to_bf16_rne(double x) {
   // fp64 -> fp32 with round-to-odd keeps enough information for a second, exact RNE step
   float f = __double2float_rz(x);
+  if (f != f) return 0x7FFF;                                 // (the addition below would carry into the sign: -0)
   if (static_cast<double>(f) != x) f = __uint_as_float(__float_as_uint(f) | 1u);   // sticky bit
   uint32_t u = __float_as_uint(f);
   u += 0x7FFFu + ((u >> 16) & 1u);

@@ -117,6 +117,26 @@ def test_few_query_rows_deep_and_shallow_rings(B, w, Hq, Hkv, d, Nk):
         assert np.abs(res["lse"][b:b + 1].cpu().numpy() - LSE).max() <= 2e-3
 
 
+@pytest.mark.parametrize("w,Hq,Hkv,d", [(1, 8, 2, 128), (8, 4, 1, 64), (4, 8, 1, 128), (64, 4, 2, 128)])      # 4, 32, 32 and 128 rows
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_queries_that_are_no_numbers(w, Hq, Hkv, d, bad):
+    """A NaN (or an infinity: a logit of inf - inf) in one query makes that row NaN and no other."""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(w)
+    t = [to_dev(_bits(rng, s)) for s in ((1, w, Hq, d), (1, Hkv, 900, d), (1, Hkv, 900, d), (1, w, Hkv, d), (1, w, Hkv, d))]
+    want = pc.parallel_attn(*t, q_pos0=70, rope_theta=1e4, want_lse=True)
+    t[0] = t[0].clone()
+    t[0][0, w - 1, Hq - 1, [3, 3 + d // 2]] = bad
+    got = pc.parallel_attn(*t, q_pos0=70, rope_theta=1e4, want_lse=True)
+    torch.cuda.synchronize()
+    assert int(got["status"].item()) == 0
+    assert got["out"][0, w - 1, Hq - 1].isnan().all() and got["lse"][0, Hq - 1, w - 1].isnan()
+    got["out"][0, w - 1, Hq - 1] = want["out"][0, w - 1, Hq - 1]
+    got["lse"][0, Hq - 1, w - 1] = want["lse"][0, Hq - 1, w - 1]
+    # two bf16 roundings of P and of the result: the row's neighbours may be taken against another reference maximum
+    assert (got["out"].float() - want["out"].float()).abs().max() <= 1e-2 and (got["lse"] - want["lse"]).abs().max() <= 2e-3
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,d,Nk0,cap,steps", [
     (2, 8, 2, 128, 250, 260, (1, 1, 4, 1)),   # crosses a tile boundary of the cache (256) while generating
     (3, 4, 4, 64, 40, 48, (1, 2, 1)),         # MHA, head size 64

@@ -265,6 +265,26 @@ def test_rope_with_and_without_a_table_kernel(C, L, H, d):
     assert np.array_equal(got, orc.rope_bf16(bits, 10000.0))
 
 
+@pytest.mark.parametrize("C,L", [(1, 40), (4, 2500)])             # with and without a table kernel
+def test_rope_of_infinities_and_nans(C, L):
+    """As the fp64 formula gives them: infinities keep their sign, inf - inf and 0 * inf are NaN."""
+    import paper_2502_14317_b200 as pc
+    H, d, inf = 2, 128, np.inf
+    x = np.random.default_rng(L).standard_normal((C, L, H, d)).astype(np.float32)
+    x[..., 0, 5], x[..., 0, 6 + d // 2], x[..., 1, 9], x[..., 1, 9 + d // 2] = inf, -inf, inf, -inf
+    bits = pc_inputs.f32_to_bf16_bits(x)
+    bits[..., 1, 7] = 0x7FC0                                       # NaN
+    got = to_f64(pc.rope_position_reuse(to_dev(bits), rope_theta=1e4))
+    torch.cuda.synchronize()
+    a = np.arange(L)[:, None] * 1e4 ** (-2.0 * np.arange(d // 2) / d)
+    c, s = np.cos(a)[None, :, None], np.sin(a)[None, :, None]
+    u = orc.bf16_to_f64(bits)
+    with np.errstate(invalid="ignore"):
+        ref = np.concatenate([u[..., : d // 2] * c - u[..., d // 2:] * s, u[..., d // 2:] * c + u[..., : d // 2] * s], axis=-1)
+    odd = ~np.isfinite(ref)
+    assert np.array_equal(got[odd], ref[odd], equal_nan=True) and np.isfinite(got[~odd]).all()
+
+
 @pytest.mark.parametrize("L,w,Hq,Hkv,d,lens", [
     (640, 64, 4, 2, 128, [640, 500, 129, 65, 384]),      # CTA pairs: full, ragged, two tiles, one tile, tile-aligned
     (520, 24, 4, 1, 128, [300, 520, 25, 256]),           # w = 24, the shortest chunk has a single context token
