@@ -17,7 +17,7 @@
 // both 55 % busy.  Measured in a loop, whole call, against one block per CTA of a pair (d = 128, even G) and a single-CTA kernel
 // without these roles (the rest): 128K tokens in chunks of 8192, 32/8 heads 9.8 -> 8.5 ms (the kernel from an idle GPU
 // 8.12 -> 7.17 ms = 1227 TFLOP/s); 32/32 heads, chunks of 4096 6.35 -> 5.66 ms; 24/8 heads, ragged 1.70 -> 1.39 ms; head size
-// 64, 32K tokens 1.27 -> 0.93 ms.
+// 64, 32K tokens 1.27 -> 0.93 ms.  A third build, head size 128 on single CTAs, takes short chunks of odd groups (launch_prefill_t).
 //
 // Window scores: the unit that runs the last query tiles of a (chunk, kv-head) group then sweeps the keys once more
 // with the transposed product K_j Qw^T (the CTAs of a pair take alternate key tiles; keys on TMEM lanes, window
@@ -31,8 +31,6 @@ namespace pc {
 namespace {
 
 using namespace flash;
-template <int D> using PCfg = Cfg<D, D == 128>;
-
 // ------------------------------------------------------------------ work decomposition
 // Groups = (chunk, kv-head).  A unit is what the blocks (four of a pair, two of a single CTA) take at a time.  Pair:
 //   G % 4 == 0   one query tile of four q-heads (block A: heads 0, 1 of the four; B: heads 2, 3; one per CTA)
@@ -54,12 +52,12 @@ template <int D> using PCfg = Cfg<D, D == 128>;
 struct Sched2 {
   int T, G, hpu, tpu, P, U, ntu, ipg, batch, hp, n_pass, wp;
 };
-template <int D, bool SPREAD>
+template <class C, bool SPREAD>
 __device__ __forceinline__ Sched2 make_sched2(const PrefillParams& p) {
   Sched2 s;
   s.T = (p.L + TILE - 1) / TILE;
   s.G = p.Hq / p.Hkv;
-  constexpr int BLOCKS = 2 * PCfg<D>::NCTA;
+  constexpr int BLOCKS = 2 * C::NCTA;
   s.hpu = s.G % BLOCKS == 0 ? BLOCKS : (s.G % 2 == 0 ? 2 : 1);      // q-heads and tiles of a unit
   s.tpu = BLOCKS / s.hpu;
   s.P = s.G / s.hpu;
@@ -70,7 +68,7 @@ __device__ __forceinline__ Sched2 make_sched2(const PrefillParams& p) {
   s.ntu = (ntt + s.tpu - 1) / s.tpu;
   if (s.ntu > s.U) s.ntu = s.U;
   s.ipg = SPREAD ? s.U * s.P : 1 + (s.U - s.ntu) * s.P;
-  const long long kv_bytes = (long long)p.L * (4 * D);    // K and V of a group
+  const long long kv_bytes = (long long)p.L * (4 * C::D);    // K and V of a group
   s.batch = (int)((48ll << 20) / kv_bytes);
   if (s.batch < 1) s.batch = 1;
   s.wp = (p.w + 7) & ~7;                                  // window rows of a head in the sweep operand (multiple of 8)
@@ -95,7 +93,7 @@ __device__ __forceinline__ int chunk_length(const PrefillParams& p, int c) {
   return len <= p.w ? p.w + 1 : len;
 }
 // blocks of unit x of a group, counted from the last tile of the chunk
-template <int D>
+template <class C>
 __device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, int x, Desc& d) {
   const int unit = x / s.P, set = x - unit * s.P;
   const int hi = s.T - 1 - unit * s.tpu - (s.T - (d.len + TILE - 1) / TILE);      // upper tile of the unit
@@ -103,7 +101,7 @@ __device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, 
 #pragma unroll
   for (int b = 0; b < 2; ++b) {
     int top;                                              // upper tile of the block over both CTAs
-    if (!PCfg<D>::PAIR) {
+    if (!C::PAIR) {
       d.h[b] = s.hpu == 2 ? h0 + b : h0;
       top = s.hpu == 2 ? hi : hi - 1 + b;
       d.t[b] = top;
@@ -121,15 +119,15 @@ __device__ __forceinline__ void decode_unit(const Sched2& s, int rank, int hkv, 
 // ====================================================================================
 // tensor maps (boxes of 64 d): tm_q (128 tokens), tm_kh (rotated keys, 64 tokens), tm_k (rotated keys, 128 tokens), tm_v
 // (128 tokens), tm_o (store, 128 tokens), tm_qw (wp tokens)
-template <int D, bool SPREAD>
+template <int D, bool PAIR, bool SPREAD>
 __global__ void __launch_bounds__(NT2, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kh,
                const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ CUtensorMap tm_qw,
                const __grid_constant__ PrefillParams prm) {
-  using C = PCfg<D>;
-  constexpr bool PAIR = C::PAIR;
+  using C = Cfg<D, PAIR>;
   constexpr int NCTA = C::NCTA, Q_BYTES = C::Q_BYTES, NQ = C::NQ;
+  constexpr int TILE_STAGES = TILE * D * 2 / C::STAGE_BYTES, STAGE_ATOMS = C::ATOMS / TILE_STAGES;   // of a full key tile (score sweep)
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0;
@@ -148,7 +146,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     if (warp == WARP_PRODUCER) {
       // ================================================================ TMA producer (both CTAs of a pair)
       if (elect_one()) {
-        const Sched2 sch = make_sched2<D, SPREAD>(prm);
+        const Sched2 sch = make_sched2<C, SPREAD>(prm);
         const int n_groups = prm.C * prm.Hkv, n_unit_items = n_groups * sch.ipg, slices = SPREAD ? prm.sweep_slices : 1;
         const int n_items = n_unit_items + (SPREAD ? n_groups * slices : 0);
         const int rows_half = sch.hp * sch.wp;           // sweep operand rows per CTA and pass (B operand half)
@@ -172,7 +170,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           const int nsub = tail ? sch.ntu * sch.P : (unit_item ? 1 : 0);
           for (int sub = 0; sub < nsub; ++sub) {
             d.kind = KIND_FLASH;
-            decode_unit<D>(sch, rank, d.hkv, first + sub, d);
+            decode_unit<C>(sch, rank, d.hkv, first + sub, d);
             if (d.n[1] == 0) continue;                    // (n[0] <= n[1])
             publish<C>(cx, p, d);
             for (int b = 0; b < 2; ++b) {
@@ -190,10 +188,13 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               if (kbar) {
                 if constexpr (PAIR)
                   for (int a = 0; a < 2; ++a) load_box<C>(dst + a * 8192, &tm_kh, kbar, a * 64, d.hkv, j * TILE + (int)rank * 64, d.c);
-                else load_box<C>(dst, &tm_k, kbar, 0, d.hkv, j * TILE, d.c);
+                else
+                  for (int a = 0; a < C::ATOMS; ++a) load_box<C>(dst + a * 16384, &tm_k, kbar, a * 64, d.hkv, j * TILE, d.c);
               }
               const uint32_t vbar = ring_stage<C>(cx, p, leader, &dst);
-              if (vbar) load_box<C>(dst, &tm_v, vbar, (int)rank * 64, d.hkv, j * TILE, d.c);
+              if (vbar)
+                for (int a = 0; a < (PAIR ? 1 : C::ATOMS); ++a)
+                  load_box<C>(dst + a * 16384, &tm_v, vbar, PAIR ? (int)rank * 64 : a * 64, d.hkv, j * TILE, d.c);
             }
           }
           if (tail || !unit_item) {
@@ -222,26 +223,28 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 }
                 ++p.q;
               }
-              // a full key tile takes ATOMS consecutive stages (of a pair: two that start on an even one, everything uses
+              // a full key tile takes TILE_STAGES consecutive stages (of a pair: two that start on an even one, everything uses
               // stages in twos)
               for (int jj = 0; jj < n_steps; ++jj)
-                for (int a = 0; a < C::ATOMS; ++a) {
+                for (int i = 0; i < TILE_STAGES; ++i) {
                   const uint32_t kbar = ring_stage<C>(cx, p, leader, &dst);
-                  if (kbar) load_box<C>(dst, &tm_k, kbar, a * 64, d.hkv, (NCTA * (step0 + jj) + (int)rank) * TILE, d.c);
+                  if (kbar)
+                    for (int a = 0; a < STAGE_ATOMS; ++a)
+                      load_box<C>(dst + a * 16384, &tm_k, kbar, (i * STAGE_ATOMS + a) * 64, d.hkv, (NCTA * (step0 + jj) + (int)rank) * TILE, d.c);
                 }
             }
           }
         }
         Desc d;
         d.kind = KIND_DONE; d.c = d.hkv = d.len = 0;
-        publish<C>(cx, p, d, PAIR || prm.skip_final_publication == 0);
+        publish<C>(cx, p, d, D == 128 || prm.skip_final_publication == 0);
         drain_copies<C>(cx, p, leader);
       }
       __syncwarp();
     } else if (warp == WARP_MMA && leader) {
       // ================================================================ issuer (of a pair: leader CTA)
       if (elect_one()) {
-        const Sched2 sch = make_sched2<D, SPREAD>(prm);
+        const Sched2 sch = make_sched2<C, SPREAD>(prm);
         const int rows_half = sch.hp * sch.wp;
         const uint32_t idesc_sw = make_idesc_bf16_f32(TILE * NCTA, PAIR ? 2 * rows_half : (rows_half + 15) & ~15, false, false);
         Issuer<C> is(cx);
@@ -259,12 +262,14 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             }
             Desc nx;
             nx.kind = KIND_DONE; nx.n[0] = nx.n[1] = 0;
-            // the next unit's first S follows the last tile without a gap
+            // the next unit's first S follows the last tile without a gap, where there are query slots for two units (with fewer
+            // its queries, and behind them its first keys, wait for this unit's end)
+            constexpr bool PRIMES = NQ >= 4;
             for (int j = 0; j < n; ++j) {                        // is.kv: V of tile j; is.kv + 1: the next K
               bool more = j + 1 < n;
               uint32_t k_u32 = 0;
               auto look_ahead = [&]() {
-                if (j + 1 == n) { nx = next_desc<C>(cx, is.nd, false); more = nx.kind == KIND_FLASH; }
+                if (j + 1 == n) { nx = next_desc<C>(cx, is.nd, false); more = PRIMES && nx.kind == KIND_FLASH; }
                 if (more) k_u32 = is.wait_kv(is.kv + 1);
               };
               auto next_s = [&](int b, int nb) {
@@ -295,7 +300,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               if (!C::SEP_P && more) is.free_kv(is.kv + 1);
               is.kv += more ? 2 : 1;
             }
-            primed = nx.kind == KIND_FLASH;
+            primed = PRIMES && nx.kind == KIND_FLASH;
             d = nx;
           } else {
             // ---- score sweep, one pass: S^T = K_j Qw^T.  Its two [128 keys x 256 rows] buffers overlay all of TMEM:
@@ -313,10 +318,13 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 mma_ss_pair_k128<false>(cx.tmem + e * 256, k_u32, is.qa[0], idesc_sw);
               } else {
                 tc_fence_after_sync();
-                for (int b = 0; b < 2; ++b) mma_ss_k64(cx.tmem + e * 256 + b * 128, k_u32, is.qa[b], idesc_sw);
+                for (int b = 0; b < 2; ++b) {
+                  if constexpr (D == 128) mma_ss_k128(cx.tmem + e * 256 + b * 128, k_u32, is.qa[b], idesc_sw);
+                  else mma_ss_k64(cx.tmem + e * 256 + b * 128, k_u32, is.qa[b], idesc_sw);
+                }
               }
               commit<C>(&mi.t_full[e]);
-              for (int a = 0; a < C::ATOMS; ++a) is.free_kv(is.kv++);
+              for (int i = 0; i < TILE_STAGES; ++i) is.free_kv(is.kv++);
             }
             // what follows overwrites the sweep buffers: wait until both were read
             WAIT2S(&mi.t_free[nt & 1], free_par(nt >> 1), W2_TFREE);
@@ -332,7 +340,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     // ================================================================ epilogue: normalise, stage bf16 rows in the block's
     // (now idle) query slot, TMA store
     setmaxnreg_dec<REGS_EPI>();
-    const Sched2 sch = make_sched2<D, SPREAD>(prm);
+    const Sched2 sch = make_sched2<C, SPREAD>(prm);
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
     uint32_t nd = 0, nq = 0, no[2] = {0, 0};
@@ -412,7 +420,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   } else {
     // ================================================================ softmax
     setmaxnreg_inc<REGS_SOFTMAX>();
-    const Sched2 sch = make_sched2<D, SPREAD>(prm);
+    const Sched2 sch = make_sched2<C, SPREAD>(prm);
     const int b = warp >> 2;
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
@@ -557,9 +565,9 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 // heads, d: 1 x 2048, 32/8, 64 (3.1 times) 99 / 54; 1 x 8192, 16/4, 64 (1.7) 332 / 231; 2 x 1024, 8/2, 128 (5.5) 41.6 / 38.1;
 // 2 x 2048, 32/8, 128 (0.8) 100 / 105; 3 x 3000, 24/8, 128 (1.0) 215 / 223.  Not for two tiles, where the count in memory costs more
 // than it spreads (1 x 192, 32/8, 128 20.5 / 21.6; 4 x 256, 4/2, 64 18.4 / 19.1).
-template <int D>
+template <class C>
 static int sweep_slices(const PrefillParams& p, int units) {
-  constexpr int NCTA = PCfg<D>::NCTA, BLOCKS = 2 * NCTA;
+  constexpr int NCTA = C::NCTA, BLOCKS = 2 * NCTA;
   const long long groups = (long long)p.C * p.Hkv;
   const int T = (p.L + TILE - 1) / TILE;
   if (groups > MAX_SPREAD_GROUPS || T < 6) return 0;
@@ -572,22 +580,29 @@ static int sweep_slices(const PrefillParams& p, int units) {
   return n < 1 ? 1 : n;
 }
 
-template <int D, bool SPREAD>
+template <int D, bool PAIR, bool SPREAD>
 static cudaError_t launch_build(const CUtensorMap* maps, const PrefillParams& prm, int grid, cudaStream_t st) {
   // the opt-in to large dynamic shared memory is a per-device attribute of the function: set it on every call
   // (a host-side call of a few hundred nanoseconds) rather than remember which devices have it
-  constexpr auto kernel = prefill_kernel<D, SPREAD>;
-  if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Off<PCfg<D>>::TOTAL); e != cudaSuccess) return e;
-  return launch_chained(kernel, dim3((unsigned)grid), dim3(NT2), Off<PCfg<D>>::TOTAL, st, PCfg<D>::NCTA, maps[0], maps[5], maps[1], maps[2],
+  using C = Cfg<D, PAIR>;
+  constexpr auto kernel = prefill_kernel<D, PAIR, SPREAD>;
+  if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Off<C>::TOTAL); e != cudaSuccess) return e;
+  return launch_chained(kernel, dim3((unsigned)grid), dim3(NT2), Off<C>::TOTAL, st, C::NCTA, maps[0], maps[5], maps[1], maps[2],
                         maps[3], maps[4], prm);
 }
 template <int D>
 static cudaError_t launch_prefill_t(const CUtensorMap* maps, PrefillParams prm, int sm_count, cudaStream_t st) {
-  constexpr int NCTA = PCfg<D>::NCTA;
-  const int grid = sm_count / NCTA * NCTA;               // one CTA per SM, a whole number of pairs
+  using C = Cfg<D, D == 128>;
+  const int grid = sm_count / C::NCTA * C::NCTA;         // one CTA per SM, a whole number of pairs
   if (grid < 1) return cudaErrorInvalidConfiguration;
-  prm.sweep_slices = sweep_slices<D>(prm, grid / NCTA);
-  return prm.sweep_slices > 0 ? launch_build<D, true>(maps, prm, grid, st) : launch_build<D, false>(maps, prm, grid, st);
+  prm.sweep_slices = sweep_slices<C>(prm, grid / C::NCTA);
+  // Odd G and chunks that do not fill a pair's unit of four tiles: single CTAs (two tiles) where there are more groups than pairs, so
+  // that a group per CTA is not what counts.  us, pairs / single CTAs, C x L, heads, d = 128: 128 x 128, 32/32 508 / 314;
+  // 32 x 256, 32/32 186 / 145; 128 x 256, 24/8 373 / 303; 128 x 300, 32/32 953 / 720; fewer groups: 12 x 256, 28/4 (48) 63 / 80.
+  if constexpr (C::PAIR)
+    if (prm.Hq / prm.Hkv % 2 != 0 && prm.L <= 3 * TILE && (long long)prm.C * prm.Hkv > grid / C::NCTA)
+      return launch_build<D, false, false>(maps, prm, sm_count, st);
+  return prm.sweep_slices > 0 ? launch_build<D, C::PAIR, true>(maps, prm, grid, st) : launch_build<D, C::PAIR, false>(maps, prm, grid, st);
 }
 
 // maps: 0 q (box 64 x 128 tokens), 1 rotated keys (64 x 128), 2 v (64 x 128), 3 o (store), 4 q with a

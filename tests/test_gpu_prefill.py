@@ -104,6 +104,18 @@ def test_units_of_a_cta_pair(L, Hq, Hkv, chunk_len):
         assert not res["o"][c, n:].any() and not res["win_score"][c, :, n:].any()
 
 
+@pytest.mark.parametrize("C,L,w,Hq,Hkv,chunk_len", [
+    (3, 100, 8, 32, 32, None), (10, 129, 100, 24, 8, None), (40, 256, 16, 6, 2, None), (20, 300, 24, 20, 4, None), (25, 384, 128, 9, 3, None),
+    (38, 128, 1, 2, 2, None), (5, 384, 40, 16, 16, [384, 41, 129, 256, 300]), (3, 260, 64, 75, 25, [65, 260, 128]),
+])
+def test_short_chunks_of_odd_groups(C, L, w, Hq, Hkv, chunk_len):
+    """Head size 128 on single CTAs: up to three query tiles, an odd number of q-heads per kv-head, more groups than CTA pairs."""
+    if chunk_len is None:
+        test_shapes(C, L, w, Hq, Hkv, 128, 10000.0)
+    else:
+        test_score_sweeps_as_items_of_their_own(C, L, w, Hq, Hkv, 128, chunk_len)
+
+
 @pytest.mark.parametrize("d", [64, 128])
 def test_growing_logits_rescale_path(d):
     """Keys whose norm grows along the chunk make the running row maximum jump by more than the lazy
