@@ -431,22 +431,25 @@ ParallelPlan parallel_plan(int B, int w, int Hq, int Hkv, int d, int Nk, int sm_
   if (room > 1) off += align_up((size_t)B * Hq * room * w * d * sizeof(float));
   p.total = off;
 
-  // Blocks of 128 rows per CTA (256 per pair) come in twos: an even number of them is filled with different rows that share
-  // every key tile, an odd number (in most cases one) holds the rows twice and takes alternate tiles.
+  // Blocks of 128 rows per CTA (256 per pair) come in twos.  An odd number of them (in most cases one) holds the rows twice and takes
+  // alternate tiles; an even number can do that too, or be filled with different rows that share every key tile, with half
+  // the items.  Rows and key splits: least time by a model in microseconds - rounds of the grid x (about 5 for an item + 1.4
+  // a tile, 2.8 where a tile serves two blocks of rows, 1.5 where the other blocks' items read it again) + 4 for the merge of
+  // splits.  Measured, us, shared / alternate tiles: 64/4 heads of 128, window of 32, 8 sequences of 3000 entries (32 or 64 items
+  // on 74 pairs) 60.7 / 40.1, 64 of 8192 (256 / 512 items) 512 / 503; 32/8, window of 128, 12 of 8192 (96 / 192) 260 / 218, 16 of 4096 159 / 169.
   p.pair = d == 128 && G * w > 128 && sm_count >= 2;
   const int block_heads = (p.pair ? 256 : 128) / w, blocks = (G + block_heads - 1) / block_heads;
-  p.alt = blocks % 2;
-  p.n_rg = p.alt ? blocks : blocks / 2;
-  // Key splits: least time by a model in microseconds - rounds of the grid x (about 5 for an item + 1.4 a tile, twice that
-  // where a tile is used by two blocks of rows) + 4 for the merge of splits.
   const int units = p.pair ? sm_count / 2 : sm_count, n_all = p.n_cache_tiles + 1;
-  const long long groups = (long long)B * Hkv * p.n_rg;
   double least_us = -1.0;
-  p.n_split = 1;
-  for (int s = 1; s <= room && s <= 64 && 2 * s <= n_all + 1; ++s) {
-    const double rounds = std::ceil((double)groups * s / units);
-    const double cost = rounds * (5.0 + (p.alt ? 1.4 : 2.8) * std::ceil((double)n_all / s)) + (s > 1 ? 4.0 : 0.0);
-    if (least_us < 0.0 || cost < least_us) { least_us = cost; p.n_split = s; }
+  for (int alt = blocks % 2; alt <= 1; ++alt) {
+    const int n_rg = alt ? blocks : blocks / 2;
+    const double tile_us = alt ? (blocks % 2 ? 1.4 : 1.5) : 2.8;
+    const long long groups = (long long)B * Hkv * n_rg;
+    for (int s = 1; s == 1 || (s <= room && s <= 64 && 2 * s <= n_all + 1); ++s) {
+      const double rounds = std::ceil((double)groups * s / units);
+      const double cost = rounds * (5.0 + tile_us * std::ceil((double)n_all / s)) + (s > 1 ? 4.0 : 0.0);
+      if (least_us < 0.0 || cost < least_us) { least_us = cost; p.alt = alt; p.n_rg = n_rg; p.n_split = s; }
+    }
   }
   return p;
 }

@@ -5,12 +5,13 @@
 #include "pc_attn.h"
 #include "pc_kernels.h"
 
-static int g_fail_at = -1, g_launches = 0, g_attention = 0;
+static int g_fail_at = -1, g_launches = 0, g_attention = 0, g_items = 0;
 static cudaError_t g_last = cudaSuccess;
 
 extern "C" {
 __attribute__((visibility("default"))) void fake_reset(int fail_at) { g_fail_at = fail_at; g_launches = g_attention = 0; g_last = cudaSuccess; }
 __attribute__((visibility("default"))) int fake_attention_launches() { return g_attention; }
+__attribute__((visibility("default"))) int fake_window_items() { return g_items; }
 __attribute__((visibility("default"))) int fake_last_error() { return (int)g_last; }
 
 void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
@@ -42,7 +43,10 @@ static cudaError_t attention() {                                  // (the real o
   return g_launches++ == g_fail_at ? (g_last = cudaErrorLaunchOutOfResources) : cudaSuccess;
 }
 cudaError_t launch_prefill_attn(const CUtensorMap*, const PrefillParams&, int, int, cudaStream_t) { return attention(); }
-cudaError_t launch_parallel_attn(const CUtensorMap*, const ParallelParams&, int, bool, int, cudaStream_t) { return attention(); }
+cudaError_t launch_parallel_attn(const CUtensorMap*, const ParallelParams& p, int, bool, int, cudaStream_t) {
+  g_items = p.B * p.Hkv * p.n_rg * p.n_split;
+  return attention();
+}
 cudaError_t launch_decode_attn(const CUtensorMap*, const DecodeParams&, int, cudaStream_t) { return attention(); }
 int decode_clusters(int, bool) { return 8; }
 void launch_chunk_score(const float*, int, int, float*, cudaStream_t) {}

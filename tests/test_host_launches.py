@@ -83,3 +83,13 @@ def test_whole_path_refuses_values_that_are_not_contiguous(fake):
         assert _hot_path(fake, _desc(v_stride=v_stride)) == (-1, 1, 0), v_stride
     for C, Hkv, v_stride in ((2, 2, (0, 0, 0)), (2, 2, (300 * 256, 256, 128)), (1, 2, (900 * 256, 256, 128)), (2, 1, (300 * 128, 128, 38400))):
         assert _hot_path(fake, _desc(C=C, Hkv=Hkv, v_stride=v_stride)) == (0, 0, 2), v_stride
+
+
+@pytest.mark.parametrize("B,w,Hq,Hkv,Nk,items", [
+    (8, 32, 64, 4, 3000, 64), (16, 64, 16, 1, 4096, 64), (12, 128, 32, 8, 8192, 192),    # 512 rows a kv-head: one item of 512 would idle pairs
+    (16, 128, 32, 8, 4096, 128), (64, 64, 64, 4, 8192, 512),                               # here it does not
+])
+def test_row_groups_that_fill_the_gpu(fake, B, w, Hq, Hkv, Nk, items):
+    fake.fake_reset(-1)
+    assert fake.pc_parallel_attn(B, w, Hq, Hkv, 128, Nk, P, 0, 1e4, 0.0, P, P, P, P, P, None, None, P, 1 << 40, None) == 0
+    assert fake.fake_window_items() == items
