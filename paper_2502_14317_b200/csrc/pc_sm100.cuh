@@ -332,11 +332,8 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
 __device__ __forceinline__ uint16_t f64_to_bf16_rne(double x) {
   // fp64 -> fp32 with round-to-odd keeps enough information for a second, exact RNE step
   float f = __double2float_rz(x);
-  if (f != f) return 0x7FFF;                                 // (the addition below would carry into the sign: -0)
   if (static_cast<double>(f) != x) f = __uint_as_float(__float_as_uint(f) | 1u);   // sticky bit
-  uint32_t u = __float_as_uint(f);
-  u += 0x7FFFu + ((u >> 16) & 1u);
-  return static_cast<uint16_t>(u >> 16);
+  return __bfloat16_as_ushort(__float2bfloat16_rn(f));
 }
 
 // ------------------------------------------------------------------ CTA pairs (cluster of 2, cta_group::2)
