@@ -478,14 +478,20 @@ int few_clusters(int n, bool deep) {
 struct FewPlan { int split; bool deep; };
 FewPlan few_plan(int B, int w, int Hq, int Hkv, int d, int n_cache_tiles) {
   FewPlan p = {0, false};
-  if (Hq / Hkv * w > 32) return p;
+  const int rows = Hq / Hkv * w;
+  if (rows > 32) return p;
+  // Long caches: a (sequence, kv-head) has at most 16 CTAs here and up to 64 splits in the wide kernel.  Measured, us, here / wide: one
+  // sequence, 8/1 heads of 128, 32 rows 65536 entries 45.5 / 27.3 but with four sequences 47.1 / 49.4, 131072 82 / 36 and 82 / 68; 28 rows, 14/2
+  // heads of 64 32768 27.7 / 25.1 and 38.5 / 29.9, 65536 46.8 / 27.9 and 70.7 / 44.6; one row, 8/1 heads of 128 65536 28.5 / 25.4, 131072 49.8 / 34.2 but
+  // with four sequences 53.9 / 64.6, 524288 174 / 81 and 195 / 179.
+  if (rows > 16 ? n_cache_tiles >= 8 * d : n_cache_tiles >= 1024ll * B * Hkv) return p;
   // Least time by a model in microseconds: rounds of clusters x (6.5 for prologue, pipeline fill and merge + a tile at the
   // CTA's share of the memory bandwidth, no faster than one CTA alone takes it).  Head size 128 has a build with six 32 KB stages and one
   // CTA per SM: alone it takes a tile in 0.67 us, with three stages in 1.43 (the load of the next but one tile then waits for
   // the products of this one).  Measured, us, three stages / six, best split of each: 16401 entries x 8 kv-heads, one
   // sequence 20.5 (16 CTAs) / 17.0 (10), two 27.9 (12) / 26.0 (6), four 44.7 (8) / 43.4 (4); 4 kv-heads 18.0 (16) / 13.5 (16);
   // 16 sequences of 8192 81.6 (2) / 81.1 (1).
-  const bool wide = Hq / Hkv * w > 16;
+  const bool wide = rows > 16;
   const double tile_us = 512.0 * d / 6.5e6;
   double least = -1.0;
   for (int deep = 0; deep <= (d == 128 ? 1 : 0); ++deep) {

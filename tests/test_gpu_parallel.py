@@ -137,6 +137,26 @@ def test_queries_that_are_no_numbers(w, Hq, Hkv, d, bad):
     assert (got["out"].float() - want["out"].float()).abs().max() <= 1e-2 and (got["lse"] - want["lse"]).abs().max() <= 2e-3
 
 
+@pytest.mark.parametrize("w,Hq,Hkv,d,Nk,one_launch", [
+    (8, 4, 1, 64, 511 * 128, True), (8, 4, 1, 64, 511 * 128 + 1, False), (1, 17, 1, 128, 1023 * 128 + 5, False),
+    (1, 2, 1, 128, 1023 * 128, True), (1, 2, 1, 128, 1024 * 128, False), (2, 1, 1, 64, 1023 * 128 + 70, False),
+])
+def test_few_query_rows_over_long_caches(w, Hq, Hkv, d, Nk, one_launch):
+    """At both sides of the cache lengths from which the wide kernel, which splits keys further, takes few rows too."""
+    import paper_2502_14317_b200 as pc
+    g = torch.Generator(device="cuda").manual_seed(Nk)
+    t = [torch.randn(s, generator=g, device="cuda").bfloat16() for s in ((1, w, Hq, d), (1, Hkv, Nk, d), (1, Hkv, Nk, d), (1, w, Hkv, d), (1, w, Hkv, d))]
+    n = pc.launch_count()
+    res = pc.parallel_attn(*t, q_pos0=500, rope_theta=1e4, want_lse=True)
+    assert (pc.launch_count() - n == 1) == one_launch
+    torch.cuda.synchronize()
+    assert int(res["status"].item()) == 0
+    q, kc, vc, kw, vw = (to_bits(x) for x in t)
+    Fg, LSE = orc.parallel_attention(q, 500, 1e4, None, kc, vc, kw, vw)
+    check_attention_output(to_f64(res["out"]), Fg, "Fg")
+    assert np.abs(res["lse"].cpu().numpy() - LSE).max() <= 2e-3
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,d,Nk0,cap,steps", [
     (2, 8, 2, 128, 250, 260, (1, 1, 4, 1)),   # crosses a tile boundary of the cache (256) while generating
     (3, 4, 4, 64, 40, 48, (1, 2, 1)),         # MHA, head size 64
