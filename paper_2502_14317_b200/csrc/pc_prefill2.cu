@@ -467,7 +467,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             }
             named_barrier_sync(3, 256);
           } else {
-            mbar_wait_cluster(&mi.lse_rdy, full_par(n_lse), cx.abort_flag, cx.status, W2_LSE);
+            mbar_wait_cluster(&mi.lse_rdy, full_par(n_lse), cx.abort_flag, cx.status, C::CODE + W2_LSE);
             ++n_lse;
           }
         }
