@@ -60,6 +60,7 @@ struct __align__(16) Misc2 {
   uint64_t lse_rdy;
   uint64_t mma_done;
   Desc desc[NDESC];
+  int left[2];                               // warps of the epilogue / the softmax that are through (leave_group)
   int item;
   uint32_t tmem_base;
   int abort_flag;                            // the two words after tmem_base stay adjacent: bounded waits read the limit
@@ -168,6 +169,7 @@ __device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool
   mbar_init(&mi.item_full, 1); mbar_init(&mi.item_free, 1);
   mbar_init(&mi.lse_rdy, 4 * N);
   mbar_init(&mi.mma_done, 1);
+  mi.left[0] = mi.left[1] = 0;
   mi.abort_flag = 0;
   mi.wait_kcycles = wait_kcycles;
   fence_mbar_init();
@@ -184,6 +186,24 @@ __device__ __forceinline__ Desc next_desc(const Ctx2& cx, uint32_t& n, bool whol
   if (whole_warp) warp_arrive(&mi.d_free[slot]); else mbar_arrive(&mi.d_free[slot]);
   ++n;
   return d;
+}
+
+// A warp of a group that meets at hardware barrier `id` leaves its loop.  After a wait has run out the warps of a group see the abort
+// flag at different times: one may leave while another goes on to such a barrier, which has no limit.  So a warp that is
+// through keeps meeting the others there until all are through.  Every warp takes part in every meeting, so that they
+// agree on its number (odd: whether this warp has taken part in an odd number so far): arrivals are counted after an even one and
+// looked at after an odd one, and all see the same count.
+template <int WARPS>
+__device__ __forceinline__ void leave_group(int id, bool odd, int* left) {
+  if (odd) named_barrier_sync(id, 32 * WARPS);
+  if ((threadIdx.x & 31) == 0) atomicAdd(left, 1);
+  __syncwarp();
+  while (true) {
+    named_barrier_sync(id, 32 * WARPS);
+    const bool all = *reinterpret_cast<volatile int*>(left) == WARPS;
+    if (all) break;
+    named_barrier_sync(id, 32 * WARPS);
+  }
 }
 
 // ------------------------------------------------------------------ producer

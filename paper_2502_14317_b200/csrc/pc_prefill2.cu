@@ -416,6 +416,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
       }
     }
+    leave_group<4>(1, (no[0] + no[1]) & 1u, &mi.left[0]);        // (a meeting per block)
     if (r == 0) tma_store_wait_all();
   } else {
     // ================================================================ softmax
@@ -466,6 +467,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               wait_count(prm.counter + 1 + d.c * prm.Hkv + d.hkv, tiles * sch.G, cx.abort_flag, cx.status, C::CODE + W2_LSE);
             }
             named_barrier_sync(3, 256);
+            ++n_lse;
           } else {
             mbar_wait_cluster(&mi.lse_rdy, full_par(n_lse), cx.abort_flag, cx.status, C::CODE + W2_LSE);
             ++n_lse;
@@ -552,6 +554,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         nq += 3 - NCTA;
       }
     }
+    // (meetings of a sweep pass: one per step and two more, with SPREAD a third in the first pass)
+    leave_group<8>(3, (nt + (SPREAD ? n_lse : 0u)) & 1u, &mi.left[1]);
   }
 
   teardown<C>(cx);
