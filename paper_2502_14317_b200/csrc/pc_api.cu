@@ -188,11 +188,20 @@ int32_t prefill_attn_impl(const pc_prefill_desc* desc, const void* q, const void
   prm.C = desc->C; prm.L = desc->L; prm.w = desc->w; prm.Hq = desc->Hq; prm.Hkv = desc->Hkv;
   const double scale = desc->softmax_scale > 0.0f ? (double)desc->softmax_scale : 1.0 / std::sqrt((double)d);
   prm.scale_log2 = (float)(scale * 1.4426950408889634);
-  prm.lse = lse; prm.win_lse = win_lse; prm.win_score = win_score;
+  // The score sweep takes the window rows' log-sum-exp in log2 units, as the blocks have it (from the natural logarithm
+  // that is returned it would be rounded twice more).  It stands where the rotation's tables were, which nothing needs any more; where
+  // they are too small (very short chunks, many of them) in win_lse itself, converted in place afterwards.
+  const long long n_win = (long long)desc->C * desc->Hq * desc->w;
+  const bool in_tables = (size_t)n_win * sizeof(float) <= lay.off_qrot - lay.off_table;
+  prm.win_lse = in_tables ? win_lse : nullptr;
+  prm.win_lse2 = in_tables ? reinterpret_cast<float*>(table) : win_lse;
+  prm.lse = lse; prm.win_score = win_score;
   prm.status = status_word; prm.counter = counter;
   prm.wait_kcycles = pc::g_wait_kcycles.load();
   prm.skip_final_publication = pc::g_skip_final_publication.load();
-  return launched(pc::launch_prefill_attn(maps, prm, d, dev.sm_count, st));
+  cudaError_t e = pc::launch_prefill_attn(maps, prm, d, dev.sm_count, st);
+  if (e == cudaSuccess && !in_tables) e = pc::launch_win_lse_natural(win_lse, n_win, st);
+  return launched(e);
 }
 
 }  // namespace

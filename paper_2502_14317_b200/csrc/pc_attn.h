@@ -15,7 +15,8 @@ struct PrefillParams {
   float scale_log2;              // softmax scale * log2(e)
   const int* chunk_len;          // [C] tokens per chunk (window included) or null: all L
   float* lse;                    // [C,Hq,L] or null
-  float* win_lse;                // [C,Hq,w]
+  float* win_lse;                // [C,Hq,w], or null: win_lse2 is converted afterwards (launch_win_lse_natural)
+  float* win_lse2;               // [C,Hq,w] in log2 units, as the score sweep needs it
   float* win_score;              // [C,Hkv,L]
   int* status;                   // device status word or null
   int* counter;                  // work-queue counter and COUNTER_WORDS - 1 words behind it, zeroed before launch
@@ -26,6 +27,9 @@ struct PrefillParams {
 
 // maps: rotated q (box 64 x 1 x 128 tokens), k_rot, v, o (store), rotated q with a wp-row box, k_rot with a 64-token box
 cudaError_t launch_prefill_attn(const CUtensorMap* maps, const PrefillParams& prm, int d, int sm_count, cudaStream_t st);
+
+// x[i] *= ln 2: log-sum-exp in log2 units to natural ones
+cudaError_t launch_win_lse_natural(float* x, long long n, cudaStream_t st);
 
 // Parallel attention, more than 32 query rows per kv-head (pc_parallel.cu).
 struct ParallelParams {

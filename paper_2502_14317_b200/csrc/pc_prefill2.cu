@@ -398,7 +398,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           const size_t row = (size_t)d.c * prm.Hq + h;
           if (prm.lse) prm.lse[row * prm.L + token] = lse2 * 0.6931471805599453f;
           const int wi = token - (d.len - prm.w);
-          if (wi >= 0) prm.win_lse[row * prm.w + wi] = lse2 * 0.6931471805599453f;
+          if (wi >= 0) {
+            prm.win_lse2[row * prm.w + wi] = lse2;               // for the score sweep
+            if (prm.win_lse != nullptr) prm.win_lse[row * prm.w + wi] = lse2 * 0.6931471805599453f;
+          }
         }
         fence_proxy_async_smem();
         named_barrier_sync(1, 128);
@@ -477,16 +480,12 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const int g0 = u * 2 * sch.hp + b * sch.hp;
         const int heads = sch.G - g0 < sch.hp ? (sch.G > g0 ? sch.G - g0 : 0) : sch.hp;
         const int cols = heads * sch.wp;
-        // log-sum-exp of the columns' window rows in log2 units; +inf (probability 0) in columns that are no window rows.
-        // (The outputs win_lse are read back, from both CTAs: exact to half an ulp of the natural logarithm.)
+        // log-sum-exp of the columns' window rows in log2 units; +inf (probability 0) in columns that are no window rows
         float* const lse_cols = &mi.lm[1][b][0];
         if (r < cols) {
           const int wi = r % sch.wp - (sch.wp - prm.w);
           float x = INFINITY;
-          if (wi >= 0) {
-            const float nat = __ldcg(prm.win_lse + ((size_t)d.c * prm.Hq + d.hkv * sch.G + g0 + r / sch.wp) * prm.w + wi);
-            x = fmaf(nat, 1.442695040888963f, nat * 1.925963033500e-8f);     // log2(e) as a sum of two floats
-          }
+          if (wi >= 0) x = __ldcg(prm.win_lse2 + ((size_t)d.c * prm.Hq + d.hkv * sch.G + g0 + r / sch.wp) * prm.w + wi);
           lse_cols[r] = x;
         }
         named_barrier_sync(3, 256);
@@ -607,6 +606,14 @@ static cudaError_t launch_prefill_t(const CUtensorMap* maps, PrefillParams prm, 
     if (prm.Hq / prm.Hkv % 2 != 0 && prm.L <= 3 * TILE && (long long)prm.C * prm.Hkv > grid / C::NCTA)
       return launch_build<D, false, false>(maps, prm, sm_count, st);
   return prm.sweep_slices > 0 ? launch_build<D, C::PAIR, true>(maps, prm, grid, st) : launch_build<D, C::PAIR, false>(maps, prm, grid, st);
+}
+
+__global__ void __launch_bounds__(256) win_lse_natural_kernel(float* x, long long n) {
+  chain();
+  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256) x[i] *= 0.6931471805599453f;
+}
+cudaError_t launch_win_lse_natural(float* x, long long n, cudaStream_t st) {
+  return launch_chained(win_lse_natural_kernel, dim3((unsigned)((n + 255) / 256 < 1184 ? (n + 255) / 256 : 1184)), dim3(256), 0, st, 1, x, n);
 }
 
 // maps: 0 q (box 64 x 128 tokens), 1 rotated keys (64 x 128), 2 v (64 x 128), 3 o (store), 4 q with a

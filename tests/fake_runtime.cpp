@@ -48,6 +48,7 @@ cudaError_t launch_parallel_attn(const CUtensorMap*, const ParallelParams& p, in
   return attention();
 }
 cudaError_t launch_decode_attn(const CUtensorMap*, const DecodeParams&, int, cudaStream_t) { return attention(); }
+cudaError_t launch_win_lse_natural(float*, long long, cudaStream_t) { return cudaSuccess; }
 int decode_clusters(int, bool) { return 8; }
 void launch_chunk_score(const float*, int, int, float*, cudaStream_t) {}
 void launch_select_chunks(const float*, int, int, int, int*, cudaStream_t) {}

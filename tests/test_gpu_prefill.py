@@ -265,6 +265,33 @@ def test_several_short_score_sweeps_on_one_cta(C, L, w, Hq, Hkv, d, chunk_len):
     test_score_sweeps_as_items_of_their_own(C, L, w, Hq, Hkv, d, chunk_len)
 
 
+@pytest.mark.parametrize("C,L,w,Hq,Hkv,d,gain", [
+    (1, 2048, 64, 8, 2, 128, 40.0), (1, 1500, 50, 6, 2, 64, 20.0),
+    (20, 130, 128, 16, 8, 64, 20.0), (30, 200, 64, 60, 20, 128, 30.0),      # more window rows than the rotation's tables have room for
+])
+def test_window_scores_are_as_precise_as_their_log_sum_exp(C, L, w, Hq, Hkv, d, gain):
+    """Large logits: what limits a score is the log-sum-exp of its rows, rounded once to fp32 in log2 units.  The 2-norm of the error may
+    exceed what that rounding alone gives (evaluated here in fp64) by a quarter, for the fp32 logits; a second rounding, of the natural
+    logarithm, would double it."""
+    import paper_2502_14317_b200 as pc
+    theta, G, log2e = 10000.0, Hq // Hkv, np.log2(np.e)
+    rng = np.random.default_rng(3)
+    q, k, v = (pc_inputs.f32_to_bf16_bits(rng.standard_normal((C, L, h, d)).astype(np.float32) * g) for h, g in ((Hq, 1.0), (Hkv, gain), (Hkv, 1.0)))
+    res = pc.chunk_prefill_attn(to_dev(q), to_dev(k), to_dev(v), w=w, rope_theta=theta)
+    torch.cuda.synchronize()
+    assert int(res["status"].item()) == 0
+    qr, kr = orc.bf16_to_f64(orc.rope_bf16(q, theta)), orc.bf16_to_f64(orc.rope_bf16(k, theta))
+    s = np.einsum("cigd,cjgd->cgij", qr[:, L - w:], np.repeat(kr, G, axis=2)) * (log2e / np.sqrt(d))
+    s[:, :, np.arange(L)[None] > (L - w + np.arange(w))[:, None]] = -np.inf
+    m = s.max(-1, keepdims=True)
+    lse = m + np.log2(np.exp2(s - m).sum(-1, keepdims=True))
+    score = lambda l: np.exp2(s - l).sum(2).reshape(C, Hkv, G, L).sum(2)
+    S = score(lse)
+    one_rounding = np.linalg.norm(score(lse.astype(np.float32)) - S)
+    assert np.linalg.norm(res["win_score"].cpu().numpy() - S) <= 1.25 * one_rounding
+    assert np.abs(res["win_lse"].cpu().numpy() - lse[..., 0] / log2e).max() <= 2e-3
+
+
 @pytest.mark.parametrize("C,L,H,d", [(1, 1, 1, 64), (1, 1, 1, 128), (5, 9, 3, 64), (2, 512, 8, 128), (1, 1025, 8, 128), (1, 2049, 8, 64), (3, 700, 37, 128)])
 def test_rope_with_and_without_a_table_kernel(C, L, H, d):
     """Up to 2^20 values the warps of the rotation pass compute their own table rows, above that a kernel of its own does: the
