@@ -16,24 +16,24 @@ def _bits(rng, shape):
 
 @pytest.mark.parametrize("B,w,Hq,Hkv,d,Nk,q_pos0,theta", [
     (2, 16, 4, 2, 64, 128, 240, 1e4),         # cfg0-like compressed cache
-    (1, 64, 8, 2, 128, 1000, 8128, 5e5),      # ragged last cache tile, G*w = 256 rows (both blocks)
-    (1, 64, 32, 8, 128, 4096, 8128, 5e5),     # B = 1: keys split across CTAs + merge kernel
-    (3, 8, 2, 2, 64, 300, 4088, 1e4),         # MHA, smallest window, one block
-    (1, 64, 8, 1, 128, 700, 8128, 5e5),       # G*w = 512 rows: two row groups per kv-head
+    (1, 64, 8, 2, 128, 1000, 8128, 5e5),      # ragged last cache tile, G*w = 256 rows: a CTA pair, both blocks of each CTA on alternate tiles
+    (1, 64, 32, 8, 128, 4096, 8128, 5e5),     # B = 1: keys split, partial results merged
+    (3, 8, 2, 2, 64, 300, 4088, 1e4),         # MHA, 8 rows: the kernel for few rows
+    (1, 64, 8, 1, 128, 700, 8128, 5e5),       # G*w = 512 rows: two row groups of 256 per kv-head
     (2, 128, 2, 1, 64, 77, 0, 1e4),           # cache shorter than one tile, widest window
     (1, 32, 6, 2, 128, 2049, 100, 1e4),       # G = 3, one key past a tile boundary
     (2, 1, 8, 2, 128, 3000, 8191, 5e5),       # decoding step: one query token over the cache (+ its own key)
     (3, 2, 4, 4, 64, 500, 4094, 1e4),         # two query tokens, MHA
     (1, 4, 32, 8, 128, 16384, 8188, 5e5),     # four query tokens over a 16K cache, Llama-3 heads
-    (2, 4, 8, 2, 128, 50, 77, 1e4),           # rows fill one block: two streams; one cache tile to one, the window tile to the other
+    (2, 4, 8, 2, 128, 50, 77, 1e4),           # 16 rows, a cache of one tile and the window's
     (5, 1, 4, 4, 64, 128, 4095, 1e4),         # decoding, MHA, head size 64, cache of exactly one tile
     (1, 16, 8, 2, 128, 5000, 300, 5e5),       # 64 rows per kv-head, 40 cache tiles split over the CTAs, two streams each
-    # batches whose 256-row groups fill the CTA pairs (head size 128, G*w a multiple of 256): the pair kernel
+    # batches that fill the CTA pairs
     (8, 64, 32, 8, 128, 300, 8128, 5e5),      # 64 groups, ragged last cache tile
     (15, 64, 32, 8, 128, 256, 8128, 5e5),     # 120 groups: two rounds per pair, cache of whole tiles
-    (28, 32, 16, 2, 128, 520, 100, 1e4),      # G = 8, w = 32: four heads per CTA
-    (16, 128, 8, 2, 128, 130, 0, 1e4),        # G*w = 512: two groups per kv-head, one head per CTA, two keys in the last tile
-    (60, 8, 32, 1, 128, 129, 5, 1e4),         # smallest window of that kernel: sixteen heads per CTA
+    (28, 32, 16, 2, 128, 520, 100, 1e4),      # G = 8, w = 32: four heads per block
+    (16, 128, 8, 2, 128, 130, 0, 1e4),        # G*w = 512 rows on shared tiles, one head per block, two keys in the last tile
+    (60, 8, 32, 1, 128, 129, 5, 1e4),         # window of 8: sixteen heads per block
 ])
 def test_parallel_attn_shapes(B, w, Hq, Hkv, d, Nk, q_pos0, theta):
     import paper_2502_14317_b200 as pc
@@ -49,6 +49,27 @@ def test_parallel_attn_shapes(B, w, Hq, Hkv, d, Nk, q_pos0, theta):
     Fg, LSE = orc.parallel_attention(qw, q_pos0, theta, None, kc, vc, kw, vw)
     check_attention_output(to_f64(res["out"]), Fg, "Fg")
     assert np.abs(res["lse"].cpu().numpy() - LSE).max() <= 2e-3
+
+
+@pytest.mark.parametrize("B", [1, 64])                            # keys split; whole items, blocks of different rows where that fills the GPU
+@pytest.mark.parametrize("w,G,Hkv,d,Nk", [
+    (64, 3, 2, 128, 1700), (64, 7, 1, 128, 1500), (128, 5, 1, 128, 2300), (16, 9, 2, 128, 2500),   # pairs: 2 + 1 heads; second block 2 + 1; three row groups, the last of one head
+    (64, 7, 1, 64, 1600), (64, 3, 2, 64, 2500), (128, 2, 2, 64, 2000), (64, 4, 2, 64, 1900), (128, 4, 1, 64, 1500),
+])
+def test_row_blocks_that_are_not_full(B, w, G, Hkv, d, Nk):
+    """Wide windows whose rows do not fill their blocks, on CTA pairs and single CTAs, with enough key tiles for the rings to go round."""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(Nk + w + B)
+    Hq = G * Hkv
+    qw, kw, vw = (_bits(rng, (B, w, h, d)) for h in (Hq, Hkv, Hkv))
+    kc, vc = _bits(rng, (B, Hkv, Nk, d)), _bits(rng, (B, Hkv, Nk, d))
+    res = pc.parallel_attn(to_dev(qw), to_dev(kc), to_dev(vc), to_dev(kw), to_dev(vw), q_pos0=333, rope_theta=1e4, want_lse=True)
+    torch.cuda.synchronize()
+    assert int(res["status"].item()) == 0
+    for b in sorted({0, B // 2, B - 1}):
+        Fg, LSE = orc.parallel_attention(qw[b:b + 1], 333, 1e4, None, *(x[b:b + 1] for x in (kc, vc, kw, vw)))
+        check_attention_output(to_f64(res["out"][b:b + 1]), Fg, "Fg")
+        assert np.abs(res["lse"][b:b + 1].cpu().numpy() - LSE).max() <= 2e-3
 
 
 @pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 128), (4, 2, 128), (4, 2, 64)])

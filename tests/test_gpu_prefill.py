@@ -47,11 +47,11 @@ def test_cfg0_full(cfg0_inputs):
     (1, 100, 32, 8, 1, 64, 10000.0),       # single ragged tile, G*w = 256 window rows
     (1, 640, 64, 8, 1, 128, 500000.0),     # G*w = 512 window rows: two score passes
     (1, 130, 64, 1, 1, 64, 10000.0),       # single head, MHA, two tiles with a 2-token tail
-    # head size 128 runs on CTA pairs: two q-heads (or two adjacent query tiles) per pair
-    (2, 300, 16, 2, 1, 128, 10000.0),      # G=2: one head pair, ragged last tile
-    (1, 100, 32, 1, 1, 128, 10000.0),      # MHA, a single ragged tile: the second CTA of the pair has no block
+    # head size 128 runs on CTA pairs: four (q-head, query tile) blocks per pair
+    (2, 300, 16, 2, 1, 128, 10000.0),      # G=2: two heads, two tiles a unit, ragged last tile
+    (1, 100, 32, 1, 1, 128, 10000.0),      # MHA, a single ragged tile: one of the four blocks is there
     (1, 256, 128, 4, 2, 128, 500000.0),    # widest window = exactly the last tile, two kv-heads
-    (2, 1100, 64, 6, 2, 128, 10000.0),     # G=3 (odd): tile-pair mode, 9 tiles, ragged
+    (2, 1100, 64, 6, 2, 128, 10000.0),     # G=3 (odd): units of four tiles of a head, 9 tiles, ragged
     (1, 1024, 8, 2, 2, 128, 10000.0),      # MHA, even tile count, smallest window
     (1, 200, 128, 8, 1, 128, 10000.0),     # G*w = 1024 window rows: four score passes, window over two tiles
     # windows that are no power of two (the sweep pads a head's rows to a multiple of 8 and leaves the pad out)
@@ -59,7 +59,7 @@ def test_cfg0_full(cfg0_inputs):
     (1, 700, 100, 4, 1, 128, 500000.0),    # CTA pairs, w = 100 (the region size of App. C), window over two tiles
     (1, 300, 5, 2, 1, 128, 10000.0),       # CTA pairs, w = 5 < 8
     (1, 260, 1, 4, 2, 128, 10000.0),       # CTA pairs, a single query token
-    (2, 400, 24, 3, 3, 128, 10000.0),      # multi-head (single-CTA kernel, tile-pair mode), w = 24
+    (2, 400, 24, 3, 3, 128, 10000.0),      # multi-head, units of four tiles, w = 24
     (1, 520, 100, 6, 2, 128, 10000.0),     # G = 3, w = 100
     (2, 300, 24, 4, 2, 64, 10000.0),       # head size 64, w = 24
     (1, 333, 100, 2, 1, 64, 10000.0),      # head size 64, w = 100
@@ -132,9 +132,9 @@ def test_growing_logits_rescale_path(d):
 
 @pytest.mark.parametrize("Hq,Hkv", [(4, 2), (2, 2), (6, 2)])
 def test_growing_logits_many_tiles(Hq, Hkv):
-    """The same stress over 13 key tiles, two chunks, even and odd group sizes: the softmax warpgroups, the three
-    issuing threads and the TMEM buffers go through many rounds in which a warpgroup stalls in the rescale path
-    while the other runs ahead, including across query blocks and the score sweep."""
+    """The same stress over 13 key tiles, two chunks, even and odd group sizes: the softmax warpgroups and the TMEM
+    buffers go through many rounds in which a warpgroup stalls in the rescale path while the other runs ahead,
+    including across query blocks and the score sweep."""
     rng = np.random.default_rng(7 + Hq)
     C, L, w, d = 2, 1600, 64, 128
     q = rng.standard_normal((C, L, Hq, d)).astype(np.float32)
@@ -163,7 +163,7 @@ def test_deterministic_and_strided(cfg0_inputs):
 
 
 def test_deterministic_head_size_128():
-    """The CTA-pair kernel (two issuing threads, two softmax warpgroups on alternate tiles) must give the same
+    """The kernel on CTA pairs (work dealt out by a counter, a softmax warpgroup per query block) must give the same
     bits run to run: accumulation order and score sums are fixed by construction."""
     import paper_2502_14317_b200 as pc
     rng = np.random.default_rng(5)
@@ -206,15 +206,15 @@ def test_argument_errors():
 
 
 @pytest.mark.parametrize("C,L,H,d,theta", [
-    (2, 8192, 4, 128, 500000.0),           # the routine of the tile prologue, positions up to 8191 (angles up to 8191 rad)
+    (2, 8192, 4, 128, 500000.0),           # positions up to 8191 (angles up to 8191 rad)
     (1, 4096, 8, 128, 10000.0),
     (3, 333, 2, 128, 10000.0),             # ragged last tile
-    (2, 1000, 3, 64, 10000.0),             # head size 64: the fp64 pre-pass kernel
+    (2, 1000, 3, 64, 10000.0),             # head size 64
 ])
 def test_rope_position_reuse_equals_fp64_rotation_rounded_once(C, L, H, d, theta):
-    """The query rotation of the tile prologue is fp32 with two exact fallbacks; its bits must be those of the
-    oracle's fp64 rotation.  Mixed magnitudes so that many outputs sit near a bf16 rounding boundary; with
-    millions of outputs the second level (about 1 in 4000) runs thousands of times."""
+    """The rotation is fp32 with two exact fallbacks; its bits must be those of the oracle's fp64 rotation.  Mixed
+    magnitudes so that many outputs sit near a bf16 rounding boundary; with millions of outputs the second level
+    (about 1 in 1300) runs thousands of times."""
     import paper_2502_14317_b200 as pc
     rng = np.random.default_rng(5 + L + d)
     x = rng.standard_normal((C, L, H, d)).astype(np.float32) * np.exp2(rng.integers(-6, 7, size=(C, L, H, 1))).astype(np.float32)
@@ -327,7 +327,7 @@ def test_rope_of_infinities_and_nans(C, L):
 @pytest.mark.parametrize("L,w,Hq,Hkv,d,lens", [
     (640, 64, 4, 2, 128, [640, 500, 129, 65, 384]),      # CTA pairs: full, ragged, two tiles, one tile, tile-aligned
     (520, 24, 4, 1, 128, [300, 520, 25, 256]),           # w = 24, the shortest chunk has a single context token
-    (640, 64, 3, 3, 128, [640, 333, 130, 65]),           # multi-head, single-CTA kernel (tile-pair mode)
+    (640, 64, 3, 3, 128, [640, 333, 130, 65]),           # multi-head: units of four tiles, fewer in the shorter chunks
     (400, 16, 4, 2, 64, [400, 17, 250, 128]),            # head size 64
     (300, 100, 2, 2, 64, [101, 300, 229]),               # head size 64, multi-head, w = 100
 ])
