@@ -323,7 +323,8 @@ PC_API int32_t pc_parallel_attn_append(int32_t B, int32_t w, int32_t Hq, int32_t
  * Shapes as in those calls; v and k_rot contiguous (PC_ERR_INVALID_ARG for other strides of v), q_win [w,Hq,d] contiguous (the window rows
  * of chunk 0: for a contiguous q, q + (L-w)*Hq*d).  With clear_status the status word, which
  * both attention calls share, is set to 0 first.  Returns the first failing call's code and
- * names that call in *failed (may be NULL; 0: none).
+ * names that call in *failed (may be NULL; 0: none).  Arguments of a later stage are checked when its turn
+ * comes: the stages before it have been launched by then, as if the calls had been made one by one.
  * pc_hot_path_workspace_bytes gives the size of ws_prefill and, in *parallel_bytes, that of
  * ws_parallel.
  */

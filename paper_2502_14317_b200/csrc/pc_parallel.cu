@@ -13,9 +13,9 @@
 // by a second kernel.
 //
 // What bounds it: many sequences, the power cap and then the tile's softmax (tensor and MUFU pipes 54 % busy, DRAM 43 % of
-// its peak): 64 sequences of 64 queries over 16384 entries, 32/8 heads 1.24 -> 1.21 ms against the kernel that held one
-// block per CTA.  One sequence: latencies, 24 K of 44 K cycles in the tiles of an item, 5 K writing its partial rows, the rest cold
-// code, setup and exit: 54.8 -> 36.6 us (with the rotation and the merge).
+// its peak): 64 sequences of 64 queries over 16384 entries, 32/8 heads take 1.02 ms from an idle GPU and 1.29 ms in a loop, as
+// with one block per CTA before.  One sequence: latencies, 24 K of 44 K cycles in the tiles of an item, 5 K writing its partial rows, the rest
+// cold code, setup and exit: 54.8 -> 36.7 us (with the rotation and the merge).
 #include "pc_attn.h"
 #include "pc_flash.cuh"
 #include "pc_kernels.h"

@@ -15,8 +15,8 @@
 //
 // What bounds it: the board's power cap (1000 W) in any loop of these calls, so energy a tile; tensor and MUFU pipes are
 // both 55 % busy.  Measured in a loop, whole call, against one block per CTA of a pair (d = 128, even G) and a single-CTA kernel
-// without these roles (the rest): 128K tokens in chunks of 8192, 32/8 heads 9.8 -> 8.5 ms (the kernel from an idle GPU
-// 8.12 -> 7.17 ms = 1227 TFLOP/s); 32/32 heads, chunks of 4096 6.35 -> 5.66 ms; 24/8 heads, ragged 1.70 -> 1.39 ms; head size
+// without these roles (the rest): 128K tokens in chunks of 8192, 32/8 heads 9.6 -> 8.4 ms (the kernel from an idle GPU
+// 8.12 -> 7.17 ms = 1227 TFLOP/s); 32/32 heads, chunks of 4096 6.1 -> 5.5 ms; 24/8 heads, ragged 1.70 -> 1.41 ms; head size
 // 64, 32K tokens 1.27 -> 0.93 ms.  A third build, head size 128 on single CTAs, takes short chunks of odd groups (launch_prefill_t).
 //
 // Window scores: the unit that runs the last query tiles of a (chunk, kv-head) group then sweeps the keys once more

@@ -5,7 +5,7 @@
 // small fraction of the fp32 rate) is almost never executed.  Three levels:
 //   1. fp32 with the fp32 heads of the table entries.  Its error is below 2^-22 (|x1| + |x2|); when
 //      y - tol and y + tol round to the same bf16 value, that value is the correctly rounded one.
-//   2. otherwise (about one output in a few thousand) the value is re-evaluated as an unevaluated sum of two
+//   2. otherwise (about one output in 1300 on N(0,1) inputs) the value is re-evaluated as an unevaluated sum of two
 //      fp32 numbers (products with their exact FMA residuals, the fp32 tails of the table entries), good to
 //      2^-43 (|x1| + |x2|), and rounded from there;
 //   3. if that is still too close to a rounding boundary (practically never), fp64 on the fp64 table.
