@@ -302,12 +302,14 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
   return d;
 }
 
-// Round an fp64 value to bf16, ties to even, in one rounding (no fp32 detour).  NaN stays NaN.
+// Round an fp64 value to bf16, ties to even, in one rounding (no fp32 detour).
 __device__ __forceinline__ uint16_t f64_to_bf16_rne(double x) {
   // fp64 -> fp32 with round-to-odd keeps enough information for a second, exact RNE step
   float f = __double2float_rz(x);
   if (static_cast<double>(f) != x) f = __uint_as_float(__float_as_uint(f) | 1u);   // sticky bit
-  return __bfloat16_as_ushort(__float2bfloat16_rn(f));
+  uint32_t u = __float_as_uint(f);
+  u += 0x7FFFu + ((u >> 16) & 1u);
+  return static_cast<uint16_t>(u >> 16);
 }
 
 // ------------------------------------------------------------------ CTA pairs (cluster of 2, cta_group::2)
