@@ -30,6 +30,7 @@
 #include "pc_attn.h"
 #include "pc_kernels.h"
 #include "pc_softmax.cuh"
+#include <cfloat>
 
 namespace pc {
 
@@ -337,6 +338,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
         if (tid < N) {
           m_old = -mi.negm[tid];
           m_new = fmaxf(fmaxf(fmaxf(mi.red[0][tid], mi.red[1][tid]), fmaxf(mi.red[2][tid], mi.red[3][tid])), m_old);
+          m_new = fmaxf(m_new, -FLT_MAX);                     // every logit so far -inf: the probabilities are 0, not exp2(-inf + inf)
         }
         named_barrier_sync(1, 128);
         if (tid < N) {

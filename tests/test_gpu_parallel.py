@@ -158,6 +158,30 @@ def test_queries_that_are_no_numbers(w, Hq, Hkv, d, bad):
     assert (got["out"].float() - want["out"].float()).abs().max() <= 1e-2 and (got["lse"] - want["lse"]).abs().max() <= 2e-3
 
 
+@pytest.mark.parametrize("G,d,Nk", [(8, 64, 50), (8, 64, 128), (4, 128, 3000), (17, 128, 700), (40, 64, 1500), (130, 128, 700)])
+@pytest.mark.parametrize("where", ["window", "first tile", "every key"])
+def test_logits_of_minus_infinity(G, d, Nk, where):
+    """Keys whose logits are -inf for every query count nothing, also where they are all that a key split or a row's first tile holds;
+    with no other key a row is NaN, as a softmax over nothing is.  (One token at position 0: its queries are not turned.)"""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(Nk + G)
+    q, kc, vc, kw, vw = (to_dev(_bits(rng, s)) for s in ((1, 1, G, d), (1, 1, Nk, d), (1, 1, Nk, d), (1, 1, 1, d), (1, 1, 1, d)))
+    q[..., 0], kc[..., 0], kw[..., 0] = 1.0, 0.0, 0.0
+    if where != "first tile":
+        kw[..., 0] = float("-inf")
+    if where != "window":
+        kc[:, :, :128 if where == "first tile" else Nk, 0] = float("-inf")
+    res = pc.parallel_attn(q, kc, vc, kw, vw, q_pos0=0, rope_theta=1e4)
+    torch.cuda.synchronize()
+    assert int(res["status"].item()) == 0
+    s = torch.cat([kc, kw.transpose(1, 2)], dim=2)[0, 0].double() @ q[0, 0].double().T / d ** 0.5
+    ref = torch.softmax(s, dim=0).T @ torch.cat([vc, vw.transpose(1, 2)], dim=2)[0, 0].double()
+    if where == "every key":
+        assert res["out"].isnan().all()
+    else:
+        check_attention_output(to_f64(res["out"])[0, 0], ref.cpu().numpy(), "Fg", sharp=True)
+
+
 @pytest.mark.parametrize("w,Hq,Hkv,d,Nk,one_launch", [
     (8, 4, 1, 64, 511 * 128, True), (8, 4, 1, 64, 511 * 128 + 1, False), (1, 17, 1, 128, 1023 * 128 + 5, False),
     (1, 2, 1, 128, 1023 * 128, True), (1, 2, 1, 128, 1024 * 128, False), (2, 1, 1, 64, 1023 * 128 + 70, False),
