@@ -80,7 +80,9 @@ PC_API uint64_t pc_launch_count(void);
  * against the final log-sum-exp); it is not a separate launch.
  *
  * q [C,L,Hq,d], k, v [C,L,Hkv,d]: inputs before RoPE, addressed through the element
- * strides (chunk, token, head) in the descriptor.  Queries and keys are rotated by a pass
+ * strides (chunk, token, head) in the descriptor.  Values meet zero probabilities where a key is masked: a
+ * NaN or infinity in v reaches, besides the rows that attend to it, the earlier rows of its 128-token tile (head size 128
+ * and odd G: also of the tile before).  Queries and keys are rotated by a pass
  * of their own ahead of the attention kernel (the rotated queries live in the workspace).
  * chunk_len [C] int32 (device; NULL: every chunk holds L tokens): tokens of chunk c, window
  * included - the paper cuts the input into chunks of AT MOST the trained length.  The
