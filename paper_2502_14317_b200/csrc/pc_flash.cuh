@@ -5,6 +5,12 @@
 // cores work for the other.  Warps (16): 0-3 softmax of block A, 4-7 softmax of block B (thread = query row = TMEM lane),
 // 8-11 epilogue (the softmax warps go straight on to the next block), 12 TMA producer, 13 issuer of all MMAs (of a
 // CTA pair: in the leader only), 14-15 idle.  Registers are dealt out by role: 184 / 80 / 64.
+//
+// Tensor memory, 512 columns: one S (128), P of both blocks (64 each), both accumulators (128 each).  The blocks take turns on
+// S: the softmax warps take a whole S into registers at once, and the product for the other block runs under their
+// exponentials.  A block therefore finds its next S ready when it is through with a tile, and the blocks' exponentials are kept half a
+// step apart.  (With an S of its own for each block and P over its first half, the next product waited for P V of the tile
+// before, 1000 of 3300 cycles a step.)
 // Cfg<D, PAIR>: head size, and whether two CTAs of a cluster work as one unit (cta_group::2: blocks of 2 x 128 rows, every
 // K/V tile split between the two shared memories).
 #pragma once
@@ -29,10 +35,8 @@ struct Cfg {
   static constexpr int STAGE_BYTES = TILE * D * 2 / NCTA;  // K/V ring: a tile, or of a pair 64 keys of K / half the columns of V
   static constexpr int NQ = STAGE_BYTES == 16384 ? 4 : 2;  // query slots
   static constexpr int NS = STAGE_BYTES == 16384 ? 6 : 5;
-  // TMEM: S of block b at 128 b, its accumulator at TM_O + D b.  Head size 128 has no room for P but over S; head size 64
-  // keeps it apart, so that the next S can be computed as soon as the present one is in registers
-  static constexpr bool SEP_P = D == 64;
-  static constexpr uint32_t TM_O = 256, TM_P = 384;
+  // TMEM: one S for both blocks in turn, P of block b at TM_P + 64 b, its accumulator at TM_O + D b
+  static constexpr uint32_t TM_S = 0, TM_P = 128, TM_O = 256;
   static constexpr int CODE = PAIR ? 200 : 100;            // wait codes in the status word
 };
 
@@ -53,7 +57,7 @@ struct __align__(16) Misc2 {
   uint64_t kv_full[MAX_NS], kv_free[MAX_NS];
   uint64_t s_full[2], o_full[2], t_full[2];
   uint64_t p_half[2], p_full[2], o_free[2], t_free[2];
-  uint64_t s_read[2], pv_done[2];            // head size 64: S is in registers / P V of a tile has run
+  uint64_t s_read, pv_done[2];               // S is in registers / P V of a tile has run
   uint64_t lm_full[2], lm_free[2];
   uint64_t d_full[NDESC], d_free[NDESC];
   uint64_t item_full, item_free;             // work items from the leader's producer to its peer's
@@ -162,11 +166,12 @@ __device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool
     mbar_init(&mi.s_full[b], 1); mbar_init(&mi.o_full[b], 1); mbar_init(&mi.t_full[b], 1);
     mbar_init(&mi.p_half[b], 4 * N); mbar_init(&mi.p_full[b], 4 * N); // 4 softmax warps of the block in each CTA
     mbar_init(&mi.o_free[b], 4 * N); mbar_init(&mi.t_free[b], 8 * N); // epilogue warps / softmax warps of the CTAs
-    mbar_init(&mi.s_read[b], 4); mbar_init(&mi.pv_done[b], 1);
+    mbar_init(&mi.pv_done[b], 1);
     mbar_init(&mi.lm_full[b], 4); mbar_init(&mi.lm_free[b], 4);
   }
   for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 13 : 12); }   // softmax and epilogue warps, issuer
   mbar_init(&mi.item_full, 1); mbar_init(&mi.item_free, 1);
+  mbar_init(&mi.s_read, 4 * N);
   mbar_init(&mi.lse_rdy, 4 * N);
   mbar_init(&mi.mma_done, 1);
   mi.left[0] = mi.left[1] = 0;
@@ -306,7 +311,7 @@ template <class C>
 struct Issuer {
   const Ctx2& cx;
   uint32_t ring_u32, q_u32;
-  uint32_t nd = 0, kv = 0, nq = 0, np[2] = {0, 0}, no[2] = {0, 0};   // descriptors, ring, query slots, tiles and blocks done
+  uint32_t nd = 0, kv = 0, nq = 0, ns = 0, np[2] = {0, 0}, no[2] = {0, 0};   // descriptors, ring, query slots, uses of S, tiles and blocks done
   uint32_t qa[2] = {0, 0};                                           // query operands of the two blocks in work
   __device__ __forceinline__ explicit Issuer(const Ctx2& c) : cx(c), ring_u32(smem_u32(c.ring)), q_u32(smem_u32(c.sQ)) {}
   // operand of ring use i, once its copy has landed
@@ -321,20 +326,22 @@ struct Issuer {
     ++nq;
     return q;
   }
-  // S of block b = Q K^T
+  // S = Q K^T for block b, once the S before it is in registers
   __device__ __forceinline__ void qk(int b, uint32_t k_smem) {
     constexpr uint32_t idesc = make_idesc_bf16_f32(TILE * C::NCTA, TILE, false, false);
+    WAIT2S(&cx.mi->s_read, free_par(ns), W2_SREAD);
+    ++ns;
     tc_fence_after_sync();
-    if constexpr (C::PAIR) mma_ss_pair_k128<true>(cx.tmem + b * 128, qa[b], k_smem, idesc);
-    else if constexpr (C::D == 128) mma_ss_k128(cx.tmem + b * 128, qa[b], k_smem, idesc);
-    else mma_ss_k64(cx.tmem + b * 128, qa[b], k_smem, idesc);
+    if constexpr (C::PAIR) mma_ss_pair_k128<true>(cx.tmem + C::TM_S, qa[b], k_smem, idesc);
+    else if constexpr (C::D == 128) mma_ss_k128(cx.tmem + C::TM_S, qa[b], k_smem, idesc);
+    else mma_ss_k64(cx.tmem + C::TM_S, qa[b], k_smem, idesc);
     commit<C>(&cx.mi->s_full[b]);
   }
   // O of block b += P V of a tile, in two halves as P arrives
   __device__ __forceinline__ void pv(int b, uint32_t v_smem, bool first, bool last) {
     Misc2& mi = *cx.mi;
     constexpr uint32_t idesc = make_idesc_bf16_f32(TILE * C::NCTA, C::D, false, true);
-    const uint32_t tO = cx.tmem + C::TM_O + b * C::D, tP = C::SEP_P ? cx.tmem + C::TM_P + b * 64 : cx.tmem + b * 128;
+    const uint32_t tO = cx.tmem + C::TM_O + b * C::D, tP = cx.tmem + C::TM_P + b * 64;
     if (first) { WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE); ++no[b]; }       // accumulator of the previous block read out
     WAIT2S(&mi.p_half[b], full_par(np[b]), W2_PHALF);                                // keys 0..63 of P
     tc_fence_after_sync();
@@ -343,10 +350,9 @@ struct Issuer {
     ++np[b];
     tc_fence_after_sync();
     mma_ts_k64<C::PAIR>(tO, tP + 32, v_smem + 8192, idesc, true);
-    if (C::SEP_P) commit<C>(&mi.pv_done[b]);
+    commit<C>(&mi.pv_done[b]);
     if (last) commit<C>(&mi.o_full[b]);
   }
-  __device__ __forceinline__ void wait_s_read(int b) { WAIT2S(&cx.mi->s_read[b], full_par(np[b]), W2_SREAD); }
 };
 
 // ------------------------------------------------------------------ softmax warps: hooks of softmax_tile for block b
@@ -357,14 +363,10 @@ struct Hooks {
   uint64_t* pv_done;
   uint32_t tiles;                                            // tiles of this block before the present one
   __device__ __forceinline__ Hooks(const Ctx2& c, int b)
-      : cx(c), p_half(in_cta<C>(&c.mi->p_half[b], 0)), p_full(in_cta<C>(&c.mi->p_full[b], 0)), s_read(in_cta<C>(&c.mi->s_read[b], 0)),
+      : cx(c), p_half(in_cta<C>(&c.mi->p_half[b], 0)), p_full(in_cta<C>(&c.mi->p_full[b], 0)), s_read(in_cta<C>(&c.mi->s_read, 0)),
         pv_done(&c.mi->pv_done[b]), tiles(0) {}
-  __device__ __forceinline__ void on_read() const { if (C::SEP_P) warp_arrive_leader(s_read); }
-  // P over S: S of this tile was issued after P V of the tile before, and P overwrites S, which is in registers
-  __device__ __forceinline__ void before_p() const {
-    if (C::SEP_P && tiles > 0) { WAIT2S(pv_done, full_par(tiles - 1), W2_PV); tc_fence_after_sync(); }
-  }
-  __device__ __forceinline__ void before_rescale() const { before_p(); }
+  __device__ __forceinline__ void on_read() const { warp_arrive_leader(s_read); }
+  __device__ __forceinline__ void before_p() const { WAIT2S(pv_done, free_par(tiles), W2_PV); tc_fence_after_sync(); }
   __device__ __forceinline__ void on_half() const { warp_arrive_leader(p_half); }
   __device__ __forceinline__ void on_full() const { warp_arrive_leader(p_full); }
 };

@@ -12,10 +12,10 @@
 // count.  Queries arrive rotated.  Small batches split the keys; the splits' fp32 partial results are merged
 // by a second kernel.
 //
-// What bounds it: many sequences, the power cap and then the tile's softmax (tensor and MUFU pipes 54 % busy, DRAM 43 % of
-// its peak): 64 sequences of 64 queries over 16384 entries, 32/8 heads take 1.02 ms from an idle GPU and 1.29 ms in a loop, as
-// with one block per CTA before.  One sequence: latencies, 24 K of 44 K cycles in the tiles of an item, 5 K writing its partial rows, the rest
-// cold code, setup and exit: 54.8 -> 36.7 us (with the rotation and the merge).
+// What bounds it: many sequences, the power cap and then the tile's softmax (2048 of some 2700 cycles a step on the MUFU pipe): 64
+// sequences of 64 queries over 16384 entries, 32/8 heads 1.23 -> 1.17 ms in a loop with one S for both blocks in turn (pc_flash.cuh).  One
+// sequence: latencies, half of the cycles in the tiles of an item, the rest writing its partial rows, cold code, setup and
+// exit: 34.6 -> 33.0 us (with the rotation and the merge).
 #include "pc_attn.h"
 #include "pc_flash.cuh"
 #include "pc_kernels.h"
@@ -154,13 +154,9 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             for (int t = 0; t < n; ++t) {
               const int b = t & 1;
               const bool more = t + 2 < n;
-              if (C::SEP_P) {                                                // the next S as soon as the present one is in registers
-                is.wait_s_read(b);
-                if (more) { is.qk(b, is.wait_kv(is.kv + 1)); is.free_kv(is.kv + 1); }
-              }
+              if (more) { is.qk(b, is.wait_kv(is.kv + 1)); is.free_kv(is.kv + 1); }
               is.pv(b, is.wait_kv(is.kv), t < 2, !more);
               is.free_kv(is.kv);
-              if (!C::SEP_P && more) { is.qk(b, is.wait_kv(is.kv + 1)); is.free_kv(is.kv + 1); }
               is.kv += more ? 2 : 1;
             }
           } else {
@@ -170,23 +166,15 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             is.free_kv(is.kv++);
             for (int t = 0; t < n; ++t) {
               const bool more = t + 1 < n;
-              if constexpr (C::SEP_P) {
-                uint32_t k_u32 = 0;
-                if (more) k_u32 = is.wait_kv(is.kv + 1);
-                for (int b = 0; b < 2; ++b)
-                  if (d.n[b] > 0) { is.wait_s_read(b); if (more) is.qk(b, k_u32); }
-                if (more) is.free_kv(is.kv + 1);
-                const uint32_t v_u32 = is.wait_kv(is.kv);
-                for (int b = 0; b < 2; ++b) if (d.n[b] > 0) is.pv(b, v_u32, t == 0, !more);
-              } else {
-                const uint32_t v_u32 = is.wait_kv(is.kv);
-                for (int b = 0; b < 2; ++b) {
-                  if (d.n[b] == 0) continue;
-                  is.pv(b, v_u32, t == 0, !more);
-                  if (more) is.qk(b, is.wait_kv(is.kv + 1));
-                }
-                if (more) is.free_kv(is.kv + 1);
+              uint32_t k_u32 = 0;
+              if (more) k_u32 = is.wait_kv(is.kv + 1);
+              const uint32_t v_u32 = is.wait_kv(is.kv);
+              for (int b = 0; b < 2; ++b) {
+                if (d.n[b] == 0) continue;
+                if (more) is.qk(b, k_u32);
+                is.pv(b, v_u32, t == 0, !more);
               }
+              if (more) is.free_kv(is.kv + 1);
               is.free_kv(is.kv);
               is.kv += more ? 2 : 1;
             }
@@ -288,8 +276,7 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     const int b = warp >> 2;
     const int r = tid & 127, wi = r % w;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tS = cx.tmem + b * 128 + lane_sel, tO = cx.tmem + C::TM_O + b * D + lane_sel;
-    const uint32_t tP = C::SEP_P ? cx.tmem + C::TM_P + b * 64 + lane_sel : tS;
+    const uint32_t tS = cx.tmem + C::TM_S + lane_sel, tP = cx.tmem + C::TM_P + b * 64 + lane_sel, tO = cx.tmem + C::TM_O + b * D + lane_sel;
     const float scale_log2 = prm.scale_log2;
     Hooks<C> hk(cx, b);
     uint32_t nd = 0, n_s = 0, n_blk = 0;

@@ -6,18 +6,17 @@
 // Head size 128 runs on CTA pairs (cluster of two, tcgen05 cta_group::2): four blocks share the tiles, every
 // 128-key tile is split between the two shared memories (each CTA stages 64 keys of K and 64 head-dim columns of V) and
 // one MMA of M = 256 feeds both SMs.  A single CTA's 128 x 128 x 128 product reads 128 bytes a cycle, all that shared
-// memory gives; on a pair it reads 96, and the L2 traffic is halved.  TMEM of a CTA: S of both blocks with P over
-// its first half (128 columns each) and both accumulators (128 each).
-// Head size 64 runs on single CTAs: its products are half as long, the softmax is what bounds it, and there is room in
-// TMEM for P beside S, so the next tile's S is computed as soon as the present one is in registers.
+// memory gives; on a pair it reads 96, and the L2 traffic is halved.
+// Head size 64 runs on single CTAs: its products are half as long, and the softmax is what bounds it.
 //
-// Roles, rings and barriers: pc_flash.cuh.
+// Roles, rings, barriers and the tensor memory: pc_flash.cuh.
 //
-// What bounds it: the board's power cap (1000 W) in any loop of these calls, so energy a tile; tensor and MUFU pipes are
-// both 55 % busy.  Measured in a loop, whole call, against one block per CTA of a pair (d = 128, even G) and a single-CTA kernel
-// without these roles (the rest): 128K tokens in chunks of 8192, 32/8 heads 9.6 -> 8.4 ms (the kernel from an idle GPU
-// 8.12 -> 7.17 ms = 1227 TFLOP/s); 32/32 heads, chunks of 4096 6.1 -> 5.5 ms; 24/8 heads, ragged 1.70 -> 1.41 ms; head size
-// 64, 32K tokens 1.27 -> 0.93 ms.  A third build, head size 128 on single CTAs, takes short chunks of odd groups (launch_prefill_t).
+// What bounds it: the board's power cap (1000 W) in any loop of these calls, so energy a tile, and beside it the MUFU pipe: a step
+// (a key tile for both blocks of a CTA) takes some 2700 cycles, of which the exponentials keep that pipe busy for 2048, the
+// products the tensor cores as long (head size 64: half as long).  Measured in a loop, whole call, with an S of each block
+// under P (3300 cycles a step) -> with one S for both in turn: 128K tokens in chunks of 8192, 32/8 heads 8.39 -> 7.89 ms; 32/32
+// heads, chunks of 4096 5.49 -> 5.31 ms; 24/8 heads, ragged 1.39 -> 1.33 ms; head size 64, 32K tokens 0.898 -> 0.886 ms.
+// A third build, head size 128 on single CTAs, takes short chunks of odd groups (launch_prefill_t).
 //
 // Window scores: the unit that runs the last query tiles of a (chunk, kv-head) group then sweeps the keys once more
 // with the transposed product K_j Qw^T (the CTAs of a pair take alternate key tiles; keys on TMEM lanes, window
@@ -276,28 +275,15 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 if (j + 1 < nb) is.qk(b, k_u32);
                 else if (j + 1 == n && more && nx.n[b] > 0) first_qk(b, k_u32);
               };
-              if constexpr (!C::SEP_P) {
-                // per block: P V, then the next S over P; the pipe runs them in order
-                const uint32_t v_u32 = is.wait_kv(is.kv);
-                if (j < n0) is.pv(0, v_u32, j == 0, j == n0 - 1);
-                look_ahead();
-                next_s(0, n0);
-                is.pv(1, v_u32, j == 0, j == n - 1);
-                next_s(1, n);
-              } else {
-                // next S as soon as the present one is in registers, then P V
-                look_ahead();
-                if (j < n0) is.wait_s_read(0);
-                next_s(0, n0);
-                is.wait_s_read(1);
-                next_s(1, n);
-                if (more) is.free_kv(is.kv + 1);
-                const uint32_t v_u32 = is.wait_kv(is.kv);
-                if (j < n0) is.pv(0, v_u32, j == 0, j == n0 - 1);
-                is.pv(1, v_u32, j == 0, j == n - 1);
-              }
+              // per block: the next S, then P V of the present tile; the two blocks take turns on S
+              look_ahead();
+              next_s(0, n0);
+              const uint32_t v_u32 = is.wait_kv(is.kv);
+              if (j < n0) is.pv(0, v_u32, j == 0, j == n0 - 1);
+              next_s(1, n);
+              if (more) is.free_kv(is.kv + 1);
+              is.pv(1, v_u32, j == 0, j == n - 1);
               is.free_kv(is.kv);
-              if (!C::SEP_P && more) is.free_kv(is.kv + 1);
               is.kv += more ? 2 : 1;
             }
             primed = PRIMES && nx.kind == KIND_FLASH;
@@ -428,8 +414,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const int b = warp >> 2;
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tS = cx.tmem + b * 128 + lane_sel, tO = cx.tmem + C::TM_O + b * D + lane_sel;
-    const uint32_t tP = C::SEP_P ? cx.tmem + C::TM_P + b * 64 + lane_sel : tS;
+    const uint32_t tS = cx.tmem + C::TM_S + lane_sel, tP = cx.tmem + C::TM_P + b * 64 + lane_sel, tO = cx.tmem + C::TM_O + b * D + lane_sel;
     const float scale_log2 = prm.scale_log2;
     Hooks<C> hk(cx, b);
     uint32_t nd = 0, n_s = 0, n_blk = 0, nq = 0, nt = 0, n_lse = 0;

@@ -60,42 +60,39 @@ __device__ __forceinline__ void rescale_rows(uint32_t o_taddr, float alpha) {
   }
 }
 
-// One 128-key tile.  The exponentials of the first 64 keys are taken against the reference maximum of the tiles BEFORE
-// this one, while the maximum of this tile is found on the ALU pipe beside them; they are stored only when that maximum
+// One 128-key tile.  The logits are taken into registers at once and their columns given back (on_read), so that the next
+// logits are computed meanwhile.  The exponentials of the first 64 keys are taken against the reference maximum of the tiles BEFORE
+// this one, while the maximum of this tile is found on the ALU pipe beside them; they are published only when that maximum
 // is known not to exceed the reference by more than 2^8 in any row of the warp (otherwise the reference is raised, the
 // accumulator rescaled and the first half repeated).  So the row maximum is off the path from logits to exponentials.
 // GEN: tiles with masked columns (columns >= vis; vis <= 0: all) and the first tile of a block; the tiles between
 // run straight-line code (the branches around the masks cost 300 of 1240 cycles).
-// Hooks: on_read() - all logits are in registers; before_rescale() - called before the accumulator is touched;
-// before_p() - called before probabilities are stored at p_taddr (64 columns); on_half(), on_full() - keys 0..63 / all
-// keys of P are in TMEM.
+// Hooks: on_read() - all logits are in registers; before_p() - called before the accumulator is touched and before
+// probabilities are stored at p_taddr (64 columns); on_half(), on_full() - keys 0..63 / all keys of P are in TMEM.
 template <int D, bool GEN, class Hooks>
 __device__ __forceinline__ void softmax_tile(uint32_t s_taddr, uint32_t p_taddr, uint32_t o_taddr, int vis, bool first_tile,
                                              float scale_log2, RowState& st, const Hooks& hk) {
   const uint64_t scale2 = dup2(scale_log2);
   uint64_t sum2[2] = {0ull, 0ull};
-  uint32_t pk[2][16], c2[32], c3[32];
-  float mx;
-  {
-    uint32_t c0[32], c1[32];
-    tmem_ld32(s_taddr, c0);
-    tmem_ld32(s_taddr + 32, c1);
-    tmem_wait_ld();
-    loaded(c0); loaded(c1);
-    tmem_ld32(s_taddr + 64, c2);
-    tmem_ld32(s_taddr + 96, c3);
-    if (GEN) { mask32(c0, 0, vis); mask32(c1, 32, vis); }
-    const uint64_t negm2 = dup2(st.m == -INFINITY ? 0.0f : -st.m);  // nothing visible so far: exp2(-inf) = 0
-    mx = fmaxf(max32(c0), max32(c1));
-    if (!GEN || !first_tile) {
-      exps32(c0, scale2, negm2, sum2, pk[0]);
-      exps32(c1, scale2, negm2, sum2, pk[1]);
-    }
-  }
+  uint32_t pk[16], c0[32], c1[32], c2[32], c3[32];
+  tmem_ld32(s_taddr, c0);
+  tmem_ld32(s_taddr + 32, c1);
+  tmem_ld32(s_taddr + 64, c2);
+  tmem_ld32(s_taddr + 96, c3);
   tmem_wait_ld();
-  loaded(c2); loaded(c3);
-  if (GEN) { mask32(c2, 64, vis); mask32(c3, 96, vis); }
-  mx = fmaxf(mx, fmaxf(max32(c2), max32(c3))) * scale_log2;
+  loaded(c0); loaded(c1); loaded(c2); loaded(c3);
+  hk.on_read();
+  if (GEN) { mask32(c0, 0, vis); mask32(c1, 32, vis); mask32(c2, 64, vis); mask32(c3, 96, vis); }
+  auto first_half = [&]() {
+    const uint64_t negm2 = dup2(st.m == -INFINITY ? 0.0f : -st.m);  // nothing visible so far: exp2(-inf) = 0
+    exps32(c0, scale2, negm2, sum2, pk);
+    tmem_st16(p_taddr, pk);
+    exps32(c1, scale2, negm2, sum2, pk);
+    tmem_st16(p_taddr + 16, pk);
+  };
+  hk.before_p();
+  if (!GEN || !first_tile) first_half();
+  const float mx = fmaxf(fmaxf(max32(c0), max32(c1)), fmaxf(max32(c2), max32(c3))) * scale_log2;
   const bool raise = mx > st.m + LAZY_RESCALE_LOG2 || (GEN && first_tile);
   if (__any_sync(0xFFFFFFFFu, raise)) {                            // rare; warp-uniform: each warp owns its 32 lanes of O
     float alpha = 1.0f;
@@ -106,31 +103,19 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_taddr, uint32_t p_taddr,
       st.l *= alpha;
     }
     if (!GEN || !first_tile) {
-      hk.before_rescale();
       rescale_rows<D>(o_taddr, alpha);
+      tmem_wait_st();                                              // the first half is about to be stored again
     }
-    uint32_t c0[32], c1[32];
-    tmem_ld32(s_taddr, c0);
-    tmem_ld32(s_taddr + 32, c1);
-    tmem_wait_ld();
-    loaded(c0); loaded(c1);
-    if (GEN) { mask32(c0, 0, vis); mask32(c1, 32, vis); }
-    const uint64_t negm2 = dup2(st.m == -INFINITY ? 0.0f : -st.m);
     sum2[0] = sum2[1] = 0ull;
-    exps32(c0, scale2, negm2, sum2, pk[0]);
-    exps32(c1, scale2, negm2, sum2, pk[1]);
+    first_half();
   }
-  hk.on_read();
-  hk.before_p();
-  tmem_st16(p_taddr, pk[0]);
-  tmem_st16(p_taddr + 16, pk[1]);
   tmem_wait_st();
   hk.on_half();
   const uint64_t negm2 = dup2(st.m == -INFINITY ? 0.0f : -st.m);
-  exps32(c2, scale2, negm2, sum2, pk[0]);
-  tmem_st16(p_taddr + 32, pk[0]);
-  exps32(c3, scale2, negm2, sum2, pk[1]);
-  tmem_st16(p_taddr + 48, pk[1]);
+  exps32(c2, scale2, negm2, sum2, pk);
+  tmem_st16(p_taddr + 32, pk);
+  exps32(c3, scale2, negm2, sum2, pk);
+  tmem_st16(p_taddr + 48, pk);
   tmem_wait_st();
   hk.on_full();
   float a0, a1;
