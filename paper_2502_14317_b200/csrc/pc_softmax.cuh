@@ -5,6 +5,7 @@
 namespace pc {
 
 constexpr float LAZY_RESCALE_LOG2 = 8.0f;      // the reference maximum is raised only when it grows by more than 2^8
+constexpr float MAX_HALF_SUM = 256.0f;         // 2^8, see softmax_tile
 // All exponentials run on the MUFU pipe (ex2), 1024 cycles a tile and warp.  Evaluating every fourth pair as a polynomial on
 // the FMA pipe took a seventh off a tile's cycles and made every workload slower: these kernels run at the board's
 // power cap, and twenty FMA-pipe instructions cost more energy than the two ex2 they replace (128K tokens, 32/8 heads
@@ -62,9 +63,12 @@ __device__ __forceinline__ void rescale_rows(uint32_t o_taddr, float alpha) {
 
 // One 128-key tile.  The logits are taken into registers at once and their columns given back (on_read), so that the next
 // logits are computed meanwhile.  The exponentials of the first 64 keys are taken against the reference maximum of the tiles BEFORE
-// this one, while the maximum of this tile is found on the ALU pipe beside them; they are published only when that maximum
-// is known not to exceed the reference by more than 2^8 in any row of the warp (otherwise the reference is raised, the
-// accumulator rescaled and the first half repeated).  So the row maximum is off the path from logits to exponentials.
+// this one and published only when none of them, and no logit of the other half, exceeds it by more than 2^8 in any row of the
+// warp (otherwise the reference is raised to the maximum, the accumulator rescaled and the first half repeated).  Of the first
+// half the sum tells, which is needed anyway: while it is at most 2^8, so is every term; if it is more, or no number, the
+// maximum is looked up.  Of the other half the maximum is found beside the exponentials.  (With the maximum of both halves, in
+// a loop: 128K tokens, 32/8 heads 7894 -> 7839 us, 32/32 heads 5307 -> 5265, head size 64, 32K tokens 886 -> 874.  The second
+// half by its sum as well, with a barrier for the first half's P V: 7842, 5283, 888.)
 // GEN: tiles with masked columns (columns >= vis; vis <= 0: all) and the first tile of a block; the tiles between
 // run straight-line code (the branches around the masks cost 300 of 1240 cycles).
 // Hooks: on_read() - all logits are in registers; before_p() - called before the accumulator is touched and before
@@ -91,10 +95,17 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_taddr, uint32_t p_taddr,
     tmem_st16(p_taddr + 16, pk);
   };
   hk.before_p();
-  if (!GEN || !first_tile) first_half();
-  const float mx = fmaxf(fmaxf(max32(c0), max32(c1)), fmaxf(max32(c2), max32(c3))) * scale_log2;
-  const bool raise = mx > st.m + LAZY_RESCALE_LOG2 || (GEN && first_tile);
+  float a0, a1, half_sum = 0.0f;
+  bool raise = GEN && first_tile;
+  if (!GEN || !first_tile) {
+    first_half();
+    unpack_f32x2(add_f32x2(sum2[0], sum2[1]), a0, a1);
+    half_sum = a0 + a1;
+    raise = !(half_sum <= (st.m == -INFINITY ? -1.0f : MAX_HALF_SUM));
+  }
+  raise |= fmaxf(max32(c2), max32(c3)) * scale_log2 > st.m + LAZY_RESCALE_LOG2;
   if (__any_sync(0xFFFFFFFFu, raise)) {                            // rare; warp-uniform: each warp owns its 32 lanes of O
+    const float mx = fmaxf(fmaxf(max32(c0), max32(c1)), fmaxf(max32(c2), max32(c3))) * scale_log2;
     float alpha = 1.0f;
     if (raise) {
       const float m_new = fmaxf(st.m, mx);
@@ -108,9 +119,13 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_taddr, uint32_t p_taddr,
     }
     sum2[0] = sum2[1] = 0ull;
     first_half();
+    unpack_f32x2(add_f32x2(sum2[0], sum2[1]), a0, a1);
+    half_sum = a0 + a1;
   }
   tmem_wait_st();
   hk.on_half();
+  st.l += half_sum;
+  sum2[0] = sum2[1] = 0ull;
   const uint64_t negm2 = dup2(st.m == -INFINITY ? 0.0f : -st.m);
   exps32(c2, scale2, negm2, sum2, pk);
   tmem_st16(p_taddr + 32, pk);
@@ -118,7 +133,6 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_taddr, uint32_t p_taddr,
   tmem_st16(p_taddr + 48, pk);
   tmem_wait_st();
   hk.on_full();
-  float a0, a1;
   unpack_f32x2(add_f32x2(sum2[0], sum2[1]), a0, a1);
   st.l += a0 + a1;
 }

@@ -130,6 +130,22 @@ def test_growing_logits_rescale_path(d):
     _run_and_compare(bits[0], bits[1], bits[2], w, 10000.0, sharp=True)
 
 
+@pytest.mark.parametrize("d,rise", [(64, 2.0), (64, 6.0), (128, 4.0), (128, 6.0)])
+def test_logits_that_rise_less_than_the_threshold_a_tile(d, rise):
+    """Every key tile lies `rise` (in log2) above the one before: no logit exceeds the reference maximum by 2^8, but 64
+    probabilities of 2^rise sum up to more than 2^8 (rise = 2: about as much, so that some rows of a warp are raised and others are
+    not).  The rise goes through the slowest pair, which the rotation leaves as it is."""
+    rng = np.random.default_rng(31 + d)
+    C, L, Hq, Hkv, w = 1, 900, 4, 2, 32
+    q = 0.3 * rng.standard_normal((C, L, Hq, d)).astype(np.float32)
+    k = 0.3 * rng.standard_normal((C, L, Hkv, d)).astype(np.float32)
+    v = rng.standard_normal((C, L, Hkv, d)).astype(np.float32)
+    q[..., d // 2 - 1] = 8.0
+    k[..., d // 2 - 1] = (np.arange(L) // 128 * rise * np.sqrt(d) / (8.0 * np.log2(np.e)))[None, :, None]
+    bits = [pc_inputs.f32_to_bf16_bits(x) for x in (q, k, v)]
+    _run_and_compare(bits[0], bits[1], bits[2], w, 1.0e9, sharp=True)
+
+
 @pytest.mark.parametrize("Hq,Hkv", [(4, 2), (2, 2), (6, 2)])
 def test_growing_logits_many_tiles(Hq, Hkv):
     """The same stress over 13 key tiles, two chunks, even and odd group sizes: the softmax warpgroups and the TMEM
