@@ -319,6 +319,7 @@ struct Issuer {
     WAIT2S(&cx.mi->kv_full[i % C::NS], full_par(i / C::NS), W2_KVFULL);
     return ring_u32 + (i % C::NS) * C::STAGE_BYTES;
   }
+  __device__ __forceinline__ bool landed(uint32_t i) { return mbar_test_wait(&cx.mi->kv_full[i % C::NS], full_par(i / C::NS)); }
   __device__ __forceinline__ void free_kv(uint32_t i) { commit<C>(&cx.mi->kv_free[i % C::NS]); }
   __device__ __forceinline__ uint32_t wait_q() {
     WAIT2S(&cx.mi->q_full[nq % C::NQ], full_par(nq / C::NQ), W2_QFULL);

@@ -154,9 +154,16 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             for (int t = 0; t < n; ++t) {
               const int b = t & 1;
               const bool more = t + 2 < n;
-              if (more) { is.qk(b, is.wait_kv(is.kv + 1)); is.free_kv(is.kv + 1); }
+              // The next S before P V of the present tile.  On single CTAs of head size 128, which hold two and a half tiles, only
+              // where its keys are there: else the values' stage is given back first (us, always before / by that rule: 16 sequences of 12000
+              // entries, window of 16, 32/8 heads 158.9 / 156.2; 33 of 2000, window of 64, 32/32 heads 254.0 / 250.4; always after: 3 of 15000,
+              // window of 16, 28/4 heads 36.7, by the rule 35.3).
+              const bool early = more && (PAIR || D == 64 || is.landed(is.kv + 1));
+              auto next_s = [&]() { is.qk(b, is.wait_kv(is.kv + 1)); is.free_kv(is.kv + 1); };
+              if (early) next_s();
               is.pv(b, is.wait_kv(is.kv), t < 2, !more);
               is.free_kv(is.kv);
+              if (more && !early) next_s();
               is.kv += more ? 2 : 1;
             }
           } else {
