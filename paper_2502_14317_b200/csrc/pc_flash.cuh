@@ -3,8 +3,13 @@
 //
 // A CTA owns two 128-row query blocks A and B, one softmax warpgroup each; while the softmax of one runs the tensor
 // cores work for the other.  Warps (16): 0-3 softmax of block A, 4-7 softmax of block B (thread = query row = TMEM lane),
-// 8-11 epilogue (the softmax warps go straight on to the next block), 12 TMA producer, 13 issuer of all MMAs (of a
-// CTA pair: in the leader only), 14-15 idle.  Registers are dealt out by role: 184 / 80 / 64.
+// 8-11 epilogue (the softmax warps go straight on to the next block), 12 TMA producer, 13 issuer of S = Q K^T and of the score
+// sweeps, 14 issuer of O += P V (of a CTA pair: in the leader only), 15 idle.  Registers are dealt out by role.
+// The issuers are two because their waits have nothing to do with each other: S is due when the S before it has been read, P V
+// when P arrives.  One thread in a fixed order was busy for two thirds of a step and late for both.  In a loop, us, one thread / two (and the registers
+// below): 8 chunks of 8192, 32/8 heads 3924 / 3865, 8 of 4096, 32/32 heads 1346 / 1333, 4 of 1257, 32/32 heads 138.1 / 135.8, query window of
+// one sequence 33.2 / 31.6.
+// Keys and values have rings of their own, so that each of them is consumed by one issuer.
 //
 // Tensor memory, 512 columns: one S (128), P of both blocks (64 each), both accumulators (128 each).  The blocks take turns on
 // S: the softmax warps take a whole S into registers at once, and the product for the other block runs under their
@@ -21,8 +26,11 @@ namespace flash {
 
 constexpr int TILE = 128;
 constexpr int NT2 = 512;                     // threads per CTA
-constexpr int WARP_EPI = 8, WARP_PRODUCER = 12, WARP_MMA = 13;
-constexpr int REGS_SOFTMAX = 184, REGS_EPI = 80, REGS_SERVICE = 64;      // 128 * (2 * 184 + 80 + 64) = 64 K registers
+constexpr int WARP_EPI = 8, WARP_PRODUCER = 12, WARP_QK = 13, WARP_PV = 14;
+// registers by role, 128 * (2 * softmax + epilogue + service) = 64 K
+// (prefill, 8 chunks of 8192, 32/8 heads: softmax 184 3920 us, 192 3872, 200 3870 with spills in the other roles; over caches 184 619, 192 631)
+struct Regs { int softmax, epilogue, service; };
+constexpr Regs REGS_PREFILL = {192, 80, 48}, REGS_PARALLEL = {184, 80, 64};
 constexpr int NDESC = 4;                     // work descriptors in flight
 constexpr int MAX_NQ = 4, MAX_NS = 6;
 template <int D_, bool PAIR_>
@@ -32,16 +40,20 @@ struct Cfg {
   static constexpr int NCTA = PAIR ? 2 : 1;
   static constexpr int ATOMS = D / 64;
   static constexpr int Q_BYTES = TILE * D * 2;
-  static constexpr int STAGE_BYTES = TILE * D * 2 / NCTA;  // K/V ring: a tile, or of a pair 64 keys of K / half the columns of V
+  static constexpr int STAGE_BYTES = TILE * D * 2 / NCTA;  // K/V rings: a tile, or of a pair 64 keys of K / half the columns of V
   static constexpr int NQ = STAGE_BYTES == 16384 ? 4 : 2;  // query slots
-  static constexpr int NS = STAGE_BYTES == 16384 ? 6 : 5;
+  static constexpr int NS = STAGE_BYTES == 16384 ? 6 : 5;  // stages: even ones for keys, odd ones for values
+  static constexpr int NK = (NS + 1) / 2, NV = NS / 2;
   // TMEM: one S for both blocks in turn, P of block b at TM_P + 64 b, its accumulator at TM_O + D b
   static constexpr uint32_t TM_S = 0, TM_P = 128, TM_O = 256;
+  // pause of the issuers between two polls, ns.  us, 20 / 0: head size 64, 32K tokens 872 / 869, windows of 64 over 32 caches of 8192,
+  // 14/2 heads 113.0 / 111.3; head size 128 on pairs, windows of 64 over 32 caches of 16384, 32/8 heads 619 / 630
+  static constexpr unsigned ISSUER_NS = D == 64 ? 0 : 20;
   static constexpr int CODE = PAIR ? 200 : 100;            // wait codes in the status word
 };
 
 enum { W2_DESC = 1, W2_ITEM, W2_QFULL, W2_QFREE, W2_KVFULL, W2_KVFREE, W2_SFULL, W2_PHALF, W2_PFULL, W2_OFULL, W2_OFREE, W2_LM,
-       W2_LMFREE, W2_LSE, W2_TFULL, W2_TFREE, W2_SREAD, W2_PV };
+       W2_LMFREE, W2_LSE, W2_TFULL, W2_TFREE, W2_SREAD, W2_PV, W2_SWEEP };
 
 enum { KIND_DONE = 0, KIND_FLASH = 1, KIND_SWEEP = 2 };
 struct __align__(16) Desc {
@@ -62,6 +74,7 @@ struct __align__(16) Misc2 {
   uint64_t d_full[NDESC], d_free[NDESC];
   uint64_t item_full, item_free;             // work items from the leader's producer to its peer's
   uint64_t lse_rdy;
+  uint64_t sweep_go;                         // the accumulators have been read out: a score sweep may overwrite them
   uint64_t mma_done;
   Desc desc[NDESC];
   int left[2];                               // warps of the epilogue / the softmax that are through (leave_group)
@@ -92,8 +105,9 @@ struct Ctx2 {
   int* status;
 };
 
-// waits of the single-thread service roles (long pause between polls) / of the softmax and epilogue warps
+// waits of the single-thread service roles (long pause between polls) / of the issuers / of the softmax and epilogue warps
 #define WAIT2(bar, par, code) mbar_wait_ns<SERVICE_BACKOFF_NS>((bar), (par), cx.abort_flag, cx.status, C::CODE + (code))
+#define WAIT2I(bar, par, code) mbar_wait_ns<C::ISSUER_NS>((bar), (par), cx.abort_flag, cx.status, C::CODE + (code))
 #define WAIT2S(bar, par, code) mbar_wait((bar), (par), cx.abort_flag, cx.status, C::CODE + (code))
 
 __device__ __forceinline__ void warp_arrive(uint64_t* bar) {
@@ -169,11 +183,12 @@ __device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool
     mbar_init(&mi.pv_done[b], 1);
     mbar_init(&mi.lm_full[b], 4); mbar_init(&mi.lm_free[b], 4);
   }
-  for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 13 : 12); }   // softmax and epilogue warps, issuer
+  for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 14 : 12); }   // softmax and epilogue warps, issuers
   mbar_init(&mi.item_full, 1); mbar_init(&mi.item_free, 1);
   mbar_init(&mi.s_read, 4 * N);
   mbar_init(&mi.lse_rdy, 4 * N);
-  mbar_init(&mi.mma_done, 1);
+  mbar_init(&mi.sweep_go, 1);
+  mbar_init(&mi.mma_done, 2);
   mi.left[0] = mi.left[1] = 0;
   mi.abort_flag = 0;
   mi.wait_kcycles = wait_kcycles;
@@ -212,7 +227,7 @@ __device__ __forceinline__ void leave_group(int id, bool odd, int* left) {
 }
 
 // ------------------------------------------------------------------ producer
-struct Prod { uint32_t kv = 0, q = 0, d = 0, item = 0; };
+struct Prod { uint32_t k = 0, v = 0, q = 0, d = 0, item = 0; };
 template <class C>
 __device__ __forceinline__ void publish(const Ctx2& cx, Prod& p, const Desc& d, bool signal = true) {
   Misc2& mi = *cx.mi;
@@ -242,17 +257,23 @@ __device__ __forceinline__ int next_item(const Ctx2& cx, Prod& p, bool leader, i
   ++p.item;
   return item;
 }
-// expects a stage's bytes over both CTAs on the leader's barrier of the next ring stage; returns that barrier's address
+// stage of the n-th use of the key ring (V: of the value ring), and how often the stage has been used before
+template <class C, bool V>
+__device__ __forceinline__ int stage_of(uint32_t n) { return V ? 2 * (n % C::NV) + 1 : 2 * (n % C::NK); }
+template <class C, bool V>
+__device__ __forceinline__ uint32_t lap_of(uint32_t n) { return n / (V ? C::NV : C::NK); }
+// expects a stage's bytes over both CTAs on the leader's barrier of the ring's next stage; returns that barrier's address
 // for the copies and the stage's place; 0 once a wait has run out (no copy is issued into a ring that nobody drains)
-template <class C>
+template <class C, bool V>
 __device__ __forceinline__ uint32_t ring_stage(const Ctx2& cx, Prod& p, bool leader, uint8_t** dst) {
   Misc2& mi = *cx.mi;
   if (*cx.abort_flag) return 0;
-  const int s = p.kv % C::NS;
-  if (!WAIT2(&mi.kv_free[s], free_par(p.kv / C::NS), W2_KVFREE)) return 0;
+  uint32_t& n = V ? p.v : p.k;
+  const int s = stage_of<C, V>(n);
+  if (!WAIT2(&mi.kv_free[s], free_par((lap_of<C, V>(n))), W2_KVFREE)) return 0;
   if (leader) mbar_arrive_expect_tx(&mi.kv_full[s], C::NCTA * C::STAGE_BYTES);
   *dst = cx.ring + s * C::STAGE_BYTES;
-  ++p.kv;
+  ++n;
   return in_cta<C>(&mi.kv_full[s], 0);
 }
 
@@ -266,7 +287,7 @@ __device__ __forceinline__ void setup(Ctx2& cx, uint8_t* smem, int* status, int 
   cx.abort_flag = &mi.abort_flag;
   cx.status = status;
   if (threadIdx.x == 0) init_barriers2<C>(mi, wait_kcycles, leader);
-  if (threadIdx.x / 32 == WARP_MMA) { if constexpr (C::PAIR) tmem_alloc_pair(&mi.tmem_base, 512); else tmem_alloc(&mi.tmem_base, 512); }
+  if (threadIdx.x / 32 == WARP_QK) { if constexpr (C::PAIR) tmem_alloc_pair(&mi.tmem_base, 512); else tmem_alloc(&mi.tmem_base, 512); }
   tc_fence_before_sync();
   __syncthreads();
   if constexpr (C::PAIR) cluster_sync_all();             // both CTAs' barriers exist before any remote arrive
@@ -280,8 +301,8 @@ __device__ __forceinline__ void teardown(const Ctx2& cx) {
   tc_fence_before_sync();
   __syncthreads();
   if constexpr (C::PAIR) cluster_sync_all();
-  if (threadIdx.x / 32 == WARP_MMA) {
-    // no tensor-core operation may still be running when its accumulators are freed: the issuer ended with a
+  if (threadIdx.x / 32 == WARP_QK) {
+    // no tensor-core operation may still be running when its accumulators are freed: each issuer ended with a
     // commit to mma_done (an arrival in both CTAs of a pair).  Immediate in a clean run; after an abort this is what
     // makes the exit safe.  The wait ignores the abort flag and is bounded.
     mbar_wait_drain(&cx.mi->mma_done, 0, cx.abort_flag);
@@ -300,55 +321,74 @@ __device__ __forceinline__ void drain_copies(const Ctx2& cx, const Prod& p, bool
   Misc2& mi = *cx.mi;
   if (!*cx.abort_flag) return;
   if (leader) {
-    for (uint32_t i = (p.kv > C::NS ? p.kv - C::NS : 0); i < p.kv; ++i) mbar_wait_drain(&mi.kv_full[i % C::NS], full_par(i / C::NS), cx.abort_flag);
+    for (uint32_t i = (p.k > C::NK ? p.k - C::NK : 0); i < p.k; ++i) mbar_wait_drain(&mi.kv_full[stage_of<C, false>(i)], full_par(lap_of<C, false>(i)), cx.abort_flag);
+    for (uint32_t i = (p.v > C::NV ? p.v - C::NV : 0); i < p.v; ++i) mbar_wait_drain(&mi.kv_full[stage_of<C, true>(i)], full_par(lap_of<C, true>(i)), cx.abort_flag);
     for (uint32_t i = (p.q > C::NQ ? p.q - C::NQ : 0); i < p.q; ++i) mbar_wait_drain(&mi.q_full[i % C::NQ], full_par(i / C::NQ), cx.abort_flag);
   }
   abort_grace_pause(cx.abort_flag);
 }
 
-// ------------------------------------------------------------------ issuer (one elected thread; of a pair: of the leader CTA)
+// ------------------------------------------------------------------ issuers (one elected thread each; of a pair: of the leader CTA)
+// operand of the n-th use of a ring, once its copy has landed / the stage is free once what this thread has issued has run
+template <class C, bool V>
+__device__ __forceinline__ uint32_t wait_stage(const Ctx2& cx, uint32_t n) {
+  const int s = stage_of<C, V>(n);
+  WAIT2I(&cx.mi->kv_full[s], full_par((lap_of<C, V>(n))), W2_KVFULL);
+  return smem_u32(cx.ring) + s * C::STAGE_BYTES;
+}
+template <class C, bool V>
+__device__ __forceinline__ void free_stage(const Ctx2& cx, uint32_t n) { commit<C>(&cx.mi->kv_free[stage_of<C, V>(n)]); }
+
 template <class C>
-struct Issuer {
+struct IssuerQK {
   const Ctx2& cx;
-  uint32_t ring_u32, q_u32;
-  uint32_t nd = 0, kv = 0, nq = 0, ns = 0, np[2] = {0, 0}, no[2] = {0, 0};   // descriptors, ring, query slots, uses of S, tiles and blocks done
+  uint32_t nd = 0, k = 0, nq = 0, ns = 0;                            // descriptors, key ring, query slots, uses of S
   uint32_t qa[2] = {0, 0};                                           // query operands of the two blocks in work
-  __device__ __forceinline__ explicit Issuer(const Ctx2& c) : cx(c), ring_u32(smem_u32(c.ring)), q_u32(smem_u32(c.sQ)) {}
-  // operand of ring use i, once its copy has landed
-  __device__ __forceinline__ uint32_t wait_kv(uint32_t i) {
-    WAIT2S(&cx.mi->kv_full[i % C::NS], full_par(i / C::NS), W2_KVFULL);
-    return ring_u32 + (i % C::NS) * C::STAGE_BYTES;
-  }
-  __device__ __forceinline__ bool landed(uint32_t i) { return mbar_test_wait(&cx.mi->kv_full[i % C::NS], full_par(i / C::NS)); }
-  __device__ __forceinline__ void free_kv(uint32_t i) { commit<C>(&cx.mi->kv_free[i % C::NS]); }
+  __device__ __forceinline__ explicit IssuerQK(const Ctx2& c) : cx(c) {}
   __device__ __forceinline__ uint32_t wait_q() {
-    WAIT2S(&cx.mi->q_full[nq % C::NQ], full_par(nq / C::NQ), W2_QFULL);
-    const uint32_t q = q_u32 + (nq % C::NQ) * C::Q_BYTES;
+    WAIT2I(&cx.mi->q_full[nq % C::NQ], full_par(nq / C::NQ), W2_QFULL);
+    const uint32_t q = smem_u32(cx.sQ) + (nq % C::NQ) * C::Q_BYTES;
     ++nq;
     return q;
   }
+  __device__ __forceinline__ uint32_t wait_k() { return wait_stage<C, false>(cx, k); }
+  __device__ __forceinline__ void free_k() { free_stage<C, false>(cx, k++); }
   // S = Q K^T for block b, once the S before it is in registers
   __device__ __forceinline__ void qk(int b, uint32_t k_smem) {
     constexpr uint32_t idesc = make_idesc_bf16_f32(TILE * C::NCTA, TILE, false, false);
-    WAIT2S(&cx.mi->s_read, free_par(ns), W2_SREAD);
+    const uint32_t q_smem = b ? qa[1] : qa[0];
+    WAIT2I(&cx.mi->s_read, free_par(ns), W2_SREAD);
     ++ns;
     tc_fence_after_sync();
-    if constexpr (C::PAIR) mma_ss_pair_k128<true>(cx.tmem + C::TM_S, qa[b], k_smem, idesc);
-    else if constexpr (C::D == 128) mma_ss_k128(cx.tmem + C::TM_S, qa[b], k_smem, idesc);
-    else mma_ss_k64(cx.tmem + C::TM_S, qa[b], k_smem, idesc);
+    if constexpr (C::PAIR) mma_ss_pair_k128<true>(cx.tmem + C::TM_S, q_smem, k_smem, idesc);
+    else if constexpr (C::D == 128) mma_ss_k128(cx.tmem + C::TM_S, q_smem, k_smem, idesc);
+    else mma_ss_k64(cx.tmem + C::TM_S, q_smem, k_smem, idesc);
     commit<C>(&cx.mi->s_full[b]);
   }
-  // O of block b += P V of a tile, in two halves as P arrives
-  __device__ __forceinline__ void pv(int b, uint32_t v_smem, bool first, bool last) {
+};
+
+template <class C>
+struct IssuerPV {
+  const Ctx2& cx;
+  uint32_t nd = 0, v = 0, tiles = 0, blocks = 0;                     // descriptors, value ring; tiles and blocks so far, modulo 2 in bit b
+  __device__ __forceinline__ explicit IssuerPV(const Ctx2& c) : cx(c) {}
+  __device__ __forceinline__ void free_v() { free_stage<C, true>(cx, v++); }
+  // the accumulator of the block before has been read out
+  __device__ __forceinline__ void wait_read_out(int b) { WAIT2I(&cx.mi->o_free[b], free_par(blocks >> b), W2_OFREE); }
+  // O of block b += P V of the values next in the ring, in two halves as P arrives.  The values are waited for after P: by then
+  // every earlier use of their stage is known to have landed (of a pair the other issuer takes sweep tiles through this ring).
+  __device__ __forceinline__ void pv(int b, bool first, bool last) {
     Misc2& mi = *cx.mi;
     constexpr uint32_t idesc = make_idesc_bf16_f32(TILE * C::NCTA, C::D, false, true);
     const uint32_t tO = cx.tmem + C::TM_O + b * C::D, tP = cx.tmem + C::TM_P + b * 64;
-    if (first) { WAIT2S(&mi.o_free[b], free_par(no[b]), W2_OFREE); ++no[b]; }       // accumulator of the previous block read out
-    WAIT2S(&mi.p_half[b], full_par(np[b]), W2_PHALF);                                // keys 0..63 of P
+    if (first) { wait_read_out(b); blocks ^= 1u << b; }
+    const uint32_t par = full_par(tiles >> b);
+    tiles ^= 1u << b;
+    WAIT2I(&mi.p_half[b], par, W2_PHALF);                                            // keys 0..63 of P
+    const uint32_t v_smem = wait_stage<C, true>(cx, v);
     tc_fence_after_sync();
     mma_ts_k64<C::PAIR>(tO, tP, v_smem, idesc, !first);
-    WAIT2S(&mi.p_full[b], full_par(np[b]), W2_PFULL);
-    ++np[b];
+    WAIT2I(&mi.p_full[b], par, W2_PFULL);
     tc_fence_after_sync();
     mma_ts_k64<C::PAIR>(tO, tP + 32, v_smem + 8192, idesc, true);
     commit<C>(&mi.pv_done[b]);

@@ -15,7 +15,7 @@
 // What bounds it: many sequences, the power cap and then the tile's softmax (2048 of some 2700 cycles a step on the MUFU pipe): 64
 // sequences of 64 queries over 16384 entries, 32/8 heads 1.23 -> 1.17 ms in a loop with one S for both blocks in turn (pc_flash.cuh).  One
 // sequence: latencies, half of the cycles in the tiles of an item, the rest writing its partial rows, cold code, setup and
-// exit: 34.6 -> 33.0 us (with the rotation and the merge).
+// exit: 34.6 -> 33.0 us (with the rotation and the merge), 31.6 with two issuing warps.
 #include "pc_attn.h"
 #include "pc_flash.cuh"
 #include "pc_kernels.h"
@@ -73,7 +73,7 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
   chain();
 
   if (warp >= WARP_PRODUCER) {
-    setmaxnreg_dec<REGS_SERVICE>();
+    setmaxnreg_dec<REGS_PARALLEL.service>();
     if (warp == WARP_PRODUCER) {
       // ================================================================ TMA producer (both CTAs of a pair)
       if (elect_one()) {
@@ -108,10 +108,10 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                             it.hkv * G + first_head(it.rg, b, rank) + i, 0, it.seq);
             ++p.q;
           }
-          // ring order: K of the first tile (alt: of the first two), then V of tile t and the K that follows it in use
+          // order of the copies: K of the first tile (alt: of the first two), then V of tile t and the K that follows it in use
           uint8_t* dst;
           auto load_k = [&](int t) {
-            const uint32_t bar = ring_stage<C>(cx, p, leader, &dst);
+            const uint32_t bar = ring_stage<C, false>(cx, p, leader, &dst);
             if (!bar) return;
             const int j = it.j0 + t, key0 = PAIR ? (int)rank * 64 : 0;
             for (int a = 0; a < C::ATOMS; ++a) {
@@ -123,7 +123,7 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
           const int lag = alt ? 2 : 1;
           for (int t = 0; t < lag && t < it.n; ++t) load_k(t);
           for (int t = 0; t < it.n; ++t) {
-            const uint32_t bar = ring_stage<C>(cx, p, leader, &dst);
+            const uint32_t bar = ring_stage<C, true>(cx, p, leader, &dst);
             const int j = it.j0 + t;
             if (bar)
               for (int a = 0; a < (PAIR ? 1 : C::ATOMS); ++a) {
@@ -140,60 +140,53 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         drain_copies<C>(cx, p, leader);
       }
       __syncwarp();
-    } else if (warp == WARP_MMA && leader) {
-      // ================================================================ issuer (of a pair: leader CTA)
+    } else if (warp == WARP_QK && leader) {
+      // ================================================================ issuer of Q K^T (of a pair: leader CTA)
       if (elect_one()) {
-        Issuer<C> is(cx);
+        IssuerQK<C> is(cx);
         while (true) {
           const Desc d = next_desc<C>(cx, is.nd, false);
           if (d.kind == KIND_DONE) break;
           const int n = d.t[1];
-          if (alt) {
-            is.qa[0] = is.qa[1] = is.wait_q();
-            for (int t = 0; t < 2 && t < n; ++t) { is.qk(t, is.wait_kv(is.kv)); is.free_kv(is.kv++); }
-            for (int t = 0; t < n; ++t) {
-              const int b = t & 1;
-              const bool more = t + 2 < n;
-              // The next S before P V of the present tile.  On single CTAs of head size 128, which hold two and a half tiles, only
-              // where its keys are there: else the values' stage is given back first (us, always before / by that rule: 16 sequences of 12000
-              // entries, window of 16, 32/8 heads 158.9 / 156.2; 33 of 2000, window of 64, 32/32 heads 254.0 / 250.4; always after: 3 of 15000,
-              // window of 16, 28/4 heads 36.7, by the rule 35.3).
-              const bool early = more && (PAIR || D == 64 || is.landed(is.kv + 1));
-              auto next_s = [&]() { is.qk(b, is.wait_kv(is.kv + 1)); is.free_kv(is.kv + 1); };
-              if (early) next_s();
-              is.pv(b, is.wait_kv(is.kv), t < 2, !more);
-              is.free_kv(is.kv);
-              if (more && !early) next_s();
-              is.kv += more ? 2 : 1;
+          is.qa[0] = is.qa[1] = is.wait_q();
+          if (!alt && d.n[1] > 0) is.qa[1] = is.wait_q();
+          for (int t = 0; t < n; ++t) {
+            const uint32_t k_u32 = is.wait_k();
+            if (alt) is.qk(t & 1, k_u32);
+            else {
+              is.qk(0, k_u32);
+              if (d.n[1] > 0) is.qk(1, k_u32);
             }
-          } else {
-            for (int b = 0; b < 2; ++b) if (d.n[b] > 0) is.qa[b] = is.wait_q();
-            const uint32_t k0 = is.wait_kv(is.kv);
-            for (int b = 0; b < 2; ++b) if (d.n[b] > 0) is.qk(b, k0);
-            is.free_kv(is.kv++);
-            for (int t = 0; t < n; ++t) {
-              const bool more = t + 1 < n;
-              uint32_t k_u32 = 0;
-              if (more) k_u32 = is.wait_kv(is.kv + 1);
-              const uint32_t v_u32 = is.wait_kv(is.kv);
-              for (int b = 0; b < 2; ++b) {
-                if (d.n[b] == 0) continue;
-                if (more) is.qk(b, k_u32);
-                is.pv(b, v_u32, t == 0, !more);
-              }
-              if (more) is.free_kv(is.kv + 1);
-              is.free_kv(is.kv);
-              is.kv += more ? 2 : 1;
-            }
+            is.free_k();
           }
         }
-        commit<C>(&mi.mma_done);                                             // teardown waits for everything this thread issued
+        commit<C>(&mi.mma_done);                                             // teardown waits for everything the issuers issued
+      }
+      __syncwarp();
+    } else if (warp == WARP_PV && leader) {
+      // ================================================================ issuer of P V (of a pair: leader CTA)
+      if (elect_one()) {
+        IssuerPV<C> is(cx);
+        while (true) {
+          const Desc d = next_desc<C>(cx, is.nd, false);
+          if (d.kind == KIND_DONE) break;
+          const int n = d.t[1];
+          for (int t = 0; t < n; ++t) {
+            if (alt) is.pv(t & 1, t < 2, t + 2 >= n);
+            else {
+              is.pv(0, t == 0, t + 1 == n);
+              if (d.n[1] > 0) is.pv(1, t == 0, t + 1 == n);
+            }
+            is.free_v();
+          }
+        }
+        commit<C>(&mi.mma_done);
       }
       __syncwarp();
     }
   } else if (warp >= WARP_EPI) {
     // ================================================================ epilogue: thread = query row
-    setmaxnreg_dec<REGS_EPI>();
+    setmaxnreg_dec<REGS_PARALLEL.epilogue>();
     const int r = tid & 127, wi = r % w;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const bool sectors = (reinterpret_cast<uintptr_t>(prm.part_o) & 31) == 0;  // a workspace is aligned to 16 bytes only
@@ -279,7 +272,7 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     }
   } else {
     // ================================================================ softmax
-    setmaxnreg_inc<REGS_SOFTMAX>();
+    setmaxnreg_inc<REGS_PARALLEL.softmax>();
     const int b = warp >> 2;
     const int r = tid & 127, wi = r % w;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;

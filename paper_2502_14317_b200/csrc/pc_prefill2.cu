@@ -13,9 +13,9 @@
 //
 // What bounds it: the board's power cap (1000 W) in any loop of these calls, so energy a tile, and beside it the MUFU pipe: a step
 // (a key tile for both blocks of a CTA) takes some 2700 cycles, of which the exponentials keep that pipe busy for 2048, the
-// products the tensor cores as long (head size 64: half as long).  Measured in a loop, whole call, with an S of each block
-// under P (3300 cycles a step) -> with one S for both in turn: 128K tokens in chunks of 8192, 32/8 heads 8.39 -> 7.89 ms; 32/32
-// heads, chunks of 4096 5.49 -> 5.31 ms; 24/8 heads, ragged 1.39 -> 1.33 ms; head size 64, 32K tokens 0.898 -> 0.886 ms.
+// products the tensor cores as long (head size 64: half as long); at any time at least one block is at its exponentials, but a warp alone
+// does not fill the pipe.  Measured in a loop, whole call, with an S of each block under P (3300 cycles a step) -> with one S
+// for both in turn: 128K tokens in chunks of 8192, 32/8 heads 8.39 -> 7.89 ms; 32/32 heads, chunks of 4096 5.49 -> 5.31 ms; 24/8 heads, ragged 1.39 -> 1.33 ms; head size 64, 32K tokens 0.898 -> 0.886 ms.  Two issuing warps: figures in pc_flash.cuh.
 // A third build, head size 128 on single CTAs, takes short chunks of odd groups (launch_prefill_t).
 //
 // Window scores: the unit that runs the last query tiles of a (chunk, kv-head) group then sweeps the keys once more
@@ -141,7 +141,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   chain();
 
   if (warp >= WARP_PRODUCER) {
-    setmaxnreg_dec<REGS_SERVICE>();
+    setmaxnreg_dec<REGS_PREFILL.service>();
     if (warp == WARP_PRODUCER) {
       // ================================================================ TMA producer (both CTAs of a pair)
       if (elect_one()) {
@@ -183,14 +183,14 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               ++p.q;
             }
             for (int j = 0; j < d.n[1]; ++j) {
-              const uint32_t kbar = ring_stage<C>(cx, p, leader, &dst);
+              const uint32_t kbar = ring_stage<C, false>(cx, p, leader, &dst);
               if (kbar) {
                 if constexpr (PAIR)
                   for (int a = 0; a < 2; ++a) load_box<C>(dst + a * 8192, &tm_kh, kbar, a * 64, d.hkv, j * TILE + (int)rank * 64, d.c);
                 else
                   for (int a = 0; a < C::ATOMS; ++a) load_box<C>(dst + a * 16384, &tm_k, kbar, a * 64, d.hkv, j * TILE, d.c);
               }
-              const uint32_t vbar = ring_stage<C>(cx, p, leader, &dst);
+              const uint32_t vbar = ring_stage<C, true>(cx, p, leader, &dst);
               if (vbar)
                 for (int a = 0; a < (PAIR ? 1 : C::ATOMS); ++a)
                   load_box<C>(dst + a * 16384, &tm_v, vbar, PAIR ? (int)rank * 64 : a * 64, d.hkv, j * TILE, d.c);
@@ -222,11 +222,11 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 }
                 ++p.q;
               }
-              // a full key tile takes TILE_STAGES consecutive stages (of a pair: two that start on an even one, everything uses
-              // stages in twos)
+              // a full key tile takes a stage of the key ring, of a pair also the one of the value ring that follows it in memory
+              // (everything uses a pair's rings in step)
               for (int jj = 0; jj < n_steps; ++jj)
                 for (int i = 0; i < TILE_STAGES; ++i) {
-                  const uint32_t kbar = ring_stage<C>(cx, p, leader, &dst);
+                  const uint32_t kbar = i == 0 ? ring_stage<C, false>(cx, p, leader, &dst) : ring_stage<C, true>(cx, p, leader, &dst);
                   if (kbar)
                     for (int a = 0; a < STAGE_ATOMS; ++a)
                       load_box<C>(dst + a * 16384, &tm_k, kbar, (i * STAGE_ATOMS + a) * 64, d.hkv, (NCTA * (step0 + jj) + (int)rank) * TILE, d.c);
@@ -240,66 +240,43 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         drain_copies<C>(cx, p, leader);
       }
       __syncwarp();
-    } else if (warp == WARP_MMA && leader) {
-      // ================================================================ issuer (of a pair: leader CTA)
+    } else if (warp == WARP_QK && leader) {
+      // ================================================================ issuer of Q K^T (of a pair: leader CTA)
       if (elect_one()) {
         const Sched2 sch = make_sched2<C, SPREAD>(prm);
         const int rows_half = sch.hp * sch.wp;
         const uint32_t idesc_sw = make_idesc_bf16_f32(TILE * NCTA, PAIR ? 2 * rows_half : (rows_half + 15) & ~15, false, false);
-        Issuer<C> is(cx);
-        uint32_t nt = 0;
-        auto first_qk = [&](int b, uint32_t k_smem) { is.qa[b] = is.wait_q(); is.qk(b, k_smem); };
-        Desc d = next_desc<C>(cx, is.nd, false);
-        bool primed = false;                                     // first S of the unit already issued
-        while (d.kind != KIND_DONE) {
+        IssuerQK<C> is(cx);
+        uint32_t nt = 0, n_go = 0;
+        bool flashed = false;                                    // a unit since the last sweep: both issuers agree on it
+        while (true) {
+          const Desc d = next_desc<C>(cx, is.nd, false);
+          if (d.kind == KIND_DONE) break;
           if (d.kind == KIND_FLASH) {
-            const int n0 = d.n[0], n = d.n[1];
-            if (!primed) {
-              const uint32_t k_u32 = is.wait_kv(is.kv);
-              for (int b = 0; b < 2; ++b) if (d.n[b] > 0) first_qk(b, k_u32);
-              is.free_kv(is.kv++);
+            flashed = true;
+            for (int j = 0; j < d.n[1]; ++j) {                   // the blocks take turns on S
+              const uint32_t k_u32 = is.wait_k();
+#pragma unroll
+              for (int b = 0; b < 2; ++b) {
+                if (j >= d.n[b]) continue;
+                if (j == 0) is.qa[b] = is.wait_q();
+                is.qk(b, k_u32);
+              }
+              is.free_k();
             }
-            Desc nx;
-            nx.kind = KIND_DONE; nx.n[0] = nx.n[1] = 0;
-            // the next unit's first S follows the last tile without a gap, where there are query slots for two units (with fewer
-            // its queries, and behind them its first keys, wait for this unit's end)
-            constexpr bool PRIMES = NQ >= 4;
-            for (int j = 0; j < n; ++j) {                        // is.kv: V of tile j; is.kv + 1: the next K
-              bool more = j + 1 < n;
-              uint32_t k_u32 = 0;
-              auto look_ahead = [&]() {
-                if (j + 1 == n) { nx = next_desc<C>(cx, is.nd, false); more = PRIMES && nx.kind == KIND_FLASH; }
-                if (more) k_u32 = is.wait_kv(is.kv + 1);
-              };
-              auto next_s = [&](int b, int nb) {
-                if (j + 1 < nb) is.qk(b, k_u32);
-                else if (j + 1 == n && more && nx.n[b] > 0) first_qk(b, k_u32);
-              };
-              // per block: the next S, then P V of the present tile; the two blocks take turns on S
-              look_ahead();
-              next_s(0, n0);
-              const uint32_t v_u32 = is.wait_kv(is.kv);
-              if (j < n0) is.pv(0, v_u32, j == 0, j == n0 - 1);
-              next_s(1, n);
-              if (more) is.free_kv(is.kv + 1);
-              is.pv(1, v_u32, j == 0, j == n - 1);
-              is.free_kv(is.kv);
-              is.kv += more ? 2 : 1;
-            }
-            primed = PRIMES && nx.kind == KIND_FLASH;
-            d = nx;
           } else {
             // ---- score sweep, one pass: S^T = K_j Qw^T.  Its two [128 keys x 256 rows] buffers overlay all of TMEM:
-            // every S / P buffer is consumed and the accumulators have been read out once o_free completes.
+            // every S / P buffer is consumed and the accumulators have been read out.
             const int n_steps = SPREAD ? d.t[1] : ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
-            for (int b = 0; b < 2; ++b) WAIT2S(&mi.o_free[b], free_par(is.no[b]), W2_OFREE);
+            if (flashed) { WAIT2S(&mi.sweep_go, full_par(n_go), W2_SWEEP); ++n_go; }
+            flashed = false;
             for (int b = 0; b < 3 - NCTA; ++b) is.qa[b] = is.wait_q();
             for (int jj = 0; jj < n_steps; ++jj, ++nt) {
               const int e = nt & 1;
               WAIT2S(&mi.t_free[e], free_par(nt >> 1), W2_TFREE);
-              const uint32_t k_u32 = is.wait_kv(is.kv);
+              const uint32_t k_u32 = is.wait_k();
               if constexpr (PAIR) {
-                is.wait_kv(is.kv + 1);
+                wait_stage<C, true>(cx, is.k);                   // (the rings are in step)
                 tc_fence_after_sync();
                 mma_ss_pair_k128<false>(cx.tmem + e * 256, k_u32, is.qa[0], idesc_sw);
               } else {
@@ -310,22 +287,53 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 }
               }
               commit<C>(&mi.t_full[e]);
-              for (int i = 0; i < TILE_STAGES; ++i) is.free_kv(is.kv++);
+              if constexpr (PAIR) free_stage<C, true>(cx, is.k);
+              is.free_k();
             }
             // what follows overwrites the sweep buffers: wait until both were read
             WAIT2S(&mi.t_free[nt & 1], free_par(nt >> 1), W2_TFREE);
             WAIT2S(&mi.t_free[(nt + 1) & 1], free_par((nt + 1) >> 1), W2_TFREE);
-            d = next_desc<C>(cx, is.nd, false);
           }
         }
-        commit<C>(&mi.mma_done);                                 // teardown waits for everything this thread issued
+        commit<C>(&mi.mma_done);                                 // teardown waits for everything the issuers issued
+      }
+      __syncwarp();
+    } else if (warp == WARP_PV && leader) {
+      // ================================================================ issuer of P V (of a pair: leader CTA)
+      if (elect_one()) {
+        IssuerPV<C> is(cx);
+        bool flashed = false;
+        while (true) {
+          const Desc d = next_desc<C>(cx, is.nd, false);
+          if (d.kind == KIND_DONE) break;
+          if (d.kind == KIND_FLASH) {
+            flashed = true;
+            for (int j = 0; j < d.n[1]; ++j) {
+#pragma unroll
+              for (int b = 0; b < 2; ++b)
+                if (j < d.n[b]) is.pv(b, j == 0, j == d.n[b] - 1);
+              is.free_v();
+            }
+          } else {
+            // (one signal per run of sweeps: with one per sweep this thread could be two phases ahead of the one that waits)
+            if (flashed) {
+              for (int b = 0; b < 2; ++b) is.wait_read_out(b);
+              tc_fence_after_sync();
+              tc_fence_before_sync();
+              mbar_arrive(&mi.sweep_go);
+            }
+            flashed = false;
+            if (PAIR) is.v += SPREAD ? d.t[1] : ((d.len + TILE - 1) / TILE + NCTA - 1) / NCTA;
+          }
+        }
+        commit<C>(&mi.mma_done);
       }
       __syncwarp();
     }
   } else if (warp >= WARP_EPI) {
     // ================================================================ epilogue: normalise, stage bf16 rows in the block's
     // (now idle) query slot, TMA store
-    setmaxnreg_dec<REGS_EPI>();
+    setmaxnreg_dec<REGS_PREFILL.epilogue>();
     const Sched2 sch = make_sched2<C, SPREAD>(prm);
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
@@ -409,7 +417,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     if (r == 0) tma_store_wait_all();
   } else {
     // ================================================================ softmax
-    setmaxnreg_inc<REGS_SOFTMAX>();
+    setmaxnreg_inc<REGS_PREFILL.softmax>();
     const Sched2 sch = make_sched2<C, SPREAD>(prm);
     const int b = warp >> 2;
     const int r = tid & 127;
