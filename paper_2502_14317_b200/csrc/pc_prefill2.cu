@@ -559,16 +559,19 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 // Slices of a group's score sweep as items of their own (SPREAD), or 0 for sweeps inside the tail items.  Where a tail item has more
 // steps (tiles of its units and of the sweep) than 1.2 times what a CTA or pair gets on average: us without / with, C x L,
 // heads, d: 1 x 2048, 32/8, 64 (3.1 times) 99 / 54; 1 x 8192, 16/4, 64 (1.7) 332 / 231; 2 x 1024, 8/2, 128 (5.5) 41.6 / 38.1;
-// 2 x 2048, 32/8, 128 (0.8) 100 / 105; 3 x 3000, 24/8, 128 (1.0) 215 / 223.  Not for two tiles, where the count in memory costs more
-// than it spreads (1 x 192, 32/8, 128 20.5 / 21.6; 4 x 256, 4/2, 64 18.4 / 19.1).
+// 2 x 2048, 32/8, 128 (0.8) 100 / 105; 3 x 3000, 24/8, 128 (1.0) 215 / 223.  Chunks of a few tiles only where the heads
+// of a group are several units (1 x 206, 14/2, 64 44.0 / 20.9; 1 x 250, 32/8, 64 22.3 / 19.5; 4 x 300, 24/8, 128 43.7 / 38.0; 4 x 500, 28/4, 128 79 / 43): with
+// one unit the count in memory costs more than it spreads (1 x 192, 32/8, 128 20.5 / 21.6; 8 x 512, 8/2, 128 31.5 / 33.3).
 template <class C>
 static int sweep_slices(const PrefillParams& p, int units) {
   constexpr int NCTA = C::NCTA, BLOCKS = 2 * NCTA;
   const long long groups = (long long)p.C * p.Hkv;
   const int T = (p.L + TILE - 1) / TILE;
-  if (groups > MAX_SPREAD_GROUPS || T < 6) return 0;
+  if (groups > MAX_SPREAD_GROUPS || T < 2) return 0;
   const int G = p.Hq / p.Hkv, hpu = G % BLOCKS == 0 ? BLOCKS : (G % 2 == 0 ? 2 : 1), tpu = BLOCKS / hpu;
-  const int P = G / hpu, U = (T + tpu - 1) / tpu, steps = (T + NCTA - 1) / NCTA;
+  const int P = G / hpu, U = (T + tpu - 1) / tpu;
+  if (P == 1 && T < 6) return 0;
+  const int steps = (T + NCTA - 1) / NCTA;
   const double all = (double)groups * (P * U * (T + tpu) / 2.0 + steps), tail = (double)P * T + steps;
   if (tail < 1.2 * all / units) return 0;
   int n = (int)(units / groups) < 8 ? (int)(units / groups) : 8;

@@ -271,6 +271,15 @@ def test_score_sweeps_as_items_of_their_own(C, L, w, Hq, Hkv, d, chunk_len):
 
 
 @pytest.mark.parametrize("C,L,w,Hq,Hkv,d,chunk_len", [
+    (1, 206, 37, 14, 2, 64, None), (2, 129, 1, 6, 2, 64, None), (1, 256, 128, 8, 1, 64, None), (1, 640, 64, 32, 8, 64, None),
+    (2, 300, 50, 6, 2, 128, None), (1, 512, 128, 7, 1, 128, None), (3, 640, 16, 12, 2, 128, [640, 17, 400]), (3, 260, 24, 14, 2, 64, [25, 260, 128]),
+])
+def test_short_chunks_with_several_units_of_heads(C, L, w, Hq, Hkv, d, chunk_len):
+    """Few groups of two to five tiles whose heads are several units: dealt out one by one as well; score sweeps of several passes."""
+    test_score_sweeps_as_items_of_their_own(C, L, w, Hq, Hkv, d, chunk_len)
+
+
+@pytest.mark.parametrize("C,L,w,Hq,Hkv,d,chunk_len", [
     (1, 2048, 128, 24, 8, 128, None),                         # 64 sweeps of one step and two passes each
     (4, 1500, 50, 5, 1, 128, [1500, 100, 900, 1300]),         # sweeps of one step or none
     (4, 1536, 50, 8, 8, 64, [1536, 100, 900, 1300]), (1, 2304, 8, 16, 8, 64, None), (1, 900, 16, 62, 62, 64, None),
