@@ -11,11 +11,12 @@
 // one sequence 33.2 / 31.6.
 // Keys and values have rings of their own, so that each of them is consumed by one issuer.
 //
-// Tensor memory, 512 columns: one S (128), P of both blocks (64 each), both accumulators (128 each).  The blocks take turns on
+// Tensor memory, 512 columns.  Head size 128: one S (128), P of both blocks (64 each), both accumulators (128 each).  The blocks take turns on
 // S: the softmax warps take a whole S into registers at once, and the product for the other block runs under their
 // exponentials.  A block therefore finds its next S ready when it is through with a tile, and the blocks' exponentials are kept half a
 // step apart.  (With an S of its own for each block and P over its first half, the next product waited for P V of the tile
-// before, 1000 of 3300 cycles a step.)
+// before, 1000 of 3300 cycles a step.)  Head size 64, whose accumulators take half the columns: an S of each block and P beside them, so
+// that no block waits for the other to read (in a loop, 32K tokens 912 -> 901 us, the whole path on 22 chunks of 958, 32/8 heads 314 -> 310).
 // Cfg<D, PAIR>: head size, and whether two CTAs of a cluster work as one unit (cta_group::2: blocks of 2 x 128 rows, every
 // K/V tile split between the two shared memories).
 #pragma once
@@ -44,8 +45,10 @@ struct Cfg {
   static constexpr int NQ = STAGE_BYTES == 16384 ? 4 : 2;  // query slots
   static constexpr int NS = STAGE_BYTES == 16384 ? 6 : 5;  // stages: even ones for keys, odd ones for values
   static constexpr int NK = (NS + 1) / 2, NV = NS / 2;
-  // TMEM: one S for both blocks in turn, P of block b at TM_P + 64 b, its accumulator at TM_O + D b
-  static constexpr uint32_t TM_S = 0, TM_P = 128, TM_O = 256;
+  // TMEM: S of block b (head size 128: one for both in turn), its P at TM_P + 64 b, its accumulator at TM_O + D b
+  static constexpr bool TWO_S = D == 64;
+  static constexpr uint32_t TM_P = TWO_S ? 256 : 128, TM_O = TWO_S ? 384 : 256;
+  static constexpr __host__ __device__ uint32_t tm_s(int b) { return TWO_S ? 128u * b : 0u; }
   // pause of the issuers between two polls, ns.  us, 20 / 0: head size 64, 32K tokens 872 / 869, windows of 64 over 32 caches of 8192,
   // 14/2 heads 113.0 / 111.3; head size 128 on pairs, windows of 64 over 32 caches of 16384, 32/8 heads 619 / 630
   static constexpr unsigned ISSUER_NS = D == 64 ? 0 : 20;
@@ -69,7 +72,7 @@ struct __align__(16) Misc2 {
   uint64_t kv_full[MAX_NS], kv_free[MAX_NS];
   uint64_t s_full[2], o_full[2], t_full[2];
   uint64_t p_half[2], p_full[2], o_free[2], t_free[2];
-  uint64_t s_read, pv_done[2];               // S is in registers / P V of a tile has run
+  uint64_t s_read[2], pv_done[2];            // S is in registers (one S: [0]) / P V of a tile has run
   uint64_t lm_full[2], lm_free[2];
   uint64_t d_full[NDESC], d_free[NDESC];
   uint64_t item_full, item_free;             // work items from the leader's producer to its peer's
@@ -180,12 +183,11 @@ __device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool
     mbar_init(&mi.s_full[b], 1); mbar_init(&mi.o_full[b], 1); mbar_init(&mi.t_full[b], 1);
     mbar_init(&mi.p_half[b], 4 * N); mbar_init(&mi.p_full[b], 4 * N); // 4 softmax warps of the block in each CTA
     mbar_init(&mi.o_free[b], 4 * N); mbar_init(&mi.t_free[b], 8 * N); // epilogue warps / softmax warps of the CTAs
-    mbar_init(&mi.pv_done[b], 1);
+    mbar_init(&mi.s_read[b], 4 * N); mbar_init(&mi.pv_done[b], 1);
     mbar_init(&mi.lm_full[b], 4); mbar_init(&mi.lm_free[b], 4);
   }
   for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 14 : 12); }   // softmax and epilogue warps, issuers
   mbar_init(&mi.item_full, 1); mbar_init(&mi.item_free, 1);
-  mbar_init(&mi.s_read, 4 * N);
   mbar_init(&mi.lse_rdy, 4 * N);
   mbar_init(&mi.sweep_go, 1);
   mbar_init(&mi.mma_done, 2);
@@ -342,7 +344,7 @@ __device__ __forceinline__ void free_stage(const Ctx2& cx, uint32_t n) { commit<
 template <class C>
 struct IssuerQK {
   const Ctx2& cx;
-  uint32_t nd = 0, k = 0, nq = 0, ns = 0;                            // descriptors, key ring, query slots, uses of S
+  uint32_t nd = 0, k = 0, nq = 0, ns = 0;                            // descriptors, key ring, query slots; uses of S so far, modulo 2 in its bit
   uint32_t qa[2] = {0, 0};                                           // query operands of the two blocks in work
   __device__ __forceinline__ explicit IssuerQK(const Ctx2& c) : cx(c) {}
   __device__ __forceinline__ uint32_t wait_q() {
@@ -357,12 +359,13 @@ struct IssuerQK {
   __device__ __forceinline__ void qk(int b, uint32_t k_smem) {
     constexpr uint32_t idesc = make_idesc_bf16_f32(TILE * C::NCTA, TILE, false, false);
     const uint32_t q_smem = b ? qa[1] : qa[0];
-    WAIT2I(&cx.mi->s_read, free_par(ns), W2_SREAD);
-    ++ns;
+    const int sb = C::TWO_S ? b : 0;
+    WAIT2I(&cx.mi->s_read[sb], free_par(ns >> sb), W2_SREAD);
+    ns ^= 1u << sb;
     tc_fence_after_sync();
-    if constexpr (C::PAIR) mma_ss_pair_k128<true>(cx.tmem + C::TM_S, q_smem, k_smem, idesc);
-    else if constexpr (C::D == 128) mma_ss_k128(cx.tmem + C::TM_S, q_smem, k_smem, idesc);
-    else mma_ss_k64(cx.tmem + C::TM_S, q_smem, k_smem, idesc);
+    if constexpr (C::PAIR) mma_ss_pair_k128<true>(cx.tmem + C::tm_s(b), q_smem, k_smem, idesc);
+    else if constexpr (C::D == 128) mma_ss_k128(cx.tmem + C::tm_s(b), q_smem, k_smem, idesc);
+    else mma_ss_k64(cx.tmem + C::tm_s(b), q_smem, k_smem, idesc);
     commit<C>(&cx.mi->s_full[b]);
   }
 };
@@ -404,7 +407,7 @@ struct Hooks {
   uint64_t* pv_done;
   uint32_t tiles;                                            // tiles of this block before the present one
   __device__ __forceinline__ Hooks(const Ctx2& c, int b)
-      : cx(c), p_half(in_cta<C>(&c.mi->p_half[b], 0)), p_full(in_cta<C>(&c.mi->p_full[b], 0)), s_read(in_cta<C>(&c.mi->s_read, 0)),
+      : cx(c), p_half(in_cta<C>(&c.mi->p_half[b], 0)), p_full(in_cta<C>(&c.mi->p_full[b], 0)), s_read(in_cta<C>(&c.mi->s_read[C::TWO_S ? b : 0], 0)),
         pv_done(&c.mi->pv_done[b]), tiles(0) {}
   __device__ __forceinline__ void on_read() const { warp_arrive_leader(s_read); }
   __device__ __forceinline__ void before_p() const { WAIT2S(pv_done, free_par(tiles), W2_PV); tc_fence_after_sync(); }

@@ -422,7 +422,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const int b = warp >> 2;
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tS = cx.tmem + C::TM_S + lane_sel, tP = cx.tmem + C::TM_P + b * 64 + lane_sel, tO = cx.tmem + C::TM_O + b * D + lane_sel;
+    const uint32_t tS = cx.tmem + C::tm_s(b) + lane_sel, tP = cx.tmem + C::TM_P + b * 64 + lane_sel, tO = cx.tmem + C::TM_O + b * D + lane_sel;
     const float scale_log2 = prm.scale_log2;
     Hooks<C> hk(cx, b);
     uint32_t nd = 0, n_s = 0, n_blk = 0, nq = 0, nt = 0, n_lse = 0;
