@@ -15,7 +15,12 @@
 // What bounds it: many sequences, the power cap and then the tile's softmax (2048 of some 2700 cycles a step on the MUFU pipe): 64
 // sequences of 64 queries over 16384 entries, 32/8 heads 1.23 -> 1.17 ms in a loop with one S for both blocks in turn (pc_flash.cuh).  One
 // sequence: latencies, half of the cycles in the tiles of an item, the rest writing its partial rows, cold code, setup and
-// exit: 34.6 -> 33.0 us (with the rotation and the merge), 31.6 with two issuing warps.
+// exit: 34.6 -> 33.0 us (with the rotation and the merge), 31.6 with two issuing warps, 30.2 with one copy of their code (below).
+//
+// The issuers' loops hold one copy of a product each, whatever block takes it.  With copies of their own for the two blocks every
+// warp was slower; probably the instruction caches, which all warps share.  In a loop, us, one issuing thread / two with copies / two
+// without: head size 64, window of 16 over 64 caches of 16000, 32/8 heads 449 / 513 / 446, window of 64 over one of 16384 28.6 / 30.2 / 27.9;
+// head size 128, window of 64 over 64 caches of 16384, 32/8 heads 1140 / 1175 / 1107, over one 33.2 / 31.2 / 30.1.
 #include "pc_attn.h"
 #include "pc_flash.cuh"
 #include "pc_kernels.h"
@@ -152,11 +157,9 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
           if (!alt && d.n[1] > 0) is.qa[1] = is.wait_q();
           for (int t = 0; t < n; ++t) {
             const uint32_t k_u32 = is.wait_k();
-            if (alt) is.qk(t & 1, k_u32);
-            else {
-              is.qk(0, k_u32);
-              if (d.n[1] > 0) is.qk(1, k_u32);
-            }
+            const int first = alt ? t & 1 : 0, last = alt ? first : (d.n[1] > 0 ? 1 : 0);       // blocks that take the tile
+#pragma unroll 1
+            for (int b = first; b <= last; ++b) is.qk(b, k_u32);
             is.free_k();
           }
         }
@@ -172,11 +175,9 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
           if (d.kind == KIND_DONE) break;
           const int n = d.t[1];
           for (int t = 0; t < n; ++t) {
-            if (alt) is.pv(t & 1, t < 2, t + 2 >= n);
-            else {
-              is.pv(0, t == 0, t + 1 == n);
-              if (d.n[1] > 0) is.pv(1, t == 0, t + 1 == n);
-            }
+            const int first = alt ? t & 1 : 0, last = alt ? first : (d.n[1] > 0 ? 1 : 0), step = alt ? 2 : 1;
+#pragma unroll 1
+            for (int b = first; b <= last; ++b) is.pv(b, t < step, t + step >= n);
             is.free_v();
           }
         }

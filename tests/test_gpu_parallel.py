@@ -72,6 +72,37 @@ def test_row_blocks_that_are_not_full(B, w, G, Hkv, d, Nk):
         assert np.abs(res["lse"][b:b + 1].cpu().numpy() - LSE).max() <= 2e-3
 
 
+WIDE = [                                                                     # both ways to fill the blocks, keys split and whole, rings that go round
+    (1, 64, 8, 2, 128, 1700), (40, 64, 8, 2, 128, 900),                      # pairs, alternate tiles
+    (6, 128, 16, 4, 128, 1800), (74, 64, 8, 1, 128, 2000),                   # pairs, shared tiles
+    (3, 16, 8, 2, 128, 1700), (80, 16, 8, 2, 128, 900),                      # single CTAs, alternate tiles
+    (1, 64, 4, 2, 64, 1700), (80, 32, 8, 2, 64, 900),                        # head size 64, alternate tiles
+    (12, 64, 16, 4, 64, 2600), (74, 64, 8, 2, 64, 1700),                     # head size 64, shared tiles
+]
+
+
+def _check_some_sequences(res, q, kc, vc, kw, vw, q_pos0, theta):
+    assert int(res["status"].item()) == 0
+    for b in sorted({0, q.shape[0] // 2, q.shape[0] - 1}):
+        Fg, LSE = orc.parallel_attention(q[b:b + 1], q_pos0, theta, None, *(x[b:b + 1] for x in (kc, vc, kw, vw)))
+        check_attention_output(to_f64(res["out"][b:b + 1]), Fg, "Fg", sharp=True)
+        assert np.abs(res["lse"][b:b + 1].cpu().numpy() - LSE).max() <= 2e-3
+
+
+@pytest.mark.parametrize("B,w,Hq,Hkv,d,Nk", WIDE)
+def test_many_query_rows_over_growing_keys(B, w, Hq, Hkv, d, Nk):
+    """More than 32 query rows: the reference maxima are raised by factors other than zero in most tiles, in streams that hold
+    different maxima, and the accumulators rescaled."""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(Nk + w + d)
+    grow = np.linspace(1.0, 40.0, Nk, dtype=np.float32)[None, None, :, None]
+    kc = pc_inputs.f32_to_bf16_bits(rng.standard_normal((B, Hkv, Nk, d)).astype(np.float32) * grow)
+    q, kw, vw, vc = (_bits(rng, s) for s in ((B, w, Hq, d), (B, w, Hkv, d), (B, w, Hkv, d), (B, Hkv, Nk, d)))
+    res = pc.parallel_attn(*(to_dev(x) for x in (q, kc, vc, kw, vw)), q_pos0=500, rope_theta=1e4, want_lse=True)
+    torch.cuda.synchronize()
+    _check_some_sequences(res, q, kc, vc, kw, vw, 500, 1e4)
+
+
 @pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 128), (4, 2, 128), (4, 2, 64)])
 @pytest.mark.parametrize("shift", [16, 32, 48])
 def test_workspace_at_any_multiple_of_16_bytes(Hq, Hkv, d, shift):
