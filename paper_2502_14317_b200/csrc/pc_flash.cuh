@@ -9,7 +9,7 @@
 // when P arrives.  One thread in a fixed order was busy for two thirds of a step and late for both.  In a loop, us, one thread / two (and the registers
 // below): 8 chunks of 8192, 32/8 heads 3924 / 3865, 8 of 4096, 32/32 heads 1346 / 1333, 4 of 1257, 32/32 heads 138.1 / 135.8, query window of
 // one sequence 33.2 / 31.6.
-// Keys and values have rings of their own, so that each of them is consumed by one issuer.
+// Keys and values have rings of their own, so that each of them is consumed by one issuer (of a pair's value ring the sweeps take stages too).
 //
 // Tensor memory, 512 columns.  Head size 128: one S (128), P of both blocks (64 each), both accumulators (128 each).  The blocks take turns on
 // S: the softmax warps take a whole S into registers at once, and the product for the other block runs under their
@@ -43,8 +43,11 @@ struct Cfg {
   static constexpr int Q_BYTES = TILE * D * 2;
   static constexpr int STAGE_BYTES = TILE * D * 2 / NCTA;  // K/V rings: a tile, or of a pair 64 keys of K / half the columns of V
   static constexpr int NQ = STAGE_BYTES == 16384 ? 4 : 2;  // query slots
-  static constexpr int NS = STAGE_BYTES == 16384 ? 6 : 5;  // stages: even ones for keys, odd ones for values
-  static constexpr int NK = (NS + 1) / 2, NV = NS / 2;
+  static constexpr int NS = STAGE_BYTES == 16384 ? 6 : 5;
+  // Stages of keys and of values, alternating.  Of five the values get three: they stay until P has been found, keys only until the
+  // next product.  Caches read at the memory's rate, us, 3 + 2 / 2 + 3: window of 16 over 64 caches of 16000, 32/8 heads 768 / 735, 64 of 2000
+  // 121 / 116, window of 64 over 18 of 8000, 32/32 heads 441 / 421; chunks on single CTAs the same (64 x 384, 32/32 heads 423 / 421).
+  static constexpr int NK = NS / 2, NV = NS - NK;
   // TMEM: S of block b (head size 128: one for both in turn), its P at TM_P + 64 b, its accumulator at TM_O + D b
   static constexpr bool TWO_S = D == 64;
   static constexpr uint32_t TM_P = TWO_S ? 256 : 128, TM_O = TWO_S ? 384 : 256;
@@ -261,7 +264,7 @@ __device__ __forceinline__ int next_item(const Ctx2& cx, Prod& p, bool leader, i
 }
 // stage of the n-th use of the key ring (V: of the value ring), and how often the stage has been used before
 template <class C, bool V>
-__device__ __forceinline__ int stage_of(uint32_t n) { return V ? 2 * (n % C::NV) + 1 : 2 * (n % C::NK); }
+__device__ __forceinline__ int stage_of(uint32_t n) { return V ? 2 * (n % C::NV) + (C::NV == C::NK) : 2 * (n % C::NK) + (C::NV != C::NK); }
 template <class C, bool V>
 __device__ __forceinline__ uint32_t lap_of(uint32_t n) { return n / (V ? C::NV : C::NK); }
 // expects a stage's bytes over both CTAs on the leader's barrier of the ring's next stage; returns that barrier's address
