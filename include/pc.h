@@ -120,10 +120,11 @@ PC_API int32_t pc_chunk_prefill_attn(const pc_prefill_desc* desc, const void* q,
  * flight and return; the host then treats the call's results as undefined (PC_ERR_TIMEOUT).
  *   wait_limit_cycles      limit for all later launches of this process (0: the default of
  *                          about 2e9 cycles, a second);
- *   skip_final_publication non-zero: the chunk-prefill kernels leave out ONE signal that
- *                          carries no data - the "no more work" message to the consumer warps after the last work
- *                          item, when nothing is in flight any more - so that their wait, and the producer's for
- *                          the message to be taken, run out.  Outputs of such a call are complete (not the scores of a call whose
+ *   skip_final_publication non-zero: the chunk-prefill kernel of head size 64 and the parallel-attention kernel for more
+ *                          than 32 query rows leave out ONE signal that carries no data - the "no more work"
+ *                          message to the consumer warps after the last work item, when nothing is in flight any
+ *                          more - so that their wait (in the latter also the producer's for the message to be
+ *                          taken, behind which it drains its copies) runs out.  Outputs of such a call are complete (not the scores of a call whose
  *                          sweeps are items of their own: they wait for blocks that end with that signal); its status_word
  *                          is non-zero.  Zero switches the hook off again.
  * Host-side settings, read at every launch.

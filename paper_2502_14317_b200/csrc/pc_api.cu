@@ -623,6 +623,7 @@ int32_t parallel_attn_impl(int32_t B, int32_t w, int32_t Hq, int32_t Hkv, int32_
   prm.status = status_word;
   prm.counter = counter;
   prm.wait_kcycles = pc::g_wait_kcycles.load();
+  prm.skip_final_publication = pc::g_skip_final_publication.load();
   cudaError_t e = pc::launch_parallel_attn(maps, prm, d, plan.pair, dev.sm_count, st);
   // the attention reads entries below Nk only (rows behind them read as zeros and are masked): the new rows can follow
   // on the same stream

@@ -46,6 +46,7 @@ struct ParallelParams {
   int* status;
   int* counter;                  // work-queue counter, zeroed before launch
   int wait_kcycles;              // limit of every device-side wait, in units of 1024 cycles
+  int skip_final_publication;    // test hook of the bounded waits (see pc_debug_bounded_wait_test in pc.h)
 };
 // maps: rotated q_win (w-row box), k_cache (128-key box; pair: 64), v_cache (128), k_win (128-row box over w tokens; pair:
 // 64), v_win (128)

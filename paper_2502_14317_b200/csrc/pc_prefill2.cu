@@ -236,9 +236,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
         Desc d;
         d.kind = KIND_DONE; d.c = d.hkv = d.len = 0;
-        publish<C>(cx, p, d, prm.skip_final_publication == 0);
-        // test hook: nobody takes the message, so this wait runs out as the consumers' do, and the copies are drained as after any abort
-        if (prm.skip_final_publication != 0) WAIT2(&mi.d_free[(p.d - 1) % NDESC], free_par((p.d - 1) / NDESC + 1), W2_DESC);
+        publish<C>(cx, p, d, D == 128 || prm.skip_final_publication == 0);
         drain_copies<C>(cx, p, leader);
       }
       __syncwarp();

@@ -103,6 +103,54 @@ def test_many_query_rows_over_growing_keys(B, w, Hq, Hkv, d, Nk):
     _check_some_sequences(res, q, kc, vc, kw, vw, 500, 1e4)
 
 
+@pytest.mark.parametrize("B,w,Hq,Hkv,d,Nk", WIDE[1::2])          # keys whole: the tile is no stream's first
+@pytest.mark.parametrize("at", [522, 612])                        # in the first / in the second half of a key tile
+def test_many_query_rows_and_one_logit_far_above_the_others(B, w, Hq, Hkv, d, Nk, at):
+    """A single key whose probability, against the maximum of the tiles before, is beyond fp32: it has to be noticed in either half of
+    a tile.  (Through the slowest pair, which the rotation leaves as it is.)"""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(Nk + at)
+    q, kc, vc, kw, vw = (rng.standard_normal(s).astype(np.float32) * g for s, g in (
+        ((B, w, Hq, d), 0.3), ((B, Hkv, Nk, d), 0.3), ((B, Hkv, Nk, d), 1.0), ((B, w, Hkv, d), 0.3), ((B, w, Hkv, d), 1.0)))
+    q[..., d // 2 - 1], kc[..., d // 2 - 1], kw[..., d // 2 - 1] = 8.0, 0.0, 0.0
+    kc[:, :, at, d // 2 - 1] = 150.0 * np.sqrt(d) / (8.0 * np.log2(np.e))
+    q, kc, vc, kw, vw = (pc_inputs.f32_to_bf16_bits(x) for x in (q, kc, vc, kw, vw))
+    res = pc.parallel_attn(*(to_dev(x) for x in (q, kc, vc, kw, vw)), q_pos0=500, rope_theta=1e9, want_lse=True)
+    torch.cuda.synchronize()
+    _check_some_sequences(res, q, kc, vc, kw, vw, 500, 1e9)
+
+
+@pytest.mark.parametrize("B,w,Hq,Hkv,d,Nk,code", [
+    (1, 64, 8, 2, 128, 1700, 201), (74, 64, 8, 1, 128, 2000, 201), (3, 16, 8, 2, 128, 1700, 101), (80, 32, 8, 2, 64, 900, 101),
+])
+def test_a_wait_that_runs_out_in_the_wide_kernel(B, w, Hq, Hkv, d, Nk, code):
+    """CTA pairs and single CTAs: the producers leave out the data-free "no more work" signal after the last work item, when no copy
+    and no product is in flight.  The waits for it give up after about a millisecond, the status word holds their code, the producer
+    drains its copies, both CTAs of a pair return, the outputs are complete and the next call gives the bits of a clean run."""
+    import paper_2502_14317_b200 as pc
+    rng = np.random.default_rng(Nk)
+    t = [to_dev(_bits(rng, s)) for s in ((B, w, Hq, d), (B, Hkv, Nk, d), (B, Hkv, Nk, d), (B, w, Hkv, d), (B, w, Hkv, d))]
+    lib = pc.load_library()
+
+    def run():
+        r = pc.parallel_attn(*t, q_pos0=300, rope_theta=1e4, want_lse=True)
+        torch.cuda.synchronize()
+        return r
+
+    clean = run()
+    assert int(clean["status"].item()) == 0
+    assert lib.pc_debug_bounded_wait_test(2_000_000, 1) == 0          # waits give up after 2e6 cycles (about 1 ms)
+    try:
+        hit = run()
+    finally:
+        assert lib.pc_debug_bounded_wait_test(0, 0) == 0
+    assert int(hit["status"].item()) == code
+    again = run()
+    assert int(again["status"].item()) == 0
+    for r in (hit, again):
+        assert torch.equal(r["out"], clean["out"]) and torch.equal(r["lse"], clean["lse"])
+
+
 @pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 128), (4, 2, 128), (4, 2, 64)])
 @pytest.mark.parametrize("shift", [16, 32, 48])
 def test_workspace_at_any_multiple_of_16_bytes(Hq, Hkv, d, shift):

@@ -392,25 +392,20 @@ def test_chunks_of_different_lengths_in_one_call(L, w, Hq, Hkv, d, lens):
         assert np.all(got_o[c, n:] == 0.0) and np.all(got_S[c, :, n:] == 0.0) and np.all(got_lse[c, :, n:] == 0.0)
 
 
-@pytest.mark.parametrize("d,code", [(64, 101), (128, 201)])           # single CTAs; CTA pairs
-def test_a_wait_that_runs_out_returns_a_status_and_leaves_the_device_usable(cfg0_inputs, d, code):
+def test_a_wait_that_runs_out_returns_a_status_and_leaves_the_device_usable(cfg0_inputs):
     """Every device-side wait is bounded.  Here one is made to run out without faulting anything: the producer
-    warps leave out the data-free "no more work" signal after the last work item, when no copy and no tensor-core
-    operation is in flight; the consumer warps wait for it for about a millisecond (limit set through the test hook),
-    store the code of that wait in the status word, drain and return, on a pair in both CTAs.  The outputs of that call
-    are complete, and the next call on the same stream is bit-identical to a clean run."""
+    warp of the single-CTA kernel (head size 64) leaves out the data-free "no more work" signal after the last
+    work item, when no copy and no tensor-core operation is in flight; the consumer warps wait for it for about a
+    millisecond (limit set through the test hook), store the code of that wait in the status word, drain and
+    return.  The outputs of that call are complete, and the next call on the same stream is bit-identical to a
+    clean run."""
     import paper_2502_14317_b200 as pc
     cfg, inp = cfg0_inputs
-    if d == 64:
-        q, k, v, w = to_dev(inp["q"]), to_dev(inp["k"]), to_dev(inp["v"]), cfg.w
-    else:
-        rng = np.random.default_rng(d)
-        q, k, v = (to_dev(pc_inputs.f32_to_bf16_bits(rng.standard_normal((3, 600, h, d)).astype(np.float32))) for h in (8, 2, 2))
-        w = 32
+    q, k, v = to_dev(inp["q"]), to_dev(inp["k"]), to_dev(inp["v"])
     lib = pc.load_library()
 
     def run():
-        r = pc.chunk_prefill_attn(q, k, v, w=w, rope_theta=1e4, want_lse=True)
+        r = pc.chunk_prefill_attn(q, k, v, w=cfg.w, rope_theta=cfg.rope_theta, want_lse=True)
         torch.cuda.synchronize()
         return r
 
@@ -421,8 +416,8 @@ def test_a_wait_that_runs_out_returns_a_status_and_leaves_the_device_usable(cfg0
         hit = run()
     finally:
         assert lib.pc_debug_bounded_wait_test(0, 0) == 0
-    got = int(hit["status"].item())
-    assert got == code, f"expected the code of the work-item wait in the status word, got {got}"
+    code = int(hit["status"].item())
+    assert code == 101, f"expected the code of the work-item wait in the status word, got {code}"
     for key in ("o", "win_score", "win_lse", "lse", "k_rot"):
         assert torch.equal(hit[key], clean[key]), key                 # all work was done before the missing signal
     again = run()
