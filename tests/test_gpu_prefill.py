@@ -134,7 +134,8 @@ def test_growing_logits_rescale_path(d):
 def test_logits_that_rise_less_than_the_threshold_a_tile(d, rise):
     """Every key tile lies `rise` (in log2) above the one before: no logit exceeds the reference maximum by 2^8, but 64
     probabilities of 2^rise sum up to more than 2^8 (rise = 2: about as much, so that some rows of a warp are raised and others are
-    not).  The rise goes through the slowest pair, which the rotation leaves as it is."""
+    not).  The rise goes through the slowest pair, which the rotation leaves as it is.  (What is tested is the repeated half; that a
+    logit is noticed in either half: the next test.)"""
     rng = np.random.default_rng(31 + d)
     C, L, Hq, Hkv, w = 1, 900, 4, 2, 32
     q = 0.3 * rng.standard_normal((C, L, Hq, d)).astype(np.float32)
@@ -142,6 +143,24 @@ def test_logits_that_rise_less_than_the_threshold_a_tile(d, rise):
     v = rng.standard_normal((C, L, Hkv, d)).astype(np.float32)
     q[..., d // 2 - 1] = 8.0
     k[..., d // 2 - 1] = (np.arange(L) // 128 * rise * np.sqrt(d) / (8.0 * np.log2(np.e)))[None, :, None]
+    bits = [pc_inputs.f32_to_bf16_bits(x) for x in (q, k, v)]
+    _run_and_compare(bits[0], bits[1], bits[2], w, 1.0e9, sharp=True)
+
+
+@pytest.mark.parametrize("d,Hq,Hkv", [(64, 4, 2), (128, 8, 2), (128, 4, 2), (128, 3, 1)])
+@pytest.mark.parametrize("at", [266, 356])                 # in the first / in the second half of a key tile
+def test_one_logit_far_above_the_others(d, Hq, Hkv, at):
+    """A single key lies more than 2^130 above all the others: taken against the maximum of the tiles before, its probability is beyond
+    fp32, so it has to be noticed in whichever half of a tile it stands, also by rows whose second half is masked (query rows 266 to
+    319 for the key at 266).  It goes through the slowest pair, which the rotation leaves as it is."""
+    rng = np.random.default_rng(at + d)
+    C, L, w = 1, 700, 32
+    q, k, v = (rng.standard_normal((C, L, h, d)).astype(np.float32) * g for h, g in ((Hq, 0.3), (Hkv, 0.3), (Hkv, 1.0)))
+    q[..., d // 2 - 1], k[..., d // 2 - 1] = 8.0, 0.0
+    k[:, at, :, d // 2 - 1] = 150.0 * np.sqrt(d) / (8.0 * np.log2(np.e))
+    s = np.einsum("ihd,jd->hij", q[0, :, :Hq // Hkv], k[0, :, 0]) * (np.log2(np.e) / np.sqrt(d))
+    with np.errstate(over="ignore"):
+        assert np.isinf(np.exp2(s[:, at:, at] - s[:, at:, :at].max(-1)).astype(np.float32)).all()
     bits = [pc_inputs.f32_to_bf16_bits(x) for x in (q, k, v)]
     _run_and_compare(bits[0], bits[1], bits[2], w, 1.0e9, sharp=True)
 
