@@ -444,8 +444,11 @@ ParallelPlan parallel_plan(int B, int w, int Hq, int Hkv, int d, int Nk, int sm_
   // alternate tiles; an even number can do that too, or be filled with different rows that share every key tile, with half
   // the items.  Rows and key splits: least time by a model in microseconds - rounds of the grid x (about 5 for an item + 1.4
   // a tile, 2.8 where a tile serves two blocks of rows, 1.5 where the other blocks' items read it again) + 4 for the merge of
-  // splits.  Measured, us, shared / alternate tiles: 64/4 heads of 128, window of 32, 8 sequences of 3000 entries (32 or 64 items
-  // on 74 pairs) 60.7 / 40.1, 64 of 8192 (256 / 512 items) 512 / 503; 32/8, window of 128, 12 of 8192 (96 / 192) 260 / 218, 16 of 4096 159 / 169.
+  // splits.  Measured, us, shared / alternate tiles: 64/4 heads of 128, window of 32, 8 sequences of 3000 entries (32 or 64
+  // items on 74 pairs) 53.8 / 35.7, 64 of 8192 (256 / 512 items) 584 / 555; 32/8, window of 128, 12 of 8192 (96 / 192) 271 / 218,
+  // 16 of 4096 156 / 166; head size 64, 32/8 heads, window of 64, 38 of 2731 124 / 115, 64 of 700 68 / 74.  The kernel's tiles have
+  // become faster than the model's (some 1.1 and 2.1) by about the same factor, so that the order of the two stands; splits
+  // it takes a little too readily (16/4 heads of 128, window of 128, 6 of 1800: shared in three splits 33.0, alternate, whole 26.4).
   p.pair = d == 128 && G * w > 128 && sm_count >= 2;
   const int block_heads = (p.pair ? 256 : 128) / w, blocks = (G + block_heads - 1) / block_heads;
   const int units = p.pair ? sm_count / 2 : sm_count, n_all = p.n_cache_tiles + 1;

@@ -5,18 +5,20 @@
 // cores work for the other.  Warps (16): 0-3 softmax of block A, 4-7 softmax of block B (thread = query row = TMEM lane),
 // 8-11 epilogue (the softmax warps go straight on to the next block), 12 TMA producer, 13 issuer of S = Q K^T and of the score
 // sweeps, 14 issuer of O += P V (of a CTA pair: in the leader only), 15 idle.  Registers are dealt out by role.
-// The issuers are two because their waits have nothing to do with each other: S is due when the S before it has been read, P V
-// when P arrives.  One thread in a fixed order was busy for two thirds of a step and late for both.  In a loop, us, one thread / two (and the registers
-// below): 8 chunks of 8192, 32/8 heads 3924 / 3865, 8 of 4096, 32/32 heads 1346 / 1333, 4 of 1257, 32/32 heads 138.1 / 135.8, query window of
-// one sequence 33.2 / 31.6.
-// Keys and values have rings of their own, so that each of them is consumed by one issuer (of a pair's value ring the sweeps take stages too).
+// The issuers are two because their waits have nothing to do with each other: S is due when the S before it has been read,
+// P V when P arrives.  One thread in a fixed order was busy for two thirds of a step and late for both.  In a loop, us, one
+// thread / two (and, in the prefill, the registers below): 8 chunks of 8192, 32/8 heads 3924 / 3865, 8 of 4096, 32/32 heads
+// 1346 / 1333, 4 of 1257, 32/32 heads 138.1 / 135.8; query windows: pc_parallel.cu.
+// Keys and values have rings of their own, so that each of them is consumed by one issuer (of a pair's value ring the sweeps
+// take stages too).
 //
-// Tensor memory, 512 columns.  Head size 128: one S (128), P of both blocks (64 each), both accumulators (128 each).  The blocks take turns on
-// S: the softmax warps take a whole S into registers at once, and the product for the other block runs under their
-// exponentials.  A block therefore finds its next S ready when it is through with a tile, and the blocks' exponentials are kept half a
-// step apart.  (With an S of its own for each block and P over its first half, the next product waited for P V of the tile
-// before, 1000 of 3300 cycles a step.)  Head size 64, whose accumulators take half the columns: an S of each block and P beside them, so
-// that no block waits for the other to read (in a loop, 32K tokens 912 -> 901 us, the whole path on 22 chunks of 958, 32/8 heads 314 -> 310).
+// Tensor memory, 512 columns.  Head size 128: one S (128), P of both blocks (64 each), both accumulators (128 each).  The
+// blocks take turns on S: the softmax warps take a whole S into registers at once, and the product for the other block runs
+// under their exponentials.  A block therefore finds its next S ready when it is through with a tile, and the blocks'
+// exponentials are kept half a step apart.  (With an S of its own for each block and P over its first half, the next product
+// waited for P V of the tile before, 1000 of 3300 cycles a step.)  Head size 64, whose accumulators take half the columns: an
+// S of each block and P beside them, so that no block waits for the other to read (prefill in a loop, one S / two, us: 8 chunks
+// of 4096, 32/32 heads 923 / 909, 22 of 958, 32/8 heads 284 / 278; query windows the same).
 // Cfg<D, PAIR>: head size, and whether two CTAs of a cluster work as one unit (cta_group::2: blocks of 2 x 128 rows, every
 // K/V tile split between the two shared memories).
 #pragma once
@@ -28,8 +30,10 @@ namespace flash {
 constexpr int TILE = 128;
 constexpr int NT2 = 512;                     // threads per CTA
 constexpr int WARP_EPI = 8, WARP_PRODUCER = 12, WARP_QK = 13, WARP_PV = 14;
-// registers by role, 128 * (2 * softmax + epilogue + service) = 64 K
-// (prefill, 8 chunks of 8192, 32/8 heads: softmax 184 3920 us, 192 3872, 200 3870 with spills in the other roles; over caches 184 619, 192 631)
+// Registers by role, 128 * (2 * softmax + epilogue + service) = 64 K.  In a loop, us: prefill, 8 chunks of 8192, 32/8 heads
+// 184/80/64 4073, 192/80/48 3983, 192/64/64 3993, 8 of 4096, 32/32 heads 1399 / 1366 / 1378; over caches softmax 184 619, 192 631.
+// With 48 registers the service roles spill (-Xptxas -v: 64 bytes stored, 84 loaded at head size 128 on pairs; 192/64/64
+// spills nothing and is no faster).
 struct Regs { int softmax, epilogue, service; };
 constexpr Regs REGS_PREFILL = {192, 80, 48}, REGS_PARALLEL = {184, 80, 64};
 constexpr int NDESC = 4;                     // work descriptors in flight
@@ -44,16 +48,18 @@ struct Cfg {
   static constexpr int STAGE_BYTES = TILE * D * 2 / NCTA;  // K/V rings: a tile, or of a pair 64 keys of K / half the columns of V
   static constexpr int NQ = STAGE_BYTES == 16384 ? 4 : 2;  // query slots
   static constexpr int NS = STAGE_BYTES == 16384 ? 6 : 5;
-  // Stages of keys and of values, alternating.  Of five the values get three: they stay until P has been found, keys only until the
-  // next product.  Caches read at the memory's rate, us, 3 + 2 / 2 + 3: window of 16 over 64 caches of 16000, 32/8 heads 768 / 735, 64 of 2000
-  // 121 / 116, window of 64 over 18 of 8000, 32/32 heads 441 / 421; chunks on single CTAs the same (64 x 384, 32/32 heads 423 / 421).
+  // Stages of keys and of values, alternating.  Of five the values get three: they stay until P has been found, keys only
+  // until the next product.  Caches read at the memory's rate, us, 3 + 2 / 2 + 3: window of 16 over 64 caches of 16000, 32/8
+  // heads 768 / 735, 64 of 2000 121 / 116, window of 64 over 18 of 8000, 32/32 heads 441 / 421; chunks on single CTAs the same
+  // (64 x 384, 32/32 heads 423 / 421).
   static constexpr int NK = NS / 2, NV = NS - NK;
   // TMEM: S of block b (head size 128: one for both in turn), its P at TM_P + 64 b, its accumulator at TM_O + D b
   static constexpr bool TWO_S = D == 64;
   static constexpr uint32_t TM_P = TWO_S ? 256 : 128, TM_O = TWO_S ? 384 : 256;
   static constexpr __host__ __device__ uint32_t tm_s(int b) { return TWO_S ? 128u * b : 0u; }
-  // pause of the issuers between two polls, ns.  us, 20 / 0: head size 64, 32K tokens 872 / 869, windows of 64 over 32 caches of 8192,
-  // 14/2 heads 113.0 / 111.3; head size 128 on pairs, windows of 64 over 32 caches of 16384, 32/8 heads 619 / 630
+  // Pause of the issuers between two polls, ns.  us, 20 / 0: head size 64, windows of 64 over 32 caches of 8192, 14/2 heads
+  // 112.4 / 111.0, over one of 16384, 32/8 heads 28.1 / 27.8, 8 chunks of 4096 the same; head size 128, within the noise of a
+  // loop at the power cap: 8 chunks of 8192 3983 / 3941, 8 of 4096, 32/32 heads 1366 / 1378, windows over 32 caches of 16384 625 / 619
   static constexpr unsigned ISSUER_NS = D == 64 ? 0 : 20;
   static constexpr int CODE = PAIR ? 200 : 100;            // wait codes in the status word
 };
@@ -189,7 +195,7 @@ __device__ __forceinline__ void init_barriers2(Misc2& mi, int wait_kcycles, bool
     mbar_init(&mi.s_read[b], 4 * N); mbar_init(&mi.pv_done[b], 1);
     mbar_init(&mi.lm_full[b], 4); mbar_init(&mi.lm_free[b], 4);
   }
-  for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 14 : 12); }   // softmax and epilogue warps, issuers
+  for (int i = 0; i < NDESC; ++i) { mbar_init(&mi.d_full[i], 1); mbar_init(&mi.d_free[i], leader ? 14 : 12); }   // warps, issuers
   mbar_init(&mi.item_full, 1); mbar_init(&mi.item_free, 1);
   mbar_init(&mi.lse_rdy, 4 * N);
   mbar_init(&mi.sweep_go, 1);
@@ -326,9 +332,12 @@ __device__ __forceinline__ void drain_copies(const Ctx2& cx, const Prod& p, bool
   Misc2& mi = *cx.mi;
   if (!*cx.abort_flag) return;
   if (leader) {
-    for (uint32_t i = (p.k > C::NK ? p.k - C::NK : 0); i < p.k; ++i) mbar_wait_drain(&mi.kv_full[stage_of<C, false>(i)], full_par(lap_of<C, false>(i)), cx.abort_flag);
-    for (uint32_t i = (p.v > C::NV ? p.v - C::NV : 0); i < p.v; ++i) mbar_wait_drain(&mi.kv_full[stage_of<C, true>(i)], full_par(lap_of<C, true>(i)), cx.abort_flag);
-    for (uint32_t i = (p.q > C::NQ ? p.q - C::NQ : 0); i < p.q; ++i) mbar_wait_drain(&mi.q_full[i % C::NQ], full_par(i / C::NQ), cx.abort_flag);
+    for (uint32_t i = (p.k > C::NK ? p.k - C::NK : 0); i < p.k; ++i)
+      mbar_wait_drain(&mi.kv_full[stage_of<C, false>(i)], full_par(lap_of<C, false>(i)), cx.abort_flag);
+    for (uint32_t i = (p.v > C::NV ? p.v - C::NV : 0); i < p.v; ++i)
+      mbar_wait_drain(&mi.kv_full[stage_of<C, true>(i)], full_par(lap_of<C, true>(i)), cx.abort_flag);
+    for (uint32_t i = (p.q > C::NQ ? p.q - C::NQ : 0); i < p.q; ++i)
+      mbar_wait_drain(&mi.q_full[i % C::NQ], full_par(i / C::NQ), cx.abort_flag);
   }
   abort_grace_pause(cx.abort_flag);
 }
@@ -347,7 +356,7 @@ __device__ __forceinline__ void free_stage(const Ctx2& cx, uint32_t n) { commit<
 template <class C>
 struct IssuerQK {
   const Ctx2& cx;
-  uint32_t nd = 0, k = 0, nq = 0, ns = 0;                            // descriptors, key ring, query slots; uses of S so far, modulo 2 in its bit
+  uint32_t nd = 0, k = 0, nq = 0, ns = 0;                            // descriptors, key ring, query slots; uses of S, modulo 2 in bits
   uint32_t qa[2] = {0, 0};                                           // query operands of the two blocks in work
   __device__ __forceinline__ explicit IssuerQK(const Ctx2& c) : cx(c) {}
   __device__ __forceinline__ uint32_t wait_q() {
@@ -410,8 +419,8 @@ struct Hooks {
   uint64_t* pv_done;
   uint32_t tiles;                                            // tiles of this block before the present one
   __device__ __forceinline__ Hooks(const Ctx2& c, int b)
-      : cx(c), p_half(in_cta<C>(&c.mi->p_half[b], 0)), p_full(in_cta<C>(&c.mi->p_full[b], 0)), s_read(in_cta<C>(&c.mi->s_read[C::TWO_S ? b : 0], 0)),
-        pv_done(&c.mi->pv_done[b]), tiles(0) {}
+      : cx(c), p_half(in_cta<C>(&c.mi->p_half[b], 0)), p_full(in_cta<C>(&c.mi->p_full[b], 0)),
+        s_read(in_cta<C>(&c.mi->s_read[C::TWO_S ? b : 0], 0)), pv_done(&c.mi->pv_done[b]), tiles(0) {}
   __device__ __forceinline__ void on_read() const { warp_arrive_leader(s_read); }
   __device__ __forceinline__ void before_p() const { WAIT2S(pv_done, free_par(tiles), W2_PV); tc_fence_after_sync(); }
   __device__ __forceinline__ void on_half() const { warp_arrive_leader(p_half); }

@@ -12,15 +12,17 @@
 // count.  Queries arrive rotated.  Small batches split the keys; the splits' fp32 partial results are merged
 // by a second kernel.
 //
-// What bounds it: many sequences, the power cap and then the tile's softmax (2048 of some 2700 cycles a step on the MUFU pipe): 64
-// sequences of 64 queries over 16384 entries, 32/8 heads 1.23 -> 1.17 ms in a loop with one S for both blocks in turn (pc_flash.cuh).  One
-// sequence: latencies, half of the cycles in the tiles of an item, the rest writing its partial rows, cold code, setup and
-// exit: 34.6 -> 33.0 us (with the rotation and the merge), 31.6 with two issuing warps, 30.2 with one copy of their code (below).
+// What bounds it: many sequences, the power cap and the tile's softmax (2048 cycles a step on the MUFU pipe at the least): 64
+// sequences of 64 queries over 16384 entries, 32/8 heads 1.23 -> 1.17 ms in a loop with one S for both blocks in turn
+// (pc_flash.cuh).  Head size 128 with few rows: caches are read at 5 TB/s.  One sequence: latencies, half of the cycles in the
+// tiles of an item, the rest writing its partial rows, cold code, setup and exit: 34.6 -> 33.0 us (with the rotation and the
+// merge) with one S, 31.6 with two issuing warps, 30.2 with one copy of their code.
 //
-// The issuers' loops hold one copy of a product each, whatever block takes it.  With copies of their own for the two blocks every
-// warp was slower; probably the instruction caches, which all warps share.  In a loop, us, one issuing thread / two with copies / two
-// without: head size 64, window of 16 over 64 caches of 16000, 32/8 heads 449 / 513 / 446, window of 64 over one of 16384 28.6 / 30.2 / 27.9;
-// head size 128, window of 64 over 64 caches of 16384, 32/8 heads 1140 / 1175 / 1107, over one 33.2 / 31.2 / 30.1.
+// The issuers' loops hold one copy of a product each, whatever block takes it.  With copies of their own for the two blocks
+// every warp was slower; probably the instruction caches, which all warps share.  In a loop, us, one issuing thread / two with
+// copies / two without: head size 64, window of 16 over 64 caches of 16000, 32/8 heads 449 / 513 / 446, window of 64 over one
+// of 16384 28.6 / 30.2 / 27.9; head size 128, window of 64 over 64 caches of 16384, 32/8 heads 1140 / 1175 / 1107, over one
+// 33.2 / 31.2 / 30.1.
 #include "pc_attn.h"
 #include "pc_flash.cuh"
 #include "pc_kernels.h"
@@ -280,7 +282,8 @@ parallel_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     const int b = warp >> 2;
     const int r = tid & 127, wi = r % w;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tS = cx.tmem + C::tm_s(b) + lane_sel, tP = cx.tmem + C::TM_P + b * 64 + lane_sel, tO = cx.tmem + C::TM_O + b * D + lane_sel;
+    const uint32_t tS = cx.tmem + C::tm_s(b) + lane_sel, tP = cx.tmem + C::TM_P + b * 64 + lane_sel;
+    const uint32_t tO = cx.tmem + C::TM_O + b * D + lane_sel;
     const float scale_log2 = prm.scale_log2;
     Hooks<C> hk(cx, b);
     uint32_t nd = 0, n_s = 0, n_blk = 0;

@@ -11,11 +11,12 @@
 //
 // Roles, rings, barriers and the tensor memory: pc_flash.cuh.
 //
-// What bounds it: the board's power cap (1000 W) in any loop of these calls, so energy a tile, and beside it the MUFU pipe: a step
-// (a key tile for both blocks of a CTA) takes some 2700 cycles, of which the exponentials keep that pipe busy for 2048, the
-// products the tensor cores as long (head size 64: half as long); at any time at least one block is at its exponentials, but a warp alone
-// does not fill the pipe.  Measured in a loop, whole call, with an S of each block under P (3300 cycles a step) -> with one S
-// for both in turn: 128K tokens in chunks of 8192, 32/8 heads 8.39 -> 7.89 ms; 32/32 heads, chunks of 4096 5.49 -> 5.31 ms; 24/8 heads, ragged 1.39 -> 1.33 ms; head size 64, 32K tokens 0.898 -> 0.886 ms.  Two issuing warps: figures in pc_flash.cuh.
+// What bounds it: the board's power cap (1000 W) in any loop of these calls, so energy a tile, and beside it the MUFU pipe: a
+// step (a key tile for both blocks of a CTA) takes some 2700 cycles, of which the exponentials keep that pipe busy for 2048, the
+// products the tensor cores as long (head size 64: half as long); at any time at least one block is at its exponentials, but a
+// warp alone does not fill the pipe.  Head size 128, in a loop, whole call, with an S of each block under P (3300 cycles a step)
+// -> with one S for both in turn: 128K tokens in chunks of 8192, 32/8 heads 8.39 -> 7.89 ms; 32/32 heads, chunks of 4096
+// 5.49 -> 5.31 ms; 24/8 heads, ragged 1.39 -> 1.33 ms.  Two issuing warps, and head size 64: figures in pc_flash.cuh.
 // A third build, head size 128 on single CTAs, takes short chunks of odd groups (launch_prefill_t).
 //
 // Window scores: the unit that runs the last query tiles of a (chunk, kv-head) group then sweeps the keys once more
@@ -422,7 +423,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const int b = warp >> 2;
     const int r = tid & 127;
     const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tS = cx.tmem + C::tm_s(b) + lane_sel, tP = cx.tmem + C::TM_P + b * 64 + lane_sel, tO = cx.tmem + C::TM_O + b * D + lane_sel;
+    const uint32_t tS = cx.tmem + C::tm_s(b) + lane_sel, tP = cx.tmem + C::TM_P + b * 64 + lane_sel;
+    const uint32_t tO = cx.tmem + C::TM_O + b * D + lane_sel;
     const float scale_log2 = prm.scale_log2;
     Hooks<C> hk(cx, b);
     uint32_t nd = 0, n_s = 0, n_blk = 0, nq = 0, nt = 0, n_lse = 0;
@@ -560,8 +562,9 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 // steps (tiles of its units and of the sweep) than 1.2 times what a CTA or pair gets on average: us without / with, C x L,
 // heads, d: 1 x 2048, 32/8, 64 (3.1 times) 99 / 54; 1 x 8192, 16/4, 64 (1.7) 332 / 231; 2 x 1024, 8/2, 128 (5.5) 41.6 / 38.1;
 // 2 x 2048, 32/8, 128 (0.8) 100 / 105; 3 x 3000, 24/8, 128 (1.0) 215 / 223.  Chunks of a few tiles only where the heads
-// of a group are several units (1 x 206, 14/2, 64 44.0 / 20.9; 1 x 250, 32/8, 64 22.3 / 19.5; 4 x 300, 24/8, 128 43.7 / 38.0; 4 x 500, 28/4, 128 79 / 43): with
-// one unit the count in memory costs more than it spreads (1 x 192, 32/8, 128 20.5 / 21.6; 8 x 512, 8/2, 128 31.5 / 33.3).
+// of a group are several units (1 x 206, 14/2, 64 44.0 / 20.9; 1 x 250, 32/8, 64 22.3 / 19.5; 4 x 300, 24/8, 128 43.7 / 38.0;
+// 4 x 500, 28/4, 128 79 / 43): with one unit the count in memory costs more than it spreads (1 x 192, 32/8, 128 20.5 / 21.6;
+// 8 x 512, 8/2, 128 31.5 / 33.3).
 template <class C>
 static int sweep_slices(const PrefillParams& p, int units) {
   constexpr int NCTA = C::NCTA, BLOCKS = 2 * NCTA;

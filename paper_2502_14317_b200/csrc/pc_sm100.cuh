@@ -16,10 +16,10 @@
 namespace pc {
 
 constexpr unsigned SPIN_BACKOFF_NS = 20;                 // pause between two polls of a barrier
-// The single-thread roles of the CTA-pair kernels (producer, issuers) wait much longer per poll: their waits last
-// thousands of cycles, a wake-up a few hundred cycles late costs them nothing, and every poll they do not make
-// leaves an issue slot to the softmax warp that shares their scheduler (measured: 1.2 % on the 128K shape; 640 ns
-// is too long, and for the softmax warps themselves 0, 20 or 80 ns make no difference).
+// Producers, and the epilogue where it waits for a block's statistics, pause much longer: their waits last thousands of
+// cycles, a wake-up a few hundred cycles late costs them nothing, and every poll they do not make leaves an issue slot to the
+// softmax warp that shares their scheduler (measured when the issuing thread paused as long: 1.2 % on the 128K shape; 640 ns is
+// too long, and for the softmax warps themselves 0, 20 or 80 ns make no difference).  The issuers: Cfg::ISSUER_NS in pc_flash.cuh.
 constexpr unsigned SERVICE_BACKOFF_NS = 320;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

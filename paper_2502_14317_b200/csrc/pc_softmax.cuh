@@ -8,8 +8,9 @@ constexpr float LAZY_RESCALE_LOG2 = 8.0f;      // the reference maximum is raise
 constexpr float MAX_HALF_SUM = 256.0f;         // 2^8, see softmax_tile
 // All exponentials run on the MUFU pipe (ex2), 1024 cycles a tile and warp.  Evaluating every fourth pair as a polynomial on
 // the FMA pipe took a seventh off a tile's cycles and made every workload slower: these kernels run at the board's
-// power cap, and twenty FMA-pipe instructions cost more energy than the two ex2 they replace (128K tokens, 32/8 heads
-// 9244 us with every fourth pair, 8946 with every eighth, 8725 with none; head size 64 at 32K tokens 1018, 977, 953).
+// power cap, and twenty FMA-pipe instructions cost more energy than the two ex2 they replace (with an S of each block and one
+// issuing thread: 128K tokens, 32/8 heads 9244 us with every fourth pair, 8946 with every eighth, 8725 with none; head size 64
+// at 32K tokens 1018, 977, 953).
 
 __device__ __forceinline__ uint64_t dup2(float v) { return pack_f32x2(v, v); }
 
@@ -67,8 +68,8 @@ __device__ __forceinline__ void rescale_rows(uint32_t o_taddr, float alpha) {
 // warp (otherwise the reference is raised to the maximum, the accumulator rescaled and the first half repeated).  Of the first
 // half the sum tells, which is needed anyway: while it is at most 2^8, so is every term; if it is more, or no number, the
 // maximum is looked up.  Of the other half the maximum is found beside the exponentials.  (With the maximum of both halves, in
-// a loop: 128K tokens, 32/8 heads 7894 -> 7839 us, 32/32 heads 5307 -> 5265, head size 64, 32K tokens 886 -> 874.  The second
-// half by its sum as well, with a barrier for the first half's P V: 7842, 5283, 888.)
+// a loop, one issuing thread: 128K tokens, 32/8 heads 7894 -> 7839 us, 32/32 heads 5307 -> 5265, head size 64, 32K tokens
+// 886 -> 874.  The second half by its sum as well, with a barrier for the first half's P V: 7842, 5283, 888.)
 // GEN: tiles with masked columns (columns >= vis; vis <= 0: all) and the first tile of a block; the tiles between
 // run straight-line code (the branches around the masks cost 300 of 1240 cycles).
 // Hooks: on_read() - all logits are in registers; before_p() - called before the accumulator is touched and before
