@@ -32,7 +32,7 @@ constexpr int NT2 = 512;                     // threads per CTA
 constexpr int WARP_EPI = 8, WARP_PRODUCER = 12, WARP_QK = 13, WARP_PV = 14;
 // Registers by role, 128 * (2 * softmax + epilogue + service) = 64 K.  In a loop, us: prefill, 8 chunks of 8192, 32/8 heads
 // 184/80/64 4073, 192/80/48 3983, 192/64/64 3993, 8 of 4096, 32/32 heads 1399 / 1366 / 1378; over caches softmax 184 619, 192 631.
-// With 48 registers the service roles spill (-Xptxas -v: 64 bytes stored, 84 loaded at head size 128 on pairs; 192/64/64
+// With 48 registers the service roles spill (-Xptxas -v: 28 bytes stored, 36 loaded at head size 128 on pairs; 192/64/64
 // spills nothing and is no faster).
 struct Regs { int softmax, epilogue, service; };
 constexpr Regs REGS_PREFILL = {192, 80, 48}, REGS_PARALLEL = {184, 80, 64};

@@ -255,12 +255,15 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           if (d.kind == KIND_DONE) break;
           if (d.kind == KIND_FLASH) {
             flashed = true;
-            for (int j = 0; j < d.n[1]; ++j) {                   // the blocks take turns on S
+            // The blocks take turns on S.  One copy of a product each here and below, whatever block takes it (pc_parallel.cu):
+            // us in loops of 15 ms, copies for the two blocks / one, head size 64, 8 chunks of 4096, 32/8 heads 914 / 860, 22 of 958 278 / 257; head
+            // size 128, 8 of 8192, 32/8 heads 4017 / 3962, 8 of 4096, 32/32 heads 1375 / 1334, 4 of 1257 134 / 128; of Q K^T alone:
+            // nothing, of P V alone: half of it.  In long loops, at the power cap, two thirds of that.
+            for (int j = 0; j < d.n[1]; ++j) {
               const uint32_t k_u32 = is.wait_k();
-#pragma unroll
-              for (int b = 0; b < 2; ++b) {
-                if (j >= d.n[b]) continue;
-                if (j == 0) is.qa[b] = is.wait_q();
+#pragma unroll 1
+              for (int b = j < d.n[0] ? 0 : 1; b < 2; ++b) {
+                if (j == 0) { const uint32_t q = is.wait_q(); if (b) is.qa[1] = q; else is.qa[0] = q; }
                 is.qk(b, k_u32);
               }
               is.free_k();
@@ -310,9 +313,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           if (d.kind == KIND_FLASH) {
             flashed = true;
             for (int j = 0; j < d.n[1]; ++j) {
-#pragma unroll
-              for (int b = 0; b < 2; ++b)
-                if (j < d.n[b]) is.pv(b, j == 0, j == d.n[b] - 1);
+#pragma unroll 1
+              for (int b = j < d.n[0] ? 0 : 1; b < 2; ++b) is.pv(b, j == 0, j == (b ? d.n[1] : d.n[0]) - 1);
               is.free_v();
             }
           } else {
