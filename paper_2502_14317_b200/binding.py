@@ -7,6 +7,7 @@ All calls enqueue on torch's current stream and do not synchronise.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from ctypes import c_float, c_int32, c_int64, c_size_t, c_void_p, c_char_p, POINTER, Structure
 
@@ -34,6 +35,9 @@ class _HotPathArgs(Structure):
                 ("m", c_int32), ("k_keep", c_int32), ("n_score", c_int32), ("clear_status", c_int32)]
 
 
+# outputs and workspaces of hot_path, in the order of csrc/pc_host.cpp
+_HOT_PATH_BUFFERS = ("o", "k_rot", "win_score", "win_lse", "chunk_score", "kept", "idx", "kc", "vc", "pos", "fg", "status", "ws_prefill",
+                     "ws_par")
 _STAGES = (None, "pc_chunk_prefill_attn", "pc_select_chunks", "pc_score_select_chunks", "pc_select_tokens", "pc_gather_kv",
            "pc_parallel_attn")
 
@@ -107,6 +111,12 @@ def load_library():
     lib.pc_parallel_attn_static_scratch_bytes.argtypes = []
     lib.pc_parallel_attn_static.restype = c_int32
     lib.pc_parallel_attn_static.argtypes = [c_int32] * 6 + [c_void_p, c_int32, c_float, c_float] + [c_void_p] * 8
+    try:
+        from . import _pc_host
+    except ImportError as e:
+        raise PcError("_pc_host.so cannot be loaded: build it with `python -m paper_2502_14317_b200.build` (%s)" % e) from e
+    address = lambda f: ctypes.cast(f, c_void_p).value
+    lib.pc_host_hot_path = functools.partial(_pc_host.hot_path, address(lib.pc_hot_path_workspace_bytes), address(lib.pc_hot_path))
     _LIB = lib
     return lib
 
@@ -496,62 +506,17 @@ def hot_path(q, k, v, *, w, rope_theta, m, k_keep, softmax_scale=0.0, chunk_scor
     Hkv = k.shape[2]
     m, k_keep = int(m), int(k_keep)
     get = b.get
-    o, k_rot, win_score, win_lse = get("o"), get("k_rot"), get("win_score"), get("win_lse")
-    kept, idx, kc, vc, pos, fg = get("kept"), get("idx"), get("kc"), get("vc"), get("pos"), get("fg")
-    score, status, ws_prefill, ws_par = get("chunk_score"), get("status"), get("ws_prefill"), get("ws_par")
-    clear = status is None
-    # empty_strided: 1.5 us of host time a tensor, torch.empty 2.4 for a shape of several dimensions
-    new, dev, mk = torch.empty_strided, q.device, m * k_keep
-    if o is None:
-        o = _like(q, q.shape)
-    if k_rot is None:
-        k_rot = _like(k, k.shape)
-    if win_score is None:
-        win_score = new((C, Hkv, L), (Hkv * L, L, 1), dtype=torch.float32, device=dev)
-    if win_lse is None:
-        win_lse = new((C, Hq, w), (Hq * w, w, 1), dtype=torch.float32, device=dev)
-    if chunk_score is not None:
-        score = chunk_score
-    elif score is None:
-        score = new((C,), (1,), dtype=torch.float32, device=dev)
-    if kept is None:
-        kept = new((m,), (1,), dtype=torch.int32, device=dev)
-    if idx is None:
-        idx = new((m, Hkv, k_keep), (Hkv * k_keep, k_keep, 1), dtype=torch.int32, device=dev)
-    if kc is None:
-        kc = new((Hkv, mk, d), (mk * d, d, 1), dtype=torch.bfloat16, device=dev)
-    if vc is None:
-        vc = _like(kc, (Hkv, mk, d))
-    if pos is None:
-        pos = new((Hkv, mk), (mk, 1), dtype=torch.int32, device=dev)
-    if fg is None:
-        fg = new((1, w, Hq, d), (w * Hq * d, Hq * d, d, 1), dtype=torch.bfloat16, device=dev)
-    if status is None:
-        status = new((1,), (1,), dtype=torch.int32, device=dev)
-    desc = _make_desc(q, k, v, o, w, rope_theta, softmax_scale)
-    ref = ctypes.byref(desc)
-    need_par = c_size_t()
-    need = lib.pc_hot_path_workspace_bytes(ref, m, k_keep, ctypes.byref(need_par))
-    need_par = need_par.value
-    if ws_prefill is None or ws_prefill.numel() < need:        # 0: a bad argument, which the call below names
-        ws_prefill = torch.empty(max(need, need_par, 16), dtype=torch.uint8, device=dev)
-    if ws_par is None or ws_par.numel() < need_par:            # (the prefill is done with its own by then)
-        ws_par = ws_prefill if ws_prefill.numel() >= need_par else torch.empty(max(need_par, 16), dtype=torch.uint8, device=dev)
-    if not (k_rot.is_contiguous() and v.is_contiguous()):
-        raise PcError("k_src and v_src must share strides with a contiguous head dimension")
-    # the window is the same in every chunk: take it from chunk 0
-    q_win = None if q.is_contiguous() else _window(q, L, w)
-    args = _HotPathArgs(q.data_ptr(), k.data_ptr(), v.data_ptr(),
-                        q.data_ptr() + (L - w) * Hq * d * 2 if q_win is None else q_win.data_ptr(), o.data_ptr(), k_rot.data_ptr(),
-                        win_score.data_ptr(), win_lse.data_ptr(), _ptr(chunk_score), score.data_ptr(), kept.data_ptr(),
-                        idx.data_ptr(), kc.data_ptr(), vc.data_ptr(), pos.data_ptr(), fg.data_ptr(), status.data_ptr(),
-                        ws_prefill.data_ptr(), ws_prefill.numel(), ws_par.data_ptr(), ws_par.numel(), m, k_keep, score.numel(), clear)
-    failed = c_int32()
-    rc = lib.pc_hot_path(ref, ctypes.byref(args), ctypes.byref(failed), _stream())
+    # new tensors in the place of those that are not there, workspaces, descriptor and call: csrc/pc_host.cpp
+    rc, stage, out = lib.pc_host_hot_path(_stream(), q, k, v, chunk_score, tuple([get(n) for n in _HOT_PATH_BUFFERS]),
+                                          (C, L, Hq, Hkv, d, w, m, k_keep), float(rope_theta), float(softmax_scale))
     if rc != 0:
-        _check(rc, _STAGES[failed.value])
-    res = {"o": o, "k_rot": k_rot, "win_score": win_score, "win_lse": win_lse, "chunk_score": score, "kept": kept, "idx": idx,
-           "kc": kc, "vc": vc, "pos": pos, "fg": fg, "status": status, "ws_prefill": ws_prefill, "ws_par": ws_par}
+        if rc == 1:
+            raise PcError("head dimension must be contiguous")
+        if rc == 2:
+            raise PcError("k_src and v_src must share strides with a contiguous head dimension")
+        _check(rc, _STAGES[stage])
+    score = out[4]
+    res = dict(zip(_HOT_PATH_BUFFERS, out))
     if buffers is not None:
         given = get("chunk_score") if chunk_score is not None else score
         buffers.update(res)

@@ -93,3 +93,49 @@ def test_row_groups_that_fill_the_gpu(fake, B, w, Hq, Hkv, Nk, items):
     fake.fake_reset(-1)
     assert fake.pc_parallel_attn(B, w, Hq, Hkv, 128, Nk, P, 0, 1e4, 0.0, P, P, P, P, P, None, None, P, 1 << 40, None) == 0
     assert fake.fake_window_items() == items
+
+
+def _host_call(lib, q, k, v, given=None, buffers={}, m=2, k_keep=64, w=16):
+    from paper_2502_14317_b200.binding import _HOT_PATH_BUFFERS
+    (C, L, Hq, d), Hkv = q.shape, k.shape[2]
+    lib.fake_reset(-1)
+    rc, stage, out = lib.pc_host_hot_path(0, q, k, v, given, tuple([buffers.get(n) for n in _HOT_PATH_BUFFERS]), (C, L, Hq, Hkv, d, w, m, k_keep),
+                                          1e4, 0.0)
+    return rc, stage, dict(zip(_HOT_PATH_BUFFERS, out))
+
+
+@pytest.mark.parametrize("d,Hq,Hkv,w", [(64, 4, 2, 16), (128, 6, 2, 1), (128, 4, 4, 128)])
+def test_host_side_of_the_whole_path(fake, d, Hq, Hkv, w):
+    """Tensors that are made, kept and replaced, on host memory and the fake runtime."""
+    torch = pytest.importorskip("torch")
+    C, L, m, kk = 3, 300, 2, 64
+    q, k, v = (torch.zeros((C, L, H, d), dtype=torch.bfloat16) for H in (Hq, Hkv, Hkv))
+    shapes = {"o": q.shape, "k_rot": k.shape, "win_score": (C, Hkv, L), "win_lse": (C, Hq, w), "chunk_score": (C,), "kept": (m,),
+              "idx": (m, Hkv, kk), "kc": (Hkv, m * kk, d), "vc": (Hkv, m * kk, d), "pos": (Hkv, m * kk), "fg": (1, w, Hq, d), "status": (1,)}
+    types = {n: torch.bfloat16 if n in ("o", "k_rot", "kc", "vc", "fg") else torch.int32 if n in ("kept", "idx", "pos", "status") else torch.float32
+             for n in shapes}
+    rc, _, a = _host_call(fake, q, k, v, w=w)
+    assert rc == 0 and fake.fake_attention_launches() == 2
+    for n, s in shapes.items():
+        assert a[n].shape == tuple(s) and a[n].dtype == types[n] and a[n].is_contiguous(), n
+    assert a["ws_par"] is a["ws_prefill"] or a["ws_par"].numel() > a["ws_prefill"].numel()
+    # everything is kept, a score of the caller's is passed on, a workspace that is too small is replaced
+    score = torch.zeros(C)
+    rc, _, b = _host_call(fake, q, k, v, given=score, buffers=a, w=w)
+    assert rc == 0 and b["chunk_score"] is score and all(b[n] is a[n] for n in a if n != "chunk_score")
+    small = torch.empty(16, dtype=torch.uint8)
+    rc, _, b = _host_call(fake, q, k, v, buffers=dict(a, ws_prefill=small, ws_par=small, pos=None), w=w)
+    assert rc == 0 and b["ws_prefill"].numel() == a["ws_prefill"].numel() and b["ws_par"].numel() >= 16 and b["pos"] is not a["pos"]
+    assert all(b[n] is a[n] for n in shapes if n != "pos")
+    # head-major queries go through a copy of the window; other strides of v are refused, as is a head dimension that is not innermost
+    heads = torch.zeros((C, Hq, L, d), dtype=torch.bfloat16).transpose(1, 2)
+    assert _host_call(fake, heads, k, v, w=w)[0] == 0
+    assert _host_call(fake, q, k, torch.zeros((C, Hkv, L, d), dtype=torch.bfloat16).transpose(1, 2), w=w)[0] == (2 if Hkv > 1 else 0)
+    assert _host_call(fake, torch.zeros((C, L, d, Hq), dtype=torch.bfloat16).transpose(2, 3), k, v, w=w)[0] == 1
+    # the library's own refusals come back with their stage, arguments that are none as exceptions
+    assert _host_call(fake, q, k, v, given=torch.zeros(C + 1), w=w)[:2] == (-1, 2)
+    assert _host_call(fake, q, k, v, w=w, m=C + 1)[0] == -1
+    with pytest.raises(TypeError):
+        _host_call(fake, q, k, v, given=3.0, w=w)
+    with pytest.raises(RuntimeError):
+        _host_call(fake, q, k, v, w=w, k_keep=-1)
