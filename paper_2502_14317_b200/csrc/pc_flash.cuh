@@ -57,10 +57,10 @@ struct Cfg {
   static constexpr bool TWO_S = D == 64;
   static constexpr uint32_t TM_P = TWO_S ? 256 : 128, TM_O = TWO_S ? 384 : 256;
   static constexpr __host__ __device__ uint32_t tm_s(int b) { return TWO_S ? 128u * b : 0u; }
-  // Pause of the issuers between two polls, ns.  us, 20 / 0: head size 64, windows of 64 over 32 caches of 8192, 14/2 heads
-  // 112.4 / 111.0, over one of 16384, 32/8 heads 28.1 / 27.8, 8 chunks of 4096 the same; head size 128, within the noise of a
-  // loop at the power cap: 8 chunks of 8192 3983 / 3941, 8 of 4096, 32/32 heads 1366 / 1378, windows over 32 caches of 16384 625 / 619
-  static constexpr unsigned ISSUER_NS = D == 64 ? 0 : 20;
+  // The issuers poll without a pause.  us, 20 ns / none, head size 128, in loops: 8 chunks of 8192, 32/8 heads 4027 / 3989, 2 of 873,
+  // 32/32 heads 51.0 / 50.8, 5 of 298, 28/4 heads 41.7 / 41.2, windows of 64 over 64 caches of 16384 1207 / 1191, two 51.2 / 50.5, one of
+  // 4096 20.6 / 20.5; head size 64, windows of 64 over 32 caches of 8192, 14/2 heads 112.4 / 111.0.
+  static constexpr unsigned ISSUER_NS = 0;
   static constexpr int CODE = PAIR ? 200 : 100;            // wait codes in the status word
 };
 
