@@ -133,6 +133,10 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
                    const __grid_constant__ CUtensorMap tm_kw, const __grid_constant__ CUtensorMap tm_vw,
                    const __grid_constant__ DecodeParams prm) {
   using Y = Lay<D, N, DEEP>;
+  // Pause between two polls: none where a CTA has its SM for itself (few items, every wait on the chain of a tile): one token over a
+  // cache of 16401 15.60 -> 15.38 us, over two of 16000 25.27 -> 25.15, 2 over eight of 4000, 28/4 heads 15.98 -> 15.88.  With two CTAs an
+  // SM it helps some shapes and costs others: 4 over eight of 9000, head size 64 35.8 -> 34.6, 2 over 32 of 16000 159 -> 161.
+  constexpr unsigned POLL_NS = DEEP ? 0 : SPIN_BACKOFF_NS;
   extern __shared__ __align__(1024) uint8_t smem[];
   Misc<N>& mi = *reinterpret_cast<Misc<N>*>(smem + Y::OFF_MISC);
   volatile int* const abort_flag = &mi.abort_flag;
@@ -248,7 +252,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
     if (elect_one()) {
       uint32_t kv = n_first;
       for (; kv < n_kv && !*abort_flag; ++kv) {
-        if (!mbar_wait(&mi.kv_free[kv % Y::NS], free_par(kv / Y::NS), abort_flag, prm.status, WD_FREE)) break;
+        if (!mbar_wait_ns<POLL_NS>(&mi.kv_free[kv % Y::NS], free_par(kv / Y::NS), abort_flag, prm.status, WD_FREE)) break;
         load_half(kv);
       }
       for (uint32_t i = kv > (uint32_t)Y::NS ? kv - Y::NS : 0; i < kv; ++i)             // every copy has landed before exit
@@ -263,7 +267,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
       constexpr uint32_t V_LBO = D == 128 ? 16384 : 1024;
       auto issue_qk = [&](int i) {
         const uint32_t kv = 2 * (uint32_t)i, st = kv % Y::NS;
-        mbar_wait(&mi.kv_full[st], full_par(kv / Y::NS), abort_flag, prm.status, WD_KV);
+        mbar_wait_ns<POLL_NS>(&mi.kv_full[st], full_par(kv / Y::NS), abort_flag, prm.status, WD_KV);
         tc_fence_after_sync();
         const uint32_t k = sK + st * Y::TILE_BYTES;
 #pragma unroll
@@ -277,8 +281,8 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
       for (int i = 0; i < n && !*abort_flag; ++i) {
         if (i + 1 < n) issue_qk(i + 1);                       // P of tile i-1 was there, so its S buffer has been read
         const uint32_t kv = 2 * (uint32_t)i + 1, st = kv % Y::NS;
-        mbar_wait(&mi.kv_full[st], full_par(kv / Y::NS), abort_flag, prm.status, WD_KV);
-        mbar_wait(&mi.p_full, full_par(i), abort_flag, prm.status, WD_P);
+        mbar_wait_ns<POLL_NS>(&mi.kv_full[st], full_par(kv / Y::NS), abort_flag, prm.status, WD_KV);
+        mbar_wait_ns<POLL_NS>(&mi.p_full, full_par(i), abort_flag, prm.status, WD_P);
         tc_fence_after_sync();
         const uint32_t v = sK + st * Y::TILE_BYTES;
 #pragma unroll
@@ -299,7 +303,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
 #pragma unroll
     for (int r = 0; r < N; ++r) l[r] = 0.0f;
     for (int i = 0; i < n; ++i) {
-      mbar_wait(&mi.s_full[i & 1], full_par(i >> 1), abort_flag, prm.status, WD_S);
+      mbar_wait_ns<POLL_NS>(&mi.s_full[i & 1], full_par(i >> 1), abort_flag, prm.status, WD_S);
       tc_fence_after_sync();
       float s[N];
       load_cols<N>(tmem + (i & 1) * N + lane_sel, s);
@@ -347,7 +351,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
         }
         named_barrier_sync(1, 128);
         if (i > 0) {
-          mbar_wait(&mi.pv_done, full_par(i - 1), abort_flag, prm.status, WD_PV);
+          mbar_wait_ns<POLL_NS>(&mi.pv_done, full_par(i - 1), abort_flag, prm.status, WD_PV);
           tc_fence_after_sync();
           float o[N];
           load_cols<N>(tO + lane_sel, o);
@@ -363,7 +367,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
 #pragma unroll
         for (int r = 0; r < N; ++r) l[r] *= mi.red[0][r];
       }
-      if (i > 0) mbar_wait(&mi.pv_done, full_par(i - 1), abort_flag, prm.status, WD_PV);   // P of the tile before has been read
+      if (i > 0) mbar_wait_ns<POLL_NS>(&mi.pv_done, full_par(i - 1), abort_flag, prm.status, WD_PV);   // P of the tile before has been read
       uint8_t* const pdst = smem + Y::OFF_P + (tid / 64) * (N * 128) + (tid % 8) * 2;
 #pragma unroll
       for (int q = 0; q < N / 8; ++q) {
@@ -384,7 +388,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_const
       if (lane == 0) mbar_arrive(&mi.p_full);
     }
     // ---- row sums over the keys, then O^T (thread = head-dim column)
-    mbar_wait(&mi.pv_done, full_par(n - 1), abort_flag, prm.status, WD_PV);
+    mbar_wait_ns<POLL_NS>(&mi.pv_done, full_par(n - 1), abort_flag, prm.status, WD_PV);
     tc_fence_after_sync();
     const float row_sum = lane_sums<N>(l, lane);
     if (lane < N) mi.red[warp][lane] = row_sum;
