@@ -156,3 +156,22 @@ def test_score_and_chunk_ranking_in_one_call(C, Hq, w, m):
     torch.cuda.synchronize()
     assert torch.equal(score_a.view(torch.int32), score_b.view(torch.int32)) and torch.equal(kept_a, kept_b)
     assert np.array_equal(kept_b.cpu().numpy(), orc.select_chunks(score_b.cpu().numpy(), m, True))
+
+
+@pytest.mark.parametrize("m,Hkv,k,d", [(5, 32, 959, 128), (5, 32, 961, 128), (3, 8, 12807, 64), (16, 31, 621, 64), (12, 32, 1024, 128)])
+def test_gather_on_both_sides_of_its_grid_rule(m, Hkv, k, d):
+    """150 MiB read and written is where the grid changes; copies to the bit, padding rows as zeros, the last rows included."""
+    import paper_2502_14317_b200 as pc
+    C, L = m + 1, k // 4 + 77
+    g = torch.Generator(device="cuda").manual_seed(k)
+    ks, vs = (torch.randn((C, L, Hkv, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    kept = torch.randperm(C, generator=g, device="cuda")[:m].sort().values.int()
+    idx = torch.randint(-1, L, (m, Hkv, k), generator=g, device="cuda", dtype=torch.int32)
+    kc, vc, pos = pc.gather_kv(ks, vs, kept, idx)
+    rows = idx.permute(1, 0, 2).reshape(Hkv, m * k)
+    assert torch.equal(pos, rows)
+    hk, ch = torch.arange(Hkv, device="cuda")[:, None], kept.long().repeat_interleave(k)[None]
+    for got, src in ((kc, ks), (vc, vs)):
+        want = src[ch, rows.clamp(min=0).long(), hk]
+        want[rows < 0] = 0
+        assert torch.equal(got, want)
