@@ -111,14 +111,21 @@ def load_library():
     lib.pc_parallel_attn_static_scratch_bytes.argtypes = []
     lib.pc_parallel_attn_static.restype = c_int32
     lib.pc_parallel_attn_static.argtypes = [c_int32] * 6 + [c_void_p, c_int32, c_float, c_float] + [c_void_p] * 8
-    try:
-        from . import _pc_host
-    except ImportError as e:
-        raise PcError("_pc_host.so cannot be loaded: build it with `python -m paper_2502_14317_b200.build` (%s)" % e) from e
-    address = lambda f: ctypes.cast(f, c_void_p).value
-    lib.pc_host_hot_path = functools.partial(_pc_host.hot_path, address(lib.pc_hot_path_workspace_bytes), address(lib.pc_hot_path))
     _LIB = lib
     return lib
+
+
+def _host_hot_path(lib):
+    """hot_path of csrc/pc_host.cpp on this library's entry points."""
+    call = getattr(lib, "_host_hot_path", None)
+    if call is None:
+        try:
+            from . import _pc_host
+        except ImportError as e:
+            raise PcError("_pc_host.so cannot be loaded: build it with `python -m paper_2502_14317_b200.build` (%s)" % e) from e
+        address = lambda f: ctypes.cast(f, c_void_p).value
+        call = lib._host_hot_path = functools.partial(_pc_host.hot_path, address(lib.pc_hot_path_workspace_bytes), address(lib.pc_hot_path))
+    return call
 
 
 def version() -> int:
@@ -507,8 +514,8 @@ def hot_path(q, k, v, *, w, rope_theta, m, k_keep, softmax_scale=0.0, chunk_scor
     m, k_keep = int(m), int(k_keep)
     get = b.get
     # new tensors in the place of those that are not there, workspaces, descriptor and call: csrc/pc_host.cpp
-    rc, stage, out = lib.pc_host_hot_path(_stream(), q, k, v, chunk_score, tuple([get(n) for n in _HOT_PATH_BUFFERS]),
-                                          (C, L, Hq, Hkv, d, w, m, k_keep), float(rope_theta), float(softmax_scale))
+    rc, stage, out = _host_hot_path(lib)(_stream(), q, k, v, chunk_score, tuple([get(n) for n in _HOT_PATH_BUFFERS]),
+                                         (C, L, Hq, Hkv, d, w, m, k_keep), float(rope_theta), float(softmax_scale))
     if rc != 0:
         if rc == 1:
             raise PcError("head dimension must be contiguous")

@@ -96,11 +96,11 @@ def test_row_groups_that_fill_the_gpu(fake, B, w, Hq, Hkv, Nk, items):
 
 
 def _host_call(lib, q, k, v, given=None, buffers={}, m=2, k_keep=64, w=16):
-    from paper_2502_14317_b200.binding import _HOT_PATH_BUFFERS
+    from paper_2502_14317_b200.binding import _HOT_PATH_BUFFERS, _host_hot_path
     (C, L, Hq, d), Hkv = q.shape, k.shape[2]
     lib.fake_reset(-1)
-    rc, stage, out = lib.pc_host_hot_path(0, q, k, v, given, tuple([buffers.get(n) for n in _HOT_PATH_BUFFERS]), (C, L, Hq, Hkv, d, w, m, k_keep),
-                                          1e4, 0.0)
+    rc, stage, out = _host_hot_path(lib)(0, q, k, v, given, tuple([buffers.get(n) for n in _HOT_PATH_BUFFERS]), (C, L, Hq, Hkv, d, w, m, k_keep),
+                                         1e4, 0.0)
     return rc, stage, dict(zip(_HOT_PATH_BUFFERS, out))
 
 
@@ -108,6 +108,8 @@ def _host_call(lib, q, k, v, given=None, buffers={}, m=2, k_keep=64, w=16):
 def test_host_side_of_the_whole_path(fake, d, Hq, Hkv, w):
     """Tensors that are made, kept and replaced, on host memory and the fake runtime."""
     torch = pytest.importorskip("torch")
+    from paper_2502_14317_b200 import build
+    build.build_library()
     C, L, m, kk = 3, 300, 2, 64
     q, k, v = (torch.zeros((C, L, H, d), dtype=torch.bfloat16) for H in (Hq, Hkv, Hkv))
     shapes = {"o": q.shape, "k_rot": k.shape, "win_score": (C, Hkv, L), "win_lse": (C, Hq, w), "chunk_score": (C,), "kept": (m,),
