@@ -38,6 +38,7 @@ class _HotPathArgs(Structure):
 # outputs and workspaces of hot_path, in the order of csrc/pc_host.cpp
 _HOT_PATH_BUFFERS = ("o", "k_rot", "win_score", "win_lse", "chunk_score", "kept", "idx", "kc", "vc", "pos", "fg", "status", "ws_prefill",
                      "ws_par")
+_BAD_INPUT = "q, k and v must be bfloat16, k and v [C, L, Hkv, d] with the C, L and d of q, everything on one device"
 _STAGES = (None, "pc_chunk_prefill_attn", "pc_select_chunks", "pc_score_select_chunks", "pc_select_tokens", "pc_gather_kv",
            "pc_parallel_attn")
 
@@ -502,7 +503,7 @@ def hot_path(q, k, v, *, w, rope_theta, m, k_keep, softmax_scale=0.0, chunk_scor
 
     ``chunk_score`` (device fp32 [C]) stands for the self-information of Eq. 3; if None the
     single-layer stand-in computed from the window log-sum-exp is used.
-    ``buffers`` (dict) lets repeated calls reuse outputs and workspaces.
+    ``buffers`` (dict) lets repeated calls reuse outputs and workspaces; what is too small for this call is replaced in it.
     """
     b = {} if buffers is None else buffers
     lib = load_library()
@@ -521,6 +522,10 @@ def hot_path(q, k, v, *, w, rope_theta, m, k_keep, softmax_scale=0.0, chunk_scor
             raise PcError("head dimension must be contiguous")
         if rc == 2:
             raise PcError("k_src and v_src must share strides with a contiguous head dimension")
+        if rc == 3:
+            raise PcError(_BAD_INPUT)
+        if rc == 4:
+            raise PcError("buffers[%r] is of another type or device, or not contiguous" % _HOT_PATH_BUFFERS[stage])
         _check(rc, _STAGES[stage])
     score = out[4]
     res = dict(zip(_HOT_PATH_BUFFERS, out))

@@ -17,8 +17,8 @@ namespace {
 
 // outputs and workspaces, in the order of binding.py's _HOT_PATH_BUFFERS
 enum { O, K_ROT, WIN_SCORE, WIN_LSE, SCORE, KEPT, IDX, KC, VC, POS, FG, STATUS, WS_PREFILL, WS_PAR, N_BUFFERS };
-// result codes beside the library's own
-enum { NOT_INNERMOST = 1, NOT_CONTIGUOUS = 2 };
+// result codes beside the library's own; with BAD_BUFFER the stage is the buffer's place
+enum { NOT_INNERMOST = 1, NOT_CONTIGUOUS = 2, BAD_INPUT = 3, BAD_BUFFER = 4 };
 
 using ws_bytes_fn = size_t (*)(const pc_prefill_desc*, int32_t, int32_t, size_t*);
 using hot_path_fn = int32_t (*)(const pc_prefill_desc*, const pc_hot_path_args*, int32_t*, void*);
@@ -33,30 +33,47 @@ struct Call {
   void* stream;
   int32_t rc, stage = 0;
 
-  void make(int i, at::IntArrayRef sizes, at::ScalarType type) {
-    if (t[i].defined()) return;
+  // Whether buffer i can be written as contiguous elements of that type (any type for a workspace, whose bytes are counted).
+  bool writable(int i, at::ScalarType type) {
+    if (t[i].scalar_type() == type && t[i].device() == q.device() && t[i].is_contiguous()) return true;
+    rc = BAD_BUFFER; stage = i;
+    return false;
+  }
+  // Buffer i of these sizes.  One that is there may be of an earlier call with other sizes: it serves as it is, or through a view of its
+  // first elements where it has enough, and is replaced where it has not.  False: one that cannot be written.
+  bool make(int i, at::IntArrayRef sizes, at::ScalarType type) {
+    if (t[i].defined()) {
+      if (i == O && t[i].sizes().equals(sizes) && t[i].scalar_type() == type && t[i].device() == q.device()) return true;   // any strides
+      if (!writable(i, type)) return false;
+      if (t[i].sizes().equals(sizes)) return true;
+      int64_t n = 1;
+      for (int64_t s : sizes) n *= s;
+      if (n >= 0 && t[i].numel() >= n) {
+        t[i] = t[i].view(-1).narrow(0, 0, n).view(sizes);
+        made[i] = true;
+        return true;
+      }
+    }
     t[i] = at::empty(sizes, at::TensorOptions().dtype(type).device(q.device()));
-    made[i] = true;
+    return made[i] = true;
   }
   void operator()();
 };
 
 void Call::operator()() {
-  const bool clear = !t[STATUS].defined();
+  // The launches go by q's sizes alone: keys and values of others would be read out of range.
+  for (const at::Tensor* x : {&q, &k, &v})
+    if (x->scalar_type() != at::kBFloat16 || x->device() != q.device()) { rc = BAD_INPUT; return; }
+  if (!k.sizes().equals({C, L, Hkv, d}) || !v.sizes().equals(k.sizes()) || (has_given && given.device() != q.device())) { rc = BAD_INPUT; return; }
   const int64_t mk = m * k_keep;
-  make(O, q.sizes(), at::kBFloat16);
-  make(K_ROT, k.sizes(), at::kBFloat16);
-  make(WIN_SCORE, {C, Hkv, L}, at::kFloat);
-  make(WIN_LSE, {C, Hq, w}, at::kFloat);
   if (has_given) t[SCORE] = given;
-  else make(SCORE, {C}, at::kFloat);
-  make(KEPT, {m}, at::kInt);
-  make(IDX, {m, Hkv, k_keep}, at::kInt);
-  make(KC, {Hkv, mk, d}, at::kBFloat16);
-  make(VC, {Hkv, mk, d}, at::kBFloat16);
-  make(POS, {Hkv, mk}, at::kInt);
-  make(FG, {1, w, Hq, d}, at::kBFloat16);
-  make(STATUS, {1}, at::kInt);
+  if (!(make(O, q.sizes(), at::kBFloat16) && make(K_ROT, k.sizes(), at::kBFloat16) && make(WIN_SCORE, {C, Hkv, L}, at::kFloat) &&
+        make(WIN_LSE, {C, Hq, w}, at::kFloat) && (has_given || make(SCORE, {C}, at::kFloat)) && make(KEPT, {m}, at::kInt) &&
+        make(IDX, {m, Hkv, k_keep}, at::kInt) && make(KC, {Hkv, mk, d}, at::kBFloat16) && make(VC, {Hkv, mk, d}, at::kBFloat16) &&
+        make(POS, {Hkv, mk}, at::kInt) && make(FG, {1, w, Hq, d}, at::kBFloat16)))
+    return;
+  const bool clear = !t[STATUS].defined() || t[STATUS].numel() < 1;
+  if (!make(STATUS, {1}, at::kInt)) return;
 
   pc_prefill_desc desc;
   desc.C = (int32_t)C; desc.L = (int32_t)L; desc.w = (int32_t)w; desc.Hq = (int32_t)Hq; desc.Hkv = (int32_t)Hkv; desc.d = (int32_t)d;
@@ -69,6 +86,8 @@ void Call::operator()() {
     if (in[i]->stride(3) != 1) { rc = NOT_INNERMOST; return; }
     for (int j = 0; j < 3; ++j) strides[i][j] = in[i]->stride(j);
   }
+  for (int i : {WS_PREFILL, WS_PAR})
+    if (t[i].defined() && !writable(i, t[i].scalar_type())) return;
   size_t need_par = 0;
   const size_t need = ws_bytes(&desc, (int32_t)m, (int32_t)k_keep, &need_par);
   auto scratch = [&](size_t bytes) { return at::empty({(int64_t)std::max<size_t>(bytes, 16)}, at::TensorOptions().dtype(at::kByte).device(q.device())); };
@@ -104,7 +123,7 @@ void Call::operator()() {
 }
 
 // hot_path(ws_bytes, run, stream, q, k, v, chunk_score or None, buffers, (C, L, Hq, Hkv, d, w, m, k_keep), rope_theta, softmax_scale)
-// -> (result code, stage, buffers): those given, or new ones in the place of None and of workspaces that are too small
+// -> (result code, stage, buffers): those given, or new ones in the place of None and of those that are too small
 PyObject* hot_path(PyObject*, PyObject* args) {
   HANDLE_TH_ERRORS
   unsigned long long ws_bytes, run, stream;

@@ -141,3 +141,50 @@ def test_host_side_of_the_whole_path(fake, d, Hq, Hkv, w):
         _host_call(fake, q, k, v, given=3.0, w=w)
     with pytest.raises(RuntimeError):
         _host_call(fake, q, k, v, w=w, k_keep=-1)
+
+
+def _path_shapes(C, L, Hq, Hkv, d, w, m, k_keep):
+    return {"o": (C, L, Hq, d), "k_rot": (C, L, Hkv, d), "win_score": (C, Hkv, L), "win_lse": (C, Hq, w), "chunk_score": (C,), "kept": (m,),
+            "idx": (m, Hkv, k_keep), "kc": (Hkv, m * k_keep, d), "vc": (Hkv, m * k_keep, d), "pos": (Hkv, m * k_keep), "fg": (1, w, Hq, d),
+            "status": (1,)}
+
+
+def _zeros(torch, C, L, Hq, Hkv, d):
+    return tuple(torch.zeros((C, L, H, d), dtype=torch.bfloat16) for H in (Hq, Hkv, Hkv))
+
+
+def test_whole_path_with_buffers_of_another_call(fake):
+    """The launches go by the sizes of this call: what an earlier call of other sizes left is big enough, or replaced, and has this call's shape."""
+    torch = pytest.importorskip("torch")
+    sizes = [(3, 300, 4, 2, 64, 16, 2, 64), (6, 900, 8, 2, 128, 16, 4, 128), (2, 200, 4, 4, 64, 8, 1, 64), (3, 300, 4, 2, 64, 64, 2, 65), (3, 300, 4, 1, 64, 64, 3, 64)]
+    kept = {}
+    for C, L, Hq, Hkv, d, w, m, kk in sizes:
+        rc, _, kept = _host_call(fake, *_zeros(torch, C, L, Hq, Hkv, d), buffers=kept, w=w, m=m, k_keep=kk)
+        assert rc == 0
+        for n, s in _path_shapes(C, L, Hq, Hkv, d, w, m, kk).items():
+            assert kept[n].shape == s and kept[n].is_contiguous(), n
+    # the caller's own memory is written wherever it is big enough
+    C, L, Hq, Hkv, d, w, m, kk = sizes[0]
+    flat = torch.empty(Hkv * m * kk * d + 8, dtype=torch.bfloat16)
+    strided = torch.empty((C, Hq, L, d), dtype=torch.bfloat16).transpose(1, 2)
+    rc, _, out = _host_call(fake, *_zeros(torch, C, L, Hq, Hkv, d), buffers={"kc": flat, "vc": flat[8:].view(-1, d), "o": strided}, w=w, m=m, k_keep=kk)
+    assert rc == 0 and out["kc"].data_ptr() == flat.data_ptr() and out["vc"].data_ptr() == flat[8:].data_ptr() and out["o"] is strided
+    assert out["kc"].shape == out["vc"].shape == (Hkv, m * kk, d)
+
+
+def test_whole_path_refuses_tensors_that_do_not_go_together(fake):
+    torch = pytest.importorskip("torch")
+    from paper_2502_14317_b200.binding import _HOT_PATH_BUFFERS
+    q, k, v = _zeros(torch, 6, 900, 4, 2, 64)
+    assert _host_call(fake, q, k, v)[0] == 0
+    for wrong in (k[:3], k[:, :300], k[..., :32], k.float(), k.half()):
+        assert _host_call(fake, q, wrong, v)[0] == 3 and fake.fake_attention_launches() == 0
+        assert _host_call(fake, q, k, wrong)[0] == 3 and fake.fake_attention_launches() == 0
+    assert _host_call(fake, q, k, v[:, :, :1])[0] == 3 and _host_call(fake, q.float(), k, v)[0] == 3
+    assert _host_call(fake, q, k.to("meta"), v)[0] == 3 and _host_call(fake, q, k, v, given=torch.zeros(6, device="meta"))[0] == 3
+    good = _host_call(fake, q, k, v)[2]
+    for n, t in good.items():
+        wrong = [t.to("meta")] + ([t.new_empty(t.numel() * 2)[::2]] if t.numel() > 1 else []) + ([] if n.startswith("ws") else [t.double()])
+        for bad in wrong:
+            assert _host_call(fake, q, k, v, buffers=dict(good, **{n: bad}))[:2] == (4, _HOT_PATH_BUFFERS.index(n)), n
+            assert fake.fake_attention_launches() == 0
