@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import functools
+import math
 import os
 from ctypes import c_float, c_int32, c_int64, c_size_t, c_void_p, c_char_p, POINTER, Structure
 
@@ -184,13 +185,36 @@ def _need_cuda(*tensors):
             raise PcError("tensors must live on a CUDA device")
 
 
+def _kept(b, name, shape, dtype, device):
+    """Tensor ``name`` of the buffers b for an output of this shape, as csrc/pc_host.cpp takes it: as it is, or a view of its first elements
+    where it has enough of them (an earlier call had other sizes); None (make a new one) where it is absent or too small."""
+    t = b.get(name)
+    if t is None:
+        return None
+    if t.dtype is not dtype or t.device != device or not (t.is_contiguous() or (name == "o" and t.shape == shape)):
+        raise PcError("buffers[%r] is of another type or device, or not contiguous" % name)
+    if t.shape == shape:
+        return t
+    n = math.prod(shape)
+    return t.view(-1)[:n].view(shape) if t.numel() >= n else None
+
+
+def _check_inputs(q, k, v, dev):
+    """The launches go by q's sizes: keys and values of others would be read out of range."""
+    C, L, _, d = q.shape
+    ks, bf16 = k.shape, torch.bfloat16
+    if not (ks == v.shape and len(ks) == 4 and ks[0] == C and ks[1] == L and ks[3] == d and q.dtype is k.dtype is v.dtype is bf16 and
+            q.device == k.device == v.device == dev):
+        raise PcError(_BAD_INPUT)
+
+
 def _make_desc(q, k, v, o, w, rope_theta, softmax_scale):
     C, L, Hq, d = q.shape
     Hkv = k.shape[2]
-    strides = [t.stride() for t in (q, k, v, o)]
-    if any(st[3] != 1 for st in strides):
+    sq, sk, sv, so = q.stride(), k.stride(), v.stride(), o.stride()
+    if not sq[3] == sk[3] == sv[3] == so[3] == 1:
         raise PcError("head dimension must be contiguous")
-    return _PrefillDesc(C, L, w, Hq, Hkv, d, float(rope_theta), float(softmax_scale), *(st[:3] for st in strides))
+    return _PrefillDesc(C, L, w, Hq, Hkv, d, float(rope_theta), float(softmax_scale), sq[:3], sk[:3], sv[:3], so[:3])
 
 
 def chunk_prefill_attn_workspace_bytes(C, L, w, Hq, Hkv, d, k_rot_in_workspace=False) -> int:
@@ -230,9 +254,9 @@ def chunk_prefill_attn(q, k, v, *, w, rope_theta, softmax_scale=0.0, want_lse=Fa
         workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
     if chunk_len is not None and (chunk_len.dtype != torch.int32 or chunk_len.numel() != C or not chunk_len.is_cuda):
         raise PcError("chunk_len must be an int32 CUDA tensor with one entry per chunk")
-    rc = lib.pc_chunk_prefill_attn(ctypes.byref(desc), _ptr(q), _ptr(k), _ptr(v), _ptr(chunk_len), _ptr(o), _ptr(k_rot),
-                                   _ptr(lse), _ptr(win_score), _ptr(win_lse), _ptr(status), _ptr(workspace),
-                                   workspace.numel(), _stream())
+    rc = lib.pc_chunk_prefill_attn(ctypes.byref(desc), q.data_ptr(), k.data_ptr(), v.data_ptr(), _ptr(chunk_len), o.data_ptr(),
+                                   k_rot.data_ptr(), _ptr(lse), win_score.data_ptr(), win_lse.data_ptr(), status.data_ptr(),
+                                   workspace.data_ptr(), workspace.numel(), _stream())
     _check(rc, "pc_chunk_prefill_attn")
     return {"o": o, "k_rot": k_rot, "win_score": win_score, "win_lse": win_lse, "lse": lse, "status": status,
             "workspace": workspace}
@@ -356,9 +380,9 @@ def queue_update(state, chunk_score, chunk_id0, lower_is_better=True):
     _need_cuda(chunk_score)
     if chunk_score.dtype != torch.float32 or not chunk_score.is_contiguous():
         raise PcError("chunk_score must be contiguous float32")
-    _check(lib.pc_queue_update(_ptr(chunk_score), chunk_score.numel(), int(chunk_id0), 1 if lower_is_better else 0,
-                               state["m"], _ptr(state["q_score"]), _ptr(state["q_chunk"]), _ptr(state["slot_src"]),
-                               _stream()), "pc_queue_update")
+    _check(lib.pc_queue_update(chunk_score.data_ptr(), chunk_score.numel(), int(chunk_id0), 1 if lower_is_better else 0, state["m"],
+                               state["q_score"].data_ptr(), state["q_chunk"].data_ptr(), state["slot_src"].data_ptr(), _stream()),
+           "pc_queue_update")
     return state["slot_src"]
 
 
@@ -390,9 +414,9 @@ def queue_select_gather(state, win_score, k_src, v_src, n_cand):
     if not _same_rows(k_src, v_src):
         raise PcError("k_src and v_src must share strides with a contiguous head dimension")
     strides = (c_int64 * 3)(k_src.stride(0), k_src.stride(1), k_src.stride(2))
-    _check(lib.pc_queue_select_gather(_ptr(win_score), _ptr(k_src), _ptr(v_src), strides, _ptr(state["slot_src"]), state["m"],
-                                      Hkv, L, int(n_cand), state["k"], d, _ptr(state["q_k"]), _ptr(state["q_v"]),
-                                      _ptr(state["q_pos"]), _stream()), "pc_queue_select_gather")
+    _check(lib.pc_queue_select_gather(win_score.data_ptr(), k_src.data_ptr(), v_src.data_ptr(), strides, state["slot_src"].data_ptr(),
+                                      state["m"], Hkv, L, int(n_cand), state["k"], d, state["q_k"].data_ptr(), state["q_v"].data_ptr(),
+                                      state["q_pos"].data_ptr(), _stream()), "pc_queue_select_gather")
 
 
 def queue_emit(state, k_out=None, v_out=None, pos_out=None, kept_out=None):
@@ -561,29 +585,41 @@ def hot_path_streaming(q, k, v, *, w, rope_theta, m, k_keep, batch=None, softmax
         if batch is None:
             raise PcError("hot_path_streaming needs a batch size for whole tensors")
         batches = [(q[c0:c0 + batch], k[c0:c0 + batch], v[c0:c0 + batch]) for c0 in range(0, q.shape[0], batch)]
+    for of_batch in batches if isinstance(q, (list, tuple)) else (batches[0], batches[-1]):   # whole tensors: those between are as the first
+        _check_inputs(*of_batch, batches[0][0].device)
     q0, k0, v0 = batches[0]
     _, L0, Hq, d = q0.shape
     Hkv = k0.shape[2]
     dev = q0.device
     n_max = max(bq.shape[0] for bq, _, _ in batches)
-    if "queue" not in b:
+    f32, i32, bf16 = torch.float32, torch.int32, torch.bfloat16
+    qu = b.get("queue")
+    if qu is None or (qu["m"], qu["Hkv"], qu["k"], qu["d"], qu["q_k"].device) != (m, Hkv, k_keep, d, dev):
         b["queue"] = queue_init(m, Hkv, k_keep, d, dev)
     else:
         lib = load_library()
-        _check(lib.pc_queue_init(m, _ptr(b["queue"]["q_score"]), _ptr(b["queue"]["q_chunk"]), _stream()), "pc_queue_init")
+        _check(lib.pc_queue_init(m, _ptr(qu["q_score"]), _ptr(qu["q_chunk"]), _stream()), "pc_queue_init")
     if "ids" not in b or b["ids"].numel() < n_max:
         b["ids"] = torch.arange(n_max, dtype=torch.int32, device=dev)
     qu = b["queue"]
+    b["status"] = _kept(b, "status", (1,), i32, dev)
     c0 = 0
-    k_win = None
+    k_win, fitted = None, {}
     for bq, bk, bv in batches:
-        n, L = bq.shape[0], bq.shape[1]
+        n, L, hq, dq = bq.shape
+        hkv = bk.shape[2]
         if L - w < k_keep:
             raise PcError("a chunk of %d tokens has fewer than k_keep = %d context tokens" % (L, k_keep))
         pb = b.setdefault("pre_%dx%d" % (n, L), {})            # buffers per batch shape
+        if fitted.get((n, L)) != (hq, hkv, dq):                # to this call's other sizes, with its first batch of the shape
+            fitted[n, L] = hq, hkv, dq
+            for name, shape, dtype in (("o", (n, L, hq, dq), bf16), ("k_rot", (n, L, hkv, dq), bf16), ("win_score", (n, hkv, L), f32),
+                                       ("win_lse", (n, hq, w), f32), ("score", (n,), f32), ("idx", (n, hkv, k_keep), i32)):
+                if name in pb:
+                    pb[name] = _kept(pb, name, shape, dtype, dev)
         pre = chunk_prefill_attn(bq, bk, bv, w=w, rope_theta=rope_theta, softmax_scale=softmax_scale,
                                  out=pb.get("o"), k_rot=pb.get("k_rot"), win_score=pb.get("win_score"),
-                                 win_lse=pb.get("win_lse"), status=b.get("status"), workspace=pb.get("workspace"))
+                                 win_lse=pb.get("win_lse"), status=b["status"], workspace=pb.get("workspace"))
         b["status"] = pre["status"]
         pb.update({"o": pre["o"], "k_rot": pre["k_rot"], "win_score": pre["win_score"], "win_lse": pre["win_lse"],
                    "workspace": pre["workspace"]})
@@ -600,17 +636,19 @@ def hot_path_streaming(q, k, v, *, w, rope_theta, m, k_keep, batch=None, softmax
             pb["idx"] = idx
             queue_gather(qu, pre["k_rot"], bv, idx)
         if k_win is None:                                      # the window is the same in every chunk: keep the first
-            k_win = b.get("k_win")
-            if k_win is None or k_win.shape != (1, w, Hkv, d):
+            k_win = _kept(b, "k_win", (1, w, Hkv, d), bf16, dev)
+            if k_win is None:
                 k_win = torch.empty((1, w, Hkv, d), dtype=torch.bfloat16, device=dev)
             k_win.copy_(pre["k_rot"][0:1, L - w:])
             b["k_win"] = k_win
         c0 += n
-    kept, kc, vc, pos = queue_emit(qu, k_out=b.get("kc"), v_out=b.get("vc"), pos_out=b.get("pos"), kept_out=b.get("kept"))
+    rows = (Hkv, m * k_keep)
+    kept, kc, vc, pos = queue_emit(qu, k_out=_kept(b, "kc", (*rows, d), bf16, dev), v_out=_kept(b, "vc", (*rows, d), bf16, dev),
+                                   pos_out=_kept(b, "pos", rows, i32, dev), kept_out=_kept(b, "kept", (m,), i32, dev))
     b.update({"kc": kc, "vc": vc, "pos": pos, "kept": kept})
     q_win, v_win = _window(q0, L0, w), _window(v0, L0, w)
     pa = parallel_attn(q_win, kc.unsqueeze(0), vc.unsqueeze(0), k_win, v_win, q_pos0=L0 - w, rope_theta=rope_theta,
-                       softmax_scale=softmax_scale, out=b.get("fg"), status=b["status"], workspace=b.get("ws_par"))
+                       softmax_scale=softmax_scale, out=_kept(b, "fg", (1, w, Hq, d), bf16, dev), status=b["status"], workspace=b.get("ws_par"))
     b.update({"fg": pa["out"], "ws_par": pa["workspace"]})
     return {"kept": kept, "kc": kc, "vc": vc, "pos": pos, "fg": pa["out"], "status": b["status"]}
 

@@ -188,3 +188,70 @@ def test_whole_path_refuses_tensors_that_do_not_go_together(fake):
         for bad in wrong:
             assert _host_call(fake, q, k, v, buffers=dict(good, **{n: bad}))[:2] == (4, _HOT_PATH_BUFFERS.index(n)), n
             assert fake.fake_attention_launches() == 0
+
+
+@pytest.fixture
+def on_host(fake, monkeypatch):
+    """The binding's calls on host memory and the fake runtime."""
+    from paper_2502_14317_b200 import binding
+    monkeypatch.setattr(binding, "_LIB", fake)
+    monkeypatch.setattr(binding, "_need_cuda", lambda *tensors: None)
+    monkeypatch.setattr(binding, "_stream", lambda: 0)
+    return binding
+
+
+def _stream_sizes():
+    """C, L, Hq, Hkv, d, w, m, k_keep: larger, smaller and other heads; the batches have the same chunks and tokens throughout"""
+    return [(4, 300, 4, 2, 64, 16, 2, 64), (4, 300, 8, 4, 128, 32, 4, 128), (4, 300, 2, 1, 64, 8, 1, 32), (4, 300, 4, 1, 128, 64, 3, 100)]
+
+
+def _written(binding, monkeypatch):
+    """Tensors that the streamed path's calls are given to write, with the sizes that the library writes."""
+    seen = []
+    prefill, emit, parallel, score = binding.chunk_prefill_attn, binding.queue_emit, binding.parallel_attn, binding.chunk_score_from_lse
+
+    def spy_prefill(q, k, v, *, w, **kw):
+        (C, L, Hq, d), Hkv = q.shape, k.shape[2]
+        seen.extend((n, kw.get(n), s) for n, s in (("out", (C, L, Hq, d)), ("k_rot", (C, L, Hkv, d)), ("win_score", (C, Hkv, L)), ("win_lse", (C, Hq, w))))
+        return prefill(q, k, v, w=w, **kw)
+
+    def spy_emit(state, **kw):
+        rows = (state["Hkv"], state["m"] * state["k"])
+        seen.extend((n, kw.get(n), s) for n, s in (("k_out", (*rows, state["d"])), ("v_out", (*rows, state["d"])), ("pos_out", rows), ("kept_out", (state["m"],))))
+        return emit(state, **kw)
+
+    def spy_parallel(q_win, *args, **kw):
+        seen.append(("out", kw.get("out"), tuple(q_win.shape)))
+        return parallel(q_win, *args, **kw)
+
+    def spy_score(win_lse, out=None):
+        seen.append(("score", out, (win_lse.shape[0],)))
+        return score(win_lse, out=out)
+    for n, f in (("chunk_prefill_attn", spy_prefill), ("queue_emit", spy_emit), ("parallel_attn", spy_parallel), ("chunk_score_from_lse", spy_score)):
+        monkeypatch.setattr(binding, n, f)
+    return seen
+
+
+def test_streamed_path_with_buffers_of_another_call(on_host, monkeypatch):
+    torch = pytest.importorskip("torch")
+    seen, b = _written(on_host, monkeypatch), {}
+    for C, L, Hq, Hkv, d, w, m, kk in _stream_sizes():
+        for _ in range(2):
+            seen.clear()
+            got = on_host.hot_path_streaming(*_zeros(torch, C, L, Hq, Hkv, d), w=w, rope_theta=1e4, m=m, k_keep=kk, batch=2, buffers=b)
+            assert all(t is None or t.shape == s for _, t, s in seen), [(n, t.shape, s) for n, t, s in seen if t is not None and t.shape != s]
+        assert all(t is not None for n, t, _ in seen), "everything is reused by a call of the same sizes"
+        shapes = _path_shapes(C, L, Hq, Hkv, d, w, m, kk)
+        assert all(got[n].shape == shapes[n] for n in ("kept", "kc", "vc", "pos", "fg", "status"))
+        assert (b["queue"]["q_k"].shape, b["queue"]["q_score"].shape) == (shapes["kc"], (m,))
+    q, k, v = _zeros(torch, 4, 300, 4, 2, 64)
+    args = dict(w=16, rope_theta=1e4, m=2, k_keep=64, batch=2)
+    for wrong in ((q, k[:, :200], v), (q, k, v[:, :, :1]), (q.float(), k, v), (q, k[:2], v[:2])):
+        with pytest.raises(on_host.PcError, match="bfloat16|C, L"):
+            on_host.hot_path_streaming(*wrong, **args)
+        if wrong[0].shape[0] == 4:                                # in a list, where only the second batch is wrong
+            parts = [(t[:2], t[2:]) for t in (q, k, v)]
+            with pytest.raises(on_host.PcError, match="C, L"):
+                on_host.hot_path_streaming(*([a, t[2:]] for (a, _), t in zip(parts, wrong)), **args)
+    with pytest.raises(on_host.PcError, match="'kc'"):
+        on_host.hot_path_streaming(q, k, v, buffers={"kc": torch.empty(2, 128, 64)}, **args)
