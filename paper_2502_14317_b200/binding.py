@@ -202,9 +202,9 @@ def _kept(b, name, shape, dtype, device):
 def _check_inputs(q, k, v, dev):
     """The launches go by q's sizes: keys and values of others would be read out of range."""
     C, L, _, d = q.shape
-    ks, bf16 = k.shape, torch.bfloat16
-    if not (ks == v.shape and len(ks) == 4 and ks[0] == C and ks[1] == L and ks[3] == d and q.dtype is k.dtype is v.dtype is bf16 and
-            q.device == k.device == v.device == dev):
+    rows = (L, k.shape[2], d)
+    if not (k.shape[1:] == v.shape[1:] == rows and k.shape[0] >= C and v.shape[0] >= C and
+            q.dtype is k.dtype is v.dtype is torch.bfloat16 and q.device == k.device == v.device == dev):
         raise PcError(_BAD_INPUT)
 
 

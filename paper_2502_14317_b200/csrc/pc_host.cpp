@@ -64,7 +64,9 @@ void Call::operator()() {
   // The launches go by q's sizes alone: keys and values of others would be read out of range.
   for (const at::Tensor* x : {&q, &k, &v})
     if (x->scalar_type() != at::kBFloat16 || x->device() != q.device()) { rc = BAD_INPUT; return; }
-  if (!k.sizes().equals({C, L, Hkv, d}) || !v.sizes().equals(k.sizes()) || (has_given && given.device() != q.device())) { rc = BAD_INPUT; return; }
+  for (const at::Tensor* x : {&k, &v})                             // (chunks beyond the queries' are not looked at)
+    if (x->dim() != 4 || x->size(0) < C || x->size(1) != L || x->size(2) != Hkv || x->size(3) != d) { rc = BAD_INPUT; return; }
+  if (has_given && given.device() != q.device()) { rc = BAD_INPUT; return; }
   const int64_t mk = m * k_keep;
   if (has_given) t[SCORE] = given;
   if (!(make(O, q.sizes(), at::kBFloat16) && make(K_ROT, k.sizes(), at::kBFloat16) && make(WIN_SCORE, {C, Hkv, L}, at::kFloat) &&

@@ -182,6 +182,7 @@ def test_whole_path_refuses_tensors_that_do_not_go_together(fake):
         assert _host_call(fake, q, k, wrong)[0] == 3 and fake.fake_attention_launches() == 0
     assert _host_call(fake, q, k, v[:, :, :1])[0] == 3 and _host_call(fake, q.float(), k, v)[0] == 3
     assert _host_call(fake, q, k.to("meta"), v)[0] == 3 and _host_call(fake, q, k, v, given=torch.zeros(6, device="meta"))[0] == 3
+    assert _host_call(fake, q[:5], k, v)[0] == _host_call(fake, q[:5], k[:5], v)[0] == 0       # chunks that no query asks for
     good = _host_call(fake, q, k, v)[2]
     for n, t in good.items():
         wrong = [t.to("meta")] + ([t.new_empty(t.numel() * 2)[::2]] if t.numel() > 1 else []) + ([] if n.startswith("ws") else [t.double()])
