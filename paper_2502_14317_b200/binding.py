@@ -665,18 +665,18 @@ def hot_path_from_host(hq, hk, hv, *, w, rope_theta, m, k_keep, softmax_scale=0.
     C, L, Hq, d = hq.shape
     Hkv = hk.shape[2]
     dev = torch.device("cuda", torch.cuda.current_device())
-    if "q" not in b:
-        b["q"] = torch.empty(hq.shape, dtype=torch.bfloat16, device=dev)
-        b["k"] = torch.empty(hk.shape, dtype=torch.bfloat16, device=dev)
-        b["v"] = torch.empty(hv.shape, dtype=torch.bfloat16, device=dev)
-        b["o"] = torch.empty(hq.shape, dtype=torch.bfloat16, device=dev)
-        b["k_rot"] = torch.empty(hk.shape, dtype=torch.bfloat16, device=dev)
-        b["win_score"] = torch.empty((C, Hkv, L), dtype=torch.float32, device=dev)
-        b["win_lse"] = torch.empty((C, Hq, w), dtype=torch.float32, device=dev)
-        b["status"] = torch.zeros(1, dtype=torch.int32, device=dev)
-        b["copy_stream"] = torch.cuda.Stream(device=dev)
-        b["uploaded"] = [torch.cuda.Event() for _ in range(n_groups)]
-        b["consumed"] = torch.cuda.Event()
+    if not (hk.shape[1:] == hv.shape[1:] == (L, Hkv, d) and hk.shape[0] >= C and hv.shape[0] >= C):
+        raise PcError("hk and hv must be [C, L, Hkv, d] with the C, L and d of hq")
+    f32, i32, bf16 = torch.float32, torch.int32, torch.bfloat16
+    for name, shape, dtype in (("q", hq.shape, bf16), ("k", hk.shape, bf16), ("v", hv.shape, bf16), ("o", hq.shape, bf16), ("k_rot", hk.shape, bf16),
+                               ("win_score", (C, Hkv, L), f32), ("win_lse", (C, Hq, w), f32)):
+        t = _kept(b, name, shape, dtype, dev)
+        b[name] = torch.empty(shape, dtype=dtype, device=dev) if t is None else t
+    t = _kept(b, "status", (1,), i32, dev)
+    b["status"] = torch.zeros(1, dtype=i32, device=dev) if t is None else t
+    if "copy_stream" not in b:
+        b["copy_stream"], b["uploaded"] = torch.cuda.Stream(device=dev), []
+    b["uploaded"] += [torch.cuda.Event() for _ in range(n_groups - len(b["uploaded"]))]
     q, k, v = b["q"], b["k"], b["v"]
     main, copy = torch.cuda.current_stream(), b["copy_stream"]
     copy.wait_stream(main)                       # the previous call may still read q, k, v
@@ -695,11 +695,14 @@ def hot_path_from_host(hq, hk, hv, *, w, rope_theta, m, k_keep, softmax_scale=0.
                                  out=b["o"][c0:c1], k_rot=b["k_rot"][c0:c1], win_score=b["win_score"][c0:c1],
                                  win_lse=b["win_lse"][c0:c1], status=b["status"], workspace=b.get("ws_prefill"))
         b["ws_prefill"] = pre["workspace"]
-    score, kept = score_select_chunks(b["win_lse"], m, True, score_out=b.get("chunk_score"), kept_out=b.get("kept"))
-    idx = select_tokens(b["win_score"], kept, L - w, k_keep, out=b.get("idx"))
-    kc, vc, pos = gather_kv(b["k_rot"], v, kept, idx, k_out=b.get("kc"), v_out=b.get("vc"), pos_out=b.get("pos"))
+    score, kept = score_select_chunks(b["win_lse"], m, True, score_out=_kept(b, "chunk_score", (C,), f32, dev),
+                                      kept_out=_kept(b, "kept", (m,), i32, dev))
+    idx = select_tokens(b["win_score"], kept, L - w, k_keep, out=_kept(b, "idx", (m, Hkv, k_keep), i32, dev))
+    rows = (Hkv, m * k_keep)
+    kc, vc, pos = gather_kv(b["k_rot"], v, kept, idx, k_out=_kept(b, "kc", (*rows, d), bf16, dev), v_out=_kept(b, "vc", (*rows, d), bf16, dev),
+                            pos_out=_kept(b, "pos", rows, i32, dev))
     pa = parallel_attn(q[0:1, L - w:], kc.unsqueeze(0), vc.unsqueeze(0), b["k_rot"][0:1, L - w:], v[0:1, L - w:],
-                       q_pos0=L - w, rope_theta=rope_theta, softmax_scale=softmax_scale, out=b.get("fg"),
+                       q_pos0=L - w, rope_theta=rope_theta, softmax_scale=softmax_scale, out=_kept(b, "fg", (1, w, Hq, d), bf16, dev),
                        status=b["status"], workspace=b.get("ws_par"))
     b.update(chunk_score=score, kept=kept, idx=idx, kc=kc, vc=vc, pos=pos, fg=pa["out"], ws_par=pa["workspace"])
     return {"o": b["o"], "k_rot": b["k_rot"], "win_score": b["win_score"], "win_lse": b["win_lse"], "chunk_score": score,

@@ -478,3 +478,24 @@ def test_hot_path_from_host_matches_device_path(cfg0_inputs):
         assert int(got["status"].item()) == 0
         for key in ("o", "k_rot", "win_score", "win_lse", "kept", "idx", "kc", "vc", "fg"):
             assert torch.equal(got[key], ref[key]), key
+
+
+@pytest.mark.parametrize("path", ["at once", "streamed", "from host"])
+def test_buffers_of_a_call_of_other_sizes(path):
+    """One dict for prompts of other sizes (larger, smaller, the same elements in another shape), head counts, head sizes, windows and kept
+    tokens: the same results as with buffers of the call's own, to the bit."""
+    import paper_2502_14317_b200 as pc
+    run = {"at once": pc.hot_path, "streamed": lambda *t, **kw: pc.hot_path_streaming(*t, batch=2, **kw),
+           "from host": lambda *t, **kw: pc.hot_path_from_host(*(x.cpu().pin_memory() for x in t), n_groups=3, **kw)}[path]
+    g = torch.Generator(device="cuda").manual_seed(5)
+    b = {}
+    for C, L, Hq, Hkv, d, w, m, kk in [(4, 300, 4, 2, 64, 16, 2, 64), (4, 300, 8, 4, 128, 32, 3, 128), (4, 300, 2, 1, 128, 64, 1, 100),
+                                       (6, 200, 4, 2, 64, 8, 4, 32), (2, 700, 8, 2, 64, 64, 2, 300)]:
+        q, k, v = (torch.randn((C, L, H, d), generator=g, device="cuda").bfloat16() for H in (Hq, Hkv, Hkv))
+        args = dict(w=w, rope_theta=1e4, m=m, k_keep=kk)
+        want, got = run(q, k, v, **args), run(q, k, v, buffers=b, **args)
+        torch.cuda.synchronize()
+        assert int(got["status"].item()) == 0
+        for n in ("o", "k_rot", "win_score", "win_lse", "chunk_score", "kept", "idx", "kc", "vc", "pos", "fg"):
+            if n in want:
+                assert got[n].shape == want[n].shape and torch.equal(got[n], want[n]), n

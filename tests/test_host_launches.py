@@ -256,3 +256,28 @@ def test_streamed_path_with_buffers_of_another_call(on_host, monkeypatch):
                 on_host.hot_path_streaming(*([a, t[2:]] for (a, _), t in zip(parts, wrong)), **args)
     with pytest.raises(on_host.PcError, match="'kc'"):
         on_host.hot_path_streaming(q, k, v, buffers={"kc": torch.empty(2, 128, 64)}, **args)
+
+
+def test_path_from_host_memory_with_buffers_of_another_call(on_host, monkeypatch):
+    import contextlib
+    import types
+    torch = pytest.importorskip("torch")
+    stream = types.SimpleNamespace(wait_stream=lambda other: None, wait_event=lambda event: None)
+    cuda = types.SimpleNamespace(current_device=lambda: 0, current_stream=lambda: stream, Stream=lambda device: stream,
+                                 stream=lambda s: contextlib.nullcontext(), Event=lambda: types.SimpleNamespace(record=lambda s: None))
+
+    class OnHost:                                                 # torch with its GPU calls on host memory
+        device = staticmethod(lambda *a: torch.device("cpu"))
+
+        def __getattr__(self, name):
+            return cuda if name == "cuda" else getattr(torch, name)
+    monkeypatch.setattr(on_host, "torch", OnHost())
+    b = {}
+    for n_groups, (C, L, Hq, Hkv, d, w, m, kk) in zip((1, 3, 2, 4), _stream_sizes()):
+        for extra in (0, 3):
+            q, k, v = _zeros(torch, C + extra, L, Hq, Hkv, d)
+            got = on_host.hot_path_from_host(q, k, v, w=w, rope_theta=1e4, m=m, k_keep=kk, n_groups=n_groups, buffers=b)
+            assert all(got[n].shape == s for n, s in _path_shapes(C + extra, L, Hq, Hkv, d, w, m, kk).items())
+    for wrong in ((q, k[:, :200], v), (q, k[:2], v), (q, k, v[:, :, :, :64])):
+        with pytest.raises(on_host.PcError, match="C, L"):
+            on_host.hot_path_from_host(*wrong, w=64, rope_theta=1e4, m=2, k_keep=64)
