@@ -10,6 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB_PATH = os.path.join(HERE, "libpc.so")
 HOST_PATH = os.path.join(HERE, "_pc_host.so")
+HOST_SOURCE = "pc_host.cpp"
 SOURCES = ["pc_api.cu", "pc_prefill2.cu", "pc_parallel.cu", "pc_decode.cu", "pc_rope.cu", "pc_select_gather.cu", "pc_queue.cu", "pc_static_scratch.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
@@ -22,51 +23,86 @@ def _nvcc() -> str:
     return cand if os.path.exists(cand) else "nvcc"
 
 
+def _older(path, sources) -> bool:
+    return not os.path.exists(path) or any(os.path.getmtime(p) > os.path.getmtime(path) for p in sources)
+
+
+def _header() -> str:
+    return os.path.join(HERE, "..", "include", "pc.h")
+
+
 def needs_build() -> bool:
-    if not os.path.exists(LIB_PATH) or not os.path.exists(HOST_PATH):
-        return True
-    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(HOST_PATH))
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "pc.h")]
-    return any(os.path.getmtime(p) > t for p in deps)
+    return _older(LIB_PATH, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != HOST_SOURCE] + [_header()])
+
+
+def _host_needs_build() -> bool:
+    return _older(HOST_PATH, [os.path.join(CSRC, HOST_SOURCE), _header()])
 
 
 def _host_command():
-    """Command that compiles csrc/pc_host.cpp against the installed torch."""
-    import torch
-    root = os.path.join(os.path.dirname(torch.__file__))
+    """Command that compiles csrc/pc_host.cpp against the installed torch; None where there is none (or one that cannot be loaded)."""
+    try:
+        import torch
+    except (ImportError, OSError):
+        return None
+    root = os.path.dirname(torch.__file__)
     inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"]]
     lib = os.path.join(root, "lib")
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
-            "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI, *("-isystem" + d for d in inc), os.path.join(CSRC, "pc_host.cpp"),
-            "-o", HOST_PATH, "-L" + lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch_cpu", "-lc10"]
+            "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI, *("-isystem" + d for d in inc), os.path.join(CSRC, HOST_SOURCE),
+            "-L" + lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch_cpu", "-lc10"]
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into one shared library; returns its path."""
-    if not force and not needs_build():
-        return LIB_PATH
-    objs = []
-    procs = []
+    """Compile every .cu under csrc/ into one shared library, and beside it csrc/pc_host.cpp into _pc_host.so; returns the library's path.
+
+    The library needs nvcc alone.  _pc_host.so, the host side of the binding's hot_path, needs torch, the Python headers and a C++ compiler: where
+    one of them is missing or fails that is said on stderr, the library is built all the same, and hot_path raises PcError."""
     os.makedirs(os.path.join(HERE, "_build"), exist_ok=True)
-    for src in SOURCES:
-        obj = os.path.join(HERE, "_build", src.replace(".cu", ".o"))
-        cmd = [_nvcc(), *NVCC_FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
-        if verbose:
-            cmd.insert(1, "-Xptxas=-v")
-        procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-        objs.append(obj)
-    procs.append(("pc_host.cpp", subprocess.Popen(_host_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    new_lib, new_host = (os.path.join(HERE, "_build", os.path.basename(p)) for p in (LIB_PATH, HOST_PATH))
+    host = None
+    if force or _host_needs_build():
+        cmd = _host_command()
+        if cmd is None:
+            sys.stderr.write("_pc_host.so is not built: torch cannot be imported\n")
+        else:
+            try:
+                host = subprocess.Popen(cmd + ["-o", new_host], stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+            except OSError as e:
+                sys.stderr.write("_pc_host.so is not built: %s\n" % e)
+    procs, objs = [], []
+    if force or needs_build():
+        for src in SOURCES:
+            obj = os.path.join(HERE, "_build", src.replace(".cu", ".o"))
+            cmd = [_nvcc(), *NVCC_FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+            if verbose:
+                cmd.insert(1, "-Xptxas=-v")
+            procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+            objs.append(obj)
+    failed = []
     for src, p in procs:
         out, _ = p.communicate()
         if verbose or p.returncode != 0:
             sys.stderr.write(out)
         if p.returncode != 0:
-            raise RuntimeError(f"compiling {src} failed")
-    link = [_nvcc(), "-shared", "-o", LIB_PATH, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
-    r = subprocess.run(link, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
-    if r.returncode != 0:
-        sys.stderr.write(r.stdout)
-        raise RuntimeError("link failed")
+            failed.append(src)
+    if host is not None:
+        out, _ = host.communicate()
+        if verbose or host.returncode != 0:
+            sys.stderr.write(out)
+        if host.returncode == 0:
+            os.replace(new_host, HOST_PATH)                # (a process that has the old one mapped keeps it)
+        else:
+            sys.stderr.write("_pc_host.so is not built: compiling %s failed\n" % HOST_SOURCE)
+    if failed:
+        raise RuntimeError("compiling %s failed" % ", ".join(failed))
+    if objs:
+        link = [_nvcc(), "-shared", "-o", new_lib, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
+        r = subprocess.run(link, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+        if r.returncode != 0:
+            sys.stderr.write(r.stdout)
+            raise RuntimeError("link failed")
+        os.replace(new_lib, LIB_PATH)
     return LIB_PATH
 
 

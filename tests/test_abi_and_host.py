@@ -213,3 +213,27 @@ def test_header_is_plain_c(tmp_path):
     r = subprocess.run([gcc, "-std=c99", "-Wall", "-Wextra", "-pedantic", "-Werror", "-fsyntax-only",
                         "-I", os.path.join(root, "include"), str(src)], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
+
+
+def _build_with_stand_ins(tmp_path, *, torch=True, **env):
+    """build.py on a copy of the sources with a stand-in for nvcc that makes empty files; the files that it leaves beside the package."""
+    import shutil
+    pkg = tmp_path / "pkg"
+    if not pkg.exists():
+        shutil.copytree(os.path.join(ROOT, "paper_2502_14317_b200", "csrc"), pkg / "csrc")
+        shutil.copy(os.path.join(ROOT, "paper_2502_14317_b200", "build.py"), pkg)
+        shutil.copytree(os.path.join(ROOT, "include"), tmp_path / "include")
+    nvcc = tmp_path / "cuda" / "bin" / "nvcc"
+    nvcc.parent.mkdir(parents=True, exist_ok=True)
+    nvcc.write_text('#!/bin/sh\nwhile [ "$1" != -o ]; do shift; done\n: > "$2"\n')
+    nvcc.chmod(0o755)
+    code = ("import sys; sys.path.insert(0, %r)\n" % str(pkg)) + ("" if torch else "sys.modules['torch'] = None\n") + "import build; print(build.build_library())"
+    r = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, CUDA_HOME=str(tmp_path / "cuda"), **env), capture_output=True, text=True)
+    return r, sorted(f for f in os.listdir(pkg) if f.endswith(".so"))
+
+
+def test_library_is_built_without_torch_or_a_compiler_for_its_binding(tmp_path):
+    for kw in (dict(CXX="/bin/false"), dict(CXX=str(tmp_path / "none")), dict(torch=False)):
+        r, built = _build_with_stand_ins(tmp_path, **kw)
+        assert r.returncode == 0 and built == ["libpc.so"] and "_pc_host.so is not built" in r.stderr, (kw, r.stderr)
+        os.remove(tmp_path / "pkg" / "libpc.so")
