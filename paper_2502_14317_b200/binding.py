@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import functools
+import importlib.util
 import math
 import os
 from ctypes import c_float, c_int32, c_int64, c_size_t, c_void_p, c_char_p, POINTER, Structure
@@ -121,12 +122,16 @@ def _host_hot_path(lib):
     """hot_path of csrc/pc_host.cpp on this library's entry points."""
     call = getattr(lib, "_host_hot_path", None)
     if call is None:
+        from .build import host_path
+        path = host_path(torch.__version__)
         try:
-            from . import _pc_host
+            spec = importlib.util.spec_from_file_location(__package__ + "._pc_host", path)
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
         except ImportError as e:
-            raise PcError("_pc_host.so cannot be loaded: build it with `python -m paper_2502_14317_b200.build` (%s)" % e) from e
+            raise PcError("%s cannot be loaded: build it with `python -m paper_2502_14317_b200.build` (%s)" % (path, e)) from e
         address = lambda f: ctypes.cast(f, c_void_p).value
-        call = lib._host_hot_path = functools.partial(_pc_host.hot_path, address(lib.pc_hot_path_workspace_bytes), address(lib.pc_hot_path))
+        call = lib._host_hot_path = functools.partial(module.hot_path, address(lib.pc_hot_path_workspace_bytes), address(lib.pc_hot_path))
     return call
 
 

@@ -227,7 +227,14 @@ def _build_with_stand_ins(tmp_path, *, torch=True, **env):
     nvcc.parent.mkdir(parents=True, exist_ok=True)
     nvcc.write_text('#!/bin/sh\nwhile [ "$1" != -o ]; do shift; done\n: > "$2"\n')
     nvcc.chmod(0o755)
-    code = ("import sys; sys.path.insert(0, %r)\n" % str(pkg)) + ("" if torch else "sys.modules['torch'] = None\n") + "import build; print(build.build_library())"
+    cxx = tmp_path / "cxx"
+    cxx.write_text(nvcc.read_text())
+    cxx.chmod(0o755)
+    env.setdefault("CXX", str(cxx))
+    code = ("import sys; sys.path.insert(0, %r)\n" % str(pkg)) + ("" if torch else "sys.modules['torch'] = None\n")
+    if isinstance(torch, str):
+        code += "import torch; torch.__version__ = %r\n" % torch
+    code += "import build; print(build.build_library())"
     r = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, CUDA_HOME=str(tmp_path / "cuda"), **env), capture_output=True, text=True)
     return r, sorted(f for f in os.listdir(pkg) if f.endswith(".so"))
 
@@ -237,3 +244,23 @@ def test_library_is_built_without_torch_or_a_compiler_for_its_binding(tmp_path):
         r, built = _build_with_stand_ins(tmp_path, **kw)
         assert r.returncode == 0 and built == ["libpc.so"] and "_pc_host.so is not built" in r.stderr, (kw, r.stderr)
         os.remove(tmp_path / "pkg" / "libpc.so")
+
+
+def test_host_module_goes_with_one_torch_and_one_python(tmp_path):
+    """A module of another torch or Python is neither taken for this one's nor loaded."""
+    import sysconfig
+    from paper_2502_14317_b200 import binding, build
+    suffix = sysconfig.get_config_var("EXT_SUFFIX")
+    names = ["_pc_host-torch%s%s" % (v, suffix) for v in ("2.0", "2.1+x")]
+    r, built = _build_with_stand_ins(tmp_path, torch="2.0")
+    assert built == [names[0], "libpc.so"], r.stderr
+    old = os.path.getmtime(tmp_path / "pkg" / names[0])
+    r, built = _build_with_stand_ins(tmp_path, torch="2.1+x")
+    assert built == [*names, "libpc.so"] and os.path.getmtime(tmp_path / "pkg" / names[0]) == old, r.stderr
+    with pytest.MonkeyPatch.context() as mp:
+        mp.setattr(build, "HERE", str(tmp_path / "pkg"))
+        with pytest.raises(binding.PcError, match="cannot be loaded"):   # no file of the installed torch
+            binding._host_hot_path(ctypes.CDLL(None))
+    build.build_library()
+    path = build.host_path(__import__("torch").__version__)
+    assert os.path.exists(path) and binding._host_hot_path(binding.load_library())
