@@ -499,7 +499,10 @@ cudaError_t launch_gather_kv(const void* k_src, const void* v_src, const long lo
   // beyond it.  The blocks are set up while the ranking ahead still holds some SMs, and those that come late then end late (and a
   // turn of blocks costs little beside DRAM).  Ranking and gather, us, 8 / 64 an SM: 96 MB 20.9 / 23.5, 105 MB 23.5 / 26.1, 134 MB
   // 29.4 / 31.1, 164 MB 36.7 / 36.1, 201 MB 44.2 / 42.0, 268 MB 56.9 / 52.1, 403 MB 81.7 / 73.4, 671 MB 131 / 118 (16 an SM 125, 32 120, 128 116).
-  const long long moved = n_rows * d * 8, per_sm = moved > (150ll << 20) ? 64 : 8;
+  // Slots of the queue: the host does not know how many take a chunk, and late in a stream most do not.  Eight slots of 8 kv-heads, 8 / 64 an
+  // SM: 2500 tokens each (164 MB if all take one) none 8.2 / 13.7, one 9.3 / 14.6, four 15.1 / 18.4, all 29.8 / 29.5; 10241 tokens (671 MB) none
+  // 27.9 / 31.3, one 33.0 / 34.6, two 38.5 / 39.9, four 64.0 / 57.3, all 121 / 107: eight.
+  const long long moved = n_rows * d * 8, per_sm = !by_slot && moved > (150ll << 20) ? 64 : 8;
   int blocks = (int)(want < sm_count * per_sm ? want : sm_count * per_sm);
   if (blocks < 1) blocks = 1;
   const long long sc = stride_elems[0] / 8, stok = stride_elems[1] / 8, sh = stride_elems[2] / 8;

@@ -242,3 +242,30 @@ def test_rank_and_compact_in_one_launch_equals_the_two_calls(Cb, L, w, Hkv, d, k
 def test_rank_and_compact_with_several_blocks_a_row(Cb, L, w, Hkv, d, k, m):
     """One block a row (33 kept), eight with uneven shares, and more rows than there are SMs."""
     test_rank_and_compact_in_one_launch_equals_the_two_calls(Cb, L, w, Hkv, d, k, m)
+
+
+@pytest.mark.parametrize("d,k", [(128, 2401), (64, 4803)])
+def test_slots_that_keep_their_contents_in_a_large_queue(d, k):
+    """Above 150 MiB of slots, where the gather of whole caches takes another grid: rows of slots that take a chunk, to the bit; others untouched."""
+    import paper_2502_14317_b200 as pc
+    m, Hkv, Cb, L = 8, 8, 3, 5000
+    g = torch.Generator(device="cuda").manual_seed(k)
+    ks, vs = (torch.randn((Cb, L, Hkv, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    idx = torch.randint(-1, L, (Cb, Hkv, k), generator=g, device="cuda", dtype=torch.int32)
+    for takes in ([-1] * m, [-1, 2, -1, -1, 0, -1, -1, 1], [0, 1, 2, 0, 1, 2, 0, 1]):
+        st = pc.queue_init(m, Hkv, k, d, torch.device("cuda:0"))
+        st["slot_src"].copy_(torch.tensor(takes, dtype=torch.int32))
+        for key in ("q_k", "q_v"):
+            st[key].view(torch.int16).fill_(0x1234)
+        st["q_pos"].fill_(-7)
+        pc.queue_gather(st, ks, vs, idx)
+        for s, c in enumerate(takes):
+            at = slice(s * k, (s + 1) * k)
+            if c < 0:
+                assert (st["q_pos"][:, at] == -7).all() and all((st[key][:, at].view(torch.int16) == 0x1234).all() for key in ("q_k", "q_v"))
+                continue
+            assert torch.equal(st["q_pos"][:, at], idx[c])
+            for key, src in (("q_k", ks), ("q_v", vs)):
+                want = src[c].transpose(0, 1).gather(1, idx[c].clamp(min=0).long()[..., None].expand(-1, -1, d))
+                want[idx[c] < 0] = 0
+                assert torch.equal(st[key][:, at], want), (key, s)

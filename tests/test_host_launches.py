@@ -9,19 +9,24 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-@pytest.fixture(scope="module")
-def fake(tmp_path_factory):
+def _fake(tmp_path_factory, *more):
+    """libpc on the fake runtime: the entry points, the rotation and further source files."""
     from paper_2502_14317_b200 import binding, build
     csrc, out = build.CSRC, str(tmp_path_factory.mktemp("fake") / "libpc_fake.so")
     subprocess.run([build._nvcc(), "-shared", "-cudart", "none", "-gencode", "arch=compute_100a,code=sm_100a", "-O1", "-std=c++17",
                     "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", "-I", csrc, "-Xlinker", "-Bsymbolic", "-Xlinker", "--no-undefined",
                     os.path.join(ROOT, "tests", "fake_runtime.cpp"), "-o", out] +
-                   [os.path.join(csrc, f) for f in ("pc_api.cu", "pc_rope.cu", "pc_static_scratch.cu")],
+                   [os.path.join(csrc, f) for f in ("pc_api.cu", "pc_rope.cu", "pc_static_scratch.cu", *more)],
                    check=True, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)
     with pytest.MonkeyPatch.context() as mp:
         mp.setattr(binding, "_LIB", None)
         mp.setattr(binding, "lib_path", lambda: out)
         return binding.load_library()
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return _fake(tmp_path_factory)
 
 
 P = 1 << 20                                                       # a device address that nothing follows
@@ -281,3 +286,13 @@ def test_path_from_host_memory_with_buffers_of_another_call(on_host, monkeypatch
     for wrong in ((q, k[:, :200], v), (q, k[:2], v), (q, k, v[:, :, :, :64])):
         with pytest.raises(on_host.PcError, match="C, L"):
             on_host.hot_path_from_host(*wrong, w=64, rope_theta=1e4, m=2, k_keep=64)
+
+
+def test_grid_of_the_gather(tmp_path_factory):
+    """More blocks than the SMs hold only where all the rows move: slots of the queue may keep theirs, which the host cannot see."""
+    lib = _fake(tmp_path_factory, "pc_select_gather.cu")
+    strides = (ctypes.c_int64 * 3)(8 << 20, 1024, 128)
+    for m, Hkv, k, d, blocks in [(1, 1, 1, 64, 1), (1, 2, 100, 128, 13), (8, 8, 2048, 128, 1184), (8, 8, 2400, 128, 1184),
+                                 (8, 8, 2401, 128, 9472), (8, 8, 10241, 128, 9472), (8, 16, 10241, 64, 9472)]:
+        assert lib.pc_gather_kv(P, P, strides, P, P, m, Hkv, k, d, P, P, P, None) == 0 and lib.fake_last_grid() == blocks
+        assert lib.pc_queue_gather(P, P, strides, P, P, m, Hkv, k, d, P, P, P, None) == 0 and lib.fake_last_grid() == min(blocks, 1184)
