@@ -30,7 +30,7 @@ class _PrefillDesc(Structure):
                 ("o_stride", c_int64 * 3)]
 
 
-class _HotPathArgs(Structure):
+class _HotPathArgs(Structure):                             # pc_hot_path_args for callers through ctypes; hot_path fills it in csrc/pc_host.cpp
     _fields_ = [(n, c_void_p) for n in ("q", "k", "v", "q_win", "o", "k_rot", "win_score", "win_lse", "given_score", "chunk_score",
                                         "kept", "idx", "kc", "vc", "pos", "fg", "status_word", "ws_prefill")] + \
                [("ws_prefill_bytes", c_size_t), ("ws_parallel", c_void_p), ("ws_parallel_bytes", c_size_t),

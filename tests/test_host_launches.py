@@ -109,7 +109,7 @@ def _host_call(lib, q, k, v, given=None, buffers={}, m=2, k_keep=64, w=16):
     return rc, stage, dict(zip(_HOT_PATH_BUFFERS, out))
 
 
-@pytest.mark.parametrize("d,Hq,Hkv,w", [(64, 4, 2, 16), (128, 6, 2, 1), (128, 4, 4, 128)])
+@pytest.mark.parametrize("d,Hq,Hkv,w", [(64, 4, 2, 16), (128, 6, 2, 1), (128, 4, 4, 128), (64, 4, 1, 16)])
 def test_host_side_of_the_whole_path(fake, d, Hq, Hkv, w):
     """Tensors that are made, kept and replaced, on host memory and the fake runtime."""
     torch = pytest.importorskip("torch")
@@ -132,7 +132,10 @@ def test_host_side_of_the_whole_path(fake, d, Hq, Hkv, w):
     assert rc == 0 and b["chunk_score"] is score and all(b[n] is a[n] for n in a if n != "chunk_score")
     small = torch.empty(16, dtype=torch.uint8)
     rc, _, b = _host_call(fake, q, k, v, buffers=dict(a, ws_prefill=small, ws_par=small, pos=None), w=w)
-    assert rc == 0 and b["ws_prefill"].numel() == a["ws_prefill"].numel() and b["ws_par"].numel() >= 16 and b["pos"] is not a["pos"]
+    need = ctypes.c_size_t()
+    fake.pc_hot_path_workspace_bytes(ctypes.byref(_desc(C, L, w, Hq, Hkv, d)), m, kk, ctypes.byref(need))
+    assert rc == 0 and b["ws_prefill"].numel() == a["ws_prefill"].numel() and b["ws_par"].numel() >= need.value > small.numel()
+    assert b["pos"] is not a["pos"]
     assert all(b[n] is a[n] for n in shapes if n != "pos")
     # head-major queries go through a copy of the window; other strides of v are refused, as is a head dimension that is not innermost
     heads = torch.zeros((C, Hq, L, d), dtype=torch.bfloat16).transpose(1, 2)
@@ -146,6 +149,47 @@ def test_host_side_of_the_whole_path(fake, d, Hq, Hkv, w):
         _host_call(fake, q, k, v, given=3.0, w=w)
     with pytest.raises(RuntimeError):
         _host_call(fake, q, k, v, w=w, k_keep=-1)
+
+
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("packed", [False, True])
+def test_arguments_of_the_whole_path(fake, packed, given):
+    """What pc_hot_path is called with: pointers and strides of the tensors that come back, sizes and flags."""
+    torch = pytest.importorskip("torch")
+    from paper_2502_14317_b200 import binding
+    C, L, Hq, Hkv, d, w, m, kk = 3, 300, 6, 2, 64, 16, 2, 70
+    got = {}
+
+    @ctypes.CFUNCTYPE(ctypes.c_int32, ctypes.POINTER(binding._PrefillDesc), ctypes.POINTER(binding._HotPathArgs), ctypes.POINTER(ctypes.c_int32), ctypes.c_void_p)
+    def run(desc, args, failed, stream):
+        read = lambda s: {n: list(x) if isinstance(x, ctypes.Array) else x for n, x in ((n, getattr(s, n)) for n, _ in s._fields_)}
+        got.update(read(args[0]), desc=read(desc[0]), stream=stream)
+        if got["q_win"] != q[0, L - w:].data_ptr():
+            got["window"] = ctypes.string_at(got["q_win"], w * Hq * d * 2)
+        return 0
+    ints = lambda *size: torch.randint(-32768, 32767, size, dtype=torch.int16).view(torch.bfloat16)
+    q, k, v, o = ints(C, L, Hq, d), ints(C, L, Hkv, d), ints(C, L, Hkv, d), ints(C, L, Hq, d)
+    if not packed:                                                # head-major, and keys between others
+        q, o, k = ints(C, Hq, L, d).transpose(1, 2), ints(C, Hq, L, d).transpose(1, 2), ints(C, L, 3 * Hkv, d)[:, :, Hkv:2 * Hkv]
+    score = torch.zeros(C - 1) if given else None
+    buffers = {"o": o} if packed else {"o": o, "status": torch.zeros(1, dtype=torch.int32)}
+    call = binding._host_hot_path(fake)
+    rc, _, out = call.func(call.args[0], ctypes.cast(run, ctypes.c_void_p).value, 77, q, k, v, score,
+                           tuple([buffers.get(n) for n in binding._HOT_PATH_BUFFERS]), (C, L, Hq, Hkv, d, w, m, kk), 5e5, 0.25)
+    out = dict(zip(binding._HOT_PATH_BUFFERS, out))
+    assert rc == 0 and out["o"] is o
+    for n, t in dict(out, q=q, k=k, v=v).items():
+        field = {"status": "status_word", "ws_par": "ws_parallel"}.get(n, n)
+        assert got[field] == t.data_ptr(), n
+    assert got["given_score"] == (score.data_ptr() if given else None) and got["n_score"] == (C - 1 if given else C)
+    assert (got["m"], got["k_keep"], got["clear_status"], got["stream"]) == (m, kk, packed, 77)
+    assert (got["ws_prefill_bytes"], got["ws_parallel_bytes"]) == (out["ws_prefill"].numel(), out["ws_par"].numel())
+    assert got["desc"] == dict(C=C, L=L, w=w, Hq=Hq, Hkv=Hkv, d=d, rope_theta=5e5, softmax_scale=0.25,
+                               **{n + "_stride": list(t.stride()[:3]) for n, t in (("q", q), ("k", k), ("v", v), ("o", o))})
+    if packed:
+        assert got["q_win"] == q[0, L - w:].data_ptr()
+    else:
+        assert got["window"] == q[0, L - w:].contiguous().view(torch.int16).numpy().tobytes()
 
 
 def _path_shapes(C, L, Hq, Hkv, d, w, m, k_keep):
