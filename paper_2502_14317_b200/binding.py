@@ -41,6 +41,7 @@ class _HotPathArgs(Structure):                             # pc_hot_path_args fo
 _HOT_PATH_BUFFERS = ("o", "k_rot", "win_score", "win_lse", "chunk_score", "kept", "idx", "kc", "vc", "pos", "fg", "status", "ws_prefill",
                      "ws_par")
 _BAD_INPUT = "q, k and v must be bfloat16, k and v [C, L, Hkv, d] with the C, L and d of q, everything on one device"
+_Strides = c_int64 * 3
 _STAGES = (None, "pc_chunk_prefill_attn", "pc_select_chunks", "pc_score_select_chunks", "pc_select_tokens", "pc_gather_kv",
            "pc_parallel_attn")
 
@@ -355,7 +356,7 @@ def gather_kv(k_src, v_src, kept, idx, k_out=None, v_out=None, pos_out=None, wan
     v_out = _like(k_out, (Hkv, m * k, d)) if v_out is None else v_out
     if pos_out is None and want_pos:
         pos_out = torch.empty((Hkv, m * k), dtype=torch.int32, device=dev)
-    strides = (c_int64 * 3)(k_src.stride(0), k_src.stride(1), k_src.stride(2))
+    strides = _Strides(*k_src.stride()[:3])
     _check(lib.pc_gather_kv(_ptr(k_src), _ptr(v_src), strides, _ptr(kept), _ptr(idx), m, Hkv, k, d, _ptr(k_out),
                             _ptr(v_out), _ptr(pos_out), _stream()), "pc_gather_kv")
     return k_out, v_out, pos_out
@@ -402,7 +403,7 @@ def queue_gather(state, k_src, v_src, idx):
         raise PcError("idx must be [Cb, Hkv, k] for the queue's k; Hkv and d must match the queue")
     if not _same_rows(k_src, v_src):
         raise PcError("k_src and v_src must share strides with a contiguous head dimension")
-    strides = (c_int64 * 3)(k_src.stride(0), k_src.stride(1), k_src.stride(2))
+    strides = _Strides(*k_src.stride()[:3])
     _check(lib.pc_queue_gather(_ptr(k_src), _ptr(v_src), strides, _ptr(state["slot_src"]), _ptr(idx), state["m"], Hkv,
                                state["k"], d, _ptr(state["q_k"]), _ptr(state["q_v"]), _ptr(state["q_pos"]), _stream()),
            "pc_queue_gather")
@@ -418,7 +419,7 @@ def queue_select_gather(state, win_score, k_src, v_src, n_cand):
         raise PcError("win_score must be contiguous [Cb, Hkv, L]; Hkv and d must match the queue")
     if not _same_rows(k_src, v_src):
         raise PcError("k_src and v_src must share strides with a contiguous head dimension")
-    strides = (c_int64 * 3)(k_src.stride(0), k_src.stride(1), k_src.stride(2))
+    strides = _Strides(*k_src.stride()[:3])
     _check(lib.pc_queue_select_gather(win_score.data_ptr(), k_src.data_ptr(), v_src.data_ptr(), strides, state["slot_src"].data_ptr(),
                                       state["m"], Hkv, L, int(n_cand), state["k"], d, state["q_k"].data_ptr(), state["q_v"].data_ptr(),
                                       state["q_pos"].data_ptr(), _stream()), "pc_queue_select_gather")
@@ -433,10 +434,12 @@ def queue_emit(state, k_out=None, v_out=None, pos_out=None, kept_out=None):
     v_out = torch.empty((Hkv, m * k, d), dtype=torch.bfloat16, device=dev) if v_out is None else v_out
     pos_out = torch.empty((Hkv, m * k), dtype=torch.int32, device=dev) if pos_out is None else pos_out
     kept_out = torch.empty(m, dtype=torch.int32, device=dev) if kept_out is None else kept_out
-    order = state.setdefault("slot_order", torch.empty(m, dtype=torch.int32, device=dev))
-    _check(lib.pc_queue_emit(_ptr(state["q_chunk"]), m, Hkv, k, d, _ptr(state["q_k"]), _ptr(state["q_v"]),
-                             _ptr(state["q_pos"]), _ptr(kept_out), _ptr(order), _ptr(k_out), _ptr(v_out), _ptr(pos_out),
-                             _stream()), "pc_queue_emit")
+    order = state.get("slot_order")
+    if order is None:
+        order = state["slot_order"] = torch.empty(m, dtype=torch.int32, device=dev)
+    _check(lib.pc_queue_emit(state["q_chunk"].data_ptr(), m, Hkv, k, d, state["q_k"].data_ptr(), state["q_v"].data_ptr(),
+                             state["q_pos"].data_ptr(), kept_out.data_ptr(), order.data_ptr(), k_out.data_ptr(), v_out.data_ptr(),
+                             pos_out.data_ptr(), _stream()), "pc_queue_emit")
     return kept_out, k_out, v_out, pos_out
 
 
