@@ -32,8 +32,8 @@ constexpr int NT2 = 512;                     // threads per CTA
 constexpr int WARP_EPI = 8, WARP_PRODUCER = 12, WARP_QK = 13, WARP_PV = 14;
 // Registers by role, 128 * (2 * softmax + epilogue + service) = 64 K.  In a loop, us: prefill, 8 chunks of 8192, 32/8 heads
 // 184/80/64 4073, 192/80/48 3983, 192/64/64 3993, 8 of 4096, 32/32 heads 1399 / 1366 / 1378; over caches softmax 184 619, 192 631.
-// With 48 registers the service roles spill (-Xptxas -v: 28 bytes stored, 36 loaded at head size 128 on pairs; 192/64/64
-// spills nothing and is no faster).
+// The service roles spill (-Xptxas -v, bytes stored / loaded at head size 128 on pairs: 48 / 60, spread 72 / 92; with 192/64/64, no
+// faster, 32 / 32 and 28 / 28).
 struct Regs { int softmax, epilogue, service; };
 constexpr Regs REGS_PREFILL = {192, 80, 48}, REGS_PARALLEL = {184, 80, 64};
 constexpr int NDESC = 4;                     // work descriptors in flight
@@ -58,8 +58,8 @@ struct Cfg {
   static constexpr uint32_t TM_P = TWO_S ? 256 : 128, TM_O = TWO_S ? 384 : 256;
   static constexpr __host__ __device__ uint32_t tm_s(int b) { return TWO_S ? 128u * b : 0u; }
   // The issuers poll without a pause.  us, 20 ns / none, head size 128, in loops: 8 chunks of 8192, 32/8 heads 4027 / 3989, 2 of 873,
-  // 32/32 heads 51.0 / 50.8, 5 of 298, 28/4 heads 41.7 / 41.2, windows of 64 over 64 caches of 16384 1207 / 1191, two 51.2 / 50.5, one of
-  // 4096 20.6 / 20.5; head size 64, windows of 64 over 32 caches of 8192, 14/2 heads 112.4 / 111.0.
+  // 32/32 heads 51.0 / 50.8, 5 of 298, 28/4 heads 41.7 / 41.2, windows of 64 over two caches of 16384 51.2 / 50.5, one of 4096 20.6 / 20.5,
+  // 64 of 16384 (power cap) nothing; head size 64, windows of 64 over 32 caches of 8192, 14/2 heads 112.4 / 111.0.
   static constexpr unsigned ISSUER_NS = 0;
   static constexpr int CODE = PAIR ? 200 : 100;            // wait codes in the status word
 };

@@ -56,7 +56,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // waits in a kernel, all its warps share the instruction caches, and these lines at every one of them cost (us in loops of 15 ms, in
 // line / out of line) head size 64, 8 chunks of 4096, 32/8 heads 877 / 857, 22 of 958 259 / 249; head size 128, 3 of 2372, 28/4 heads
 // 188 / 179, 5 of 298 42.5 / 41.1; window of 16 over 64 caches of 16000, head size 64 496 / 478; a decoding step over one cache of
-// 16401 15.7 / 15.6; at the power cap (8 of 8192, 32/8 heads of 128 4018 / 4034) nothing.
+// 16401 15.7 / 15.6; at the power cap (8 of 8192, 32/8 heads of 128 4018 / 4034) nothing.  What is alive across the call costs the roles
+// registers: spills stored, bytes, prefill 20 / 48 at head size 64, 28 / 48 at 128 on pairs, query windows 0 / 16 to 24 (in those times).
 static __device__ __noinline__ bool mbar_wait_over(long long t0, volatile int* abort_flag, int* status_word, int where) {
   if (*abort_flag) return true;
   if (clock64() - t0 <= (static_cast<long long>(abort_flag[1]) << 10)) return false;
