@@ -191,6 +191,13 @@ def _need_cuda(*tensors):
             raise PcError("tensors must live on a CUDA device")
 
 
+def _let_go(t, stream=None):
+    """A kept tensor is about to be dropped.  Its memory belongs to the stream it was made on; the calls that used it may have been on the
+    present one, and it is not given out again before that has come here."""
+    if t is not None and t.is_cuda:
+        t.record_stream(torch.cuda.current_stream(t.device) if stream is None else stream)
+
+
 def _kept(b, name, shape, dtype, device):
     """Tensor ``name`` of the buffers b for an output of this shape, as csrc/pc_host.cpp takes it: as it is, or a view of its first elements
     where it has enough of them (an earlier call had other sizes); None (make a new one) where it is absent or too small."""
@@ -202,7 +209,10 @@ def _kept(b, name, shape, dtype, device):
     if t.shape == shape:
         return t
     n = math.prod(shape)
-    return t.view(-1)[:n].view(shape) if t.numel() >= n else None
+    if t.numel() >= n:
+        return t.view(-1)[:n].view(shape)
+    _let_go(t)
+    return None
 
 
 def _check_inputs(q, k, v, dev):
@@ -257,6 +267,7 @@ def chunk_prefill_attn(q, k, v, *, w, rope_theta, softmax_scale=0.0, want_lse=Fa
     desc = _make_desc(q, k, v, o, w, rope_theta, softmax_scale)
     need = int(lib.pc_chunk_prefill_attn_workspace_bytes(ctypes.byref(desc)))
     if workspace is None or workspace.numel() < need:          # need == 0: a bad descriptor, which the call below names
+        _let_go(workspace)
         workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
     if chunk_len is not None and (chunk_len.dtype != torch.int32 or chunk_len.numel() != C or not chunk_len.is_cuda):
         raise PcError("chunk_len must be an int32 CUDA tensor with one entry per chunk")
@@ -465,6 +476,7 @@ def parallel_attn(q_win, k_cache, v_cache, k_win, v_win, *, q_pos0, rope_theta, 
         status = torch.zeros(1, dtype=torch.int32, device=dev)
     need = parallel_attn_workspace_bytes(B, w, Hq, Hkv, d, Nk)
     if workspace is None or workspace.numel() < need:
+        _let_go(workspace)
         workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
     rc = lib.pc_parallel_attn(B, w, Hq, Hkv, d, Nk, _ptr(q_win), int(q_pos0), float(rope_theta), float(softmax_scale),
                               _ptr(k_cache), _ptr(v_cache), _ptr(k_win), _ptr(v_win), _ptr(out), _ptr(lse_out),
@@ -603,11 +615,15 @@ def hot_path_streaming(q, k, v, *, w, rope_theta, m, k_keep, batch=None, softmax
     f32, i32, bf16 = torch.float32, torch.int32, torch.bfloat16
     qu = b.get("queue")
     if qu is None or (qu["m"], qu["Hkv"], qu["k"], qu["d"], qu["q_k"].device) != (m, Hkv, k_keep, d, dev):
+        for t in () if qu is None else qu.values():
+            if torch.is_tensor(t):
+                _let_go(t)
         b["queue"] = queue_init(m, Hkv, k_keep, d, dev)
     else:
         lib = load_library()
         _check(lib.pc_queue_init(m, _ptr(qu["q_score"]), _ptr(qu["q_chunk"]), _stream()), "pc_queue_init")
     if "ids" not in b or b["ids"].numel() < n_max:
+        _let_go(b.get("ids"))
         b["ids"] = torch.arange(n_max, dtype=torch.int32, device=dev)
     qu = b["queue"]
     b["status"] = _kept(b, "status", (1,), i32, dev)
@@ -679,7 +695,11 @@ def hot_path_from_host(hq, hk, hv, *, w, rope_theta, m, k_keep, softmax_scale=0.
     for name, shape, dtype in (("q", hq.shape, bf16), ("k", hk.shape, bf16), ("v", hv.shape, bf16), ("o", hq.shape, bf16), ("k_rot", hk.shape, bf16),
                                ("win_score", (C, Hkv, L), f32), ("win_lse", (C, Hq, w), f32)):
         t = _kept(b, name, shape, dtype, dev)
-        b[name] = torch.empty(shape, dtype=dtype, device=dev) if t is None else t
+        if t is None:
+            if "copy_stream" in b:                              # a call that failed half-way may have left uploads into it
+                _let_go(b.get(name), b["copy_stream"])
+            t = torch.empty(shape, dtype=dtype, device=dev)
+        b[name] = t
     t = _kept(b, "status", (1,), i32, dev)
     b["status"] = torch.zeros(1, dtype=i32, device=dev) if t is None else t
     if "copy_stream" not in b:

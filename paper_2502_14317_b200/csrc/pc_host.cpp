@@ -7,6 +7,7 @@
 // The library's entry points come as addresses with each call: this module holds no state.
 #include <Python.h>
 #include <ATen/ATen.h>
+#include <c10/core/impl/VirtualGuardImpl.h>
 #include <pybind11/pybind11.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -39,6 +40,11 @@ struct Call {
     rc = BAD_BUFFER; stage = i;
     return false;
   }
+  // Buffer i is about to be dropped.  Its memory belongs to the stream it was made on; the calls that used it may have been on the present
+  // one, and it is not given out again before that has come here.
+  void let_go(int i) {
+    if (t[i].is_cuda()) t[i].record_stream(c10::impl::VirtualGuardImpl(t[i].device().type()).getStream(t[i].device()));
+  }
   // Buffer i of these sizes.  One that is there may be of an earlier call with other sizes: it serves as it is, or through a view of its
   // first elements where it has enough, and is replaced where it has not.  False: one that cannot be written.
   bool make(int i, at::IntArrayRef sizes, at::ScalarType type) {
@@ -53,6 +59,7 @@ struct Call {
         made[i] = true;
         return true;
       }
+      let_go(i);
     }
     t[i] = at::empty(sizes, at::TensorOptions().dtype(type).device(q.device()));
     return made[i] = true;
@@ -94,10 +101,12 @@ void Call::operator()() {
   const size_t need = ws_bytes(&desc, (int32_t)m, (int32_t)k_keep, &need_par);
   auto scratch = [&](size_t bytes) { return at::empty({(int64_t)std::max<size_t>(bytes, 16)}, at::TensorOptions().dtype(at::kByte).device(q.device())); };
   if (!t[WS_PREFILL].defined() || (size_t)t[WS_PREFILL].numel() < need) {      // 0: a bad argument, which the call below names
+    if (t[WS_PREFILL].defined()) let_go(WS_PREFILL);
     t[WS_PREFILL] = scratch(std::max(need, need_par));
     made[WS_PREFILL] = true;
   }
   if (!t[WS_PAR].defined() || (size_t)t[WS_PAR].numel() < need_par) {          // (the prefill is done with its own by then)
+    if (t[WS_PAR].defined()) let_go(WS_PAR);
     t[WS_PAR] = (size_t)t[WS_PREFILL].numel() >= need_par ? t[WS_PREFILL] : scratch(need_par);
     made[WS_PAR] = true;
   }

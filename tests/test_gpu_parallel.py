@@ -499,3 +499,40 @@ def test_buffers_of_a_call_of_other_sizes(path):
         for n in ("o", "k_rot", "win_score", "win_lse", "chunk_score", "kept", "idx", "kc", "vc", "pos", "fg"):
             if n in want:
                 assert got[n].shape == want[n].shape and torch.equal(got[n], want[n]), n
+
+
+@pytest.mark.parametrize("path", ["at once", "streamed", "from host"])
+def test_buffers_dropped_on_another_stream(path):
+    """Buffers of one stream, used and then replaced on another that has not come there yet: their memory is not given out meanwhile."""
+    import paper_2502_14317_b200 as pc
+    run = {"at once": pc.hot_path, "streamed": lambda *t, **kw: pc.hot_path_streaming(*t, batch=2, **kw), "from host": pc.hot_path_from_host}[path]
+    g = torch.Generator(device="cuda").manual_seed(6)
+
+    def inputs(L, Hq, Hkv):
+        t = [torch.randn((4, L, H, 64), generator=g, device="cuda").bfloat16() for H in (Hq, Hkv, Hkv)]
+        return [x.cpu().pin_memory() for x in t] if path == "from host" else t
+    # (the streamed path keeps a set of buffers for each batch shape: other head counts there)
+    small, large = inputs(500, 4, 2), inputs(500, 8, 4) if path == "streamed" else inputs(900, 4, 2)
+    small_args, args, b = dict(w=16, rope_theta=1e4, m=2, k_keep=100), dict(w=16, rope_theta=1e4, m=3, k_keep=200), {}
+
+    def tensors(x):
+        return [t for v in x.values() for t in (tensors(v) if isinstance(v, dict) else [v] if torch.is_tensor(v) else [])]
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):                                  # kernels are loaded, the side stream has memory to give
+        want = {n: t.clone() for n, t in run(*large, **args).items()}
+    run(*small, buffers=b, **small_args)
+    old = {t.untyped_storage().data_ptr(): t.untyped_storage().nbytes() for t in tensors(b)}
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(1 << 30)                                 # half a second
+        out = run(*large, buffers=b, **args)
+        done = torch.cuda.Event()
+        done.record()
+    dropped = set(old) - {t.untyped_storage().data_ptr() for t in tensors(b)}
+    new = [torch.empty(old[p], dtype=torch.uint8, device="cuda") for p in dropped]
+    assert not done.query() and len(dropped) >= 8
+    assert not dropped & {t.data_ptr() for t in new}
+    torch.cuda.synchronize()
+    assert int(out["status"].item()) == 0
+    for n in ("kept", "kc", "vc", "pos", "fg"):
+        assert torch.equal(out[n], want[n]), n
