@@ -478,9 +478,9 @@ def parallel_attn(q_win, k_cache, v_cache, k_win, v_win, *, q_pos0, rope_theta, 
     if workspace is None or workspace.numel() < need:
         _let_go(workspace)
         workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
-    rc = lib.pc_parallel_attn(B, w, Hq, Hkv, d, Nk, _ptr(q_win), int(q_pos0), float(rope_theta), float(softmax_scale),
-                              _ptr(k_cache), _ptr(v_cache), _ptr(k_win), _ptr(v_win), _ptr(out), _ptr(lse_out),
-                              _ptr(status), _ptr(workspace), workspace.numel(), _stream())
+    rc = lib.pc_parallel_attn(B, w, Hq, Hkv, d, Nk, q_win.data_ptr(), int(q_pos0), float(rope_theta), float(softmax_scale),
+                              k_cache.data_ptr(), v_cache.data_ptr(), k_win.data_ptr(), v_win.data_ptr(), out.data_ptr(), _ptr(lse_out),
+                              status.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream())
     _check(rc, "pc_parallel_attn")
     return {"out": out, "lse": lse_out, "status": status, "workspace": workspace}
 
@@ -601,17 +601,20 @@ def hot_path_streaming(q, k, v, *, w, rope_theta, m, k_keep, batch=None, softmax
     b = {} if buffers is None else buffers
     if isinstance(q, (list, tuple)):
         batches = list(zip(q, k, v))
+        for of_batch in batches:
+            _check_inputs(*of_batch, batches[0][0].device)
     else:
         if batch is None:
             raise PcError("hot_path_streaming needs a batch size for whole tensors")
-        batches = [(q[c0:c0 + batch], k[c0:c0 + batch], v[c0:c0 + batch]) for c0 in range(0, q.shape[0], batch)]
-    for of_batch in batches if isinstance(q, (list, tuple)) else (batches[0], batches[-1]):   # whole tensors: those between are as the first
-        _check_inputs(*of_batch, batches[0][0].device)
+        _check_inputs(q, k, v, q.device)
+        if batch >= q.shape[0] == k.shape[0] == v.shape[0] > 0:
+            batches = [(q, k, v)]
+        else:
+            batches = [(q[c0:c0 + batch], k[c0:c0 + batch], v[c0:c0 + batch]) for c0 in range(0, q.shape[0], batch)]
     q0, k0, v0 = batches[0]
     _, L0, Hq, d = q0.shape
     Hkv = k0.shape[2]
     dev = q0.device
-    n_max = max(bq.shape[0] for bq, _, _ in batches)
     f32, i32, bf16 = torch.float32, torch.int32, torch.bfloat16
     qu = b.get("queue")
     if qu is None or (qu["m"], qu["Hkv"], qu["k"], qu["d"], qu["q_k"].device) != (m, Hkv, k_keep, d, dev):
@@ -622,9 +625,6 @@ def hot_path_streaming(q, k, v, *, w, rope_theta, m, k_keep, batch=None, softmax
     else:
         lib = load_library()
         _check(lib.pc_queue_init(m, _ptr(qu["q_score"]), _ptr(qu["q_chunk"]), _stream()), "pc_queue_init")
-    if "ids" not in b or b["ids"].numel() < n_max:
-        _let_go(b.get("ids"))
-        b["ids"] = torch.arange(n_max, dtype=torch.int32, device=dev)
     qu = b["queue"]
     b["status"] = _kept(b, "status", (1,), i32, dev)
     c0 = 0
@@ -656,6 +656,9 @@ def hot_path_streaming(q, k, v, *, w, rope_theta, m, k_keep, batch=None, softmax
         if k_keep <= 10240:                                    # rank and compact the chunks that entered, one launch
             queue_select_gather(qu, pre["win_score"], pre["k_rot"], bv, L - w)
         else:
+            if "ids" not in b or b["ids"].numel() < n:
+                _let_go(b.get("ids"))
+                b["ids"] = torch.arange(n, dtype=torch.int32, device=dev)
             idx = select_tokens(pre["win_score"], b["ids"][:n], L - w, k_keep, out=pb.get("idx"))
             pb["idx"] = idx
             queue_gather(qu, pre["k_rot"], bv, idx)
@@ -663,7 +666,7 @@ def hot_path_streaming(q, k, v, *, w, rope_theta, m, k_keep, batch=None, softmax
             k_win = _kept(b, "k_win", (1, w, Hkv, d), bf16, dev)
             if k_win is None:
                 k_win = torch.empty((1, w, Hkv, d), dtype=torch.bfloat16, device=dev)
-            k_win.copy_(pre["k_rot"][0:1, L - w:])
+            k_win.copy_(_window(pre["k_rot"], L, w))
             b["k_win"] = k_win
         c0 += n
     rows = (Hkv, m * k_keep)
@@ -713,13 +716,14 @@ def hot_path_from_host(hq, hk, hv, *, w, rope_theta, m, k_keep, softmax_scale=0.
         c0, c1 = bounds[g], bounds[g + 1]
         if c1 == c0:
             continue
+        qg, kg, vg = q[c0:c1], k[c0:c1], v[c0:c1]
         with torch.cuda.stream(copy):
-            q[c0:c1].copy_(hq[c0:c1], non_blocking=True)
-            k[c0:c1].copy_(hk[c0:c1], non_blocking=True)
-            v[c0:c1].copy_(hv[c0:c1], non_blocking=True)
+            qg.copy_(hq[c0:c1], non_blocking=True)
+            kg.copy_(hk[c0:c1], non_blocking=True)
+            vg.copy_(hv[c0:c1], non_blocking=True)
             b["uploaded"][g].record(copy)
         main.wait_event(b["uploaded"][g])
-        pre = chunk_prefill_attn(q[c0:c1], k[c0:c1], v[c0:c1], w=w, rope_theta=rope_theta, softmax_scale=softmax_scale,
+        pre = chunk_prefill_attn(qg, kg, vg, w=w, rope_theta=rope_theta, softmax_scale=softmax_scale,
                                  out=b["o"][c0:c1], k_rot=b["k_rot"][c0:c1], win_score=b["win_score"][c0:c1],
                                  win_lse=b["win_lse"][c0:c1], status=b["status"], workspace=b.get("ws_prefill"))
         b["ws_prefill"] = pre["workspace"]
@@ -729,7 +733,7 @@ def hot_path_from_host(hq, hk, hv, *, w, rope_theta, m, k_keep, softmax_scale=0.
     rows = (Hkv, m * k_keep)
     kc, vc, pos = gather_kv(b["k_rot"], v, kept, idx, k_out=_kept(b, "kc", (*rows, d), bf16, dev), v_out=_kept(b, "vc", (*rows, d), bf16, dev),
                             pos_out=_kept(b, "pos", rows, i32, dev))
-    pa = parallel_attn(q[0:1, L - w:], kc.unsqueeze(0), vc.unsqueeze(0), b["k_rot"][0:1, L - w:], v[0:1, L - w:],
+    pa = parallel_attn(_window(q, L, w), kc.unsqueeze(0), vc.unsqueeze(0), _window(b["k_rot"], L, w), _window(v, L, w),
                        q_pos0=L - w, rope_theta=rope_theta, softmax_scale=softmax_scale, out=_kept(b, "fg", (1, w, Hq, d), bf16, dev),
                        status=b["status"], workspace=b.get("ws_par"))
     b.update(chunk_score=score, kept=kept, idx=idx, kc=kc, vc=vc, pos=pos, fg=pa["out"], ws_par=pa["workspace"])
